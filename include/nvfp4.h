@@ -236,7 +236,7 @@ NVFP4_API nvfp4_status nvfp4_sq_error(const void* ref, int32_t ref_is_fp32, int6
  *   When both GEMMs are requested they run in one launch of the CTA-pair kernel.
  * Ordering: both calls are stream-ordered as a whole (everything enqueued before them on the stream has
  *   finished before their first kernel starts, and their results are complete for whatever is enqueued after
- *   them).  Inside a call the kernels overlap only their set-up with the tail of the kernel before them
+ *   them).  The kernels of this library overlap only their set-up with the tail of the kernel before them
  *   (programmatic dependent launch) and never read each other's output early; in the NVFP4 bf16 path the tensor
  *   amax of W (Appendix B.1) is taken inside the kernel that quantizes X.  Results are bit-identical to the
  *   same steps issued one by one through nvfp4_quantize and nvfp4_gemm.

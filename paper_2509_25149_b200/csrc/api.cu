@@ -126,7 +126,10 @@ nvfp4_status quantize_impl(const void* x, int64_t rows, int64_t cols, int64_t ld
   if (mx)  // no tensor-level scale, hence no amax pass
     return launch_quantize_mx(a, hr, hc, b2, o->rht_colwise != 0, sr, s) == cudaSuccess ? NVFP4_OK : NVFP4_ERR_CUDA;
   if (f32) {
-    if (!(o->flags & NVFP4_AMAX_PROVIDED) && launch_amax_f32(a, hr, hc, s) != cudaSuccess) return NVFP4_ERR_CUDA;
+    if (!(o->flags & NVFP4_AMAX_PROVIDED)) {
+      if (launch_amax_f32(a, hr, hc, s) != cudaSuccess) return NVFP4_ERR_CUDA;
+      a.chained = 1;
+    }
     return launch_quantize_f32(a, hr, hc, b2, sr, s) == cudaSuccess ? NVFP4_OK : NVFP4_ERR_CUDA;
   }
   if (other_dim) {
@@ -145,13 +148,12 @@ nvfp4_status quantize_impl(const void* x, int64_t rows, int64_t cols, int64_t ld
     return launch_quantize_rht(ra, (o->flags & NVFP4_AMAX_PROVIDED) != 0, sr, s) == cudaSuccess ? NVFP4_OK
                                                                                                   : NVFP4_ERR_CUDA;
   }
-  // pass 2 may become resident while the previous kernel of this call drains (its own pass 1, or the caller's launch)
+  // pass 2 may read the source while the previous kernel of this call drains (its own pass 1, or the kernel before)
   a.chained = chained;
   // only the forward pass's activation quantize carries a side job (see side_amax_fits); checked before any launch
-  if (side && (!hr || b2 || sr || o->rht_rowwise || (hc && !o->rht_colwise))) return NVFP4_ERR_ARG;
-  if (side && zero_side_amax(*side, s) != cudaSuccess) return NVFP4_ERR_CUDA;  // not between pass 1 and pass 2
+  if (side && (!hr || (o->flags & NVFP4_AMAX_PROVIDED) || b2 || sr || o->rht_rowwise || (hc && !o->rht_colwise))) return NVFP4_ERR_ARG;
   if (!(o->flags & NVFP4_AMAX_PROVIDED)) {
-    if (launch_amax(a, hr, hc, o->rht_rowwise != 0, o->rht_colwise != 0, s) != cudaSuccess) return NVFP4_ERR_CUDA;
+    if (launch_amax(a, hr, hc, o->rht_rowwise != 0, o->rht_colwise != 0, side, s) != cudaSuccess) return NVFP4_ERR_CUDA;
     a.chained = 1;
   }
   if (side) {
@@ -222,11 +224,10 @@ int gemm_tile(const GemmArgs& g) {
 }
 
 nvfp4_status gemm_impl(const nvfp4_tensor* A, const nvfp4_tensor* B, void* D, int32_t d_is_fp32, int64_t ldd,
-                       int32_t accumulate, cudaStream_t s, bool chained = false) {
+                       int32_t accumulate, cudaStream_t s) {
   GemmArgs g;
   nvfp4_status st = gemm_prepare(A, B, D, d_is_fp32, ldd, accumulate, g);
   if (st != NVFP4_OK) return st;
-  g.chained = chained;
   if (launch_gemm(g, A->codes, B->codes, gemm_tile(g), s) != cudaSuccess) return NVFP4_ERR_CUDA;
   return NVFP4_OK;
 }
@@ -336,12 +337,11 @@ nvfp4_status nvfp4_linear_fwd(const void* X, const void* W, int64_t M, int64_t N
     if ((st = quantize_impl(X, M, K, K, &xo, &x_row, X_col_saved, s, false, &w_amax)) != NVFP4_OK) return st;
     wo.flags |= NVFP4_AMAX_PROVIDED;
     if ((st = quantize_impl(W, N, K, K, &wo, W_row, W_col_saved, s, false, nullptr, true)) != NVFP4_OK) return st;
-    return gemm_impl(&x_row, W_row, Y_bf16, 0, N, 0, s, true);
+    return gemm_impl(&x_row, W_row, Y_bf16, 0, N, 0, s);
   }
   if (!w_is_cached && (st = quantize_impl(W, N, K, K, &wo, W_row, W_col_saved, s)) != NVFP4_OK) return st;
   if ((st = quantize_impl(X, M, K, K, &xo, &x_row, X_col_saved, s)) != NVFP4_OK) return st;
-  // behind a quantizer of this call the GEMM may set itself up while that kernel drains
-  return gemm_impl(&x_row, W_row, Y_bf16, 0, N, 0, s, true);
+  return gemm_impl(&x_row, W_row, Y_bf16, 0, N, 0, s);
 }
 
 nvfp4_status nvfp4_linear_bwd(const void* dY, const nvfp4_tensor* X_col_saved, const nvfp4_tensor* W_col_saved,
@@ -391,7 +391,6 @@ nvfp4_status nvfp4_linear_bwd(const void* dY, const nvfp4_tensor* X_col_saved, c
     GemmArgs gd, gw;
     if ((st = gemm_prepare(&g_row, W_col_saved, dX_bf16, 0, K, 0, gd)) != NVFP4_OK) return st;
     if ((st = gemm_prepare(&g_col, X_col_saved, dW_fp32, 1, K, accumulate_dw, gw)) != NVFP4_OK) return st;
-    gd.chained = gw.chained = 1;  // behind the quantizer of dY
     const int td = gemm_tile(gd), tw = gemm_tile(gw);
     if ((td == 512 || td == 768) && (tw == 512 || tw == 768)) {
       const bool forced = g_tile_n.load(std::memory_order_relaxed) != 0;
@@ -403,7 +402,7 @@ nvfp4_status nvfp4_linear_bwd(const void* dY, const nvfp4_tensor* X_col_saved, c
       return e == cudaSuccess ? NVFP4_OK : NVFP4_ERR_CUDA;
     }
   }
-  if (dX_bf16 && (st = gemm_impl(&g_row, W_col_saved, dX_bf16, 0, K, 0, s, true)) != NVFP4_OK) return st;
+  if (dX_bf16 && (st = gemm_impl(&g_row, W_col_saved, dX_bf16, 0, K, 0, s)) != NVFP4_OK) return st;
   if (dW_fp32 && (st = gemm_impl(&g_col, X_col_saved, dW_fp32, 1, K, accumulate_dw, s)) != NVFP4_OK) return st;
   return NVFP4_OK;
 }

@@ -55,10 +55,14 @@ __device__ __forceinline__ void fence_mbarrier_init() {
 // orders this thread's earlier generic-proxy accesses to shared memory before later asynchronous-proxy ones (TMA)
 __device__ __forceinline__ void fence_proxy_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
-// ---- programmatic dependent launch: a kernel launched with `launch_kernel(..., after_own_kernel = true)` may become
-// resident while the previous kernel of the stream drains; it runs its set-up (barriers, tensor memory, descriptor
-// prefetch, loads of data the previous kernel does not write) and then waits here for that kernel to finish with all
-// its writes visible.  A no-op for a kernel that was launched the ordinary way.
+// ---- programmatic dependent launch: every kernel launched with `launch_kernel` may become resident while the previous
+// kernel of the stream drains; it runs its set-up (barriers, tensor memory, descriptor prefetch) and then waits here for
+// that kernel to finish with all its writes visible.  Behind a kernel that does not know the scheme (a caller's own) the
+// launch is held until that kernel's CTAs have exited, and the wait covers its writes.  Rules that keep it transitive:
+//   - every kernel waits before it finishes, so "kernel n has finished" implies "kernel n - 1 has finished";
+//   - before its wait a kernel touches only what no kernel that may still run writes: the kernel that zeroes the words of
+//     a call (zero_words_kernel) waits first and only then lets its dependent start, so the reductions behind it may read
+//     their inputs at once and wait just before their first atomic.
 __device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // lets the next kernel of the stream, if it was launched that way, become resident as CTAs of this grid retire
 __device__ __forceinline__ void griddep_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
@@ -66,7 +70,7 @@ __device__ __forceinline__ void griddep_launch_dependents() { asm volatile("grid
 #ifdef __CUDACC__
 template <typename... Params, typename... Args>
 inline cudaError_t launch_kernel(void (*kern)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
-                                 bool after_own_kernel, Args&&... args) {
+                                 Args&&... args) {
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = grid;
   cfg.blockDim = block;
@@ -76,7 +80,7 @@ inline cudaError_t launch_kernel(void (*kern)(Params...), dim3 grid, dim3 block,
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = after_own_kernel ? 1 : 0;
+  cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kern, static_cast<Params>(args)...);
 }
 #endif

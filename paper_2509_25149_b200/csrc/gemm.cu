@@ -162,6 +162,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  griddep_wait();  // the set-up above ran beside the previous kernel; from here on its output is touched
+  griddep_launch_dependents();
 
   if (warp == 0) {
     // ------------------------------------------------------------------ producer ----
@@ -363,9 +365,9 @@ cudaError_t launch_t(const GemmArgs& g, const void* a_codes, const void* b_codes
   }
   const int n_tiles = (g.M / BM) * (g.N / BN);
   const int grid = n_tiles < num_sms ? n_tiles : num_sms;
-  kern<<<grid, kThreads, C::kSmemBytes, s>>>(map_a, map_b, g);
+  const cudaError_t le = launch_kernel(kern, dim3(grid), dim3(kThreads), C::kSmemBytes, s, map_a, map_b, g);
   count_launch();
-  return cudaGetLastError();
+  return le;
 }
 
 bool make_pair_maps(const GemmArgs& g, const void* a_codes, const void* b_codes, CUtensorMap* map_a, CUtensorMap* map_b,
@@ -432,20 +434,19 @@ cudaError_t launch_pair(const GemmArgs& g0, const void* a0, const void* b0, cons
       device_configured(configured_rows, dev);
     }
   }
-  const bool chained = g0.chained != 0;
   const dim3 grid(2 * pairs), block(pair::kThreads);
   cudaError_t le;
   if (rows)
-    le = launch_kernel(pair::gemm_pair_kernel<false, true>, grid, block, pair::kSmemBytes, s, chained, m[0], m[1], m[2],
+    le = launch_kernel(pair::gemm_pair_kernel<false, true>, grid, block, pair::kSmemBytes, s, m[0], m[1], m[2],
                        m[3], m[4], m[5], a);
   else if (g0.mx)
-    le = launch_kernel(pair::gemm_pair_kernel<true>, grid, block, pair::kSmemBytes, s, chained, m[0], m[1], m[2], m[3],
+    le = launch_kernel(pair::gemm_pair_kernel<true>, grid, block, pair::kSmemBytes, s, m[0], m[1], m[2], m[3],
                        m[4], m[5], a);
   else
-    le = launch_kernel(pair::gemm_pair_kernel<false>, grid, block, pair::kSmemBytes, s, chained, m[0], m[1], m[2], m[3],
+    le = launch_kernel(pair::gemm_pair_kernel<false>, grid, block, pair::kSmemBytes, s, m[0], m[1], m[2], m[3],
                        m[4], m[5], a);
   count_launch();
-  return le != cudaSuccess ? le : cudaGetLastError();
+  return le;
 }
 
 // N = 128 q = 384 a + 256 b with b in {0, 1, 2}: a wide column tiles, b narrow ones (q >= 2)
@@ -549,12 +550,12 @@ cudaError_t launch_wide(const GemmArgs& g0, const void* a0, const void* b0, cons
   const int pairs = a.n_tiles < max_pairs ? a.n_tiles : max_pairs;
   const dim3 grid(2 * pairs), block(wide::kWThreads);
   const cudaError_t le =
-      g0.mx ? launch_kernel(wide::gemm_wide_kernel<true>, grid, block, wide::kWSmemBytes, s, g0.chained != 0, m[0], m[1],
+      g0.mx ? launch_kernel(wide::gemm_wide_kernel<true>, grid, block, wide::kWSmemBytes, s, m[0], m[1],
                             m[2], m[3], m[4], m[5], m[6], m[7], a)
-            : launch_kernel(wide::gemm_wide_kernel<false>, grid, block, wide::kWSmemBytes, s, g0.chained != 0, m[0], m[1],
+            : launch_kernel(wide::gemm_wide_kernel<false>, grid, block, wide::kWSmemBytes, s, m[0], m[1],
                             m[2], m[3], m[4], m[5], m[6], m[7], a);
   count_launch();
-  return le != cudaSuccess ? le : cudaGetLastError();
+  return le;
 }
 
 cudaError_t sm_count(int* n) {
@@ -657,9 +658,10 @@ cudaError_t launch_gemm_bf16(const DenseGemmArgs& g, cudaStream_t s) {
   dense::Args a{g.M, g.N, g.K, g.a_mn, g.b_mn, g.d_is_fp32, g.accumulate};
   const int n_tiles = ((g.M + 255) / 256) * ((g.N + 255) / 256), max_pairs = num_sms / 2;
   const int pairs = n_tiles < max_pairs ? n_tiles : max_pairs;
-  dense::gemm_bf16_pair_kernel<<<2 * pairs, dense::kThreads, dense::kSmemBytes, s>>>(map_a, map_b, map_d, a);
+  e = launch_kernel(dense::gemm_bf16_pair_kernel, dim3(2 * pairs), dim3(dense::kThreads), dense::kSmemBytes, s, map_a,
+                    map_b, map_d, a);
   count_launch();
-  return cudaGetLastError();
+  return e;
 }
 
 // Test aid: one warp waits, with the given limit, on a barrier nobody arrives at.  The wait runs out, the code lands

@@ -115,6 +115,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   cluster_sync_all();  // both CTAs' barriers are initialised before any remote signal
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  griddep_wait();  // the set-up above ran beside the previous kernel; from here on its output is touched
+  griddep_launch_dependents();
 
   if (warp == 0) {
     // ------------------------------------------------------------------ producer ----

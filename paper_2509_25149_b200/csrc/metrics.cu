@@ -9,6 +9,7 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
+#include "async_ptx.cuh"
 #include "common.cuh"
 #include "quantize.h"
 #include "quantize_common.cuh"
@@ -31,6 +32,7 @@ __device__ __forceinline__ void block_reduce_add(double err, double ref, double*
   }
   __syncthreads();
   if (threadIdx.x < 2) {
+    griddep_wait();  // the sums are zero
     double s = 0.0;
 #pragma unroll
     for (int w = 0; w < 8; ++w) s += red[threadIdx.x][w];
@@ -156,41 +158,38 @@ cudaError_t grid_for(int64_t units, unsigned* grid) {
   return cudaSuccess;
 }
 
+cudaError_t zero_sums(double* out, cudaStream_t s) {  // the kernel behind it reads its tensors meanwhile
+  float* w = reinterpret_cast<float*>(out);
+  return launch_zero_words(w, w + 1, w + 2, w + 3, s);
+}
+
 }  // namespace
 
 cudaError_t launch_quant_error(const void* x, int64_t rows, int64_t cols, int64_t ld, const nvfp4_tensor& q,
                                double* out, cudaStream_t s) {
-  cudaError_t e = cudaMemsetAsync(out, 0, 2 * sizeof(double), s);
+  cudaError_t e = zero_sums(out, s);
   if (e != cudaSuccess) return e;
   unsigned grid;
   if ((e = grid_for(rows * (cols >> 4), &grid)) != cudaSuccess) return e;
   const int swz = q.sf_layout == NVFP4_SF_SWIZZLED;
-  if (q.format == NVFP4_FORMAT_MXFP4)
-    quant_error_kernel<true><<<grid, 256, 0, s>>>(static_cast<const uint16_t*>(x), rows, cols, ld, q.codes, q.scales,
-                                                  q.global, swz, 0, out);
-  else
-    quant_error_kernel<false><<<grid, 256, 0, s>>>(static_cast<const uint16_t*>(x), rows, cols, ld, q.codes, q.scales,
-                                                   q.global, swz, q.format == NVFP4_FORMAT_NVFP4_ROWSCALE, out);
+  e = launch_kernel(q.format == NVFP4_FORMAT_MXFP4 ? quant_error_kernel<true> : quant_error_kernel<false>, dim3(grid),
+                    dim3(256), 0, s, static_cast<const uint16_t*>(x), rows, cols, ld, q.codes, q.scales, q.global, swz,
+                    q.format == NVFP4_FORMAT_NVFP4_ROWSCALE, out);
   count_launch();
-  return cudaGetLastError();
+  return e;
 }
 
 cudaError_t launch_sq_error(const void* ref, bool ref_fp32, int64_t ld_ref, const void* test, bool test_fp32,
                             int64_t ld_test, int64_t rows, int64_t cols, double* out, cudaStream_t s) {
-  cudaError_t e = cudaMemsetAsync(out, 0, 2 * sizeof(double), s);
+  cudaError_t e = zero_sums(out, s);
   if (e != cudaSuccess) return e;
   unsigned grid;
   if ((e = grid_for(rows * (cols >> 3), &grid)) != cudaSuccess) return e;
-#define NVFP4_SQ(R, T)                                                                                        \
-  if (ref_fp32 == R && test_fp32 == T)                                                                        \
-    sq_error_kernel<R, T><<<grid, 256, 0, s>>>(ref, ld_ref, test, ld_test, rows, cols, out);
-  NVFP4_SQ(false, false)
-  NVFP4_SQ(false, true)
-  NVFP4_SQ(true, false)
-  NVFP4_SQ(true, true)
-#undef NVFP4_SQ
+  auto kern = ref_fp32 ? (test_fp32 ? sq_error_kernel<true, true> : sq_error_kernel<true, false>)
+                       : (test_fp32 ? sq_error_kernel<false, true> : sq_error_kernel<false, false>);
+  e = launch_kernel(kern, dim3(grid), dim3(256), 0, s, ref, ld_ref, test, ld_test, rows, cols, out);
   count_launch();
-  return cudaGetLastError();
+  return e;
 }
 
 }  // namespace nvfp4

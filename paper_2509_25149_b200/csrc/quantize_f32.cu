@@ -2,6 +2,7 @@
 // e.g. weights quantized straight from their FP32 master copy.  Same two passes and the same arithmetic as the bf16
 // kernels of quantize.cu, only the element read differs: the tile is staged as FP32 (64 KB), a chunk is two 32-byte
 // loads.  No Hadamard transform (the recipe transforms activations and gradients, which are bf16).
+#include "async_ptx.cuh"
 #include "quantize.h"
 #include "quantize_common.cuh"
 
@@ -20,7 +21,8 @@ __global__ void __launch_bounds__(256) amax_f32_kernel(const float* __restrict__
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t tr = blockIdx.x / tiles_c, tc = blockIdx.x % tiles_c;
   const int64_t r0 = tr * 128 + warp * 16, c0 = tc * 128 + lane * 4;
-  float m = 0.f;
+  griddep_launch_dependents();  // pass 2 may load its tiles while the last CTAs of this pass run
+  float m = 0.f;  // (the source is complete: zero_words_kernel has waited for it)
   if (r0 < rows && c0 < cols) {  // rows % 16 == 0, cols % 16 == 0
     uint4 v[16];
 #pragma unroll
@@ -35,6 +37,7 @@ __global__ void __launch_bounds__(256) amax_f32_kernel(const float* __restrict__
   if (lane == 0) red[warp] = m;
   __syncthreads();
   if (threadIdx.x == 0) {
+    griddep_wait();  // the words are zero
     float t = 0.f;
 #pragma unroll
     for (int w = 0; w < 8; ++w) t = fmaxf(t, red[w]);
@@ -70,7 +73,10 @@ __global__ void __launch_bounds__(256, 2) quantize_f32_kernel(const QuantArgs a)
   const int64_t n_cb = a.cols >> 4, n_rb = a.rows >> 4;
 
   float* g_sc = reinterpret_cast<float*>(smem + F32Smem::kGlobalScales);
+  if (!a.chained) griddep_wait();  // the source may be the previous kernel's output
+  griddep_launch_dependents();
   if (threadIdx.x == 0) {  // Eq. 1 once per CTA
+    griddep_wait();  // (every other thread passes the barrier in front of the first output only after this wait)
     float re = 1.f, rd = 1.f, ce = 1.f, cd = 1.f;
     if (HAS_ROW || BLOCK2D) global_scales(HAS_ROW ? a.r_global[0] : a.c_global[0], re, rd);
     if (HAS_COL) {
@@ -269,15 +275,14 @@ __global__ void __launch_bounds__(256, 2) quantize_f32_kernel(const QuantArgs a)
 }
 
 cudaError_t launch_amax_f32(const QuantArgs& a, bool has_row, bool has_col, cudaStream_t s) {
-  cudaError_t e;
-  if (has_row && (e = cudaMemsetAsync(a.r_global, 0, sizeof(float), s)) != cudaSuccess) return e;
-  if (has_col && (e = cudaMemsetAsync(a.c_global, 0, sizeof(float), s)) != cudaSuccess) return e;
+  cudaError_t e = launch_zero_words(has_row ? a.r_global : nullptr, has_col ? a.c_global : nullptr, nullptr, nullptr, s);
+  if (e != cudaSuccess) return e;
   const int tiles_c = (int)((a.cols + 127) / 128);
   const unsigned tiles = (unsigned)(((a.rows + 127) / 128) * tiles_c);
-  amax_f32_kernel<<<tiles, 256, 0, s>>>(reinterpret_cast<const float*>(a.x), a.rows, a.cols, a.ld, tiles_c,
-                                        has_row ? a.r_global : nullptr, has_col ? a.c_global : nullptr);
+  e = launch_kernel(amax_f32_kernel, dim3(tiles), dim3(256), 0, s, reinterpret_cast<const float*>(a.x), a.rows, a.cols,
+                    a.ld, tiles_c, has_row ? a.r_global : nullptr, has_col ? a.c_global : nullptr);
   count_launch();
-  return cudaGetLastError();
+  return e;
 }
 
 template <bool HR, bool HC, bool B2, bool SR>
@@ -291,9 +296,9 @@ static cudaError_t launch_f32_t(const QuantArgs& a, cudaStream_t s) {
     if (e != cudaSuccess) return e;
     device_configured(configured, dev);
   }
-  kern<<<(unsigned)((int64_t)a.tiles_r * a.tiles_c), 256, smem, s>>>(a);
+  const cudaError_t e = launch_kernel(kern, dim3((unsigned)((int64_t)a.tiles_r * a.tiles_c)), dim3(256), smem, s, a);
   count_launch();
-  return cudaGetLastError();
+  return e;
 }
 
 cudaError_t launch_quantize_f32(const QuantArgs& a, bool has_row, bool has_col, bool block2d, bool sr, cudaStream_t s) {

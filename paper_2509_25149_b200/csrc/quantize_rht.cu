@@ -345,8 +345,8 @@ cudaError_t launch_quantize_rht(const RhtArgs& ra, bool amax_provided, bool sr, 
     // the recipe's case (plain row-wise copy, transformed transposed copy): pass 1 on the tensor cores, HBM-bound
     if ((e = launch_amax_rot_col_small(ra.q, ra.has_row != 0, ra.mask16, ra.d, ra.norm, s)) != cudaSuccess) return e;
   } else if (!amax_provided) {
-    if (ra.has_row && (e = cudaMemsetAsync(ra.q.r_global, 0, sizeof(float), s)) != cudaSuccess) return e;
-    if (ra.has_col && (e = cudaMemsetAsync(ra.q.c_global, 0, sizeof(float), s)) != cudaSuccess) return e;
+    e = launch_zero_words(ra.has_row ? ra.q.r_global : nullptr, ra.has_col ? ra.q.c_global : nullptr, nullptr, nullptr, s);
+    if (e != cudaSuccess) return e;
     if ((e = launch_mode<0, false>(ra, s)) != cudaSuccess) return e;
   }
   return sr ? launch_mode<1, true>(ra, s) : launch_mode<1, false>(ra, s);

@@ -1,0 +1,90 @@
+"""Kernels of consecutive calls overlap their set-up with the kernel before them (programmatic dependent launch).  Whatever
+precedes a call on the stream (another kernel, a copy, a fill, an event of another stream), directly or inside a captured
+graph, the call sees its finished result: outputs are bit-identical to those of the same call on a quiet GPU."""
+import pytest
+import torch
+
+from paper_2509_25149_b200 import binding as B
+from paper_2509_25149_b200 import synth
+
+pytestmark = pytest.mark.gpu
+M, N, K = 512, 768, 1024
+
+
+def _call(kind, x, w_q, out):
+    """One public call whose first kernel reads x; returns the tensors to compare."""
+    if kind == "bf16":
+        B.nvfp4_gemm_bf16(x, x, out["d32"])
+        return [out["d32"]]
+    if kind == "error":
+        return [B.nvfp4_quant_error(x, out["row"], out["sums"]).float()]  # (FP64 atomics: the order varies)
+    opts = {"nvfp4": B.quant_opts(rounding=1, rht_colwise=True, rht_sign_mask=synth.DEFAULT_RHT_SIGN_MASK, seed=1),
+            "mxfp4": B.quant_opts(rht_colwise=True, rht_sign_mask=0x73E5), "rows": B.quant_opts(),
+            "provided": B.quant_opts(flags=B.AMAX_PROVIDED)}[kind]
+    t = {"mxfp4": "mx", "rows": "rs"}.get(kind, "")
+    row, col = out[t + "row"], None if kind in ("rows", "provided") else out[t + "col"]
+    B.nvfp4_quantize(x, opts, row, col)
+    res = [row.codes, row.scales, row.glob] + ([col.codes, col.scales, col.glob] if col else [])
+    if kind != "mxfp4":
+        B.nvfp4_gemm(row, w_q, out["d"])
+        res.append(out["d"])
+    return res
+
+
+@pytest.mark.parametrize("before", ["kernel", "copy", "fill", "other stream"])
+@pytest.mark.parametrize("kind", ["nvfp4", "mxfp4", "rows", "provided", "bf16", "error"])
+def test_a_call_sees_what_precedes_it(kind, before):
+    src = torch.randn((M, K), generator=torch.Generator("cuda").manual_seed(1), device="cuda").to(torch.bfloat16)
+    w_q = B.alloc_tensor(N, K)
+    B.nvfp4_quantize(src[:256].repeat(3, 1).contiguous(), B.quant_opts(), w_q, None)
+    out = {"row": B.alloc_tensor(M, K), "col": B.alloc_tensor(K, M),
+           "mxrow": B.alloc_tensor(M, K, format=B.FORMAT_MXFP4), "mxcol": B.alloc_tensor(K, M, format=B.FORMAT_MXFP4),
+           "rsrow": B.alloc_tensor(M, K, format=B.FORMAT_NVFP4_ROWSCALE),
+           "d": torch.empty((M, N), dtype=torch.bfloat16, device="cuda"),
+           "d32": torch.empty((M, M), dtype=torch.float32, device="cuda"),
+           "sums": torch.empty(2, dtype=torch.float64, device="cuda")}
+    B.nvfp4_quantize(src, B.quant_opts(), out["row"], None)
+    if kind == "provided":
+        out["row"].glob.fill_(8.0)
+    big = torch.randn((4096, 4096), device="cuda")
+    x, other = torch.empty_like(src), torch.cuda.Stream()
+
+    def produce():  # x = src (or zeros for "fill"), the last operation before the call a slow or non-kernel one
+        if before == "fill":
+            x.copy_(src)
+            x.view(torch.int16).zero_()
+        elif before == "other stream":
+            other.wait_stream(torch.cuda.current_stream())
+            with torch.cuda.stream(other):
+                torch.mm(big, big)
+                x.copy_(src)
+            torch.cuda.current_stream().wait_stream(other)
+        elif before == "copy":
+            x.copy_(src)  # same type and shape: a device-to-device copy
+        else:
+            torch.mm(big, big)
+            torch.mul(src, 1.0, out=x)
+
+    produce()
+    torch.cuda.synchronize()
+    want = [t.clone() for t in _call(kind, x, w_q, out)]
+    torch.cuda.synchronize()
+    for _ in range(10):
+        x.fill_(float("nan"))
+        produce()
+        for got, ref in zip(_call(kind, x, w_q, out), want):
+            assert torch.equal(got, ref)
+    graph, side = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+    side.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(side):
+        with torch.cuda.graph(graph, stream=side):
+            produce()
+            res = _call(kind, x, w_q, out)
+    torch.cuda.synchronize()
+    for _ in range(5):
+        x.fill_(float("nan"))
+        graph.replay()
+        torch.cuda.synchronize()
+        for got, ref in zip(res, want):
+            assert torch.equal(got, ref)
+    B.nvfp4_device_status()
