@@ -153,7 +153,7 @@ NVFP4_API nvfp4_status nvfp4_quantize(const void* x_bf16, int64_t rows, int64_t 
  * nvfp4_gemm -- Eq. 5: D[i][j] = s_dec^A * s_dec^B * sum_blocks S^A[i,b] S^B[j,b] sum_{k in b} a[i,k] b[j,k]
  *   A [M x K], B [N x K]: quantized copies whose columns are the contraction dimension, scales in
  *   the NVFP4_SF_SWIZZLED layout, M % 128 == 0, N % 128 == 0, K % 256 == 0 (K = A->cols = B->cols).
- *   Shapes with M % 256 == 0 run on CTA pairs (256 x 256 or 256 x 384 tiles), others on one CTA per tile.
+ *   Runs on CTA pairs with 256 x 128, 256 x 256 or 256 x 384 tiles, whichever schedule is estimated shorter.
  *   D: device, row-major [M x N] with leading dimension ldd (elements, >= N, ldd*elemsize % 16 == 0),
  *   bf16 (round-to-nearest-even) when d_is_fp32 == 0, else fp32.  Partial sums are accumulated in
  *   FP32 by the tensor cores; the product of the two tensor decode scales is applied once at the end.
@@ -318,11 +318,10 @@ NVFP4_API nvfp4_status nvfp4_device_status(void* cuda_stream, uint32_t* detail);
  */
 NVFP4_API nvfp4_status nvfp4_test_wait_timeout(uint64_t limit_ns, void* cuda_stream);
 
-/* Tuning knob: which GEMM tiling to use.  128 / 256 = one CTA per 128 x 128 / 128 x 256 output tile;
- * 512 = a CTA pair per 256 x 256 tile (needs M % 256 == 0 and N % 256 == 0, otherwise 128 is used);
- * 768 = a CTA pair per 256 x 384 tile, plus up to two 256-wide tiles per row of tiles (needs M % 256 == 0,
- * N % 128 == 0 and N >= 256, otherwise as 512);
- * 0 = choose by shape (for the pair kernels: the tile width whose static schedule is estimated shorter).
+/* Tuning knob: which GEMM tiling to use.  128 / 256 = one CTA per 128 x 128 / 128 x 256 output tile (256 needs
+ * N % 256 == 0, otherwise 128 is used); CTA pairs: 640 = 256 x 128 tiles, 512 = 256 x 256 tiles, 768 = 256 x 384 tiles plus
+ * up to two 256-wide ones per row of tiles (needs N >= 256 and per-tensor scales, otherwise as 512);
+ * 0 = choose by shape (the CTA-pair tile whose static schedule is estimated shortest).
  * Returns 0, or -1 for any other value.  Process-wide; results do not depend on it
  * beyond FP32 summation order. */
 NVFP4_API int32_t nvfp4_set_gemm_tile_n(int32_t tile_n);

@@ -204,23 +204,10 @@ nvfp4_status gemm_prepare(const nvfp4_tensor* A, const nvfp4_tensor* B, void* D,
   return NVFP4_OK;
 }
 
-int gemm_tile(const GemmArgs& g) {
-  const int M = g.M, N = g.N, K = g.K;
-  const int d_is_fp32 = g.d_is_fp32;
-  // CTA pairs on 256 x 256 tiles whenever the shape allows (half the operand traffic per flop, half the
-  // scale-copy and MMA issue work per SM).  Otherwise one CTA per tile: 128 x 256 tiles hold one accumulator
-  // (exposed epilogue), 128 x 128 tiles two (the epilogue overlaps the next tile), so the wide tile pays off
-  // once the main loop is long enough to amortise the epilogue.
-  int tile_n = g_tile_n.load(std::memory_order_relaxed);
-  if (tile_n != 128 && tile_n != 256 && tile_n != 512 && tile_n != 768) {
-    if (M % 256 == 0 && N % 256 == 0)
-      tile_n = prefer_wide_tiles(g, nullptr) ? 768 : 512;  // CTA pairs: the tile width with the shorter schedule
-    else if (M % 256 == 0 && N % 128 == 0 && N >= 256)
-      tile_n = 768;
-    else
-      tile_n = (K >= (d_is_fp32 ? 16384 : 8192)) ? 256 : 128;
-  }
-  return tile_n;
+// The tile of a launch: the caller's (nvfp4_set_gemm_tile_n), or the CTA-pair tile with the shortest estimated schedule
+int gemm_tile(const GemmArgs& g0, const GemmArgs* g1 = nullptr) {
+  const int forced = g_tile_n.load(std::memory_order_relaxed);
+  return forced ? forced : best_pair_tile(g0, g1);
 }
 
 nvfp4_status gemm_impl(const nvfp4_tensor* A, const nvfp4_tensor* B, void* D, int32_t d_is_fp32, int64_t ldd,
@@ -391,14 +378,12 @@ nvfp4_status nvfp4_linear_bwd(const void* dY, const nvfp4_tensor* X_col_saved, c
     GemmArgs gd, gw;
     if ((st = gemm_prepare(&g_row, W_col_saved, dX_bf16, 0, K, 0, gd)) != NVFP4_OK) return st;
     if ((st = gemm_prepare(&g_col, X_col_saved, dW_fp32, 1, K, accumulate_dw, gw)) != NVFP4_OK) return st;
-    const int td = gemm_tile(gd), tw = gemm_tile(gw);
-    if ((td == 512 || td == 768) && (tw == 512 || tw == 768)) {
-      const bool forced = g_tile_n.load(std::memory_order_relaxed) != 0;
-      const bool dgrad_first = gd.K >= gw.K;
-      const bool wide = forced ? td == 768 : prefer_wide_tiles(dgrad_first ? gd : gw, dgrad_first ? &gw : &gd);
+    const bool dgrad_first = gd.K >= gw.K;
+    const int tile = dgrad_first ? gemm_tile(gd, &gw) : gemm_tile(gw, &gd);
+    if (tile >= kTilePair256) {
       const cudaError_t e =
-          dgrad_first ? launch_gemm_two(gd, g_row.codes, W_col_saved->codes, gw, g_col.codes, X_col_saved->codes, wide, s)
-                      : launch_gemm_two(gw, g_col.codes, X_col_saved->codes, gd, g_row.codes, W_col_saved->codes, wide, s);
+          dgrad_first ? launch_gemm_two(gd, g_row.codes, W_col_saved->codes, gw, g_col.codes, X_col_saved->codes, tile, s)
+                      : launch_gemm_two(gw, g_col.codes, X_col_saved->codes, gd, g_row.codes, W_col_saved->codes, tile, s);
       return e == cudaSuccess ? NVFP4_OK : NVFP4_ERR_CUDA;
     }
   }
@@ -548,7 +533,8 @@ int32_t nvfp4_set_gemm_experiment(int32_t mode, int32_t max_pairs, void* probe) 
 }
 
 int32_t nvfp4_set_gemm_tile_n(int32_t tile_n) {
-  if (tile_n != 0 && tile_n != 128 && tile_n != 256 && tile_n != 512 && tile_n != 768) return -1;
+  if (tile_n != 0 && tile_n != 128 && tile_n != 256 && tile_n != 512 && tile_n != 640 && tile_n != 768)
+    return -1;
   g_tile_n.store(tile_n, std::memory_order_relaxed);
   return 0;
 }

@@ -12,8 +12,8 @@
 // Every wait is bounded: when one expires the kernel records a code in a device status word, every role
 // leaves its loop, tensor memory is released and the kernel returns.
 //
-// This file holds the one-CTA kernel (shapes with M or N not a multiple of 256), the tensor-map helpers and the
-// launchers of both kernels; the CTA-pair kernel that carries the large shapes is in gemm_2cta.cuh.
+// This file holds the one-CTA kernel (only on request, nvfp4_set_gemm_tile_n), the tensor-map helpers and the launchers of
+// all kernels; the CTA-pair kernels that take every shape are in gemm_2cta.cuh and gemm_wide.cuh.
 #include <cuda.h>
 #include <cuda_bf16.h>
 
@@ -370,12 +370,12 @@ cudaError_t launch_t(const GemmArgs& g, const void* a_codes, const void* b_codes
   return le;
 }
 
-bool make_pair_maps(const GemmArgs& g, const void* a_codes, const void* b_codes, CUtensorMap* map_a, CUtensorMap* map_b,
-                    CUtensorMap* map_d) {
-  bool ok = make_code_map(map_a, a_codes, g.M, g.K / 2, 128) && make_code_map(map_b, b_codes, g.N, g.K / 2, 128);
+bool make_pair_maps(const GemmArgs& g, const void* a_codes, const void* b_codes, int bn, CUtensorMap* map_a,
+                    CUtensorMap* map_b, CUtensorMap* map_d) {
+  bool ok = make_code_map(map_a, a_codes, g.M, g.K / 2, 128) && make_code_map(map_b, b_codes, g.N, g.K / 2, bn / 2);
   if (g.d_is_fp32)
     ok = ok && make_map_2d(map_d, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, g.d, (uint64_t)g.N, (uint64_t)g.M,
-                           (uint64_t)g.ldd * 4, 32, 128, true);
+                           (uint64_t)g.ldd * 4, 16, 128, 2);
   else
     ok = ok && make_map_2d(map_d, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, g.d, (uint64_t)g.N, (uint64_t)g.M,
                            (uint64_t)g.ldd * 2, 64, 128, true);
@@ -390,63 +390,59 @@ pair::Problem pair_problem(const GemmArgs& g) {
   return pair::Problem{g.M, g.N, g.K, g.sfa, g.sfb, g.a_global, g.b_global, g.d_is_fp32, g.accumulate, g.a_rows, g.b_rows};
 }
 
+// tiles of a problem on CTA pairs with BN columns; the last one in either direction may be half outside
+inline int pair_tiles(const GemmArgs& g, int bn) { return ((g.M + 255) / 256) * ((g.N + bn - 1) / bn); }
+
 // g1 == nullptr: one problem
-cudaError_t launch_pair(const GemmArgs& g0, const void* a0, const void* b0, const GemmArgs* g1, const void* a1,
-                        const void* b1, int num_sms, cudaStream_t s) {
+template <bool MX, bool ROWS, int BN>
+cudaError_t launch_pair_t(const GemmArgs& g0, const void* a0, const void* b0, const GemmArgs* g1, const void* a1,
+                          const void* b1, int num_sms, cudaStream_t s) {
+  auto kern = pair::gemm_pair_kernel<MX, ROWS, BN>;
+  constexpr int smem = pair::Cfg<BN>::kSmemBytes;
   CUtensorMap m[6];
-  if (!make_pair_maps(g0, a0, b0, &m[0], &m[1], &m[2])) return cudaErrorInvalidValue;
+  if (!make_pair_maps(g0, a0, b0, BN, &m[0], &m[1], &m[2])) return cudaErrorInvalidValue;
   if (g1) {
-    if (!make_pair_maps(*g1, a1, b1, &m[3], &m[4], &m[5])) return cudaErrorInvalidValue;
+    if (!make_pair_maps(*g1, a1, b1, BN, &m[3], &m[4], &m[5])) return cudaErrorInvalidValue;
   } else {
     m[3] = m[0]; m[4] = m[1]; m[5] = m[2];
   }
-  if (g1 && g1->mx != g0.mx) return cudaErrorInvalidValue;
   static std::atomic<uint64_t> configured{0};  // per call site (template instantiation) and device
   int dev;
   if (device_needs_config(configured, &dev)) {
-    cudaError_t e = cudaFuncSetAttribute(pair::gemm_pair_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         pair::kSmemBytes);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(pair::gemm_pair_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             pair::kSmemBytes);
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
     device_configured(configured, dev);
   }
   pair::Args a{};
   a.p[0] = pair_problem(g0);
   a.p[1] = pair_problem(g1 ? *g1 : g0);
-  a.n_tiles0 = (g0.M / 256) * (g0.N / 256);
-  a.n_tiles = a.n_tiles0 + (g1 ? (g1->M / 256) * (g1->N / 256) : 0);
+  a.n_tiles0 = pair_tiles(g0, BN);
+  a.n_tiles = a.n_tiles0 + (g1 ? pair_tiles(*g1, BN) : 0);
   int max_pairs = num_sms / 2;
   const int cap = g_exp_max_pairs.load(std::memory_order_relaxed);  // measurement aids, 0 / NULL normally
   if (cap > 0 && cap < max_pairs) max_pairs = cap;
   a.exp = g_exp_mode.load(std::memory_order_relaxed);
   a.probe = g_exp_probe.load(std::memory_order_relaxed);
   const int pairs = a.n_tiles < max_pairs ? a.n_tiles : max_pairs;
-  const bool rows = a.p[0].a_rows || a.p[0].b_rows || a.p[1].a_rows || a.p[1].b_rows;
-  if (rows) {
-    if (g0.mx) return cudaErrorInvalidValue;
-    static std::atomic<uint64_t> configured_rows{0};
-    if (device_needs_config(configured_rows, &dev)) {
-      cudaError_t e = cudaFuncSetAttribute(pair::gemm_pair_kernel<false, true>,
-                                           cudaFuncAttributeMaxDynamicSharedMemorySize, pair::kSmemBytes);
-      if (e != cudaSuccess) return e;
-      device_configured(configured_rows, dev);
-    }
-  }
-  const dim3 grid(2 * pairs), block(pair::kThreads);
-  cudaError_t le;
-  if (rows)
-    le = launch_kernel(pair::gemm_pair_kernel<false, true>, grid, block, pair::kSmemBytes, s, m[0], m[1], m[2],
-                       m[3], m[4], m[5], a);
-  else if (g0.mx)
-    le = launch_kernel(pair::gemm_pair_kernel<true>, grid, block, pair::kSmemBytes, s, m[0], m[1], m[2], m[3],
-                       m[4], m[5], a);
-  else
-    le = launch_kernel(pair::gemm_pair_kernel<false>, grid, block, pair::kSmemBytes, s, m[0], m[1], m[2], m[3],
-                       m[4], m[5], a);
+  const cudaError_t e =
+      launch_kernel(kern, dim3(2 * pairs), dim3(pair::kThreads), smem, s, m[0], m[1], m[2], m[3], m[4], m[5], a);
   count_launch();
-  return le;
+  return e;
+}
+
+cudaError_t launch_pair(const GemmArgs& g0, const void* a0, const void* b0, const GemmArgs* g1, const void* a1,
+                        const void* b1, int bn, int num_sms, cudaStream_t s) {
+  if (g1 && g1->mx != g0.mx) return cudaErrorInvalidValue;
+  if (g0.a_rows || g0.b_rows || (g1 && (g1->a_rows || g1->b_rows))) {
+    if (g0.mx) return cudaErrorInvalidValue;
+    return bn == 128 ? launch_pair_t<false, true, 128>(g0, a0, b0, g1, a1, b1, num_sms, s)
+                     : launch_pair_t<false, true, 256>(g0, a0, b0, g1, a1, b1, num_sms, s);
+  }
+  if (bn == 128)
+    return g0.mx ? launch_pair_t<true, false, 128>(g0, a0, b0, g1, a1, b1, num_sms, s)
+                 : launch_pair_t<false, false, 128>(g0, a0, b0, g1, a1, b1, num_sms, s);
+  return g0.mx ? launch_pair_t<true, false, 256>(g0, a0, b0, g1, a1, b1, num_sms, s)
+               : launch_pair_t<false, false, 256>(g0, a0, b0, g1, a1, b1, num_sms, s);
 }
 
 // N = 128 q = 384 a + 256 b with b in {0, 1, 2}: a wide column tiles, b narrow ones (q >= 2)
@@ -462,7 +458,7 @@ bool wide_split(int N, int* n_wide, int* n_narrow) {
 
 bool wide_eligible(const GemmArgs& g) {
   int a, b;
-  return g.M % 256 == 0 && g.K % 256 == 0 && wide_split(g.N, &a, &b);
+  return !g.a_rows && !g.b_rows && wide_split(g.N, &a, &b);
 }
 
 wide::WProblem wide_problem(const GemmArgs& g) {
@@ -485,27 +481,30 @@ bool make_wide_maps(const GemmArgs& g, const void* a_codes, const void* b_codes,
   return ok;
 }
 
-// Estimated makespan (in units of one 256-deep k-block of a 256 x 256 tile) of the static round-robin schedule
-// the pair kernels use, for one or two problems: round r hands tiles r * pairs .. to the pairs in order, odd rounds
-// in reverse order.  A tile
-// costs its k-blocks times its width factor plus the accumulator hand-over.
-double pair_makespan(const GemmArgs* const* gs, int n_problems, bool wide_tiles, int pairs) {
+// Estimated time (microseconds, without the launch) of the static round-robin schedule the pair kernels use, for one or
+// two problems: round r hands tiles r * pairs .. to the pairs in order, odd rounds in reverse order.  A tile costs its
+// k-blocks plus the accumulator hand-over, and no less than its output takes to store.  The constants are a fit to 90
+// shapes drawn over M 128 .. 16384, N 256 .. 20480, K 512 .. 20480, both output types, timed with all three tiles (rms
+// error 5 %); choosing by them loses 0.1 % on average against the best tile of each shape, always 256 x 256 loses 17 %.
+double pair_makespan(const GemmArgs* const* gs, int n_problems, int tile, int pairs) {
   std::vector<double> load((size_t)pairs, 0.0);
   constexpr int kGroupM = 8;
   int64_t t = 0;
   for (int pi = 0; pi < n_problems; ++pi) {
     const GemmArgs& g = *gs[pi];
-    int n_wide = 0, n_narrow = g.N / 256;
-    if (wide_tiles) wide_split(g.N, &n_wide, &n_narrow);
-    const int tiles_m = g.M / 256, tiles_n = n_wide + n_narrow;
+    int n_wide = 0, n_narrow = tile == kTilePair128 ? (g.N + 127) / 128 : (g.N + 255) / 256;
+    if (tile == kTileWide) wide_split(g.N, &n_wide, &n_narrow);
+    const int tiles_m = (g.M + 255) / 256, tiles_n = n_wide + n_narrow;
     const double kb = g.K / 256.0;
+    const bool f = g.d_is_fp32;
+    const double wide_cost = std::max(0.505 * kb + (f ? 3.56 : 2.03), f ? 4.9 : 0.0);
+    const double narrow_cost = tile == kTilePair128 ? std::max(0.323 * kb + (f ? 0.97 : 0.64), f ? 1.8 : 1.4)
+                               : tile == kTileWide  ? std::max(0.383 * kb + 2.0, f ? 3.3 : 0.0)
+                                                    : std::max(0.383 * kb + (f ? 2.5 : 1.83), f ? 4.9 : 0.0);
     for (int m0 = 0; m0 < tiles_m; m0 += kGroupM) {
       const int gm = tiles_m - m0 < kGroupM ? tiles_m - m0 : kGroupM;
       for (int n_idx = 0; n_idx < tiles_n; ++n_idx) {
-        const bool w = n_idx < n_wide;
-        // hand-over per tile in k-block units, fitted to 24 layer shapes timed with both tile widths (the fp32 figure
-        // of the wide tile refitted after its store chunks stopped waiting for each other)
-        const double cost = w ? 1.5 * kb + (g.d_is_fp32 ? 3.8 : 3.3) : kb + (wide_tiles ? 2.9 : 2.5);
+        const double cost = n_idx < n_wide ? wide_cost : narrow_cost;
         for (int i = 0; i < gm; ++i, ++t) {
           const int64_t rnd = t / pairs, p = t % pairs;
           load[(size_t)((rnd & 1) ? pairs - 1 - p : p)] += cost;  // odd rounds run through the pairs in reverse
@@ -515,8 +514,7 @@ double pair_makespan(const GemmArgs* const* gs, int n_problems, bool wide_tiles,
   }
   double worst = 0.0;
   for (double v : load) worst = v > worst ? v : worst;
-  // the wide tiles move 17 % fewer operand bytes per flop; under the power cap that showed as ~3 % more clock
-  return wide_tiles ? worst * 0.97 : worst;
+  return worst;
 }
 
 // g1 == nullptr: one problem
@@ -544,8 +542,8 @@ cudaError_t launch_wide(const GemmArgs& g0, const void* a0, const void* b0, cons
   wide::WArgs a{};
   a.p[0] = wide_problem(g0);
   a.p[1] = wide_problem(g1 ? *g1 : g0);
-  a.n_tiles0 = (g0.M / 256) * a.p[0].tiles_n;
-  a.n_tiles = a.n_tiles0 + (g1 ? (g1->M / 256) * a.p[1].tiles_n : 0);
+  a.n_tiles0 = ((g0.M + 255) / 256) * a.p[0].tiles_n;
+  a.n_tiles = a.n_tiles0 + (g1 ? ((g1->M + 255) / 256) * a.p[1].tiles_n : 0);
   const int max_pairs = num_sms / 2;
   const int pairs = a.n_tiles < max_pairs ? a.n_tiles : max_pairs;
   const dim3 grid(2 * pairs), block(wide::kWThreads);
@@ -575,60 +573,65 @@ cudaError_t sm_count(int* n) {
 
 }  // namespace
 
-cudaError_t launch_gemm(const GemmArgs& g, const void* a_codes, const void* b_codes, int tile_n, cudaStream_t s) {
+cudaError_t launch_gemm(const GemmArgs& g, const void* a_codes, const void* b_codes, int tile, cudaStream_t s) {
   int num_sms = 0;
   cudaError_t e = sm_count(&num_sms);
   if (e != cudaSuccess) return e;
-  if (g.a_rows || g.b_rows) {  // scale vectors are applied by the 256 x 256 pair kernel's epilogue only
-    if (g.M % 256 != 0 || g.N % 256 != 0) return cudaErrorInvalidValue;
-    return launch_pair(g, a_codes, b_codes, nullptr, nullptr, nullptr, num_sms, s);
-  }
-  if (tile_n == 768 && wide_eligible(g)) return launch_wide(g, a_codes, b_codes, nullptr, nullptr, nullptr, num_sms, s);
-  if ((tile_n == 512 || tile_n == 768) && g.M % 256 == 0 && g.N % 256 == 0)
-    return launch_pair(g, a_codes, b_codes, nullptr, nullptr, nullptr, num_sms, s);
-  if (tile_n == 256 && g.N % 256 == 0)
+  const bool rows = g.a_rows || g.b_rows;  // scale vectors: the pair kernel's epilogue only
+  if (tile == kTileWide && wide_eligible(g)) return launch_wide(g, a_codes, b_codes, nullptr, nullptr, nullptr, num_sms, s);
+  if (tile >= kTilePair256 || rows)
+    return launch_pair(g, a_codes, b_codes, nullptr, nullptr, nullptr, tile == kTilePair128 ? 128 : 256, num_sms, s);
+  if (tile == 256 && g.N % 256 == 0)
     return g.mx ? launch_t<256, true>(g, a_codes, b_codes, num_sms, s) : launch_t<256, false>(g, a_codes, b_codes, num_sms, s);
   return g.mx ? launch_t<128, true>(g, a_codes, b_codes, num_sms, s) : launch_t<128, false>(g, a_codes, b_codes, num_sms, s);
 }
 
 cudaError_t launch_gemm_two(const GemmArgs& g0, const void* a0, const void* b0, const GemmArgs& g1, const void* a1,
-                            const void* b1, bool wide_tiles, cudaStream_t s) {
+                            const void* b1, int tile, cudaStream_t s) {
   int num_sms = 0;
   cudaError_t e = sm_count(&num_sms);
   if (e != cudaSuccess) return e;
-  if (wide_tiles && wide_eligible(g0) && wide_eligible(g1)) return launch_wide(g0, a0, b0, &g1, a1, b1, num_sms, s);
-  return launch_pair(g0, a0, b0, &g1, a1, b1, num_sms, s);
+  if (tile == kTileWide && wide_eligible(g0) && wide_eligible(g1)) return launch_wide(g0, a0, b0, &g1, a1, b1, num_sms, s);
+  return launch_pair(g0, a0, b0, &g1, a1, b1, tile == kTilePair128 ? 128 : 256, num_sms, s);
 }
 
-bool prefer_wide_tiles(const GemmArgs& g0, const GemmArgs* g1) {
-  if (!wide_eligible(g0) || (g1 && !wide_eligible(*g1))) return false;
-  if (g0.N % 256 != 0 || (g1 && g1->N % 256 != 0)) return true;  // only the wide kernel takes N = 128 (2k + 1)
+int best_pair_tile(const GemmArgs& g0, const GemmArgs* g1) {
   int num_sms = 0;
-  if (sm_count(&num_sms) != cudaSuccess) return false;
-  // the estimate walks every tile of both schedules: remember the answers for the shapes seen (a training loop
+  if (sm_count(&num_sms) != cudaSuccess) return kTilePair256;
+  const bool wide_fits = wide_eligible(g0) && (!g1 || wide_eligible(*g1));
+  // the estimate walks every tile of the schedules: remember the answers for the shapes seen (a training loop
   // repeats a handful of them)
-  struct Entry { int key[8]; bool wide; };
+  struct Entry { int key[8]; int tile; };
   static std::mutex mu;
   static std::vector<Entry> seen;
   // (the output type is part of the key: an fp32 output changes the hand-over cost and with it the choice)
   const int key[8] = {g0.M, g0.N, g0.K, g1 ? g1->M : 0, g1 ? g1->N : 0, g1 ? g1->K : 0, num_sms,
-                      (g0.d_is_fp32 ? 1 : 0) | (g1 && g1->d_is_fp32 ? 2 : 0)};
+                      (g0.d_is_fp32 ? 1 : 0) | (g1 && g1->d_is_fp32 ? 2 : 0) | (wide_fits ? 4 : 0)};
   {
     std::lock_guard<std::mutex> lock(mu);
     for (const Entry& e : seen)
-      if (std::equal(key, key + 8, e.key)) return e.wide;
+      if (std::equal(key, key + 8, e.key)) return e.tile;
   }
   const GemmArgs* gs[2] = {&g0, g1};
   const int n = g1 ? 2 : 1, pairs = num_sms / 2;
-  const bool wide = pair_makespan(gs, n, true, pairs) < pair_makespan(gs, n, false, pairs);
+  int best = kTilePair256;
+  double least = pair_makespan(gs, n, kTilePair256, pairs);
+  for (int tile : {kTilePair128, kTileWide}) {
+    if (tile == kTileWide && !wide_fits) continue;
+    const double v = pair_makespan(gs, n, tile, pairs);
+    if (v < least) {
+      least = v;
+      best = tile;
+    }
+  }
   std::lock_guard<std::mutex> lock(mu);
   if (seen.size() < 256) {
     Entry e{};
     std::copy(key, key + 8, e.key);
-    e.wide = wide;
+    e.tile = best;
     seen.push_back(e);
   }
-  return wide;
+  return best;
 }
 
 cudaError_t launch_gemm_bf16(const DenseGemmArgs& g, cudaStream_t s) {
@@ -643,7 +646,7 @@ cudaError_t launch_gemm_bf16(const DenseGemmArgs& g, cudaStream_t s) {
                      : make_map_2d(&map_b, bf, 2, g.b, (uint64_t)g.K, (uint64_t)g.N, (uint64_t)g.ldb * 2, 64, 128, true));
   if (g.d_is_fp32)
     ok = ok && make_map_2d(&map_d, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, g.d, (uint64_t)g.N, (uint64_t)g.M,
-                           (uint64_t)g.ldd * 4, 32, 128, true);
+                           (uint64_t)g.ldd * 4, 16, 128, 2);
   else
     ok = ok && make_map_2d(&map_d, bf, 2, g.d, (uint64_t)g.N, (uint64_t)g.M, (uint64_t)g.ldd * 2, 64, 128, true);
   if (!ok) return cudaErrorInvalidValue;

@@ -19,16 +19,18 @@ struct GemmArgs {
   const float* b_rows;    // (CTA-pair kernel with 256 x 256 tiles only)
 };
 
-// tile_n: 128 or 256 (one CTA per tile; 256 needs N % 256 == 0, otherwise 128 is used), 512 (CTA pairs, 256 x 256
-// tiles; M, N % 256 == 0) or 768 (CTA pairs, 256 x 384 tiles; M % 256 == 0, N % 128 == 0, N >= 256)
-cudaError_t launch_gemm(const GemmArgs& g, const void* a_codes, const void* b_codes, int tile_n, cudaStream_t s);
-// Two independent GEMMs in one launch of the CTA-pair kernel (all of M, N multiples of 256, K of 256): the tiles of
-// g0 are worked through first, then those of g1, on one persistent grid.
-// wide_tiles: 256 x 384 tiles (gemm_wide.cuh) when both shapes allow, else 256 x 256.
+// Tiles: 128 or 256 = one CTA per 128 x 128 / 128 x 256 tile (256 needs N % 256 == 0, otherwise 128 is used); the others
+// run on CTA pairs and take any M and N that are multiples of 128 (a half beyond the edge is computed on zeros and clipped).
+constexpr int kTilePair256 = 512;  // 256 x 256
+constexpr int kTilePair128 = 640;  // 256 x 128
+constexpr int kTileWide = 768;     // 256 x 384, needs N >= 256 and tensor-level scales
+cudaError_t launch_gemm(const GemmArgs& g, const void* a_codes, const void* b_codes, int tile, cudaStream_t s);
+// Two independent GEMMs in one launch of a CTA-pair kernel: the tiles of g0 are worked through first, then those of g1,
+// on one persistent grid.
 cudaError_t launch_gemm_two(const GemmArgs& g0, const void* a0, const void* b0, const GemmArgs& g1, const void* a1,
-                            const void* b1, bool wide_tiles, cudaStream_t s);
-// Scheduling estimate: do 256 x 384 tiles beat 256 x 256 tiles for this problem (or pair of problems in one launch)?
-bool prefer_wide_tiles(const GemmArgs& g0, const GemmArgs* g1);
+                            const void* b1, int tile, cudaStream_t s);
+// Scheduling estimate: the CTA-pair tile for this problem (or pair of problems in one launch)
+int best_pair_tile(const GemmArgs& g0, const GemmArgs* g1);
 // Measurement aids of the CTA-pair kernel with 256 x 256 tiles (0, 0, NULL = normal operation): mode bit 0 = no MMAs,
 // bit 1 = no operand loads, bit 2 = no scale loads / copies, bit 3 = accumulator handed back unread and nothing
 // stored, bit 4 = the issuer does not wait for the accumulator (results meaningless with any bit set); max_pairs caps the

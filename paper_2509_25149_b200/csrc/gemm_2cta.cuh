@@ -1,6 +1,7 @@
 // Block-scaled NVFP4 GEMM on CTA pairs (tcgen05 cta_group::2): a cluster of two CTAs on one TPC computes a
-// 256 x 256 output tile.  Each CTA keeps its own 128 rows of A, HALF of the B tile (128 of its 256 rows) and the
-// accumulator of its 128 output rows in its own tensor memory; the pair's tensor cores exchange the B halves, so
+// 256 x 256 output tile (or 256 x 128: twice the tiles for shapes that leave pairs idle, and with the tensor memory
+// that frees a second accumulator).  Each CTA keeps its own 128 rows of A, HALF of the B tile (128 of its 256 rows) and
+// the accumulator of its 128 output rows in its own tensor memory; the pair's tensor cores exchange the B halves, so
 // every byte of B is fetched from L2 and read from shared memory once per pair.  That halving of the operand
 // traffic per flop is the point: the one-CTA kernel is bound by shared-memory bandwidth, not by the tensor pipe.
 //
@@ -9,6 +10,9 @@
 // registers -> tensor memory, one warp per 32-lane quadrant), 3-10 epilogue (both; two groups of four warps, one per
 // 128-column half: tensor memory -> registers -> swizzled staging -> TMA store; the accumulator is released as
 // soon as it has been read).
+// M and N may be odd multiples of 128: the half of the last tile beyond the edge reads zero codes (tensor map) and its
+// output is clipped.  Half a tile of padding costs less than the one-CTA kernel that used to take these shapes:
+// 4224 x 5248 x 5120 85 -> 60 us, 2048 x 7040 x 512 (odd N) 23 -> 11 us.
 // Included by gemm.cu only.
 #pragma once
 
@@ -21,20 +25,27 @@ namespace nvfp4 {
 namespace pair {
 
 constexpr int kThreads = 448;      // producer, MMA, 2 x 4 epilogue warps, 4 scale warps (2, 11, 12, 13)
-constexpr int kStages = 5;
 constexpr int kABytes = 128 * 128;   // 128 rows x 256 K elements
-constexpr int kBBytes = 128 * 128;   // this CTA's half of the 256-row B tile
 constexpr int kSfaBytes = 4 * 512;   // own 128 rows, four K64 steps
-constexpr int kSfbBytes = 8 * 512;   // all 256 rows of B (both CTAs need them), four K64 steps
-constexpr int kStageBytes = kABytes + kBBytes + kSfaBytes + kSfbBytes;  // 38 KB
 constexpr int kStagingBytes = 2 * 16384;  // one 128 x 128-byte store buffer per epilogue group
 constexpr int kBetaBytes = 2 * 128 * 4;   // column scales of the tile, one half per epilogue group (row-scaled B)
-constexpr int kSmemBytes = kStages * kStageBytes + kStagingBytes + 1024 /*alignment*/ + 256 /*barriers*/ + kBetaBytes;
 constexpr uint32_t kTmemCols = 512;
-constexpr int kSfCol = 256;          // after the 256 accumulator columns: one 48-column slot per stage
-constexpr int kSfSlotCols = 48;      // SFA 4 x 4, SFB 4 x 8
-static_assert(kSfCol + kStages * kSfSlotCols <= 512, "tensor memory budget");
-static_assert(kStageBytes % 1024 == 0, "stages must keep the 1024-byte swizzle alignment");
+template <int BN>
+struct Cfg {
+  static constexpr int kGroups = BN / 128;              // 128-row groups of B = scale atoms per K64 step
+  static constexpr int kStages = BN == 256 ? 5 : 6;
+  static constexpr int kAcc = BN == 256 ? 1 : 2;        // accumulators in tensor memory
+  static constexpr int kBBytes = BN / 2 * 128;          // this CTA's half of the B tile
+  static constexpr int kSfbBytes = 4 * kGroups * 512;   // all rows of B (both CTAs need them), four K64 steps
+  static constexpr int kStageBytes = kABytes + kBBytes + kSfaBytes + kSfbBytes;  // 38 / 28 KB
+  static constexpr int kSmemBytes =
+      kStages * kStageBytes + kStagingBytes + 1024 /*alignment*/ + 256 /*barriers*/ + kBetaBytes;
+  static constexpr int kSfCol = 256;                    // after the accumulator columns: one slot per stage
+  static constexpr int kSfSlotCols = 16 + 16 * kGroups; // SFA 4 x 4, SFB 4 x 4 per group
+  static_assert(kSfCol + kStages * kSfSlotCols <= 512, "tensor memory budget");
+  static_assert(kStageBytes % 1024 == 0, "stages must keep the 1024-byte swizzle alignment");
+  static_assert(kSmemBytes <= 232448, "shared memory budget");
+};
 
 struct Problem {
   int M, N, K;
@@ -164,6 +175,11 @@ __device__ __forceinline__ void tc_st16(uint32_t taddr, const uint32_t* r) {
       "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
       : "memory");
 }
+__device__ __forceinline__ void tc_st8(uint32_t taddr, const uint32_t* r) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"r"(taddr), "r"(r[0]), "r"(r[1]),
+               "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
+               : "memory");
+}
 __device__ __forceinline__ void tc_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ uint4 lds128(uint32_t addr) {
   uint4 v;
@@ -195,30 +211,43 @@ __device__ __forceinline__ void tc2_mma_mxf4(uint32_t d_tmem, uint64_t adesc, ui
       : "memory");
 }
 
-// Epilogue helper: 128 accumulator columns of one row per thread (registers) -> alpha, conversion -> 128-byte
-// swizzled rows of the group's staging buffer -> TMA store (or reduce-add) of 128 x 128-byte boxes.  A group has
-// ONE 16 KB buffer: a chunk is converted only after the store of the previous chunk has finished reading it.
-// BETA: the 128 columns additionally carry their own factors (float[128] in shared memory at `beta`).
-template <bool FP32, bool BETA = false>
-__device__ __forceinline__ void store_half(const uint32_t (&r)[128], float alpha, int et, int bar_id, int row_in_tile,
-                                           uint32_t stage_buf, const CUtensorMap* map_d, int x0, int row0,
-                                           int accumulate, const float* beta = nullptr, int skip = 0) {
+// Epilogue helper: COLS accumulator columns of one row per thread (registers) -> alpha, conversion -> swizzled rows of
+// the group's 16 KB staging buffer -> TMA store (or reduce-add).
+// bf16: chunks of 64 columns (128-byte rows) through the whole buffer, each converted once the store before it has
+// finished reading.  fp32: chunks of 16 columns (64-byte rows) through the two 8 KB halves in turn, so that a chunk waits
+// only for the store of two chunks before it; with 32-column chunks through the whole buffer the stores were a serial
+// chain that bounded tiles of few k-blocks.  (An even number of fp32 chunks: a tile starts with the first half, and only a
+// store of the other kind from the tile before, `drain`, can reach into it.)
+// BETA: the columns additionally carry their own factors (float[COLS] in shared memory at `beta`).
+template <bool FP32, bool BETA = false, int COLS = 128>
+__device__ __forceinline__ void store_half(const uint32_t (&r)[COLS], float alpha, int et, int bar_id, int row_in_tile,
+                                           uint32_t stage_buf16k, const CUtensorMap* map_d, int x0, int row0,
+                                           int accumulate, bool drain, const float* beta = nullptr, int skip = 0) {
   // skip (measurement aid): bit 0 = the converted values are not written to the staging buffer, bit 1 = no TMA store
-  constexpr int kChunks = FP32 ? 4 : 2;
-  constexpr int kChunkCols = FP32 ? 32 : 64;
+  constexpr int kChunkCols = FP32 ? 16 : 64, kUnits = FP32 ? 4 : 8;  // 16-byte units of a staged row
+  constexpr int kChunks = COLS / kChunkCols;
+  static_assert(!FP32 || kChunks % 2 == 0, "a tile starts with the first half of the buffer");
 #pragma unroll
   for (int c = 0; c < kChunks; ++c) {
-    if (et == 0) bulk_wait_read<0>();
+    const uint32_t stage_buf = stage_buf16k + (FP32 ? (c & 1) * 8192 : 0);
+    if (et == 0) {
+      if (!FP32 || (c == 0 && drain))
+        bulk_wait_read<0>();
+      else
+        bulk_wait_read<1>();
+    }
     asm volatile("bar.sync %0, 128;" ::"r"(bar_id) : "memory");
-    const uint32_t srow = stage_buf + row_in_tile * 128;
+    const uint32_t srow = stage_buf + row_in_tile * (16 * kUnits);
+    // 128-byte swizzle: unit index XOR address bits 7-9 = row & 7; 64-byte swizzle: XOR bits 7-8 = (row >> 1) & 3
+    const uint32_t x = FP32 ? (row_in_tile >> 1) & 3 : row_in_tile & 7;
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
+    for (int j = 0; j < kUnits; ++j) {
       uint32_t p[4];
       if (FP32) {
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-          float v = __uint_as_float(r[c * 32 + 4 * j + e]) * alpha;
-          if (BETA) v *= beta[c * 32 + 4 * j + e];
+          float v = __uint_as_float(r[c * 16 + 4 * j + e]) * alpha;
+          if (BETA) v *= beta[c * 16 + 4 * j + e];
           p[e] = __float_as_uint(v);
         }
       } else {
@@ -235,8 +264,8 @@ __device__ __forceinline__ void store_half(const uint32_t (&r)[128], float alpha
         }
       }
       if (!(skip & 1) || (p[0] ^ p[1] ^ p[2] ^ p[3]) == 0x9E3779B9u)  // (the aid keeps the conversion alive)
-        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(srow + ((j ^ (row_in_tile & 7)) << 4)), "r"(p[0]),
-                     "r"(p[1]), "r"(p[2]), "r"(p[3])
+        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(srow + ((j ^ x) << 4)), "r"(p[0]), "r"(p[1]),
+                     "r"(p[2]), "r"(p[3])
                      : "memory");
     }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -257,12 +286,16 @@ __device__ __forceinline__ void store_half(const uint32_t (&r)[128], float alpha
 // ROWS = true: at least one operand carries its global scale per row (a_rows / b_rows); the epilogue then applies a
 // factor per output row and / or per output column.  A separate instantiation so that the common kernel keeps its
 // register budget.
-template <bool MX, bool ROWS = false>
+// BN: columns of a tile (256 or 128).
+template <bool MX, bool ROWS = false, int BN = 256>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant__ CUtensorMap map_b0,
                      const __grid_constant__ CUtensorMap map_d0, const __grid_constant__ CUtensorMap map_a1,
                      const __grid_constant__ CUtensorMap map_b1, const __grid_constant__ CUtensorMap map_d1,
                      const __grid_constant__ Args g) {
+  using C = Cfg<BN>;
+  constexpr int kStages = C::kStages, kStageBytes = C::kStageBytes, kBBytes = C::kBBytes, kGroups = C::kGroups;
+  constexpr int kSfCol = C::kSfCol, kSfSlotCols = C::kSfSlotCols;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t* base_ptr = smem_raw + (base - smem_u32(smem_raw));
@@ -272,11 +305,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   auto sff_bar = [&](int s) { return bar_base + 8u * (kStages + s); };       // leader only: scales of both CTAs in TMEM
   auto empty_bar = [&](int s) { return bar_base + 8u * (2 * kStages + s); }; // one per CTA
   auto sfl_bar = [&](int s) { return bar_base + 8u * (3 * kStages + s); };   // one per CTA: own scale atoms landed
-  const uint32_t accf_bar = bar_base + 8u * (4 * kStages);                   // one per CTA
-  const uint32_t acce_bar = bar_base + 8u * (4 * kStages + 1);               // leader only, 16 arrivals
-  const uint32_t done_bar = bar_base + 8u * (4 * kStages + 2);               // one per CTA, peer arrives
-  volatile uint32_t* tmem_slot =
-      reinterpret_cast<volatile uint32_t*>(base_ptr + kStages * kStageBytes + kStagingBytes + 8 * (4 * kStages + 3));
+  auto accf_bar = [&](int b) { return bar_base + 8u * (4 * kStages + b); };             // per accumulator, one per CTA
+  auto acce_bar = [&](int b) { return bar_base + 8u * (4 * kStages + C::kAcc + b); };   // leader only, 16 arrivals
+  const uint32_t done_bar = bar_base + 8u * (4 * kStages + 2 * C::kAcc);                // one per CTA, peer arrives
+  volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(base_ptr + kStages * kStageBytes + kStagingBytes +
+                                                                      8 * (4 * kStages + 2 * C::kAcc + 1));
   volatile uint32_t* abort_flag = tmem_slot + 1;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -290,7 +323,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   auto tile_coords = [&](int tile, int& prob, int& m_blk, int& n_blk) {
     prob = tile >= g.n_tiles0 ? 1 : 0;
     if (prob) tile -= g.n_tiles0;
-    const int tiles_m = g.p[prob].M / 256, tiles_n = g.p[prob].N / 256;
+    const int tiles_m = (g.p[prob].M + 255) / 256, tiles_n = (g.p[prob].N + BN - 1) / BN;
     const int per_group = kGroupM * tiles_n;
     const int grp = tile / per_group, in_grp = tile - grp * per_group;
     const int m0 = grp * kGroupM;
@@ -311,8 +344,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       mbar_init(empty_bar(s), 1);
       mbar_init(sfl_bar(s), 1);
     }
-    mbar_init(accf_bar, 1);
-    mbar_init(acce_bar, 16);       // eight epilogue warps in each CTA
+    for (int b = 0; b < C::kAcc; ++b) {
+      mbar_init(accf_bar(b), 1);
+      mbar_init(acce_bar(b), 16);  // eight epilogue warps in each CTA
+    }
     mbar_init(done_bar, 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -350,9 +385,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         const int sf_atoms_k = pr.K / (MX ? 128 : 64);  // atoms along K per 128-row group
         constexpr int kAtomsKb = MX ? 2 : 4;              // atoms per 256-deep k-block and 128-row group
         const int row_a = m_blk * 256 + (int)rank * 128;       // this CTA's A rows
-        const int row_b = n_blk * 256 + (int)rank * 128;       // this CTA's half of the B tile
-        const uint8_t* sfa = pr.sfa + (int64_t)(m_blk * 2 + (int)rank) * sf_atoms_k * 512;  // own 128 rows
-        const uint8_t* sfb = pr.sfb + (int64_t)(n_blk * 2) * sf_atoms_k * 512;               // all 256 rows of B
+        const int row_b = n_blk * BN + (int)rank * (BN / 2);   // this CTA's half of the B tile
+        // Scale atoms: own 128 rows, all BN rows of B.  M or N may be an odd multiple of 128: the codes of the half
+        // beyond the edge are zero-filled by the tensor map, and its scales (any valid ones do) are those of the last
+        // group inside; its outputs are clipped.
+        const int grp_a = min(m_blk * 2 + (int)rank, pr.M / 128 - 1), last_b = pr.N / 128 - 1;
+        const uint8_t* sfa = pr.sfa + (int64_t)grp_a * sf_atoms_k * 512;
+        const uint8_t* sfb0 = pr.sfb + (int64_t)min(n_blk * kGroups, last_b) * sf_atoms_k * 512;
+        const uint8_t* sfb1 = pr.sfb + (int64_t)min(n_blk * kGroups + 1, last_b) * sf_atoms_k * 512;
         for (int kb = 0; kb < k_blocks; ++kb) {
           if (!(ok = mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag, 0x100u + stage))) break;
           const uint32_t st = base + stage * kStageBytes;
@@ -368,12 +408,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
           if (g.exp & 4) {
             mbar_expect_tx(sfl_bar(stage), 0);  // measurement aid: no scale loads
           } else {
-            mbar_expect_tx(sfl_bar(stage), 3 * kAtomsKb * 512);
+            mbar_expect_tx(sfl_bar(stage), (1 + kGroups) * kAtomsKb * 512);
             bulk_load(st + kABytes + kBBytes, sfa + (int64_t)kb * kAtomsKb * 512, kAtomsKb * 512, sfl_bar(stage));
-            bulk_load(st + kABytes + kBBytes + kSfaBytes, sfb + (int64_t)kb * kAtomsKb * 512, kAtomsKb * 512,
+            bulk_load(st + kABytes + kBBytes + kSfaBytes, sfb0 + (int64_t)kb * kAtomsKb * 512, kAtomsKb * 512,
                       sfl_bar(stage));
-            bulk_load(st + kABytes + kBBytes + kSfaBytes + 2048, sfb + ((int64_t)sf_atoms_k + kb * kAtomsKb) * 512,
-                      kAtomsKb * 512, sfl_bar(stage));
+            if (kGroups == 2)
+              bulk_load(st + kABytes + kBBytes + kSfaBytes + 2048, sfb1 + (int64_t)kb * kAtomsKb * 512, kAtomsKb * 512,
+                        sfl_bar(stage));
           }
           if (++stage == kStages) {
             stage = 0;
@@ -386,7 +427,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     // ------------------------------- scale atoms: shared memory -> registers -> tensor memory (both CTAs) ----
     // One warp per 32-lane quadrant of tensor memory (warps 2, 11, 12, 13 -> quadrants 2, 3, 0, 1).  Lane l of
     // every quadrant holds row l of each 512-byte atom: columns [4j, 4j+4) of the stage's slot for SFA of K64-step
-    // j, columns [16 + 8j + 4g, ..) for SFB of step j and 128-row group g.  The tensor-memory copy engine
+    // j, columns [16 + 4 * groups * j + 4g, ..) for SFB of step j and 128-row group g.  The tensor-memory copy engine
     // (tcgen05.cp) moves one atom per instruction and was the bottleneck of the main loop; twelve 16-byte loads
     // and three tcgen05.st per warp do the same work off the critical path.
     const int quad = warp & 3;
@@ -410,7 +451,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
           continue;
         }
         const uint32_t sf_s = base + stage * kStageBytes + kABytes + kBBytes + lane * 16;
-        uint32_t r[48];
+        uint32_t r[kSfSlotCols];
         constexpr int kAtomsKb = MX ? 2 : 4;  // atoms per k-block and 128-row group
 #pragma unroll
         for (int j = 0; j < kAtomsKb; ++j) {
@@ -421,20 +462,21 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 #pragma unroll
         for (int j = 0; j < kAtomsKb; ++j)
 #pragma unroll
-          for (int grp = 0; grp < 2; ++grp) {
+          for (int grp = 0; grp < kGroups; ++grp) {
             const uint4 b = lds128(sf_s + kSfaBytes + grp * 2048 + j * 512);
-            r[16 + 8 * j + 4 * grp] = b.x; r[16 + 8 * j + 4 * grp + 1] = b.y;
-            r[16 + 8 * j + 4 * grp + 2] = b.z; r[16 + 8 * j + 4 * grp + 3] = b.w;
+            const int c = 16 + 4 * kGroups * j + 4 * grp;
+            r[c] = b.x; r[c + 1] = b.y; r[c + 2] = b.z; r[c + 3] = b.w;
           }
         if (MX) {
-          asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"r"(sf_t), "r"(r[0]),
-                       "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
-                       : "memory");
-          tc_st16(sf_t + 16, &r[16]);
+          tc_st8(sf_t, &r[0]);
+          if (kGroups == 2)
+            tc_st16(sf_t + 16, &r[16]);
+          else
+            tc_st8(sf_t + 16, &r[16]);
         } else {
           tc_st16(sf_t, &r[0]);
           tc_st16(sf_t + 16, &r[16]);
-          tc_st16(sf_t + 32, &r[32]);
+          if (kGroups == 2) tc_st16(sf_t + 32, &r[32]);
         }
         tc_wait_st();
         tc_fence_before();
@@ -451,10 +493,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     // ---------------------------------------------------------------- MMA issuer (leader) ----
     if (leader && lane == 0) {
       int stage = 0;
-      uint32_t phase = 0, acc_phase = 0;
+      uint32_t phase = 0, acc_phase = 0;  // bit b: phase of accumulator b's barriers
+      int acc = 0;
       bool ok = true;
-      constexpr uint32_t idesc = instr_desc_nvf4(256, 256);
-      constexpr uint32_t idesc_mx[2] = {instr_desc_mxf4(256, 256, 0), instr_desc_mxf4(256, 256, 2)};
+      constexpr uint32_t idesc = instr_desc_nvf4(256, BN);
+      constexpr uint32_t idesc_mx[2] = {instr_desc_mxf4(256, BN, 0), instr_desc_mxf4(256, BN, 2)};
       const uint32_t a_lo0 = ((base >> 4) & 0x3fffu) | (1u << 16);
       const uint32_t b_lo0 = (((base + kABytes) >> 4) & 0x3fffu) | (1u << 16);
       const long long probe_c0 = g.probe ? clock64() : 0;
@@ -462,9 +505,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       unsigned long long probe_kb = 0, probe_tiles = 0;
       long long probe_wait = 0, probe_mark = probe_c0;  // cycles spent waiting for the accumulator to be handed back
       for (int rnd = 0, tile = pair_id; tile < n_tiles && ok; tile = next_tile(++rnd)) {
-        if (!(g.exp & 16) && !(ok = mbar_wait_cluster(acce_bar, acc_phase ^ 1u, abort_flag, 0x300u))) break;
+        if (!(g.exp & 16) && !(ok = mbar_wait_cluster(acce_bar(acc), ((acc_phase >> acc) & 1u) ^ 1u, abort_flag, 0x300u)))
+          break;
         if (g.probe) probe_wait += clock64() - probe_mark;
         tc_fence_after();
+        const uint32_t d_tmem = tmem + acc * BN;
         const int k_blocks = k_blocks_of(tile);
         for (int kb = 0; kb < k_blocks; ++kb) {
           if (!(ok = mbar_wait_cluster(full_bar(stage), phase, abort_flag, 0x200u + stage))) break;
@@ -480,19 +525,19 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
             for (int j = 0; j < kAtomsKb; ++j) {
               tc2_cp_sf(sf_t + j * 4, make_desc(sf_lo + j * 32, kDescHiSf));
 #pragma unroll
-              for (int grp = 0; grp < 2; ++grp)
-                tc2_cp_sf(sf_t + 16 + 8 * j + 4 * grp, make_desc(sf_lo + (kSfaBytes >> 4) + grp * 128 + j * 32, kDescHiSf));
+              for (int grp = 0; grp < kGroups; ++grp)
+                tc2_cp_sf(sf_t + 16 + 4 * kGroups * j + 4 * grp, make_desc(sf_lo + (kSfaBytes >> 4) + grp * 128 + j * 32, kDescHiSf));
             }
           }
 #pragma unroll
           for (int j = 0; j < 4; ++j) {
             if (g.exp & 1) break;  // measurement aid: no MMAs
             if (MX)  // one atom (4 columns) serves two K = 64 steps: bytes 0-1, then bytes 2-3
-              tc2_mma_mxf4(tmem, make_desc(a_lo + 2 * j, kDescHiOperand), make_desc(b_lo + 2 * j, kDescHiOperand),
-                           idesc_mx[j & 1], sf_t + (j >> 1) * 4, sf_t + 16 + (j >> 1) * 8, (kb > 0 || j > 0) ? 1u : 0u);
+              tc2_mma_mxf4(d_tmem, make_desc(a_lo + 2 * j, kDescHiOperand), make_desc(b_lo + 2 * j, kDescHiOperand),
+                           idesc_mx[j & 1], sf_t + (j >> 1) * 4, sf_t + 16 + (j >> 1) * 4 * kGroups, (kb > 0 || j > 0) ? 1u : 0u);
             else
-              tc2_mma_nvf4(tmem, make_desc(a_lo + 2 * j, kDescHiOperand), make_desc(b_lo + 2 * j, kDescHiOperand), idesc,
-                           sf_t + j * 4, sf_t + 16 + j * 8, (kb > 0 || j > 0) ? 1u : 0u);
+              tc2_mma_nvf4(d_tmem, make_desc(a_lo + 2 * j, kDescHiOperand), make_desc(b_lo + 2 * j, kDescHiOperand), idesc,
+                           sf_t + j * 4, sf_t + 16 + j * 4 * kGroups, (kb > 0 || j > 0) ? 1u : 0u);
           }
           tc2_commit_both(empty_bar(stage), 3);  // both CTAs' stages are free once these MMAs have read them
           if (++stage == kStages) {
@@ -501,8 +546,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
           }
         }
         if (!ok) break;
-        tc2_commit_both(accf_bar, 3);  // accumulators of both CTAs complete
-        acc_phase ^= 1u;
+        tc2_commit_both(accf_bar(acc), 3);  // this accumulator is complete in both CTAs
+        acc_phase ^= 1u << acc;
+        if (++acc == C::kAcc) acc = 0;
         probe_kb += (unsigned long long)k_blocks;
         ++probe_tiles;
         if (g.probe) probe_mark = clock64();
@@ -510,7 +556,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       if (g.probe) {
         // the last commit has been issued, not completed: wait for the accumulator hand-over of the last tile so that
         // the interval covers the work (bounded like every other wait)
-        mbar_wait_cluster(acce_bar, acc_phase ^ 1u, abort_flag, 0x380u);
+        const int last = C::kAcc - 1 - acc;  // (one accumulator: itself; two: the one used last)
+        mbar_wait_cluster(acce_bar(last), ((acc_phase >> last) & 1u) ^ 1u, abort_flag, 0x380u);
         probe_wait += clock64() - probe_mark;
         g.probe[8 * pair_id] = (unsigned long long)(clock64() - probe_c0);
         g.probe[8 * pair_id + 1] = globaltimer_ns() - probe_t0;
@@ -521,71 +568,79 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     }
   } else if (warp >= 3 && warp <= 10) {
     // ------------------------------------------------------------------ epilogue ----
-    // Two groups of four warps; group h drains columns [128h, 128h + 128) of the accumulator through its own
-    // pair of staging buffers, so the two halves leave tensor memory concurrently.
+    // Two groups of four warps; group h drains its half of the accumulator's columns through its own staging buffer, so
+    // the two halves leave tensor memory concurrently.
+    constexpr int kHalf = BN / 2;
     const int quad = warp & 3;              // tensor-memory lanes this warp may read
     const int half = (warp - 3) >> 2;       // column half / epilogue group
     const int et = (threadIdx.x - 96) & 127;  // 0..127 inside the group
     const int bar_id = 1 + half;
     uint32_t acc_phase = 0;
+    int acc = 0, last_prob = 0;
     // per-tensor decode scales; an operand with per-row scales contributes 1 here and its vector below
     const float alpha0 = __fmul_rn((ROWS && g.p[0].a_rows) ? 1.f : g.p[0].a_global[1], (ROWS && g.p[0].b_rows) ? 1.f : g.p[0].b_global[1]);
     const float alpha1 = __fmul_rn((ROWS && g.p[1].a_rows) ? 1.f : g.p[1].a_global[1], (ROWS && g.p[1].b_rows) ? 1.f : g.p[1].b_global[1]);
     float* beta = reinterpret_cast<float*>(base_ptr + kStages * kStageBytes + kStagingBytes + 256) + half * 128;
-    const uint32_t acce_leader = map_to_cta(acce_bar, 0);
+    const uint32_t acce_leader = map_to_cta(acce_bar(0), 0);
     const int row_in_tile = quad * 32 + lane;
-    const uint32_t t_row = tmem + ((uint32_t)(quad * 32) << 16) + half * 128;
+    const uint32_t t_row0 = tmem + ((uint32_t)(quad * 32) << 16) + half * kHalf;
     const uint32_t stage_buf = staging + half * 16384;
+    auto next_acc = [&] {
+      acc_phase ^= 1u << acc;
+      if (++acc == C::kAcc) acc = 0;
+    };
     for (int rnd = 0, tile = pair_id; tile < n_tiles; tile = next_tile(++rnd)) {
       int prob, m_blk, n_blk;
       tile_coords(tile, prob, m_blk, n_blk);
       const CUtensorMap* map_d = prob ? &map_d1 : &map_d0;
       float alpha = prob ? alpha1 : alpha0;
       const int d_is_fp32 = g.p[prob].d_is_fp32, accumulate = g.p[prob].accumulate;
+      const bool drain = prob != last_prob;  // the problems of a launch may have different output types
+      last_prob = prob;
       const float* a_rows = ROWS ? g.p[prob].a_rows : nullptr;
       const float* b_rows = ROWS ? g.p[prob].b_rows : nullptr;
       if (a_rows) alpha *= a_rows[2 * (int64_t)(m_blk * 256 + (int)rank * 128 + quad * 32 + lane) + 1];
       // the group's 128 column factors; the first barrier inside store_half orders this write before their use, its
       // last one orders their use before the next tile's write
-      if (b_rows) beta[et] = b_rows[2 * (int64_t)(n_blk * 256 + half * 128 + et) + 1];
-      mbar_wait_cluster(accf_bar, acc_phase, abort_flag, 0x400u);
+      if (b_rows && et < kHalf) beta[et] = b_rows[2 * (int64_t)(n_blk * BN + half * kHalf + et) + 1];
+      mbar_wait_cluster(accf_bar(acc), (acc_phase >> acc) & 1u, abort_flag, 0x400u);
       // agree on giving up: a warp that timed out still joins this barrier, and all 128 threads take ONE decision
       if (group_gave_up(abort_flag, bar_id, 128)) break;
       tc_fence_after();
       if (g.exp & 8) {  // measurement aid: the accumulator is handed back unread, nothing is stored
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive_cluster(acce_leader);
-        acc_phase ^= 1u;
+        if (lane == 0) mbar_arrive_cluster(acce_leader + 8u * acc);
+        next_acc();
         continue;
       }
       const int row0 = m_blk * 256 + (int)rank * 128;
-      // read this warp's 32 lanes x 128 columns in one go and hand the accumulator back at once: the MMA issuer
+      // read this warp's 32 lanes x BN / 2 columns in one go and hand the accumulator back at once: the MMA issuer
       // can start the next tile while the values are converted and stored from registers
-      uint32_t r[128];
+      const uint32_t t_row = t_row0 + acc * BN;
+      const int x0 = n_blk * BN + half * kHalf;
+      uint32_t r[kHalf];
       // sixteen columns per load: measured per tile 1830 cycles of hand-over with x16 loads against 2400 with x32
       // and 3500 with x64 (wider loads want longer runs of consecutive registers)
 #pragma unroll
-      for (int q = 0; q < 8; ++q) tc_ld16(t_row + q * 16, *reinterpret_cast<uint32_t(*)[16]>(&r[q * 16]));
+      for (int q = 0; q < kHalf / 16; ++q) tc_ld16(t_row + q * 16, *reinterpret_cast<uint32_t(*)[16]>(&r[q * 16]));
       tc_wait_ld();
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive_cluster(acce_leader);
+      if (lane == 0) mbar_arrive_cluster(acce_leader + 8u * acc);
       if (ROWS && b_rows) {
         if (d_is_fp32)
-          store_half<true, true>(r, alpha, et, bar_id, row_in_tile, stage_buf, map_d, n_blk * 256 + half * 128,
-                                 row0, accumulate, beta);
+          store_half<true, true, kHalf>(r, alpha, et, bar_id, row_in_tile, stage_buf, map_d, x0, row0, accumulate, drain, beta);
         else
-          store_half<false, true>(r, alpha, et, bar_id, row_in_tile, stage_buf, map_d, n_blk * 256 + half * 128,
-                                  row0, accumulate, beta);
+          store_half<false, true, kHalf>(r, alpha, et, bar_id, row_in_tile, stage_buf, map_d, x0, row0, accumulate, drain, beta);
       } else if (d_is_fp32) {
-        store_half<true>(r, alpha, et, bar_id, row_in_tile, stage_buf, map_d, n_blk * 256 + half * 128, row0,
-                         accumulate, nullptr, (g.exp >> 6) & 3);
+        store_half<true, false, kHalf>(r, alpha, et, bar_id, row_in_tile, stage_buf, map_d, x0, row0, accumulate, drain,
+                                       nullptr, (g.exp >> 6) & 3);
       } else {
-        store_half<false>(r, alpha, et, bar_id, row_in_tile, stage_buf, map_d, n_blk * 256 + half * 128, row0,
-                          accumulate, nullptr, (g.exp >> 6) & 3);
+        store_half<false, false, kHalf>(r, alpha, et, bar_id, row_in_tile, stage_buf, map_d, x0, row0, accumulate, drain,
+                                        nullptr, (g.exp >> 6) & 3);
       }
-      acc_phase ^= 1u;
+      next_acc();
     }
     if (et == 0) bulk_wait_all<0>();  // all stores have left shared memory and are visible
   }

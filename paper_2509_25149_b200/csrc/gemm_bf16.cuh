@@ -222,10 +222,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       if (lane == 0) mbar_arrive_cluster(map_to_cta(acce_bar(buf), 0));
       if (g.d_is_fp32)
         store_half<true>(r, 1.0f, et, bar_id, row_in_tile, stage_buf, &map_d, n_blk * 256 + half * 128, row0,
-                         g.accumulate);
+                         g.accumulate, false);
       else
         store_half<false>(r, 1.0f, et, bar_id, row_in_tile, stage_buf, &map_d, n_blk * 256 + half * 128, row0,
-                          g.accumulate);
+                          g.accumulate, false);
       acc_phase ^= 1u << buf;
     }
     if (et == 0) bulk_wait_all<0>();  // all stores have left shared memory and are visible

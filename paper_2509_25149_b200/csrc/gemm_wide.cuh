@@ -158,7 +158,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kWThreads, 1)
   auto tile_coords = [&](int tile, int& prob, int& m_blk, int& n0, int& width) {
     prob = tile >= g.n_tiles0 ? 1 : 0;
     if (prob) tile -= g.n_tiles0;
-    const int tiles_m = g.p[prob].M / 256, tiles_n = g.p[prob].tiles_n, n_wide = g.p[prob].n_wide;
+    const int tiles_m = (g.p[prob].M + 255) / 256, tiles_n = g.p[prob].tiles_n, n_wide = g.p[prob].n_wide;
     const int per_group = kGroupM * tiles_n;
     const int grp = tile / per_group, in_grp = tile - grp * per_group;
     const int m0 = grp * kGroupM;
@@ -225,7 +225,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kWThreads, 1)
         const int row_b = n0 + (int)rank * 128;            // its 128 rows of the tile's first 256 columns
         const int row_c = n0 + 256 + (int)rank * 64;       // its 64 rows of the last 128 columns (wide tiles)
         const int groups = width / 128;
-        const uint8_t* sfa = pr.sfa + (int64_t)(m_blk * 2 + (int)rank) * sf_atoms_k * 512;  // own 128 rows
+        // own 128 rows; M may be an odd multiple of 128: the last pair's second half reads zero codes (tensor map) under
+        // the scales of the group before it, and its outputs are clipped
+        const uint8_t* sfa = pr.sfa + (int64_t)min(m_blk * 2 + (int)rank, pr.M / 128 - 1) * sf_atoms_k * 512;
         const uint8_t* sfb = pr.sfb + (int64_t)(n0 / 128) * sf_atoms_k * 512;               // all rows of the B tile
         for (int kb = 0; kb < k_blocks; ++kb) {
           if (!(ok = mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag, 0x100u + stage))) break;

@@ -1,0 +1,77 @@
+"""CTA-pair tiles at the edges: M and N odd multiples of 128 (half of the last tile lies outside), one tile and many, one
+k-block and many, both output types, both formats, accumulation, two problems in one launch."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import parity as P
+from paper_2509_25149_b200 import binding as B
+from paper_2509_25149_b200 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("shape", [(128, 128, 256), (128, 640, 768), (384, 256, 512), (640, 384, 2304), (1152, 2688, 512)])
+@pytest.mark.parametrize("tile", [512, 640, 768, 0])
+@pytest.mark.parametrize("fp32", [False, True])
+@pytest.mark.parametrize("fmt", ["nvfp4", "mxfp4"])
+def test_odd_multiples_of_128(shape, tile, fp32, fmt):
+    M, N, K = shape
+    X = synth.normal_with_outliers_bf16((M, K), 0.01, 50.0, M + N, M + N + 1)
+    W = synth.normal_bf16((N, K), 0.02, M + N + 2)
+    f = B.FORMAT_MXFP4 if fmt == "mxfp4" else B.FORMAT_NVFP4
+    # the operands sit inside larger buffers filled with NaN scale bytes: nothing beyond the last group may be used
+    A, Bt = B.alloc_tensor(M, K, format=f), B.alloc_tensor(N, K, format=f)
+    for t in (A, Bt):
+        big = torch.full((t.scales.numel() * 2 + 65536,), 0xFF, dtype=torch.uint8, device="cuda")
+        t.scales = big[: t.scales.numel()]
+    B.nvfp4_quantize(X.cuda(), B.quant_opts(), A, None)
+    B.nvfp4_quantize(W.cuda(), B.quant_opts(block_rows=32 if fmt == "mxfp4" else 16), Bt, None)
+    # exact reference: the decoded operands in binary64 (their codes are checked by the quantizer tests)
+    a, b = (B.nvfp4_dequantize(t).double() for t in (A, Bt))
+    Dref, T = (a @ b.T).cpu().numpy(), (a.abs() @ b.abs().T).cpu().numpy()
+    wide = torch.full((M + 8, N + 64), 7.0, dtype=torch.float32 if fp32 else torch.bfloat16, device="cuda")
+    D = wide[:M, :N]
+    B.nvfp4_set_gemm_tile_n(tile)
+    try:
+        B.nvfp4_gemm(A, Bt, D)
+        B.nvfp4_device_status()
+        P.assert_gemm_close(D.float().cpu().numpy(), Dref, T, not fp32, f"{fmt} {shape} tile {tile}")
+        assert torch.all(wide[M:] == 7.0) and torch.all(wide[:, N:] == 7.0)
+        if fp32:  # what is added is the very product
+            once = D.clone()
+            B.nvfp4_gemm(A, Bt, D, accumulate=True)
+            B.nvfp4_device_status()
+            assert torch.equal(D, once + once)
+    finally:
+        B.nvfp4_set_gemm_tile_n(0)
+
+
+@pytest.mark.parametrize("shape", [(256, 512, 256), (768, 1280, 1024)])
+@pytest.mark.parametrize("tile", [512, 640, 768])
+def test_layer_is_the_same_on_every_tile(shape, tile):
+    """Dgrad and Wgrad share a launch; the sums are exact enough that every tile gives the same bits here."""
+    M, N, K = shape
+    X, W = synth.normal_bf16((M, K), 1.0, 1).cuda(), synth.normal_bf16((N, K), 0.02, 2).cuda()
+    dY = synth.normal_bf16((M, N), 1e-3, 3).cuda()
+    opts = B.quant_opts(rht_sign_mask=synth.DEFAULT_RHT_SIGN_MASK, seed=1)
+    ws_f = torch.empty(B.nvfp4_linear_fwd_workspace_bytes(M, K), dtype=torch.uint8, device="cuda")
+    ws_b = torch.empty(B.nvfp4_linear_bwd_workspace_bytes(M, N), dtype=torch.uint8, device="cuda")
+
+    def run(t):
+        X_col, W_row, W_col = B.alloc_tensor(K, M), B.alloc_tensor(N, K), B.alloc_tensor(K, N)
+        Y, dX = (torch.empty(s, dtype=torch.bfloat16, device="cuda") for s in ((M, N), (M, K)))
+        dW = torch.empty((N, K), dtype=torch.float32, device="cuda")
+        B.nvfp4_set_gemm_tile_n(t)
+        try:
+            B.nvfp4_linear_fwd(X, W, opts, Y, X_col, W_row, W_col, False, ws_f)
+            B.nvfp4_linear_bwd(dY, X_col, W_col, K, opts, dX, dW, False, ws_b)
+            B.nvfp4_device_status()
+        finally:
+            B.nvfp4_set_gemm_tile_n(0)
+        return Y, dX, dW
+
+    for got, ref in zip(run(tile), run(0)):
+        d = (got.double() - ref.double()).norm() / ref.double().norm()
+        assert float(d) < 5e-5  # FP32 sums in another order, at most a bf16 boundary crossed here and there
