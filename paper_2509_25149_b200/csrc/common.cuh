@@ -29,6 +29,7 @@ inline bool device_needs_config(const std::atomic<uint64_t>& seen, int* dev) {
 inline void device_configured(std::atomic<uint64_t>& seen, int dev) {
   if (dev >= 0 && dev < 64) seen.fetch_or(1ull << dev, std::memory_order_release);
 }
+cudaError_t sm_count(int* n);  // SMs of the current device (looked up once per device)
 
 // ---------------------------------------------------------------------------------------------
 // Formats

@@ -82,6 +82,21 @@ bool make_map_2d(CUtensorMap* map, CUtensorMapDataType dtype, int elem_bytes, co
   return true;
 }
 
+cudaError_t sm_count(int* n) {
+  static std::atomic<int> cache[64] = {};  // per device ordinal
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  int v = (dev >= 0 && dev < 64) ? cache[dev].load(std::memory_order_relaxed) : 0;
+  if (!v) {
+    e = cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    if (dev >= 0 && dev < 64) cache[dev].store(v, std::memory_order_relaxed);
+  }
+  *n = v;
+  return cudaSuccess;
+}
+
 namespace {
 
 constexpr int BM = 128;
@@ -554,21 +569,6 @@ cudaError_t launch_wide(const GemmArgs& g0, const void* a0, const void* b0, cons
                             m[2], m[3], m[4], m[5], m[6], m[7], a);
   count_launch();
   return le;
-}
-
-cudaError_t sm_count(int* n) {
-  static std::atomic<int> cache[64] = {};  // per device ordinal
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  int v = (dev >= 0 && dev < 64) ? cache[dev].load(std::memory_order_relaxed) : 0;
-  if (!v) {
-    e = cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess) return e;
-    if (dev >= 0 && dev < 64) cache[dev].store(v, std::memory_order_relaxed);
-  }
-  *n = v;
-  return cudaSuccess;
 }
 
 }  // namespace

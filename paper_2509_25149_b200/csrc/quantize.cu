@@ -265,39 +265,6 @@ struct QuantSmem {
   static constexpr int bytes(bool rand, bool row_codes) { return kRand + (rand ? 16384 : row_codes ? 8192 : 0); }
 };
 
-// Bounded wait for a tile (2 s): on expiry the abort word of the CTA and the device status word are set.
-constexpr uint32_t kQuantWaitCode = 0x51000001u;
-__device__ __forceinline__ bool quant_wait(uint32_t bar, uint32_t parity, volatile uint32_t* abort_flag,
-                                           unsigned int* status) {
-  if (mbar_try(bar, parity)) return true;
-  const unsigned long long t0 = globaltimer_ns();
-  uint32_t spins = 0;
-  while (true) {
-    if (mbar_try(bar, parity)) return true;
-    if ((++spins & 63u) == 0u) {
-      if (*abort_flag) return false;
-      if (globaltimer_ns() - t0 > kWaitLimitNs) {
-        *abort_flag = kQuantWaitCode;
-        if (status) atomicCAS(status, 0u, kQuantWaitCode);
-        return false;
-      }
-    }
-  }
-}
-
-// max(m, |a|, |b|)
-__device__ __forceinline__ float amax3(float m, float a, float b) {
-  float r;
-  asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(m), "f"(fabsf(a)), "f"(fabsf(b)));
-  return r;
-}
-__device__ __forceinline__ float amax16_3(const float (&f)[16]) {
-  float m = 0.f;
-#pragma unroll
-  for (int i = 0; i < 16; i += 2) m = amax3(m, f[i], f[i + 1]);
-  return m;
-}
-
 // Eq. 2-3: the stored E4M3 byte of a block, S_b = e4m3(fl(fl(amax_b / 6) * s_enc))
 __device__ __forceinline__ uint32_t block_scale_byte(float amax_b, float s_enc) {
   const float t = __fmul_rn(div6_rn(amax_b), s_enc);

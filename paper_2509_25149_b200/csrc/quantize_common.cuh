@@ -4,6 +4,7 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
+#include "async_ptx.cuh"
 #include "common.cuh"
 
 namespace nvfp4 {
@@ -42,6 +43,39 @@ __device__ __forceinline__ float warp_max(float v) {
 // sign word for a bf16 pair whose two elements are inputs j0 and j1 of a Hadamard chunk
 __device__ __forceinline__ uint32_t sign_pair(uint32_t mask, int j0, int j1) {
   return (((mask >> j0) & 1u) << 15) | (((mask >> j1) & 1u) << 31);
+}
+
+// Bounded wait for a tile (2 s): on expiry the abort word of the CTA and the device status word are set.
+constexpr uint32_t kQuantWaitCode = 0x51000001u;
+__device__ __forceinline__ bool quant_wait(uint32_t bar, uint32_t parity, volatile uint32_t* abort_flag,
+                                           unsigned int* status) {
+  if (mbar_try(bar, parity)) return true;
+  const unsigned long long t0 = globaltimer_ns();
+  uint32_t spins = 0;
+  while (true) {
+    if (mbar_try(bar, parity)) return true;
+    if ((++spins & 63u) == 0u) {
+      if (*abort_flag) return false;
+      if (globaltimer_ns() - t0 > kWaitLimitNs) {
+        *abort_flag = kQuantWaitCode;
+        if (status) atomicCAS(status, 0u, kQuantWaitCode);
+        return false;
+      }
+    }
+  }
+}
+
+// max(m, |a|, |b|)
+__device__ __forceinline__ float amax3(float m, float a, float b) {
+  float r;
+  asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(m), "f"(fabsf(a)), "f"(fabsf(b)));
+  return r;
+}
+__device__ __forceinline__ float amax16_3(const float (&f)[16]) {
+  float m = 0.f;
+#pragma unroll
+  for (int i = 0; i < 16; i += 2) m = amax3(m, f[i], f[i + 1]);
+  return m;
 }
 
 // Eq. 4 for sixteen values: v = fl(y * s_enc,b), two lanes per instruction; for stochastic rounding the result is

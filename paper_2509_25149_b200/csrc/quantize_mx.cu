@@ -37,261 +37,321 @@ __device__ __forceinline__ void fwht32_pairs(float2 v[32]) {
 }
 
 struct MxSmem {
-  static constexpr int kTile = 0;                   // 128 rows x 256 B of bf16
-  static constexpr int kColCodes = 32768;           // 128 columns x 64 B
-  static constexpr int kSfRow = kColCodes + 8192;   // one 512-byte atom: 128 rows x 4 blocks of 32
-  static constexpr int kSfCol = kSfRow + 512;
-  static constexpr int kBlk = kSfCol + 512;         // 32x32 mode: amax of (warp's 16 rows) x (4 column blocks)
-  static constexpr int kRand = kBlk + 128;          // 128 rows x 128 B (stochastic rounding only), chunk cb of row r
-                                                    // at slot cb ^ ((r >> 2) & 7)
-  static constexpr int kBytesNoRand = kRand;
-  static constexpr int kBytesRand = kRand + 16384;
+  static constexpr int kTileBytes = 32768;
+  static constexpr int kTile = 0;                       // 2 x (128 rows x 256 B of bf16), filled by TMA
+  static constexpr int kColCodes = 2 * kTileBytes;      // 2 x (64 column pairs x 128 B)
+  static constexpr int kSfRow = kColCodes + 2 * 8192;   // 2 x one 512-byte atom: 128 rows x 4 blocks of 32
+  static constexpr int kSfCol = kSfRow + 2 * 512;
+  static constexpr int kBlk = kSfCol + 2 * 512;         // 32x32 mode: amax of (warp's 16 rows) x (4 column blocks)
+  static constexpr int kBlkByte = kBlk + 128;           // 32x32 mode: scale byte by (32-row group, column block)
+  static constexpr int kBars = kBlkByte + 32;           // two "tile landed" barriers, then the abort word
+  static constexpr int kRand = kBars + 32;              // 128 rows x 128 B of complemented draws (stochastic rounding),
+                                                        // or 128 rows x 64 B of row-wise codes (32x32, both copies)
+  static constexpr int bytes(bool rand, bool row_codes) { return kRand + (rand ? 16384 : row_codes ? 8192 : 0); }
 };
 
 constexpr float kInvSqrt32 = 0.176776695296636893f;  // fl(1 / sqrt(32))
 
-// One CTA (256 threads) per 128 x 128 tile of the source.
-//   phase 1  each thread owns four 1x16 chunks (32-byte loads); a 1x32 block is the two chunks of an even / odd lane
-//            pair; the row-wise copy is produced from registers, the raw tile (and the random bytes) are staged;
-//   phase 2  each thread owns 32 rows x 2 columns of the staged tile and produces the transposed copy;
-//   phase 3  staged codes and scale bytes leave with 16-byte stores.
+// Persistent CTAs (two per SM) going through 128 x 128 tiles of the source that arrive by TMA in a ring of two buffers, as
+// in quantize_kernel; bound by instruction issue.  One CTA per tile, each loading its own registers and waiting for them,
+// took 45 us for a 8192 x 5120 activation, 80 us for a 8192 x 7168 gradient and 27 us for a 7168 x 5120 weight.
+//   phase 1  each thread owns four 1x16 chunks of the tile; a 1x32 block is the two chunks of an even / odd lane pair;
+//            produces the row-wise copy (and stages the random bytes for stochastic rounding);
+//   phase 2  each thread owns 32 rows x 2 columns of the tile and produces the transposed copy: a pair of warps reads what
+//            the same pair staged, so the 64 threads meet at a barrier of their own;
+//   phase 3  staged codes and scale bytes leave with 16-byte stores (staging double buffered: one CTA barrier per tile).
 template <bool HAS_ROW, bool HAS_COL, bool BLOCK2D, bool RHT_COL, bool SR>
-__global__ void __launch_bounds__(256, RHT_COL ? 2 : 3) quantize_mx_kernel(const QuantArgs a) {
+__global__ void __launch_bounds__(256, 2) quantize_mx_kernel(const __grid_constant__ CUtensorMap src_map,
+                                                             const QuantArgs a) {
+  using S = MxSmem;
   extern __shared__ __align__(128) uint8_t smem[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int tile = (int)blockIdx.x;
-  griddep_launch_dependents();  // the GEMM of a composed call may set itself up while the last CTAs run
-  const int64_t row0 = (int64_t)(tile / a.tiles_c) * 128;
-  const int64_t col0 = (int64_t)(tile % a.tiles_c) * 128;
   const int64_t n_cb = a.cols >> 4;  // 16-chunks per source row (index of the random draws)
+  // 32x32 blocks with both copies requested: the transposed copy holds the very codes of the row-wise one
+  constexpr bool kNibbleTranspose = BLOCK2D && HAS_ROW && HAS_COL;
+  constexpr bool kStageRand = SR && HAS_COL && !kNibbleTranspose;
+  volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(smem + S::kBars + 16);
+  const uint32_t bar0 = smem_u32(smem + S::kBars), tile0 = smem_u32(smem + S::kTile);
 
-  // ------------------------------------------------------------------ phase 1 ----
-  const int cb = lane & 7;  // 16-chunk column inside the tile
-  uint32_t raw[4][8];
-  bool ok[4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int r = warp * 16 + i * 4 + (lane >> 3);
-    ok[i] = (row0 + r < a.rows) && (col0 + cb * 16 < a.cols);
-    if (ok[i]) {
-      ldg256_stream(a.x + (row0 + r) * a.ld + col0 + cb * 16, raw[i]);
-    } else {
-#pragma unroll
-      for (int k = 0; k < 8; ++k) raw[i][k] = 0u;
+  const int total = a.tiles_r * a.tiles_c, stride = (int)gridDim.x;
+  const int n_mine = (total - 1 - (int)blockIdx.x) / stride + 1;  // gridDim.x <= total
+  auto issue = [&](int j) {  // the CTA's tile j into buffer j & 1 (one thread)
+    const int t = (int)blockIdx.x + j * stride, tr = t / a.tiles_c, tc = t - tr * a.tiles_c;
+    mbar_expect_tx(bar0 + 8 * (j & 1), S::kTileBytes);
+    tma_load_2d(tile0 + (j & 1) * S::kTileBytes, &src_map, tc * 128, tr * 128, bar0 + 8 * (j & 1));
+  };
+  if (threadIdx.x == 0) {
+    mbar_init(bar0, 1);
+    mbar_init(bar0 + 8, 1);
+    *abort_flag = 0u;
+    fence_mbarrier_init();
+    fence_proxy_async_smem();
+    griddep_wait();  // the source may be the previous kernel's output; the barrier below holds everybody else's writes
+    issue(0);
+    if (n_mine > 1) issue(1);
+    // no tensor-level scale in this format: the copies' global words read {0, 1} so that the GEMM epilogue's
+    // product of decode scales is 1
+    if (blockIdx.x == 0) {
+      if (HAS_ROW) { a.r_global[0] = 0.f; a.r_global[1] = 1.f; }
+      if (HAS_COL) { a.c_global[0] = 0.f; a.c_global[1] = 1.f; }
     }
   }
-  if (HAS_COL) {
-    const int first = (lane >> 2) & 1;  // halves in lane-dependent order: a quarter warp covers all banks
+  __syncthreads();
+  griddep_launch_dependents();
+
+  const int cb = lane & 7, rl = warp * 16 + (lane >> 3);  // phase 1: chunk column, row of chunk 0 (chunk i: + 4 i)
+  const int q32 = threadIdx.x >> 6, cp = threadIdx.x & 63;  // phase 2: 32-row group, column pair
+  const uint32_t sign2 = a.sign_mask;
+  float* const blk = reinterpret_cast<float*>(smem + S::kBlk);
+  auto pair_sync = [&] { asm volatile("bar.sync %0, 64;" ::"r"(1 + q32) : "memory"); };
+  const int sf_row_pos = a.r_swz ? ((rl & 31) * 16 + (rl >> 5) * 4 + (cb >> 1)) : (rl * 4 + (cb >> 1));
+  const int sf_row_step = a.r_swz ? 64 : 16;  // four rows further (never across a 32-row quarter)
+  const int sf_col_pos = a.c_swz ? (((2 * cp) & 31) * 16 + (cp >> 4) * 4 + q32) : (2 * cp * 4 + q32);
+  const int sf_col_odd = a.c_swz ? 16 : 4;
+  const int64_t r_pitch = a.cols >> 1;
+
+  int j = 0;
+  for (; j < n_mine; ++j) {
+    const int tile = (int)blockIdx.x + j * stride, tr = tile / a.tiles_c, tc = tile - tr * a.tiles_c;
+    const int64_t row0 = (int64_t)tr * 128, col0 = (int64_t)tc * 128;
+    const int buf = j & 1;
+    const uint8_t* const tile_buf = smem + S::kTile + buf * S::kTileBytes;
+    uint8_t* const col_codes = smem + S::kColCodes + buf * 8192;
+    uint8_t* const sf_row = smem + S::kSfRow + buf * 512;
+    uint8_t* const sf_col = smem + S::kSfCol + buf * 512;
+    quant_wait(bar0 + 8 * buf, (uint32_t)(j >> 1) & 1u, abort_flag, a.status);
+
+    // ---------------------------------------------------------------- phase 1 ----
+    uint32_t raw[4][8];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-      const int r = warp * 16 + i * 4 + (lane >> 3);
-      uint8_t* dst = smem + MxSmem::kTile + r * 256 + cb * 32;
-      const uint4 h0 = make_uint4(raw[i][0], raw[i][1], raw[i][2], raw[i][3]);
-      const uint4 h1 = make_uint4(raw[i][4], raw[i][5], raw[i][6], raw[i][7]);
-      if (first) {
-        *reinterpret_cast<uint4*>(dst + 16) = h1;
-        *reinterpret_cast<uint4*>(dst) = h0;
-      } else {
-        *reinterpret_cast<uint4*>(dst) = h0;
-        *reinterpret_cast<uint4*>(dst + 16) = h1;
+      const uint4 h0 = *reinterpret_cast<const uint4*>(tile_buf + rl * 256 + cb * 32 + i * 1024);
+      const uint4 h1 = *reinterpret_cast<const uint4*>(tile_buf + rl * 256 + cb * 32 + i * 1024 + 16);
+      raw[i][0] = h0.x; raw[i][1] = h0.y; raw[i][2] = h0.z; raw[i][3] = h0.w;
+      raw[i][4] = h1.x; raw[i][5] = h1.y; raw[i][6] = h1.z; raw[i][7] = h1.w;
+    }
+    float am[4];  // amax of the 1x32 block each chunk belongs to (the chunk of the neighbouring lane completes it)
+    if (HAS_ROW || BLOCK2D) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        uint32_t acc = 0;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) acc = absmax_bf16x2(acc, raw[i][k]);
+        const float own = fmaxf(bf16_lo(acc), bf16_hi(acc));
+        am[i] = fmaxf(own, __shfl_xor_sync(0xffffffffu, own, 1));
       }
     }
-  }
-
-  // amax of the 1x32 block each chunk belongs to (the chunk of the neighbouring lane completes it)
-  float am[4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    uint32_t acc = 0;
-#pragma unroll
-    for (int k = 0; k < 8; ++k) acc = absmax_bf16x2(acc, raw[i][k]);
-    const float own = fmaxf(bf16_lo(acc), bf16_hi(acc));
-    am[i] = fmaxf(own, __shfl_xor_sync(0xffffffffu, own, 1));
-  }
-  float* blk = reinterpret_cast<float*>(smem + MxSmem::kBlk);
-  if (BLOCK2D) {
-    // 32x32 blocks: the warp's 16 rows first, then the neighbouring warp's 16 rows through shared memory
-    float m = fmaxf(fmaxf(am[0], am[1]), fmaxf(am[2], am[3]));
-    m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 8));
-    m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 16));
-    if (lane < 8 && !(lane & 1)) blk[warp * 4 + (cb >> 1)] = m;
-    __syncthreads();
-    m = fmaxf(blk[warp * 4 + (cb >> 1)], blk[(warp ^ 1) * 4 + (cb >> 1)]);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) am[i] = m;
-  }
-
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int r = warp * 16 + i * 4 + (lane >> 3);
-    uint32_t rnd[4] = {0u, 0u, 0u, 0u};
-    if (SR) {
-      const uint64_t g = (uint64_t)(row0 + r) * (uint64_t)n_cb + (uint64_t)((col0 >> 4) + cb);
-      uint4 q = philox4x32_10((uint32_t)g, (uint32_t)(g >> 32), a.off_lo, a.off_hi, a.rk);
-      rnd[0] = q.x; rnd[1] = q.y; rnd[2] = q.z; rnd[3] = q.w;
-      if (HAS_COL) {
-        uint4 qc = q;
-        if (a.off_hi_col != a.off_hi)
-          qc = philox4x32_10((uint32_t)g, (uint32_t)(g >> 32), a.off_lo, a.off_hi_col, a.rk);
-        *reinterpret_cast<uint4*>(smem + MxSmem::kRand + r * 128 + ((cb ^ ((r >> 2) & 7)) << 4)) = qc;
-      }
-    }
-    if (HAS_ROW) {
-      float f[16];
-#pragma unroll
-      for (int k = 0; k < 8; ++k) {
-        f[2 * k] = bf16_lo(raw[i][k]);
-        f[2 * k + 1] = bf16_hi(raw[i][k]);
-      }
-      uint32_t byte;
-      float enc;
-      mx_scales(am[i], byte, enc);
-      const uint2 codes = convert16<SR>(f, enc, Nu14FromWords{rnd});
-      if (ok[i])
-        *reinterpret_cast<uint2*>(a.r_codes + (row0 + r) * (a.cols >> 1) + ((col0 + cb * 16) >> 1)) = codes;
-      if (!(cb & 1)) {
-        const int pos = a.r_swz ? ((r & 31) * 16 + (r >> 5) * 4 + (cb >> 1)) : (r * 4 + (cb >> 1));
-        smem[MxSmem::kSfRow + pos] = (uint8_t)byte;
-      }
-    }
-  }
-  __syncthreads();
-
-  // ------------------------------------------------------------------ phase 2 ----
-  if (HAS_COL) {
-    const int q32 = threadIdx.x >> 6;  // 32-row group inside the tile
-    const int cp = threadIdx.x & 63;   // column pair: tile columns 2cp, 2cp + 1
-    float2 v[32];
-#pragma unroll
-    for (int j = 0; j < 32; ++j) {
-      uint32_t word = *reinterpret_cast<const uint32_t*>(smem + MxSmem::kTile + (q32 * 32 + j) * 256 + cp * 4);
-      if (RHT_COL) word ^= sign_pair(a.sign_mask, j, j);
-      v[j] = make_float2(bf16_lo(word), bf16_hi(word));
-    }
-    if (RHT_COL) {
-      fwht32_pairs(v);
-      // y = fl(sum * fl(1 / sqrt(32))): Section 5, transform size 32
-      const float2 c2 = make_float2(kInvSqrt32, kInvSqrt32);
-#pragma unroll
-      for (int j = 0; j < 32; ++j) v[j] = mul2(v[j], c2);
-    }
-    float a0 = 0.f, a1 = 0.f;
     if (BLOCK2D) {
-      a0 = a1 = fmaxf(blk[(2 * q32) * 4 + (cp >> 4)], blk[(2 * q32 + 1) * 4 + (cp >> 4)]);
-    } else {
+      // 32x32 blocks: the warp's 16 rows first, then the other warp of the pair's through shared memory
+      float m = fmaxf(fmaxf(am[0], am[1]), fmaxf(am[2], am[3]));
+      m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 8));
+      m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 16));
+      if (lane < 8 && !(lane & 1)) blk[warp * 4 + (cb >> 1)] = m;
+      pair_sync();
+      m = fmaxf(blk[warp * 4 + (cb >> 1)], blk[(warp ^ 1) * 4 + (cb >> 1)]);
 #pragma unroll
-      for (int j = 0; j < 32; ++j) {
-        a0 = fmaxf(a0, fabsf(v[j].x));
-        a1 = fmaxf(a1, fabsf(v[j].y));
-      }
+      for (int i = 0; i < 4; ++i) am[i] = m;
     }
-    uint32_t byte0, byte1;
-    float enc0, enc1;
-    mx_scales(a0, byte0, enc0);
-    mx_scales(a1, byte1, enc1);
-    uint4 out0, out1;  // 32 nibbles of column 2cp / 2cp + 1
+    const bool col_ok = col0 + cb * 16 < a.cols;
+    uint64_t g = 0;
+    if (SR) g = (uint64_t)(row0 + rl) * (uint64_t)n_cb + (uint64_t)((col0 >> 4) + cb);
+    uint8_t* r_out = HAS_ROW ? a.r_codes + (row0 + rl) * r_pitch + ((col0 + cb * 16) >> 1) : nullptr;
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      float f0[16], f1[16];
-      uint32_t two[16];
-#pragma unroll
-      for (int j = 0; j < 16; ++j) {
-        f0[j] = v[16 * h + j].x;
-        f1[j] = v[16 * h + j].y;
-        two[j] = 0u;
-        if (SR) {
-          // low / high byte = draw of source element (row 32 q32 + 16 h + j, column 2cp / 2cp + 1)
-          const int r = q32 * 32 + 16 * h + j;
-          two[j] = *reinterpret_cast<const uint16_t*>(smem + MxSmem::kRand + r * 128 +
-                                                      (((cp >> 3) ^ ((r >> 2) & 7)) << 4) + (cp & 7) * 2);
+    for (int i = 0; i < 4; ++i) {
+      const bool ok = col_ok && row0 + rl + 4 * i < a.rows;
+      uint32_t rnd[4] = {0u, 0u, 0u, 0u};
+      if (SR) {
+        const uint64_t gi = g + (uint64_t)(4 * i) * (uint64_t)n_cb;
+        const uint4 q = philox4x32_10((uint32_t)gi, (uint32_t)(gi >> 32), a.off_lo, a.off_hi, a.rk);
+        rnd[0] = q.x; rnd[1] = q.y; rnd[2] = q.z; rnd[3] = q.w;
+        if (kStageRand) {
+          uint4 qc = q;
+          if (a.off_hi_col != a.off_hi)
+            qc = philox4x32_10((uint32_t)gi, (uint32_t)(gi >> 32), a.off_lo, a.off_hi_col, a.rk);
+          *reinterpret_cast<uint4*>(smem + S::kRand + (rl + 4 * i) * 128 + cb * 16) = make_uint4(~qc.x, ~qc.y, ~qc.z, ~qc.w);
         }
       }
-      const uint2 c0 = convert16<SR>(f0, enc0, Nu14FromPairs<0>{two});
-      const uint2 c1 = convert16<SR>(f1, enc1, Nu14FromPairs<1>{two});
-      if (h == 0) {
-        out0.x = c0.x; out0.y = c0.y; out1.x = c1.x; out1.y = c1.y;
-      } else {
-        out0.z = c0.x; out0.w = c0.y; out1.z = c1.x; out1.w = c1.y;
+      if (HAS_ROW) {
+        float f[16];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          f[2 * k] = bf16_lo(raw[i][k]);
+          f[2 * k + 1] = bf16_hi(raw[i][k]);
+        }
+        uint32_t byte;
+        float enc;
+        mx_scales(am[i], byte, enc);
+        const uint2 codes = convert16<SR>(f, enc, Nu14FromWords{rnd});
+        if (ok) *reinterpret_cast<uint2*>(r_out + (int64_t)(4 * i) * r_pitch) = codes;
+        if (kNibbleTranspose)
+          *reinterpret_cast<uint2*>(smem + S::kRand + (rl + 4 * i) * 64 + cb * 8) = ok ? codes : make_uint2(0u, 0u);
+        if (!(cb & 1)) sf_row[sf_row_pos + i * sf_row_step] = (uint8_t)byte;
+        if (kNibbleTranspose && i == 0 && lane < 8 && !(cb & 1)) smem[S::kBlkByte + warp * 4 + (cb >> 1)] = (uint8_t)byte;
       }
     }
-    // staging as in the NVFP4 kernel: column c holds eight 8-byte units (16 rows each), unit u stored at
-    // (u ^ (c >> 1)) & 7.  The two units of this thread (2 q32, 2 q32 + 1) stay adjacent, swapped when the XOR is
-    // odd; the column written first alternates with the XOR so that a quarter warp covers all banks.
-    const int x = cp & 7;
-#pragma unroll
-    for (int s = 0; s < 2; ++s) {
-      const int odd = s ^ (x & 1);
-      const int c = 2 * cp + odd;
-      uint4 val = odd ? out1 : out0;
-      if (x & 1) val = make_uint4(val.z, val.w, val.x, val.y);
-      *reinterpret_cast<uint4*>(smem + MxSmem::kColCodes + c * 64 + ((((2 * q32) ^ x) & 6) << 3)) = val;
-      const uint32_t byte = odd ? byte1 : byte0;
-      const int pos = a.c_swz ? ((c & 31) * 16 + (c >> 5) * 4 + q32) : (c * 4 + q32);
-      smem[MxSmem::kSfCol + pos] = (uint8_t)byte;
-    }
-  }
-  __syncthreads();
+    if (kStageRand || kNibbleTranspose) pair_sync();  // (otherwise phase 2 reads the tile alone)
 
-  // ------------------------------------------------------------------ phase 3 ----
-  if (HAS_COL) {
-    const int64_t pitch = a.rows >> 1;  // bytes per row of the transposed copy
+    // ---------------------------------------------------------------- phase 2 ----
+    if (HAS_COL) {
+      uint4 out0, out1;  // 32 nibbles of column 2cp / 2cp + 1
+      uint32_t byte0, byte1;
+      if (kNibbleTranspose) {
+        byte0 = byte1 = smem[S::kBlkByte + 2 * q32 * 4 + (cp >> 4)];
+        uint32_t lo[8], hi[8];
 #pragma unroll
-    for (int k = 0; k < 2; ++k) {
-      const int unit = threadIdx.x + 256 * k;
-      const int c = unit >> 2, m = unit & 3;  // column, 32-row group
-      if (col0 + c >= a.cols) continue;
-      const int x = (c >> 1) & 7;
-      uint4 val = *reinterpret_cast<const uint4*>(smem + MxSmem::kColCodes + c * 64 + ((((2 * m) ^ x) & 6) << 3));
-      if (x & 1) val = make_uint4(val.z, val.w, val.x, val.y);
-      if (row0 + 32 * m < a.rows)  // rows % 32 == 0: a 32-row group is inside or outside
-        *reinterpret_cast<uint4*>(a.c_codes + (col0 + c) * pitch + (row0 >> 1) + m * 16) = val;
-    }
-  }
+        for (int m = 0; m < 8; ++m) {
+          // byte [row][cp] of the staged row-wise codes = (column 2cp in the low nibble, 2cp + 1 in the high one)
+          uint32_t b[4];
 #pragma unroll
-  for (int which = 0; which < 2; ++which) {
-    if (which == 0 && !HAS_ROW) continue;
-    if (which == 1 && !HAS_COL) continue;
-    const uint8_t* src = smem + (which == 0 ? MxSmem::kSfRow : MxSmem::kSfCol);
-    uint8_t* dst = which == 0 ? a.r_scales : a.c_scales;
-    const int swz = which == 0 ? a.r_swz : a.c_swz;
-    const int64_t R0 = which == 0 ? row0 : col0, K0 = which == 0 ? (col0 >> 5) : (row0 >> 5);
-    const int64_t Rn = which == 0 ? a.rows : a.cols, n_kb = which == 0 ? (a.cols >> 5) : (a.rows >> 5);
-    if (swz) {
-      if (threadIdx.x < 32) {  // one 512-byte atom per tile and copy
-        const int64_t off = ((R0 >> 7) * (n_kb >> 2) + (K0 >> 2)) * 512 + threadIdx.x * 16;
-        *reinterpret_cast<uint4*>(dst + off) = *reinterpret_cast<const uint4*>(src + threadIdx.x * 16);
+          for (int k = 0; k < 4; ++k) b[k] = smem[S::kRand + (q32 * 32 + 4 * m + k) * 64 + cp];
+          const uint32_t w = __byte_perm(__byte_perm(b[0], b[1], 0x0040), __byte_perm(b[2], b[3], 0x0040), 0x5410);
+          const uint32_t l = w & 0x0F0F0F0Fu, h = (w >> 4) & 0x0F0F0F0Fu;  // four nibbles, one per byte -> 16 bits
+          const uint32_t tl = (l | (l >> 4)) & 0x00FF00FFu, th = (h | (h >> 4)) & 0x00FF00FFu;
+          lo[m] = (tl | (tl >> 8)) & 0xFFFFu;
+          hi[m] = (th | (th >> 8)) & 0xFFFFu;
+        }
+        out0 = make_uint4(lo[0] | (lo[1] << 16), lo[2] | (lo[3] << 16), lo[4] | (lo[5] << 16), lo[6] | (lo[7] << 16));
+        out1 = make_uint4(hi[0] | (hi[1] << 16), hi[2] | (hi[3] << 16), hi[4] | (hi[5] << 16), hi[6] | (hi[7] << 16));
+      } else {
+        float2 v[32];
+        const uint8_t* tp = tile_buf + q32 * 32 * 256 + cp * 4;
+#pragma unroll
+        for (int k = 0; k < 32; ++k) {
+          uint32_t word = *reinterpret_cast<const uint32_t*>(tp + k * 256);
+          if (RHT_COL) word ^= ((sign2 << (31 - k)) & 0x80000000u) | ((k < 16 ? sign2 << (15 - k) : sign2 >> (k - 15)) & 0x8000u);
+          v[k] = make_float2(bf16_lo(word), bf16_hi(word));
+        }
+        if (RHT_COL) {
+          fwht32_pairs(v);
+          // y = fl(sum * fl(1 / sqrt(32))): Section 5, transform size 32
+          const float2 c2 = make_float2(kInvSqrt32, kInvSqrt32);
+#pragma unroll
+          for (int k = 0; k < 32; ++k) v[k] = mul2(v[k], c2);
+        }
+        float a0 = 0.f, a1 = 0.f;
+        if (BLOCK2D) {
+          a0 = a1 = fmaxf(blk[(2 * q32) * 4 + (cp >> 4)], blk[(2 * q32 + 1) * 4 + (cp >> 4)]);
+        } else {
+#pragma unroll
+          for (int k = 0; k < 32; k += 2) {
+            a0 = amax3(a0, v[k].x, v[k + 1].x);
+            a1 = amax3(a1, v[k].y, v[k + 1].y);
+          }
+        }
+        float enc0, enc1;
+        mx_scales(a0, byte0, enc0);
+        mx_scales(a1, byte1, enc1);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          float f0[16], f1[16];
+#pragma unroll
+          for (int k = 0; k < 16; ++k) {
+            f0[k] = v[16 * h + k].x;
+            f1[k] = v[16 * h + k].y;
+          }
+          uint2 c0, c1;
+          if (SR) {
+            // low / high byte of ntwo[k] = 255 - draw of source element (row 32 q32 + 16 h + k, column 2cp / 2cp + 1)
+            uint32_t ntwo[16];
+            const uint8_t* rp = smem + S::kRand + (q32 * 32 + 16 * h) * 128 + cp * 2;
+#pragma unroll
+            for (int k = 0; k < 16; ++k) ntwo[k] = *reinterpret_cast<const uint16_t*>(rp + k * 128);
+            convert16x2_sr(f0, f1, enc0, enc1, ntwo, c0, c1);
+          } else {
+            const uint32_t none[4] = {0u, 0u, 0u, 0u};
+            c0 = convert16<false>(f0, enc0, Nu14FromWords{none});
+            c1 = convert16<false>(f1, enc1, Nu14FromWords{none});
+          }
+          if (h == 0) {
+            out0.x = c0.x; out0.y = c0.y; out1.x = c1.x; out1.y = c1.y;
+          } else {
+            out0.z = c0.x; out0.w = c0.y; out1.z = c1.x; out1.w = c1.y;
+          }
+        }
       }
-    } else {
+      // staging: a column pair has 128 bytes, eight 16-byte units (column parity, 32-row group); unit u sits at u ^ cp
+      *reinterpret_cast<uint4*>(col_codes + cp * 128 + (((q32 ^ cp) & 7) << 4)) = out0;
+      *reinterpret_cast<uint4*>(col_codes + cp * 128 + ((((4 + q32) ^ cp) & 7) << 4)) = out1;
+      sf_col[sf_col_pos] = (uint8_t)byte0;
+      sf_col[sf_col_pos + sf_col_odd] = (uint8_t)byte1;
+    }
+    __syncthreads();
+    if (*abort_flag) break;  // a wait expired (the word is read after the barrier: the same for every thread)
+    if (threadIdx.x == 0 && j + 2 < n_mine) issue(j + 2);  // every warp is done with this buffer
+
+    // ---------------------------------------------------------------- phase 3 ----
+    if (HAS_COL) {
+      const int64_t pitch = a.rows >> 1;  // bytes per row of the transposed copy
 #pragma unroll
       for (int k = 0; k < 2; ++k) {
-        const int idx = threadIdx.x * 2 + k;
-        const int r = idx >> 2, kb = idx & 3;
-        if (R0 + r < Rn && K0 + kb < n_kb) dst[(R0 + r) * n_kb + K0 + kb] = src[idx];
+        const int unit = threadIdx.x + 256 * k;
+        const int c = unit >> 2, m = unit & 3;  // column, 32-row group
+        if (col0 + c >= a.cols || row0 + 32 * m >= a.rows) continue;  // rows % 32 == 0: a group is inside or outside
+        const uint4 val = *reinterpret_cast<const uint4*>(col_codes + (c >> 1) * 128 +
+                                                          (((((c & 1) * 4 + m) ^ (c >> 1)) & 7) << 4));
+        *reinterpret_cast<uint4*>(a.c_codes + (col0 + c) * pitch + (row0 >> 1) + m * 16) = val;
+      }
+    }
+#pragma unroll
+    for (int which = 0; which < 2; ++which) {
+      if (which == 0 ? !HAS_ROW : !HAS_COL) continue;
+      const uint8_t* src = which == 0 ? sf_row : sf_col;
+      uint8_t* dst = which == 0 ? a.r_scales : a.c_scales;
+      const int swz = which == 0 ? a.r_swz : a.c_swz;
+      const int64_t R0 = which == 0 ? row0 : col0, K0 = which == 0 ? (col0 >> 5) : (row0 >> 5);
+      const int64_t Rn = which == 0 ? a.rows : a.cols, n_kb = which == 0 ? (a.cols >> 5) : (a.rows >> 5);
+      if (swz) {
+        if (threadIdx.x < 32) {  // one 512-byte atom per tile and copy
+          const int64_t off = ((R0 >> 7) * (n_kb >> 2) + (K0 >> 2)) * 512 + threadIdx.x * 16;
+          *reinterpret_cast<uint4*>(dst + off) = *reinterpret_cast<const uint4*>(src + threadIdx.x * 16);
+        }
+      } else if (threadIdx.x < 128) {
+        const int r = threadIdx.x;
+        if (R0 + r < Rn) {
+          uint8_t* d = dst + (R0 + r) * n_kb + K0;
+          if (K0 + 4 <= n_kb && (n_kb & 3) == 0) {
+            *reinterpret_cast<uint32_t*>(d) = *reinterpret_cast<const uint32_t*>(src + r * 4);
+          } else {
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+              if (K0 + k < n_kb) d[k] = src[r * 4 + k];
+          }
+        }
       }
     }
   }
-  // no tensor-level scale in this format: the copies' global words read {0, 1} so that the GEMM epilogue's
-  // product of decode scales is 1
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    if (HAS_ROW) { a.r_global[0] = 0.f; a.r_global[1] = 1.f; }
-    if (HAS_COL) { a.c_global[0] = 0.f; a.c_global[1] = 1.f; }
+  if (j < n_mine && threadIdx.x == 0) {
+    // left early: tiles j and j + 1 may still be in flight; one more bounded wait each, so that no copy lands in shared
+    // memory after the CTA has gone
+    for (int i = j; i < j + 2 && i < n_mine; ++i) {
+      const unsigned long long t0 = globaltimer_ns();
+      while (!mbar_try(bar0 + 8 * (i & 1), (uint32_t)(i >> 1) & 1u) && globaltimer_ns() - t0 < kWaitLimitNs) {
+      }
+    }
   }
 }
 
 template <bool HR, bool HC, bool B2, bool RC, bool SR>
 static cudaError_t launch_mx_t(const QuantArgs& a, cudaStream_t s) {
   auto kern = quantize_mx_kernel<HR, HC, B2, RC, SR>;
-  const int smem = (SR && HC) ? MxSmem::kBytesRand : MxSmem::kBytesNoRand;
+  constexpr bool kRowCodes = B2 && HR && HC;
+  constexpr int smem = MxSmem::bytes(SR && HC && !kRowCodes, kRowCodes);
+  CUtensorMap map;
+  if (!make_map_2d(&map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, a.x, (uint64_t)a.cols, (uint64_t)a.rows,
+                   (uint64_t)a.ld * 2, 128, 128, 0))
+    return cudaErrorInvalidValue;
   static std::atomic<uint64_t> configured{0};  // per call site (template instantiation) and device
-  int dev;
+  int dev, sms = 0;
+  cudaError_t e = sm_count(&sms);
+  if (e != cudaSuccess) return e;
   if (device_needs_config(configured, &dev)) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, MxSmem::kBytesRand);
-    if (e != cudaSuccess) return e;
+    if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess) return e;
     device_configured(configured, dev);
   }
-  kern<<<(unsigned)((int64_t)a.tiles_r * a.tiles_c), 256, smem, s>>>(a);
+  const int64_t tiles = (int64_t)a.tiles_r * a.tiles_c;
+  e = launch_kernel(kern, dim3((unsigned)(tiles < 2 * sms ? tiles : 2 * sms)), dim3(256), smem, s, map, a);
   count_launch();
-  return cudaGetLastError();
+  return e;
 }
 
 cudaError_t launch_quantize_mx(const QuantArgs& a, bool has_row, bool has_col, bool block2d, bool rht_col, bool sr,
