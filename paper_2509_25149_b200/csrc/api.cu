@@ -110,6 +110,7 @@ nvfp4_status quantize_impl(const void* x, int64_t rows, int64_t cols, int64_t ld
     a.c_swz = colwise->sf_layout == NVFP4_SF_SWIZZLED;
   }
   a.sign_mask = mx ? o->rht_sign_mask : (o->rht_sign_mask & 0xffffu);
+  for (int j = 0; j < 32; ++j) a.row_sign[j] = ((a.sign_mask >> j) & 1u) ? 0x80008000u : 0u;
   a.seed_lo = (uint32_t)o->seed; a.seed_hi = (uint32_t)(o->seed >> 32);
   for (uint32_t r = 0; r < 10; ++r) {  // Philox key schedule
     a.rk[2 * r] = a.seed_lo + r * 0x9E3779B9u;

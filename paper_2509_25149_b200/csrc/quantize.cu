@@ -379,9 +379,6 @@ __global__ void __launch_bounds__(256, 2) quantize_kernel(const __grid_constant_
   const int cb = lane & 7, rl = warp * 16 + (lane >> 3);
   const uint32_t tile_ld = rl * 256 + cb * 32;     // chunk i of the thread inside a tile buffer: + 1024 i
   const uint32_t rand_st = QuantSmem::kRand + rl * 128 + cb * 16;  // + 512 i
-  // sign of source row j of a 16-row group (the transform of the transposed copy negates whole source rows: input j
-  // of a chunk = row j of the group) for both halves of a bf16 pair: bits 15 and 31 of sign2 << (15 - j)
-  const uint32_t sign2 = (a.sign_mask & 0xffffu) * 0x10001u;
   const int sf_row_pos = a.r_swz ? ((cb >> 2) * 512 + (rl & 31) * 16 + (rl >> 5) * 4 + (cb & 3)) : (rl * 8 + cb);
   const int sf_row_step = a.r_swz ? 64 : 32;
   const int64_t r_pitch = a.cols >> 1;  // bytes per row of the row-wise codes
@@ -538,37 +535,25 @@ __global__ void __launch_bounds__(256, 2) quantize_kernel(const __grid_constant_
             sf_col[sf_col_pos + it * sf_col_it + sf_col_odd] = (uint8_t)byte;
             continue;
           }
-          float f0[16], f1[16];
+          float2 v[16];  // rows of the group, (column 2cp, column 2cp + 1)
           const uint8_t* tp = tile_buf + q * 16 * 256 + cp * 4;
 #pragma unroll
           for (int j = 0; j < 16; ++j) {
             uint32_t word = *reinterpret_cast<const uint32_t*>(tp + j * 256);
-            if (RHT_COL) word ^= (sign2 << (15 - j)) & 0x80008000u;
-            f0[j] = bf16_lo(word);
-            f1[j] = bf16_hi(word);
+            if (RHT_COL) word ^= a.row_sign[j];
+            v[j] = make_float2(bf16_lo(word), bf16_hi(word));
           }
-          if (RHT_COL) {  // values are 4 * y from here on
-            float2 v[16];
-#pragma unroll
-            for (int j = 0; j < 16; ++j) v[j] = make_float2(f0[j], f1[j]);
-            fwht16_pairs(v);  // both columns in one pass of packed adds
-#pragma unroll
-            for (int j = 0; j < 16; ++j) {
-              f0[j] = v[j].x;
-              f1[j] = v[j].y;
-            }
-          }
+          if (RHT_COL) fwht16_pairs(v);  // both columns in one pass of packed adds; values are 4 * y from here on
           uint32_t byte0, byte1;
-          float enc0, enc1;
+          float2 enc;
           if (BLOCK2D) {
-            enc0 = enc1 = reinterpret_cast<const float*>(smem + QuantSmem::kBlkEnc)[q * 8 + (cp >> 3)];
+            enc.x = enc.y = reinterpret_cast<const float*>(smem + QuantSmem::kBlkEnc)[q * 8 + (cp >> 3)];
             byte0 = byte1 = smem[QuantSmem::kBlkByte + q * 8 + (cp >> 3)];
           } else {
-            const float m0 = amax16_3(f0), m1 = amax16_3(f1);
-            byte0 = block_scale_byte(RHT_COL ? 0.25f * m0 : m0, c_senc);
-            byte1 = block_scale_byte(RHT_COL ? 0.25f * m1 : m1, c_senc);
-            enc0 = enc_col[byte0];
-            enc1 = enc_col[byte1];
+            const float2 m = amax_pairs(v);
+            byte0 = block_scale_byte(RHT_COL ? 0.25f * m.x : m.x, c_senc);
+            byte1 = block_scale_byte(RHT_COL ? 0.25f * m.y : m.y, c_senc);
+            enc = make_float2(enc_col[byte0], enc_col[byte1]);
           }
           uint2 codes0, codes1;
           if (SR) {
@@ -577,11 +562,9 @@ __global__ void __launch_bounds__(256, 2) quantize_kernel(const __grid_constant_
             const uint8_t* rp = smem + QuantSmem::kRand + q * 16 * 128 + cp * 2;
 #pragma unroll
             for (int j = 0; j < 16; ++j) ntwo[j] = *reinterpret_cast<const uint16_t*>(rp + j * 128);
-            convert16x2_sr(f0, f1, enc0, enc1, ntwo, codes0, codes1);
+            convert16x2_sr(v, enc, ntwo, codes0, codes1);
           } else {
-            const uint32_t none[4] = {0u, 0u, 0u, 0u};
-            codes0 = convert16<false>(f0, enc0, Nu14FromWords{none});
-            codes1 = convert16<false>(f1, enc1, Nu14FromWords{none});
+            convert16x2_rne(v, enc, codes0, codes1);
           }
           // staging: both columns' eight bytes in one 16-byte unit (conflict-free: eight consecutive column pairs hit
           // eight different units of a 128-byte line)

@@ -132,26 +132,62 @@ struct Nu14FromPairs {
   }
 };
 
-// Two columns of sixteen rows at once (the transposed copy of the main kernel): element j of both columns goes into
-// one conversion.  ntwo[j]: low byte = 255 - draw of (row j, first column), next byte = the same for the second one.
-__device__ __forceinline__ void convert16x2_sr(const float (&f0)[16], const float (&f1)[16], float enc0, float enc1,
-                                               const uint32_t (&ntwo)[16], uint2& out0, uint2& out1) {
-  float v0[16], v1[16];
-  scale16<true>(f0, enc0, v0);
-  scale16<true>(f1, enc1, v1);
+// Two columns of sixteen rows at once (the transposed copy): y[r] = (row r of the first column, of the second), which is
+// how the tile is read and transformed, so that a packed multiplication scales a row of both without moving registers.
+template <bool SR>
+__device__ __forceinline__ float2 scale_row_pair(float2 y, float2 enc) {  // Eq. 4 (see scale16)
+  const float2 p = mul2(y, enc);
+  return SR ? mul2_rz(p, make_float2(kSrTowardsZero, kSrTowardsZero)) : p;
+}
+// Stochastic rounding, element r of both columns in one conversion.  ntwo[r]: low byte = 255 - draw of (row r, first
+// column), next byte = the same for the second one.
+__device__ __forceinline__ void convert16x2_sr(const float2* y, float2 enc, const uint32_t (&ntwo)[16], uint2& out0,
+                                               uint2& out1) {
   // rows (r, r + 1) of both columns: byte 0 = first column, byte 1 = second column; rows (r + 2, r + 3) in bytes 2, 3
   uint32_t e[4];
 #pragma unroll
   for (int m = 0; m < 4; ++m) {
     const int r = 4 * m;
-    const uint32_t a = e2m1x2_sr_pair(v0[r], v1[r], __byte_perm(ntwo[r], 0x80808080u, 0x1044u), v0[r + 2], v1[r + 2],
+    float2 v[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) v[k] = scale_row_pair<true>(y[r + k], enc);
+    const uint32_t a = e2m1x2_sr_pair(v[0].x, v[0].y, __byte_perm(ntwo[r], 0x80808080u, 0x1044u), v[2].x, v[2].y,
                                       __byte_perm(ntwo[r + 2], 0x80808080u, 0x1044u));
-    const uint32_t b = e2m1x2_sr_pair(v0[r + 1], v1[r + 1], __byte_perm(ntwo[r + 1], 0x80808080u, 0x1044u), v0[r + 3],
-                                      v1[r + 3], __byte_perm(ntwo[r + 3], 0x80808080u, 0x1044u));
+    const uint32_t b = e2m1x2_sr_pair(v[1].x, v[1].y, __byte_perm(ntwo[r + 1], 0x80808080u, 0x1044u), v[3].x, v[3].y,
+                                      __byte_perm(ntwo[r + 3], 0x80808080u, 0x1044u));
     e[m] = a + b * 16u;  // disjoint nibbles
   }
   out0 = make_uint2(__byte_perm(e[0], e[1], 0x6420u), __byte_perm(e[2], e[3], 0x6420u));
   out1 = make_uint2(__byte_perm(e[0], e[1], 0x7531u), __byte_perm(e[2], e[3], 0x7531u));
+}
+// Rounding to nearest even
+__device__ __forceinline__ void convert16x2_rne(const float2* y, float2 enc, uint2& out0, uint2& out1) {
+  uint32_t o0[2], o1[2];
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    float v0[8], v1[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const float2 v = scale_row_pair<false>(y[8 * h + k], enc);
+      v0[k] = v.x;
+      v1[k] = v.y;
+    }
+    o0[h] = e2m1x8_rne(v0);
+    o1[h] = e2m1x8_rne(v1);
+  }
+  out0 = make_uint2(o0[0], o0[1]);
+  out1 = make_uint2(o1[0], o1[1]);
+}
+// block maxima of both columns
+template <int ROWS>
+__device__ __forceinline__ float2 amax_pairs(const float2 (&y)[ROWS]) {
+  float2 m = make_float2(0.f, 0.f);
+#pragma unroll
+  for (int r = 0; r < ROWS; r += 2) {
+    m.x = amax3(m.x, y[r].x, y[r + 1].x);
+    m.y = amax3(m.y, y[r].y, y[r + 1].y);
+  }
+  return m;
 }
 
 __device__ __forceinline__ float amax16(const float (&f)[16]) {

@@ -101,7 +101,6 @@ __global__ void __launch_bounds__(256, 2) quantize_mx_kernel(const __grid_consta
 
   const int cb = lane & 7, rl = warp * 16 + (lane >> 3);  // phase 1: chunk column, row of chunk 0 (chunk i: + 4 i)
   const int q32 = threadIdx.x >> 6, cp = threadIdx.x & 63;  // phase 2: 32-row group, column pair
-  const uint32_t sign2 = a.sign_mask;
   float* const blk = reinterpret_cast<float*>(smem + S::kBlk);
   auto pair_sync = [&] { asm volatile("bar.sync %0, 64;" ::"r"(1 + q32) : "memory"); };
   const int sf_row_pos = a.r_swz ? ((rl & 31) * 16 + (rl >> 5) * 4 + (cb >> 1)) : (rl * 4 + (cb >> 1));
@@ -218,37 +217,23 @@ __global__ void __launch_bounds__(256, 2) quantize_mx_kernel(const __grid_consta
 #pragma unroll
         for (int k = 0; k < 32; ++k) {
           uint32_t word = *reinterpret_cast<const uint32_t*>(tp + k * 256);
-          if (RHT_COL) word ^= ((sign2 << (31 - k)) & 0x80000000u) | ((k < 16 ? sign2 << (15 - k) : sign2 >> (k - 15)) & 0x8000u);
+          if (RHT_COL) word ^= a.row_sign[k];
           v[k] = make_float2(bf16_lo(word), bf16_hi(word));
         }
-        if (RHT_COL) {
-          fwht32_pairs(v);
-          // y = fl(sum * fl(1 / sqrt(32))): Section 5, transform size 32
-          const float2 c2 = make_float2(kInvSqrt32, kInvSqrt32);
-#pragma unroll
-          for (int k = 0; k < 32; ++k) v[k] = mul2(v[k], c2);
-        }
-        float a0 = 0.f, a1 = 0.f;
-        if (BLOCK2D) {
-          a0 = a1 = fmaxf(blk[(2 * q32) * 4 + (cp >> 4)], blk[(2 * q32 + 1) * 4 + (cp >> 4)]);
-        } else {
-#pragma unroll
-          for (int k = 0; k < 32; k += 2) {
-            a0 = amax3(a0, v[k].x, v[k + 1].x);
-            a1 = amax3(a1, v[k].y, v[k + 1].y);
-          }
-        }
-        float enc0, enc1;
-        mx_scales(a0, byte0, enc0);
-        mx_scales(a1, byte1, enc1);
+        if (RHT_COL) fwht32_pairs(v);
+        float2 am2, enc;
+        if (BLOCK2D)
+          am2.x = am2.y = fmaxf(blk[(2 * q32) * 4 + (cp >> 4)], blk[(2 * q32 + 1) * 4 + (cp >> 4)]);
+        else
+          am2 = amax_pairs(v);
+        // Section 5, transform size 32: y = fl(sum * c), c = fl(1 / sqrt(32)).  Rounding is monotone, so the block's amax is
+        // fl(max |sum| * c); the encode scale is a power of two, so fl(y * enc) = fl(sum * (c * enc)): y is never formed.
+        if (RHT_COL) am2 = mul2(am2, make_float2(kInvSqrt32, kInvSqrt32));
+        mx_scales(am2.x, byte0, enc.x);
+        mx_scales(am2.y, byte1, enc.y);
+        if (RHT_COL) enc = mul2(enc, make_float2(kInvSqrt32, kInvSqrt32));
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-          float f0[16], f1[16];
-#pragma unroll
-          for (int k = 0; k < 16; ++k) {
-            f0[k] = v[16 * h + k].x;
-            f1[k] = v[16 * h + k].y;
-          }
           uint2 c0, c1;
           if (SR) {
             // low / high byte of ntwo[k] = 255 - draw of source element (row 32 q32 + 16 h + k, column 2cp / 2cp + 1)
@@ -256,11 +241,9 @@ __global__ void __launch_bounds__(256, 2) quantize_mx_kernel(const __grid_consta
             const uint8_t* rp = smem + S::kRand + (q32 * 32 + 16 * h) * 128 + cp * 2;
 #pragma unroll
             for (int k = 0; k < 16; ++k) ntwo[k] = *reinterpret_cast<const uint16_t*>(rp + k * 128);
-            convert16x2_sr(f0, f1, enc0, enc1, ntwo, c0, c1);
+            convert16x2_sr(&v[16 * h], enc, ntwo, c0, c1);
           } else {
-            const uint32_t none[4] = {0u, 0u, 0u, 0u};
-            c0 = convert16<false>(f0, enc0, Nu14FromWords{none});
-            c1 = convert16<false>(f1, enc1, Nu14FromWords{none});
+            convert16x2_rne(&v[16 * h], enc, c0, c1);
           }
           if (h == 0) {
             out0.x = c0.x; out0.y = c0.y; out1.x = c1.x; out1.y = c1.y;
