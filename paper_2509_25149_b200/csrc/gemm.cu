@@ -634,37 +634,47 @@ int best_pair_tile(const GemmArgs& g0, const GemmArgs* g1) {
   return best;
 }
 
-cudaError_t launch_gemm_bf16(const DenseGemmArgs& g, cudaStream_t s) {
-  int num_sms = 0;
-  cudaError_t e = sm_count(&num_sms);
-  if (e != cudaSuccess) return e;
+template <int BN>
+static cudaError_t launch_bf16_t(const DenseGemmArgs& g, int max_pairs, cudaStream_t s) {
+  auto kern = dense::gemm_bf16_pair_kernel<BN>;
   CUtensorMap map_a, map_b, map_d;
   const CUtensorMapDataType bf = CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
   bool ok = g.a_mn ? make_map_2d(&map_a, bf, 2, g.a, (uint64_t)g.M, (uint64_t)g.K, (uint64_t)g.lda * 2, 64, 64, true)
                    : make_map_2d(&map_a, bf, 2, g.a, (uint64_t)g.K, (uint64_t)g.M, (uint64_t)g.lda * 2, 64, 128, true);
   ok = ok && (g.b_mn ? make_map_2d(&map_b, bf, 2, g.b, (uint64_t)g.N, (uint64_t)g.K, (uint64_t)g.ldb * 2, 64, 64, true)
-                     : make_map_2d(&map_b, bf, 2, g.b, (uint64_t)g.K, (uint64_t)g.N, (uint64_t)g.ldb * 2, 64, 128, true));
+                     : make_map_2d(&map_b, bf, 2, g.b, (uint64_t)g.K, (uint64_t)g.N, (uint64_t)g.ldb * 2, 64, BN / 2, true));
   if (g.d_is_fp32)
     ok = ok && make_map_2d(&map_d, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, g.d, (uint64_t)g.N, (uint64_t)g.M,
                            (uint64_t)g.ldd * 4, 16, 128, 2);
   else
     ok = ok && make_map_2d(&map_d, bf, 2, g.d, (uint64_t)g.N, (uint64_t)g.M, (uint64_t)g.ldd * 2, 64, 128, true);
   if (!ok) return cudaErrorInvalidValue;
-  static std::atomic<uint64_t> configured{0};  // per device
+  static std::atomic<uint64_t> configured{0};  // per call site (template instantiation) and device
   int dev;
   if (device_needs_config(configured, &dev)) {
-    e = cudaFuncSetAttribute(dense::gemm_bf16_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             dense::kSmemBytes);
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, dense::kSmemBytes);
     if (e != cudaSuccess) return e;
     device_configured(configured, dev);
   }
   dense::Args a{g.M, g.N, g.K, g.a_mn, g.b_mn, g.d_is_fp32, g.accumulate};
-  const int n_tiles = ((g.M + 255) / 256) * ((g.N + 255) / 256), max_pairs = num_sms / 2;
+  const int n_tiles = ((g.M + 255) / 256) * ((g.N + BN - 1) / BN);
   const int pairs = n_tiles < max_pairs ? n_tiles : max_pairs;
-  e = launch_kernel(dense::gemm_bf16_pair_kernel, dim3(2 * pairs), dim3(dense::kThreads), dense::kSmemBytes, s, map_a,
-                    map_b, map_d, a);
+  const cudaError_t e =
+      launch_kernel(kern, dim3(2 * pairs), dim3(dense::kThreads), dense::kSmemBytes, s, map_a, map_b, map_d, a);
   count_launch();
   return e;
+}
+
+cudaError_t launch_gemm_bf16(const DenseGemmArgs& g, cudaStream_t s) {
+  int num_sms = 0;
+  cudaError_t e = sm_count(&num_sms);
+  if (e != cudaSuccess) return e;
+  // 256 x 128 tiles while every one of them has a pair to itself: less to load per k-block and half the epilogue (1000 x
+  // 2000 x 3000 22.9 -> 19.0 us, 512 x 4096 x 4096 24.2 -> 23.2, 512 x 1024 x 1024 9.1 -> 8.1).  Beyond one round they lose:
+  // an instruction 128 columns wide takes as long as one 256 wide (264 x 7168 x 5120 30 -> 50 us).
+  const int pairs = num_sms / 2;
+  const int64_t tiles128 = (int64_t)((g.M + 255) / 256) * ((g.N + 127) / 128);
+  return tiles128 <= pairs ? launch_bf16_t<128>(g, pairs, s) : launch_bf16_t<256>(g, pairs, s);
 }
 
 // Test aid: one warp waits, with the given limit, on a barrier nobody arrives at.  The wait runs out, the code lands

@@ -53,6 +53,7 @@ __device__ __forceinline__ void tc2_mma_bf16(uint32_t d_tmem, uint64_t adesc, ui
       : "memory");
 }
 
+template <int BN>  // columns of a tile (256 or 128)
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     gemm_bf16_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                           const __grid_constant__ CUtensorMap map_d, const __grid_constant__ Args g) {
@@ -77,7 +78,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   const bool leader = rank == 0;
   const int pair_id = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
   // ragged edges: loads beyond the operands read zeros, stores beyond D are clipped (both by the tensor maps)
-  const int tiles_m = (g.M + 255) / 256, tiles_n = (g.N + 255) / 256, n_tiles = tiles_m * tiles_n;
+  const int tiles_m = (g.M + 255) / 256, tiles_n = (g.N + BN - 1) / BN, n_tiles = tiles_m * tiles_n;
   const int k_blocks = (g.K + 63) / 64;
   // groups of eight row-blocks sweep all column-blocks before the next group starts (L2 reuse of A and B)
   constexpr int kGroupM = 8;
@@ -128,12 +129,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         int m_blk, n_blk;
         tile_coords(tile, m_blk, n_blk);
         const int row_a = m_blk * 256 + (int)rank * 128;  // this CTA's rows of A
-        const int row_b = n_blk * 256 + (int)rank * 128;  // this CTA's half of the B tile
+        const int row_b = n_blk * BN + (int)rank * (BN / 2);  // this CTA's half of the B tile
         for (int kb = 0; kb < k_blocks; ++kb) {
           if (!(ok = mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag, 0x900u + stage))) break;
           const uint32_t st = base + stage * dense::kStageBytes;
           const uint32_t bar = map_to_cta(full_bar(stage), 0);  // the leader's barrier counts both CTAs' operands
-          mbar_expect_tx_cluster(bar, dense::kStageBytes);
+          mbar_expect_tx_cluster(bar, dense::kOperandBytes + BN / 2 * 128);
           if (g.a_mn) {
             tma_load_2d_pair(st, &map_a, row_a, kb * 64, bar);
             tma_load_2d_pair(st + 8192, &map_a, row_a + 64, kb * 64, bar);
@@ -142,7 +143,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
           }
           if (g.b_mn) {
             tma_load_2d_pair(st + dense::kOperandBytes, &map_b, row_b, kb * 64, bar);
-            tma_load_2d_pair(st + dense::kOperandBytes + 8192, &map_b, row_b + 64, kb * 64, bar);
+            if (BN == 256) tma_load_2d_pair(st + dense::kOperandBytes + 8192, &map_b, row_b + 64, kb * 64, bar);
           } else {
             tma_load_2d_pair(st + dense::kOperandBytes, &map_b, kb * 64, row_b, bar);
           }
@@ -159,7 +160,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       int stage = 0;
       uint32_t phase = 0, acc_phase = 0;  // bit b: phase of accumulator b's barrier
       bool ok = true;
-      const uint32_t idesc = instr_desc_bf16(256, 256, g.a_mn, g.b_mn);
+      const uint32_t idesc = instr_desc_bf16(256, BN, g.a_mn, g.b_mn);
       // descriptor halves: start address and leading byte offset (low word), stride byte offset / version /
       // 128-byte swizzle (high word).  K-major: 8-row groups 1024 bytes apart, leading offset unused.  MN-major:
       // 64-index boxes 8192 bytes apart (leading), 8-row k groups 1024 bytes apart (stride).
@@ -212,20 +213,20 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       if (group_gave_up(abort_flag, bar_id, 128)) break;
       tc_fence_after();
       const int row0 = m_blk * 256 + (int)rank * 128;
-      const uint32_t t_row = tmem + ((uint32_t)(quad * 32) << 16) + buf * 256 + half * 128;
-      uint32_t r[128];
+      const uint32_t t_row = tmem + ((uint32_t)(quad * 32) << 16) + buf * 256 + half * (BN / 2);
+      uint32_t r[BN / 2];
 #pragma unroll
-      for (int q = 0; q < 8; ++q) tc_ld16(t_row + q * 16, *reinterpret_cast<uint32_t(*)[16]>(&r[q * 16]));
+      for (int q = 0; q < BN / 32; ++q) tc_ld16(t_row + q * 16, *reinterpret_cast<uint32_t(*)[16]>(&r[q * 16]));
       tc_wait_ld();
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive_cluster(map_to_cta(acce_bar(buf), 0));
       if (g.d_is_fp32)
-        store_half<true>(r, 1.0f, et, bar_id, row_in_tile, stage_buf, &map_d, n_blk * 256 + half * 128, row0,
-                         g.accumulate, false);
+        store_half<true, false, BN / 2>(r, 1.0f, et, bar_id, row_in_tile, stage_buf, &map_d, n_blk * BN + half * (BN / 2),
+                                        row0, g.accumulate, false);
       else
-        store_half<false>(r, 1.0f, et, bar_id, row_in_tile, stage_buf, &map_d, n_blk * 256 + half * 128, row0,
-                          g.accumulate, false);
+        store_half<false, false, BN / 2>(r, 1.0f, et, bar_id, row_in_tile, stage_buf, &map_d, n_blk * BN + half * (BN / 2),
+                                         row0, g.accumulate, false);
       acc_phase ^= 1u << buf;
     }
     if (et == 0) bulk_wait_all<0>();  // all stores have left shared memory and are visible

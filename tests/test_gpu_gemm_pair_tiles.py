@@ -75,3 +75,29 @@ def test_layer_is_the_same_on_every_tile(shape, tile):
     for got, ref in zip(run(tile), run(0)):
         d = (got.double() - ref.double()).norm() / ref.double().norm()
         assert float(d) < 5e-5  # FP32 sums in another order, at most a bf16 boundary crossed here and there
+
+
+@pytest.mark.parametrize("shape", [(8, 8, 8), (264, 520, 72), (776, 1096, 200), (2056, 2568, 136), (1032, 5128, 72)])
+@pytest.mark.parametrize("layouts", [(0, 0), (0, 1), (1, 0), (1, 1)])
+@pytest.mark.parametrize("fp32", [False, True])
+def test_bf16_ragged_on_both_tiles(shape, layouts, fp32):
+    """One round of 256 x 128 tiles (the first three shapes) and several of 256 x 256, edges of every kind, in a larger
+    buffer."""
+    M, N, K = shape
+    g = torch.Generator("cuda").manual_seed(M + N)
+    A, Bt = (torch.randn(s, generator=g, device="cuda").to(torch.bfloat16) for s in ((M, K), (N, K)))
+    ref, T = A.double() @ Bt.double().T, A.double().abs() @ Bt.double().abs().T
+    a = A.T.contiguous() if layouts[0] else A
+    b = Bt.T.contiguous() if layouts[1] else Bt
+    wide = torch.full((M + 8, N + 8), 7.0, dtype=torch.float32 if fp32 else torch.bfloat16, device="cuda")
+    D = wide[:M, :N]
+    B.nvfp4_gemm_bf16(a, b, D, *layouts)
+    B.nvfp4_device_status()
+    bound = 1e-4 * T + (0 if fp32 else 2.0 ** -8) * ref.abs()  # FP32 sums of exact products; one bf16 rounding
+    assert bool(((D.double() - ref).abs() <= bound + 1e-12).all())
+    assert torch.all(wide[M:] == 7.0) and torch.all(wide[:, N:] == 7.0)
+    if fp32:
+        once = D.clone()
+        B.nvfp4_gemm_bf16(a, b, D, *layouts, accumulate=True)
+        B.nvfp4_device_status()
+        assert torch.equal(D, once + once)
