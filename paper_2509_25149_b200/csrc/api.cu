@@ -220,6 +220,31 @@ nvfp4_status gemm_impl(const nvfp4_tensor* A, const nvfp4_tensor* B, void* D, in
   return NVFP4_OK;
 }
 
+// argument checks of one BF16 GEMM and its launch description
+nvfp4_status bf16_prepare(const void* A, int32_t a_layout, int64_t lda, const void* B, int32_t b_layout, int64_t ldb,
+                          int64_t M, int64_t N, int64_t K, void* D, int32_t d_is_fp32, int64_t ldd, int32_t accumulate,
+                          DenseGemmArgs& g) {
+  if (!A || !B || !D) return NVFP4_ERR_NULL;
+  if ((a_layout != NVFP4_K_MAJOR && a_layout != NVFP4_MN_MAJOR) || (b_layout != NVFP4_K_MAJOR && b_layout != NVFP4_MN_MAJOR))
+    return NVFP4_ERR_ARG;
+  if (M <= 0 || N <= 0 || K <= 0 || M % 8 != 0 || N % 8 != 0 || K % 8 != 0) return NVFP4_ERR_SHAPE;
+  if (M > 0x7fffff00 || N > 0x7fffff00 || K > 0x7fffff00 || ((M + 255) / 256) * ((N + 255) / 256) > 0x7fffffff)
+    return NVFP4_ERR_SHAPE;
+  if (lda < (a_layout == NVFP4_MN_MAJOR ? M : K) || ldb < (b_layout == NVFP4_MN_MAJOR ? N : K) || ldd < N)
+    return NVFP4_ERR_SHAPE;
+  if (accumulate && !d_is_fp32) return NVFP4_ERR_ARG;
+  const int64_t esz = d_is_fp32 ? 4 : 2;
+  if (lda % 8 != 0 || ldb % 8 != 0 || (ldd * esz) % 16 != 0 || !aligned(A, 16) || !aligned(B, 16) || !aligned(D, 16))
+    return NVFP4_ERR_ALIGN;
+  g = DenseGemmArgs{};
+  g.a = A; g.b = B; g.d = D;
+  g.lda = lda; g.ldb = ldb; g.ldd = ldd;
+  g.M = (int)M; g.N = (int)N; g.K = (int)K;
+  g.a_mn = a_layout == NVFP4_MN_MAJOR; g.b_mn = b_layout == NVFP4_MN_MAJOR;
+  g.d_is_fp32 = d_is_fp32 != 0; g.accumulate = accumulate != 0;
+  return NVFP4_OK;
+}
+
 inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 inline size_t copy_bytes(int64_t rows, int64_t cols) {
   return align_up((size_t)(rows * cols / 2), 256) + align_up((size_t)(rows * cols / 16), 256) + 256;
@@ -420,25 +445,10 @@ nvfp4_status nvfp4_linear_fwd_noalloc(const void* X, const void* W, int64_t M, i
 nvfp4_status nvfp4_gemm_bf16(const void* A, int32_t a_layout, int64_t lda, const void* B, int32_t b_layout, int64_t ldb,
                              int64_t M, int64_t N, int64_t K, void* D, int32_t d_is_fp32, int64_t ldd,
                              int32_t accumulate, void* cuda_stream) {
-  if (!A || !B || !D) return NVFP4_ERR_NULL;
-  if ((a_layout != NVFP4_K_MAJOR && a_layout != NVFP4_MN_MAJOR) || (b_layout != NVFP4_K_MAJOR && b_layout != NVFP4_MN_MAJOR))
-    return NVFP4_ERR_ARG;
-  if (M <= 0 || N <= 0 || K <= 0 || M % 8 != 0 || N % 8 != 0 || K % 8 != 0) return NVFP4_ERR_SHAPE;
-  if (M > 0x7fffff00 || N > 0x7fffff00 || K > 0x7fffff00 || ((M + 255) / 256) * ((N + 255) / 256) > 0x7fffffff)
-    return NVFP4_ERR_SHAPE;
-  if (lda < (a_layout == NVFP4_MN_MAJOR ? M : K) || ldb < (b_layout == NVFP4_MN_MAJOR ? N : K) || ldd < N)
-    return NVFP4_ERR_SHAPE;
-  if (accumulate && !d_is_fp32) return NVFP4_ERR_ARG;
-  const int64_t esz = d_is_fp32 ? 4 : 2;
-  if (lda % 8 != 0 || ldb % 8 != 0 || (ldd * esz) % 16 != 0 || !aligned(A, 16) || !aligned(B, 16) || !aligned(D, 16))
-    return NVFP4_ERR_ALIGN;
-  DenseGemmArgs g{};
-  g.a = A; g.b = B; g.d = D;
-  g.lda = lda; g.ldb = ldb; g.ldd = ldd;
-  g.M = (int)M; g.N = (int)N; g.K = (int)K;
-  g.a_mn = a_layout == NVFP4_MN_MAJOR; g.b_mn = b_layout == NVFP4_MN_MAJOR;
-  g.d_is_fp32 = d_is_fp32 != 0; g.accumulate = accumulate != 0;
-  return launch_gemm_bf16(g, static_cast<cudaStream_t>(cuda_stream)) == cudaSuccess ? NVFP4_OK : NVFP4_ERR_CUDA;
+  DenseGemmArgs g;
+  const nvfp4_status st = bf16_prepare(A, a_layout, lda, B, b_layout, ldb, M, N, K, D, d_is_fp32, ldd, accumulate, g);
+  if (st != NVFP4_OK) return st;
+  return launch_gemm_bf16(g, nullptr, static_cast<cudaStream_t>(cuda_stream)) == cudaSuccess ? NVFP4_OK : NVFP4_ERR_CUDA;
 }
 
 nvfp4_status nvfp4_linear_bf16_fwd(const void* X, const void* W, int64_t M, int64_t N, int64_t K, void* Y_bf16,
@@ -451,15 +461,21 @@ nvfp4_status nvfp4_linear_bf16_bwd(const void* dY, const void* X, const void* W,
   if (!dY) return NVFP4_ERR_NULL;
   if (!dX_bf16 && !dW_fp32) return NVFP4_ERR_NULL;
   nvfp4_status st;
+  DenseGemmArgs gd, gw;
   // Dgrad: dX[M x K] = dY[M x N] W[N x K]; the contraction runs over W's rows
-  if (dX_bf16 && (st = nvfp4_gemm_bf16(dY, NVFP4_K_MAJOR, N, W, NVFP4_MN_MAJOR, K, M, K, N, dX_bf16, 0, K, 0,
-                                       cuda_stream)) != NVFP4_OK)
+  if (dX_bf16 &&
+      (st = bf16_prepare(dY, NVFP4_K_MAJOR, N, W, NVFP4_MN_MAJOR, K, M, K, N, dX_bf16, 0, K, 0, gd)) != NVFP4_OK)
     return st;
   // Wgrad: dW[N x K] = dY^T X; the contraction runs over the tokens, the rows of both operands
-  if (dW_fp32 && (st = nvfp4_gemm_bf16(dY, NVFP4_MN_MAJOR, N, X, NVFP4_MN_MAJOR, K, N, K, M, dW_fp32, 1, K,
-                                       accumulate_dw, cuda_stream)) != NVFP4_OK)
+  if (dW_fp32 && (st = bf16_prepare(dY, NVFP4_MN_MAJOR, N, X, NVFP4_MN_MAJOR, K, N, K, M, dW_fp32, 1, K, accumulate_dw,
+                                    gw)) != NVFP4_OK)
     return st;
-  return NVFP4_OK;
+  // both: one launch, the longer contraction first
+  const bool both = dX_bf16 && dW_fp32, dgrad_first = dX_bf16 && (!both || gd.K >= gw.K);
+  return launch_gemm_bf16(dgrad_first ? gd : gw, both ? (dgrad_first ? &gw : &gd) : nullptr,
+                          static_cast<cudaStream_t>(cuda_stream)) == cudaSuccess
+             ? NVFP4_OK
+             : NVFP4_ERR_CUDA;
 }
 
 nvfp4_status nvfp4_quant_error(const void* x_bf16, int64_t rows, int64_t cols, int64_t ld, const nvfp4_tensor* q,

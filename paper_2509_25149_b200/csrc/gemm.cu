@@ -635,20 +635,33 @@ int best_pair_tile(const GemmArgs& g0, const GemmArgs* g1) {
 }
 
 template <int BN>
-static cudaError_t launch_bf16_t(const DenseGemmArgs& g, int max_pairs, cudaStream_t s) {
-  auto kern = dense::gemm_bf16_pair_kernel<BN>;
-  CUtensorMap map_a, map_b, map_d;
+static bool make_bf16_maps(const DenseGemmArgs& g, CUtensorMap* m) {  // A, B, D
   const CUtensorMapDataType bf = CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
-  bool ok = g.a_mn ? make_map_2d(&map_a, bf, 2, g.a, (uint64_t)g.M, (uint64_t)g.K, (uint64_t)g.lda * 2, 64, 64, true)
-                   : make_map_2d(&map_a, bf, 2, g.a, (uint64_t)g.K, (uint64_t)g.M, (uint64_t)g.lda * 2, 64, 128, true);
-  ok = ok && (g.b_mn ? make_map_2d(&map_b, bf, 2, g.b, (uint64_t)g.N, (uint64_t)g.K, (uint64_t)g.ldb * 2, 64, 64, true)
-                     : make_map_2d(&map_b, bf, 2, g.b, (uint64_t)g.K, (uint64_t)g.N, (uint64_t)g.ldb * 2, 64, BN / 2, true));
+  bool ok = g.a_mn ? make_map_2d(&m[0], bf, 2, g.a, (uint64_t)g.M, (uint64_t)g.K, (uint64_t)g.lda * 2, 64, 64, true)
+                   : make_map_2d(&m[0], bf, 2, g.a, (uint64_t)g.K, (uint64_t)g.M, (uint64_t)g.lda * 2, 64, 128, true);
+  ok = ok && (g.b_mn ? make_map_2d(&m[1], bf, 2, g.b, (uint64_t)g.N, (uint64_t)g.K, (uint64_t)g.ldb * 2, 64, 64, true)
+                     : make_map_2d(&m[1], bf, 2, g.b, (uint64_t)g.K, (uint64_t)g.N, (uint64_t)g.ldb * 2, 64, BN / 2, true));
   if (g.d_is_fp32)
-    ok = ok && make_map_2d(&map_d, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, g.d, (uint64_t)g.N, (uint64_t)g.M,
+    ok = ok && make_map_2d(&m[2], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, g.d, (uint64_t)g.N, (uint64_t)g.M,
                            (uint64_t)g.ldd * 4, 16, 128, 2);
   else
-    ok = ok && make_map_2d(&map_d, bf, 2, g.d, (uint64_t)g.N, (uint64_t)g.M, (uint64_t)g.ldd * 2, 64, 128, true);
-  if (!ok) return cudaErrorInvalidValue;
+    ok = ok && make_map_2d(&m[2], bf, 2, g.d, (uint64_t)g.N, (uint64_t)g.M, (uint64_t)g.ldd * 2, 64, 128, true);
+  return ok;
+}
+
+static int bf16_tiles(const DenseGemmArgs& g, int bn) { return ((g.M + 255) / 256) * ((g.N + bn - 1) / bn); }
+
+// g1 == nullptr: one problem
+template <int BN>
+static cudaError_t launch_bf16_t(const DenseGemmArgs& g0, const DenseGemmArgs* g1, int max_pairs, cudaStream_t s) {
+  auto kern = dense::gemm_bf16_pair_kernel<BN>;
+  CUtensorMap m[6];
+  if (!make_bf16_maps<BN>(g0, m)) return cudaErrorInvalidValue;
+  if (g1) {
+    if (!make_bf16_maps<BN>(*g1, m + 3)) return cudaErrorInvalidValue;
+  } else {
+    for (int i = 0; i < 3; ++i) m[3 + i] = m[i];
+  }
   static std::atomic<uint64_t> configured{0};  // per call site (template instantiation) and device
   int dev;
   if (device_needs_config(configured, &dev)) {
@@ -656,16 +669,22 @@ static cudaError_t launch_bf16_t(const DenseGemmArgs& g, int max_pairs, cudaStre
     if (e != cudaSuccess) return e;
     device_configured(configured, dev);
   }
-  dense::Args a{g.M, g.N, g.K, g.a_mn, g.b_mn, g.d_is_fp32, g.accumulate};
-  const int n_tiles = ((g.M + 255) / 256) * ((g.N + BN - 1) / BN);
-  const int pairs = n_tiles < max_pairs ? n_tiles : max_pairs;
-  const cudaError_t e =
-      launch_kernel(kern, dim3(2 * pairs), dim3(dense::kThreads), dense::kSmemBytes, s, map_a, map_b, map_d, a);
+  auto problem = [](const DenseGemmArgs& g) {
+    return dense::Problem{g.M, g.N, g.K, g.a_mn, g.b_mn, g.d_is_fp32, g.accumulate};
+  };
+  dense::Args a{};
+  a.p[0] = problem(g0);
+  a.p[1] = problem(g1 ? *g1 : g0);
+  a.n_tiles0 = bf16_tiles(g0, BN);
+  a.n_tiles = a.n_tiles0 + (g1 ? bf16_tiles(*g1, BN) : 0);
+  const int pairs = a.n_tiles < max_pairs ? a.n_tiles : max_pairs;
+  const cudaError_t e = launch_kernel(kern, dim3(2 * pairs), dim3(dense::kThreads), dense::kSmemBytes, s, m[0], m[1], m[2],
+                                      m[3], m[4], m[5], a);
   count_launch();
   return e;
 }
 
-cudaError_t launch_gemm_bf16(const DenseGemmArgs& g, cudaStream_t s) {
+cudaError_t launch_gemm_bf16(const DenseGemmArgs& g0, const DenseGemmArgs* g1, cudaStream_t s) {
   int num_sms = 0;
   cudaError_t e = sm_count(&num_sms);
   if (e != cudaSuccess) return e;
@@ -673,8 +692,8 @@ cudaError_t launch_gemm_bf16(const DenseGemmArgs& g, cudaStream_t s) {
   // 2000 x 3000 22.9 -> 19.0 us, 512 x 4096 x 4096 24.2 -> 23.2, 512 x 1024 x 1024 9.1 -> 8.1).  Beyond one round they lose:
   // an instruction 128 columns wide takes as long as one 256 wide (264 x 7168 x 5120 30 -> 50 us).
   const int pairs = num_sms / 2;
-  const int64_t tiles128 = (int64_t)((g.M + 255) / 256) * ((g.N + 127) / 128);
-  return tiles128 <= pairs ? launch_bf16_t<128>(g, pairs, s) : launch_bf16_t<256>(g, pairs, s);
+  const int64_t tiles128 = (int64_t)bf16_tiles(g0, 128) + (g1 ? bf16_tiles(*g1, 128) : 0);
+  return tiles128 <= pairs ? launch_bf16_t<128>(g0, g1, pairs, s) : launch_bf16_t<256>(g0, g1, pairs, s);
 }
 
 // Test aid: one warp waits, with the given limit, on a barrier nobody arrives at.  The wait runs out, the code lands

@@ -57,6 +57,7 @@ struct DenseGemmArgs {
   int a_mn, b_mn;
   int d_is_fp32, accumulate;
 };
-cudaError_t launch_gemm_bf16(const DenseGemmArgs& g, cudaStream_t s);
+// g1 (may be NULL): a second, independent product in the same launch, its tiles after those of g0
+cudaError_t launch_gemm_bf16(const DenseGemmArgs& g0, const DenseGemmArgs* g1, cudaStream_t s);
 
 }  // namespace nvfp4

@@ -30,10 +30,17 @@ constexpr int kStagingBytes = 2 * 16384;
 constexpr int kSmemBytes = kStages * kStageBytes + kStagingBytes + 1024 /*alignment*/ + 256 /*barriers*/;
 constexpr uint32_t kTmemCols = 512;                // two 256-column accumulators
 
-struct Args {
+struct Problem {
   int M, N, K;
   int a_mn, b_mn;  // 1 = the operand is stored with the output index contiguous
   int d_is_fp32, accumulate;
+};
+// One launch works through the tiles of up to two independent products (problem 0 first): Dgrad and Wgrad of a layer fill
+// each other's partial last round (4088 x 5128 x 5112: 5 + 6 rounds of tiles on 74 pairs become 10).
+struct Args {
+  Problem p[2];
+  int n_tiles0;  // tiles of problem 0
+  int n_tiles;   // tiles of both problems
 };
 
 // kind::f16 instruction descriptor: FP32 accumulator (bit 4), BF16 x BF16 (format 1 at bits 7 and 10), operand
@@ -55,8 +62,10 @@ __device__ __forceinline__ void tc2_mma_bf16(uint32_t d_tmem, uint64_t adesc, ui
 
 template <int BN>  // columns of a tile (256 or 128)
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
-    gemm_bf16_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
-                          const __grid_constant__ CUtensorMap map_d, const __grid_constant__ Args g) {
+    gemm_bf16_pair_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant__ CUtensorMap map_b0,
+                          const __grid_constant__ CUtensorMap map_d0, const __grid_constant__ CUtensorMap map_a1,
+                          const __grid_constant__ CUtensorMap map_b1, const __grid_constant__ CUtensorMap map_d1,
+                          const __grid_constant__ Args g) {
   using namespace pair;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -78,11 +87,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   const bool leader = rank == 0;
   const int pair_id = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
   // ragged edges: loads beyond the operands read zeros, stores beyond D are clipped (both by the tensor maps)
-  const int tiles_m = (g.M + 255) / 256, tiles_n = (g.N + BN - 1) / BN, n_tiles = tiles_m * tiles_n;
-  const int k_blocks = (g.K + 63) / 64;
+  const int n_tiles = g.n_tiles;
+  auto k_blocks_of = [&](int tile) { return (g.p[tile >= g.n_tiles0 ? 1 : 0].K + 63) / 64; };
   // groups of eight row-blocks sweep all column-blocks before the next group starts (L2 reuse of A and B)
   constexpr int kGroupM = 8;
-  auto tile_coords = [&](int tile, int& m_blk, int& n_blk) {
+  auto tile_coords = [&](int tile, int& prob, int& m_blk, int& n_blk) {
+    prob = tile >= g.n_tiles0 ? 1 : 0;
+    if (prob) tile -= g.n_tiles0;
+    const int tiles_m = (g.p[prob].M + 255) / 256, tiles_n = (g.p[prob].N + BN - 1) / BN;
     const int per_group = kGroupM * tiles_n;
     const int grp = tile / per_group, in_grp = tile - grp * per_group;
     const int m0 = grp * kGroupM;
@@ -126,8 +138,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       uint32_t phase = 0;
       bool ok = true;
       for (int tile = pair_id; tile < n_tiles && ok; tile += n_pairs) {
-        int m_blk, n_blk;
-        tile_coords(tile, m_blk, n_blk);
+        int prob, m_blk, n_blk;
+        tile_coords(tile, prob, m_blk, n_blk);
+        const CUtensorMap* map_a = prob ? &map_a1 : &map_a0;
+        const CUtensorMap* map_b = prob ? &map_b1 : &map_b0;
+        const int a_mn = g.p[prob].a_mn, b_mn = g.p[prob].b_mn, k_blocks = k_blocks_of(tile);
         const int row_a = m_blk * 256 + (int)rank * 128;  // this CTA's rows of A
         const int row_b = n_blk * BN + (int)rank * (BN / 2);  // this CTA's half of the B tile
         for (int kb = 0; kb < k_blocks; ++kb) {
@@ -135,17 +150,17 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
           const uint32_t st = base + stage * dense::kStageBytes;
           const uint32_t bar = map_to_cta(full_bar(stage), 0);  // the leader's barrier counts both CTAs' operands
           mbar_expect_tx_cluster(bar, dense::kOperandBytes + BN / 2 * 128);
-          if (g.a_mn) {
-            tma_load_2d_pair(st, &map_a, row_a, kb * 64, bar);
-            tma_load_2d_pair(st + 8192, &map_a, row_a + 64, kb * 64, bar);
+          if (a_mn) {
+            tma_load_2d_pair(st, map_a, row_a, kb * 64, bar);
+            tma_load_2d_pair(st + 8192, map_a, row_a + 64, kb * 64, bar);
           } else {
-            tma_load_2d_pair(st, &map_a, kb * 64, row_a, bar);
+            tma_load_2d_pair(st, map_a, kb * 64, row_a, bar);
           }
-          if (g.b_mn) {
-            tma_load_2d_pair(st + dense::kOperandBytes, &map_b, row_b, kb * 64, bar);
-            if (BN == 256) tma_load_2d_pair(st + dense::kOperandBytes + 8192, &map_b, row_b + 64, kb * 64, bar);
+          if (b_mn) {
+            tma_load_2d_pair(st + dense::kOperandBytes, map_b, row_b, kb * 64, bar);
+            if (BN == 256) tma_load_2d_pair(st + dense::kOperandBytes + 8192, map_b, row_b + 64, kb * 64, bar);
           } else {
-            tma_load_2d_pair(st + dense::kOperandBytes, &map_b, kb * 64, row_b, bar);
+            tma_load_2d_pair(st + dense::kOperandBytes, map_b, kb * 64, row_b, bar);
           }
           if (++stage == S) {
             stage = 0;
@@ -160,20 +175,23 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       int stage = 0;
       uint32_t phase = 0, acc_phase = 0;  // bit b: phase of accumulator b's barrier
       bool ok = true;
-      const uint32_t idesc = instr_desc_bf16(256, BN, g.a_mn, g.b_mn);
       // descriptor halves: start address and leading byte offset (low word), stride byte offset / version /
       // 128-byte swizzle (high word).  K-major: 8-row groups 1024 bytes apart, leading offset unused.  MN-major:
       // 64-index boxes 8192 bytes apart (leading), 8-row k groups 1024 bytes apart (stride).
-      const uint32_t a_lo0 = ((base >> 4) & 0x3fffu) | ((g.a_mn ? (8192u >> 4) : 1u) << 16);
-      const uint32_t b_lo0 = (((base + dense::kOperandBytes) >> 4) & 0x3fffu) | ((g.b_mn ? (8192u >> 4) : 1u) << 16);
-      const uint32_t a_step = g.a_mn ? (2048u >> 4) : (32u >> 4);  // one K = 16 instruction further
-      const uint32_t b_step = g.b_mn ? (2048u >> 4) : (32u >> 4);
+      const uint32_t a_lo_base = (base >> 4) & 0x3fffu, b_lo_base = ((base + dense::kOperandBytes) >> 4) & 0x3fffu;
       int it = 0;
       for (int tile = pair_id; tile < n_tiles && ok; tile += n_pairs, ++it) {
         const int buf = it & 1;
         if (!(ok = mbar_wait_cluster(acce_bar(buf), ((acc_phase >> buf) & 1u) ^ 1u, abort_flag, 0xB00u + buf))) break;
         tc_fence_after();
         const uint32_t d_t = tmem + buf * 256;
+        const Problem& pr = g.p[tile >= g.n_tiles0 ? 1 : 0];
+        const uint32_t idesc = instr_desc_bf16(256, BN, pr.a_mn, pr.b_mn);
+        const uint32_t a_lo0 = a_lo_base | ((pr.a_mn ? (8192u >> 4) : 1u) << 16);
+        const uint32_t b_lo0 = b_lo_base | ((pr.b_mn ? (8192u >> 4) : 1u) << 16);
+        const uint32_t a_step = pr.a_mn ? (2048u >> 4) : (32u >> 4);  // one K = 16 instruction further
+        const uint32_t b_step = pr.b_mn ? (2048u >> 4) : (32u >> 4);
+        const int k_blocks = k_blocks_of(tile);
         for (int kb = 0; kb < k_blocks; ++kb) {
           if (!(ok = mbar_wait_cluster(full_bar(stage), phase, abort_flag, 0xA00u + stage))) break;
           tc_fence_after();
@@ -203,11 +221,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     uint32_t acc_phase = 0;
     const int row_in_tile = quad * 32 + lane;
     const uint32_t stage_buf = staging + half * 16384;
-    int it = 0;
+    int it = 0, last_prob = 0;
     for (int tile = pair_id; tile < n_tiles; tile += n_pairs, ++it) {
       const int buf = it & 1;
-      int m_blk, n_blk;
-      tile_coords(tile, m_blk, n_blk);
+      int prob, m_blk, n_blk;
+      tile_coords(tile, prob, m_blk, n_blk);
+      const CUtensorMap* map_d = prob ? &map_d1 : &map_d0;
+      const bool drain = prob != last_prob;  // the problems of a launch may have different output types
+      last_prob = prob;
       mbar_wait_cluster(accf_bar(buf), (acc_phase >> buf) & 1u, abort_flag, 0xC00u + buf);
       // agree on giving up: a warp that timed out still joins this barrier, and all 128 threads take ONE decision
       if (group_gave_up(abort_flag, bar_id, 128)) break;
@@ -221,12 +242,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive_cluster(map_to_cta(acce_bar(buf), 0));
-      if (g.d_is_fp32)
-        store_half<true, false, BN / 2>(r, 1.0f, et, bar_id, row_in_tile, stage_buf, &map_d, n_blk * BN + half * (BN / 2),
-                                        row0, g.accumulate, false);
+      if (g.p[prob].d_is_fp32)
+        store_half<true, false, BN / 2>(r, 1.0f, et, bar_id, row_in_tile, stage_buf, map_d, n_blk * BN + half * (BN / 2),
+                                        row0, g.p[prob].accumulate, drain);
       else
-        store_half<false, false, BN / 2>(r, 1.0f, et, bar_id, row_in_tile, stage_buf, &map_d, n_blk * BN + half * (BN / 2),
-                                         row0, g.accumulate, false);
+        store_half<false, false, BN / 2>(r, 1.0f, et, bar_id, row_in_tile, stage_buf, map_d, n_blk * BN + half * (BN / 2),
+                                         row0, g.p[prob].accumulate, drain);
       acc_phase ^= 1u << buf;
     }
     if (et == 0) bulk_wait_all<0>();  // all stores have left shared memory and are visible
