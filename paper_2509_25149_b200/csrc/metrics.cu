@@ -18,13 +18,16 @@ namespace nvfp4 {
 
 namespace {
 
+// CTAs of 16 warps, two per SM: a quarter of the FP64 atomics on the two sums that CTAs of eight at eight per SM took
+constexpr int kWarps = 16, kThreads = 32 * kWarps;
+
 __device__ __forceinline__ void block_reduce_add(double err, double ref, double* out) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     err += __shfl_xor_sync(0xffffffffu, err, o);
     ref += __shfl_xor_sync(0xffffffffu, ref, o);
   }
-  __shared__ double red[2][8];
+  __shared__ double red[2][kWarps];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (lane == 0) {
     red[0][warp] = err;
@@ -35,22 +38,37 @@ __device__ __forceinline__ void block_reduce_add(double err, double ref, double*
     griddep_wait();  // the sums are zero
     double s = 0.0;
 #pragma unroll
-    for (int w = 0; w < 8; ++w) s += red[threadIdx.x][w];
+    for (int w = 0; w < kWarps; ++w) s += red[threadIdx.x][w];
     atomicAdd(out + threadIdx.x, s);
   }
 }
 
-// i = r * n + c with c < n: 32-bit division whenever the index allows (the 64-bit one costs as much as the rest of a
-// 16-element chunk)
-__device__ __forceinline__ void split_index(int64_t i, int64_t n, int64_t& r, int64_t& c) {
-  if (i <= 0xffffffffll && n <= 0xffffffffll) {
-    const uint32_t q = (uint32_t)i / (uint32_t)n;
-    r = q;
-    c = (uint32_t)i - q * (uint32_t)n;
-  } else {
-    r = i / n;
-    c = i - r * n;
+// Walks a thread through units first, first + step, ... of a [rows x n] array: coordinates move by additions (a division
+// per 16 elements cost a sixth of the instructions).
+struct Walk {
+  int64_t r, dr, c, dc, n;
+  __device__ __forceinline__ Walk(int64_t first, int64_t step, int64_t n_) : n(n_) {
+    r = first / n;
+    c = first - r * n;
+    dr = step / n;
+    dc = step - dr * n;
   }
+  __device__ __forceinline__ void next() {
+    r += dr;
+    c += dc;
+    if (c >= n) {
+      c -= n;
+      ++r;
+    }
+  }
+};
+
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+  float2 r;
+  asm("{.reg .b64 ra, rb, rc, rd; mov.b64 ra, {%2, %3}; mov.b64 rb, {%4, %5}; mov.b64 rc, {%6, %7}; "
+      "fma.rn.f32x2 rd, ra, rb, rc; mov.b64 {%0, %1}, rd;}"
+      : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+  return r;
 }
 
 // one byte of codes -> its two E2M1 values (low nibble first)
@@ -65,46 +83,62 @@ __device__ __forceinline__ float2 e2m1x2_values(uint32_t byte) {
 }
 
 template <bool MX>
-__global__ void __launch_bounds__(256) quant_error_kernel(const uint16_t* __restrict__ x, int64_t rows, int64_t cols,
+__global__ void __launch_bounds__(kThreads, 2) quant_error_kernel(const uint16_t* __restrict__ x, int64_t rows, int64_t cols,
                                                           int64_t ld, const uint8_t* __restrict__ codes,
                                                           const uint8_t* __restrict__ scales,
                                                           const float* __restrict__ global, int swz,
                                                           int per_row, double* __restrict__ out) {
   const int64_t n_cb = cols >> 4;                 // 16-element chunks per row
   const int64_t n_sb = MX ? (cols >> 5) : n_cb;   // scale blocks per row
-  const int64_t n_chunks = rows * n_cb;
   const float s_dec_t = MX ? 1.f : global[1];
   double err = 0.0, ref = 0.0;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n_chunks; i += (int64_t)gridDim.x * blockDim.x) {
-    int64_t r, cb;
-    split_index(i, n_cb, r, cb);
-    uint32_t raw[8];
-    ldg256_stream(x + r * ld + cb * 16, raw);
-    const uint2 c = *reinterpret_cast<const uint2*>(codes + r * (cols >> 1) + cb * 8);
-    const int64_t sb = MX ? (cb >> 1) : cb;
-    const uint32_t byte = scales[swz ? sf_swizzled_offset(r, sb, n_sb) : (r * n_sb + sb)];
-    float sf;
-    if (MX) {
-      sf = byte == 0 ? __uint_as_float(0x00400000u) : __uint_as_float(byte << 23);  // 2^(byte - 127)
-    } else {
-      uint32_t h2;
-      asm("cvt.rn.f16x2.e4m3x2 %0, %1;" : "=r"(h2) : "h"((uint16_t)byte));
-      sf = __half2float(__ushort_as_half((unsigned short)(h2 & 0xffffu)));
+  Walk w(blockIdx.x * (int64_t)blockDim.x + threadIdx.x, (int64_t)gridDim.x * blockDim.x, n_cb);
+  constexpr int kDepth = 3;  // chunks whose loads are in flight
+  uint32_t raw[kDepth][8];
+  uint2 codes2[kDepth];
+  uint32_t byte[kDepth];
+  float s_dec[kDepth];
+  bool live[kDepth];
+  auto load = [&](int u) {
+    live[u] = w.r < rows;
+    if (live[u]) {
+      const int64_t r = w.r, cb = w.c, sb = MX ? (cb >> 1) : cb;
+      ldg256_stream(x + r * ld + cb * 16, raw[u]);
+      codes2[u] = __ldg(reinterpret_cast<const uint2*>(codes + r * (cols >> 1) + cb * 8));
+      byte[u] = __ldg(scales + (swz ? sf_swizzled_offset(r, sb, n_sb) : (r * n_sb + sb)));
+      s_dec[u] = per_row ? __ldg(global + 2 * r + 1) : s_dec_t;  // per_row: {amax, s_dec} per row
     }
-    const float scale = __fmul_rn(sf, per_row ? global[2 * r + 1] : s_dec_t);  // per_row: {amax, s_dec} per row
-    float e = 0.f, n = 0.f;
+    w.next();
+  };
 #pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      const float2 q = e2m1x2_values(((k < 4 ? c.x : c.y) >> (8 * (k & 3))) & 0xffu);
-      const float x0 = bf16_lo(raw[k]), x1 = bf16_hi(raw[k]);
-      const float d0 = x0 - q.x * scale, d1 = x1 - q.y * scale;
-      e = fmaf(d0, d0, e);
-      e = fmaf(d1, d1, e);
-      n = fmaf(x0, x0, n);
-      n = fmaf(x1, x1, n);
+  for (int u = 0; u < kDepth; ++u) load(u);
+  while (live[0]) {
+#pragma unroll
+    for (int u = 0; u < kDepth; ++u) {
+      if (live[u]) {
+        float sf;
+        if (MX) {
+          sf = byte[u] == 0 ? __uint_as_float(0x00400000u) : __uint_as_float(byte[u] << 23);  // 2^(byte - 127)
+        } else {
+          uint32_t h2;
+          asm("cvt.rn.f16x2.e4m3x2 %0, %1;" : "=r"(h2) : "h"((uint16_t)byte[u]));
+          sf = __half2float(__ushort_as_half((unsigned short)(h2 & 0xffffu)));
+        }
+        const float neg = -__fmul_rn(sf, s_dec[u]);
+        float2 e = make_float2(0.f, 0.f), n = e;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          const float2 q = e2m1x2_values(((k < 4 ? codes2[u].x : codes2[u].y) >> (8 * (k & 3))) & 0xffu);
+          const float2 xv = make_float2(bf16_lo(raw[u][k]), bf16_hi(raw[u][k]));
+          const float2 d = fma2(q, make_float2(neg, neg), xv);
+          e = fma2(d, d, e);
+          n = fma2(xv, xv, n);
+        }
+        err += (double)(e.x + e.y);
+        ref += (double)(n.x + n.y);
+      }
+      load(u);  // the slot's next chunk, while the other slots' are worked on
     }
-    err += (double)e;
-    ref += (double)n;
   }
   block_reduce_add(err, ref, out);
 }
@@ -123,26 +157,37 @@ __device__ __forceinline__ void load8(const void* base, int64_t elem, float (&v)
 }
 
 template <bool REF32, bool TEST32>
-__global__ void __launch_bounds__(256) sq_error_kernel(const void* __restrict__ refp, int64_t ld_ref,
+__global__ void __launch_bounds__(kThreads, 2) sq_error_kernel(const void* __restrict__ refp, int64_t ld_ref,
                                                        const void* __restrict__ testp, int64_t ld_test, int64_t rows,
                                                        int64_t cols, double* __restrict__ out) {
-  const int64_t n_c8 = cols >> 3, n_units = rows * n_c8;  // units of 8 elements
+  Walk w(blockIdx.x * (int64_t)blockDim.x + threadIdx.x, (int64_t)gridDim.x * blockDim.x, cols >> 3);  // units of 8
   double err = 0.0, ref = 0.0;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n_units; i += (int64_t)gridDim.x * blockDim.x) {
-    int64_t r, c8;
-    split_index(i, n_c8, r, c8);
-    float a[8], b[8];
-    load8<REF32>(refp, r * ld_ref + c8 * 8, a);
-    load8<TEST32>(testp, r * ld_test + c8 * 8, b);
-    float e = 0.f, n = 0.f;
+  constexpr int kDepth = 2;  // units whose loads are in flight together
+  float a[kDepth][8], b[kDepth][8];
+  bool live[kDepth];
+  while (w.r < rows) {
 #pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      const float d = a[k] - b[k];
-      e = fmaf(d, d, e);
-      n = fmaf(a[k], a[k], n);
+    for (int u = 0; u < kDepth; ++u) {
+      live[u] = w.r < rows;
+      if (live[u]) {
+        load8<REF32>(refp, w.r * ld_ref + w.c * 8, a[u]);
+        load8<TEST32>(testp, w.r * ld_test + w.c * 8, b[u]);
+      }
+      w.next();
     }
-    err += (double)e;
-    ref += (double)n;
+#pragma unroll
+    for (int u = 0; u < kDepth; ++u) {
+      if (!live[u]) continue;
+      float e = 0.f, n = 0.f;
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        const float d = a[u][k] - b[u][k];
+        e = fmaf(d, d, e);
+        n = fmaf(a[u][k], a[u][k], n);
+      }
+      err += (double)e;
+      ref += (double)n;
+    }
   }
   block_reduce_add(err, ref, out);
 }
@@ -153,7 +198,7 @@ cudaError_t grid_for(int64_t units, unsigned* grid) {
   if (e != cudaSuccess) return e;
   e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
-  const int64_t want = (units + 255) / 256, cap = (int64_t)sms * 8;  // eight resident CTAs per SM
+  const int64_t want = (units + kThreads - 1) / kThreads, cap = (int64_t)sms * 2;  // resident CTAs
   *grid = (unsigned)(want < cap ? (want > 0 ? want : 1) : cap);
   return cudaSuccess;
 }
@@ -173,7 +218,7 @@ cudaError_t launch_quant_error(const void* x, int64_t rows, int64_t cols, int64_
   if ((e = grid_for(rows * (cols >> 4), &grid)) != cudaSuccess) return e;
   const int swz = q.sf_layout == NVFP4_SF_SWIZZLED;
   e = launch_kernel(q.format == NVFP4_FORMAT_MXFP4 ? quant_error_kernel<true> : quant_error_kernel<false>, dim3(grid),
-                    dim3(256), 0, s, static_cast<const uint16_t*>(x), rows, cols, ld, q.codes, q.scales, q.global, swz,
+                    dim3(kThreads), 0, s, static_cast<const uint16_t*>(x), rows, cols, ld, q.codes, q.scales, q.global, swz,
                     q.format == NVFP4_FORMAT_NVFP4_ROWSCALE, out);
   count_launch();
   return e;
@@ -187,7 +232,7 @@ cudaError_t launch_sq_error(const void* ref, bool ref_fp32, int64_t ld_ref, cons
   if ((e = grid_for(rows * (cols >> 3), &grid)) != cudaSuccess) return e;
   auto kern = ref_fp32 ? (test_fp32 ? sq_error_kernel<true, true> : sq_error_kernel<true, false>)
                        : (test_fp32 ? sq_error_kernel<false, true> : sq_error_kernel<false, false>);
-  e = launch_kernel(kern, dim3(grid), dim3(256), 0, s, ref, ld_ref, test, ld_test, rows, cols, out);
+  e = launch_kernel(kern, dim3(grid), dim3(kThreads), 0, s, ref, ld_ref, test, ld_test, rows, cols, out);
   count_launch();
   return e;
 }

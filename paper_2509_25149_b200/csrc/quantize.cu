@@ -281,6 +281,23 @@ __device__ __forceinline__ float encode_scale_of_byte(uint32_t byte, float s_dec
   return (byte == 0u) ? 0.0f : fminf(__frcp_rn(d), kFltMax);
 }
 
+// Row-by-row scale bytes of a 128 x 8-block tile (staged [128][8]): as words where the row length keeps them aligned.
+// Row lengths are any number; otherwise the bytes leave one by one, but eight lanes write the eight bytes of a row: a warp's store touches four rows, not sixteen (four bytes of a row
+// per thread made the stores a microsecond of the tile's five).
+__device__ __forceinline__ void store_linear_scales(const uint8_t* src, uint8_t* dst, int64_t R0, int64_t K0, int64_t Rn,
+                                                    int64_t n_kb, bool full_tile) {
+  if (full_tile && (n_kb & 3) == 0) {
+    *reinterpret_cast<uint32_t*>(dst + (R0 + (threadIdx.x >> 1)) * n_kb + K0 + (threadIdx.x & 1) * 4) =
+        *reinterpret_cast<const uint32_t*>(src + threadIdx.x * 4);
+    return;
+  }
+  const int r = threadIdx.x >> 3, kb = threadIdx.x & 7;
+  uint8_t* d = dst + (R0 + r) * n_kb + K0 + kb;
+#pragma unroll
+  for (int p = 0; p < 4; ++p, d += 32 * n_kb)
+    if (full_tile || (R0 + r + 32 * p < Rn && K0 + kb < n_kb)) *d = src[threadIdx.x + 256 * p];
+}
+
 template <bool HAS_ROW, bool HAS_COL, bool BLOCK2D, bool RHT_ROW, bool RHT_COL, bool SR, bool SIDE = false>
 __global__ void __launch_bounds__(256, 2) quantize_kernel(const __grid_constant__ CUtensorMap src_map,
                                                           const __grid_constant__ CUtensorMap side_map,
@@ -585,25 +602,26 @@ __global__ void __launch_bounds__(256, 2) quantize_kernel(const __grid_constant_
 
     // ------------------------------------------------------------------ phase 3 ----
     if (HAS_COL) {
-      // a thread takes column pair cp and the 16-row groups (2m, 2m + 1): 16 bytes = 32 rows of each of its two columns
       const int64_t pitch = a.rows >> 1;  // bytes per row of the transposed copy
-      const bool vec16 = (a.rows & 31) == 0;
-      const int cp = threadIdx.x >> 2, m = threadIdx.x & 3;
-      const uint8_t* unit = col_codes + cp * 128 + ((((2 * m) ^ cp) & 7) << 4);
-      const uint4 g0 = *reinterpret_cast<const uint4*>(unit);  // group 2m: (first column, second column) x 8 bytes
-      const uint4 g1 = *reinterpret_cast<const uint4*>(reinterpret_cast<const uint8_t*>((uintptr_t)unit ^ 16));
-      const int64_t rr = row0 + 32 * m;
+      if ((a.rows & 31) == 0) {
+        // a thread takes column pair cp and the 16-row groups (2m, 2m + 1): 16 bytes = 32 rows of each of its two columns
+        const int cp = threadIdx.x >> 2, m = threadIdx.x & 3;
+        const uint8_t* unit = col_codes + cp * 128 + ((((2 * m) ^ cp) & 7) << 4);
+        const uint4 g0 = *reinterpret_cast<const uint4*>(unit);  // group 2m: (first column, second column) x 8 bytes
+        const uint4 g1 = *reinterpret_cast<const uint4*>(reinterpret_cast<const uint8_t*>((uintptr_t)unit ^ 16));
+        uint8_t* dst = a.c_codes + (col0 + 2 * cp) * pitch + (row0 >> 1) + m * 16;
+        if (full_tile || (row0 + 32 * m < a.rows && col0 + 2 * cp < a.cols)) {  // cols is even, rows % 32 == 0
+          *reinterpret_cast<uint4*>(dst) = make_uint4(g0.x, g0.y, g1.x, g1.y);
+          *reinterpret_cast<uint4*>(dst + pitch) = make_uint4(g0.z, g0.w, g1.z, g1.w);
+        }
+      } else {
+        // rows % 32 == 16: rows of the copy start on 8-byte boundaries; eight lanes write the 64 bytes of a column
 #pragma unroll
-      for (int odd = 0; odd < 2; ++odd) {
-        const int c = 2 * cp + odd;
-        if (col0 + c >= a.cols) continue;
-        const uint4 v = odd ? make_uint4(g0.z, g0.w, g1.z, g1.w) : make_uint4(g0.x, g0.y, g1.x, g1.y);
-        uint8_t* dst = a.c_codes + (col0 + c) * pitch + (row0 >> 1) + m * 16;
-        if (rr + 16 < a.rows && vec16) {
-          *reinterpret_cast<uint4*>(dst) = v;
-        } else {
-          if (rr < a.rows) *reinterpret_cast<uint2*>(dst) = make_uint2(v.x, v.y);
-          if (rr + 16 < a.rows) *reinterpret_cast<uint2*>(dst + 8) = make_uint2(v.z, v.w);
+        for (int p = 0; p < 4; ++p) {
+          const int c = (threadIdx.x >> 3) + 32 * p, q = threadIdx.x & 7, cp = c >> 1;
+          const uint2 v = *reinterpret_cast<const uint2*>(col_codes + cp * 128 + (((q ^ cp) & 7) << 4) + (c & 1) * 8);
+          if (full_tile || (row0 + 16 * q < a.rows && col0 + c < a.cols))
+            *reinterpret_cast<uint2*>(a.c_codes + (col0 + c) * pitch + (row0 >> 1) + q * 8) = v;
         }
       }
     }
@@ -627,12 +645,7 @@ __global__ void __launch_bounds__(256, 2) quantize_kernel(const __grid_constant_
           }
         }
       } else {
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          const int idx = threadIdx.x * 4 + k;
-          const int r = idx >> 3, kb = idx & 7;
-          if (R0 + r < Rn && K0 + kb < n_kb) dst[(R0 + r) * n_kb + K0 + kb] = src[idx];
-        }
+        store_linear_scales(src, dst, R0, K0, Rn, n_kb, full_tile);
       }
     }
     ++k;  // on to the CTA's next own tile

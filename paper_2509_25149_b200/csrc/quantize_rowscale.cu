@@ -4,9 +4,9 @@
 // dimension, so the GEMM can apply it in its epilogue as a vector; the transposed copy of the same tensor would need
 // a statistic over all source rows, i.e. the pass this variant exists to remove.
 //
-// CTAs of four warps.  A row of up to 5120 elements is held in the registers of ONE warp between the amax step and the
-// encoding (ten 16-element chunks per lane), a row of up to 10240 / 20480 elements in those of two / four warps, which
-// exchange their partial maxima through shared memory: one read from HBM in every case.  Longer rows are read a second
+// CTAs of four warps.  A row of up to 20480 elements is held in the registers of one, two or four warps between the amax
+// step and the encoding (two, five or ten 16-element chunks per lane); the warps of a row exchange their partial maxima
+// through shared memory: one read from HBM in every case.  Longer rows are read a second
 // time (from L1 / L2).  Eq. 1 per row, Eq. 2-4 as in the main quantizer; stochastic-rounding draws are keyed by the
 // element's position in the source, as everywhere.
 #include <cuda_bf16.h>
@@ -19,8 +19,6 @@
 namespace nvfp4 {
 
 namespace {
-
-constexpr int kKeep = 10;  // chunks of 16 elements a lane holds: 10 * 32 * 16 = 5120 elements per warp
 
 __device__ __forceinline__ void ldg256_cached(const void* p, uint32_t (&r)[8]) {
   const uint4 a = __ldg(reinterpret_cast<const uint4*>(p));
@@ -54,9 +52,13 @@ __device__ __forceinline__ void encode_chunk(const QuantArgs& a, const uint32_t 
   a.r_scales[a.r_swz ? sf_swizzled_offset(row, cb, n_cb) : (row * n_cb + cb)] = (uint8_t)byte;
 }
 
-// WPR warps per row (1, 2 or 4): warp w of the CTA holds chunks [(w % WPR) * 320, ...) of row (4 / WPR) * i + w / WPR.
-template <bool SR, int WPR>
-__global__ void __launch_bounds__(128, 4) quantize_rowscale_kernel(const QuantArgs a) {
+// CTAs resident per SM by what a lane keeps (registers)
+constexpr int ctas_per_sm(int keep) { return keep <= 2 ? 8 : keep <= 5 ? 6 : 4; }
+
+// WPR warps per row (1, 2 or 4): row (4 / WPR) * i + w / WPR of iteration i belongs to warp w, whose lanes take every WPR-th
+// group of 32 chunks, so that a row of any length is spread evenly.
+template <bool SR, int WPR, int kKeep>
+__global__ void __launch_bounds__(128, ctas_per_sm(kKeep)) quantize_rowscale_kernel(const QuantArgs a) {
   __shared__ float part[2][4];  // partial maxima, double-buffered across iterations
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   constexpr int kRowsPerCta = 4 / WPR;
@@ -72,7 +74,7 @@ __global__ void __launch_bounds__(128, 4) quantize_rowscale_kernel(const QuantAr
     uint32_t acc = 0;
 #pragma unroll
     for (int i = 0; i < kKeep; ++i) {
-      const int64_t cb = (int64_t)seg * (kKeep * 32) + lane + 32 * i;
+      const int64_t cb = lane + 32 * (seg + WPR * i);
       if (live && cb < n_cb) {
         ldg256_stream(src + cb * 16, keep[i]);
       } else {
@@ -100,7 +102,7 @@ __global__ void __launch_bounds__(128, 4) quantize_rowscale_kernel(const QuantAr
     if (live) {
 #pragma unroll
       for (int i = 0; i < kKeep; ++i) {
-        const int64_t cb = (int64_t)seg * (kKeep * 32) + lane + 32 * i;
+        const int64_t cb = lane + 32 * (seg + WPR * i);
         if (cb < n_cb) encode_chunk<SR>(a, keep[i], row, cb, n_cb, s_enc, s_dec);
       }
     }
@@ -155,20 +157,27 @@ __global__ void __launch_bounds__(256) quantize_rowscale_long_kernel(const Quant
   }
 }
 
+template <bool SR, int WPR, int KEEP>
+cudaError_t launch_kept(const QuantArgs& a, int sms, cudaStream_t s) {
+  const int64_t want = (a.rows * WPR + 3) / 4, cap = (int64_t)sms * ctas_per_sm(KEEP) * 4;  // up to four rounds of CTAs
+  quantize_rowscale_kernel<SR, WPR, KEEP><<<(unsigned)(want < cap ? want : cap), 128, 0, s>>>(a);
+  return cudaGetLastError();
+}
+
 template <bool SR>
 cudaError_t launch_t(const QuantArgs& a, int sms, cudaStream_t s) {
-  const int64_t per_warp = (int64_t)kKeep * 32 * 16;
-  if (a.cols > 4 * per_warp) {
-    const int64_t want = (a.rows + 7) / 8, cap = (int64_t)sms * 6;
-    quantize_rowscale_long_kernel<SR><<<(unsigned)(want < cap ? want : cap), 256, 0, s>>>(a);
-    return cudaGetLastError();
-  }
-  const int wpr = a.cols <= per_warp ? 1 : (a.cols <= 2 * per_warp ? 2 : 4);
-  const int64_t want = (a.rows * wpr + 3) / 4, cap = (int64_t)sms * 4 * 4;  // four CTAs per SM, four rounds
-  const unsigned grid = (unsigned)(want < cap ? want : cap);
-  if (wpr == 1) quantize_rowscale_kernel<SR, 1><<<grid, 128, 0, s>>>(a);
-  else if (wpr == 2) quantize_rowscale_kernel<SR, 2><<<grid, 128, 0, s>>>(a);
-  else quantize_rowscale_kernel<SR, 4><<<grid, 128, 0, s>>>(a);
+  // The fewest registers per lane that hold the row: more warps per SM are more bytes in flight.  Ten chunks per lane for
+  // every row up to 5120 elements left rows of 1024 waiting (16384 rows: 18.7 -> 10.8 us); 2560 15.7 -> 12.0 us (8192 rows),
+  // 5120 39.6 -> 37.9 us (16384 rows).  A row that fits one warp with five chunks does not gain from a second one (15.1 us).
+  const int64_t chunks = a.cols >> 4;
+  if (chunks <= 32 * 2) return launch_kept<SR, 1, 2>(a, sms, s);
+  if (chunks <= 32 * 4) return launch_kept<SR, 2, 2>(a, sms, s);
+  if (chunks <= 32 * 5) return launch_kept<SR, 1, 5>(a, sms, s);
+  if (chunks <= 32 * 10) return launch_kept<SR, 2, 5>(a, sms, s);
+  if (chunks <= 32 * 20) return launch_kept<SR, 4, 5>(a, sms, s);
+  if (chunks <= 32 * 40) return launch_kept<SR, 4, 10>(a, sms, s);
+  const int64_t want = (a.rows + 7) / 8, cap = (int64_t)sms * 6;
+  quantize_rowscale_long_kernel<SR><<<(unsigned)(want < cap ? want : cap), 256, 0, s>>>(a);
   return cudaGetLastError();
 }
 
