@@ -320,7 +320,7 @@ NVFP4_API nvfp4_status nvfp4_test_wait_timeout(uint64_t limit_ns, void* cuda_str
 
 /* Tuning knob: which GEMM tiling to use.  128 / 256 = one CTA per 128 x 128 / 128 x 256 output tile (256 needs
  * N % 256 == 0, otherwise 128 is used); CTA pairs: 640 = 256 x 128 tiles, 512 = 256 x 256 tiles, 768 = 256 x 384 tiles plus
- * up to two 256-wide ones per row of tiles (needs N >= 256 and per-tensor scales, otherwise as 512);
+ * up to two 256-wide ones per row of tiles (needs N >= 256, otherwise as 512);
  * 0 = choose by shape (the CTA-pair tile whose static schedule is estimated shortest).
  * Returns 0, or -1 for any other value.  Process-wide; results do not depend on it
  * beyond FP32 summation order. */

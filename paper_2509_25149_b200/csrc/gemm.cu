@@ -405,6 +405,10 @@ pair::Problem pair_problem(const GemmArgs& g) {
   return pair::Problem{g.M, g.N, g.K, g.sfa, g.sfb, g.a_global, g.b_global, g.d_is_fp32, g.accumulate, g.a_rows, g.b_rows};
 }
 
+bool has_row_scales(const GemmArgs& g0, const GemmArgs* g1) {
+  return g0.a_rows || g0.b_rows || (g1 && (g1->a_rows || g1->b_rows));
+}
+
 // tiles of a problem on CTA pairs with BN columns; the last one in either direction may be half outside
 inline int pair_tiles(const GemmArgs& g, int bn) { return ((g.M + 255) / 256) * ((g.N + bn - 1) / bn); }
 
@@ -448,7 +452,7 @@ cudaError_t launch_pair_t(const GemmArgs& g0, const void* a0, const void* b0, co
 cudaError_t launch_pair(const GemmArgs& g0, const void* a0, const void* b0, const GemmArgs* g1, const void* a1,
                         const void* b1, int bn, int num_sms, cudaStream_t s) {
   if (g1 && g1->mx != g0.mx) return cudaErrorInvalidValue;
-  if (g0.a_rows || g0.b_rows || (g1 && (g1->a_rows || g1->b_rows))) {
+  if (has_row_scales(g0, g1)) {
     if (g0.mx) return cudaErrorInvalidValue;
     return bn == 128 ? launch_pair_t<false, true, 128>(g0, a0, b0, g1, a1, b1, num_sms, s)
                      : launch_pair_t<false, true, 256>(g0, a0, b0, g1, a1, b1, num_sms, s);
@@ -473,13 +477,14 @@ bool wide_split(int N, int* n_wide, int* n_narrow) {
 
 bool wide_eligible(const GemmArgs& g) {
   int a, b;
-  return !g.a_rows && !g.b_rows && wide_split(g.N, &a, &b);
+  return wide_split(g.N, &a, &b);
 }
 
 wide::WProblem wide_problem(const GemmArgs& g) {
   int a = 0, b = 0;
   wide_split(g.N, &a, &b);
-  return wide::WProblem{g.M, g.N, g.K, g.sfa, g.sfb, g.a_global, g.b_global, g.d_is_fp32, g.accumulate, a, a + b};
+  return wide::WProblem{g.M, g.N, g.K, g.sfa, g.sfb, g.a_global, g.b_global, g.d_is_fp32, g.accumulate, a, a + b, g.a_rows,
+                        g.b_rows};
 }
 
 bool make_wide_maps(const GemmArgs& g, const void* a_codes, const void* b_codes, CUtensorMap* m) {
@@ -533,8 +538,10 @@ double pair_makespan(const GemmArgs* const* gs, int n_problems, int tile, int pa
 }
 
 // g1 == nullptr: one problem
-cudaError_t launch_wide(const GemmArgs& g0, const void* a0, const void* b0, const GemmArgs* g1, const void* a1,
-                        const void* b1, int num_sms, cudaStream_t s) {
+template <bool MX, bool ROWS>
+cudaError_t launch_wide_t(const GemmArgs& g0, const void* a0, const void* b0, const GemmArgs* g1, const void* a1,
+                          const void* b1, int num_sms, cudaStream_t s) {
+  auto kern = wide::gemm_wide_kernel<MX, ROWS>;
   CUtensorMap m[8];
   if (!make_wide_maps(g0, a0, b0, &m[0])) return cudaErrorInvalidValue;
   if (g1) {
@@ -542,15 +549,10 @@ cudaError_t launch_wide(const GemmArgs& g0, const void* a0, const void* b0, cons
   } else {
     for (int i = 0; i < 4; ++i) m[4 + i] = m[i];
   }
-  if (g1 && g1->mx != g0.mx) return cudaErrorInvalidValue;
-  static std::atomic<uint64_t> configured{0};  // per device
+  static std::atomic<uint64_t> configured{0};  // per call site (template instantiation) and device
   int dev;
   if (device_needs_config(configured, &dev)) {
-    cudaError_t e = cudaFuncSetAttribute(wide::gemm_wide_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         wide::kWSmemBytes);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(wide::gemm_wide_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             wide::kWSmemBytes);
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, wide::kWSmemBytes);
     if (e != cudaSuccess) return e;
     device_configured(configured, dev);
   }
@@ -561,14 +563,19 @@ cudaError_t launch_wide(const GemmArgs& g0, const void* a0, const void* b0, cons
   a.n_tiles = a.n_tiles0 + (g1 ? ((g1->M + 255) / 256) * a.p[1].tiles_n : 0);
   const int max_pairs = num_sms / 2;
   const int pairs = a.n_tiles < max_pairs ? a.n_tiles : max_pairs;
-  const dim3 grid(2 * pairs), block(wide::kWThreads);
-  const cudaError_t le =
-      g0.mx ? launch_kernel(wide::gemm_wide_kernel<true>, grid, block, wide::kWSmemBytes, s, m[0], m[1],
-                            m[2], m[3], m[4], m[5], m[6], m[7], a)
-            : launch_kernel(wide::gemm_wide_kernel<false>, grid, block, wide::kWSmemBytes, s, m[0], m[1],
-                            m[2], m[3], m[4], m[5], m[6], m[7], a);
+  const cudaError_t le = launch_kernel(kern, dim3(2 * pairs), dim3(wide::kWThreads), wide::kWSmemBytes, s, m[0], m[1], m[2],
+                                       m[3], m[4], m[5], m[6], m[7], a);
   count_launch();
   return le;
+}
+
+cudaError_t launch_wide(const GemmArgs& g0, const void* a0, const void* b0, const GemmArgs* g1, const void* a1,
+                        const void* b1, int num_sms, cudaStream_t s) {
+  if (g1 && g1->mx != g0.mx) return cudaErrorInvalidValue;
+  if (has_row_scales(g0, g1))
+    return g0.mx ? cudaErrorInvalidValue : launch_wide_t<false, true>(g0, a0, b0, g1, a1, b1, num_sms, s);
+  return g0.mx ? launch_wide_t<true, false>(g0, a0, b0, g1, a1, b1, num_sms, s)
+               : launch_wide_t<false, false>(g0, a0, b0, g1, a1, b1, num_sms, s);
 }
 
 }  // namespace
@@ -577,7 +584,7 @@ cudaError_t launch_gemm(const GemmArgs& g, const void* a_codes, const void* b_co
   int num_sms = 0;
   cudaError_t e = sm_count(&num_sms);
   if (e != cudaSuccess) return e;
-  const bool rows = g.a_rows || g.b_rows;  // scale vectors: the pair kernel's epilogue only
+  const bool rows = has_row_scales(g, nullptr);  // scale vectors: the pair kernels' epilogues only
   if (tile == kTileWide && wide_eligible(g)) return launch_wide(g, a_codes, b_codes, nullptr, nullptr, nullptr, num_sms, s);
   if (tile >= kTilePair256 || rows)
     return launch_pair(g, a_codes, b_codes, nullptr, nullptr, nullptr, tile == kTilePair128 ? 128 : 256, num_sms, s);

@@ -16,14 +16,14 @@ struct GemmArgs {
   int d_is_fp32, accumulate;
   int mx;                 // operands are MXFP4 (UE8M0 scale per 32 elements) instead of NVFP4
   const float* a_rows;    // per-row {amax, s_dec} pairs of A / B when their global scale is taken per row, else NULL
-  const float* b_rows;    // (CTA-pair kernel with 256 x 256 tiles only)
+  const float* b_rows;    // (CTA-pair kernels only)
 };
 
 // Tiles: 128 or 256 = one CTA per 128 x 128 / 128 x 256 tile (256 needs N % 256 == 0, otherwise 128 is used); the others
 // run on CTA pairs and take any M and N that are multiples of 128 (a half beyond the edge is computed on zeros and clipped).
 constexpr int kTilePair256 = 512;  // 256 x 256
 constexpr int kTilePair128 = 640;  // 256 x 128
-constexpr int kTileWide = 768;     // 256 x 384, needs N >= 256 and tensor-level scales
+constexpr int kTileWide = 768;     // 256 x 384, needs N >= 256
 cudaError_t launch_gemm(const GemmArgs& g, const void* a_codes, const void* b_codes, int tile, cudaStream_t s);
 // Two independent GEMMs in one launch of a CTA-pair kernel: the tiles of g0 are worked through first, then those of g1,
 // on one persistent grid.

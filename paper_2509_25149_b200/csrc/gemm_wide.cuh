@@ -34,7 +34,8 @@ constexpr int kWSfaBytes = 4 * 512;
 constexpr int kWSfbBytes = 12 * 512;  // three 128-row groups x four K64 steps
 constexpr int kWStageBytes = kWABytes + kWBBytes + kWSfaBytes + kWSfbBytes;  // 48 KB
 constexpr int kWStagingBytes = 2 * 16384;
-constexpr int kWSmemBytes = kWStages * kWStageBytes + kWStagingBytes + 1024 /*alignment*/ + 256 /*barriers*/;
+constexpr int kWBetaBytes = 384 * 4;  // column scales of the tile, one half per epilogue group (row-scaled B)
+constexpr int kWSmemBytes = kWStages * kWStageBytes + kWStagingBytes + 1024 /*alignment*/ + 256 /*barriers*/ + kWBetaBytes;
 constexpr uint32_t kWTmemCols = 512;
 constexpr int kWSfCol = 384;      // after the accumulator columns
 constexpr int kWSfSlotCols = 64;  // SFA 4 x 4, SFB 4 x 12
@@ -51,6 +52,8 @@ struct WProblem {
   int d_is_fp32, accumulate;
   int n_wide;   // 384-wide column tiles (they come first)
   int tiles_n;  // all column tiles
+  const float* a_rows;  // {amax, s_dec} pairs per row of the operand, or NULL (see pair::Problem)
+  const float* b_rows;
 };
 struct WArgs {
   WProblem p[2];
@@ -66,10 +69,11 @@ struct WArgs {
 // other half) may still be in flight, so the tensor-memory reads between the chunks do not wait for a store.  (The same
 // scheme for bf16 outputs, with 32-column chunks, was measured slower than the single buffer: twice the barriers and
 // stores of half the width.)  n_chunks counts the group's fp32 chunks; the caller drains all stores before a tile.
-template <bool FP32>
+// BETA: the columns additionally carry their own factors (float[64] in shared memory at `beta`).
+template <bool FP32, bool BETA = false>
 __device__ __forceinline__ void store_cols64(const uint32_t (&r)[64], float alpha, int et, int bar_id, int row_in_tile,
                                              uint32_t stage_buf16k, uint32_t& n_chunks, const CUtensorMap* map_d, int x0,
-                                             int row0, int accumulate) {
+                                             int row0, int accumulate, const float* beta = nullptr) {
   if (FP32) {
 #pragma unroll
     for (int c = 0; c < 4; ++c, ++n_chunks) {
@@ -81,7 +85,11 @@ __device__ __forceinline__ void store_cols64(const uint32_t (&r)[64], float alph
       for (int j = 0; j < 4; ++j) {
         uint32_t p[4];
 #pragma unroll
-        for (int e = 0; e < 4; ++e) p[e] = __float_as_uint(__uint_as_float(r[c * 16 + 4 * j + e]) * alpha);
+        for (int e = 0; e < 4; ++e) {
+          float v = __uint_as_float(r[c * 16 + 4 * j + e]) * alpha;
+          if (BETA) v *= beta[c * 16 + 4 * j + e];
+          p[e] = __float_as_uint(v);
+        }
         // 64-byte swizzle: the 16-byte unit index is XORed with bits 7-8 of the address, i.e. with (row >> 1) & 3
         asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(srow + ((j ^ ((row_in_tile >> 1) & 3)) << 4)),
                      "r"(p[0]), "r"(p[1]), "r"(p[2]), "r"(p[3])
@@ -106,8 +114,12 @@ __device__ __forceinline__ void store_cols64(const uint32_t (&r)[64], float alph
       uint32_t p[4];
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
-        __nv_bfloat162 h = __floats2bfloat162_rn(__uint_as_float(r[8 * j + 2 * e]) * alpha,
-                                                 __uint_as_float(r[8 * j + 2 * e + 1]) * alpha);
+        float v0 = __uint_as_float(r[8 * j + 2 * e]) * alpha, v1 = __uint_as_float(r[8 * j + 2 * e + 1]) * alpha;
+        if (BETA) {
+          v0 *= beta[8 * j + 2 * e];
+          v1 *= beta[8 * j + 2 * e + 1];
+        }
+        __nv_bfloat162 h = __floats2bfloat162_rn(v0, v1);
         p[e] = *reinterpret_cast<uint32_t*>(&h);
       }
       asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(srow + ((j ^ (row_in_tile & 7)) << 4)), "r"(p[0]),
@@ -123,7 +135,8 @@ __device__ __forceinline__ void store_cols64(const uint32_t (&r)[64], float alph
   }
 }
 
-template <bool MX>
+// ROWS = true: an operand carries its global scale per row (a separate instantiation, as in the pair kernel).
+template <bool MX, bool ROWS = false>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kWThreads, 1)
     gemm_wide_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant__ CUtensorMap map_b0,
                      const __grid_constant__ CUtensorMap map_c0, const __grid_constant__ CUtensorMap map_d0,
@@ -371,8 +384,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kWThreads, 1)
     const int et = (threadIdx.x - 96) & 127;  // 0..127 inside the group
     const int bar_id = 1 + half;
     uint32_t acc_phase = 0;
-    const float alpha0 = __fmul_rn(g.p[0].a_global[1], g.p[0].b_global[1]);
-    const float alpha1 = __fmul_rn(g.p[1].a_global[1], g.p[1].b_global[1]);
+    // per-tensor decode scales; an operand with per-row scales contributes 1 here and its vector below
+    const float alpha0 = __fmul_rn((ROWS && g.p[0].a_rows) ? 1.f : g.p[0].a_global[1], (ROWS && g.p[0].b_rows) ? 1.f : g.p[0].b_global[1]);
+    const float alpha1 = __fmul_rn((ROWS && g.p[1].a_rows) ? 1.f : g.p[1].a_global[1], (ROWS && g.p[1].b_rows) ? 1.f : g.p[1].b_global[1]);
+    float* const beta = reinterpret_cast<float*>(base_ptr + kWStages * kWStageBytes + kWStagingBytes + 256) + half * 192;
     const uint32_t acce_leader = map_to_cta(acce_bar, 0);
     const int row_in_tile = quad * 32 + lane;
     const uint32_t stage_bufs = staging + half * 16384;
@@ -381,9 +396,16 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kWThreads, 1)
       int prob, m_blk, n0, width;
       tile_coords(tile, prob, m_blk, n0, width);
       const CUtensorMap* map_d = prob ? &map_d1 : &map_d0;
-      const float alpha = prob ? alpha1 : alpha0;
+      float alpha = prob ? alpha1 : alpha0;
       const int d_is_fp32 = g.p[prob].d_is_fp32, accumulate = g.p[prob].accumulate;
       const int cols_half = width >> 1, passes = cols_half >> 6;  // 192 / 3 or 128 / 2
+      const float* b_rows = ROWS ? g.p[prob].b_rows : nullptr;
+      if (ROWS && g.p[prob].a_rows)
+        alpha *= g.p[prob].a_rows[2 * (int64_t)(m_blk * 256 + (int)rank * 128 + row_in_tile) + 1];
+      // the group's column factors; the barriers inside store_cols64 order this write before their use and their last use
+      // before the next tile's write
+      if (b_rows)
+        for (int c = et; c < cols_half; c += 128) beta[c] = b_rows[2 * (int64_t)(n0 + half * cols_half + c) + 1];
       mbar_wait_cluster(accf_bar, acc_phase, abort_flag, 0x400u);
       // agree on giving up: a warp that timed out still joins this barrier, and all 128 threads take ONE decision
       if (group_gave_up(abort_flag, bar_id, 128)) break;
@@ -404,10 +426,18 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kWThreads, 1)
           if (lane == 0) mbar_arrive_cluster(acce_leader);
         }
         const int x0 = n0 + half * cols_half + p * 64;
-        if (d_is_fp32)
+        if (ROWS && b_rows) {
+          if (d_is_fp32)
+            store_cols64<true, ROWS>(r, alpha, et, bar_id, row_in_tile, stage_bufs, n_chunks, map_d, x0, row0, accumulate,
+                                     beta + p * 64);
+          else
+            store_cols64<false, ROWS>(r, alpha, et, bar_id, row_in_tile, stage_bufs, n_chunks, map_d, x0, row0, accumulate,
+                                      beta + p * 64);
+        } else if (d_is_fp32) {
           store_cols64<true>(r, alpha, et, bar_id, row_in_tile, stage_bufs, n_chunks, map_d, x0, row0, accumulate);
-        else
+        } else {
           store_cols64<false>(r, alpha, et, bar_id, row_in_tile, stage_bufs, n_chunks, map_d, x0, row0, accumulate);
+        }
       }
       acc_phase ^= 1u;
     }

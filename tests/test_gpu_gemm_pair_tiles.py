@@ -101,3 +101,30 @@ def test_bf16_ragged_on_both_tiles(shape, layouts, fp32):
         B.nvfp4_gemm_bf16(a, b, D, *layouts, accumulate=True)
         B.nvfp4_device_status()
         assert torch.equal(D, once + once)
+
+
+@pytest.mark.parametrize("shape", [(256, 256, 256), (256, 768, 512), (512, 1280, 1024)])
+@pytest.mark.parametrize("tile", [512, 640, 768])
+@pytest.mark.parametrize("rows_on", ["A", "B", "AB"])
+@pytest.mark.parametrize("fp32", [False, True])
+def test_scale_vectors_on_every_pair_tile(shape, tile, rows_on, fp32):
+    M, N, K = shape
+
+    def operand(R, per_row, seed):
+        x = synth.normal_bf16((R, K), 1.0, seed)
+        x *= torch.exp2(torch.arange(R) % 13 - 6).to(torch.bfloat16)[:, None]  # rows far apart: a mixed-up factor shows
+        t = B.alloc_tensor(R, K, format=B.FORMAT_NVFP4_ROWSCALE if per_row else B.FORMAT_NVFP4)
+        B.nvfp4_quantize(x.cuda(), B.quant_opts(), t, None)
+        return t
+
+    A, Bt = operand(M, "A" in rows_on, 3), operand(N, "B" in rows_on, 4)
+    a, b = (B.nvfp4_dequantize(t).double() for t in (A, Bt))
+    D = torch.full((M, N), float("nan"), dtype=torch.float32 if fp32 else torch.bfloat16, device="cuda")
+    B.nvfp4_set_gemm_tile_n(tile)
+    try:
+        B.nvfp4_gemm(A, Bt, D)
+        B.nvfp4_device_status()
+    finally:
+        B.nvfp4_set_gemm_tile_n(0)
+    P.assert_gemm_close(D.float().cpu().numpy(), (a @ b.T).cpu().numpy(), (a.abs() @ b.abs().T).cpu().numpy(), not fp32,
+                        f"rows {rows_on} tile {tile}")
