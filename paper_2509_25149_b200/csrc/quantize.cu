@@ -232,8 +232,8 @@ __global__ void __launch_bounds__(256) amax_rot_col_kernel(const uint16_t* __res
 }
 
 // ---------------------------------------------------------------------------------------------
-// Pass 2: persistent CTAs (two per SM), each working through 128 x 128 tiles of the source.  The tiles arrive by
-// TMA (cp.async.bulk.tensor, this GPU's memory, no multicast) in a ring of two 32 KB buffers: the load of tile
+// Pass 2: persistent CTAs (two per SM), each working through tiles of 128 rows x 128 (few tiles: 64) columns of the source.
+// The tiles arrive by TMA (cp.async.bulk.tensor, this GPU's memory, no multicast) in a ring of two buffers: the load of tile
 // k + 2 is issued as soon as tile k has been consumed, so a tile is in flight during the whole of the previous one;
 // out-of-range parts of a ragged tile are zero-filled by the copy.
 //   set-up   once per CTA: Eq. 1, and the table  E4M3 byte -> encode scale  of each copy (the text after Eq. 3:
@@ -248,21 +248,27 @@ __global__ void __launch_bounds__(256) amax_rot_col_kernel(const uint16_t* __res
 // buffered, so a tile needs one CTA barrier.  Tiles are visited in reverse order so that the end of the tensor,
 // which pass 1 touched last, is read first while it may still sit in L2.
 // ---------------------------------------------------------------------------------------------
+// TC: columns of a tile.
+template <int TC>
 struct QuantSmem {
-  static constexpr int kTile = 0;                     // 2 x (128 rows x 256 B of bf16), filled by TMA
-  static constexpr int kColCodes = 65536;             // 2 x (128 columns x 64 B)
-  static constexpr int kSfRow = kColCodes + 2 * 8192; // 2 x 1 KB
-  static constexpr int kSfCol = kSfRow + 2 * 1024;    // 2 x 1 KB
-  static constexpr int kBlkEnc = kSfCol + 2 * 1024;   // 64 floats (16x16 mode)
-  static constexpr int kBlkByte = kBlkEnc + 256;      // 64 bytes
-  static constexpr int kGlobalScales = kBlkByte + 64; // s_enc, s_dec of the row-wise and the column-wise copy
-  static constexpr int kEncRow = kGlobalScales + 64;  // 128 floats: encode scale by E4M3 byte, row-wise copy
-  static constexpr int kEncCol = kEncRow + 512;       // the same for the transposed copy
-  static constexpr int kBars = kEncCol + 512;         // two "tile landed" barriers, then the abort word
-  static constexpr int kRand = kBars + 32;            // 128 rows x 128 B of complemented draws (stochastic rounding),
-                                                      // or 128 rows x 64 B of row-wise codes (16x16 blocks, both copies)
-  static constexpr int kTileBytes = 32768;
-  static constexpr int bytes(bool rand, bool row_codes) { return kRand + (rand ? 16384 : row_codes ? 8192 : 0); }
+  static constexpr int kChunks = TC / 16;                // 1x16 chunks per tile row
+  static constexpr int kRow = 2 * TC;                    // bytes per tile row
+  static constexpr int kTileBytes = 128 * kRow;
+  static constexpr int kTile = 0;                        // 2 tiles of bf16, filled by TMA
+  static constexpr int kColBytes = TC * 64;
+  static constexpr int kColCodes = 2 * kTileBytes;       // 2 x (TC columns x 64 B)
+  static constexpr int kSfBytes = 8 * TC;                // 128 rows x kChunks bytes, or TC columns x 8
+  static constexpr int kSfRow = kColCodes + 2 * kColBytes;
+  static constexpr int kSfCol = kSfRow + 2 * kSfBytes;
+  static constexpr int kBlkEnc = kSfCol + 2 * kSfBytes;  // 64 floats (16x16 mode)
+  static constexpr int kBlkByte = kBlkEnc + 256;         // 64 bytes
+  static constexpr int kGlobalScales = kBlkByte + 64;    // s_enc, s_dec of the row-wise and the column-wise copy
+  static constexpr int kEncRow = kGlobalScales + 64;     // 128 floats: encode scale by E4M3 byte, row-wise copy
+  static constexpr int kEncCol = kEncRow + 512;          // the same for the transposed copy
+  static constexpr int kBars = kEncCol + 512;            // two "tile landed" barriers, then the abort word
+  static constexpr int kRand = kBars + 32;               // 128 rows x TC B of complemented draws (stochastic rounding),
+                                                         // or 128 rows x TC / 2 B of row-wise codes (16x16, both copies)
+  static constexpr int bytes(bool rand, bool row_codes) { return kRand + (rand ? 128 * TC : row_codes ? 64 * TC : 0); }
 };
 
 // Eq. 2-3: the stored E4M3 byte of a block, S_b = e4m3(fl(fl(amax_b / 6) * s_enc))
@@ -281,27 +287,34 @@ __device__ __forceinline__ float encode_scale_of_byte(uint32_t byte, float s_dec
   return (byte == 0u) ? 0.0f : fminf(__frcp_rn(d), kFltMax);
 }
 
-// Row-by-row scale bytes of a 128 x 8-block tile (staged [128][8]): as words where the row length keeps them aligned.
-// Row lengths are any number; otherwise the bytes leave one by one, but eight lanes write the eight bytes of a row: a warp's store touches four rows, not sixteen (four bytes of a row
+// Row-by-row scale bytes of a tile of ROWS x KB blocks (staged row by row): as words where the row length keeps them aligned.
+// Row lengths are any number; otherwise the bytes leave one by one, but neighbouring lanes write the bytes of a row: a warp's store touches four rows, not sixteen (four bytes of a row
 // per thread made the stores a microsecond of the tile's five).
+template <int ROWS, int KB>
 __device__ __forceinline__ void store_linear_scales(const uint8_t* src, uint8_t* dst, int64_t R0, int64_t K0, int64_t Rn,
                                                     int64_t n_kb, bool full_tile) {
   if (full_tile && (n_kb & 3) == 0) {
-    *reinterpret_cast<uint32_t*>(dst + (R0 + (threadIdx.x >> 1)) * n_kb + K0 + (threadIdx.x & 1) * 4) =
-        *reinterpret_cast<const uint32_t*>(src + threadIdx.x * 4);
+    if (threadIdx.x < ROWS * KB / 4)
+      *reinterpret_cast<uint32_t*>(dst + (R0 + threadIdx.x / (KB / 4)) * n_kb + K0 + threadIdx.x % (KB / 4) * 4) =
+          *reinterpret_cast<const uint32_t*>(src + threadIdx.x * 4);
     return;
   }
-  const int r = threadIdx.x >> 3, kb = threadIdx.x & 7;
+  const int r = threadIdx.x / KB, kb = threadIdx.x % KB;
   uint8_t* d = dst + (R0 + r) * n_kb + K0 + kb;
 #pragma unroll
-  for (int p = 0; p < 4; ++p, d += 32 * n_kb)
-    if (full_tile || (R0 + r + 32 * p < Rn && K0 + kb < n_kb)) *d = src[threadIdx.x + 256 * p];
+  for (int p = 0; p < ROWS * KB / 256; ++p, d += 256 / KB * n_kb)
+    if (full_tile || (R0 + r + 256 / KB * p < Rn && K0 + kb < n_kb)) *d = src[threadIdx.x + 256 * p];
 }
 
-template <bool HAS_ROW, bool HAS_COL, bool BLOCK2D, bool RHT_ROW, bool RHT_COL, bool SR, bool SIDE = false>
+template <bool HAS_ROW, bool HAS_COL, bool BLOCK2D, bool RHT_ROW, bool RHT_COL, bool SR, bool SIDE, int TC>
 __global__ void __launch_bounds__(256, 2) quantize_kernel(const __grid_constant__ CUtensorMap src_map,
                                                           const __grid_constant__ CUtensorMap side_map,
                                                           const QuantArgs a) {
+  using S = QuantSmem<TC>;
+  constexpr int CH = S::kChunks;          // chunks per tile row
+  constexpr int RPP = 32 / CH;            // rows a warp covers with one chunk per lane; chunk i of a lane: RPP * i rows down
+  constexpr int NP = 16 / RPP;            // chunks per lane
+  constexpr int NIT = TC / 64;            // column pairs per lane in phase 2
   extern __shared__ __align__(128) uint8_t smem[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int n_cb = (int)(a.cols >> 4);  // 16-blocks per source row
@@ -309,8 +322,8 @@ __global__ void __launch_bounds__(256, 2) quantize_kernel(const __grid_constant_
   // 16x16 blocks with both copies requested: the transposed copy holds the very codes of the row-wise one
   // (Section 4.3), so it is made by transposing nibbles; the raw tile is not needed a second time
   constexpr bool kNibbleTranspose = BLOCK2D && HAS_ROW && HAS_COL;
-  volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(smem + QuantSmem::kBars + 16);
-  const uint32_t bar0 = smem_u32(smem + QuantSmem::kBars), tile0 = smem_u32(smem + QuantSmem::kTile);
+  volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(smem + S::kBars + 16);
+  const uint32_t bar0 = smem_u32(smem + S::kBars), tile0 = smem_u32(smem + S::kTile);
 
   const int total = a.tiles_r * a.tiles_c, stride = (int)gridDim.x;
   const int first = total - 1 - (int)blockIdx.x;         // this CTA's tiles: first, first - stride, ...
@@ -326,14 +339,14 @@ __global__ void __launch_bounds__(256, 2) quantize_kernel(const __grid_constant_
     return SIDE && sk < m_mine && (k >= n_mine || (long long)sk * n_mine < (long long)k * m_mine);
   };
   auto issue_load = [&](int j, int k, int sk) {  // job j (own tile k or side tile sk) into buffer j & 1 (one thread)
-    const uint32_t bar = bar0 + 8 * (j & 1), dst = tile0 + (j & 1) * QuantSmem::kTileBytes;
-    mbar_expect_tx(bar, QuantSmem::kTileBytes);
+    const uint32_t bar = bar0 + 8 * (j & 1), dst = tile0 + (j & 1) * S::kTileBytes;
+    mbar_expect_tx(bar, S::kTileBytes);
     if (side_next(k, sk)) {
       const int t = (int)blockIdx.x + sk * stride, tr = t / a.side_tiles_c, tc = t - tr * a.side_tiles_c;
-      tma_load_2d(dst, &side_map, tc * 128, tr * 128, bar);
+      tma_load_2d(dst, &side_map, tc * TC, tr * 128, bar);
     } else {
       const int t = first - k * stride, tr = t / a.tiles_c, tc = t - tr * a.tiles_c;
-      tma_load_2d(dst, &src_map, tc * 128, tr * 128, bar);
+      tma_load_2d(dst, &src_map, tc * TC, tr * 128, bar);
     }
   };
   int ahead_k = 0, ahead_sk = 0;  // thread 0: own / side tiles among the jobs already issued
@@ -343,7 +356,7 @@ __global__ void __launch_bounds__(256, 2) quantize_kernel(const __grid_constant_
   };
 
   // ------------------------------------------------------------------ set-up ----
-  float* g_sc = reinterpret_cast<float*>(smem + QuantSmem::kGlobalScales);
+  float* g_sc = reinterpret_cast<float*>(smem + S::kGlobalScales);
   if (threadIdx.x == 0) {
     mbar_init(bar0, 1);
     mbar_init(bar0 + 8, 1);
@@ -376,46 +389,50 @@ __global__ void __launch_bounds__(256, 2) quantize_kernel(const __grid_constant_
   __syncthreads();
   griddep_launch_dependents();
   const float r_senc = g_sc[0], r_sdec = g_sc[1], c_senc = g_sc[2], c_sdec = g_sc[3];
-  const float* enc_row = reinterpret_cast<const float*>(smem + QuantSmem::kEncRow);
-  const float* enc_col = reinterpret_cast<const float*>(smem + QuantSmem::kEncCol);
+  const float* enc_row = reinterpret_cast<const float*>(smem + S::kEncRow);
+  const float* enc_col = reinterpret_cast<const float*>(smem + S::kEncCol);
   if (!BLOCK2D) {
     // with the transform the kernel works on 4 * y: the 1/4 is folded into the block amax and the encode scale (exact)
     if (threadIdx.x < 128) {
       if (HAS_ROW)
-        reinterpret_cast<float*>(smem + QuantSmem::kEncRow)[threadIdx.x] =
+        reinterpret_cast<float*>(smem + S::kEncRow)[threadIdx.x] =
             encode_scale_of_byte(threadIdx.x, r_sdec) * (RHT_ROW ? 0.25f : 1.0f);
     } else {
       if (HAS_COL)
-        reinterpret_cast<float*>(smem + QuantSmem::kEncCol)[threadIdx.x - 128] =
+        reinterpret_cast<float*>(smem + S::kEncCol)[threadIdx.x - 128] =
             encode_scale_of_byte(threadIdx.x - 128, c_sdec) * (RHT_COL ? 0.25f : 1.0f);
     }
     __syncthreads();
   }
 
-  // per-thread constants of phase 1: chunk column cb, row rl + 4 i for chunk i
-  const int cb = lane & 7, rl = warp * 16 + (lane >> 3);
-  const uint32_t tile_ld = rl * 256 + cb * 32;     // chunk i of the thread inside a tile buffer: + 1024 i
-  const uint32_t rand_st = QuantSmem::kRand + rl * 128 + cb * 16;  // + 512 i
-  const int sf_row_pos = a.r_swz ? ((cb >> 2) * 512 + (rl & 31) * 16 + (rl >> 5) * 4 + (cb & 3)) : (rl * 8 + cb);
-  const int sf_row_step = a.r_swz ? 64 : 32;
+  // per-thread constants of phase 1: chunk column cb, row rl + RPP * i for chunk i
+  const int cb = lane % CH, rl = warp * 16 + lane / CH;
+  const uint32_t tile_ld = rl * S::kRow + cb * 32;     // chunk i of the thread inside a tile buffer: + RPP * kRow * i
+  const uint32_t rand_st = S::kRand + rl * TC + cb * 16;  // + RPP * TC * i
+  const int sf_row_pos = a.r_swz ? ((cb >> 2) * 512 + (rl & 31) * 16 + (rl >> 5) * 4 + (cb & 3)) : (rl * CH + cb);
+  const int sf_row_step = a.r_swz ? RPP * 16 : RPP * CH;
   const int64_t r_pitch = a.cols >> 1;  // bytes per row of the row-wise codes
 
   // hoisted constants of phase 2: where a thread stages its two columns' codes and scale bytes (iteration it, column
   // parity odd); the 16-byte unit of column pair cp and 16-row group q sits at cp * 128 + ((q ^ cp) & 7) * 16
   const int col_codes_st = lane * 128 + (((warp ^ lane) & 7) << 4);  // + 4096 it
-  const int sf_col_pos = a.c_swz ? ((warp >> 2) * 512 + (lane & 15) * 32 + (lane >> 4) * 4 + (warp & 3)) : (lane * 16 + warp);
-  const int sf_col_odd = a.c_swz ? 16 : 8, sf_col_it = a.c_swz ? 8 : 512;
+  // scale bytes of the transposed copy: two whole atoms (TC = 128) or half of the rows of two atoms (TC = 64: 8 bytes of
+  // each 16)
+  constexpr int kAtomRow = TC == 128 ? 16 : 8;
+  const int sf_col_pos = a.c_swz ? ((warp >> 2) * (32 * kAtomRow) + (lane & 15) * (2 * kAtomRow) + (lane >> 4) * 4 + (warp & 3))
+                                 : (lane * 16 + warp);
+  const int sf_col_odd = a.c_swz ? kAtomRow : 8, sf_col_it = a.c_swz ? 8 : 512;
 
   const int step_r = stride / a.tiles_c, step_c = stride - step_r * a.tiles_c;  // tile coordinates move by these
   int tr = first >= 0 ? first / a.tiles_c : 0, tc = first >= 0 ? first - tr * a.tiles_c : 0;
   int k = 0, sk = 0, j = 0;  // own tiles done, side tiles done, jobs done (the ring position)
   uint32_t side_acc = 0;     // |.| maximum of the side tiles, two bf16 lanes
   for (; j < n_jobs; ++j) {
-    const uint8_t* const tile_buf = smem + QuantSmem::kTile + (j & 1) * QuantSmem::kTileBytes;
+    const uint8_t* const tile_buf = smem + S::kTile + (j & 1) * S::kTileBytes;
     quant_wait(bar0 + 8 * (j & 1), (uint32_t)(j >> 1) & 1u, abort_flag, a.status);  // the tile has landed
     if (SIDE && side_next(k, sk)) {
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {  // zero fill outside the tensor leaves the maximum alone
+      for (int i = 0; i < S::kTileBytes / 4096; ++i) {  // zero fill outside the tensor leaves the maximum alone
         const uint4 v = *reinterpret_cast<const uint4*>(tile_buf + i * 4096 + threadIdx.x * 16);
         side_acc = absmax_bf16x2(absmax_bf16x2(side_acc, v.x), v.y);
         side_acc = absmax_bf16x2(absmax_bf16x2(side_acc, v.z), v.w);
@@ -427,22 +444,22 @@ __global__ void __launch_bounds__(256, 2) quantize_kernel(const __grid_constant_
       continue;
     }
     const int buf = k & 1;  // staging buffers alternate with the CTA's own tiles
-    const int64_t row0 = (int64_t)tr * 128, col0 = (int64_t)tc * 128;
-    const bool full_tile = (row0 + 128 <= a.rows) && (col0 + 128 <= a.cols);
-    uint8_t* const col_codes = smem + QuantSmem::kColCodes + buf * 8192;
-    uint8_t* const sf_row = smem + QuantSmem::kSfRow + buf * 1024;
-    uint8_t* const sf_col = smem + QuantSmem::kSfCol + buf * 1024;
+    const int64_t row0 = (int64_t)tr * 128, col0 = (int64_t)tc * TC;
+    const bool full_tile = (row0 + 128 <= a.rows) && (col0 + TC <= a.cols);
+    uint8_t* const col_codes = smem + S::kColCodes + buf * S::kColBytes;
+    uint8_t* const sf_row = smem + S::kSfRow + buf * S::kSfBytes;
+    uint8_t* const sf_col = smem + S::kSfCol + buf * S::kSfBytes;
 
     auto phases_1_2 = [&](auto full_c) {
       constexpr bool FULL = decltype(full_c)::value;
       // ---------------------------------------------------------------- phase 1 ----
-      const int rows_left = FULL ? 128 : (int)(a.rows - row0) - rl;         // chunk i exists iff 4 i < rows_left
+      const int rows_left = FULL ? 128 : (int)(a.rows - row0) - rl;         // chunk i exists iff RPP * i < rows_left
       const bool col_ok = FULL || (col0 + cb * 16 < a.cols);
-      uint32_t raw[4][8];
+      uint32_t raw[NP][8];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const uint4 h0 = *reinterpret_cast<const uint4*>(tile_buf + tile_ld + i * 1024);
-        const uint4 h1 = *reinterpret_cast<const uint4*>(tile_buf + tile_ld + i * 1024 + 16);
+      for (int i = 0; i < NP; ++i) {
+        const uint4 h0 = *reinterpret_cast<const uint4*>(tile_buf + tile_ld + i * (RPP * S::kRow));
+        const uint4 h1 = *reinterpret_cast<const uint4*>(tile_buf + tile_ld + i * (RPP * S::kRow) + 16);
         raw[i][0] = h0.x; raw[i][1] = h0.y; raw[i][2] = h0.z; raw[i][3] = h0.w;
         raw[i][4] = h1.x; raw[i][5] = h1.y; raw[i][6] = h1.z; raw[i][7] = h1.w;
       }
@@ -452,18 +469,18 @@ __global__ void __launch_bounds__(256, 2) quantize_kernel(const __grid_constant_
       if (BLOCK2D) {  // amax of the lane's chunk column over the warp's 16 rows: one scale per 16 x 16 block
         float blk_amax = 0.f;
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
+        for (int i = 0; i < NP; ++i) {
           uint32_t acc = 0;
 #pragma unroll
           for (int k = 0; k < 8; ++k) acc = absmax_bf16x2(acc, raw[i][k]);
           blk_amax = fmaxf(blk_amax, fmaxf(bf16_lo(acc), bf16_hi(acc)));
         }
-        blk_amax = fmaxf(blk_amax, __shfl_xor_sync(0xffffffffu, blk_amax, 8));
-        blk_amax = fmaxf(blk_amax, __shfl_xor_sync(0xffffffffu, blk_amax, 16));
+#pragma unroll
+        for (int o = CH; o < 32; o <<= 1) blk_amax = fmaxf(blk_amax, __shfl_xor_sync(0xffffffffu, blk_amax, o));
         block_scales(blk_amax, r_senc, r_sdec, blk_byte, blk_enc);
-        if (lane < 8) {
-          reinterpret_cast<float*>(smem + QuantSmem::kBlkEnc)[warp * 8 + cb] = blk_enc;
-          smem[QuantSmem::kBlkByte + warp * 8 + cb] = (uint8_t)blk_byte;
+        if (lane < CH) {
+          reinterpret_cast<float*>(smem + S::kBlkEnc)[warp * CH + cb] = blk_enc;
+          smem[S::kBlkByte + warp * CH + cb] = (uint8_t)blk_byte;
         }
       }
 
@@ -471,10 +488,10 @@ __global__ void __launch_bounds__(256, 2) quantize_kernel(const __grid_constant_
       if (SR) g = (uint64_t)(row0 + rl) * (uint64_t)n_cb + (uint64_t)((col0 >> 4) + cb);
       uint8_t* r_out = HAS_ROW ? a.r_codes + (row0 + rl) * r_pitch + ((col0 + cb * 16) >> 1) : nullptr;
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
+      for (int i = 0; i < NP; ++i) {
         uint32_t rnd[4] = {0u, 0u, 0u, 0u};
         if (SR) {
-          const uint64_t gi = g + (uint64_t)(4 * i) * (uint64_t)n_cb;
+          const uint64_t gi = g + (uint64_t)(RPP * i) * (uint64_t)n_cb;
           uint4 q = philox4x32_10((uint32_t)gi, (uint32_t)(gi >> 32), a.off_lo, a.off_hi, a.rk);
           rnd[0] = q.x; rnd[1] = q.y; rnd[2] = q.z; rnd[3] = q.w;
           if (HAS_COL && !kNibbleTranspose) {
@@ -482,7 +499,7 @@ __global__ void __launch_bounds__(256, 2) quantize_kernel(const __grid_constant_
             if (a.off_hi_col != a.off_hi)
               qc = philox4x32_10((uint32_t)gi, (uint32_t)(gi >> 32), a.off_lo, a.off_hi_col, a.rk);
             // staged complemented: the conversion wants 255 - draw
-            *reinterpret_cast<uint4*>(smem + rand_st + i * 512) = make_uint4(~qc.x, ~qc.y, ~qc.z, ~qc.w);
+            *reinterpret_cast<uint4*>(smem + rand_st + i * (RPP * TC)) = make_uint4(~qc.x, ~qc.y, ~qc.z, ~qc.w);
           }
         }
         if (HAS_ROW) {
@@ -506,10 +523,11 @@ __global__ void __launch_bounds__(256, 2) quantize_kernel(const __grid_constant_
             enc = enc_row[byte];
           }
           const uint2 codes = convert16<SR>(f, enc, Nu14FromWords{rnd});
-          if (FULL || (col_ok && 4 * i < rows_left)) *reinterpret_cast<uint2*>(r_out + (int64_t)(4 * i) * r_pitch) = codes;
+          if (FULL || (col_ok && RPP * i < rows_left))
+            *reinterpret_cast<uint2*>(r_out + (int64_t)(RPP * i) * r_pitch) = codes;
           if (kNibbleTranspose)  // row r, bytes [8 cb, 8 cb + 8): byte k = columns (2k, 2k + 1) of the chunk
-            *reinterpret_cast<uint2*>(smem + QuantSmem::kRand + (rl + 4 * i) * 64 + cb * 8) =
-                (FULL || (col_ok && 4 * i < rows_left)) ? codes : make_uint2(0u, 0u);
+            *reinterpret_cast<uint2*>(smem + S::kRand + (rl + RPP * i) * (TC / 2) + cb * 8) =
+                (FULL || (col_ok && RPP * i < rows_left)) ? codes : make_uint2(0u, 0u);
           sf_row[sf_row_pos + i * sf_row_step] = (uint8_t)byte;
         }
       }
@@ -521,7 +539,7 @@ __global__ void __launch_bounds__(256, 2) quantize_kernel(const __grid_constant_
       if (HAS_COL) {
         const int q = warp;  // 16-row group inside the tile
 #pragma unroll
-        for (int it = 0; it < 2; ++it) {
+        for (int it = 0; it < NIT; ++it) {
           const int cp = lane + 32 * it;  // column pair: tile columns 2cp, 2cp+1
           if (kNibbleTranspose) {
             // byte [row][cp] of the staged row-wise codes = (column 2cp in the low nibble, 2cp + 1 in the high one)
@@ -530,7 +548,7 @@ __global__ void __launch_bounds__(256, 2) quantize_kernel(const __grid_constant_
             for (int m = 0; m < 4; ++m) {
               uint32_t b[4];
 #pragma unroll
-              for (int j = 0; j < 4; ++j) b[j] = smem[QuantSmem::kRand + (q * 16 + 4 * m + j) * 64 + cp];
+              for (int j = 0; j < 4; ++j) b[j] = smem[S::kRand + (q * 16 + 4 * m + j) * (TC / 2) + cp];
               w[m] = __byte_perm(__byte_perm(b[0], b[1], 0x0040), __byte_perm(b[2], b[3], 0x0040), 0x5410);
             }
             auto gather = [](uint32_t x) {  // four nibbles, one per byte -> 16 bits
@@ -545,7 +563,7 @@ __global__ void __launch_bounds__(256, 2) quantize_kernel(const __grid_constant_
             }
             const uint2 codes0 = make_uint2(lo[0] | (lo[1] << 16), lo[2] | (lo[3] << 16));
             const uint2 codes1 = make_uint2(hi[0] | (hi[1] << 16), hi[2] | (hi[3] << 16));
-            const uint32_t byte = smem[QuantSmem::kBlkByte + q * 8 + (cp >> 3)];
+            const uint32_t byte = smem[S::kBlkByte + q * CH + (cp >> 3)];
             *reinterpret_cast<uint4*>(col_codes + col_codes_st + it * 4096) =
                 make_uint4(codes0.x, codes0.y, codes1.x, codes1.y);
             sf_col[sf_col_pos + it * sf_col_it] = (uint8_t)byte;
@@ -553,10 +571,10 @@ __global__ void __launch_bounds__(256, 2) quantize_kernel(const __grid_constant_
             continue;
           }
           float2 v[16];  // rows of the group, (column 2cp, column 2cp + 1)
-          const uint8_t* tp = tile_buf + q * 16 * 256 + cp * 4;
+          const uint8_t* tp = tile_buf + q * 16 * S::kRow + cp * 4;
 #pragma unroll
           for (int j = 0; j < 16; ++j) {
-            uint32_t word = *reinterpret_cast<const uint32_t*>(tp + j * 256);
+            uint32_t word = *reinterpret_cast<const uint32_t*>(tp + j * S::kRow);
             if (RHT_COL) word ^= a.row_sign[j];
             v[j] = make_float2(bf16_lo(word), bf16_hi(word));
           }
@@ -564,8 +582,8 @@ __global__ void __launch_bounds__(256, 2) quantize_kernel(const __grid_constant_
           uint32_t byte0, byte1;
           float2 enc;
           if (BLOCK2D) {
-            enc.x = enc.y = reinterpret_cast<const float*>(smem + QuantSmem::kBlkEnc)[q * 8 + (cp >> 3)];
-            byte0 = byte1 = smem[QuantSmem::kBlkByte + q * 8 + (cp >> 3)];
+            enc.x = enc.y = reinterpret_cast<const float*>(smem + S::kBlkEnc)[q * CH + (cp >> 3)];
+            byte0 = byte1 = smem[S::kBlkByte + q * CH + (cp >> 3)];
           } else {
             const float2 m = amax_pairs(v);
             byte0 = block_scale_byte(RHT_COL ? 0.25f * m.x : m.x, c_senc);
@@ -576,9 +594,9 @@ __global__ void __launch_bounds__(256, 2) quantize_kernel(const __grid_constant_
           if (SR) {
             // low / high byte of ntwo[j] = 255 - draw of source element (row 16q + j, column 2cp / 2cp + 1)
             uint32_t ntwo[16];
-            const uint8_t* rp = smem + QuantSmem::kRand + q * 16 * 128 + cp * 2;
+            const uint8_t* rp = smem + S::kRand + q * 16 * TC + cp * 2;
 #pragma unroll
-            for (int j = 0; j < 16; ++j) ntwo[j] = *reinterpret_cast<const uint16_t*>(rp + j * 128);
+            for (int j = 0; j < 16; ++j) ntwo[j] = *reinterpret_cast<const uint16_t*>(rp + j * TC);
             convert16x2_sr(v, enc, ntwo, codes0, codes1);
           } else {
             convert16x2_rne(v, enc, codes0, codes1);
@@ -604,20 +622,30 @@ __global__ void __launch_bounds__(256, 2) quantize_kernel(const __grid_constant_
     if (HAS_COL) {
       const int64_t pitch = a.rows >> 1;  // bytes per row of the transposed copy
       if ((a.rows & 31) == 0) {
-        // a thread takes column pair cp and the 16-row groups (2m, 2m + 1): 16 bytes = 32 rows of each of its two columns
-        const int cp = threadIdx.x >> 2, m = threadIdx.x & 3;
-        const uint8_t* unit = col_codes + cp * 128 + ((((2 * m) ^ cp) & 7) << 4);
-        const uint4 g0 = *reinterpret_cast<const uint4*>(unit);  // group 2m: (first column, second column) x 8 bytes
-        const uint4 g1 = *reinterpret_cast<const uint4*>(reinterpret_cast<const uint8_t*>((uintptr_t)unit ^ 16));
-        uint8_t* dst = a.c_codes + (col0 + 2 * cp) * pitch + (row0 >> 1) + m * 16;
-        if (full_tile || (row0 + 32 * m < a.rows && col0 + 2 * cp < a.cols)) {  // cols is even, rows % 32 == 0
-          *reinterpret_cast<uint4*>(dst) = make_uint4(g0.x, g0.y, g1.x, g1.y);
-          *reinterpret_cast<uint4*>(dst + pitch) = make_uint4(g0.z, g0.w, g1.z, g1.w);
+        // 16 bytes per store: the 16-row groups (2m, 2m + 1) of a column
+        if (TC == 64) {  // a thread takes 32 rows of one column
+          const int c = threadIdx.x >> 2, m = threadIdx.x & 3, cp = c >> 1;
+          const uint8_t* unit = col_codes + cp * 128 + ((((2 * m) ^ cp) & 7) << 4) + (c & 1) * 8;
+          const uint2 g0 = *reinterpret_cast<const uint2*>(unit);
+          const uint2 g1 = *reinterpret_cast<const uint2*>(reinterpret_cast<const uint8_t*>((uintptr_t)unit ^ 16));
+          if (full_tile || (row0 + 32 * m < a.rows && col0 + c < a.cols))
+            *reinterpret_cast<uint4*>(a.c_codes + (col0 + c) * pitch + (row0 >> 1) + m * 16) =
+                make_uint4(g0.x, g0.y, g1.x, g1.y);
+        } else {  // ... or of column pair cp
+          const int cp = threadIdx.x >> 2, m = threadIdx.x & 3;
+          const uint8_t* unit = col_codes + cp * 128 + ((((2 * m) ^ cp) & 7) << 4);
+          const uint4 g0 = *reinterpret_cast<const uint4*>(unit);  // group 2m: (first column, second column) x 8 bytes
+          const uint4 g1 = *reinterpret_cast<const uint4*>(reinterpret_cast<const uint8_t*>((uintptr_t)unit ^ 16));
+          uint8_t* dst = a.c_codes + (col0 + 2 * cp) * pitch + (row0 >> 1) + m * 16;
+          if (full_tile || (row0 + 32 * m < a.rows && col0 + 2 * cp < a.cols)) {  // cols is even, rows % 32 == 0
+            *reinterpret_cast<uint4*>(dst) = make_uint4(g0.x, g0.y, g1.x, g1.y);
+            *reinterpret_cast<uint4*>(dst + pitch) = make_uint4(g0.z, g0.w, g1.z, g1.w);
+          }
         }
       } else {
         // rows % 32 == 16: rows of the copy start on 8-byte boundaries; eight lanes write the 64 bytes of a column
 #pragma unroll
-        for (int p = 0; p < 4; ++p) {
+        for (int p = 0; p < TC / 32; ++p) {
           const int c = (threadIdx.x >> 3) + 32 * p, q = threadIdx.x & 7, cp = c >> 1;
           const uint2 v = *reinterpret_cast<const uint2*>(col_codes + cp * 128 + (((q ^ cp) & 7) << 4) + (c & 1) * 8);
           if (full_tile || (row0 + 16 * q < a.rows && col0 + c < a.cols))
@@ -636,8 +664,16 @@ __global__ void __launch_bounds__(256, 2) quantize_kernel(const __grid_constant_
       // the copy's row / block coordinates of this tile
       const int64_t R0 = which == 0 ? row0 : col0, K0 = which == 0 ? (col0 >> 4) : (row0 >> 4);
       const int64_t Rn = which == 0 ? a.rows : a.cols, n_kb = which == 0 ? n_cb : n_rb;
-      if (swz) {
-        if (threadIdx.x < 64) {
+      if (swz && TC == 64 && which == 1) {
+        if (threadIdx.x < 64) {  // eight bytes (64 of the 128 rows) of each 16 of two atoms
+          const int atom = threadIdx.x >> 5, l = threadIdx.x & 31;
+          if (K0 + atom * 4 < n_kb) {
+            const int64_t off = ((R0 >> 7) * (n_kb >> 2) + (K0 >> 2) + atom) * 512 + l * 16 + ((int)(R0 & 127) >> 5) * 4;
+            *reinterpret_cast<uint2*>(dst + off) = *reinterpret_cast<const uint2*>(src + atom * 256 + l * 8);
+          }
+        }
+      } else if (swz) {
+        if (threadIdx.x < (TC == 64 ? 32 : 64)) {
           const int atom = threadIdx.x >> 5;
           if (K0 + atom * 4 < n_kb) {
             const int64_t off = ((R0 >> 7) * (n_kb >> 2) + (K0 >> 2) + atom) * 512 + (threadIdx.x & 31) * 16;
@@ -645,7 +681,10 @@ __global__ void __launch_bounds__(256, 2) quantize_kernel(const __grid_constant_
           }
         }
       } else {
-        store_linear_scales(src, dst, R0, K0, Rn, n_kb, full_tile);
+        if (which == 0)
+          store_linear_scales<128, CH>(src, dst, R0, K0, Rn, n_kb, full_tile);
+        else
+          store_linear_scales<TC, 8>(src, dst, R0, K0, Rn, n_kb, full_tile);
       }
     }
     ++k;  // on to the CTA's next own tile
@@ -668,7 +707,7 @@ __global__ void __launch_bounds__(256, 2) quantize_kernel(const __grid_constant_
     return;  // no maximum is published by a CTA that gave up
   }
   if (SIDE) {
-    float* red = reinterpret_cast<float*>(smem + QuantSmem::kBlkEnc);  // free in 1 x 16 mode
+    float* red = reinterpret_cast<float*>(smem + S::kBlkEnc);  // free in 1 x 16 mode
     const float m = warp_max(fmaxf(bf16_lo(side_acc), bf16_hi(side_acc)));
     __syncthreads();
     if (lane == 0) red[warp] = m;
@@ -828,25 +867,26 @@ cudaError_t launch_amax_rot_col_small(const QuantArgs& a, bool has_row, uint32_t
                  : launch_amax_rot_col<false>(a, mask16, nullptr, nullptr, a.c_global, d, norm, s);
 }
 
-template <bool HR, bool HC, bool B2, bool RR, bool RC, bool SR, bool SIDE = false>
-static cudaError_t launch_quant_t(const QuantArgs& a_in, cudaStream_t s, const SideAmax* side = nullptr) {
-  auto kern = quantize_kernel<HR, HC, B2, RR, RC, SR, SIDE>;
+template <bool HR, bool HC, bool B2, bool RR, bool RC, bool SR, bool SIDE, int TC>
+static cudaError_t launch_quant_tc(const QuantArgs& a_in, int sms, cudaStream_t s, const SideAmax* side) {
+  auto kern = quantize_kernel<HR, HC, B2, RR, RC, SR, SIDE, TC>;
   QuantArgs a = a_in;
+  a.tiles_c = (int)((a.cols + TC - 1) / TC);
   constexpr bool kRowCodes = B2 && HR && HC;
-  constexpr int smem = QuantSmem::bytes(SR && HC && !kRowCodes, kRowCodes);
-  // the source as a 2-D tensor map: boxes of 128 x 128 bf16 (256-byte rows, no swizzle), zero fill outside
+  constexpr int smem = QuantSmem<TC>::bytes(SR && HC && !kRowCodes, kRowCodes);
+  // the source as a 2-D tensor map: boxes of 128 rows x TC bf16 (no swizzle), zero fill outside
   CUtensorMap map;
   if (!make_map_2d(&map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, a.x, (uint64_t)a.cols, (uint64_t)a.rows,
-                   (uint64_t)a.ld * 2, 128, 128, false))
+                   (uint64_t)a.ld * 2, TC, 128, false))
     return cudaErrorInvalidValue;
   CUtensorMap side_map = map;
   int64_t side_tiles = 0;
   if (SIDE) {
     if (!side || !make_map_2d(&side_map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, side->x, (uint64_t)side->cols,
-                              (uint64_t)side->rows, (uint64_t)side->ld * 2, 128, 128, false))
+                              (uint64_t)side->rows, (uint64_t)side->ld * 2, TC, 128, false))
       return cudaErrorInvalidValue;
     a.side_tiles_r = (int)((side->rows + 127) / 128);
-    a.side_tiles_c = (int)((side->cols + 127) / 128);
+    a.side_tiles_c = (int)((side->cols + TC - 1) / TC);
     a.side_out0 = side->out0;
     a.side_out1 = side->out1;
     side_tiles = (int64_t)a.side_tiles_r * a.side_tiles_c;
@@ -860,8 +900,7 @@ static cudaError_t launch_quant_t(const QuantArgs& a_in, cudaStream_t s, const S
   if (device_needs_config(configured, &dev)) {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
-    int sms = 0, per_sm = 0;
-    if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev < 0 ? 0 : dev)) != cudaSuccess) return e;
+    int per_sm = 0;
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 256, smem)) != cudaSuccess) return e;
     if (dev >= 0 && dev < 64) resident[dev].store(sms * (per_sm > 0 ? per_sm : 1), std::memory_order_relaxed);
     device_configured(configured, dev);
@@ -872,6 +911,21 @@ static cudaError_t launch_quant_t(const QuantArgs& a_in, cudaStream_t s, const S
   const cudaError_t e = launch_kernel(kern, dim3((unsigned)grid), dim3(256), smem, s, map, side_map, a);
   count_launch();
   return e;
+}
+
+template <bool HR, bool HC, bool B2, bool RR, bool RC, bool SR, bool SIDE = false>
+static cudaError_t launch_quant_t(const QuantArgs& a, cudaStream_t s, const SideAmax* side = nullptr) {
+  int sms = 0;
+  const cudaError_t e = sm_count(&sms);
+  if (e != cudaSuccess) return e;
+  // Tiles 64 columns wide when they go round the resident CTAs in less time: a tile of half the width takes 0.535 of the time
+  // (16x16 blocks: 0.58), and the CTAs take whole rounds.  Measured (128 / 64 wide): gradient of 512 x 1024 8.6 / 7.0 us, 2048 x
+  // 1024 10.6 / 8.3, 2816 x 2304 16.4 / 14.7, 4096 x 4096 31.7 / 30.4, 8192 x 5120 63.3 / 67.2; weight of 2048 x 1024 7.0 / 6.0,
+  // 4096 x 2304 11.1 / 12.1.
+  const int64_t slots = 2 * sms, t128 = (int64_t)a.tiles_r * a.tiles_c, t64 = (int64_t)a.tiles_r * ((a.cols + 63) / 64);
+  const double r128 = (double)((t128 + slots - 1) / slots), r64 = (double)((t64 + slots - 1) / slots) * (B2 ? 0.58 : 0.535);
+  if (!RR && r64 < r128) return launch_quant_tc<HR, HC, B2, RR, RC, SR, SIDE, RR ? 128 : 64>(a, sms, s, side);
+  return launch_quant_tc<HR, HC, B2, RR, RC, SR, SIDE, 128>(a, sms, s, side);
 }
 
 cudaError_t launch_quantize_with_amax_of(const QuantArgs& a, bool has_col, const SideAmax& side, cudaStream_t s) {

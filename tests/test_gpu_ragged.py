@@ -68,3 +68,21 @@ def test_error_sums(shape, what):
         got, d = B.nvfp4_quant_error(x.contiguous(), q), x.double() - B.nvfp4_dequantize(q).double()
     want = torch.stack([d.square().sum(), x.double().square().sum()])
     assert bool(((got - want).abs() <= 16 * 2.0 ** -24 * want).all())
+
+
+@pytest.mark.parametrize("shape", [(128, 128), (640, 1152), (16, 5136), (2064, 4112), (5120, 7680)])
+@pytest.mark.parametrize("kind", ["activation", "gradient", "weight"])
+def test_both_tile_widths_of_the_quantizer(shape, kind):
+    """The tile width follows the number of tiles: one tile to 2400, ragged and whole."""
+    R, C = shape
+    g = torch.Generator("cuda").manual_seed(R + C)
+    x = torch.randn((R, C), generator=g, device="cuda").to(torch.bfloat16)
+    x[R // 2, C // 3] = 40.0
+    layout = B.SF_SWIZZLED if R % 128 == 0 and C % 128 == 0 else B.SF_LINEAR
+    opts = dict(block_rows=16) if kind == "weight" else dict(rounding=oracle.SR if kind == "gradient" else oracle.RNE,
+                                                            seed=4, sr_offset=1)
+    row, col = B.alloc_tensor(R, C, layout), B.alloc_tensor(C, R, layout)
+    B.nvfp4_quantize(x, B.quant_opts(**opts), row, col)
+    B.nvfp4_device_status()
+    P.assert_exact(row, oracle.quantize(synth.bits(x.cpu()), **opts), "row")
+    P.assert_exact(col, oracle.quantize(synth.bits(x.cpu()), colwise=True, **opts), "col")
