@@ -35,11 +35,40 @@ nvfp4_status check_copy(const nvfp4_tensor* t, int64_t rows, int64_t cols) {
   return NVFP4_OK;
 }
 
+// launch description of a quantize call whose arguments have been checked
+nvfp4_status fill_quant_args(const void* x, int64_t rows, int64_t cols, int64_t ld, const nvfp4_quant_opts* o,
+                             const nvfp4_tensor* rowwise, const nvfp4_tensor* colwise, bool mx, QuantArgs& a) {
+  a = QuantArgs{};
+  a.x = static_cast<const uint16_t*>(x);
+  a.rows = rows; a.cols = cols; a.ld = ld;
+  if (rowwise) {
+    a.r_codes = rowwise->codes; a.r_scales = rowwise->scales; a.r_global = rowwise->global;
+    a.r_swz = rowwise->sf_layout == NVFP4_SF_SWIZZLED;
+  }
+  if (colwise) {
+    a.c_codes = colwise->codes; a.c_scales = colwise->scales; a.c_global = colwise->global;
+    a.c_swz = colwise->sf_layout == NVFP4_SF_SWIZZLED;
+  }
+  a.sign_mask = mx ? o->rht_sign_mask : (o->rht_sign_mask & 0xffffu);
+  for (int j = 0; j < 32; ++j) a.row_sign[j] = ((a.sign_mask >> j) & 1u) ? 0x80008000u : 0u;
+  a.seed_lo = (uint32_t)o->seed; a.seed_hi = (uint32_t)(o->seed >> 32);
+  for (uint32_t r = 0; r < 10; ++r) {  // Philox key schedule
+    a.rk[2 * r] = a.seed_lo + r * 0x9E3779B9u;
+    a.rk[2 * r + 1] = a.seed_hi + r * 0xBB67AE85u;
+  }
+  a.off_lo = (uint32_t)o->sr_offset; a.off_hi = (uint32_t)(o->sr_offset >> 32);
+  a.off_hi_col = (o->flags & NVFP4_SR_INDEPENDENT_COPIES) ? (a.off_hi | 0x80000000u) : a.off_hi;
+  a.tiles_r = (int)((rows + 127) / 128);
+  a.tiles_c = (int)((cols + 127) / 128);
+  if (device_status_word(&a.status) != cudaSuccess) return NVFP4_ERR_CUDA;
+  return NVFP4_OK;
+}
+
 // check_only: every argument check of the call, no launch (the composed calls validate all their steps first, so
 // that a rejected call has enqueued nothing)
 nvfp4_status quantize_impl(const void* x, int64_t rows, int64_t cols, int64_t ld, const nvfp4_quant_opts* o,
                            const nvfp4_tensor* rowwise, const nvfp4_tensor* colwise, cudaStream_t s,
-                           bool check_only = false, const SideAmax* side = nullptr, bool chained = false) {
+                           bool check_only = false) {
   if (!x || !o) return NVFP4_ERR_NULL;
   if (!rowwise && !colwise) return NVFP4_ERR_NULL;
   if (rows <= 0 || cols <= 0 || rows % 16 != 0 || cols % 16 != 0) return NVFP4_ERR_SHAPE;
@@ -98,29 +127,8 @@ nvfp4_status quantize_impl(const void* x, int64_t rows, int64_t cols, int64_t ld
   if (colwise && (st = check_copy(colwise, cols, rows)) != NVFP4_OK) return st;
   if (check_only) return NVFP4_OK;
 
-  QuantArgs a{};
-  a.x = static_cast<const uint16_t*>(x);
-  a.rows = rows; a.cols = cols; a.ld = ld;
-  if (rowwise) {
-    a.r_codes = rowwise->codes; a.r_scales = rowwise->scales; a.r_global = rowwise->global;
-    a.r_swz = rowwise->sf_layout == NVFP4_SF_SWIZZLED;
-  }
-  if (colwise) {
-    a.c_codes = colwise->codes; a.c_scales = colwise->scales; a.c_global = colwise->global;
-    a.c_swz = colwise->sf_layout == NVFP4_SF_SWIZZLED;
-  }
-  a.sign_mask = mx ? o->rht_sign_mask : (o->rht_sign_mask & 0xffffu);
-  for (int j = 0; j < 32; ++j) a.row_sign[j] = ((a.sign_mask >> j) & 1u) ? 0x80008000u : 0u;
-  a.seed_lo = (uint32_t)o->seed; a.seed_hi = (uint32_t)(o->seed >> 32);
-  for (uint32_t r = 0; r < 10; ++r) {  // Philox key schedule
-    a.rk[2 * r] = a.seed_lo + r * 0x9E3779B9u;
-    a.rk[2 * r + 1] = a.seed_hi + r * 0xBB67AE85u;
-  }
-  a.off_lo = (uint32_t)o->sr_offset; a.off_hi = (uint32_t)(o->sr_offset >> 32);
-  a.off_hi_col = (o->flags & NVFP4_SR_INDEPENDENT_COPIES) ? (a.off_hi | 0x80000000u) : a.off_hi;
-  a.tiles_r = (int)((rows + 127) / 128);
-  a.tiles_c = (int)((cols + 127) / 128);
-  if (device_status_word(&a.status) != cudaSuccess) return NVFP4_ERR_CUDA;
+  QuantArgs a;
+  if ((st = fill_quant_args(x, rows, cols, ld, o, rowwise, colwise, mx, a)) != NVFP4_OK) return st;
 
   const bool hr = rowwise != nullptr, hc = colwise != nullptr;
   const bool b2 = o->block_rows == blk, sr = o->rounding == NVFP4_ROUND_STOCHASTIC;
@@ -149,27 +157,13 @@ nvfp4_status quantize_impl(const void* x, int64_t rows, int64_t cols, int64_t ld
     return launch_quantize_rht(ra, (o->flags & NVFP4_AMAX_PROVIDED) != 0, sr, s) == cudaSuccess ? NVFP4_OK
                                                                                                   : NVFP4_ERR_CUDA;
   }
-  // pass 2 may read the source while the previous kernel of this call drains (its own pass 1, or the kernel before)
-  a.chained = chained;
-  // only the forward pass's activation quantize carries a side job (see side_amax_fits); checked before any launch
-  if (side && (!hr || (o->flags & NVFP4_AMAX_PROVIDED) || b2 || sr || o->rht_rowwise || (hc && !o->rht_colwise))) return NVFP4_ERR_ARG;
   if (!(o->flags & NVFP4_AMAX_PROVIDED)) {
-    if (launch_amax(a, hr, hc, o->rht_rowwise != 0, o->rht_colwise != 0, side, s) != cudaSuccess) return NVFP4_ERR_CUDA;
+    if (launch_amax(a, hr, hc, o->rht_rowwise != 0, o->rht_colwise != 0, s) != cudaSuccess) return NVFP4_ERR_CUDA;
     a.chained = 1;
-  }
-  if (side) {
-    return launch_quantize_with_amax_of(a, hc, *side, s) == cudaSuccess ? NVFP4_OK : NVFP4_ERR_CUDA;
   }
   if (launch_quantize(a, hr, hc, b2, o->rht_rowwise != 0, o->rht_colwise != 0, sr, s) != cudaSuccess)
     return NVFP4_ERR_CUDA;
   return NVFP4_OK;
-}
-
-// Whether a quantize of the composed calls (options xo) runs `quantize_kernel`, the kernel that can take a second
-// tensor's plain amax on the side and lets the next kernel of the call set itself up early: bf16 source, NVFP4, the
-// 16-point transform or none.
-bool side_amax_fits(int32_t fmt, const nvfp4_quant_opts& xo) {
-  return fmt == NVFP4_FORMAT_NVFP4 && (xo.rht_dim == 0 || xo.rht_dim == 16) && !(xo.flags & NVFP4_INPUT_FP32);
 }
 
 // argument checks of one GEMM and its launch description
@@ -344,12 +338,13 @@ nvfp4_status nvfp4_linear_fwd(const void* X, const void* W, int64_t M, int64_t N
   if (!w_is_cached && (st = quantize_impl(W, N, K, K, &wo, W_row, W_col_saved, s, true)) != NVFP4_OK) return st;
   if ((st = quantize_impl(X, M, K, K, &xo, &x_row, X_col_saved, s, true)) != NVFP4_OK) return st;
   if ((st = gemm_prepare(&x_row, W_row, Y_bf16, 0, N, 0, gy)) != NVFP4_OK) return st;
-  if (!w_is_cached && side_amax_fits(fmt, xo)) {
-    // pass 1 of W (memory-bound) rides on pass 2 of X (issue-bound); W's pass 2 then finds its amax in place
-    const SideAmax w_amax{W, N, K, K, W_row->global, W_col_saved ? W_col_saved->global : nullptr};
-    if ((st = quantize_impl(X, M, K, K, &xo, &x_row, X_col_saved, s, false, &w_amax)) != NVFP4_OK) return st;
-    wo.flags |= NVFP4_AMAX_PROVIDED;
-    if ((st = quantize_impl(W, N, K, K, &wo, W_row, W_col_saved, s, false, nullptr, true)) != NVFP4_OK) return st;
+  if (!w_is_cached && fmt == NVFP4_FORMAT_NVFP4 && (xo.rht_dim == 0 || xo.rht_dim == 16)) {
+    // both tensors in the same launches (the kernels of the other formats and transform sizes take one tensor each)
+    QuantArgs xa, wa;
+    if ((st = fill_quant_args(X, M, K, K, &xo, &x_row, X_col_saved, false, xa)) != NVFP4_OK) return st;
+    if ((st = fill_quant_args(W, N, K, K, &wo, W_row, W_col_saved, false, wa)) != NVFP4_OK) return st;
+    if (launch_quantize_x_and_w(xa, X_col_saved != nullptr, wa, W_col_saved != nullptr, s) != cudaSuccess)
+      return NVFP4_ERR_CUDA;
     return gemm_impl(&x_row, W_row, Y_bf16, 0, N, 0, s);
   }
   if (!w_is_cached && (st = quantize_impl(W, N, K, K, &wo, W_row, W_col_saved, s)) != NVFP4_OK) return st;

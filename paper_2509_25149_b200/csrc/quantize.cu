@@ -20,14 +20,12 @@ namespace nvfp4 {
 // CTA tile 128 rows x 256 columns; a warp owns 16 rows, a lane 8 columns of each of them.
 // ---------------------------------------------------------------------------------------------
 template <bool PLAIN, bool ROT_ROW, bool ROT_COL>
-__global__ void __launch_bounds__(256) amax_kernel(const uint16_t* __restrict__ x, int64_t rows,
-                                                   int64_t cols, int64_t ld, uint32_t sign_mask,
-                                                   int tiles_c, float* __restrict__ out_plain0,
-                                                   float* __restrict__ out_plain1,
-                                                   float* __restrict__ out_rot_row,
-                                                   float* __restrict__ out_rot_col) {
+__device__ __forceinline__ void amax_tile(const uint16_t* __restrict__ x, int64_t rows, int64_t cols, int64_t ld,
+                                          uint32_t sign_mask, int tile, int tiles_c, float* __restrict__ out_plain0,
+                                          float* __restrict__ out_plain1, float* __restrict__ out_rot_row,
+                                          float* __restrict__ out_rot_col) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t tr = blockIdx.x / tiles_c, tc = blockIdx.x % tiles_c;
+  const int64_t tr = tile / tiles_c, tc = tile % tiles_c;
   const int64_t r0 = tr * 128 + warp * 16;
   const int64_t c0 = tc * 256 + lane * 8;
   const bool in_range = (r0 < rows) && (c0 < cols);  // rows % 16 == 0, cols % 8 == 0
@@ -132,6 +130,15 @@ __global__ void __launch_bounds__(256) amax_kernel(const uint16_t* __restrict__ 
   }
 }
 
+template <bool PLAIN, bool ROT_ROW, bool ROT_COL>
+__global__ void __launch_bounds__(256) amax_kernel(const uint16_t* __restrict__ x, int64_t rows, int64_t cols, int64_t ld,
+                                                   uint32_t sign_mask, int tiles_c, float* __restrict__ out_plain0,
+                                                   float* __restrict__ out_plain1, float* __restrict__ out_rot_row,
+                                                   float* __restrict__ out_rot_col) {
+  amax_tile<PLAIN, ROT_ROW, ROT_COL>(x, rows, cols, ld, sign_mask, (int)blockIdx.x, tiles_c, out_plain0, out_plain1,
+                                     out_rot_row, out_rot_col);
+}
+
 // ---------------------------------------------------------------------------------------------
 // Pass 1 for a copy transformed down the rows (the transposed copy of a Wgrad operand, Appendix C): the
 // 16-point transform of 8 columns at a time is one bf16 tensor-core product  Y(16x8) = A(16x16) * X(16x8)  with
@@ -150,14 +157,13 @@ __device__ __forceinline__ uint32_t movmatrix_trans(uint32_t v) {
 // d, norm: size of the transform (2, 4, 8 or 16: H_16 is replaced by the block-diagonal matrix of 16 / d copies of
 // H_d) and its normalisation 1 / sqrt(d), applied to the maximum.
 template <bool PLAIN>
-__global__ void __launch_bounds__(256) amax_rot_col_kernel(const uint16_t* __restrict__ x, int64_t rows,
-                                                           int64_t cols, int64_t ld, uint32_t sign_mask,
-                                                           int tiles_c, float* __restrict__ out_plain0,
-                                                           float* __restrict__ out_plain1,
-                                                           float* __restrict__ out_rot_col, int d, float norm) {
+__device__ __forceinline__ void amax_rot_col_tile(const uint16_t* __restrict__ x, int64_t rows, int64_t cols, int64_t ld,
+                                                  uint32_t sign_mask, int tile, int tiles_c, float* __restrict__ out_plain0,
+                                                  float* __restrict__ out_plain1, float* __restrict__ out_rot_col, int d,
+                                                  float norm) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int g = lane >> 2, t = lane & 3;
-  const int64_t tr = blockIdx.x / tiles_c, tc = blockIdx.x % tiles_c;
+  const int64_t tr = tile / tiles_c, tc = tile % tiles_c;
   const int64_t r0 = tr * 128 + warp * 16;
   griddep_launch_dependents();  // pass 2 may set itself up while the last CTAs of this pass run
 
@@ -229,6 +235,30 @@ __global__ void __launch_bounds__(256) amax_rot_col_kernel(const uint16_t* __res
     }
     if (threadIdx.x == 1) atomicMax(reinterpret_cast<unsigned int*>(out_rot_col), bits);
   }
+}
+
+template <bool PLAIN>
+__global__ void __launch_bounds__(256) amax_rot_col_kernel(const uint16_t* __restrict__ x, int64_t rows, int64_t cols,
+                                                           int64_t ld, uint32_t sign_mask, int tiles_c,
+                                                           float* __restrict__ out_plain0, float* __restrict__ out_plain1,
+                                                           float* __restrict__ out_rot_col, int d, float norm) {
+  amax_rot_col_tile<PLAIN>(x, rows, cols, ld, sign_mask, (int)blockIdx.x, tiles_c, out_plain0, out_plain1, out_rot_col, d,
+                           norm);
+}
+
+// Pass 1 of two tensors in one launch (see quantize_x_and_w_kernel): the first n_x CTAs take tiles of an activation (row-wise
+// copy plain, transposed copy rotated), the others of a weight (plain).
+template <bool X_COL, bool W_COL>
+__global__ void __launch_bounds__(256) amax_x_and_w_kernel(const __grid_constant__ QuantArgs x, const __grid_constant__ QuantArgs w,
+                                                           int n_x, int x_tiles_c, int w_tiles_c) {
+  const int b = (int)blockIdx.x;
+  if (b >= n_x)
+    amax_tile<true, false, false>(w.x, w.rows, w.cols, w.ld, 0u, b - n_x, w_tiles_c, w.r_global, W_COL ? w.c_global : nullptr,
+                                  nullptr, nullptr);
+  else if (X_COL)
+    amax_rot_col_tile<true>(x.x, x.rows, x.cols, x.ld, x.sign_mask, b, x_tiles_c, x.r_global, nullptr, x.c_global, 16, 0.25f);
+  else
+    amax_tile<true, false, false>(x.x, x.rows, x.cols, x.ld, 0u, b, x_tiles_c, x.r_global, nullptr, nullptr, nullptr);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -306,10 +336,9 @@ __device__ __forceinline__ void store_linear_scales(const uint8_t* src, uint8_t*
     if (full_tile || (R0 + r + 256 / KB * p < Rn && K0 + kb < n_kb)) *d = src[threadIdx.x + 256 * p];
 }
 
-template <bool HAS_ROW, bool HAS_COL, bool BLOCK2D, bool RHT_ROW, bool RHT_COL, bool SR, bool SIDE, int TC>
-__global__ void __launch_bounds__(256, 2) quantize_kernel(const __grid_constant__ CUtensorMap src_map,
-                                                          const __grid_constant__ CUtensorMap side_map,
-                                                          const QuantArgs a) {
+template <bool HAS_ROW, bool HAS_COL, bool BLOCK2D, bool RHT_ROW, bool RHT_COL, bool SR, int TC>
+__device__ __forceinline__ void quantize_tiles(const CUtensorMap* src_map, const QuantArgs& a, const int block,
+                                               const int blocks) {  // this CTA among those of the tensor
   using S = QuantSmem<TC>;
   constexpr int CH = S::kChunks;          // chunks per tile row
   constexpr int RPP = 32 / CH;            // rows a warp covers with one chunk per lane; chunk i of a lane: RPP * i rows down
@@ -325,34 +354,13 @@ __global__ void __launch_bounds__(256, 2) quantize_kernel(const __grid_constant_
   volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(smem + S::kBars + 16);
   const uint32_t bar0 = smem_u32(smem + S::kBars), tile0 = smem_u32(smem + S::kTile);
 
-  const int total = a.tiles_r * a.tiles_c, stride = (int)gridDim.x;
-  const int first = total - 1 - (int)blockIdx.x;         // this CTA's tiles: first, first - stride, ...
+  const int total = a.tiles_r * a.tiles_c, stride = blocks;
+  const int first = total - 1 - block;  // this CTA's tiles: first, first - stride, ...
   const int n_mine = first >= 0 ? first / stride + 1 : 0;
-  // SIDE: the CTA also streams its share of a second tensor's tiles through the same ring and takes their plain
-  // amax (pass 1 of that tensor, Appendix B.1): memory-bound work riding on an issue-bound kernel.  Side tiles go
-  // front to back (the tensor's own pass 2 starts from its end), interleaved in proportion with the CTA's own tiles.
-  const int side_total = SIDE ? a.side_tiles_r * a.side_tiles_c : 0;
-  const int m_mine = (int)blockIdx.x < side_total ? (side_total - 1 - (int)blockIdx.x) / stride + 1 : 0;
-  const int n_jobs = n_mine + m_mine;
-  // with k own tiles and sk side tiles behind it, the CTA's next job is a side tile iff ...
-  auto side_next = [&](int k, int sk) {
-    return SIDE && sk < m_mine && (k >= n_mine || (long long)sk * n_mine < (long long)k * m_mine);
-  };
-  auto issue_load = [&](int j, int k, int sk) {  // job j (own tile k or side tile sk) into buffer j & 1 (one thread)
-    const uint32_t bar = bar0 + 8 * (j & 1), dst = tile0 + (j & 1) * S::kTileBytes;
-    mbar_expect_tx(bar, S::kTileBytes);
-    if (side_next(k, sk)) {
-      const int t = (int)blockIdx.x + sk * stride, tr = t / a.side_tiles_c, tc = t - tr * a.side_tiles_c;
-      tma_load_2d(dst, &side_map, tc * TC, tr * 128, bar);
-    } else {
-      const int t = first - k * stride, tr = t / a.tiles_c, tc = t - tr * a.tiles_c;
-      tma_load_2d(dst, &src_map, tc * TC, tr * 128, bar);
-    }
-  };
-  int ahead_k = 0, ahead_sk = 0;  // thread 0: own / side tiles among the jobs already issued
-  auto issue_next = [&](int j) {
-    issue_load(j, ahead_k, ahead_sk);
-    if (side_next(ahead_k, ahead_sk)) ++ahead_sk; else ++ahead_k;
+  auto issue = [&](int j) {  // the CTA's tile j into buffer j & 1 (one thread)
+    const int t = first - j * stride, tr = t / a.tiles_c, tc = t - tr * a.tiles_c;
+    mbar_expect_tx(bar0 + 8 * (j & 1), S::kTileBytes);
+    tma_load_2d(tile0 + (j & 1) * S::kTileBytes, src_map, tc * TC, tr * 128, bar0 + 8 * (j & 1));
   };
 
   // ------------------------------------------------------------------ set-up ----
@@ -364,8 +372,8 @@ __global__ void __launch_bounds__(256, 2) quantize_kernel(const __grid_constant_
     fence_mbarrier_init();
     fence_proxy_async_smem();
     if (!a.chained) griddep_wait();  // the source may be the previous kernel's output
-    if (n_jobs > 0) issue_next(0);
-    if (n_jobs > 1) issue_next(1);
+    if (n_mine > 0) issue(0);
+    if (n_mine > 1) issue(1);
     // the source tiles above are nobody's output in this call; the tensor amax below is the previous kernel's.
     // Every other thread passes the barrier below only after this wait, so no output is written before it either.
     griddep_wait();
@@ -381,7 +389,7 @@ __global__ void __launch_bounds__(256, 2) quantize_kernel(const __grid_constant_
       }
     }
     g_sc[0] = re; g_sc[1] = rd; g_sc[2] = ce; g_sc[3] = cd;
-    if (blockIdx.x == 0) {
+    if (block == 0) {
       if (HAS_ROW) a.r_global[1] = rd;
       if (HAS_COL) a.c_global[1] = cd;
     }
@@ -425,25 +433,11 @@ __global__ void __launch_bounds__(256, 2) quantize_kernel(const __grid_constant_
 
   const int step_r = stride / a.tiles_c, step_c = stride - step_r * a.tiles_c;  // tile coordinates move by these
   int tr = first >= 0 ? first / a.tiles_c : 0, tc = first >= 0 ? first - tr * a.tiles_c : 0;
-  int k = 0, sk = 0, j = 0;  // own tiles done, side tiles done, jobs done (the ring position)
-  uint32_t side_acc = 0;     // |.| maximum of the side tiles, two bf16 lanes
-  for (; j < n_jobs; ++j) {
-    const uint8_t* const tile_buf = smem + S::kTile + (j & 1) * S::kTileBytes;
-    quant_wait(bar0 + 8 * (j & 1), (uint32_t)(j >> 1) & 1u, abort_flag, a.status);  // the tile has landed
-    if (SIDE && side_next(k, sk)) {
-#pragma unroll
-      for (int i = 0; i < S::kTileBytes / 4096; ++i) {  // zero fill outside the tensor leaves the maximum alone
-        const uint4 v = *reinterpret_cast<const uint4*>(tile_buf + i * 4096 + threadIdx.x * 16);
-        side_acc = absmax_bf16x2(absmax_bf16x2(side_acc, v.x), v.y);
-        side_acc = absmax_bf16x2(absmax_bf16x2(side_acc, v.z), v.w);
-      }
-      __syncthreads();
-      if (*abort_flag) break;
-      if (threadIdx.x == 0 && j + 2 < n_jobs) issue_next(j + 2);
-      ++sk;
-      continue;
-    }
-    const int buf = k & 1;  // staging buffers alternate with the CTA's own tiles
+  int j = 0;  // tiles done
+  for (; j < n_mine; ++j) {
+    const int buf = j & 1;
+    const uint8_t* const tile_buf = smem + S::kTile + buf * S::kTileBytes;
+    quant_wait(bar0 + 8 * buf, (uint32_t)(j >> 1) & 1u, abort_flag, a.status);  // the tile has landed
     const int64_t row0 = (int64_t)tr * 128, col0 = (int64_t)tc * TC;
     const bool full_tile = (row0 + 128 <= a.rows) && (col0 + TC <= a.cols);
     uint8_t* const col_codes = smem + S::kColCodes + buf * S::kColBytes;
@@ -616,7 +610,7 @@ __global__ void __launch_bounds__(256, 2) quantize_kernel(const __grid_constant_
       phases_1_2(std::false_type{});
     __syncthreads();
     if (*abort_flag) break;  // a wait expired (the word is read after the barrier: the same for every thread)
-    if (threadIdx.x == 0 && j + 2 < n_jobs) issue_next(j + 2);  // every warp is done with this buffer
+    if (threadIdx.x == 0 && j + 2 < n_mine) issue(j + 2);  // every warp is done with this buffer
 
     // ------------------------------------------------------------------ phase 3 ----
     if (HAS_COL) {
@@ -687,7 +681,6 @@ __global__ void __launch_bounds__(256, 2) quantize_kernel(const __grid_constant_
           store_linear_scales<TC, 8>(src, dst, R0, K0, Rn, n_kb, full_tile);
       }
     }
-    ++k;  // on to the CTA's next own tile
     tr -= step_r;
     tc -= step_c;
     if (tc < 0) {
@@ -695,32 +688,37 @@ __global__ void __launch_bounds__(256, 2) quantize_kernel(const __grid_constant_
       --tr;
     }
   }
-  if (j < n_jobs) {
-    // left early: jobs j and j + 1 may still be in flight; give each one more bounded wait so that no copy lands
-    // in shared memory after the CTA has gone
-    if (threadIdx.x == 0)
-      for (int i = j; i < j + 2 && i < n_jobs; ++i) {
-        const unsigned long long t0 = globaltimer_ns();
-        while (!mbar_try(bar0 + 8 * (i & 1), (uint32_t)(i >> 1) & 1u) && globaltimer_ns() - t0 < kWaitLimitNs) {
-        }
+  if (j < n_mine && threadIdx.x == 0)
+    // left early: tiles j and j + 1 may still be in flight; give each one more bounded wait so that no copy lands in shared
+    // memory after the CTA has gone
+    for (int i = j; i < j + 2 && i < n_mine; ++i) {
+      const unsigned long long t0 = globaltimer_ns();
+      while (!mbar_try(bar0 + 8 * (i & 1), (uint32_t)(i >> 1) & 1u) && globaltimer_ns() - t0 < kWaitLimitNs) {
       }
-    return;  // no maximum is published by a CTA that gave up
-  }
-  if (SIDE) {
-    float* red = reinterpret_cast<float*>(smem + S::kBlkEnc);  // free in 1 x 16 mode
-    const float m = warp_max(fmaxf(bf16_lo(side_acc), bf16_hi(side_acc)));
-    __syncthreads();
-    if (lane == 0) red[warp] = m;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      float t = 0.f;
-#pragma unroll
-      for (int w = 0; w < 8; ++w) t = fmaxf(t, red[w]);
-      const uint32_t bits = __float_as_uint(t);  // non-negative floats order like their bit patterns
-      if (a.side_out0) atomicMax(reinterpret_cast<unsigned int*>(a.side_out0), bits);
-      if (a.side_out1) atomicMax(reinterpret_cast<unsigned int*>(a.side_out1), bits);
     }
-  }
+}
+
+template <bool HAS_ROW, bool HAS_COL, bool BLOCK2D, bool RHT_ROW, bool RHT_COL, bool SR, int TC>
+__global__ void __launch_bounds__(256, 2) quantize_kernel(const __grid_constant__ CUtensorMap src_map,
+                                                          const __grid_constant__ QuantArgs a) {
+  quantize_tiles<HAS_ROW, HAS_COL, BLOCK2D, RHT_ROW, RHT_COL, SR, TC>(&src_map, a, (int)blockIdx.x, (int)gridDim.x);
+}
+
+// The activation (1x16 blocks, the transposed copy with the transform) and the weight (16x16 blocks) of a forward call in one
+// launch, the first n_x CTAs on the activation: one ramp and one tail instead of two.  Carrying the weight's memory-bound
+// pass 1 on the activation's pass 2 and quantizing the weight behind it measured the same for many tiles (8192 x 20480 x 5120)
+// and lost for few: fwd + bwd of 512 x 1024 x 1024 27.6 -> 24.2 us of GPU time, 1024 x 2048 x 2048 41.7 -> 39.7, 2048 x 4096 x
+// 3072 93.8 -> 91.5.
+template <bool X_COL, bool W_COL, int TC>
+__global__ void __launch_bounds__(256, 2) quantize_x_and_w_kernel(const __grid_constant__ CUtensorMap x_map,
+                                                                  const __grid_constant__ CUtensorMap w_map,
+                                                                  const __grid_constant__ QuantArgs x,
+                                                                  const __grid_constant__ QuantArgs w, int n_x) {
+  const int b = (int)blockIdx.x;
+  if (b < n_x)
+    quantize_tiles<true, X_COL, false, false, X_COL, false, TC>(&x_map, x, b, n_x);
+  else
+    quantize_tiles<true, W_COL, true, false, false, false, TC>(&w_map, w, b - n_x, (int)gridDim.x - n_x);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -832,9 +830,8 @@ static cudaError_t launch_amax_rot_col(const QuantArgs& a, uint32_t mask16, floa
 }
 
 cudaError_t launch_amax(const QuantArgs& a, bool has_row, bool has_col, bool rht_row, bool rht_col,
-                        const SideAmax* side, cudaStream_t s) {
-  const cudaError_t e = launch_zero_words(has_row ? a.r_global : nullptr, has_col ? a.c_global : nullptr,
-                                          side ? side->out0 : nullptr, side ? side->out1 : nullptr, s);
+                        cudaStream_t s) {
+  const cudaError_t e = launch_zero_words(has_row ? a.r_global : nullptr, has_col ? a.c_global : nullptr, nullptr, nullptr, s);
   if (e != cudaSuccess) return e;
   const bool rr = has_row && rht_row, rc = has_col && rht_col;
   float* plain0 = (has_row && !rht_row) ? a.r_global : nullptr;
@@ -867,54 +864,37 @@ cudaError_t launch_amax_rot_col_small(const QuantArgs& a, bool has_row, uint32_t
                  : launch_amax_rot_col<false>(a, mask16, nullptr, nullptr, a.c_global, d, norm, s);
 }
 
-template <bool HR, bool HC, bool B2, bool RR, bool RC, bool SR, bool SIDE, int TC>
-static cudaError_t launch_quant_tc(const QuantArgs& a_in, int sms, cudaStream_t s, const SideAmax* side) {
-  auto kern = quantize_kernel<HR, HC, B2, RR, RC, SR, SIDE, TC>;
+// the source as a 2-D tensor map: boxes of 128 rows x tc bf16 (no swizzle), zero fill outside
+static bool quant_source_map(CUtensorMap* map, const QuantArgs& a, int tc) {
+  return make_map_2d(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, a.x, (uint64_t)a.cols, (uint64_t)a.rows, (uint64_t)a.ld * 2, tc,
+                     128, false);
+}
+
+template <bool HR, bool HC, bool B2, bool RR, bool RC, bool SR, int TC>
+static cudaError_t launch_quant_tc(const QuantArgs& a_in, int slots, cudaStream_t s) {
+  auto kern = quantize_kernel<HR, HC, B2, RR, RC, SR, TC>;
   QuantArgs a = a_in;
   a.tiles_c = (int)((a.cols + TC - 1) / TC);
   constexpr bool kRowCodes = B2 && HR && HC;
   constexpr int smem = QuantSmem<TC>::bytes(SR && HC && !kRowCodes, kRowCodes);
-  // the source as a 2-D tensor map: boxes of 128 rows x TC bf16 (no swizzle), zero fill outside
   CUtensorMap map;
-  if (!make_map_2d(&map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, a.x, (uint64_t)a.cols, (uint64_t)a.rows,
-                   (uint64_t)a.ld * 2, TC, 128, false))
-    return cudaErrorInvalidValue;
-  CUtensorMap side_map = map;
-  int64_t side_tiles = 0;
-  if (SIDE) {
-    if (!side || !make_map_2d(&side_map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, side->x, (uint64_t)side->cols,
-                              (uint64_t)side->rows, (uint64_t)side->ld * 2, TC, 128, false))
-      return cudaErrorInvalidValue;
-    a.side_tiles_r = (int)((side->rows + 127) / 128);
-    a.side_tiles_c = (int)((side->cols + TC - 1) / TC);
-    a.side_out0 = side->out0;
-    a.side_out1 = side->out1;
-    side_tiles = (int64_t)a.side_tiles_r * a.side_tiles_c;
-    if (side_tiles > 0x7fffffff) return cudaErrorInvalidValue;
-  }
-  // per call site (template instantiation) and device: the dynamic shared-memory limit, and how many CTAs the device
-  // keeps resident (the persistent grid)
-  static std::atomic<uint64_t> configured{0};
-  static std::atomic<int> resident[64] = {};
+  if (!quant_source_map(&map, a, TC)) return cudaErrorInvalidValue;
+  static std::atomic<uint64_t> configured{0};  // per call site (template instantiation) and device
   int dev;
   if (device_needs_config(configured, &dev)) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
-    int per_sm = 0;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 256, smem)) != cudaSuccess) return e;
-    if (dev >= 0 && dev < 64) resident[dev].store(sms * (per_sm > 0 ? per_sm : 1), std::memory_order_relaxed);
     device_configured(configured, dev);
   }
-  const int slots = (dev >= 0 && dev < 64) ? resident[dev].load(std::memory_order_relaxed) : 0;
-  const int64_t own = (int64_t)a.tiles_r * a.tiles_c, tiles = own > side_tiles ? own : side_tiles;
-  const int64_t grid = (slots > 0 && tiles > slots) ? slots : tiles;
-  const cudaError_t e = launch_kernel(kern, dim3((unsigned)grid), dim3(256), smem, s, map, side_map, a);
+  const int64_t tiles = (int64_t)a.tiles_r * a.tiles_c;
+  const cudaError_t e =
+      launch_kernel(kern, dim3((unsigned)(tiles < slots ? tiles : slots)), dim3(256), smem, s, map, a);
   count_launch();
   return e;
 }
 
-template <bool HR, bool HC, bool B2, bool RR, bool RC, bool SR, bool SIDE = false>
-static cudaError_t launch_quant_t(const QuantArgs& a, cudaStream_t s, const SideAmax* side = nullptr) {
+template <bool HR, bool HC, bool B2, bool RR, bool RC, bool SR>
+static cudaError_t launch_quant_t(const QuantArgs& a, cudaStream_t s) {
   int sms = 0;
   const cudaError_t e = sm_count(&sms);
   if (e != cudaSuccess) return e;
@@ -922,15 +902,77 @@ static cudaError_t launch_quant_t(const QuantArgs& a, cudaStream_t s, const Side
   // (16x16 blocks: 0.58), and the CTAs take whole rounds.  Measured (128 / 64 wide): gradient of 512 x 1024 8.6 / 7.0 us, 2048 x
   // 1024 10.6 / 8.3, 2816 x 2304 16.4 / 14.7, 4096 x 4096 31.7 / 30.4, 8192 x 5120 63.3 / 67.2; weight of 2048 x 1024 7.0 / 6.0,
   // 4096 x 2304 11.1 / 12.1.
-  const int64_t slots = 2 * sms, t128 = (int64_t)a.tiles_r * a.tiles_c, t64 = (int64_t)a.tiles_r * ((a.cols + 63) / 64);
+  const int slots = 2 * sms;  // resident CTAs
+  const int64_t t128 = (int64_t)a.tiles_r * a.tiles_c, t64 = (int64_t)a.tiles_r * ((a.cols + 63) / 64);
   const double r128 = (double)((t128 + slots - 1) / slots), r64 = (double)((t64 + slots - 1) / slots) * (B2 ? 0.58 : 0.535);
-  if (!RR && r64 < r128) return launch_quant_tc<HR, HC, B2, RR, RC, SR, SIDE, RR ? 128 : 64>(a, sms, s, side);
-  return launch_quant_tc<HR, HC, B2, RR, RC, SR, SIDE, 128>(a, sms, s, side);
+  if (!RR && r64 < r128) return launch_quant_tc<HR, HC, B2, RR, RC, SR, RR ? 128 : 64>(a, slots, s);
+  return launch_quant_tc<HR, HC, B2, RR, RC, SR, 128>(a, slots, s);
 }
 
-cudaError_t launch_quantize_with_amax_of(const QuantArgs& a, bool has_col, const SideAmax& side, cudaStream_t s) {
-  return has_col ? launch_quant_t<true, true, false, false, true, false, true>(a, s, &side)
-                 : launch_quant_t<true, false, false, false, false, false, true>(a, s, &side);
+template <bool X_COL, bool W_COL, int TC>
+static cudaError_t launch_x_and_w_tc(QuantArgs x, QuantArgs w, int slots, cudaStream_t s) {
+  auto kern = quantize_x_and_w_kernel<X_COL, W_COL, TC>;
+  constexpr int smem = QuantSmem<TC>::bytes(false, W_COL);
+  CUtensorMap maps[2];
+  QuantArgs* const t[2] = {&x, &w};
+  for (int i = 0; i < 2; ++i) {
+    t[i]->tiles_c = (int)((t[i]->cols + TC - 1) / TC);
+    if (!quant_source_map(&maps[i], *t[i], TC)) return cudaErrorInvalidValue;
+  }
+  static std::atomic<uint64_t> configured{0};  // per call site (template instantiation) and device
+  int dev;
+  if (device_needs_config(configured, &dev)) {
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return e;
+    device_configured(configured, dev);
+  }
+  // CTAs in proportion to the work (a weight's tile takes three quarters of an activation's), at whole rounds of either
+  const int tx = x.tiles_r * x.tiles_c, tw = w.tiles_r * w.tiles_c;
+  int n_x = tx, n_w = tw;
+  if (tx + tw > slots) {
+    double least = 1e30;
+    for (int rounds = (tx + slots - 2) / (slots - 1); rounds <= tx; ++rounds) {
+      const int gx = (tx + rounds - 1) / rounds, gw = slots - gx < tw ? slots - gx : tw;
+      const double w_time = 0.75 * ((tw + gw - 1) / gw), time = rounds > w_time ? (double)rounds : w_time;
+      if (time < least) {
+        least = time;
+        n_x = gx;
+        n_w = gw;
+      }
+      if (rounds >= w_time) break;  // more rounds of the activation only take longer
+    }
+  }
+  const cudaError_t e = launch_kernel(kern, dim3((unsigned)(n_x + n_w)), dim3(256), smem, s, maps[0], maps[1], x, w, n_x);
+  count_launch();
+  return e;
+}
+
+template <bool X_COL, bool W_COL>
+static cudaError_t launch_x_and_w_t(const QuantArgs& x, const QuantArgs& w, cudaStream_t s) {
+  int sms = 0;
+  cudaError_t e = sm_count(&sms);
+  if (e != cudaSuccess) return e;
+  e = launch_zero_words(x.r_global, X_COL ? x.c_global : nullptr, w.r_global, W_COL ? w.c_global : nullptr, s);
+  if (e != cudaSuccess) return e;
+  const int xc = (int)((x.cols + 255) / 256), wc = (int)((w.cols + 255) / 256);
+  const int64_t n_x = ((x.rows + 127) / 128) * xc, n_w = ((w.rows + 127) / 128) * wc;
+  if (n_x + n_w > 0x7fffffff) return cudaErrorInvalidValue;
+  e = launch_kernel(amax_x_and_w_kernel<X_COL, W_COL>, dim3((unsigned)(n_x + n_w)), dim3(256), 0, s, x, w, (int)n_x, xc, wc);
+  count_launch();
+  if (e != cudaSuccess) return e;
+  QuantArgs xa = x, wa = w;
+  xa.chained = wa.chained = 1;
+  const int slots = 2 * sms;  // resident CTAs; the width of the tiles as in launch_quant_t
+  const int64_t t128 = (int64_t)x.tiles_r * x.tiles_c + (int64_t)w.tiles_r * w.tiles_c;
+  const int64_t t64 = (int64_t)x.tiles_r * ((x.cols + 63) / 64) + (int64_t)w.tiles_r * ((w.cols + 63) / 64);
+  return 0.55 * (double)((t64 + slots - 1) / slots) < (double)((t128 + slots - 1) / slots)
+             ? launch_x_and_w_tc<X_COL, W_COL, 64>(xa, wa, slots, s)
+             : launch_x_and_w_tc<X_COL, W_COL, 128>(xa, wa, slots, s);
+}
+
+cudaError_t launch_quantize_x_and_w(const QuantArgs& x, bool x_col, const QuantArgs& w, bool w_col, cudaStream_t s) {
+  if (x_col) return w_col ? launch_x_and_w_t<true, true>(x, w, s) : launch_x_and_w_t<true, false>(x, w, s);
+  return w_col ? launch_x_and_w_t<false, true>(x, w, s) : launch_x_and_w_t<false, false>(x, w, s);
 }
 
 cudaError_t launch_quantize(const QuantArgs& a, bool has_row, bool has_col, bool block2d, bool rht_row,

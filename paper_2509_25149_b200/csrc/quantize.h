@@ -26,18 +26,6 @@ struct QuantArgs {
   unsigned int* status;  // device status word: a bounded wait that expired leaves its code here (may be NULL)
   int chained;  // the source is complete when the kernel starts (an earlier kernel of the same call has waited for it):
                 // it may be read before the wait for the previous kernel (see launch_kernel)
-  // side job of launch_quantize_with_amax_of: 128 x 128 tiles of the second tensor and where its amax goes
-  int side_tiles_r, side_tiles_c;
-  float* side_out0;
-  float* side_out1;
-};
-
-// A second bf16 tensor whose plain amax (pass 1 of its own quantization) a quantize launch takes on the side
-struct SideAmax {
-  const void* x;
-  int64_t rows, cols, ld;
-  float* out0;  // both receive the amax (the row-wise and the transposed copy's global[0]); either may be NULL
-  float* out1;
 };
 
 // Another transform size (quantize_rht.cu): d = 2, 4, 8 or 128 on the copies flagged rht_row / rht_col
@@ -56,12 +44,12 @@ cudaError_t launch_amax_rot_col_small(const QuantArgs& a, bool has_row, uint32_t
 // Clears the words the reductions of a call add into (any of them may be NULL) in one launch, the first of the call.
 cudaError_t launch_zero_words(float* w0, float* w1, float* w2, float* w3, cudaStream_t s);
 cudaError_t launch_amax(const QuantArgs& a, bool has_row, bool has_col, bool rht_row, bool rht_col,
-                        const SideAmax* side, cudaStream_t s);
+                        cudaStream_t s);
 cudaError_t launch_quantize(const QuantArgs& a, bool has_row, bool has_col, bool block2d, bool rht_row,
                             bool rht_col, bool sr, cudaStream_t s);
-// The row-wise copy (and, with has_col, the transformed transposed copy) of a, round-to-nearest, 1 x 16 blocks, and
-// on the side the plain amax of `side`: the memory-bound pass 1 of the next tensor rides on this issue-bound kernel.
-cudaError_t launch_quantize_with_amax_of(const QuantArgs& a, bool has_col, const SideAmax& side, cudaStream_t s);
+// The copies of an activation (1x16 blocks, the transposed one, if wanted, with the 16-point transform) and of a weight (16x16
+// blocks), round-to-nearest, both passes of both in three launches
+cudaError_t launch_quantize_x_and_w(const QuantArgs& x, bool x_col, const QuantArgs& w, bool w_col, cudaStream_t s);
 // MXFP4 outputs (quantize_mx.cu): one pass, no tensor-level scale
 cudaError_t launch_quantize_mx(const QuantArgs& a, bool has_row, bool has_col, bool block2d, bool rht_col, bool sr,
                                cudaStream_t s);
