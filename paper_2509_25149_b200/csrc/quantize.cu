@@ -261,6 +261,39 @@ __global__ void __launch_bounds__(256) amax_x_and_w_kernel(const __grid_constant
     amax_tile<true, false, false>(x.x, x.rows, x.cols, x.ld, 0u, b, x_tiles_c, x.r_global, nullptr, nullptr, nullptr);
 }
 
+// Pass 1 of a binary32 source: plain tensor amax.  CTA tile 128 rows x 128 columns; a warp owns 16 rows, a lane 4 columns of each.
+__global__ void __launch_bounds__(256) amax_f32_kernel(const float* __restrict__ x, int64_t rows, int64_t cols,
+                                                       int64_t ld, int tiles_c, float* __restrict__ out0,
+                                                       float* __restrict__ out1) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t tr = blockIdx.x / tiles_c, tc = blockIdx.x % tiles_c;
+  const int64_t r0 = tr * 128 + warp * 16, c0 = tc * 128 + lane * 4;
+  griddep_launch_dependents();  // pass 2 may load its tiles while the last CTAs of this pass run
+  float m = 0.f;  // (the source is complete: zero_words_kernel has waited for it)
+  if (r0 < rows && c0 < cols) {  // rows % 16 == 0, cols % 16 == 0
+    uint4 v[16];
+#pragma unroll
+    for (int j = 0; j < 16; ++j) v[j] = ldg128_stream(x + (r0 + j) * ld + c0);
+#pragma unroll
+    for (int j = 0; j < 16; ++j)
+      m = fmaxf(fmaxf(m, fmaxf(fabsf(__uint_as_float(v[j].x)), fabsf(__uint_as_float(v[j].y)))),
+                fmaxf(fabsf(__uint_as_float(v[j].z)), fabsf(__uint_as_float(v[j].w))));
+  }
+  __shared__ float red[8];
+  m = warp_max(m);
+  if (lane == 0) red[warp] = m;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    griddep_wait();  // the words are zero
+    float t = 0.f;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) t = fmaxf(t, red[w]);
+    const uint32_t bits = __float_as_uint(t);  // non-negative floats order like their bit patterns
+    if (out0) atomicMax(reinterpret_cast<unsigned int*>(out0), bits);
+    if (out1) atomicMax(reinterpret_cast<unsigned int*>(out1), bits);
+  }
+}
+
 // ---------------------------------------------------------------------------------------------
 // Pass 2: persistent CTAs (two per SM), each working through tiles of 128 rows x 128 (few tiles: 64) columns of the source.
 // The tiles arrive by TMA (cp.async.bulk.tensor, this GPU's memory, no multicast) in a ring of two buffers: the load of tile
@@ -278,13 +311,13 @@ __global__ void __launch_bounds__(256) amax_x_and_w_kernel(const __grid_constant
 // buffered, so a tile needs one CTA barrier.  Tiles are visited in reverse order so that the end of the tensor,
 // which pass 1 touched last, is read first while it may still sit in L2.
 // ---------------------------------------------------------------------------------------------
-// TC: columns of a tile.
-template <int TC>
+// TC: columns of a tile; F32: the source is binary32 (tiles of 64 columns).
+template <int TC, bool F32 = false>
 struct QuantSmem {
   static constexpr int kChunks = TC / 16;                // 1x16 chunks per tile row
-  static constexpr int kRow = 2 * TC;                    // bytes per tile row
+  static constexpr int kRow = (F32 ? 4 : 2) * TC;        // bytes per tile row
   static constexpr int kTileBytes = 128 * kRow;
-  static constexpr int kTile = 0;                        // 2 tiles of bf16, filled by TMA
+  static constexpr int kTile = 0;                        // 2 tiles, filled by TMA
   static constexpr int kColBytes = TC * 64;
   static constexpr int kColCodes = 2 * kTileBytes;       // 2 x (TC columns x 64 B)
   static constexpr int kSfBytes = 8 * TC;                // 128 rows x kChunks bytes, or TC columns x 8
@@ -336,10 +369,10 @@ __device__ __forceinline__ void store_linear_scales(const uint8_t* src, uint8_t*
     if (full_tile || (R0 + r + 256 / KB * p < Rn && K0 + kb < n_kb)) *d = src[threadIdx.x + 256 * p];
 }
 
-template <bool HAS_ROW, bool HAS_COL, bool BLOCK2D, bool RHT_ROW, bool RHT_COL, bool SR, int TC>
+template <bool HAS_ROW, bool HAS_COL, bool BLOCK2D, bool RHT_ROW, bool RHT_COL, bool SR, int TC, bool F32 = false>
 __device__ __forceinline__ void quantize_tiles(const CUtensorMap* src_map, const QuantArgs& a, const int block,
                                                const int blocks) {  // this CTA among those of the tensor
-  using S = QuantSmem<TC>;
+  using S = QuantSmem<TC, F32>;
   constexpr int CH = S::kChunks;          // chunks per tile row
   constexpr int RPP = 32 / CH;            // rows a warp covers with one chunk per lane; chunk i of a lane: RPP * i rows down
   constexpr int NP = 16 / RPP;            // chunks per lane
@@ -415,11 +448,14 @@ __device__ __forceinline__ void quantize_tiles(const CUtensorMap* src_map, const
 
   // per-thread constants of phase 1: chunk column cb, row rl + RPP * i for chunk i
   const int cb = lane % CH, rl = warp * 16 + lane / CH;
-  const uint32_t tile_ld = rl * S::kRow + cb * 32;     // chunk i of the thread inside a tile buffer: + RPP * kRow * i
+  const uint32_t tile_ld = rl * S::kRow + cb * (F32 ? 64 : 32);  // chunk i of the thread inside a tile buffer: + RPP * kRow * i
   const uint32_t rand_st = S::kRand + rl * TC + cb * 16;  // + RPP * TC * i
   const int sf_row_pos = a.r_swz ? ((cb >> 2) * 512 + (rl & 31) * 16 + (rl >> 5) * 4 + (cb & 3)) : (rl * CH + cb);
   const int sf_row_step = a.r_swz ? RPP * 16 : RPP * CH;
   const int64_t r_pitch = a.cols >> 1;  // bytes per row of the row-wise codes
+  // F32: a lane reads the four 16-byte quarters of a chunk beginning with its own rot-th, so that the eight lanes of a quarter
+  // warp (chunks 64 bytes, rows 256 bytes apart) cover all banks; the codes are rotated back into place
+  const int rot = ((cb >> 1) + 2 * (rl & 1)) & 3;
 
   // hoisted constants of phase 2: where a thread stages its two columns' codes and scale bytes (iteration it, column
   // parity odd); the 16-byte unit of column pair cp and 16-row group q sits at cp * 128 + ((q ^ cp) & 7) * 16
@@ -449,13 +485,15 @@ __device__ __forceinline__ void quantize_tiles(const CUtensorMap* src_map, const
       // ---------------------------------------------------------------- phase 1 ----
       const int rows_left = FULL ? 128 : (int)(a.rows - row0) - rl;         // chunk i exists iff RPP * i < rows_left
       const bool col_ok = FULL || (col0 + cb * 16 < a.cols);
-      uint32_t raw[NP][8];
+      uint32_t raw[NP][F32 ? 16 : 8];  // F32: quarter rot first
 #pragma unroll
       for (int i = 0; i < NP; ++i) {
-        const uint4 h0 = *reinterpret_cast<const uint4*>(tile_buf + tile_ld + i * (RPP * S::kRow));
-        const uint4 h1 = *reinterpret_cast<const uint4*>(tile_buf + tile_ld + i * (RPP * S::kRow) + 16);
-        raw[i][0] = h0.x; raw[i][1] = h0.y; raw[i][2] = h0.z; raw[i][3] = h0.w;
-        raw[i][4] = h1.x; raw[i][5] = h1.y; raw[i][6] = h1.z; raw[i][7] = h1.w;
+        const uint8_t* const src = tile_buf + tile_ld + i * (RPP * S::kRow);
+#pragma unroll
+        for (int h = 0; h < (F32 ? 4 : 2); ++h) {
+          const uint4 v = *reinterpret_cast<const uint4*>(src + (F32 ? ((h + rot) & 3) : h) * 16);
+          raw[i][4 * h] = v.x; raw[i][4 * h + 1] = v.y; raw[i][4 * h + 2] = v.z; raw[i][4 * h + 3] = v.w;
+        }
       }
 
       uint32_t blk_byte = 0;
@@ -464,10 +502,16 @@ __device__ __forceinline__ void quantize_tiles(const CUtensorMap* src_map, const
         float blk_amax = 0.f;
 #pragma unroll
         for (int i = 0; i < NP; ++i) {
-          uint32_t acc = 0;
+          if constexpr (F32) {
 #pragma unroll
-          for (int k = 0; k < 8; ++k) acc = absmax_bf16x2(acc, raw[i][k]);
-          blk_amax = fmaxf(blk_amax, fmaxf(bf16_lo(acc), bf16_hi(acc)));
+            for (int k = 0; k < 16; k += 2)
+              blk_amax = amax3(blk_amax, __uint_as_float(raw[i][k]), __uint_as_float(raw[i][k + 1]));
+          } else {
+            uint32_t acc = 0;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) acc = absmax_bf16x2(acc, raw[i][k]);
+            blk_amax = fmaxf(blk_amax, fmaxf(bf16_lo(acc), bf16_hi(acc)));
+          }
         }
 #pragma unroll
         for (int o = CH; o < 32; o <<= 1) blk_amax = fmaxf(blk_amax, __shfl_xor_sync(0xffffffffu, blk_amax, o));
@@ -498,14 +542,25 @@ __device__ __forceinline__ void quantize_tiles(const CUtensorMap* src_map, const
         }
         if (HAS_ROW) {
           float f[16];
+          if constexpr (F32) {
 #pragma unroll
-          for (int k = 0; k < 8; ++k) {
-            uint32_t word = raw[i][k];
-            if (RHT_ROW) word ^= sign_pair(a.sign_mask, 2 * k, 2 * k + 1);
-            f[2 * k] = bf16_lo(word);
-            f[2 * k + 1] = bf16_hi(word);
+            for (int k = 0; k < 16; ++k) f[k] = __uint_as_float(raw[i][k]);
+            if (SR) {  // the draws of the quarters in the order they were read
+              const uint32_t a0 = (rot & 1) ? rnd[1] : rnd[0], a1 = (rot & 1) ? rnd[2] : rnd[1];
+              const uint32_t a2 = (rot & 1) ? rnd[3] : rnd[2], a3 = (rot & 1) ? rnd[0] : rnd[3];
+              rnd[0] = (rot & 2) ? a2 : a0; rnd[1] = (rot & 2) ? a3 : a1;
+              rnd[2] = (rot & 2) ? a0 : a2; rnd[3] = (rot & 2) ? a1 : a3;
+            }
+          } else {
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+              uint32_t word = raw[i][k];
+              if (RHT_ROW) word ^= sign_pair(a.sign_mask, 2 * k, 2 * k + 1);
+              f[2 * k] = bf16_lo(word);
+              f[2 * k + 1] = bf16_hi(word);
+            }
+            if (RHT_ROW) fwht16(f);  // values are 4 * y from here on
           }
-          if (RHT_ROW) fwht16(f);  // values are 4 * y from here on
           uint32_t byte;
           float enc;
           if (BLOCK2D) {
@@ -516,7 +571,11 @@ __device__ __forceinline__ void quantize_tiles(const CUtensorMap* src_map, const
             byte = block_scale_byte(RHT_ROW ? 0.25f * m : m, r_senc);
             enc = enc_row[byte];
           }
-          const uint2 codes = convert16<SR>(f, enc, Nu14FromWords{rnd});
+          uint2 codes = convert16<SR>(f, enc, Nu14FromWords{rnd});
+          if (F32) {  // 64-bit rotation to the left by rot quarters of 16 bits
+            const uint32_t x = (rot & 2) ? codes.y : codes.x, y = (rot & 2) ? codes.x : codes.y;
+            codes = make_uint2(__funnelshift_l(y, x, (rot & 1) * 16), __funnelshift_l(x, y, (rot & 1) * 16));
+          }
           if (FULL || (col_ok && RPP * i < rows_left))
             *reinterpret_cast<uint2*>(r_out + (int64_t)(RPP * i) * r_pitch) = codes;
           if (kNibbleTranspose)  // row r, bytes [8 cb, 8 cb + 8): byte k = columns (2k, 2k + 1) of the chunk
@@ -565,9 +624,13 @@ __device__ __forceinline__ void quantize_tiles(const CUtensorMap* src_map, const
             continue;
           }
           float2 v[16];  // rows of the group, (column 2cp, column 2cp + 1)
-          const uint8_t* tp = tile_buf + q * 16 * S::kRow + cp * 4;
+          const uint8_t* tp = tile_buf + q * 16 * S::kRow + cp * (F32 ? 8 : 4);
 #pragma unroll
           for (int j = 0; j < 16; ++j) {
+            if (F32) {
+              v[j] = *reinterpret_cast<const float2*>(tp + j * S::kRow);
+              continue;
+            }
             uint32_t word = *reinterpret_cast<const uint32_t*>(tp + j * S::kRow);
             if (RHT_COL) word ^= a.row_sign[j];
             v[j] = make_float2(bf16_lo(word), bf16_hi(word));
@@ -698,10 +761,10 @@ __device__ __forceinline__ void quantize_tiles(const CUtensorMap* src_map, const
     }
 }
 
-template <bool HAS_ROW, bool HAS_COL, bool BLOCK2D, bool RHT_ROW, bool RHT_COL, bool SR, int TC>
+template <bool HAS_ROW, bool HAS_COL, bool BLOCK2D, bool RHT_ROW, bool RHT_COL, bool SR, int TC, bool F32 = false>
 __global__ void __launch_bounds__(256, 2) quantize_kernel(const __grid_constant__ CUtensorMap src_map,
                                                           const __grid_constant__ QuantArgs a) {
-  quantize_tiles<HAS_ROW, HAS_COL, BLOCK2D, RHT_ROW, RHT_COL, SR, TC>(&src_map, a, (int)blockIdx.x, (int)gridDim.x);
+  quantize_tiles<HAS_ROW, HAS_COL, BLOCK2D, RHT_ROW, RHT_COL, SR, TC, F32>(&src_map, a, (int)blockIdx.x, (int)gridDim.x);
 }
 
 // The activation (1x16 blocks, the transposed copy with the transform) and the weight (16x16 blocks) of a forward call in one
@@ -864,21 +927,21 @@ cudaError_t launch_amax_rot_col_small(const QuantArgs& a, bool has_row, uint32_t
                  : launch_amax_rot_col<false>(a, mask16, nullptr, nullptr, a.c_global, d, norm, s);
 }
 
-// the source as a 2-D tensor map: boxes of 128 rows x tc bf16 (no swizzle), zero fill outside
-static bool quant_source_map(CUtensorMap* map, const QuantArgs& a, int tc) {
-  return make_map_2d(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, a.x, (uint64_t)a.cols, (uint64_t)a.rows, (uint64_t)a.ld * 2, tc,
-                     128, false);
+// the source as a 2-D tensor map: boxes of 128 rows x tc elements (no swizzle), zero fill outside
+static bool quant_source_map(CUtensorMap* map, const QuantArgs& a, int tc, bool f32 = false) {
+  return make_map_2d(map, f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, f32 ? 4 : 2, a.x,
+                     (uint64_t)a.cols, (uint64_t)a.rows, (uint64_t)a.ld * (f32 ? 4 : 2), tc, 128, false);
 }
 
-template <bool HR, bool HC, bool B2, bool RR, bool RC, bool SR, int TC>
+template <bool HR, bool HC, bool B2, bool RR, bool RC, bool SR, int TC, bool F32 = false>
 static cudaError_t launch_quant_tc(const QuantArgs& a_in, int slots, cudaStream_t s) {
-  auto kern = quantize_kernel<HR, HC, B2, RR, RC, SR, TC>;
+  auto kern = quantize_kernel<HR, HC, B2, RR, RC, SR, TC, F32>;
   QuantArgs a = a_in;
   a.tiles_c = (int)((a.cols + TC - 1) / TC);
   constexpr bool kRowCodes = B2 && HR && HC;
-  constexpr int smem = QuantSmem<TC>::bytes(SR && HC && !kRowCodes, kRowCodes);
+  constexpr int smem = QuantSmem<TC, F32>::bytes(SR && HC && !kRowCodes, kRowCodes);
   CUtensorMap map;
-  if (!quant_source_map(&map, a, TC)) return cudaErrorInvalidValue;
+  if (!quant_source_map(&map, a, TC, F32)) return cudaErrorInvalidValue;
   static std::atomic<uint64_t> configured{0};  // per call site (template instantiation) and device
   int dev;
   if (device_needs_config(configured, &dev)) {
@@ -998,6 +1061,39 @@ cudaError_t launch_quantize(const QuantArgs& a, bool has_row, bool has_col, bool
   NVFP4_Q_COPIES(false, true, true, true)
 #undef NVFP4_Q_COPIES
 #undef NVFP4_Q
+  return cudaErrorInvalidValue;
+}
+
+cudaError_t launch_amax_f32(const QuantArgs& a, bool has_row, bool has_col, cudaStream_t s) {
+  cudaError_t e = launch_zero_words(has_row ? a.r_global : nullptr, has_col ? a.c_global : nullptr, nullptr, nullptr, s);
+  if (e != cudaSuccess) return e;
+  const int tiles_c = (int)((a.cols + 127) / 128);
+  const unsigned tiles = (unsigned)(((a.rows + 127) / 128) * tiles_c);
+  e = launch_kernel(amax_f32_kernel, dim3(tiles), dim3(256), 0, s, reinterpret_cast<const float*>(a.x), a.rows, a.cols,
+                    a.ld, tiles_c, has_row ? a.r_global : nullptr, has_col ? a.c_global : nullptr);
+  count_launch();
+  return e;
+}
+
+// binary32 source (Appendix B names FP32 as well as BF16 as the precision converted from), e.g. weights quantized straight from
+// their FP32 master copy; no transform (the recipe transforms activations and gradients, which are bf16)
+cudaError_t launch_quantize_f32(const QuantArgs& a, bool has_row, bool has_col, bool block2d, bool sr, cudaStream_t s) {
+  int sms = 0;
+  const cudaError_t e = sm_count(&sms);
+  if (e != cudaSuccess) return e;
+#define NVFP4_F32Q(HR, HC, B2, SRV)                                              \
+  if (has_row == HR && has_col == HC && block2d == B2 && sr == SRV)              \
+    return launch_quant_tc<HR, HC, B2, false, false, SRV, 64, true>(a, 2 * sms, s);
+#define NVFP4_F32Q_COPIES(B2, SRV) \
+  NVFP4_F32Q(true, false, B2, SRV)  \
+  NVFP4_F32Q(false, true, B2, SRV)  \
+  NVFP4_F32Q(true, true, B2, SRV)
+  NVFP4_F32Q_COPIES(true, false)
+  NVFP4_F32Q_COPIES(true, true)
+  NVFP4_F32Q_COPIES(false, false)
+  NVFP4_F32Q_COPIES(false, true)
+#undef NVFP4_F32Q_COPIES
+#undef NVFP4_F32Q
   return cudaErrorInvalidValue;
 }
 

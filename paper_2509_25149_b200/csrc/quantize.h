@@ -53,7 +53,7 @@ cudaError_t launch_quantize_x_and_w(const QuantArgs& x, bool x_col, const QuantA
 // MXFP4 outputs (quantize_mx.cu): one pass, no tensor-level scale
 cudaError_t launch_quantize_mx(const QuantArgs& a, bool has_row, bool has_col, bool block2d, bool rht_col, bool sr,
                                cudaStream_t s);
-// binary32 source (quantize_f32.cu): plain amax pass and the quantize pass, no transform
+// binary32 source: plain amax pass and the quantize pass, no transform
 cudaError_t launch_amax_f32(const QuantArgs& a, bool has_row, bool has_col, cudaStream_t s);
 cudaError_t launch_quantize_f32(const QuantArgs& a, bool has_row, bool has_col, bool block2d, bool sr, cudaStream_t s);
 cudaError_t launch_dequantize(const nvfp4_tensor& t, float* out, cudaStream_t s);
