@@ -238,7 +238,8 @@ NVFP4_API nvfp4_status nvfp4_sq_error(const void* ref, int32_t ref_is_fp32, int6
  *   finished before their first kernel starts, and their results are complete for whatever is enqueued after
  *   them).  The kernels of this library overlap only their set-up with the tail of the kernel before them
  *   (programmatic dependent launch) and never read each other's output early; in the NVFP4 bf16 path X and a fresh W
- *   are quantized by the same launches.  Results are bit-identical to the same steps issued one by one through
+ *   are quantized by the same launches.  Y and dX also serve as scratch before the product is written (not where they
+ *   lie over an input).  Results are bit-identical to the same steps issued one by one through
  *   nvfp4_quantize and nvfp4_gemm.
  * Format: the layer runs in the format of the copies it is given (W_row / W_col_saved / X_col_saved must
  *   agree).  With MXFP4 copies the same sequence uses 1x32 and 32x32 blocks and the 32-point transform

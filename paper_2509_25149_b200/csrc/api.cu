@@ -64,11 +64,22 @@ nvfp4_status fill_quant_args(const void* x, int64_t rows, int64_t cols, int64_t 
   return NVFP4_OK;
 }
 
+// Room for the maxima of pass 1's tiles: an output which the call writes last, unless an input lies in the same memory
+float2* parts_in(void* out, int64_t out_bytes, const void* in0, int64_t bytes0, const void* in1 = nullptr, int64_t bytes1 = 0) {
+  const char* const o = static_cast<const char*>(out);
+  auto apart = [&](const void* in, int64_t n) {
+    const char* const p = static_cast<const char*>(in);
+    return !p || p + n <= o || o + out_bytes <= p;
+  };
+  return apart(in0, bytes0) && apart(in1, bytes1) ? static_cast<float2*>(out) : nullptr;
+}
+
+// parts: room for pass 1's maxima if it may leave them in parts (an activation or a gradient of a layer).
 // check_only: every argument check of the call, no launch (the composed calls validate all their steps first, so
 // that a rejected call has enqueued nothing)
 nvfp4_status quantize_impl(const void* x, int64_t rows, int64_t cols, int64_t ld, const nvfp4_quant_opts* o,
                            const nvfp4_tensor* rowwise, const nvfp4_tensor* colwise, cudaStream_t s,
-                           bool check_only = false) {
+                           bool check_only = false, float2* parts = nullptr) {
   if (!x || !o) return NVFP4_ERR_NULL;
   if (!rowwise && !colwise) return NVFP4_ERR_NULL;
   if (rows <= 0 || cols <= 0 || rows % 16 != 0 || cols % 16 != 0) return NVFP4_ERR_SHAPE;
@@ -158,6 +169,10 @@ nvfp4_status quantize_impl(const void* x, int64_t rows, int64_t cols, int64_t ld
                                                                                                   : NVFP4_ERR_CUDA;
   }
   if (!(o->flags & NVFP4_AMAX_PROVIDED)) {
+    if (parts && pass1_in_parts(amax_parts(rows, cols))) {
+      a.parts = parts;
+      a.n_parts = (int)amax_parts(rows, cols);
+    }
     if (launch_amax(a, hr, hc, o->rht_rowwise != 0, o->rht_colwise != 0, s) != cudaSuccess) return NVFP4_ERR_CUDA;
     a.chained = 1;
   }
@@ -338,17 +353,23 @@ nvfp4_status nvfp4_linear_fwd(const void* X, const void* W, int64_t M, int64_t N
   if (!w_is_cached && (st = quantize_impl(W, N, K, K, &wo, W_row, W_col_saved, s, true)) != NVFP4_OK) return st;
   if ((st = quantize_impl(X, M, K, K, &xo, &x_row, X_col_saved, s, true)) != NVFP4_OK) return st;
   if ((st = gemm_prepare(&x_row, W_row, Y_bf16, 0, N, 0, gy)) != NVFP4_OK) return st;
+  float2* const parts = parts_in(Y_bf16, 2 * M * N, X, 2 * M * K, W, 2 * N * K);
   if (!w_is_cached && fmt == NVFP4_FORMAT_NVFP4 && (xo.rht_dim == 0 || xo.rht_dim == 16)) {
     // both tensors in the same launches (the kernels of the other formats and transform sizes take one tensor each)
     QuantArgs xa, wa;
     if ((st = fill_quant_args(X, M, K, K, &xo, &x_row, X_col_saved, false, xa)) != NVFP4_OK) return st;
     if ((st = fill_quant_args(W, N, K, K, &wo, W_row, W_col_saved, false, wa)) != NVFP4_OK) return st;
+    const int64_t n_x = amax_parts(M, K), n_w = amax_parts(N, K);
+    if (parts && pass1_in_parts(n_x + n_w)) {
+      xa.parts = parts; xa.n_parts = (int)n_x;
+      wa.parts = parts + n_x; wa.n_parts = (int)n_w;
+    }
     if (launch_quantize_x_and_w(xa, X_col_saved != nullptr, wa, W_col_saved != nullptr, s) != cudaSuccess)
       return NVFP4_ERR_CUDA;
     return gemm_impl(&x_row, W_row, Y_bf16, 0, N, 0, s);
   }
   if (!w_is_cached && (st = quantize_impl(W, N, K, K, &wo, W_row, W_col_saved, s)) != NVFP4_OK) return st;
-  if ((st = quantize_impl(X, M, K, K, &xo, &x_row, X_col_saved, s)) != NVFP4_OK) return st;
+  if ((st = quantize_impl(X, M, K, K, &xo, &x_row, X_col_saved, s, false, parts)) != NVFP4_OK) return st;
   return gemm_impl(&x_row, W_row, Y_bf16, 0, N, 0, s);
 }
 
@@ -391,7 +412,10 @@ nvfp4_status nvfp4_linear_bwd(const void* dY, const nvfp4_tensor* X_col_saved, c
     if (dX_bf16 && (st = gemm_prepare(&g_row, W_col_saved, dX_bf16, 0, K, 0, gchk)) != NVFP4_OK) return st;
     if (dW_fp32 && (st = gemm_prepare(&g_col, X_col_saved, dW_fp32, 1, K, accumulate_dw, gchk)) != NVFP4_OK) return st;
   }
-  if ((st = quantize_impl(dY, M, N, N, &go, dX_bf16 ? &g_row : nullptr, dW_fp32 ? &g_col : nullptr, s)) != NVFP4_OK)
+  // without a dX the workspace's row-wise copy is free
+  float2* const parts = dX_bf16 ? parts_in(dX_bf16, 2 * M * K, dY, 2 * M * N) : reinterpret_cast<float2*>(g_row.codes);
+  if ((st = quantize_impl(dY, M, N, N, &go, dX_bf16 ? &g_row : nullptr, dW_fp32 ? &g_col : nullptr, s, false, parts)) !=
+      NVFP4_OK)
     return st;
   if (dX_bf16 && dW_fp32) {
     // Dgrad and Wgrad are independent: when both run on CTA pairs they share one launch, the longer contraction

@@ -62,7 +62,8 @@ __device__ __forceinline__ void fence_proxy_async_smem() { asm volatile("fence.p
 //   - every kernel waits before it finishes, so "kernel n has finished" implies "kernel n - 1 has finished";
 //   - before its wait a kernel touches only what no kernel that may still run writes: the kernel that zeroes the words of
 //     a call (zero_words_kernel) waits first and only then lets its dependent start, so the reductions behind it may read
-//     their inputs at once and wait just before their first atomic.
+//     their inputs at once and wait just before their first atomic (a reduction that is the first
+//     kernel of its call waits and lets its dependent start in the same order).
 __device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // lets the next kernel of the stream, if it was launched that way, become resident as CTAs of this grid retire
 __device__ __forceinline__ void griddep_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }

@@ -7,6 +7,7 @@
 #include <cuda_fp16.h>
 
 #include <type_traits>
+#include <utility>
 
 #include "async_ptx.cuh"
 #include "common.cuh"
@@ -15,23 +16,34 @@
 
 namespace nvfp4 {
 
+// Pass 1 without words to clear: the {plain, transformed} maximum of a tile goes to a place of its own and pass 2 takes the
+// maximum over the places.  For small tensors, see pass1_in_parts().
+__device__ __forceinline__ void store_part(float2* part, const float (&plain)[8], const float (&rot)[8]) {
+  if (threadIdx.x != 0) return;
+  float2 m = make_float2(plain[0], rot[0]);
+#pragma unroll
+  for (int w = 1; w < 8; ++w) m = make_float2(fmaxf(m.x, plain[w]), fmaxf(m.y, rot[w]));
+  *part = m;
+}
+
 // ---------------------------------------------------------------------------------------------
 // Pass 1: tensor amax (Appendix B.1), plain and / or in the rotated space of a transformed copy.
 // CTA tile 128 rows x 256 columns; a warp owns 16 rows, a lane 8 columns of each of them.
 // ---------------------------------------------------------------------------------------------
-template <bool PLAIN, bool ROT_ROW, bool ROT_COL>
+template <bool PLAIN, bool ROT_ROW, bool ROT_COL, bool PARTS>
 __device__ __forceinline__ void amax_tile(const uint16_t* __restrict__ x, int64_t rows, int64_t cols, int64_t ld,
                                           uint32_t sign_mask, int tile, int tiles_c, float* __restrict__ out_plain0,
                                           float* __restrict__ out_plain1, float* __restrict__ out_rot_row,
-                                          float* __restrict__ out_rot_col) {
+                                          float* __restrict__ out_rot_col, float2* __restrict__ parts) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t tr = tile / tiles_c, tc = tile % tiles_c;
   const int64_t r0 = tr * 128 + warp * 16;
   const int64_t c0 = tc * 256 + lane * 8;
   const bool in_range = (r0 < rows) && (c0 < cols);  // rows % 16 == 0, cols % 8 == 0
+  if (PARTS) griddep_wait();    // the first kernel of its call; otherwise zero_words_kernel has waited for the source
   griddep_launch_dependents();  // pass 2 may set itself up while the last CTAs of this pass run
 
-  uint4 raw[16];  // (the source is complete: zero_words_kernel has waited for it)
+  uint4 raw[16];
   if (in_range) {
     const uint16_t* p = x + r0 * ld + c0;
 #pragma unroll
@@ -114,7 +126,9 @@ __device__ __forceinline__ void amax_tile(const uint16_t* __restrict__ x, int64_
     red[2][warp] = m_col;
   }
   __syncthreads();
-  if (threadIdx.x < 3) {
+  if (PARTS) {
+    store_part(parts + tile, red[0], red[2]);
+  } else if (threadIdx.x < 3) {
     griddep_wait();  // the words are zero
     float m = 0.f;
 #pragma unroll
@@ -130,13 +144,13 @@ __device__ __forceinline__ void amax_tile(const uint16_t* __restrict__ x, int64_
   }
 }
 
-template <bool PLAIN, bool ROT_ROW, bool ROT_COL>
+template <bool PLAIN, bool ROT_ROW, bool ROT_COL, bool PARTS>
 __global__ void __launch_bounds__(256) amax_kernel(const uint16_t* __restrict__ x, int64_t rows, int64_t cols, int64_t ld,
                                                    uint32_t sign_mask, int tiles_c, float* __restrict__ out_plain0,
                                                    float* __restrict__ out_plain1, float* __restrict__ out_rot_row,
-                                                   float* __restrict__ out_rot_col) {
-  amax_tile<PLAIN, ROT_ROW, ROT_COL>(x, rows, cols, ld, sign_mask, (int)blockIdx.x, tiles_c, out_plain0, out_plain1,
-                                     out_rot_row, out_rot_col);
+                                                   float* __restrict__ out_rot_col, float2* __restrict__ parts) {
+  amax_tile<PLAIN, ROT_ROW, ROT_COL, PARTS>(x, rows, cols, ld, sign_mask, (int)blockIdx.x, tiles_c, out_plain0, out_plain1,
+                                            out_rot_row, out_rot_col, parts);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -156,16 +170,17 @@ __device__ __forceinline__ uint32_t movmatrix_trans(uint32_t v) {
 
 // d, norm: size of the transform (2, 4, 8 or 16: H_16 is replaced by the block-diagonal matrix of 16 / d copies of
 // H_d) and its normalisation 1 / sqrt(d), applied to the maximum.
-template <bool PLAIN>
+template <bool PLAIN, bool PARTS>
 __device__ __forceinline__ void amax_rot_col_tile(const uint16_t* __restrict__ x, int64_t rows, int64_t cols, int64_t ld,
                                                   uint32_t sign_mask, int tile, int tiles_c, float* __restrict__ out_plain0,
                                                   float* __restrict__ out_plain1, float* __restrict__ out_rot_col, int d,
-                                                  float norm) {
+                                                  float norm, float2* __restrict__ parts) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int g = lane >> 2, t = lane & 3;
   const int64_t tr = tile / tiles_c, tc = tile % tiles_c;
   const int64_t r0 = tr * 128 + warp * 16;
-  griddep_launch_dependents();  // pass 2 may set itself up while the last CTAs of this pass run
+  if (PARTS) griddep_wait();  // as in amax_tile
+  griddep_launch_dependents();
 
   uint32_t lo[4][8], hi[4][8];  // rows g and g + 8 of the slab, 16 columns each, four 64-column steps
 #pragma unroll
@@ -223,7 +238,9 @@ __device__ __forceinline__ void amax_rot_col_tile(const uint16_t* __restrict__ x
     red[1][warp] = m_col;
   }
   __syncthreads();
-  if (threadIdx.x < 2) {
+  if (PARTS) {
+    store_part(parts + tile, red[0], red[1]);
+  } else if (threadIdx.x < 2) {
     griddep_wait();  // the words are zero
     float m = 0.f;
 #pragma unroll
@@ -237,28 +254,31 @@ __device__ __forceinline__ void amax_rot_col_tile(const uint16_t* __restrict__ x
   }
 }
 
-template <bool PLAIN>
+template <bool PLAIN, bool PARTS>
 __global__ void __launch_bounds__(256) amax_rot_col_kernel(const uint16_t* __restrict__ x, int64_t rows, int64_t cols,
                                                            int64_t ld, uint32_t sign_mask, int tiles_c,
                                                            float* __restrict__ out_plain0, float* __restrict__ out_plain1,
-                                                           float* __restrict__ out_rot_col, int d, float norm) {
-  amax_rot_col_tile<PLAIN>(x, rows, cols, ld, sign_mask, (int)blockIdx.x, tiles_c, out_plain0, out_plain1, out_rot_col, d,
-                           norm);
+                                                           float* __restrict__ out_rot_col, int d, float norm,
+                                                           float2* __restrict__ parts) {
+  amax_rot_col_tile<PLAIN, PARTS>(x, rows, cols, ld, sign_mask, (int)blockIdx.x, tiles_c, out_plain0, out_plain1,
+                                  out_rot_col, d, norm, parts);
 }
 
 // Pass 1 of two tensors in one launch (see quantize_x_and_w_kernel): the first n_x CTAs take tiles of an activation (row-wise
 // copy plain, transposed copy rotated), the others of a weight (plain).
-template <bool X_COL, bool W_COL>
+template <bool X_COL, bool W_COL, bool PARTS>
 __global__ void __launch_bounds__(256) amax_x_and_w_kernel(const __grid_constant__ QuantArgs x, const __grid_constant__ QuantArgs w,
                                                            int n_x, int x_tiles_c, int w_tiles_c) {
   const int b = (int)blockIdx.x;
   if (b >= n_x)
-    amax_tile<true, false, false>(w.x, w.rows, w.cols, w.ld, 0u, b - n_x, w_tiles_c, w.r_global, W_COL ? w.c_global : nullptr,
-                                  nullptr, nullptr);
+    amax_tile<true, false, false, PARTS>(w.x, w.rows, w.cols, w.ld, 0u, b - n_x, w_tiles_c, w.r_global, W_COL ? w.c_global : nullptr,
+                                  nullptr, nullptr, w.parts);
   else if (X_COL)
-    amax_rot_col_tile<true>(x.x, x.rows, x.cols, x.ld, x.sign_mask, b, x_tiles_c, x.r_global, nullptr, x.c_global, 16, 0.25f);
+    amax_rot_col_tile<true, PARTS>(x.x, x.rows, x.cols, x.ld, x.sign_mask, b, x_tiles_c, x.r_global, nullptr, x.c_global, 16, 0.25f,
+                                   x.parts);
   else
-    amax_tile<true, false, false>(x.x, x.rows, x.cols, x.ld, 0u, b, x_tiles_c, x.r_global, nullptr, nullptr, nullptr);
+    amax_tile<true, false, false, PARTS>(x.x, x.rows, x.cols, x.ld, 0u, b, x_tiles_c, x.r_global, nullptr, nullptr, nullptr,
+                                         x.parts);
 }
 
 // Pass 1 of a binary32 source: plain tensor amax.  CTA tile 128 rows x 128 columns; a warp owns 16 rows, a lane 4 columns of each.
@@ -369,7 +389,8 @@ __device__ __forceinline__ void store_linear_scales(const uint8_t* src, uint8_t*
     if (full_tile || (R0 + r + 256 / KB * p < Rn && K0 + kb < n_kb)) *d = src[threadIdx.x + 256 * p];
 }
 
-template <bool HAS_ROW, bool HAS_COL, bool BLOCK2D, bool RHT_ROW, bool RHT_COL, bool SR, int TC, bool F32 = false>
+template <bool HAS_ROW, bool HAS_COL, bool BLOCK2D, bool RHT_ROW, bool RHT_COL, bool SR, int TC, bool F32 = false,
+          bool PARTS = false>
 __device__ __forceinline__ void quantize_tiles(const CUtensorMap* src_map, const QuantArgs& a, const int block,
                                                const int blocks) {  // this CTA among those of the tensor
   using S = QuantSmem<TC, F32>;
@@ -409,16 +430,42 @@ __device__ __forceinline__ void quantize_tiles(const CUtensorMap* src_map, const
     if (n_mine > 1) issue(1);
     // the source tiles above are nobody's output in this call; the tensor amax below is the previous kernel's.
     // Every other thread passes the barrier below only after this wait, so no output is written before it either.
+    if (!PARTS) griddep_wait();
+  }
+  float2 m = make_float2(0.f, 0.f);
+  if (PARTS) {
     griddep_wait();
+    for (int i = threadIdx.x; i < a.n_parts; i += 256) {
+      const float2 p = __ldcg(a.parts + i);
+      m = make_float2(fmaxf(m.x, p.x), fmaxf(m.y, RHT_COL ? p.y : p.x));
+    }
+    m = make_float2(warp_max(m.x), warp_max(m.y));
+    float2* const red = reinterpret_cast<float2*>(smem + S::kEncRow);  // the table is made behind the next barriers
+    if (lane == 0) red[warp] = m;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+#pragma unroll
+      for (int w = 1; w < 8; ++w) m = make_float2(fmaxf(m.x, red[w].x), fmaxf(m.y, red[w].y));
+      if (block == 0) {
+        if (HAS_ROW) a.r_global[0] = m.x;
+        if (HAS_COL) a.c_global[0] = m.y;
+      }
+    }
+  }
+  if (threadIdx.x == 0) {
     // Eq. 1 (two IEEE divisions per copy)
     float re = 1.f, rd = 1.f, ce = 1.f, cd = 1.f;
-    if (HAS_ROW || BLOCK2D) global_scales(HAS_ROW ? a.r_global[0] : a.c_global[0], re, rd);
+    if (!PARTS) {
+      if (HAS_ROW) m.x = a.r_global[0];
+      if (HAS_COL) m.y = a.c_global[0];
+    }
+    if (HAS_ROW || BLOCK2D) global_scales(HAS_ROW ? m.x : m.y, re, rd);
     if (HAS_COL) {
       if (BLOCK2D && HAS_ROW) {
         ce = re;
         cd = rd;
       } else {
-        global_scales(a.c_global[0], ce, cd);
+        global_scales(m.y, ce, cd);
       }
     }
     g_sc[0] = re; g_sc[1] = rd; g_sc[2] = ce; g_sc[3] = cd;
@@ -772,10 +819,11 @@ __device__ __forceinline__ void quantize_tiles(const CUtensorMap* src_map, const
     }
 }
 
-template <bool HAS_ROW, bool HAS_COL, bool BLOCK2D, bool RHT_ROW, bool RHT_COL, bool SR, int TC, bool F32 = false>
+template <bool HAS_ROW, bool HAS_COL, bool BLOCK2D, bool RHT_ROW, bool RHT_COL, bool SR, int TC, bool F32 = false,
+          bool PARTS = false>
 __global__ void __launch_bounds__(256, 2) quantize_kernel(const __grid_constant__ CUtensorMap src_map,
                                                           const __grid_constant__ QuantArgs a) {
-  quantize_tiles<HAS_ROW, HAS_COL, BLOCK2D, RHT_ROW, RHT_COL, SR, TC, F32>(&src_map, a, (int)blockIdx.x, (int)gridDim.x);
+  quantize_tiles<HAS_ROW, HAS_COL, BLOCK2D, RHT_ROW, RHT_COL, SR, TC, F32, PARTS>(&src_map, a, (int)blockIdx.x, (int)gridDim.x);
 }
 
 // The activation (1x16 blocks, the transposed copy with the transform) and the weight (16x16 blocks) of a forward call in one
@@ -783,16 +831,16 @@ __global__ void __launch_bounds__(256, 2) quantize_kernel(const __grid_constant_
 // pass 1 on the activation's pass 2 and quantizing the weight behind it measured the same for many tiles (8192 x 20480 x 5120)
 // and lost for few: fwd + bwd of 512 x 1024 x 1024 27.6 -> 24.2 us of GPU time, 1024 x 2048 x 2048 41.7 -> 39.7, 2048 x 4096 x
 // 3072 93.8 -> 91.5.
-template <bool X_COL, bool W_COL, int TC>
+template <bool X_COL, bool W_COL, int TC, bool PARTS>
 __global__ void __launch_bounds__(256, 2) quantize_x_and_w_kernel(const __grid_constant__ CUtensorMap x_map,
                                                                   const __grid_constant__ CUtensorMap w_map,
                                                                   const __grid_constant__ QuantArgs x,
                                                                   const __grid_constant__ QuantArgs w, int n_x) {
   const int b = (int)blockIdx.x;
   if (b < n_x)
-    quantize_tiles<true, X_COL, false, false, X_COL, false, TC>(&x_map, x, b, n_x);
+    quantize_tiles<true, X_COL, false, false, X_COL, false, TC, false, PARTS>(&x_map, x, b, n_x);
   else
-    quantize_tiles<true, W_COL, true, false, false, false, TC>(&w_map, w, b - n_x, (int)gridDim.x - n_x);
+    quantize_tiles<true, W_COL, true, false, false, false, TC, false, PARTS>(&w_map, w, b - n_x, (int)gridDim.x - n_x);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -863,13 +911,45 @@ __global__ void e2m1_sr_kernel(const float* __restrict__ v, const uint8_t* __res
 // ---------------------------------------------------------------------------------------------
 // Host launchers
 // ---------------------------------------------------------------------------------------------
+int64_t amax_parts(int64_t rows, int64_t cols) { return (rows + 127) / 128 * ((cols + 255) / 256); }
+
+// Pass 1 in parts while every tile of pass 2 (64 columns wide, four to a tile of pass 1) has a CTA of its own: the call has a
+// launch less.  Graph time of a layer, words / parts: fwd + bwd of 512 x 1024 x 1024 24.0 / 22.9 us, 1024 x 1024 x 1024 25.9 /
+// 24.7, 1024 x 2048 x 2048 39.1 / 38.5; bwd of 1024 x 2048 x 1024 17.2 / 16.9; and 2.3 us of the host's time.  Beyond that it
+// loses (2048 x 3328 x 3328 80.6 / 82.1): see launch_amax_parts().
+bool pass1_in_parts(int64_t parts) {
+  int sms = 0;
+  return sm_count(&sms) == cudaSuccess && 4 * parts <= 2 * sms;
+}
+
+// In parts, pass 1 is the first kernel of its call and becomes resident while the previous one drains.  At three CTAs per SM
+// it crowds on the SMs that drain first and runs there when it may begin (bwd of 1024 x 2048 x 1024 18.9 us instead of 16.9):
+// more shared memory than half of an SM's keeps it to one.
+template <auto KERN, typename... Args>
+static cudaError_t launch_amax_parts(unsigned tiles, cudaStream_t s, Args&&... args) {
+  constexpr int kSmem = 120 * 1024;
+  static std::atomic<uint64_t> configured{0};  // per kernel and device
+  int dev;
+  if (device_needs_config(configured, &dev)) {
+    const cudaError_t e = cudaFuncSetAttribute(KERN, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
+    if (e != cudaSuccess) return e;
+    device_configured(configured, dev);
+  }
+  return launch_kernel(KERN, dim3(tiles), dim3(256), kSmem, s, std::forward<Args>(args)...);
+}
+
 template <bool PLAIN, bool RR, bool RC>
 static cudaError_t launch_amax_t(const QuantArgs& a, float* plain0, float* plain1, float* rot_row,
                                  float* rot_col, cudaStream_t s) {
   const int tiles_c = (int)((a.cols + 255) / 256);
   const int64_t tiles = ((a.rows + 127) / 128) * tiles_c;
-  const cudaError_t e = launch_kernel(amax_kernel<PLAIN, RR, RC>, dim3((unsigned)tiles), dim3(256), 0, s, a.x, a.rows,
-                                      a.cols, a.ld, a.sign_mask, tiles_c, plain0, plain1, rot_row, rot_col);
+  cudaError_t e = cudaErrorInvalidValue;
+  if (!a.parts)
+    e = launch_kernel(amax_kernel<PLAIN, RR, RC, false>, dim3((unsigned)tiles), dim3(256), 0, s, a.x, a.rows, a.cols, a.ld,
+                      a.sign_mask, tiles_c, plain0, plain1, rot_row, rot_col, (float2*)nullptr);
+  else if constexpr (!RR && !RC)
+    e = launch_amax_parts<amax_kernel<PLAIN, RR, RC, true>>((unsigned)tiles, s, a.x, a.rows, a.cols, a.ld, a.sign_mask, tiles_c,
+                                                            plain0, plain1, rot_row, rot_col, a.parts);
   count_launch();
   return e;
 }
@@ -897,16 +977,21 @@ static cudaError_t launch_amax_rot_col(const QuantArgs& a, uint32_t mask16, floa
                                        int d, float norm, cudaStream_t s) {
   const int tiles_c = (int)((a.cols + 255) / 256);
   const unsigned tiles = (unsigned)(((a.rows + 127) / 128) * tiles_c);
-  const cudaError_t e = launch_kernel(amax_rot_col_kernel<PLAIN>, dim3(tiles), dim3(256), 0, s, a.x, a.rows, a.cols, a.ld,
-                                      mask16, tiles_c, plain0, plain1, rot_col, d, norm);
+  const cudaError_t e =
+      a.parts ? launch_amax_parts<amax_rot_col_kernel<PLAIN, true>>(tiles, s, a.x, a.rows, a.cols, a.ld, mask16, tiles_c, plain0,
+                                                                    plain1, rot_col, d, norm, a.parts)
+              : launch_kernel(amax_rot_col_kernel<PLAIN, false>, dim3(tiles), dim3(256), 0, s, a.x, a.rows, a.cols, a.ld,
+                              mask16, tiles_c, plain0, plain1, rot_col, d, norm, (float2*)nullptr);
   count_launch();
   return e;
 }
 
 cudaError_t launch_amax(const QuantArgs& a, bool has_row, bool has_col, bool rht_row, bool rht_col,
                         cudaStream_t s) {
-  const cudaError_t e = launch_zero_words(has_row ? a.r_global : nullptr, has_col ? a.c_global : nullptr, nullptr, nullptr, s);
-  if (e != cudaSuccess) return e;
+  if (!a.parts) {
+    const cudaError_t e = launch_zero_words(has_row ? a.r_global : nullptr, has_col ? a.c_global : nullptr, nullptr, nullptr, s);
+    if (e != cudaSuccess) return e;
+  }
   const bool rr = has_row && rht_row, rc = has_col && rht_col;
   float* plain0 = (has_row && !rht_row) ? a.r_global : nullptr;
   float* plain1 = (has_col && !rht_col) ? a.c_global : nullptr;
@@ -944,9 +1029,9 @@ static bool quant_source_map(CUtensorMap* map, const QuantArgs& a, int tc, bool 
                      (uint64_t)a.cols, (uint64_t)a.rows, (uint64_t)a.ld * (f32 ? 4 : 2), tc, 128, false);
 }
 
-template <bool HR, bool HC, bool B2, bool RR, bool RC, bool SR, int TC, bool F32 = false>
+template <bool HR, bool HC, bool B2, bool RR, bool RC, bool SR, int TC, bool F32 = false, bool PARTS = false>
 static cudaError_t launch_quant_tc(const QuantArgs& a_in, int slots, cudaStream_t s) {
-  auto kern = quantize_kernel<HR, HC, B2, RR, RC, SR, TC, F32>;
+  auto kern = quantize_kernel<HR, HC, B2, RR, RC, SR, TC, F32, PARTS>;
   QuantArgs a = a_in;
   a.tiles_c = (int)((a.cols + TC - 1) / TC);
   constexpr bool kRowCodes = B2 && HR && HC;
@@ -977,15 +1062,17 @@ static cudaError_t launch_quant_t(const QuantArgs& a, cudaStream_t s) {
   // 1024 10.6 / 8.3, 2816 x 2304 16.4 / 14.7, 4096 x 4096 31.7 / 30.4, 8192 x 5120 63.3 / 67.2; weight of 2048 x 1024 7.0 / 6.0,
   // 4096 x 2304 11.1 / 12.1.
   const int slots = 2 * sms;  // resident CTAs
+  if constexpr (!B2 && !RR && RC == HC)  // an activation or a gradient of a layer
+    if (a.parts) return launch_quant_tc<HR, HC, B2, RR, RC, SR, 64, false, true>(a, slots, s);
   const int64_t t128 = (int64_t)a.tiles_r * a.tiles_c, t64 = (int64_t)a.tiles_r * ((a.cols + 63) / 64);
   const double r128 = (double)((t128 + slots - 1) / slots), r64 = (double)((t64 + slots - 1) / slots) * (B2 ? 0.58 : 0.535);
   if (!RR && r64 < r128) return launch_quant_tc<HR, HC, B2, RR, RC, SR, RR ? 128 : 64>(a, slots, s);
   return launch_quant_tc<HR, HC, B2, RR, RC, SR, 128>(a, slots, s);
 }
 
-template <bool X_COL, bool W_COL, int TC>
+template <bool X_COL, bool W_COL, int TC, bool PARTS = false>
 static cudaError_t launch_x_and_w_tc(QuantArgs x, QuantArgs w, int slots, cudaStream_t s) {
-  auto kern = quantize_x_and_w_kernel<X_COL, W_COL, TC>;
+  auto kern = quantize_x_and_w_kernel<X_COL, W_COL, TC, PARTS>;
   constexpr int smem = QuantSmem<TC>::bytes(false, W_COL);
   CUtensorMap maps[2];
   QuantArgs* const t[2] = {&x, &w};
@@ -1026,17 +1113,22 @@ static cudaError_t launch_x_and_w_t(const QuantArgs& x, const QuantArgs& w, cuda
   int sms = 0;
   cudaError_t e = sm_count(&sms);
   if (e != cudaSuccess) return e;
-  e = launch_zero_words(x.r_global, X_COL ? x.c_global : nullptr, w.r_global, W_COL ? w.c_global : nullptr, s);
-  if (e != cudaSuccess) return e;
+  if (!x.parts) {
+    e = launch_zero_words(x.r_global, X_COL ? x.c_global : nullptr, w.r_global, W_COL ? w.c_global : nullptr, s);
+    if (e != cudaSuccess) return e;
+  }
   const int xc = (int)((x.cols + 255) / 256), wc = (int)((w.cols + 255) / 256);
   const int64_t n_x = ((x.rows + 127) / 128) * xc, n_w = ((w.rows + 127) / 128) * wc;
   if (n_x + n_w > 0x7fffffff) return cudaErrorInvalidValue;
-  e = launch_kernel(amax_x_and_w_kernel<X_COL, W_COL>, dim3((unsigned)(n_x + n_w)), dim3(256), 0, s, x, w, (int)n_x, xc, wc);
+  e = x.parts ? launch_amax_parts<amax_x_and_w_kernel<X_COL, W_COL, true>>((unsigned)(n_x + n_w), s, x, w, (int)n_x, xc, wc)
+              : launch_kernel(amax_x_and_w_kernel<X_COL, W_COL, false>, dim3((unsigned)(n_x + n_w)), dim3(256), 0, s, x, w,
+                              (int)n_x, xc, wc);
   count_launch();
   if (e != cudaSuccess) return e;
   QuantArgs xa = x, wa = w;
   xa.chained = wa.chained = 1;
   const int slots = 2 * sms;  // resident CTAs; the width of the tiles as in launch_quant_t
+  if (x.parts) return launch_x_and_w_tc<X_COL, W_COL, 64, true>(xa, wa, slots, s);
   const int64_t t128 = (int64_t)x.tiles_r * x.tiles_c + (int64_t)w.tiles_r * w.tiles_c;
   const int64_t t64 = (int64_t)x.tiles_r * ((x.cols + 63) / 64) + (int64_t)w.tiles_r * ((w.cols + 63) / 64);
   return 0.55 * (double)((t64 + slots - 1) / slots) < (double)((t128 + slots - 1) / slots)

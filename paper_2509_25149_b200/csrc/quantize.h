@@ -24,6 +24,8 @@ struct QuantArgs {
   uint32_t rk[20];       // Philox round keys (seed_lo + r * W0, seed_hi + r * W1), r = 0..9, filled by the host
   int tiles_r, tiles_c;  // 128 x 128 tiles of the source
   unsigned int* status;  // device status word: a bounded wait that expired leaves its code here (may be NULL)
+  float2* parts;  // pass 1 leaves {plain, transformed} maximum of each of its n_parts tiles here (scratch of the call); NULL: it
+  int n_parts;    // takes the maximum into the copies' first words, which are cleared before
   int chained;  // the source is complete when the kernel starts (an earlier kernel of the same call has waited for it):
                 // it may be read before the wait for the previous kernel (see launch_kernel)
 };
@@ -41,6 +43,10 @@ cudaError_t launch_quantize_rht(const RhtArgs& ra, bool amax_provided, bool sr, 
 cudaError_t launch_amax_rot_col_small(const QuantArgs& a, bool has_row, uint32_t mask16, int d, float norm,
                                       cudaStream_t s);
 
+// Pass 1 in parts: the number of its tiles, and whether the launchers below take `parts` for that many (of all tensors of the
+// launch together)
+int64_t amax_parts(int64_t rows, int64_t cols);
+bool pass1_in_parts(int64_t parts);
 // Clears the words the reductions of a call add into (any of them may be NULL) in one launch, the first of the call.
 cudaError_t launch_zero_words(float* w0, float* w1, float* w2, float* w3, cudaStream_t s);
 cudaError_t launch_amax(const QuantArgs& a, bool has_row, bool has_col, bool rht_row, bool rht_col,
