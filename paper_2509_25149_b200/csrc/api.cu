@@ -569,7 +569,8 @@ int32_t nvfp4_set_gemm_experiment(int32_t mode, int32_t max_pairs, void* probe) 
 }
 
 int32_t nvfp4_set_gemm_tile_n(int32_t tile_n) {
-  if (tile_n != 0 && tile_n != 128 && tile_n != 256 && tile_n != 512 && tile_n != 640 && tile_n != 768)
+  if (tile_n != 0 && tile_n != 128 && tile_n != 256 && tile_n != 512 && tile_n != 640 && tile_n != 768 &&
+      tile_n != kTileSplit2 && tile_n != kTileSplit4)
     return -1;
   g_tile_n.store(tile_n, std::memory_order_relaxed);
   return 0;

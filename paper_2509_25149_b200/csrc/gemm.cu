@@ -385,7 +385,7 @@ cudaError_t launch_t(const GemmArgs& g, const void* a_codes, const void* b_codes
   return le;
 }
 
-bool make_pair_maps(const GemmArgs& g, const void* a_codes, const void* b_codes, int bn, CUtensorMap* map_a,
+bool make_pair_maps(const GemmArgs& g, const void* a_codes, const void* b_codes, int bn, int store_cols, CUtensorMap* map_a,
                     CUtensorMap* map_b, CUtensorMap* map_d) {
   bool ok = make_code_map(map_a, a_codes, g.M, g.K / 2, 128) && make_code_map(map_b, b_codes, g.N, g.K / 2, bn / 2);
   if (g.d_is_fp32)
@@ -393,7 +393,7 @@ bool make_pair_maps(const GemmArgs& g, const void* a_codes, const void* b_codes,
                            (uint64_t)g.ldd * 4, 16, 128, 2);
   else
     ok = ok && make_map_2d(map_d, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, g.d, (uint64_t)g.N, (uint64_t)g.M,
-                           (uint64_t)g.ldd * 2, 64, 128, true);
+                           (uint64_t)g.ldd * 2, store_cols < 64 ? 32 : 64, 128, store_cols < 64 ? 2 : 1);
   return ok;
 }
 
@@ -413,15 +413,15 @@ bool has_row_scales(const GemmArgs& g0, const GemmArgs* g1) {
 inline int pair_tiles(const GemmArgs& g, int bn) { return ((g.M + 255) / 256) * ((g.N + bn - 1) / bn); }
 
 // g1 == nullptr: one problem
-template <bool MX, bool ROWS, int BN>
+template <bool MX, bool ROWS, int BN, int SPLIT = 1>
 cudaError_t launch_pair_t(const GemmArgs& g0, const void* a0, const void* b0, const GemmArgs* g1, const void* a1,
                           const void* b1, int num_sms, cudaStream_t s) {
-  auto kern = pair::gemm_pair_kernel<MX, ROWS, BN>;
-  constexpr int smem = pair::Cfg<BN>::kSmemBytes;
+  auto kern = pair::gemm_pair_kernel<MX, ROWS, BN, SPLIT>;
+  constexpr int smem = pair::Cfg<BN, SPLIT>::kSmemBytes, store_cols = SPLIT > 1 ? BN / SPLIT : 64;
   CUtensorMap m[6];
-  if (!make_pair_maps(g0, a0, b0, BN, &m[0], &m[1], &m[2])) return cudaErrorInvalidValue;
+  if (!make_pair_maps(g0, a0, b0, BN, store_cols, &m[0], &m[1], &m[2])) return cudaErrorInvalidValue;
   if (g1) {
-    if (!make_pair_maps(*g1, a1, b1, BN, &m[3], &m[4], &m[5])) return cudaErrorInvalidValue;
+    if (!make_pair_maps(*g1, a1, b1, BN, store_cols, &m[3], &m[4], &m[5])) return cudaErrorInvalidValue;
   } else {
     m[3] = m[0]; m[4] = m[1]; m[5] = m[2];
   }
@@ -442,9 +442,9 @@ cudaError_t launch_pair_t(const GemmArgs& g0, const void* a0, const void* b0, co
   if (cap > 0 && cap < max_pairs) max_pairs = cap;
   a.exp = g_exp_mode.load(std::memory_order_relaxed);
   a.probe = g_exp_probe.load(std::memory_order_relaxed);
-  const int pairs = a.n_tiles < max_pairs ? a.n_tiles : max_pairs;
+  const int pairs = a.n_tiles < max_pairs || SPLIT > 1 ? a.n_tiles : max_pairs;  // SPLIT > 1: a cluster for each tile
   const cudaError_t e =
-      launch_kernel(kern, dim3(2 * pairs), dim3(pair::kThreads), smem, s, m[0], m[1], m[2], m[3], m[4], m[5], a);
+      launch_kernel(kern, dim3(2 * SPLIT * pairs), dim3(pair::kThreads), smem, s, m[0], m[1], m[2], m[3], m[4], m[5], a);
   count_launch();
   return e;
 }
@@ -462,6 +462,15 @@ cudaError_t launch_pair(const GemmArgs& g0, const void* a0, const void* b0, cons
                  : launch_pair_t<false, false, 128>(g0, a0, b0, g1, a1, b1, num_sms, s);
   return g0.mx ? launch_pair_t<true, false, 256>(g0, a0, b0, g1, a1, b1, num_sms, s)
                : launch_pair_t<false, false, 256>(g0, a0, b0, g1, a1, b1, num_sms, s);
+}
+
+template <int SPLIT>
+cudaError_t launch_split(const GemmArgs& g, const void* a, const void* b, int num_sms, cudaStream_t s) {
+  if (has_row_scales(g, nullptr))
+    return g.mx ? cudaErrorInvalidValue
+                : launch_pair_t<false, true, 128, SPLIT>(g, a, b, nullptr, nullptr, nullptr, num_sms, s);
+  return g.mx ? launch_pair_t<true, false, 128, SPLIT>(g, a, b, nullptr, nullptr, nullptr, num_sms, s)
+              : launch_pair_t<false, false, 128, SPLIT>(g, a, b, nullptr, nullptr, nullptr, num_sms, s);
 }
 
 // N = 128 q = 384 a + 256 b with b in {0, 1, 2}: a wide column tiles, b narrow ones (q >= 2)
@@ -537,6 +546,51 @@ double pair_makespan(const GemmArgs* const* gs, int n_problems, int tile, int pa
   return worst;
 }
 
+// Clusters of SPLIT pairs that are resident at once on the current device (0: none)
+template <int SPLIT>
+int split_clusters() {
+  constexpr int kMaxDevices = 64;
+  static std::atomic<int> known[kMaxDevices];  // the number + 1
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return 0;
+  if (const int n = known[dev].load(std::memory_order_relaxed)) return n - 1;
+  auto kern = pair::gemm_pair_kernel<false, false, 128, SPLIT>;
+  constexpr int smem = pair::Cfg<128, SPLIT>::kSmemBytes;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(2 * SPLIT);
+  cfg.blockDim = dim3(pair::kThreads);
+  cfg.dynamicSmemBytes = smem;
+  int n = 0;
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
+      cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess)
+    n = 0;
+  known[dev].store(n + 1, std::memory_order_relaxed);
+  return n;
+}
+
+// The split of a product that has a launch to itself, or 0 (`least`: the estimate of the best tile).  A split pays where a
+// tile's contraction is long and the clusters of all tiles are resident at once; its exchange costs 1.4 us (2.1 where most of
+// the chip takes part) and it has to win by half a microsecond.  The two products of a backward call fill one launch
+// together: with one of them split and the other behind it, 512 x 3584 x 768 took 38.0 us instead of 31.8.
+// Time of a product, 256 x 128 tiles / two pairs / four pairs per tile: 256 x 512 x 5120 10.5 / 8.5 / 7.3 us, 256 x 512 x 20480
+// 29.1 / 17.8 / 12.2, 512 x 1024 x 4096 9.5 / 8.1 / 14.1 (two rounds), 1024 x 1024 x 10240 17.6 / 12.9 / 27.6; 256 x 1024 x 2048
+// 6.7 / 6.7 / 6.4, 256 x 2048 x 1024 5.5 / 6.2 / 12.1.
+int split_tile(const GemmArgs& g, double least) {
+  const int tiles = ((g.M + 255) / 256) * (g.N / 128), kb = g.K / 256;
+  const double fixed = (g.d_is_fp32 ? 0.97 : 0.64) + (tiles > 16 ? 2.1 : 1.4);
+  int best = 0;
+  least -= 0.5;
+  auto consider = [&](int split, int clusters, int tile) {
+    const double v = 0.323 * ((kb + split - 1) / split) + fixed;
+    if (kb < split || tiles > clusters || v >= least) return;
+    best = tile;
+    least = v;
+  };
+  consider(2, split_clusters<2>(), kTileSplit2);
+  consider(4, split_clusters<4>(), kTileSplit4);
+  return best;
+}
+
 // g1 == nullptr: one problem
 template <bool MX, bool ROWS>
 cudaError_t launch_wide_t(const GemmArgs& g0, const void* a0, const void* b0, const GemmArgs* g1, const void* a1,
@@ -585,6 +639,9 @@ cudaError_t launch_gemm(const GemmArgs& g, const void* a_codes, const void* b_co
   cudaError_t e = sm_count(&num_sms);
   if (e != cudaSuccess) return e;
   const bool rows = has_row_scales(g, nullptr);  // scale vectors: the pair kernels' epilogues only
+  if (tile == kTileSplit2 && g.K / 256 >= 2) return launch_split<2>(g, a_codes, b_codes, num_sms, s);
+  if (tile == kTileSplit4 && g.K / 256 >= 4) return launch_split<4>(g, a_codes, b_codes, num_sms, s);
+  if (tile == kTileSplit2 || tile == kTileSplit4) tile = kTilePair128;
   if (tile == kTileWide && wide_eligible(g)) return launch_wide(g, a_codes, b_codes, nullptr, nullptr, nullptr, num_sms, s);
   if (tile >= kTilePair256 || rows)
     return launch_pair(g, a_codes, b_codes, nullptr, nullptr, nullptr, tile == kTilePair128 ? 128 : 256, num_sms, s);
@@ -631,6 +688,8 @@ int best_pair_tile(const GemmArgs& g0, const GemmArgs* g1) {
       best = tile;
     }
   }
+  if (!g1)
+    if (const int tile = split_tile(g0, least)) best = tile;
   std::lock_guard<std::mutex> lock(mu);
   if (seen.size() < 256) {
     Entry e{};

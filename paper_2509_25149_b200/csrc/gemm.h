@@ -24,12 +24,14 @@ struct GemmArgs {
 constexpr int kTilePair256 = 512;  // 256 x 256
 constexpr int kTilePair128 = 640;  // 256 x 128
 constexpr int kTileWide = 768;     // 256 x 384, needs N >= 256
+constexpr int kTileSplit2 = 642;   // 256 x 128, a cluster of two pairs per tile shares its contraction (K >= 512)
+constexpr int kTileSplit4 = 644;   // the same with four pairs (K >= 1024)
 cudaError_t launch_gemm(const GemmArgs& g, const void* a_codes, const void* b_codes, int tile, cudaStream_t s);
 // Two independent GEMMs in one launch of a CTA-pair kernel: the tiles of g0 are worked through first, then those of g1,
 // on one persistent grid.
 cudaError_t launch_gemm_two(const GemmArgs& g0, const void* a0, const void* b0, const GemmArgs& g1, const void* a1,
                             const void* b1, int tile, cudaStream_t s);
-// Scheduling estimate: the CTA-pair tile for this problem (or pair of problems in one launch)
+// Scheduling estimate: the CTA-pair tile for this problem (or pair of problems in one launch, then no split one)
 int best_pair_tile(const GemmArgs& g0, const GemmArgs* g1);
 // Measurement aids of the CTA-pair kernel with 256 x 256 tiles (0, 0, NULL = normal operation): mode bit 0 = no MMAs,
 // bit 1 = no operand loads, bit 2 = no scale loads / copies, bit 3 = accumulator handed back unread and nothing

@@ -30,16 +30,20 @@ constexpr int kSfaBytes = 4 * 512;   // own 128 rows, four K64 steps
 constexpr int kStagingBytes = 2 * 16384;  // one 128 x 128-byte store buffer per epilogue group
 constexpr int kBetaBytes = 2 * 128 * 4;   // column scales of the tile, one half per epilogue group (row-scaled B)
 constexpr uint32_t kTmemCols = 512;
-template <int BN>
+// SPLIT > 1: a cluster of SPLIT pairs works on one tile, each pair on its share of the contraction, see gemm_pair_kernel
+template <int BN, int SPLIT = 1>
 struct Cfg {
   static constexpr int kGroups = BN / 128;              // 128-row groups of B = scale atoms per K64 step
-  static constexpr int kStages = BN == 256 ? 5 : 6;
+  static constexpr int kStages = BN == 256 || SPLIT > 1 ? 5 : 6;
   static constexpr int kAcc = BN == 256 ? 1 : 2;        // accumulators in tensor memory
   static constexpr int kBBytes = BN / 2 * 128;          // this CTA's half of the B tile
   static constexpr int kSfbBytes = 4 * kGroups * 512;   // all rows of B (both CTAs need them), four K64 steps
   static constexpr int kStageBytes = kABytes + kBBytes + kSfaBytes + kSfbBytes;  // 38 / 28 KB
+  static constexpr int kCols = BN / SPLIT;              // columns that a pair finishes and stores
+  static constexpr int kSlotBytes = 128 * kCols * 4;    // one other pair's share of them (this CTA's 128 rows)
+  static constexpr int kRecvBytes = (SPLIT - 1) * kSlotBytes;
   static constexpr int kSmemBytes =
-      kStages * kStageBytes + kStagingBytes + 1024 /*alignment*/ + 256 /*barriers*/ + kBetaBytes;
+      kStages * kStageBytes + kStagingBytes + 1024 /*alignment*/ + 256 /*barriers*/ + kBetaBytes + kRecvBytes;
   static constexpr int kSfCol = 256;                    // after the accumulator columns: one slot per stage
   static constexpr int kSfSlotCols = 16 + 16 * kGroups; // SFA 4 x 4, SFB 4 x 4 per group
   static_assert(kSfCol + kStages * kSfSlotCols <= 512, "tensor memory budget");
@@ -147,6 +151,13 @@ __device__ __forceinline__ void tma_reduce_add_2d(const CUtensorMap* map, int x,
                "r"(x), "r"(y), "r"(src)
                : "memory");
 }
+// four words into another CTA's shared memory, counted on a barrier there
+__device__ __forceinline__ void st_async16(uint32_t cluster_addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d,
+                                           uint32_t cluster_bar) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(cluster_addr),
+               "r"(a), "r"(b), "r"(c), "r"(d), "r"(cluster_bar)
+               : "memory");
+}
 __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
 template <int N>
 __device__ __forceinline__ void bulk_wait_read() {
@@ -213,7 +224,7 @@ __device__ __forceinline__ void tc2_mma_mxf4(uint32_t d_tmem, uint64_t adesc, ui
 
 // Epilogue helper: COLS accumulator columns of one row per thread (registers) -> alpha, conversion -> swizzled rows of
 // the group's 16 KB staging buffer -> TMA store (or reduce-add).
-// bf16: chunks of 64 columns (128-byte rows) through the whole buffer, each converted once the store before it has
+// bf16: chunks of 64 columns (128-byte rows; 32 columns where a call stores no more) through the whole buffer, each converted once the store before it has
 // finished reading.  fp32: chunks of 16 columns (64-byte rows) through the two 8 KB halves in turn, so that a chunk waits
 // only for the store of two chunks before it; with 32-column chunks through the whole buffer the stores were a serial
 // chain that bounded tiles of few k-blocks.  (An even number of fp32 chunks: a tile starts with the first half, and only a
@@ -224,7 +235,8 @@ __device__ __forceinline__ void store_half(const uint32_t (&r)[COLS], float alph
                                            uint32_t stage_buf16k, const CUtensorMap* map_d, int x0, int row0,
                                            int accumulate, bool drain, const float* beta = nullptr, int skip = 0) {
   // skip (measurement aid): bit 0 = the converted values are not written to the staging buffer, bit 1 = no TMA store
-  constexpr int kChunkCols = FP32 ? 16 : 64, kUnits = FP32 ? 4 : 8;  // 16-byte units of a staged row
+  constexpr int kUnits = FP32 || COLS < 64 ? 4 : 8;  // 16-byte units of a staged row
+  constexpr int kChunkCols = FP32 ? 16 : 8 * kUnits;
   constexpr int kChunks = COLS / kChunkCols;
   static_assert(!FP32 || kChunks % 2 == 0, "a tile starts with the first half of the buffer");
 #pragma unroll
@@ -239,7 +251,7 @@ __device__ __forceinline__ void store_half(const uint32_t (&r)[COLS], float alph
     asm volatile("bar.sync %0, 128;" ::"r"(bar_id) : "memory");
     const uint32_t srow = stage_buf + row_in_tile * (16 * kUnits);
     // 128-byte swizzle: unit index XOR address bits 7-9 = row & 7; 64-byte swizzle: XOR bits 7-8 = (row >> 1) & 3
-    const uint32_t x = FP32 ? (row_in_tile >> 1) & 3 : row_in_tile & 7;
+    const uint32_t x = kUnits == 4 ? (row_in_tile >> 1) & 3 : row_in_tile & 7;
 #pragma unroll
     for (int j = 0; j < kUnits; ++j) {
       uint32_t p[4];
@@ -253,11 +265,11 @@ __device__ __forceinline__ void store_half(const uint32_t (&r)[COLS], float alph
       } else {
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-          float v0 = __uint_as_float(r[c * 64 + 8 * j + 2 * e]) * alpha;
-          float v1 = __uint_as_float(r[c * 64 + 8 * j + 2 * e + 1]) * alpha;
+          float v0 = __uint_as_float(r[c * kChunkCols + 8 * j + 2 * e]) * alpha;
+          float v1 = __uint_as_float(r[c * kChunkCols + 8 * j + 2 * e + 1]) * alpha;
           if (BETA) {
-            v0 *= beta[c * 64 + 8 * j + 2 * e];
-            v1 *= beta[c * 64 + 8 * j + 2 * e + 1];
+            v0 *= beta[c * kChunkCols + 8 * j + 2 * e];
+            v1 *= beta[c * kChunkCols + 8 * j + 2 * e + 1];
           }
           __nv_bfloat162 h = __floats2bfloat162_rn(v0, v1);
           p[e] = *reinterpret_cast<uint32_t*>(&h);
@@ -287,13 +299,18 @@ __device__ __forceinline__ void store_half(const uint32_t (&r)[COLS], float alph
 // factor per output row and / or per output column.  A separate instantiation so that the common kernel keeps its
 // register budget.
 // BN: columns of a tile (256 or 128).
-template <bool MX, bool ROWS = false, int BN = 256>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
+// SPLIT > 1 (BN = 128): for few tiles and long contractions, which leave most pairs idle.  A cluster of SPLIT pairs takes one
+// tile (the only one of its life), pair s the s-th share of the k-blocks.  Then every pair finishes 128 / SPLIT columns:
+// it sends its sums of the others' columns into their shared memory and adds what it receives to its own, always in the
+// order of the pairs.  (A product of few tiles is bound by one pair's main loop, 0.31 us per k-block: shared by four 0.08; figures at
+// split_tile().)
+template <bool MX, bool ROWS = false, int BN = 256, int SPLIT = 1>
+__global__ void __cluster_dims__(2 * SPLIT, 1, 1) __launch_bounds__(kThreads, 1)
     gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant__ CUtensorMap map_b0,
                      const __grid_constant__ CUtensorMap map_d0, const __grid_constant__ CUtensorMap map_a1,
                      const __grid_constant__ CUtensorMap map_b1, const __grid_constant__ CUtensorMap map_d1,
                      const __grid_constant__ Args g) {
-  using C = Cfg<BN>;
+  using C = Cfg<BN, SPLIT>;
   constexpr int kStages = C::kStages, kStageBytes = C::kStageBytes, kBBytes = C::kBBytes, kGroups = C::kGroups;
   constexpr int kSfCol = C::kSfCol, kSfSlotCols = C::kSfSlotCols;
   extern __shared__ uint8_t smem_raw[];
@@ -308,14 +325,19 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   auto accf_bar = [&](int b) { return bar_base + 8u * (4 * kStages + b); };             // per accumulator, one per CTA
   auto acce_bar = [&](int b) { return bar_base + 8u * (4 * kStages + C::kAcc + b); };   // leader only, 16 arrivals
   const uint32_t done_bar = bar_base + 8u * (4 * kStages + 2 * C::kAcc);                // one per CTA, peer arrives
+  const uint32_t recv_bar = done_bar + 8;                                               // SPLIT > 1: all shares are here
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(base_ptr + kStages * kStageBytes + kStagingBytes +
-                                                                      8 * (4 * kStages + 2 * C::kAcc + 1));
+                                                                      8 * (4 * kStages + 2 * C::kAcc + (SPLIT > 1 ? 2 : 1)));
   volatile uint32_t* abort_flag = tmem_slot + 1;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t rank = cluster_ctarank();  // 0 = leader
+  const uint32_t cta = cluster_ctarank();
+  const uint32_t rank = SPLIT > 1 ? cta & 1u : cta;          // in the pair, 0 = leader
+  const uint32_t leader_cta = SPLIT > 1 ? cta & ~1u : 0u;    // the leader's rank in the cluster
+  const uint16_t pair_mask = (uint16_t)(3u << leader_cta);   // both CTAs of the pair
+  const int split = SPLIT > 1 ? (int)(cta >> 1) : 0;         // which share of the contraction
   const bool leader = rank == 0;
-  const int pair_id = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
+  const int pair_id = blockIdx.x / (2 * SPLIT), n_pairs = gridDim.x / (2 * SPLIT);  // (SPLIT > 1: clusters)
   const int n_tiles = g.n_tiles;
   // Tile order inside a problem: groups of kGroupM row-blocks sweep all column-blocks before the next group
   // starts, so the group's rows of A and all of B stay in L2 while they are reused.
@@ -331,7 +353,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     m_blk = m0 + in_grp % gm;
     n_blk = in_grp / gm;
   };
-  auto k_blocks_of = [&](int tile) { return g.p[tile >= g.n_tiles0 ? 1 : 0].K / 256; };
+  auto k_first = [&](int k_blocks) { return SPLIT > 1 ? k_blocks * split / SPLIT : 0; };
+  auto k_end = [&](int k_blocks) { return SPLIT > 1 ? k_blocks * (split + 1) / SPLIT : k_blocks; };
+  auto k_blocks_of = [&](int tile) {  // this pair's
+    const int n = g.p[tile >= g.n_tiles0 ? 1 : 0].K / 256;
+    return k_end(n) - k_first(n);
+  };
   // Tiles go to the pairs in rounds, odd rounds in reverse pair order (a snake): with two problems of different
   // depth in one launch, the pairs that drew the deeper or the extra tiles of one round draw the shallower ones, or
   // none, in the next.  A balance measure only: on one problem it times the same as the plain round-robin.
@@ -348,10 +375,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       mbar_init(accf_bar(b), 1);
       mbar_init(acce_bar(b), 16);  // eight epilogue warps in each CTA
     }
-    mbar_init(done_bar, 1);
+    mbar_init(done_bar, 2 * SPLIT - 1);
+    if (SPLIT > 1) mbar_init(recv_bar, 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    if (SPLIT > 1) mbar_expect_tx(recv_bar, C::kRecvBytes);
   }
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32((const void*)tmem_slot)),
@@ -393,10 +422,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         const uint8_t* sfa = pr.sfa + (int64_t)grp_a * sf_atoms_k * 512;
         const uint8_t* sfb0 = pr.sfb + (int64_t)min(n_blk * kGroups, last_b) * sf_atoms_k * 512;
         const uint8_t* sfb1 = pr.sfb + (int64_t)min(n_blk * kGroups + 1, last_b) * sf_atoms_k * 512;
-        for (int kb = 0; kb < k_blocks; ++kb) {
+        for (int kb = k_first(k_blocks); kb < k_end(k_blocks); ++kb) {
           if (!(ok = mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag, 0x100u + stage))) break;
           const uint32_t st = base + stage * kStageBytes;
-          const uint32_t bar = map_to_cta(full_bar(stage), 0);  // the leader's barrier counts both CTAs' operands
+          const uint32_t bar = map_to_cta(full_bar(stage), leader_cta);  // the leader's barrier counts both CTAs' operands
           if (g.exp & 2) {
             mbar_expect_tx_cluster(bar, 0);  // measurement aid: no operand loads
           } else {
@@ -433,7 +462,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     const int quad = warp & 3;
     int stage = 0;
     uint32_t phase = 0;
-    const uint32_t sff_leader = map_to_cta(sff_bar(0), 0);
+    const uint32_t sff_leader = map_to_cta(sff_bar(0), leader_cta);
     for (int rnd = 0, tile = pair_id; tile < n_tiles; tile = next_tile(++rnd)) {
       bool ok = true;
       const int k_blocks = k_blocks_of(tile);
@@ -539,21 +568,21 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
               tc2_mma_nvf4(d_tmem, make_desc(a_lo + 2 * j, kDescHiOperand), make_desc(b_lo + 2 * j, kDescHiOperand), idesc,
                            sf_t + j * 4, sf_t + 16 + j * 4 * kGroups, (kb > 0 || j > 0) ? 1u : 0u);
           }
-          tc2_commit_both(empty_bar(stage), 3);  // both CTAs' stages are free once these MMAs have read them
+          tc2_commit_both(empty_bar(stage), pair_mask);  // both CTAs' stages are free once these MMAs have read them
           if (++stage == kStages) {
             stage = 0;
             phase ^= 1u;
           }
         }
         if (!ok) break;
-        tc2_commit_both(accf_bar(acc), 3);  // this accumulator is complete in both CTAs
+        tc2_commit_both(accf_bar(acc), pair_mask);  // this accumulator is complete in both CTAs
         acc_phase ^= 1u << acc;
         if (++acc == C::kAcc) acc = 0;
         probe_kb += (unsigned long long)k_blocks;
         ++probe_tiles;
         if (g.probe) probe_mark = clock64();
       }
-      if (g.probe) {
+      if (g.probe && split == 0) {
         // the last commit has been issued, not completed: wait for the accumulator hand-over of the last tile so that
         // the interval covers the work (bounded like every other wait)
         const int last = C::kAcc - 1 - acc;  // (one accumulator: itself; two: the one used last)
@@ -581,7 +610,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     const float alpha0 = __fmul_rn((ROWS && g.p[0].a_rows) ? 1.f : g.p[0].a_global[1], (ROWS && g.p[0].b_rows) ? 1.f : g.p[0].b_global[1]);
     const float alpha1 = __fmul_rn((ROWS && g.p[1].a_rows) ? 1.f : g.p[1].a_global[1], (ROWS && g.p[1].b_rows) ? 1.f : g.p[1].b_global[1]);
     float* beta = reinterpret_cast<float*>(base_ptr + kStages * kStageBytes + kStagingBytes + 256) + half * 128;
-    const uint32_t acce_leader = map_to_cta(acce_bar(0), 0);
+    const uint32_t acce_leader = map_to_cta(acce_bar(0), leader_cta);
     const int row_in_tile = quad * 32 + lane;
     const uint32_t t_row0 = tmem + ((uint32_t)(quad * 32) << 16) + half * kHalf;
     const uint32_t stage_buf = staging + half * 16384;
@@ -602,7 +631,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       if (a_rows) alpha *= a_rows[2 * (int64_t)(m_blk * 256 + (int)rank * 128 + quad * 32 + lane) + 1];
       // the group's 128 column factors; the first barrier inside store_half orders this write before their use, its
       // last one orders their use before the next tile's write
-      if (b_rows && et < kHalf) beta[et] = b_rows[2 * (int64_t)(n_blk * BN + half * kHalf + et) + 1];
+      if (SPLIT > 1) {
+        if (b_rows && et < C::kCols) beta[et] = b_rows[2 * (int64_t)(n_blk * BN + split * C::kCols + et) + 1];
+      } else if (b_rows && et < kHalf) {
+        beta[et] = b_rows[2 * (int64_t)(n_blk * BN + half * kHalf + et) + 1];
+      }
       mbar_wait_cluster(accf_bar(acc), (acc_phase >> acc) & 1u, abort_flag, 0x400u);
       // agree on giving up: a warp that timed out still joins this barrier, and all 128 threads take ONE decision
       if (group_gave_up(abort_flag, bar_id, 128)) break;
@@ -628,7 +661,54 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive_cluster(acce_leader + 8u * acc);
-      if (ROWS && b_rows) {
+      if constexpr (SPLIT > 1) {
+        constexpr int kCols = C::kCols, kMine = kHalf / kCols;  // columns of a pair; pairs whose columns this group reads
+        const uint32_t recv = staging + kStagingBytes + 256 + kBetaBytes;
+        const uint32_t at = (uint32_t)row_in_tile * 16;  // of four columns: [column / 4][row][16 bytes]
+        uint32_t v[kCols];
+#pragma unroll
+        for (int q = 0; q < kMine; ++q) {
+          const int to = half * kMine + q;  // the pair that finishes them
+          if (to == split) {
+#pragma unroll
+            for (int k = 0; k < kCols; ++k) v[k] = r[q * kCols + k];
+          } else {
+            const uint32_t to_cta = 2 * to + rank;
+            const uint32_t dst = map_to_cta(recv + (split < to ? split : split - 1) * C::kSlotBytes + at, to_cta);
+            const uint32_t bar = map_to_cta(recv_bar, to_cta);
+#pragma unroll
+            for (int k = 0; k < kCols; k += 4)
+              st_async16(dst + k * 512, r[q * kCols + k], r[q * kCols + k + 1], r[q * kCols + k + 2], r[q * kCols + k + 3], bar);
+          }
+        }
+        if (split / kMine != half) break;  // the other group of this CTA finishes the pair's columns
+        mbar_wait_cluster(recv_bar, 0, abort_flag, 0x700u);
+        if (group_gave_up(abort_flag, bar_id, 128)) break;
+#pragma unroll
+        for (int k = 0; k < kCols; k += 4) {
+          float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+          for (int p = 0; p < SPLIT; ++p) {
+            uint4 w = make_uint4(v[k], v[k + 1], v[k + 2], v[k + 3]);
+            if (p != split) w = lds128(recv + (p < split ? p : p - 1) * C::kSlotBytes + at + k * 512);
+            const float4 f = make_float4(__uint_as_float(w.x), __uint_as_float(w.y), __uint_as_float(w.z), __uint_as_float(w.w));
+            sum = p == 0 ? f : make_float4(sum.x + f.x, sum.y + f.y, sum.z + f.z, sum.w + f.w);
+          }
+          v[k] = __float_as_uint(sum.x); v[k + 1] = __float_as_uint(sum.y);
+          v[k + 2] = __float_as_uint(sum.z); v[k + 3] = __float_as_uint(sum.w);
+        }
+        const int xs = n_blk * BN + split * kCols;
+        if (ROWS && b_rows) {
+          if (d_is_fp32)
+            store_half<true, true, kCols>(v, alpha, et, bar_id, row_in_tile, stage_buf, map_d, xs, row0, accumulate, drain, beta);
+          else
+            store_half<false, true, kCols>(v, alpha, et, bar_id, row_in_tile, stage_buf, map_d, xs, row0, accumulate, drain, beta);
+        } else if (d_is_fp32) {
+          store_half<true, false, kCols>(v, alpha, et, bar_id, row_in_tile, stage_buf, map_d, xs, row0, accumulate, drain);
+        } else {
+          store_half<false, false, kCols>(v, alpha, et, bar_id, row_in_tile, stage_buf, map_d, xs, row0, accumulate, drain);
+        }
+      } else if (ROWS && b_rows) {
         if (d_is_fp32)
           store_half<true, true, kHalf>(r, alpha, et, bar_id, row_in_tile, stage_buf, map_d, x0, row0, accumulate, drain, beta);
         else
@@ -651,7 +731,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   tc_fence_before();
   __syncthreads();
   if (threadIdx.x == 0) {
-    mbar_arrive_cluster(map_to_cta(done_bar, rank ^ 1u));
+    for (uint32_t k = 1; k < 2 * SPLIT; ++k) mbar_arrive_cluster(map_to_cta(done_bar, cta ^ k));
     mbar_wait_cluster(done_bar, 0, abort_flag, 0x600u);
   }
   __syncthreads();

@@ -1,0 +1,64 @@
+"""Products whose contraction several CTA pairs share: shares of equal and unequal length down to one k-block, tiles half
+outside, both output types, every scale format, accumulation, and sizes on both sides of the rule that chooses it."""
+import pytest
+import torch
+
+import parity as P
+from paper_2509_25149_b200 import binding as B
+from paper_2509_25149_b200 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+def _operands(M, N, K, fmt):
+    f = B.FORMAT_MXFP4 if fmt == "mxfp4" else B.FORMAT_NVFP4
+    A = B.alloc_tensor(M, K, format=B.FORMAT_NVFP4_ROWSCALE if fmt == "rows" else f)
+    Bt = B.alloc_tensor(N, K, format=f)
+    B.nvfp4_quantize(synth.normal_with_outliers_bf16((M, K), 0.01, 50.0, M + N, M + N + 1).cuda(), B.quant_opts(), A, None)
+    B.nvfp4_quantize(synth.normal_bf16((N, K), 0.02, M + N + 2).cuda(),
+                     B.quant_opts(block_rows=32 if fmt == "mxfp4" else 16), Bt, None)
+    a, b = B.nvfp4_dequantize(A).double(), B.nvfp4_dequantize(Bt).double()
+    return A, Bt, (a @ b.T).cpu().numpy(), (a.abs() @ b.abs().T).cpu().numpy()
+
+
+@pytest.mark.parametrize("shape", [(256, 256, 512), (256, 256, 1024), (128, 384, 1280), (512, 512, 1792), (384, 128, 5120),
+                                   (256, 8192, 1024)])
+@pytest.mark.parametrize("tile", [642, 644])
+@pytest.mark.parametrize("fp32", [False, True])
+@pytest.mark.parametrize("fmt", ["nvfp4", "mxfp4", "rows"])
+def test_shared_contraction(shape, tile, fp32, fmt):
+    M, N, K = shape
+    if fmt == "rows":
+        M, N = (M + 255) // 256 * 256, (N + 255) // 256 * 256
+    A, Bt, want, T = _operands(M, N, K, fmt)
+    wide = torch.full((M + 8, N + 64), 7.0, dtype=torch.float32 if fp32 else torch.bfloat16, device="cuda")
+    D = wide[:M, :N]
+    B.nvfp4_set_gemm_tile_n(tile)
+    try:
+        B.nvfp4_gemm(A, Bt, D)
+        B.nvfp4_device_status()
+        P.assert_gemm_close(D.float().cpu().numpy(), want, T, not fp32, f"{fmt} {shape} split {tile}")
+        assert torch.all(wide[M:] == 7.0) and torch.all(wide[:, N:] == 7.0)
+        once = D.clone()
+        B.nvfp4_gemm(A, Bt, D)
+        assert torch.equal(D, once)  # the shares are added in a fixed order
+        if fp32:  # what is added is the very product
+            B.nvfp4_gemm(A, Bt, D, accumulate=True)
+            B.nvfp4_device_status()
+            assert torch.equal(D, once + once)
+    finally:
+        B.nvfp4_set_gemm_tile_n(0)
+
+
+@pytest.mark.parametrize("shape", [(256, 256, 1280), (256, 256, 2560), (256, 1024, 4096), (1024, 1024, 8192), (1024, 1152, 8192),
+                                   (128, 128, 20480)])
+def test_sizes_around_the_rule(shape):
+    """Chosen by size: 8 products behind each other (their clusters start while the one before drains) give the same bits."""
+    M, N, K = shape
+    A, Bt, want, T = _operands(M, N, K, "nvfp4")
+    outs = [torch.empty((M, N), device="cuda") for _ in range(8)]
+    for D in outs:
+        B.nvfp4_gemm(A, Bt, D)
+    B.nvfp4_device_status()
+    P.assert_gemm_close(outs[0].cpu().numpy(), want, T, False, f"{shape}")
+    assert all(torch.equal(D, outs[0]) for D in outs)
