@@ -546,26 +546,29 @@ double pair_makespan(const GemmArgs* const* gs, int n_problems, int tile, int pa
   return worst;
 }
 
-// Clusters of SPLIT pairs that are resident at once on the current device (0: none)
-template <int SPLIT>
-int split_clusters() {
+// Clusters of 2 * SPLIT CTAs of this kernel that are resident at once on the current device (0: none)
+template <auto KERN, int SPLIT>
+int resident_clusters(int threads, int smem) {
   constexpr int kMaxDevices = 64;
   static std::atomic<int> known[kMaxDevices];  // the number + 1
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return 0;
   if (const int n = known[dev].load(std::memory_order_relaxed)) return n - 1;
-  auto kern = pair::gemm_pair_kernel<false, false, 128, SPLIT>;
-  constexpr int smem = pair::Cfg<128, SPLIT>::kSmemBytes;
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(2 * SPLIT);
-  cfg.blockDim = dim3(pair::kThreads);
+  cfg.blockDim = dim3(threads);
   cfg.dynamicSmemBytes = smem;
   int n = 0;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
-      cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess)
+  if (cudaFuncSetAttribute(KERN, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
+      cudaOccupancyMaxActiveClusters(&n, KERN, &cfg) != cudaSuccess)
     n = 0;
   known[dev].store(n + 1, std::memory_order_relaxed);
   return n;
+}
+template <int SPLIT>
+int split_clusters() {
+  return resident_clusters<pair::gemm_pair_kernel<false, false, 128, SPLIT>, SPLIT>(pair::kThreads,
+                                                                                   pair::Cfg<128, SPLIT>::kSmemBytes);
 }
 
 // The split of a product that has a launch to itself, or 0 (`least`: the estimate of the best tile).  A split pays where a
@@ -700,7 +703,7 @@ int best_pair_tile(const GemmArgs& g0, const GemmArgs* g1) {
   return best;
 }
 
-template <int BN>
+template <int BN, int SPLIT>
 static bool make_bf16_maps(const DenseGemmArgs& g, CUtensorMap* m) {  // A, B, D
   const CUtensorMapDataType bf = CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
   bool ok = g.a_mn ? make_map_2d(&m[0], bf, 2, g.a, (uint64_t)g.M, (uint64_t)g.K, (uint64_t)g.lda * 2, 64, 64, true)
@@ -711,27 +714,29 @@ static bool make_bf16_maps(const DenseGemmArgs& g, CUtensorMap* m) {  // A, B, D
     ok = ok && make_map_2d(&m[2], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, g.d, (uint64_t)g.N, (uint64_t)g.M,
                            (uint64_t)g.ldd * 4, 16, 128, 2);
   else
-    ok = ok && make_map_2d(&m[2], bf, 2, g.d, (uint64_t)g.N, (uint64_t)g.M, (uint64_t)g.ldd * 2, 64, 128, true);
+    ok = ok && make_map_2d(&m[2], bf, 2, g.d, (uint64_t)g.N, (uint64_t)g.M, (uint64_t)g.ldd * 2,
+                           SPLIT == 4 ? 32 : 64, 128, SPLIT == 4 ? 2 : 1);
   return ok;
 }
 
 static int bf16_tiles(const DenseGemmArgs& g, int bn) { return ((g.M + 255) / 256) * ((g.N + bn - 1) / bn); }
 
 // g1 == nullptr: one problem
-template <int BN>
+template <int BN, int SPLIT = 1>
 static cudaError_t launch_bf16_t(const DenseGemmArgs& g0, const DenseGemmArgs* g1, int max_pairs, cudaStream_t s) {
-  auto kern = dense::gemm_bf16_pair_kernel<BN>;
+  auto kern = dense::gemm_bf16_pair_kernel<BN, SPLIT>;
+  constexpr int smem = dense::Cfg<BN, SPLIT>::kSmemBytes;
   CUtensorMap m[6];
-  if (!make_bf16_maps<BN>(g0, m)) return cudaErrorInvalidValue;
+  if (!make_bf16_maps<BN, SPLIT>(g0, m)) return cudaErrorInvalidValue;
   if (g1) {
-    if (!make_bf16_maps<BN>(*g1, m + 3)) return cudaErrorInvalidValue;
+    if (!make_bf16_maps<BN, SPLIT>(*g1, m + 3)) return cudaErrorInvalidValue;
   } else {
     for (int i = 0; i < 3; ++i) m[3 + i] = m[i];
   }
   static std::atomic<uint64_t> configured{0};  // per call site (template instantiation) and device
   int dev;
   if (device_needs_config(configured, &dev)) {
-    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, dense::kSmemBytes);
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
     device_configured(configured, dev);
   }
@@ -743,8 +748,8 @@ static cudaError_t launch_bf16_t(const DenseGemmArgs& g0, const DenseGemmArgs* g
   a.p[1] = problem(g1 ? *g1 : g0);
   a.n_tiles0 = bf16_tiles(g0, BN);
   a.n_tiles = a.n_tiles0 + (g1 ? bf16_tiles(*g1, BN) : 0);
-  const int pairs = a.n_tiles < max_pairs ? a.n_tiles : max_pairs;
-  const cudaError_t e = launch_kernel(kern, dim3(2 * pairs), dim3(dense::kThreads), dense::kSmemBytes, s, m[0], m[1], m[2],
+  const int pairs = a.n_tiles < max_pairs || SPLIT > 1 ? a.n_tiles : max_pairs;  // SPLIT > 1: a cluster for each tile
+  const cudaError_t e = launch_kernel(kern, dim3(2 * SPLIT * pairs), dim3(dense::kThreads), smem, s, m[0], m[1], m[2],
                                       m[3], m[4], m[5], a);
   count_launch();
   return e;
@@ -759,6 +764,23 @@ cudaError_t launch_gemm_bf16(const DenseGemmArgs& g0, const DenseGemmArgs* g1, c
   // an instruction 128 columns wide takes as long as one 256 wide (264 x 7168 x 5120 30 -> 50 us).
   const int pairs = num_sms / 2;
   const int64_t tiles128 = (int64_t)bf16_tiles(g0, 128) + (g1 ? bf16_tiles(*g1, 128) : 0);
+  // Fewer tiles than clusters of several pairs: each tile's contraction is shared by two or four pairs, where what that saves
+  // of the longest contraction (0.305 us per 64 deep) exceeds the exchange, 1.1 us (1.5 where most of the chip takes part) |
+  // 1.6.  One / two / four pairs per tile: 264 x 512 x 512 6.4 / 6.0 / 6.2 us, 264 x 512 x 4096 23.6 / 14.8 / 10.4, 512 x 512 x
+  // 16384 83 / 45 / 26, 1024 x 1024 x 512 6.5 / 6.6 / 18.5 (two rounds), 1024 x 1024 x 4096 24.9 / 16.2 / 31.5.
+  auto clusters = [](auto split) {
+    constexpr int kSplit = decltype(split)::value;
+    return resident_clusters<dense::gemm_bf16_pair_kernel<128, kSplit>, kSplit>(dense::kThreads,
+                                                                             dense::Cfg<128, kSplit>::kSmemBytes);
+  };
+  const int kb0 = (g0.K + 63) / 64, kb1 = g1 ? (g1->K + 63) / 64 : kb0, kb = kb0 > kb1 ? kb0 : kb1;
+  auto gain = [&](int split) {
+    return 0.305 * (kb - (kb + split - 1) / split) - (split == 4 ? 1.6 : tiles128 > 16 ? 1.5 : 1.1);
+  };
+  if (tiles128 <= 64 && (kb0 < kb1 ? kb0 : kb1) >= 4 && gain(2) > 0.2) {
+    if (gain(4) > gain(2) && tiles128 <= clusters(std::integral_constant<int, 4>())) return launch_bf16_t<128, 4>(g0, g1, pairs, s);
+    if (tiles128 <= clusters(std::integral_constant<int, 2>())) return launch_bf16_t<128, 2>(g0, g1, pairs, s);
+  }
   return tiles128 <= pairs ? launch_bf16_t<128>(g0, g1, pairs, s) : launch_bf16_t<256>(g0, g1, pairs, s);
 }
 

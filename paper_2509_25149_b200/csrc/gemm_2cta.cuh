@@ -40,8 +40,7 @@ struct Cfg {
   static constexpr int kSfbBytes = 4 * kGroups * 512;   // all rows of B (both CTAs need them), four K64 steps
   static constexpr int kStageBytes = kABytes + kBBytes + kSfaBytes + kSfbBytes;  // 38 / 28 KB
   static constexpr int kCols = BN / SPLIT;              // columns that a pair finishes and stores
-  static constexpr int kSlotBytes = 128 * kCols * 4;    // one other pair's share of them (this CTA's 128 rows)
-  static constexpr int kRecvBytes = (SPLIT - 1) * kSlotBytes;
+  static constexpr int kRecvBytes = (SPLIT - 1) * 128 * kCols * 4;  // the other pairs' shares of them (this CTA's 128 rows)
   static constexpr int kSmemBytes =
       kStages * kStageBytes + kStagingBytes + 1024 /*alignment*/ + 256 /*barriers*/ + kBetaBytes + kRecvBytes;
   static constexpr int kSfCol = 256;                    // after the accumulator columns: one slot per stage
@@ -290,6 +289,50 @@ __device__ __forceinline__ void store_half(const uint32_t (&r)[COLS], float alph
       bulk_commit();
     }
   }
+}
+
+// The exchange of a split tile (256 x 128, SPLIT pairs, see gemm_pair_kernel): r = this pair's sums of the 64 columns that this
+// epilogue group reads.  Sends them to the pairs that finish them and, in the group that holds this pair's own columns, leaves
+// the complete sums in v.  false: nothing (more) to do in this group.  recv: [other pair][column / 4][row][four columns].
+template <int SPLIT>
+__device__ __forceinline__ bool exchange_columns(const uint32_t (&r)[64], uint32_t (&v)[128 / SPLIT], int half, int split,
+                                                 uint32_t rank, uint32_t recv, uint32_t recv_bar, int row_in_tile,
+                                                 volatile uint32_t* abort_flag, int bar_id) {
+  constexpr int kCols = 128 / SPLIT, kMine = 64 / kCols;  // columns of a pair; pairs whose columns this group reads
+  constexpr int kSlot = 128 * kCols * 4;
+  const uint32_t at = (uint32_t)row_in_tile * 16;
+#pragma unroll
+  for (int q = 0; q < kMine; ++q) {
+    const int to = half * kMine + q;  // the pair that finishes them
+    if (to == split) {
+#pragma unroll
+      for (int k = 0; k < kCols; ++k) v[k] = r[q * kCols + k];
+    } else {
+      const uint32_t to_cta = 2 * to + rank;
+      const uint32_t dst = map_to_cta(recv + (split < to ? split : split - 1) * kSlot + at, to_cta);
+      const uint32_t bar = map_to_cta(recv_bar, to_cta);
+#pragma unroll
+      for (int k = 0; k < kCols; k += 4)
+        st_async16(dst + k * 512, r[q * kCols + k], r[q * kCols + k + 1], r[q * kCols + k + 2], r[q * kCols + k + 3], bar);
+    }
+  }
+  if (split / kMine != half) return false;  // the other group of this CTA finishes the pair's columns
+  mbar_wait_cluster(recv_bar, 0, abort_flag, 0x700u);
+  if (group_gave_up(abort_flag, bar_id, 128)) return false;
+#pragma unroll
+  for (int k = 0; k < kCols; k += 4) {
+    float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int p = 0; p < SPLIT; ++p) {
+      uint4 w = make_uint4(v[k], v[k + 1], v[k + 2], v[k + 3]);
+      if (p != split) w = lds128(recv + (p < split ? p : p - 1) * kSlot + at + k * 512);
+      const float4 f = make_float4(__uint_as_float(w.x), __uint_as_float(w.y), __uint_as_float(w.z), __uint_as_float(w.w));
+      sum = p == 0 ? f : make_float4(sum.x + f.x, sum.y + f.y, sum.z + f.z, sum.w + f.w);
+    }
+    v[k] = __float_as_uint(sum.x); v[k + 1] = __float_as_uint(sum.y);
+    v[k + 2] = __float_as_uint(sum.z); v[k + 3] = __float_as_uint(sum.w);
+  }
+  return true;
 }
 
 // MX = false: NVFP4 (E4M3 scale per 16 elements: one 512-byte atom per 128 rows and K = 64).
@@ -662,41 +705,11 @@ __global__ void __cluster_dims__(2 * SPLIT, 1, 1) __launch_bounds__(kThreads, 1)
       __syncwarp();
       if (lane == 0) mbar_arrive_cluster(acce_leader + 8u * acc);
       if constexpr (SPLIT > 1) {
-        constexpr int kCols = C::kCols, kMine = kHalf / kCols;  // columns of a pair; pairs whose columns this group reads
-        const uint32_t recv = staging + kStagingBytes + 256 + kBetaBytes;
-        const uint32_t at = (uint32_t)row_in_tile * 16;  // of four columns: [column / 4][row][16 bytes]
+        constexpr int kCols = C::kCols;
         uint32_t v[kCols];
-#pragma unroll
-        for (int q = 0; q < kMine; ++q) {
-          const int to = half * kMine + q;  // the pair that finishes them
-          if (to == split) {
-#pragma unroll
-            for (int k = 0; k < kCols; ++k) v[k] = r[q * kCols + k];
-          } else {
-            const uint32_t to_cta = 2 * to + rank;
-            const uint32_t dst = map_to_cta(recv + (split < to ? split : split - 1) * C::kSlotBytes + at, to_cta);
-            const uint32_t bar = map_to_cta(recv_bar, to_cta);
-#pragma unroll
-            for (int k = 0; k < kCols; k += 4)
-              st_async16(dst + k * 512, r[q * kCols + k], r[q * kCols + k + 1], r[q * kCols + k + 2], r[q * kCols + k + 3], bar);
-          }
-        }
-        if (split / kMine != half) break;  // the other group of this CTA finishes the pair's columns
-        mbar_wait_cluster(recv_bar, 0, abort_flag, 0x700u);
-        if (group_gave_up(abort_flag, bar_id, 128)) break;
-#pragma unroll
-        for (int k = 0; k < kCols; k += 4) {
-          float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-          for (int p = 0; p < SPLIT; ++p) {
-            uint4 w = make_uint4(v[k], v[k + 1], v[k + 2], v[k + 3]);
-            if (p != split) w = lds128(recv + (p < split ? p : p - 1) * C::kSlotBytes + at + k * 512);
-            const float4 f = make_float4(__uint_as_float(w.x), __uint_as_float(w.y), __uint_as_float(w.z), __uint_as_float(w.w));
-            sum = p == 0 ? f : make_float4(sum.x + f.x, sum.y + f.y, sum.z + f.z, sum.w + f.w);
-          }
-          v[k] = __float_as_uint(sum.x); v[k + 1] = __float_as_uint(sum.y);
-          v[k + 2] = __float_as_uint(sum.z); v[k + 3] = __float_as_uint(sum.w);
-        }
+        if (!exchange_columns<SPLIT>(r, v, half, split, rank, staging + kStagingBytes + 256 + kBetaBytes, recv_bar, row_in_tile,
+                                     abort_flag, bar_id))
+          break;
         const int xs = n_blk * BN + split * kCols;
         if (ROWS && b_rows) {
           if (d_is_fp32)

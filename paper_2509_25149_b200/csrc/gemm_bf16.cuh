@@ -23,11 +23,17 @@ namespace nvfp4 {
 namespace dense {
 
 constexpr int kThreads = 320;       // producer, MMA issuer, 2 x 4 epilogue warps
-constexpr int kStages = 6;
 constexpr int kOperandBytes = 128 * 128;           // 128 rows (or output indices) x 64 bf16
-constexpr int kStageBytes = 2 * kOperandBytes;     // A, this CTA's half of B
 constexpr int kStagingBytes = 2 * 16384;
-constexpr int kSmemBytes = kStages * kStageBytes + kStagingBytes + 1024 /*alignment*/ + 256 /*barriers*/;
+constexpr int kStages = 6;
+template <int BN, int SPLIT>
+struct Cfg {
+  // A, this CTA's half of B.  (32 KB for the narrow tile as well: 24 KB apart, 1024 x 1280 x 4096 takes 24.3 us, not 23.9)
+  static constexpr int kStageBytes = SPLIT > 1 ? kOperandBytes + BN / 2 * 128 : 2 * kOperandBytes;
+  static constexpr int kRecvBytes = (SPLIT - 1) * 128 * (BN / SPLIT) * 4;
+  static constexpr int kSmemBytes = kStages * kStageBytes + kStagingBytes + 1024 /*alignment*/ + 256 /*barriers*/ + kRecvBytes;
+  static_assert(kSmemBytes <= 232448, "shared memory budget");
+};
 constexpr uint32_t kTmemCols = 512;                // two 256-column accumulators
 
 struct Problem {
@@ -60,35 +66,45 @@ __device__ __forceinline__ void tc2_mma_bf16(uint32_t d_tmem, uint64_t adesc, ui
       : "memory");
 }
 
-template <int BN>  // columns of a tile (256 or 128)
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
+// BN: columns of a tile (256 or 128).  SPLIT > 1 (BN = 128): a cluster of SPLIT pairs takes one tile, the only one of its life,
+// each pair a share of the k-blocks (the exchange: pair::exchange_columns).
+template <int BN, int SPLIT = 1>
+__global__ void __cluster_dims__(2 * SPLIT, 1, 1) __launch_bounds__(kThreads, 1)
     gemm_bf16_pair_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant__ CUtensorMap map_b0,
                           const __grid_constant__ CUtensorMap map_d0, const __grid_constant__ CUtensorMap map_a1,
                           const __grid_constant__ CUtensorMap map_b1, const __grid_constant__ CUtensorMap map_d1,
                           const __grid_constant__ Args g) {
   using namespace pair;
+  constexpr int S = dense::kStages, kStageBytes = dense::Cfg<BN, SPLIT>::kStageBytes;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t* base_ptr = smem_raw + (base - smem_u32(smem_raw));
-  const uint32_t staging = base + dense::kStages * dense::kStageBytes;
+  const uint32_t staging = base + S * kStageBytes;
   const uint32_t bar_base = staging + dense::kStagingBytes;
-  constexpr int S = dense::kStages;
   auto full_bar = [&](int s) { return bar_base + 8u * s; };              // leader only: both CTAs' operands landed
   auto empty_bar = [&](int s) { return bar_base + 8u * (S + s); };       // one per CTA
   auto accf_bar = [&](int b) { return bar_base + 8u * (2 * S + b); };    // one per CTA and accumulator
   auto acce_bar = [&](int b) { return bar_base + 8u * (2 * S + 2 + b); };  // leader only, 16 arrivals
   const uint32_t done_bar = bar_base + 8u * (2 * S + 4);
+  const uint32_t recv_bar = done_bar + 16;                               // SPLIT > 1: all shares are here
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(
-      base_ptr + S * dense::kStageBytes + dense::kStagingBytes + 8 * (2 * S + 5));
+      base_ptr + S * kStageBytes + dense::kStagingBytes + 8 * (2 * S + 5));
   volatile uint32_t* abort_flag = tmem_slot + 1;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t rank = cluster_ctarank();  // 0 = leader
+  const uint32_t cta = cluster_ctarank();
+  const uint32_t rank = SPLIT > 1 ? cta & 1u : cta;          // in the pair, 0 = leader
+  const uint32_t leader_cta = SPLIT > 1 ? cta & ~1u : 0u;    // the leader's rank in the cluster
+  const uint16_t pair_mask = (uint16_t)(3u << leader_cta);   // both CTAs of the pair
+  const int split = SPLIT > 1 ? (int)(cta >> 1) : 0;         // which share of the contraction
   const bool leader = rank == 0;
-  const int pair_id = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
+  const int pair_id = blockIdx.x / (2 * SPLIT), n_pairs = gridDim.x / (2 * SPLIT);  // (SPLIT > 1: clusters)
   // ragged edges: loads beyond the operands read zeros, stores beyond D are clipped (both by the tensor maps)
   const int n_tiles = g.n_tiles;
-  auto k_blocks_of = [&](int tile) { return (g.p[tile >= g.n_tiles0 ? 1 : 0].K + 63) / 64; };
+  auto k_begin = [&](int tile, int s) {  // first k-block of share s
+    const int n = (g.p[tile >= g.n_tiles0 ? 1 : 0].K + 63) / 64;
+    return SPLIT > 1 ? n * s / SPLIT : n * s;
+  };
   // groups of eight row-blocks sweep all column-blocks before the next group starts (L2 reuse of A and B)
   constexpr int kGroupM = 8;
   auto tile_coords = [&](int tile, int& prob, int& m_blk, int& n_blk) {
@@ -112,10 +128,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       mbar_init(accf_bar(b), 1);
       mbar_init(acce_bar(b), 16);  // eight epilogue warps in each CTA
     }
-    mbar_init(done_bar, 1);
+    mbar_init(done_bar, 2 * SPLIT - 1);
+    if (SPLIT > 1) mbar_init(recv_bar, 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    if (SPLIT > 1) mbar_expect_tx(recv_bar, dense::Cfg<BN, SPLIT>::kRecvBytes);
   }
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32((const void*)tmem_slot)),
@@ -142,13 +160,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         tile_coords(tile, prob, m_blk, n_blk);
         const CUtensorMap* map_a = prob ? &map_a1 : &map_a0;
         const CUtensorMap* map_b = prob ? &map_b1 : &map_b0;
-        const int a_mn = g.p[prob].a_mn, b_mn = g.p[prob].b_mn, k_blocks = k_blocks_of(tile);
+        const int a_mn = g.p[prob].a_mn, b_mn = g.p[prob].b_mn, k_end = k_begin(tile, split + 1);
         const int row_a = m_blk * 256 + (int)rank * 128;  // this CTA's rows of A
         const int row_b = n_blk * BN + (int)rank * (BN / 2);  // this CTA's half of the B tile
-        for (int kb = 0; kb < k_blocks; ++kb) {
+        for (int kb = k_begin(tile, split); kb < k_end; ++kb) {
           if (!(ok = mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag, 0x900u + stage))) break;
-          const uint32_t st = base + stage * dense::kStageBytes;
-          const uint32_t bar = map_to_cta(full_bar(stage), 0);  // the leader's barrier counts both CTAs' operands
+          const uint32_t st = base + stage * kStageBytes;
+          const uint32_t bar = map_to_cta(full_bar(stage), leader_cta);  // the leader's barrier counts both CTAs' operands
           mbar_expect_tx_cluster(bar, dense::kOperandBytes + BN / 2 * 128);
           if (a_mn) {
             tma_load_2d_pair(st, map_a, row_a, kb * 64, bar);
@@ -191,24 +209,24 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         const uint32_t b_lo0 = b_lo_base | ((pr.b_mn ? (8192u >> 4) : 1u) << 16);
         const uint32_t a_step = pr.a_mn ? (2048u >> 4) : (32u >> 4);  // one K = 16 instruction further
         const uint32_t b_step = pr.b_mn ? (2048u >> 4) : (32u >> 4);
-        const int k_blocks = k_blocks_of(tile);
+        const int k_blocks = k_begin(tile, split + 1) - k_begin(tile, split);
         for (int kb = 0; kb < k_blocks; ++kb) {
           if (!(ok = mbar_wait_cluster(full_bar(stage), phase, abort_flag, 0xA00u + stage))) break;
           tc_fence_after();
-          const uint32_t a_lo = a_lo0 + stage * (dense::kStageBytes >> 4);
-          const uint32_t b_lo = b_lo0 + stage * (dense::kStageBytes >> 4);
+          const uint32_t a_lo = a_lo0 + stage * (kStageBytes >> 4);
+          const uint32_t b_lo = b_lo0 + stage * (kStageBytes >> 4);
 #pragma unroll
           for (int j = 0; j < 4; ++j)
             tc2_mma_bf16(d_t, make_desc(a_lo + j * a_step, kDescHiOperand), make_desc(b_lo + j * b_step, kDescHiOperand),
                          idesc, (kb > 0 || j > 0) ? 1u : 0u);
-          tc2_commit_both(empty_bar(stage), 3);  // both CTAs' stages are free once these MMAs have read them
+          tc2_commit_both(empty_bar(stage), pair_mask);  // both CTAs' stages are free once these MMAs have read them
           if (++stage == S) {
             stage = 0;
             phase ^= 1u;
           }
         }
         if (!ok) break;
-        tc2_commit_both(accf_bar(buf), 3);  // this accumulator is complete in both CTAs
+        tc2_commit_both(accf_bar(buf), pair_mask);  // this accumulator is complete in both CTAs
         acc_phase ^= 1u << buf;
       }
     }
@@ -241,8 +259,19 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       tc_wait_ld();
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive_cluster(map_to_cta(acce_bar(buf), 0));
-      if (g.p[prob].d_is_fp32)
+      if (lane == 0) mbar_arrive_cluster(map_to_cta(acce_bar(buf), leader_cta));
+      if constexpr (SPLIT > 1) {
+        constexpr int kCols = BN / SPLIT;
+        uint32_t v[kCols];
+        if (!exchange_columns<SPLIT>(r, v, half, split, rank, staging + dense::kStagingBytes + 256, recv_bar, row_in_tile,
+                                     abort_flag, bar_id))
+          break;
+        const int xs = n_blk * BN + split * kCols;
+        if (g.p[prob].d_is_fp32)
+          store_half<true, false, kCols>(v, 1.0f, et, bar_id, row_in_tile, stage_buf, map_d, xs, row0, g.p[prob].accumulate, drain);
+        else
+          store_half<false, false, kCols>(v, 1.0f, et, bar_id, row_in_tile, stage_buf, map_d, xs, row0, g.p[prob].accumulate, drain);
+      } else if (g.p[prob].d_is_fp32)
         store_half<true, false, BN / 2>(r, 1.0f, et, bar_id, row_in_tile, stage_buf, map_d, n_blk * BN + half * (BN / 2),
                                         row0, g.p[prob].accumulate, drain);
       else
@@ -258,7 +287,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   tc_fence_before();
   __syncthreads();
   if (threadIdx.x == 0) {
-    mbar_arrive_cluster(map_to_cta(done_bar, rank ^ 1u));
+    for (uint32_t k = 1; k < 2 * SPLIT; ++k) mbar_arrive_cluster(map_to_cta(done_bar, cta ^ k));
     mbar_wait_cluster(done_bar, 0, abort_flag, 0xD00u);
   }
   __syncthreads();

@@ -1,4 +1,4 @@
-"""Products whose contraction several CTA pairs share: shares of equal and unequal length down to one k-block, tiles half
+"""Products whose contraction several CTA pairs share (block-scaled and BF16): shares of equal and unequal length down to one k-block, tiles half
 outside, both output types, every scale format, accumulation, and sizes on both sides of the rule that chooses it."""
 import pytest
 import torch
@@ -62,3 +62,26 @@ def test_sizes_around_the_rule(shape):
     B.nvfp4_device_status()
     P.assert_gemm_close(outs[0].cpu().numpy(), want, T, False, f"{shape}")
     assert all(torch.equal(D, outs[0]) for D in outs)
+
+
+# shares of one k-block (K = 256) and of unequal length, ragged sizes; the last two lie beyond the rule (33 tiles and more)
+@pytest.mark.parametrize("shape", [(256, 128, 256), (264, 520, 1000), (520, 264, 2056), (512, 1024, 4096), (1000, 1000, 1032),
+                                   (128, 4096, 1024), (1000, 2000, 1000), (1288, 1024, 776)])
+def test_bf16_products(shape):
+    """Against binary64.  A sum of K products in FP32: K roundings of 2^-23 of what the terms' magnitudes add up to at most."""
+    M, N, K = shape
+    gen = torch.Generator("cuda").manual_seed(M + N + K)
+    X, W, dY = (torch.randn(s, generator=gen, device="cuda").to(torch.bfloat16) for s in ((M, K), (N, K), (M, N)))
+    Y, dX = (torch.full((M, n), 7.0, dtype=torch.bfloat16, device="cuda") for n in (N, K))
+    dW = torch.full((N, K), 2.0, device="cuda")
+    B.nvfp4_linear_bf16_fwd(X, W, Y)
+    B.nvfp4_linear_bf16_bwd(dY, X, W, K, dX, dW, True)
+    B.nvfp4_device_status()
+    x, w, dy = X.double(), W.double(), dY.double()
+    for got, a, b, depth, bf16 in ((Y, x, w, K, True), (dX, dy, w.T, N, True), (dW - 2.0, dy.T, x.T, M, False)):
+        want, T = a @ b.T, a.abs() @ b.abs().T
+        bound = depth * 2.0 ** -23 * T + (2.0 ** -8 * want.abs() if bf16 else 2.0 ** -22 * (want.abs() + 2.0))
+        assert torch.all((got.double() - want).abs() <= bound)
+    again = torch.empty_like(Y)
+    B.nvfp4_linear_bf16_fwd(X, W, again)
+    assert torch.equal(again, Y)
