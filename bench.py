@@ -535,7 +535,7 @@ CASES = {
     "quant_w_f32": ("qw_f32", 20480, 5120, 0),      # 16x16 blocks, both copies, from a binary32 source (419 MB)
     "step": ("step", 8192, 20480, 5120),           # the whole cfg 3 fwd + bwd step, full size: ONE-PASS captures only
     "fwd_half": ("fwd", 8192, 10240, 5120),         # forward call, half the output features (X 84 MB, W 105 MB): the
-                                                    # quantize kernel of X that carries the amax pass of W
+                                                    # launches that quantize X and W together
     "gemm_bf16_fprop": ("bf16", 4096, 5120, 5120),  # BF16 layer (Section 4.1): Y = X W^T, both operands K-major
     "gemm_bf16_wgrad": ("bf16_wgrad", 5120, 5120, 4096),  # dW = dY^T X, both operands read transposed, fp32 output
     "step_bf16": ("step_bf16", 8192, 20480, 5120),  # the cfg 3 layer kept in BF16, fwd + bwd, full size
