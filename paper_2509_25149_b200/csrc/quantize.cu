@@ -370,25 +370,6 @@ __device__ __forceinline__ float encode_scale_of_byte(uint32_t byte, float s_dec
   return (byte == 0u) ? 0.0f : fminf(__frcp_rn(d), kFltMax);
 }
 
-// Row-by-row scale bytes of a tile of ROWS x KB blocks (staged row by row): as words where the row length keeps them aligned.
-// Row lengths are any number; otherwise the bytes leave one by one, but neighbouring lanes write the bytes of a row: a warp's store touches four rows, not sixteen (four bytes of a row
-// per thread made the stores a microsecond of the tile's five).
-template <int ROWS, int KB>
-__device__ __forceinline__ void store_linear_scales(const uint8_t* src, uint8_t* dst, int64_t R0, int64_t K0, int64_t Rn,
-                                                    int64_t n_kb, bool full_tile) {
-  if (full_tile && (n_kb & 3) == 0) {
-    if (threadIdx.x < ROWS * KB / 4)
-      *reinterpret_cast<uint32_t*>(dst + (R0 + threadIdx.x / (KB / 4)) * n_kb + K0 + threadIdx.x % (KB / 4) * 4) =
-          *reinterpret_cast<const uint32_t*>(src + threadIdx.x * 4);
-    return;
-  }
-  const int r = threadIdx.x / KB, kb = threadIdx.x % KB;
-  uint8_t* d = dst + (R0 + r) * n_kb + K0 + kb;
-#pragma unroll
-  for (int p = 0; p < ROWS * KB / 256; ++p, d += 256 / KB * n_kb)
-    if (full_tile || (R0 + r + 256 / KB * p < Rn && K0 + kb < n_kb)) *d = src[threadIdx.x + 256 * p];
-}
-
 template <bool HAS_ROW, bool HAS_COL, bool BLOCK2D, bool RHT_ROW, bool RHT_COL, bool SR, int TC, bool F32 = false,
           bool PARTS = false>
 __device__ __forceinline__ void quantize_tiles(const CUtensorMap* src_map, const QuantArgs& a, const int block,

@@ -197,4 +197,24 @@ __device__ __forceinline__ float amax16(const float (&f)[16]) {
   return m;
 }
 
+// Row-by-row scale bytes of a tile of ROWS x KB blocks (staged row by row): as words where the row length keeps them aligned.
+// Row lengths are any number; otherwise the bytes leave one by one, but neighbouring lanes write the bytes of a row: a warp's
+// store touches four (eight) rows, not sixteen (four bytes of a row per thread made the stores a microsecond of the tile's
+// five).
+template <int ROWS, int KB>
+__device__ __forceinline__ void store_linear_scales(const uint8_t* src, uint8_t* dst, int64_t R0, int64_t K0, int64_t Rn,
+                                                    int64_t n_kb, bool full_tile) {
+  if (full_tile && (n_kb & 3) == 0) {
+    if (threadIdx.x < ROWS * KB / 4)
+      *reinterpret_cast<uint32_t*>(dst + (R0 + threadIdx.x / (KB / 4)) * n_kb + K0 + threadIdx.x % (KB / 4) * 4) =
+          *reinterpret_cast<const uint32_t*>(src + threadIdx.x * 4);
+    return;
+  }
+  const int r = threadIdx.x / KB, kb = threadIdx.x % KB;
+  uint8_t* d = dst + (R0 + r) * n_kb + K0 + kb;
+#pragma unroll
+  for (int p = 0; p < ROWS * KB / 256; ++p, d += 256 / KB * n_kb)
+    if (full_tile || (R0 + r + 256 / KB * p < Rn && K0 + kb < n_kb)) *d = src[threadIdx.x + 256 * p];
+}
+
 }  // namespace nvfp4

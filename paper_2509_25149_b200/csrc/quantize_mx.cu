@@ -288,18 +288,8 @@ __global__ void __launch_bounds__(256, 2) quantize_mx_kernel(const __grid_consta
           const int64_t off = ((R0 >> 7) * (n_kb >> 2) + (K0 >> 2)) * 512 + threadIdx.x * 16;
           *reinterpret_cast<uint4*>(dst + off) = *reinterpret_cast<const uint4*>(src + threadIdx.x * 16);
         }
-      } else if (threadIdx.x < 128) {
-        const int r = threadIdx.x;
-        if (R0 + r < Rn) {
-          uint8_t* d = dst + (R0 + r) * n_kb + K0;
-          if (K0 + 4 <= n_kb && (n_kb & 3) == 0) {
-            *reinterpret_cast<uint32_t*>(d) = *reinterpret_cast<const uint32_t*>(src + r * 4);
-          } else {
-#pragma unroll
-            for (int k = 0; k < 4; ++k)
-              if (K0 + k < n_kb) d[k] = src[r * 4 + k];
-          }
-        }
+      } else {
+        store_linear_scales<128, 4>(src, dst, R0, K0, Rn, n_kb, row0 + 128 <= a.rows && col0 + 128 <= a.cols);
       }
     }
   }
