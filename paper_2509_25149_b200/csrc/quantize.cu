@@ -628,9 +628,8 @@ __device__ __forceinline__ void quantize_tiles(const CUtensorMap* src_map, const
       // ---------------------------------------------------------------- phase 2 ----
       if constexpr (kNibbleTranspose) {
         // The transposed copy is the row-wise one with its nibbles transposed: a lane takes eight rows (half) of CL
-        // neighbouring columns and transposes 8 x 4 nibbles at a time: 16-bit halves, bytes, nibbles.  (Two columns per lane,
-        // read byte by byte, took 2.3 instructions per element and a shared-memory read for every second one: quantizing an
-        // 8192 x 5120 weight 39.8 us, now 37.7.)
+        // neighbouring columns.  (Two columns per lane, read byte by byte, took 2.3 instructions per element and a shared-memory
+        // read for every second one: quantizing an 8192 x 5120 weight 39.8 us, now 37.7.)
         constexpr int CL = TC / 16;
         const int q = warp, o = lane & 15, half = lane >> 4;
         const uint8_t* const src = smem + S::kRand + (q * 16 + half * 8) * (TC / 2) + o * (CL / 2);
@@ -640,19 +639,7 @@ __device__ __forceinline__ void quantize_tiles(const CUtensorMap* src_map, const
           w[k] = CL == 8 ? *reinterpret_cast<const uint32_t*>(src + k * (TC / 2))
                          : (uint32_t) * reinterpret_cast<const uint16_t*>(src + k * (TC / 2));
         uint32_t col[CL];
-#pragma unroll
-        for (int h = 0; h < CL / 4; ++h) {  // columns 4h .. 4h + 3
-          uint32_t p[4];                     // [row k | row k + 4]
-#pragma unroll
-          for (int k = 0; k < 4; ++k) p[k] = __byte_perm(w[k], w[k + 4], h ? 0x7632 : 0x5410);
-#pragma unroll
-          for (int b = 0; b < 2; ++b) {  // the pair of columns in bytes b and b + 2
-            const uint32_t even = __byte_perm(p[0], p[2], b ? 0x7351 : 0x6240);  // rows 0, 2, 4, 6
-            const uint32_t odd = __byte_perm(p[1], p[3], b ? 0x7351 : 0x6240);   // rows 1, 3, 5, 7
-            col[4 * h + 2 * b] = (even & 0x0F0F0F0Fu) | ((odd << 4) & 0xF0F0F0F0u);
-            col[4 * h + 2 * b + 1] = ((even >> 4) & 0x0F0F0F0Fu) | (odd & 0xF0F0F0F0u);
-          }
-        }
+        transpose_nibbles(w, col);
 #pragma unroll
         for (int k = 0; k < CL; ++k) {
           const int cp = CL / 2 * o + (k >> 1);

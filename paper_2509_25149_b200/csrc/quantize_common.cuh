@@ -217,4 +217,23 @@ __device__ __forceinline__ void store_linear_scales(const uint8_t* src, uint8_t*
     if (full_tile || (R0 + r + 256 / KB * p < Rn && K0 + kb < n_kb)) *d = src[threadIdx.x + 256 * p];
 }
 
+// Eight rows of CL nibbles (a word each, columns from the low end) -> CL columns of eight nibbles (rows from the low end): 16-bit
+// halves, then bytes, then nibbles.
+template <int CL>
+__device__ __forceinline__ void transpose_nibbles(const uint32_t (&w)[8], uint32_t (&col)[CL]) {
+#pragma unroll
+  for (int h = 0; h < CL / 4; ++h) {  // columns 4h .. 4h + 3
+    uint32_t p[4];                     // [row k | row k + 4]
+#pragma unroll
+    for (int k = 0; k < 4; ++k) p[k] = __byte_perm(w[k], w[k + 4], h ? 0x7632 : 0x5410);
+#pragma unroll
+    for (int b = 0; b < 2; ++b) {  // the pair of columns in bytes b and b + 2
+      const uint32_t even = __byte_perm(p[0], p[2], b ? 0x7351 : 0x6240);  // rows 0, 2, 4, 6
+      const uint32_t odd = __byte_perm(p[1], p[3], b ? 0x7351 : 0x6240);   // rows 1, 3, 5, 7
+      col[4 * h + 2 * b] = (even & 0x0F0F0F0Fu) | ((odd << 4) & 0xF0F0F0F0u);
+      col[4 * h + 2 * b + 1] = ((even >> 4) & 0x0F0F0F0Fu) | (odd & 0xF0F0F0F0u);
+    }
+  }
+}
+
 }  // namespace nvfp4

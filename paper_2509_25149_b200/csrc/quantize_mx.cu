@@ -109,6 +109,8 @@ __global__ void __launch_bounds__(256, 2) quantize_mx_kernel(const __grid_consta
   const int sf_col_odd = a.c_swz ? 16 : 4;
   const int64_t r_pitch = a.cols >> 1;
 
+  auto spread = [](int p) { return p ^ (p >> 2); };  // eight consecutive column pairs, and every fourth, in different units
+
   int j = 0;
   for (; j < n_mine; ++j) {
     const int tile = (int)blockIdx.x + j * stride, tr = tile / a.tiles_c, tc = tile - tr * a.tiles_c;
@@ -195,22 +197,18 @@ __global__ void __launch_bounds__(256, 2) quantize_mx_kernel(const __grid_consta
       uint4 out0, out1;  // 32 nibbles of column 2cp / 2cp + 1
       uint32_t byte0, byte1;
       if (kNibbleTranspose) {
+        // nibbles of the row-wise copy, 8 rows x 8 columns per thread, see transpose_nibbles()
         byte0 = byte1 = smem[S::kBlkByte + 2 * q32 * 4 + (cp >> 4)];
-        uint32_t lo[8], hi[8];
+        const int o = lane & 15, rg = cp >> 4;  // columns 8 o .., rows 8 rg .. of the group
+        const uint8_t* const src = smem + S::kRand + (q32 * 32 + rg * 8) * 64 + o * 4;
+        uint32_t w[8], col[8];
 #pragma unroll
-        for (int m = 0; m < 8; ++m) {
-          // byte [row][cp] of the staged row-wise codes = (column 2cp in the low nibble, 2cp + 1 in the high one)
-          uint32_t b[4];
+        for (int k = 0; k < 8; ++k) w[k] = *reinterpret_cast<const uint32_t*>(src + k * 64);
+        transpose_nibbles(w, col);
 #pragma unroll
-          for (int k = 0; k < 4; ++k) b[k] = smem[S::kRand + (q32 * 32 + 4 * m + k) * 64 + cp];
-          const uint32_t w = __byte_perm(__byte_perm(b[0], b[1], 0x0040), __byte_perm(b[2], b[3], 0x0040), 0x5410);
-          const uint32_t l = w & 0x0F0F0F0Fu, h = (w >> 4) & 0x0F0F0F0Fu;  // four nibbles, one per byte -> 16 bits
-          const uint32_t tl = (l | (l >> 4)) & 0x00FF00FFu, th = (h | (h >> 4)) & 0x00FF00FFu;
-          lo[m] = (tl | (tl >> 8)) & 0xFFFFu;
-          hi[m] = (th | (th >> 8)) & 0xFFFFu;
-        }
-        out0 = make_uint4(lo[0] | (lo[1] << 16), lo[2] | (lo[3] << 16), lo[4] | (lo[5] << 16), lo[6] | (lo[7] << 16));
-        out1 = make_uint4(hi[0] | (hi[1] << 16), hi[2] | (hi[3] << 16), hi[4] | (hi[5] << 16), hi[6] | (hi[7] << 16));
+        for (int k = 0; k < 8; ++k)
+          *reinterpret_cast<uint32_t*>(col_codes + (4 * o + (k >> 1)) * 128 +
+                                       ((((k & 1) * 4 + q32) ^ spread(4 * o + (k >> 1))) & 7) * 16 + rg * 4) = col[k];
       } else {
         float2 v[32];
         const uint8_t* tp = tile_buf + q32 * 32 * 256 + cp * 4;
@@ -252,9 +250,11 @@ __global__ void __launch_bounds__(256, 2) quantize_mx_kernel(const __grid_consta
           }
         }
       }
-      // staging: a column pair has 128 bytes, eight 16-byte units (column parity, 32-row group); unit u sits at u ^ cp
-      *reinterpret_cast<uint4*>(col_codes + cp * 128 + (((q32 ^ cp) & 7) << 4)) = out0;
-      *reinterpret_cast<uint4*>(col_codes + cp * 128 + ((((4 + q32) ^ cp) & 7) << 4)) = out1;
+      // staging: a column pair has 128 bytes, eight 16-byte units (column parity, 32-row group); unit u sits at u ^ spread(cp)
+      if (!kNibbleTranspose) {
+        *reinterpret_cast<uint4*>(col_codes + cp * 128 + (((q32 ^ spread(cp)) & 7) << 4)) = out0;
+        *reinterpret_cast<uint4*>(col_codes + cp * 128 + ((((4 + q32) ^ spread(cp)) & 7) << 4)) = out1;
+      }
       sf_col[sf_col_pos] = (uint8_t)byte0;
       sf_col[sf_col_pos + sf_col_odd] = (uint8_t)byte1;
     }
@@ -271,7 +271,7 @@ __global__ void __launch_bounds__(256, 2) quantize_mx_kernel(const __grid_consta
         const int c = unit >> 2, m = unit & 3;  // column, 32-row group
         if (col0 + c >= a.cols || row0 + 32 * m >= a.rows) continue;  // rows % 32 == 0: a group is inside or outside
         const uint4 val = *reinterpret_cast<const uint4*>(col_codes + (c >> 1) * 128 +
-                                                          (((((c & 1) * 4 + m) ^ (c >> 1)) & 7) << 4));
+                                                          (((((c & 1) * 4 + m) ^ spread(c >> 1)) & 7) << 4));
         *reinterpret_cast<uint4*>(a.c_codes + (col0 + c) * pitch + (row0 >> 1) + m * 16) = val;
       }
     }
