@@ -721,10 +721,9 @@ static bool make_bf16_maps(const DenseGemmArgs& g, CUtensorMap* m) {  // A, B, D
 
 static int bf16_tiles(const DenseGemmArgs& g, int bn) { return ((g.M + 255) / 256) * ((g.N + bn - 1) / bn); }
 
-// g1 == nullptr: one problem
-template <int BN, int SPLIT = 1>
-static cudaError_t launch_bf16_t(const DenseGemmArgs& g0, const DenseGemmArgs* g1, int max_pairs, cudaStream_t s) {
-  auto kern = dense::gemm_bf16_pair_kernel<BN, SPLIT>;
+template <int BN, int SPLIT, bool TWO>
+static cudaError_t launch_bf16_problems(const DenseGemmArgs& g0, const DenseGemmArgs* g1, int max_pairs, cudaStream_t s) {
+  auto kern = dense::gemm_bf16_pair_kernel<BN, SPLIT, TWO>;
   constexpr int smem = dense::Cfg<BN, SPLIT>::kSmemBytes;
   CUtensorMap m[6];
   if (!make_bf16_maps<BN, SPLIT>(g0, m)) return cudaErrorInvalidValue;
@@ -753,6 +752,13 @@ static cudaError_t launch_bf16_t(const DenseGemmArgs& g0, const DenseGemmArgs* g
                                       m[3], m[4], m[5], a);
   count_launch();
   return e;
+}
+
+// g1 == nullptr: one problem
+template <int BN, int SPLIT = 1>
+static cudaError_t launch_bf16_t(const DenseGemmArgs& g0, const DenseGemmArgs* g1, int max_pairs, cudaStream_t s) {
+  return g1 ? launch_bf16_problems<BN, SPLIT, true>(g0, g1, max_pairs, s)
+            : launch_bf16_problems<BN, SPLIT, false>(g0, nullptr, max_pairs, s);
 }
 
 cudaError_t launch_gemm_bf16(const DenseGemmArgs& g0, const DenseGemmArgs* g1, cudaStream_t s) {

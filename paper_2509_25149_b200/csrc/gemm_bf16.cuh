@@ -68,7 +68,8 @@ __device__ __forceinline__ void tc2_mma_bf16(uint32_t d_tmem, uint64_t adesc, ui
 
 // BN: columns of a tile (256 or 128).  SPLIT > 1 (BN = 128): a cluster of SPLIT pairs takes one tile, the only one of its life,
 // each pair a share of the k-blocks (the exchange: pair::exchange_columns).
-template <int BN, int SPLIT = 1>
+// TWO: the launch has two problems.
+template <int BN, int SPLIT = 1, bool TWO = true>
 __global__ void __cluster_dims__(2 * SPLIT, 1, 1) __launch_bounds__(kThreads, 1)
     gemm_bf16_pair_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant__ CUtensorMap map_b0,
                           const __grid_constant__ CUtensorMap map_d0, const __grid_constant__ CUtensorMap map_a1,
@@ -102,13 +103,13 @@ __global__ void __cluster_dims__(2 * SPLIT, 1, 1) __launch_bounds__(kThreads, 1)
   // ragged edges: loads beyond the operands read zeros, stores beyond D are clipped (both by the tensor maps)
   const int n_tiles = g.n_tiles;
   auto k_begin = [&](int tile, int s) {  // first k-block of share s
-    const int n = (g.p[tile >= g.n_tiles0 ? 1 : 0].K + 63) / 64;
+    const int n = (g.p[TWO && tile >= g.n_tiles0 ? 1 : 0].K + 63) / 64;
     return SPLIT > 1 ? n * s / SPLIT : n * s;
   };
   // groups of eight row-blocks sweep all column-blocks before the next group starts (L2 reuse of A and B)
   constexpr int kGroupM = 8;
   auto tile_coords = [&](int tile, int& prob, int& m_blk, int& n_blk) {
-    prob = tile >= g.n_tiles0 ? 1 : 0;
+    prob = TWO && tile >= g.n_tiles0 ? 1 : 0;
     if (prob) tile -= g.n_tiles0;
     const int tiles_m = (g.p[prob].M + 255) / 256, tiles_n = (g.p[prob].N + BN - 1) / BN;
     const int per_group = kGroupM * tiles_n;
@@ -158,33 +159,40 @@ __global__ void __cluster_dims__(2 * SPLIT, 1, 1) __launch_bounds__(kThreads, 1)
       for (int tile = pair_id; tile < n_tiles && ok; tile += n_pairs) {
         int prob, m_blk, n_blk;
         tile_coords(tile, prob, m_blk, n_blk);
-        const CUtensorMap* map_a = prob ? &map_a1 : &map_a0;
-        const CUtensorMap* map_b = prob ? &map_b1 : &map_b0;
-        const int a_mn = g.p[prob].a_mn, b_mn = g.p[prob].b_mn, k_end = k_begin(tile, split + 1);
         const int row_a = m_blk * 256 + (int)rank * 128;  // this CTA's rows of A
         const int row_b = n_blk * BN + (int)rank * (BN / 2);  // this CTA's half of the B tile
-        for (int kb = k_begin(tile, split); kb < k_end; ++kb) {
-          if (!(ok = mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag, 0x900u + stage))) break;
-          const uint32_t st = base + stage * kStageBytes;
-          const uint32_t bar = map_to_cta(full_bar(stage), leader_cta);  // the leader's barrier counts both CTAs' operands
-          mbar_expect_tx_cluster(bar, dense::kOperandBytes + BN / 2 * 128);
-          if (a_mn) {
-            tma_load_2d_pair(st, map_a, row_a, kb * 64, bar);
-            tma_load_2d_pair(st + 8192, map_a, row_a + 64, kb * 64, bar);
-          } else {
-            tma_load_2d_pair(st, map_a, kb * 64, row_a, bar);
+        const int k_end = k_begin(tile, split + 1);
+        // One copy of the loop for each problem of the launch, with its tensor maps and layouts at fixed places of the parameter
+        // bank: with the maps picked by pointer the loads of a stage were issued so late that a pair could not go faster even
+        // when it had L2 to itself (last rounds): forward of 3632 x 1552 x 3136 41.0 us, now 35.4, backward 67.6, now 63.4.
+        auto load_tile = [&](const CUtensorMap* map_a, const CUtensorMap* map_b, const Problem& pr) {
+          for (int kb = k_begin(tile, split); kb < k_end; ++kb) {
+            if (!(ok = mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag, 0x900u + stage))) break;
+            const uint32_t st = base + stage * kStageBytes;
+            const uint32_t bar = map_to_cta(full_bar(stage), leader_cta);  // the leader's barrier counts both CTAs' operands
+            mbar_expect_tx_cluster(bar, dense::kOperandBytes + BN / 2 * 128);
+            if (pr.a_mn) {
+              tma_load_2d_pair(st, map_a, row_a, kb * 64, bar);
+              tma_load_2d_pair(st + 8192, map_a, row_a + 64, kb * 64, bar);
+            } else {
+              tma_load_2d_pair(st, map_a, kb * 64, row_a, bar);
+            }
+            if (pr.b_mn) {
+              tma_load_2d_pair(st + dense::kOperandBytes, map_b, row_b, kb * 64, bar);
+              if (BN == 256) tma_load_2d_pair(st + dense::kOperandBytes + 8192, map_b, row_b + 64, kb * 64, bar);
+            } else {
+              tma_load_2d_pair(st + dense::kOperandBytes, map_b, kb * 64, row_b, bar);
+            }
+            if (++stage == S) {
+              stage = 0;
+              phase ^= 1u;
+            }
           }
-          if (b_mn) {
-            tma_load_2d_pair(st + dense::kOperandBytes, map_b, row_b, kb * 64, bar);
-            if (BN == 256) tma_load_2d_pair(st + dense::kOperandBytes + 8192, map_b, row_b + 64, kb * 64, bar);
-          } else {
-            tma_load_2d_pair(st + dense::kOperandBytes, map_b, kb * 64, row_b, bar);
-          }
-          if (++stage == S) {
-            stage = 0;
-            phase ^= 1u;
-          }
-        }
+        };
+        if (!TWO || prob == 0)
+          load_tile(&map_a0, &map_b0, g.p[0]);
+        else
+          load_tile(&map_a1, &map_b1, g.p[1]);
       }
     }
   } else if (warp == 1) {
@@ -203,28 +211,34 @@ __global__ void __cluster_dims__(2 * SPLIT, 1, 1) __launch_bounds__(kThreads, 1)
         if (!(ok = mbar_wait_cluster(acce_bar(buf), ((acc_phase >> buf) & 1u) ^ 1u, abort_flag, 0xB00u + buf))) break;
         tc_fence_after();
         const uint32_t d_t = tmem + buf * 256;
-        const Problem& pr = g.p[tile >= g.n_tiles0 ? 1 : 0];
-        const uint32_t idesc = instr_desc_bf16(256, BN, pr.a_mn, pr.b_mn);
-        const uint32_t a_lo0 = a_lo_base | ((pr.a_mn ? (8192u >> 4) : 1u) << 16);
-        const uint32_t b_lo0 = b_lo_base | ((pr.b_mn ? (8192u >> 4) : 1u) << 16);
-        const uint32_t a_step = pr.a_mn ? (2048u >> 4) : (32u >> 4);  // one K = 16 instruction further
-        const uint32_t b_step = pr.b_mn ? (2048u >> 4) : (32u >> 4);
         const int k_blocks = k_begin(tile, split + 1) - k_begin(tile, split);
-        for (int kb = 0; kb < k_blocks; ++kb) {
-          if (!(ok = mbar_wait_cluster(full_bar(stage), phase, abort_flag, 0xA00u + stage))) break;
-          tc_fence_after();
-          const uint32_t a_lo = a_lo0 + stage * (kStageBytes >> 4);
-          const uint32_t b_lo = b_lo0 + stage * (kStageBytes >> 4);
+        // (one copy of the loop for each problem, as in the producer)
+        auto main_loop = [&](const Problem& pr) {
+          const uint32_t idesc = instr_desc_bf16(256, BN, pr.a_mn, pr.b_mn);
+          const uint32_t a_lo0 = a_lo_base | ((pr.a_mn ? (8192u >> 4) : 1u) << 16);
+          const uint32_t b_lo0 = b_lo_base | ((pr.b_mn ? (8192u >> 4) : 1u) << 16);
+          const uint32_t a_step = pr.a_mn ? (2048u >> 4) : (32u >> 4);  // one K = 16 instruction further
+          const uint32_t b_step = pr.b_mn ? (2048u >> 4) : (32u >> 4);
+          for (int kb = 0; kb < k_blocks; ++kb) {
+            if (!(ok = mbar_wait_cluster(full_bar(stage), phase, abort_flag, 0xA00u + stage))) break;
+            tc_fence_after();
+            const uint32_t a_lo = a_lo0 + stage * (kStageBytes >> 4);
+            const uint32_t b_lo = b_lo0 + stage * (kStageBytes >> 4);
 #pragma unroll
-          for (int j = 0; j < 4; ++j)
-            tc2_mma_bf16(d_t, make_desc(a_lo + j * a_step, kDescHiOperand), make_desc(b_lo + j * b_step, kDescHiOperand),
-                         idesc, (kb > 0 || j > 0) ? 1u : 0u);
-          tc2_commit_both(empty_bar(stage), pair_mask);  // both CTAs' stages are free once these MMAs have read them
-          if (++stage == S) {
-            stage = 0;
-            phase ^= 1u;
+            for (int j = 0; j < 4; ++j)
+              tc2_mma_bf16(d_t, make_desc(a_lo + j * a_step, kDescHiOperand), make_desc(b_lo + j * b_step, kDescHiOperand),
+                           idesc, (kb > 0 || j > 0) ? 1u : 0u);
+            tc2_commit_both(empty_bar(stage), pair_mask);  // both CTAs' stages are free once these MMAs have read them
+            if (++stage == S) {
+              stage = 0;
+              phase ^= 1u;
+            }
           }
-        }
+        };
+        if (!TWO || tile < g.n_tiles0)
+          main_loop(g.p[0]);
+        else
+          main_loop(g.p[1]);
         if (!ok) break;
         tc2_commit_both(accf_bar(buf), pair_mask);  // this accumulator is complete in both CTAs
         acc_phase ^= 1u << buf;
