@@ -60,7 +60,8 @@ enum { NVFP4_SF_LINEAR = 0, NVFP4_SF_SWIZZLED = 1 };
 enum { NVFP4_FORMAT_NVFP4 = 0, NVFP4_FORMAT_MXFP4 = 1, NVFP4_FORMAT_NVFP4_ROWSCALE = 2 };
 enum {
   /* the column-wise copy draws its stochastic-rounding bits from a second stream (bit 63 of
-     sr_offset set) instead of sharing the draw of the same source element with the row-wise copy */
+     sr_offset set) instead of sharing the draw of the same source element with the row-wise copy.  Where both copies of
+     square blocks are requested of a bf16 source in NVFP4 it has no effect: they hold the same values */
   NVFP4_SR_INDEPENDENT_COPIES = 1,
   /* global[0] of each requested copy already holds the tensor amax: skip the reduction pass */
   NVFP4_AMAX_PROVIDED = 2,
@@ -136,7 +137,8 @@ typedef struct nvfp4_quant_opts {
  *             Section 4.3: the backward pass contracts over the other dimension):
  *             colwise->rows == cols, colwise->cols == rows.
  *   At least one copy must be requested.  With block_rows == 16 both copies hold the same
- *   quantized values (transposed) and no Hadamard transform is allowed.
+ *   quantized values (transposed; a binary32 source rounded stochastically with NVFP4_SR_INDEPENDENT_COPIES, and 32x32
+ *   MXFP4 blocks likewise, excepted) and no Hadamard transform is allowed.
  *   rowwise->format == NVFP4_FORMAT_NVFP4_ROWSCALE: one pass, colwise must be NULL, block_rows 1, no transform,
  *   bf16 source; rowwise->global receives 2 * rows floats.
  * Two passes over x: a tensor-amax reduction (in the rotated space for a transformed copy),

@@ -1158,6 +1158,10 @@ cudaError_t launch_amax_f32(const QuantArgs& a, bool has_row, bool has_col, cuda
 // binary32 source (Appendix B names FP32 as well as BF16 as the precision converted from), e.g. weights quantized straight from
 // their FP32 master copy; no transform (the recipe transforms activations and gradients, which are bf16)
 cudaError_t launch_quantize_f32(const QuantArgs& a, bool has_row, bool has_col, bool block2d, bool sr, cudaStream_t s) {
+  if (block2d && sr && has_row && has_col && a.off_hi_col != a.off_hi) {  // independent draws: the copies' codes differ
+    const cudaError_t e = launch_quantize_f32(a, true, false, true, true, s);
+    return e != cudaSuccess ? e : launch_quantize_f32(a, false, true, true, true, s);
+  }
   int sms = 0;
   const cudaError_t e = sm_count(&sms);
   if (e != cudaSuccess) return e;

@@ -67,7 +67,8 @@ __global__ void __launch_bounds__(256, 2) quantize_mx_kernel(const __grid_consta
   extern __shared__ __align__(128) uint8_t smem[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t n_cb = a.cols >> 4;  // 16-chunks per source row (index of the random draws)
-  // 32x32 blocks with both copies requested: the transposed copy holds the very codes of the row-wise one
+  // 32x32 blocks with both copies requested: the transposed copy holds the very codes of the row-wise one (with draws of its
+  // own it is made by a launch of its own, see launch_quantize_mx)
   constexpr bool kNibbleTranspose = BLOCK2D && HAS_ROW && HAS_COL;
   constexpr bool kStageRand = SR && HAS_COL && !kNibbleTranspose;
   volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(smem + S::kBars + 16);
@@ -330,6 +331,10 @@ static cudaError_t launch_mx_t(const QuantArgs& a, cudaStream_t s) {
 cudaError_t launch_quantize_mx(const QuantArgs& a, bool has_row, bool has_col, bool block2d, bool rht_col, bool sr,
                                cudaStream_t s) {
   rht_col = rht_col && has_col;
+  if (block2d && sr && has_row && has_col && a.off_hi_col != a.off_hi) {  // independent draws: the copies' codes differ
+    const cudaError_t e = launch_quantize_mx(a, true, false, true, false, true, s);
+    return e != cudaSuccess ? e : launch_quantize_mx(a, false, true, true, false, true, s);
+  }
 #define NVFP4_MXQ(HR, HC, B2, RC, SRV)                                                        \
   if (has_row == HR && has_col == HC && block2d == B2 && rht_col == RC && sr == SRV)         \
     return launch_mx_t<HR, HC, B2, RC, SRV>(a, s);

@@ -74,6 +74,30 @@ def test_sr_16x16_and_seed_zero():
     P.assert_exact(col, oracle.quantize(synth.bits(w), block_rows=16, rounding=oracle.SR, colwise=True), "2D SR col")
 
 
+@pytest.mark.parametrize("shape", [(32, 32), (256, 384), (160, 224)])
+@pytest.mark.parametrize("fmt", ["mxfp4", "binary32", "binary32, amax provided"])
+def test_square_blocks_with_draws_of_their_own(shape, fmt):
+    """Both copies of a weight in one call, the transposed one rounded with the second stream."""
+    w = rand_bf16(shape, 5, std=0.02)
+    layout = B.SF_SWIZZLED if shape[0] % 128 == 0 and shape[1] % 128 == 0 else B.SF_LINEAR
+    opt = dict(rounding=B.ROUND_STOCHASTIC, seed=11, sr_offset=6, flags=B.SR_INDEPENDENT_COPIES)
+    sr = dict(rounding=oracle.SR, seed=11)
+    if fmt == "mxfp4":
+        row, col = P.gpu_quantize_mx(w, colwise=True, sf_layout=layout, block_rows=32, **opt)
+        P.assert_exact_mx(row, oracle.quantize_mx(synth.bits(w), block_rows=32, sr_offset=6, **sr), "row")
+        P.assert_exact_mx(col, oracle.quantize_mx(synth.bits(w), block_rows=32, colwise=True, sr_offset=6 | (1 << 63), **sr),
+                          "col")
+        return
+    w = w.float()
+    row, col = (B.alloc_tensor(*s, layout) for s in (shape, shape[::-1]))
+    if "provided" in fmt:
+        opt["flags"] |= B.AMAX_PROVIDED
+        row.glob[0] = col.glob[0] = float(w.abs().max())
+    B.nvfp4_quantize(w.cuda(), B.quant_opts(block_rows=16, **opt), row, col)
+    P.assert_exact(row, oracle.quantize(w.numpy(), block_rows=16, sr_offset=6, **sr), "row")
+    P.assert_exact(col, oracle.quantize(w.numpy(), block_rows=16, colwise=True, sr_offset=6 | (1 << 63), **sr), "col")
+
+
 @pytest.mark.parametrize("shape", [(128, 128), (256, 384), (144, 208)])
 @pytest.mark.parametrize("rounding", [B.ROUND_NEAREST_EVEN, B.ROUND_STOCHASTIC])
 def test_rht_copies_follow_the_tolerance_protocol(shape, rounding):
