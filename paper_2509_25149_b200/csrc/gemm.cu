@@ -438,10 +438,12 @@ cudaError_t launch_pair_t(const GemmArgs& g0, const void* a0, const void* b0, co
   a.n_tiles0 = pair_tiles(g0, BN);
   a.n_tiles = a.n_tiles0 + (g1 ? pair_tiles(*g1, BN) : 0);
   int max_pairs = num_sms / 2;
-  const int cap = g_exp_max_pairs.load(std::memory_order_relaxed);  // measurement aids, 0 / NULL normally
-  if (cap > 0 && cap < max_pairs) max_pairs = cap;
-  a.exp = g_exp_mode.load(std::memory_order_relaxed);
-  a.probe = g_exp_probe.load(std::memory_order_relaxed);
+  if (BN == 256) {  // measurement aids (0 / NULL normally) of the kernel with 256 x 256 tiles; no other launch may see them
+    const int cap = g_exp_max_pairs.load(std::memory_order_relaxed);
+    if (cap > 0 && cap < max_pairs) max_pairs = cap;
+    a.exp = g_exp_mode.load(std::memory_order_relaxed);
+    a.probe = g_exp_probe.load(std::memory_order_relaxed);
+  }
   const int pairs = a.n_tiles < max_pairs || SPLIT > 1 ? a.n_tiles : max_pairs;  // SPLIT > 1: a cluster for each tile
   const cudaError_t e =
       launch_kernel(kern, dim3(2 * SPLIT * pairs), dim3(pair::kThreads), smem, s, m[0], m[1], m[2], m[3], m[4], m[5], a);

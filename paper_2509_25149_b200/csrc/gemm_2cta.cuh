@@ -69,7 +69,7 @@ struct Args {
   Problem p[2];
   int n_tiles0;  // tiles of problem 0
   int n_tiles;   // tiles of both problems
-  // Measurement aids (0 / NULL in normal operation).  exp: bit 0 = the issuer skips the MMAs, bit 1 = the producer
+  // Measurement aids of the kernel with 256 x 256 tiles (0 / NULL in normal operation and for the others).  exp: bit 0 = the issuer skips the MMAs, bit 1 = the producer
   // skips the operand loads, bit 2 = scale atoms are neither loaded nor copied to tensor memory, bit 3 = the epilogue hands the
   // accumulator back unread and stores nothing, bit 4 = the issuer does not wait for the accumulator (results are
   // meaningless with any bit set; the barriers are signalled as usual).  probe: per pair eight 64-bit words, five

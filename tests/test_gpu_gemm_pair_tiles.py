@@ -128,3 +128,23 @@ def test_scale_vectors_on_every_pair_tile(shape, tile, rows_on, fp32):
         B.nvfp4_set_gemm_tile_n(0)
     P.assert_gemm_close(D.float().cpu().numpy(), (a @ b.T).cpu().numpy(), (a.abs() @ b.abs().T).cpu().numpy(), not fp32,
                         f"rows {rows_on} tile {tile}")
+
+
+@pytest.mark.parametrize("tile", [640, 642, 644, 768, 128])
+def test_measurement_aids_leave_the_other_tiles_alone(tile):
+    """No MMAs, no output, a capped grid and a probe are asked for: only the kernel with 256 x 256 tiles heeds them."""
+    A, Bt = B.alloc_tensor(256, 1024), B.alloc_tensor(512, 1024)
+    for t, seed in ((A, 1), (Bt, 2)):
+        B.nvfp4_quantize(synth.normal_bf16((t.rows, t.cols), 1.0, seed).cuda(), B.quant_opts(), t, None)
+    D, want = (torch.zeros((256, 512), device="cuda") for _ in range(2))
+    probe = torch.zeros(8 * 74, dtype=torch.int64, device="cuda")
+    B.nvfp4_set_gemm_tile_n(tile)
+    try:
+        B.nvfp4_gemm(A, Bt, want)
+        B.nvfp4_set_gemm_experiment(1 | 8, 1, probe)
+        B.nvfp4_gemm(A, Bt, D)
+        B.nvfp4_device_status()
+    finally:
+        B.nvfp4_set_gemm_experiment()
+        B.nvfp4_set_gemm_tile_n(0)
+    assert torch.equal(D, want) and not probe.any()
