@@ -322,6 +322,14 @@ NVFP4_API nvfp4_status nvfp4_device_status(void* cuda_stream, uint32_t* detail);
  */
 NVFP4_API nvfp4_status nvfp4_test_wait_timeout(uint64_t limit_ns, void* cuda_stream);
 
+/*
+ * Test aid for the same path: enqueues a cluster of eight blocks of which the first has given up when it reaches the exit of
+ * the GEMM kernels, and block k gets there after k / 7 of `delay_ns` (1 .. 100 000 000).  `times` (DEVICE, 24 words) receives
+ * when each block got there and when it was let go (nanoseconds, two words per block), then each block's abort word
+ * (0x7E570002: it heard of it).  No block may go before the last has arrived.  The status word is left alone.
+ */
+NVFP4_API nvfp4_status nvfp4_test_cluster_leave(uint64_t delay_ns, uint64_t* times, void* cuda_stream);
+
 /* Tuning knob: which GEMM tiling to use.  128 / 256 = one CTA per 128 x 128 / 128 x 256 output tile (256 needs
  * N % 256 == 0, otherwise 128 is used); CTA pairs: 640 = 256 x 128 tiles, 512 = 256 x 256 tiles, 768 = 256 x 384 tiles plus
  * up to two 256-wide ones per row of tiles (needs N >= 256, otherwise as 512); 642 / 644 = 256 x 128 tiles whose

@@ -562,6 +562,15 @@ nvfp4_status nvfp4_test_wait_timeout(uint64_t limit_ns, void* cuda_stream) {
   return launch_wait_probe(limit_ns, static_cast<cudaStream_t>(cuda_stream)) == cudaSuccess ? NVFP4_OK : NVFP4_ERR_CUDA;
 }
 
+nvfp4_status nvfp4_test_cluster_leave(uint64_t delay_ns, uint64_t* times, void* cuda_stream) {
+  if (!times) return NVFP4_ERR_NULL;
+  if (delay_ns == 0 || delay_ns > 100000000ull) return NVFP4_ERR_ARG;  // at most 0.1 s
+  return launch_leave_probe(delay_ns, reinterpret_cast<unsigned long long*>(times), static_cast<cudaStream_t>(cuda_stream)) ==
+                 cudaSuccess
+             ? NVFP4_OK
+             : NVFP4_ERR_CUDA;
+}
+
 int32_t nvfp4_set_gemm_experiment(int32_t mode, int32_t max_pairs, void* probe) {
   if (mode < 0 || mode > 255 || max_pairs < 0) return -1;
   set_gemm_experiment(mode, max_pairs, static_cast<unsigned long long*>(probe));

@@ -811,6 +811,37 @@ cudaError_t launch_wait_probe(unsigned long long limit_ns, cudaStream_t s) {
   return cudaGetLastError();
 }
 
+// Test aid: a cluster of eight whose first CTA has given up while the others arrive at the exit after k / 7 of the delay.
+// times[2 k], [2 k + 1]: when CTA k got to the exit and when it was let go; times[16 + k]: its abort word then.
+__global__ void __cluster_dims__(8, 1, 1) leave_probe_kernel(unsigned long long delay_ns, unsigned long long* times) {
+  __shared__ __align__(8) unsigned long long bar;
+  __shared__ uint32_t abort_flag;
+  const uint32_t cta = pair::cluster_ctarank();
+  if (threadIdx.x == 0) {
+    mbar_init(smem_u32(&bar), 7);
+    abort_flag = cta == 0 ? kLeaveProbeCode : 0u;
+    fence_mbarrier_init();
+  }
+  __syncthreads();
+  pair::cluster_sync_all();
+  if (threadIdx.x == 0) {
+    const unsigned long long t0 = globaltimer_ns();
+    while (globaltimer_ns() - t0 < delay_ns / 7 * cta) __nanosleep(1000);
+    times[2 * cta] = globaltimer_ns();
+  }
+  pair::leave_cluster<8>(smem_u32(&bar), cta, &abort_flag, 0x610u);
+  if (threadIdx.x == 0) {
+    times[2 * cta + 1] = globaltimer_ns();
+    times[16 + cta] = abort_flag;
+  }
+}
+
+cudaError_t launch_leave_probe(unsigned long long delay_ns, unsigned long long* times, cudaStream_t s) {
+  leave_probe_kernel<<<8, 32, 0, s>>>(delay_ns, times);
+  count_launch();
+  return cudaGetLastError();
+}
+
 void set_gemm_experiment(int mode, int max_pairs, unsigned long long* probe) {
   g_exp_mode.store(mode, std::memory_order_relaxed);
   g_exp_max_pairs.store(max_pairs, std::memory_order_relaxed);

@@ -44,6 +44,9 @@ cudaError_t read_device_status(cudaStream_t s, uint32_t* code);
 // status word and returns by itself
 constexpr uint32_t kWaitProbeCode = 0x7E570001u;
 cudaError_t launch_wait_probe(unsigned long long limit_ns, cudaStream_t s);
+// test aid: how a cluster in which one CTA has given up is left (times: device array of 24 words)
+constexpr uint32_t kLeaveProbeCode = 0x7E570002u;
+cudaError_t launch_leave_probe(unsigned long long delay_ns, unsigned long long* times, cudaStream_t s);
 // device address of the status word on the current device (for kernels of other translation units)
 cudaError_t device_status_word(unsigned int** word);
 

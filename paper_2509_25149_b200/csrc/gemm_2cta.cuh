@@ -132,6 +132,41 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity,
   }
 }
 
+// Leaving a cluster of CTAS CTAs (every thread calls it).  None may go while another can still signal its barriers, read its shared
+// memory or write into it: each tells the others that it is done and waits for their word.  One that gave up (a wait of
+// kWaitLimitNs expired) sets its peers' abort words first, so that those who still wait for it stop at once.  The wait for the
+// others has a limit of its own and does not look at the abort word: with the word set it used to end after 64 tries,
+// with peers that had up to two seconds of their own waits left.
+constexpr unsigned long long kLeaveLimitNs = 2 * kWaitLimitNs;
+template <int CTAS>
+__device__ __forceinline__ void leave_cluster(uint32_t done_bar, uint32_t cta, volatile uint32_t* abort_flag, uint32_t code) {
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    const uint32_t gave_up = *abort_flag, flag = smem_u32(const_cast<const uint32_t*>(abort_flag));
+    for (uint32_t k = 1; k < CTAS; ++k) {
+      if (gave_up)
+        asm volatile("st.relaxed.cluster.shared::cluster.u32 [%0], %1;" ::"r"(map_to_cta(flag, cta ^ k)), "r"(gave_up)
+                     : "memory");
+      mbar_arrive_cluster(map_to_cta(done_bar, cta ^ k));
+    }
+    if (!mbar_try_cluster(done_bar, 0)) {
+      const unsigned long long t0 = globaltimer_ns();
+      while (!mbar_try_cluster(done_bar, 0)) {
+        if (globaltimer_ns() - t0 > kLeaveLimitNs) {
+          *abort_flag = code;
+          atomicCAS(&g_device_status, 0u, code);
+          break;
+        }
+      }
+    }
+  }
+  __syncthreads();
+  if (*abort_flag) {
+    // give copies that may still be in flight time to land before the shared memory is handed back
+    for (int i = 0; i < 100; ++i) __nanosleep(1000);
+  }
+}
+
 // pair-aware TMA load: the data lands in this CTA's shared memory, the bytes are counted on `bar`, which may be
 // the peer's barrier (cluster address)
 __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap* map, int x, int y, uint32_t bar) {
@@ -739,18 +774,8 @@ __global__ void __cluster_dims__(2 * SPLIT, 1, 1) __launch_bounds__(kThreads, 1)
   }
 
   // ------------------------------------------------------------------ teardown ----
-  // Neither CTA may leave while the other can still signal its barriers or read its shared memory: each tells
-  // the peer it is done and waits (bounded) for the peer's word.
   tc_fence_before();
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    for (uint32_t k = 1; k < 2 * SPLIT; ++k) mbar_arrive_cluster(map_to_cta(done_bar, cta ^ k));
-    mbar_wait_cluster(done_bar, 0, abort_flag, 0x600u);
-  }
-  __syncthreads();
-  if (*abort_flag) {
-    for (int i = 0; i < 100; ++i) __nanosleep(1000);
-  }
+  leave_cluster<2 * SPLIT>(done_bar, cta, abort_flag, 0x600u);
   if (warp == 1) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");

@@ -445,17 +445,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kWThreads, 1)
   }
 
   // ------------------------------------------------------------------ teardown ----
-  // Neither CTA may leave while the other can still signal its barriers or read its shared memory.
   tc_fence_before();
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    mbar_arrive_cluster(map_to_cta(done_bar, rank ^ 1u));
-    mbar_wait_cluster(done_bar, 0, abort_flag, 0x600u);
-  }
-  __syncthreads();
-  if (*abort_flag) {
-    for (int i = 0; i < 100; ++i) __nanosleep(1000);
-  }
+  leave_cluster<2>(done_bar, rank, abort_flag, 0x600u);
   if (warp == 1) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kWTmemCols) : "memory");

@@ -44,3 +44,19 @@ def test_expired_wait_is_reported_and_the_device_stays_usable():
     B.nvfp4_device_status()
     Dref, T = P.gemm_reference(oracle.quantize(synth.bits(a)), oracle.quantize(synth.bits(b), block_rows=16))
     P.assert_gemm_close(D.float().cpu().numpy(), Dref, T, True, "GEMM after an expired wait")
+
+
+def test_nobody_leaves_a_cluster_before_the_last_has_arrived():
+    """Also when one block has given up: the others hear of it, and its shared memory stays until they are through."""
+    times = torch.zeros(24, dtype=torch.int64, device="cuda")
+    B.nvfp4_test_cluster_leave(21_000_000, times)  # blocks arrive every 3 ms
+    B.nvfp4_device_status()
+    arrived, left = times[:16].view(8, 2).T.tolist()
+    assert max(arrived) - min(arrived) >= 20_000_000
+    assert min(left) >= max(arrived) - 10_000  # (10 us: the clock's step)
+    assert max(left) - max(arrived) < 50_000_000
+    assert times[16:].tolist() == [0x7E570002] * 8
+    for delay in (0, 10 ** 9):
+        with pytest.raises(B.NVFP4Error) as e:
+            B.nvfp4_test_cluster_leave(delay, times)
+        assert e.value.status == ERR_ARG
