@@ -391,6 +391,8 @@ __global__ void __cluster_dims__(2 * SPLIT, 1, 1) __launch_bounds__(kThreads, 1)
   using C = Cfg<BN, SPLIT>;
   constexpr int kStages = C::kStages, kStageBytes = C::kStageBytes, kBBytes = C::kBBytes, kGroups = C::kGroups;
   constexpr int kSfCol = C::kSfCol, kSfSlotCols = C::kSfSlotCols;
+  auto exp = [&] { return BN == 256 ? g.exp : 0; };  // the measurement aids are this kernel's alone
+  auto probe = [&] { return BN == 256 ? g.probe : nullptr; };
   extern __shared__ uint8_t smem_raw[];
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t* base_ptr = smem_raw + (base - smem_u32(smem_raw));
@@ -504,7 +506,7 @@ __global__ void __cluster_dims__(2 * SPLIT, 1, 1) __launch_bounds__(kThreads, 1)
           if (!(ok = mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag, 0x100u + stage))) break;
           const uint32_t st = base + stage * kStageBytes;
           const uint32_t bar = map_to_cta(full_bar(stage), leader_cta);  // the leader's barrier counts both CTAs' operands
-          if (g.exp & 2) {
+          if (exp() & 2) {
             mbar_expect_tx_cluster(bar, 0);  // measurement aid: no operand loads
           } else {
             mbar_expect_tx_cluster(bar, kABytes + kBBytes);
@@ -512,7 +514,7 @@ __global__ void __cluster_dims__(2 * SPLIT, 1, 1) __launch_bounds__(kThreads, 1)
             tma_load_2d_pair(st + kABytes, map_b, kb * 128, row_b, bar);
           }
           // scale atoms: plain bulk copies counted on this CTA's own barrier (its scale warps wait on it)
-          if (g.exp & 4) {
+          if (exp() & 4) {
             mbar_expect_tx(sfl_bar(stage), 0);  // measurement aid: no scale loads
           } else {
             mbar_expect_tx(sfl_bar(stage), (1 + kGroups) * kAtomsKb * 512);
@@ -548,7 +550,7 @@ __global__ void __cluster_dims__(2 * SPLIT, 1, 1) __launch_bounds__(kThreads, 1)
         ok = mbar_wait(sfl_bar(stage), phase, abort_flag, 0x500u + stage);
         ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
         if (!ok) break;
-        if (g.exp & (4 | 32)) {  // measurement aids: no scale copies / the issuer copies, this warp only relays
+        if (exp() & (4 | 32)) {  // measurement aids: no scale copies / the issuer copies, this warp only relays
           __syncwarp();
           if (lane == 0) mbar_arrive_cluster(sff_leader + 8u * stage);
           if (++stage == kStages) {
@@ -607,14 +609,14 @@ __global__ void __cluster_dims__(2 * SPLIT, 1, 1) __launch_bounds__(kThreads, 1)
       constexpr uint32_t idesc_mx[2] = {instr_desc_mxf4(256, BN, 0), instr_desc_mxf4(256, BN, 2)};
       const uint32_t a_lo0 = ((base >> 4) & 0x3fffu) | (1u << 16);
       const uint32_t b_lo0 = (((base + kABytes) >> 4) & 0x3fffu) | (1u << 16);
-      const long long probe_c0 = g.probe ? clock64() : 0;
-      const unsigned long long probe_t0 = g.probe ? globaltimer_ns() : 0;
+      const long long probe_c0 = probe() ? clock64() : 0;
+      const unsigned long long probe_t0 = probe() ? globaltimer_ns() : 0;
       unsigned long long probe_kb = 0, probe_tiles = 0;
       long long probe_wait = 0, probe_mark = probe_c0;  // cycles spent waiting for the accumulator to be handed back
       for (int rnd = 0, tile = pair_id; tile < n_tiles && ok; tile = next_tile(++rnd)) {
-        if (!(g.exp & 16) && !(ok = mbar_wait_cluster(acce_bar(acc), ((acc_phase >> acc) & 1u) ^ 1u, abort_flag, 0x300u)))
+        if (!(exp() & 16) && !(ok = mbar_wait_cluster(acce_bar(acc), ((acc_phase >> acc) & 1u) ^ 1u, abort_flag, 0x300u)))
           break;
-        if (g.probe) probe_wait += clock64() - probe_mark;
+        if (probe()) probe_wait += clock64() - probe_mark;
         tc_fence_after();
         const uint32_t d_tmem = tmem + acc * BN;
         const int k_blocks = k_blocks_of(tile);
@@ -625,7 +627,7 @@ __global__ void __cluster_dims__(2 * SPLIT, 1, 1) __launch_bounds__(kThreads, 1)
           const uint32_t a_lo = a_lo0 + stage * (kStageBytes >> 4);
           const uint32_t b_lo = b_lo0 + stage * (kStageBytes >> 4);
           const uint32_t sf_t = tmem + kSfCol + stage * kSfSlotCols;
-          if (g.exp & 32) {  // measurement aid: the scale atoms go through the copy engine, issued here
+          if (exp() & 32) {  // measurement aid: the scale atoms go through the copy engine, issued here
             const uint32_t sf_lo = (((base + kABytes + kBBytes) >> 4) & 0x3fffu) + stage * (kStageBytes >> 4);
             constexpr int kAtomsKb = MX ? 2 : 4;
 #pragma unroll
@@ -638,7 +640,7 @@ __global__ void __cluster_dims__(2 * SPLIT, 1, 1) __launch_bounds__(kThreads, 1)
           }
 #pragma unroll
           for (int j = 0; j < 4; ++j) {
-            if (g.exp & 1) break;  // measurement aid: no MMAs
+            if (exp() & 1) break;  // measurement aid: no MMAs
             if (MX)  // one atom (4 columns) serves two K = 64 steps: bytes 0-1, then bytes 2-3
               tc2_mma_mxf4(d_tmem, make_desc(a_lo + 2 * j, kDescHiOperand), make_desc(b_lo + 2 * j, kDescHiOperand),
                            idesc_mx[j & 1], sf_t + (j >> 1) * 4, sf_t + 16 + (j >> 1) * 4 * kGroups, (kb > 0 || j > 0) ? 1u : 0u);
@@ -658,19 +660,19 @@ __global__ void __cluster_dims__(2 * SPLIT, 1, 1) __launch_bounds__(kThreads, 1)
         if (++acc == C::kAcc) acc = 0;
         probe_kb += (unsigned long long)k_blocks;
         ++probe_tiles;
-        if (g.probe) probe_mark = clock64();
+        if (probe()) probe_mark = clock64();
       }
-      if (g.probe && split == 0) {
+      if (probe() && split == 0) {
         // the last commit has been issued, not completed: wait for the accumulator hand-over of the last tile so that
         // the interval covers the work (bounded like every other wait)
         const int last = C::kAcc - 1 - acc;  // (one accumulator: itself; two: the one used last)
         mbar_wait_cluster(acce_bar(last), ((acc_phase >> last) & 1u) ^ 1u, abort_flag, 0x380u);
         probe_wait += clock64() - probe_mark;
-        g.probe[8 * pair_id] = (unsigned long long)(clock64() - probe_c0);
-        g.probe[8 * pair_id + 1] = globaltimer_ns() - probe_t0;
-        g.probe[8 * pair_id + 2] = probe_kb;
-        g.probe[8 * pair_id + 3] = probe_tiles;
-        g.probe[8 * pair_id + 4] = (unsigned long long)probe_wait;
+        probe()[8 * pair_id] = (unsigned long long)(clock64() - probe_c0);
+        probe()[8 * pair_id + 1] = globaltimer_ns() - probe_t0;
+        probe()[8 * pair_id + 2] = probe_kb;
+        probe()[8 * pair_id + 3] = probe_tiles;
+        probe()[8 * pair_id + 4] = (unsigned long long)probe_wait;
       }
     }
   } else if (warp >= 3 && warp <= 10) {
@@ -718,7 +720,7 @@ __global__ void __cluster_dims__(2 * SPLIT, 1, 1) __launch_bounds__(kThreads, 1)
       // agree on giving up: a warp that timed out still joins this barrier, and all 128 threads take ONE decision
       if (group_gave_up(abort_flag, bar_id, 128)) break;
       tc_fence_after();
-      if (g.exp & 8) {  // measurement aid: the accumulator is handed back unread, nothing is stored
+      if (exp() & 8) {  // measurement aid: the accumulator is handed back unread, nothing is stored
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive_cluster(acce_leader + 8u * acc);
@@ -763,10 +765,10 @@ __global__ void __cluster_dims__(2 * SPLIT, 1, 1) __launch_bounds__(kThreads, 1)
           store_half<false, true, kHalf>(r, alpha, et, bar_id, row_in_tile, stage_buf, map_d, x0, row0, accumulate, drain, beta);
       } else if (d_is_fp32) {
         store_half<true, false, kHalf>(r, alpha, et, bar_id, row_in_tile, stage_buf, map_d, x0, row0, accumulate, drain,
-                                       nullptr, (g.exp >> 6) & 3);
+                                       nullptr, (exp() >> 6) & 3);
       } else {
         store_half<false, false, kHalf>(r, alpha, et, bar_id, row_in_tile, stage_buf, map_d, x0, row0, accumulate, drain,
-                                        nullptr, (g.exp >> 6) & 3);
+                                        nullptr, (exp() >> 6) & 3);
       }
       next_acc();
     }
