@@ -242,8 +242,7 @@ NVFP4_API nvfp4_status nvfp4_sq_error(const void* ref, int32_t ref_is_fp32, int6
  *   (programmatic dependent launch) and never read each other's output early; in the NVFP4 bf16 path X and a fresh W
  *   are quantized by the same launches.  Y and dX also serve as scratch before the product is written (not where they
  *   lie over an input).  Results are bit-identical to the same steps issued one by one through
- *   nvfp4_quantize and nvfp4_gemm; a backward call for both products is so up to the order of the FP32 sums where
- *   nvfp4_gemm splits the contraction of one of them (few output tiles, K of thousands).
+ *   nvfp4_quantize and nvfp4_gemm, and a product of a backward call does not depend on whether the other is asked for.
  * Format: the layer runs in the format of the copies it is given (W_row / W_col_saved / X_col_saved must
  *   agree).  With MXFP4 copies the same sequence uses 1x32 and 32x32 blocks and the 32-point transform
  *   (Section 5); opts->rht_sign_mask then supplies 32 sign bits.
@@ -333,7 +332,8 @@ NVFP4_API nvfp4_status nvfp4_test_cluster_leave(uint64_t delay_ns, uint64_t* tim
 /* Tuning knob: which GEMM tiling to use.  128 / 256 = one CTA per 128 x 128 / 128 x 256 output tile (256 needs
  * N % 256 == 0, otherwise 128 is used); CTA pairs: 640 = 256 x 128 tiles, 512 = 256 x 256 tiles, 768 = 256 x 384 tiles plus
  * up to two 256-wide ones per row of tiles (needs N >= 256, otherwise as 512); 642 / 644 = 256 x 128 tiles whose
- * contraction two / four CTA pairs share (K >= 512 / 1024, otherwise, and for two products in one launch, as 640 / 512);
+ * contraction two / four CTA pairs share (K >= 512 / 1024, otherwise as 640; two products in one launch: as 640, summed in
+ * the same order);
  * 0 = choose by shape (the CTA-pair tile whose static schedule is estimated shortest).
  * Returns 0, or -1 for any other value.  Process-wide; results do not depend on it
  * beyond FP32 summation order. */

@@ -211,6 +211,7 @@ nvfp4_status gemm_prepare(const nvfp4_tensor* A, const nvfp4_tensor* B, void* D,
   g.mx = A->format == NVFP4_FORMAT_MXFP4;
   g.a_rows = a_rs ? A->global : nullptr;
   g.b_rows = b_rs ? B->global : nullptr;
+  g.shares = 1;
   return NVFP4_OK;
 }
 
@@ -419,10 +420,13 @@ nvfp4_status nvfp4_linear_bwd(const void* dY, const nvfp4_tensor* X_col_saved, c
     return st;
   if (dX_bf16 && dW_fp32) {
     // Dgrad and Wgrad are independent: when both run on CTA pairs they share one launch, the longer contraction
-    // first, so the partial last round of one is filled with tiles of the other
+    // first, so the partial last round of one is filled with tiles of the other.  Their bits are those of the separate products:
+    // one that is split when it is alone is summed in the same order here.
     GemmArgs gd, gw;
     if ((st = gemm_prepare(&g_row, W_col_saved, dX_bf16, 0, K, 0, gd)) != NVFP4_OK) return st;
     if ((st = gemm_prepare(&g_col, X_col_saved, dW_fp32, 1, K, accumulate_dw, gw)) != NVFP4_OK) return st;
+    gd.shares = split_of(gd, gemm_tile(gd));
+    gw.shares = split_of(gw, gemm_tile(gw));
     const bool dgrad_first = gd.K >= gw.K;
     const int tile = dgrad_first ? gemm_tile(gd, &gw) : gemm_tile(gw, &gd);
     if (tile >= kTilePair256) {

@@ -402,7 +402,8 @@ std::atomic<int> g_exp_mode{0}, g_exp_max_pairs{0};
 std::atomic<unsigned long long*> g_exp_probe{nullptr};
 
 pair::Problem pair_problem(const GemmArgs& g) {
-  return pair::Problem{g.M, g.N, g.K, g.sfa, g.sfb, g.a_global, g.b_global, g.d_is_fp32, g.accumulate, g.a_rows, g.b_rows};
+  return pair::Problem{g.M,         g.N,          g.K,      g.sfa,    g.sfb,   g.a_global, g.b_global,
+                       g.d_is_fp32, g.accumulate, g.a_rows, g.b_rows, g.shares == 4 ? 2 : g.shares == 2 ? 1 : 0};
 }
 
 bool has_row_scales(const GemmArgs& g0, const GemmArgs* g1) {
@@ -413,10 +414,10 @@ bool has_row_scales(const GemmArgs& g0, const GemmArgs* g1) {
 inline int pair_tiles(const GemmArgs& g, int bn) { return ((g.M + 255) / 256) * ((g.N + bn - 1) / bn); }
 
 // g1 == nullptr: one problem
-template <bool MX, bool ROWS, int BN, int SPLIT = 1>
+template <bool MX, bool ROWS, int BN, int SPLIT = 1, bool SHARES = false>
 cudaError_t launch_pair_t(const GemmArgs& g0, const void* a0, const void* b0, const GemmArgs* g1, const void* a1,
                           const void* b1, int num_sms, cudaStream_t s) {
-  auto kern = pair::gemm_pair_kernel<MX, ROWS, BN, SPLIT>;
+  auto kern = pair::gemm_pair_kernel<MX, ROWS, BN, SPLIT, SHARES>;
   constexpr int smem = pair::Cfg<BN, SPLIT>::kSmemBytes, store_cols = SPLIT > 1 ? BN / SPLIT : 64;
   CUtensorMap m[6];
   if (!make_pair_maps(g0, a0, b0, BN, store_cols, &m[0], &m[1], &m[2])) return cudaErrorInvalidValue;
@@ -639,13 +640,19 @@ cudaError_t launch_wide(const GemmArgs& g0, const void* a0, const void* b0, cons
 
 }  // namespace
 
+int split_of(const GemmArgs& g, int tile) {
+  const int split = tile == kTileSplit2 ? 2 : tile == kTileSplit4 ? 4 : 1;
+  return g.K / 256 >= split ? split : 1;  // a pair has a k-block at least
+}
+
 cudaError_t launch_gemm(const GemmArgs& g, const void* a_codes, const void* b_codes, int tile, cudaStream_t s) {
   int num_sms = 0;
   cudaError_t e = sm_count(&num_sms);
   if (e != cudaSuccess) return e;
   const bool rows = has_row_scales(g, nullptr);  // scale vectors: the pair kernels' epilogues only
-  if (tile == kTileSplit2 && g.K / 256 >= 2) return launch_split<2>(g, a_codes, b_codes, num_sms, s);
-  if (tile == kTileSplit4 && g.K / 256 >= 4) return launch_split<4>(g, a_codes, b_codes, num_sms, s);
+  const int split = split_of(g, tile);
+  if (split == 2) return launch_split<2>(g, a_codes, b_codes, num_sms, s);
+  if (split == 4) return launch_split<4>(g, a_codes, b_codes, num_sms, s);
   if (tile == kTileSplit2 || tile == kTileSplit4) tile = kTilePair128;
   if (tile == kTileWide && wide_eligible(g)) return launch_wide(g, a_codes, b_codes, nullptr, nullptr, nullptr, num_sms, s);
   if (tile >= kTilePair256 || rows)
@@ -660,8 +667,13 @@ cudaError_t launch_gemm_two(const GemmArgs& g0, const void* a0, const void* b0, 
   int num_sms = 0;
   cudaError_t e = sm_count(&num_sms);
   if (e != cudaSuccess) return e;
+  if (g0.shares > 1 || g1.shares > 1) {
+    if (g1.mx != g0.mx || has_row_scales(g0, &g1)) return cudaErrorInvalidValue;
+    return g0.mx ? launch_pair_t<true, false, 128, 1, true>(g0, a0, b0, &g1, a1, b1, num_sms, s)
+                 : launch_pair_t<false, false, 128, 1, true>(g0, a0, b0, &g1, a1, b1, num_sms, s);
+  }
   if (tile == kTileWide && wide_eligible(g0) && wide_eligible(g1)) return launch_wide(g0, a0, b0, &g1, a1, b1, num_sms, s);
-  return launch_pair(g0, a0, b0, &g1, a1, b1, tile == kTilePair128 ? 128 : 256, num_sms, s);
+  return launch_pair(g0, a0, b0, &g1, a1, b1, tile == kTilePair256 || tile == kTileWide ? 256 : 128, num_sms, s);
 }
 
 int best_pair_tile(const GemmArgs& g0, const GemmArgs* g1) {

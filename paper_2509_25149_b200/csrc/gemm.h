@@ -17,6 +17,7 @@ struct GemmArgs {
   int mx;                 // operands are MXFP4 (UE8M0 scale per 32 elements) instead of NVFP4
   const float* a_rows;    // per-row {amax, s_dec} pairs of A / B when their global scale is taken per row, else NULL
   const float* b_rows;    // (CTA-pair kernels only)
+  int shares;             // launch_gemm_two: parts of the contraction that are summed apart (split_of; 1 otherwise)
 };
 
 // Tiles: 128 or 256 = one CTA per 128 x 128 / 128 x 256 tile (256 needs N % 256 == 0, otherwise 128 is used); the others
@@ -27,8 +28,11 @@ constexpr int kTileWide = 768;     // 256 x 384, needs N >= 256
 constexpr int kTileSplit2 = 642;   // 256 x 128, a cluster of two pairs per tile shares its contraction (K >= 512)
 constexpr int kTileSplit4 = 644;   // the same with four pairs (K >= 1024)
 cudaError_t launch_gemm(const GemmArgs& g, const void* a_codes, const void* b_codes, int tile, cudaStream_t s);
+// CTA pairs that share a tile's contraction when `tile` is asked for: 4, 2 or 1
+int split_of(const GemmArgs& g, int tile);
 // Two independent GEMMs in one launch of a CTA-pair kernel: the tiles of g0 are worked through first, then those of g1,
-// on one persistent grid.
+// on one persistent grid.  Where either is split when it has a launch to itself (GemmArgs::shares), the sums of both are taken
+// in the same order here, on 256 x 128 tiles whatever `tile` says.
 cudaError_t launch_gemm_two(const GemmArgs& g0, const void* a0, const void* b0, const GemmArgs& g1, const void* a1,
                             const void* b1, int tile, cudaStream_t s);
 // Scheduling estimate: the CTA-pair tile for this problem (or pair of problems in one launch, then no split one)

@@ -61,6 +61,7 @@ struct Problem {
   // the operand; NULL = the operand carries the usual per-tensor words in a_global / b_global
   const float* a_rows;
   const float* b_rows;
+  int shares_log2;  // SHARES: the sums are taken in 1 << shares_log2 shares, as so many pairs would take them
 };
 // One launch works through the tiles of up to two independent GEMMs (problem 0 first): Dgrad and Wgrad of a
 // linear layer share no output, so their tiles can fill the same persistent grid and the partial last round of
@@ -382,12 +383,17 @@ __device__ __forceinline__ bool exchange_columns(const uint32_t (&r)[64], uint32
 // it sends its sums of the others' columns into their shared memory and adds what it receives to its own, always in the
 // order of the pairs.  (A product of few tiles is bound by one pair's main loop, 0.31 us per k-block: shared by four 0.08; figures at
 // split_tile().)
-template <bool MX, bool ROWS = false, int BN = 256, int SPLIT = 1>
+// SHARES (BN = 128): the contraction of a problem is cut into 1 << shares_log2 parts, which a pair sums one after the other into the
+// two accumulators; the epilogue adds them in the order in which SPLIT pairs add theirs.  For the two products of a backward call in
+// one launch: each comes out bit for bit as the launch that it would have to itself makes it.  (In one sum / in shares / the two
+// products behind each other: backward call of 512 x 3584 x 768 16.0 / 16.3 / 22.6 us, 2048 x 512 x 512 14.0 / 14.4 / 18.5.)
+template <bool MX, bool ROWS = false, int BN = 256, int SPLIT = 1, bool SHARES = false>
 __global__ void __cluster_dims__(2 * SPLIT, 1, 1) __launch_bounds__(kThreads, 1)
     gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant__ CUtensorMap map_b0,
                      const __grid_constant__ CUtensorMap map_d0, const __grid_constant__ CUtensorMap map_a1,
                      const __grid_constant__ CUtensorMap map_b1, const __grid_constant__ CUtensorMap map_d1,
                      const __grid_constant__ Args g) {
+  static_assert(!SHARES || (BN == 128 && SPLIT == 1 && !ROWS), "two accumulators, one pair per tile");
   using C = Cfg<BN, SPLIT>;
   constexpr int kStages = C::kStages, kStageBytes = C::kStageBytes, kBBytes = C::kBBytes, kGroups = C::kGroups;
   constexpr int kSfCol = C::kSfCol, kSfSlotCols = C::kSfSlotCols;
@@ -614,53 +620,56 @@ __global__ void __cluster_dims__(2 * SPLIT, 1, 1) __launch_bounds__(kThreads, 1)
       unsigned long long probe_kb = 0, probe_tiles = 0;
       long long probe_wait = 0, probe_mark = probe_c0;  // cycles spent waiting for the accumulator to be handed back
       for (int rnd = 0, tile = pair_id; tile < n_tiles && ok; tile = next_tile(++rnd)) {
-        if (!(exp() & 16) && !(ok = mbar_wait_cluster(acce_bar(acc), ((acc_phase >> acc) & 1u) ^ 1u, abort_flag, 0x300u)))
-          break;
-        if (probe()) probe_wait += clock64() - probe_mark;
-        tc_fence_after();
-        const uint32_t d_tmem = tmem + acc * BN;
-        const int k_blocks = k_blocks_of(tile);
-        for (int kb = 0; kb < k_blocks; ++kb) {
-          if (!(ok = mbar_wait_cluster(full_bar(stage), phase, abort_flag, 0x200u + stage))) break;
-          if (!(ok = mbar_wait_cluster(sff_bar(stage), phase, abort_flag, 0x280u + stage))) break;
+        const int k_all = k_blocks_of(tile), shares_log2 = SHARES ? g.p[tile >= g.n_tiles0 ? 1 : 0].shares_log2 : 0;
+        for (int share = 0; share < 1 << shares_log2 && ok; ++share) {
+          if (!(exp() & 16) && !(ok = mbar_wait_cluster(acce_bar(acc), ((acc_phase >> acc) & 1u) ^ 1u, abort_flag, 0x300u)))
+            break;
+          if (probe()) probe_wait += clock64() - probe_mark;
           tc_fence_after();
-          const uint32_t a_lo = a_lo0 + stage * (kStageBytes >> 4);
-          const uint32_t b_lo = b_lo0 + stage * (kStageBytes >> 4);
-          const uint32_t sf_t = tmem + kSfCol + stage * kSfSlotCols;
-          if (exp() & 32) {  // measurement aid: the scale atoms go through the copy engine, issued here
-            const uint32_t sf_lo = (((base + kABytes + kBBytes) >> 4) & 0x3fffu) + stage * (kStageBytes >> 4);
-            constexpr int kAtomsKb = MX ? 2 : 4;
+          const uint32_t d_tmem = tmem + acc * BN;
+          const int k_blocks = SHARES ? (k_all * (share + 1) >> shares_log2) - (k_all * share >> shares_log2) : k_all;
+          for (int kb = 0; kb < k_blocks; ++kb) {
+            if (!(ok = mbar_wait_cluster(full_bar(stage), phase, abort_flag, 0x200u + stage))) break;
+            if (!(ok = mbar_wait_cluster(sff_bar(stage), phase, abort_flag, 0x280u + stage))) break;
+            tc_fence_after();
+            const uint32_t a_lo = a_lo0 + stage * (kStageBytes >> 4);
+            const uint32_t b_lo = b_lo0 + stage * (kStageBytes >> 4);
+            const uint32_t sf_t = tmem + kSfCol + stage * kSfSlotCols;
+            if (exp() & 32) {  // measurement aid: the scale atoms go through the copy engine, issued here
+              const uint32_t sf_lo = (((base + kABytes + kBBytes) >> 4) & 0x3fffu) + stage * (kStageBytes >> 4);
+              constexpr int kAtomsKb = MX ? 2 : 4;
 #pragma unroll
-            for (int j = 0; j < kAtomsKb; ++j) {
-              tc2_cp_sf(sf_t + j * 4, make_desc(sf_lo + j * 32, kDescHiSf));
+              for (int j = 0; j < kAtomsKb; ++j) {
+                tc2_cp_sf(sf_t + j * 4, make_desc(sf_lo + j * 32, kDescHiSf));
 #pragma unroll
-              for (int grp = 0; grp < kGroups; ++grp)
-                tc2_cp_sf(sf_t + 16 + 4 * kGroups * j + 4 * grp, make_desc(sf_lo + (kSfaBytes >> 4) + grp * 128 + j * 32, kDescHiSf));
+                for (int grp = 0; grp < kGroups; ++grp)
+                  tc2_cp_sf(sf_t + 16 + 4 * kGroups * j + 4 * grp, make_desc(sf_lo + (kSfaBytes >> 4) + grp * 128 + j * 32, kDescHiSf));
+              }
+            }
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              if (exp() & 1) break;  // measurement aid: no MMAs
+              if (MX)  // one atom (4 columns) serves two K = 64 steps: bytes 0-1, then bytes 2-3
+                tc2_mma_mxf4(d_tmem, make_desc(a_lo + 2 * j, kDescHiOperand), make_desc(b_lo + 2 * j, kDescHiOperand),
+                             idesc_mx[j & 1], sf_t + (j >> 1) * 4, sf_t + 16 + (j >> 1) * 4 * kGroups, (kb > 0 || j > 0) ? 1u : 0u);
+              else
+                tc2_mma_nvf4(d_tmem, make_desc(a_lo + 2 * j, kDescHiOperand), make_desc(b_lo + 2 * j, kDescHiOperand), idesc,
+                             sf_t + j * 4, sf_t + 16 + j * 4 * kGroups, (kb > 0 || j > 0) ? 1u : 0u);
+            }
+            tc2_commit_both(empty_bar(stage), pair_mask);  // both CTAs' stages are free once these MMAs have read them
+            if (++stage == kStages) {
+              stage = 0;
+              phase ^= 1u;
             }
           }
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            if (exp() & 1) break;  // measurement aid: no MMAs
-            if (MX)  // one atom (4 columns) serves two K = 64 steps: bytes 0-1, then bytes 2-3
-              tc2_mma_mxf4(d_tmem, make_desc(a_lo + 2 * j, kDescHiOperand), make_desc(b_lo + 2 * j, kDescHiOperand),
-                           idesc_mx[j & 1], sf_t + (j >> 1) * 4, sf_t + 16 + (j >> 1) * 4 * kGroups, (kb > 0 || j > 0) ? 1u : 0u);
-            else
-              tc2_mma_nvf4(d_tmem, make_desc(a_lo + 2 * j, kDescHiOperand), make_desc(b_lo + 2 * j, kDescHiOperand), idesc,
-                           sf_t + j * 4, sf_t + 16 + j * 4 * kGroups, (kb > 0 || j > 0) ? 1u : 0u);
-          }
-          tc2_commit_both(empty_bar(stage), pair_mask);  // both CTAs' stages are free once these MMAs have read them
-          if (++stage == kStages) {
-            stage = 0;
-            phase ^= 1u;
-          }
+          if (!ok) break;
+          tc2_commit_both(accf_bar(acc), pair_mask);  // this accumulator is complete in both CTAs
+          acc_phase ^= 1u << acc;
+          if (++acc == C::kAcc) acc = 0;
+          probe_kb += (unsigned long long)k_blocks;
+          ++probe_tiles;
+          if (probe()) probe_mark = clock64();
         }
-        if (!ok) break;
-        tc2_commit_both(accf_bar(acc), pair_mask);  // this accumulator is complete in both CTAs
-        acc_phase ^= 1u << acc;
-        if (++acc == C::kAcc) acc = 0;
-        probe_kb += (unsigned long long)k_blocks;
-        ++probe_tiles;
-        if (probe()) probe_mark = clock64();
       }
       if (probe() && split == 0) {
         // the last commit has been issued, not completed: wait for the accumulator hand-over of the last tile so that
@@ -741,6 +750,28 @@ __global__ void __cluster_dims__(2 * SPLIT, 1, 1) __launch_bounds__(kThreads, 1)
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive_cluster(acce_leader + 8u * acc);
+      if constexpr (SHARES) {
+        bool gave_up = false;
+#pragma unroll 1
+        for (int more = (1 << g.p[prob].shares_log2) - 1; more > 0; --more) {
+          next_acc();
+          mbar_wait_cluster(accf_bar(acc), (acc_phase >> acc) & 1u, abort_flag, 0x400u);
+          if ((gave_up = group_gave_up(abort_flag, bar_id, 128))) break;
+          tc_fence_after();
+#pragma unroll
+          for (int q = 0; q < kHalf; q += 16) {
+            uint32_t part[16];
+            tc_ld16(t_row0 + acc * BN + q, part);
+            tc_wait_ld();
+#pragma unroll
+            for (int k = 0; k < 16; ++k) r[q + k] = __float_as_uint(__uint_as_float(r[q + k]) + __uint_as_float(part[k]));
+          }
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive_cluster(acce_leader + 8u * acc);
+        }
+        if (gave_up) break;
+      }
       if constexpr (SPLIT > 1) {
         constexpr int kCols = C::kCols;
         uint32_t v[kCols];

@@ -85,3 +85,42 @@ def test_bf16_products(shape):
     again = torch.empty_like(Y)
     B.nvfp4_linear_bf16_fwd(X, W, again)
     assert torch.equal(again, Y)
+
+
+# the first two are split by the rule (dX, dW); 1280 and 1792: shares of unequal length
+@pytest.mark.parametrize("size", [(512, 3584, 768), (2048, 512, 512), (256, 1280, 1792), (1792, 256, 1280), (256, 256, 512)])
+@pytest.mark.parametrize("tile", [0, 642, 644])
+@pytest.mark.parametrize("fmt", [B.FORMAT_NVFP4, B.FORMAT_MXFP4])
+def test_backward_call_sums_as_its_products_do(size, tile, fmt):
+    """Blocks far apart in magnitude, so that the FP32 sums are not exact: the bits tell the order of the additions."""
+    M, N, K = size
+    gen = torch.Generator("cuda").manual_seed(M + N + K)
+
+    def source(rows, cols):
+        x = torch.randn((rows, cols), generator=gen, device="cuda")
+        return (x * torch.exp2(torch.randint(-9, 10, (rows // 32, cols // 32), generator=gen, device="cuda").float())
+                .repeat_interleave(32, 0).repeat_interleave(32, 1)).to(torch.bfloat16)
+
+    dy = source(M, N)
+    xc, wc, gr, gc = (B.alloc_tensor(r, c, format=fmt) for r, c in ((K, M), (K, N), (M, N), (N, M)))
+    B.nvfp4_quantize(source(K, M), B.quant_opts(), xc)
+    B.nvfp4_quantize(source(K, N), B.quant_opts(), wc)
+    opts = B.quant_opts(rounding=B.ROUND_STOCHASTIC, rht_colwise=True, rht_sign_mask=0x73E5, seed=3)
+    B.nvfp4_quantize(dy, opts, gr, gc)
+    ws = torch.empty(B.nvfp4_linear_bwd_workspace_bytes(M, N), dtype=torch.uint8, device="cuda")
+
+    def buffers():
+        return torch.zeros((M, K), dtype=torch.bfloat16, device="cuda"), torch.full((N, K), 0.5, device="cuda")
+
+    B.nvfp4_set_gemm_tile_n(tile)
+    try:
+        (dx0, dw0), (dx1, dw1), (dx2, dw2) = buffers(), buffers(), buffers()
+        B.nvfp4_gemm(gr, wc, dx0)
+        B.nvfp4_gemm(gc, xc, dw0, accumulate=True)
+        B.nvfp4_linear_bwd(dy, xc, wc, K, opts, dx1, dw1, True, ws)
+        B.nvfp4_linear_bwd(dy, xc, wc, K, opts, dx2, None, True, ws)
+        B.nvfp4_linear_bwd(dy, xc, wc, K, opts, None, dw2, True, ws)
+        B.nvfp4_device_status()
+    finally:
+        B.nvfp4_set_gemm_tile_n(0)
+    assert torch.equal(dx1, dx0) and torch.equal(dw1, dw0) and torch.equal(dx2, dx0) and torch.equal(dw2, dw0)
