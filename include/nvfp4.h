@@ -334,7 +334,8 @@ NVFP4_API nvfp4_status nvfp4_test_cluster_leave(uint64_t delay_ns, uint64_t* tim
  * up to two 256-wide ones per row of tiles (needs N >= 256, otherwise as 512); 642 / 644 = 256 x 128 tiles whose
  * contraction two / four CTA pairs share (K >= 512 / 1024, otherwise as 640; two products in one launch: as 640, summed in
  * the same order);
- * 0 = choose by shape (the CTA-pair tile whose static schedule is estimated shortest).
+ * 0 = choose by shape (the CTA-pair tile whose static schedule is estimated shortest; whether a contraction is
+ * shared, and so the order of the FP32 sums, also depends on how many such clusters the GPU keeps resident).
  * Returns 0, or -1 for any other value.  Process-wide; results do not depend on it
  * beyond FP32 summation order. */
 NVFP4_API int32_t nvfp4_set_gemm_tile_n(int32_t tile_n);

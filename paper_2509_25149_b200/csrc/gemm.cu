@@ -19,11 +19,11 @@
 
 #include "common.cuh"
 #include <algorithm>
-#include <mutex>
 #include <vector>
 
 #include "gemm.h"
 #include "tc_ptx.cuh"
+#include "tile_memo.h"
 #include "gemm_2cta.cuh"
 #include "gemm_wide.cuh"
 #include "gemm_bf16.cuh"
@@ -680,22 +680,16 @@ int best_pair_tile(const GemmArgs& g0, const GemmArgs* g1) {
   int num_sms = 0;
   if (sm_count(&num_sms) != cudaSuccess) return kTilePair256;
   const bool wide_fits = wide_eligible(g0) && (!g1 || wide_eligible(*g1));
-  // the estimate walks every tile of the schedules: remember the answers for the shapes seen (a training loop
-  // repeats a handful of them)
-  struct Entry { int key[8]; int tile; };
-  static std::mutex mu;
-  static std::vector<Entry> seen;
+  int dev = 0, best = kTilePair256;
+  if (cudaGetDevice(&dev) != cudaSuccess) return best;
+  static TileMemo memo;
   // (the output type is part of the key: an fp32 output changes the hand-over cost and with it the choice)
-  const int key[8] = {g0.M, g0.N, g0.K, g1 ? g1->M : 0, g1 ? g1->N : 0, g1 ? g1->K : 0, num_sms,
-                      (g0.d_is_fp32 ? 1 : 0) | (g1 && g1->d_is_fp32 ? 2 : 0) | (wide_fits ? 4 : 0)};
-  {
-    std::lock_guard<std::mutex> lock(mu);
-    for (const Entry& e : seen)
-      if (std::equal(key, key + 8, e.key)) return e.tile;
-  }
+  const int key[TileMemo::kKey] = {g0.M, g0.N, g0.K, g1 ? g1->M : 0, g1 ? g1->N : 0, g1 ? g1->K : 0,
+                                   (g0.d_is_fp32 ? 1 : 0) | (g1 && g1->d_is_fp32 ? 2 : 0), dev};
+  if (memo.find(key, &best)) return best;
   const GemmArgs* gs[2] = {&g0, g1};
   const int n = g1 ? 2 : 1, pairs = num_sms / 2;
-  int best = kTilePair256;
+  best = kTilePair256;
   double least = pair_makespan(gs, n, kTilePair256, pairs);
   for (int tile : {kTilePair128, kTileWide}) {
     if (tile == kTileWide && !wide_fits) continue;
@@ -707,13 +701,7 @@ int best_pair_tile(const GemmArgs& g0, const GemmArgs* g1) {
   }
   if (!g1)
     if (const int tile = split_tile(g0, least)) best = tile;
-  std::lock_guard<std::mutex> lock(mu);
-  if (seen.size() < 256) {
-    Entry e{};
-    std::copy(key, key + 8, e.key);
-    e.tile = best;
-    seen.push_back(e);
-  }
+  memo.put(key, best);
   return best;
 }
 
