@@ -346,7 +346,7 @@ def nvfp4_set_gemm_experiment(mode: int = 0, max_pairs: int = 0, probe: Optional
 
 def nvfp4_set_gemm_tile_n(tile_n: int) -> None:
     if lib().nvfp4_set_gemm_tile_n(tile_n) != 0:
-        raise ValueError("tile_n must be 0, 128, 256, 512, 640 or 768")
+        raise ValueError("tile_n must be 0, 128, 256, 512, 640, 642, 644 or 768")
 
 
 def nvfp4_launch_count() -> int:

@@ -143,3 +143,12 @@ def test_plain_c_client_runs():
                        check=True)
         r = subprocess.run([exe], capture_output=True, text=True, timeout=120)
         assert r.returncode == 0 and r.stdout.startswith("ok"), (r.returncode, r.stdout, r.stderr)
+
+
+def test_the_message_names_every_tile_that_is_accepted():
+    with pytest.raises(ValueError) as e:
+        B.nvfp4_set_gemm_tile_n(1)
+    named = {int(n) for n in re.findall(r"\d+", str(e.value))}
+    accepted = {n for n in range(1100) if B.lib().nvfp4_set_gemm_tile_n(n) == 0}
+    B.nvfp4_set_gemm_tile_n(0)
+    assert named == accepted
