@@ -106,9 +106,16 @@ def _check(status: int, where: str) -> None:
         raise NVFP4Error(status, where)
 
 
+# torch.cuda.current_stream() builds a Stream object around the handle, 3 us of host time per call; these return it as it is, where
+# this torch has them
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_get_device = getattr(torch._C, "_cuda_getDevice", None)
+
+
 def _stream() -> int:
-    # the handle itself: torch.cuda.current_stream() builds a Stream object around it, 3 us of host time per call
-    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    if _raw_stream is None or _get_device is None or not torch.cuda.is_initialized():
+        return torch.cuda.current_stream().cuda_stream  # (initialises CUDA)
+    return _raw_stream(_get_device())
 
 
 _TENSOR_FIELDS = struct.Struct("PPPqqii")  # nvfp4_tensor

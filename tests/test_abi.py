@@ -4,6 +4,7 @@ import os
 import re
 
 import pytest
+import torch
 
 from paper_2509_25149_b200 import binding as B
 
@@ -152,3 +153,18 @@ def test_the_message_names_every_tile_that_is_accepted():
     accepted = {n for n in range(1100) if B.lib().nvfp4_set_gemm_tile_n(n) == 0}
     B.nvfp4_set_gemm_tile_n(0)
     assert named == accepted
+
+
+@pytest.mark.parametrize("missing", ["_raw_stream", "_get_device", "CUDA not initialised"])
+def test_stream_handle_comes_from_the_public_call_where_it_has_to(monkeypatch, missing):
+    class Stream:
+        cuda_stream = 0x1234
+
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda *a: Stream())
+    monkeypatch.setattr(torch.cuda, "is_initialized", lambda: missing != "CUDA not initialised")
+    monkeypatch.setattr(B, "_get_device", lambda: 0)
+    monkeypatch.setattr(B, "_raw_stream", lambda device: 0x5678)
+    assert B._stream() == (0x1234 if missing == "CUDA not initialised" else 0x5678)
+    if missing.startswith("_"):
+        monkeypatch.setattr(B, missing, None)
+        assert B._stream() == 0x1234
