@@ -36,6 +36,10 @@ class CTensor(ctypes.Structure):
                 ("rows", ctypes.c_int64), ("cols", ctypes.c_int64), ("sf_layout", ctypes.c_int32),
                 ("format", ctypes.c_int32)]
 
+    @property
+    def _as_parameter_(self):  # a struct itself may be passed where its address is wanted
+        return ctypes.byref(self)
+
 
 class CQuantOpts(ctypes.Structure):
     _fields_ = [("block_rows", ctypes.c_int32), ("rounding", ctypes.c_int32), ("rht_rowwise", ctypes.c_int32),

@@ -168,3 +168,11 @@ def test_stream_handle_comes_from_the_public_call_where_it_has_to(monkeypatch, m
     if missing.startswith("_"):
         monkeypatch.setattr(B, missing, None)
         assert B._stream() == 0x1234
+
+
+def test_tensor_structs_are_taken_in_every_form():
+    """The struct, its address, a pointer to it, its bytes; NULL in its place is an error of the call, not of ctypes."""
+    L, t, o = B.lib(), B.CTensor(), B.quant_opts()
+    for form in (t, ctypes.byref(t), ctypes.pointer(t), bytes(t), None):
+        assert L.nvfp4_gemm(form, form, None, 0, 0, 0, None) == 1
+        assert L.nvfp4_quantize(None, 16, 16, 16, ctypes.byref(o), form, None, None) == 1
