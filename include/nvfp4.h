@@ -178,8 +178,8 @@ NVFP4_API nvfp4_status nvfp4_gemm(const nvfp4_tensor* A, const nvfp4_tensor* B, 
  *   B: device bf16.  b_layout NVFP4_K_MAJOR : stored [N][K], ldb >= K;  NVFP4_MN_MAJOR: stored [K][N], ldb >= N.
  *   D: device, row-major [M x N], ldd >= N, bf16 (round-to-nearest-even) or fp32 (d_is_fp32 != 0);
  *      accumulate != 0 adds into an fp32 D.
- *   M, N, K multiples of 8 (the kernel works on 256 x 256 x 64 tiles; ragged edges are zero-filled on load and
- *   clipped on store by the tensor maps); pointers 16-byte aligned, lda, ldb multiples of 8, ldd * elemsize of 16.
+ *   M, N, K multiples of 8 (the kernel works on 256 x 256 or 256 x 128 tiles, 64 deep, and a narrow tile's contraction may be
+ *   shared by two or four CTA pairs; ragged edges are zero-filled on load and clipped on store by the tensor maps); pointers 16-byte aligned, lda, ldb multiples of 8, ldd * elemsize of 16.
  *   Nothing is enqueued on error.
  */
 enum { NVFP4_K_MAJOR = 0, NVFP4_MN_MAJOR = 1 };
@@ -191,7 +191,8 @@ NVFP4_API nvfp4_status nvfp4_gemm_bf16(const void* A, int32_t a_layout, int64_t 
  * The same layer as nvfp4_linear_fwd / _bwd without quantization (Section 4.1, Appendix D), on the same row-major
  * operands X [M x K], W [N x K], dY [M x N], all contiguous bf16; no transposed copies are made:
  *   fwd: Y  = X W^T (bf16);   bwd: dX = dY W (bf16), dW = dY^T X (fp32, accumulate_dw != 0 adds into it);
- *   dX or dW may be NULL to skip that GEMM.  M, N, K multiples of 8.
+ *   dX or dW may be NULL to skip that GEMM.  M, N, K multiples of 8.  Both are made in one launch; whether their
+ *   contractions are shared, and so the order of the FP32 sums, is decided for the launch.
  */
 NVFP4_API nvfp4_status nvfp4_linear_bf16_fwd(const void* X, const void* W, int64_t M, int64_t N, int64_t K,
                                              void* Y_bf16, void* cuda_stream);
@@ -333,12 +334,16 @@ NVFP4_API nvfp4_status nvfp4_test_cluster_leave(uint64_t delay_ns, uint64_t* tim
  * N % 256 == 0, otherwise 128 is used); CTA pairs: 640 = 256 x 128 tiles, 512 = 256 x 256 tiles, 768 = 256 x 384 tiles plus
  * up to two 256-wide ones per row of tiles (needs N >= 256, otherwise as 512); 642 / 644 = 256 x 128 tiles whose
  * contraction two / four CTA pairs share (K >= 512 / 1024, otherwise as 640; two products in one launch: as 640, summed in
- * the same order);
+ * the same order); these two are heeded by BF16 products as well (K > 64 / 192, otherwise by size), the others are not;
  * 0 = choose by shape (the CTA-pair tile whose static schedule is estimated shortest; whether a contraction is
  * shared, and so the order of the FP32 sums, also depends on how many such clusters the GPU keeps resident).
  * Returns 0, or -1 for any other value.  Process-wide; results do not depend on it
  * beyond FP32 summation order. */
 NVFP4_API int32_t nvfp4_set_gemm_tile_n(int32_t tile_n);
+
+/* The tile (a value of nvfp4_set_gemm_tile_n) of one M x N x K product with a launch to itself on the current device: nvfp4_gemm,
+ * or nvfp4_gemm_bf16 when bf16 != 0.  -1 for a size that the call would refuse.  Launches nothing. */
+NVFP4_API int32_t nvfp4_gemm_tile(int32_t bf16, int64_t M, int64_t N, int64_t K, int32_t d_is_fp32);
 
 /*
  * Measurement aid for the main loop of the CTA-pair GEMM with 256 x 256 tiles (what bounds a 256-deep k-block):

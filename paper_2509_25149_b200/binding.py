@@ -25,7 +25,7 @@ EXPORTED = (
     "nvfp4_quantize", "nvfp4_gemm", "nvfp4_linear_fwd_workspace_bytes", "nvfp4_linear_bwd_workspace_bytes",
     "nvfp4_linear_fwd", "nvfp4_linear_bwd", "nvfp4_dequantize", "nvfp4_rht16", "nvfp4_e2m1_sr", "nvfp4_test_wait_timeout",
     "nvfp4_test_cluster_leave", "nvfp4_device_status",
-    "nvfp4_set_gemm_tile_n", "nvfp4_set_gemm_experiment", "nvfp4_status_string", "nvfp4_launch_count",
+    "nvfp4_set_gemm_tile_n", "nvfp4_gemm_tile", "nvfp4_set_gemm_experiment", "nvfp4_status_string", "nvfp4_launch_count",
     "nvfp4_linear_fwd_noalloc", "nvfp4_linear_fwd_noalloc_max_bytes",
     "nvfp4_gemm_bf16", "nvfp4_linear_bf16_fwd", "nvfp4_linear_bf16_bwd", "nvfp4_quant_error", "nvfp4_sq_error",
 )
@@ -94,6 +94,7 @@ def lib() -> ctypes.CDLL:
         L.nvfp4_test_cluster_leave.restype, L.nvfp4_test_cluster_leave.argtypes = i32, [ctypes.c_uint64, vp, vp]
         L.nvfp4_device_status.restype, L.nvfp4_device_status.argtypes = i32, [vp, c.POINTER(u32)]
         L.nvfp4_set_gemm_tile_n.restype, L.nvfp4_set_gemm_tile_n.argtypes = i32, [i32]
+        L.nvfp4_gemm_tile.restype, L.nvfp4_gemm_tile.argtypes = i32, [i32, i64, i64, i64, i32]
         L.nvfp4_set_gemm_experiment.restype, L.nvfp4_set_gemm_experiment.argtypes = i32, [i32, i32, vp]
         L.nvfp4_status_string.restype, L.nvfp4_status_string.argtypes = c.c_char_p, [i32]
         L.nvfp4_launch_count.restype, L.nvfp4_launch_count.argtypes = c.c_uint64, []
@@ -358,6 +359,11 @@ def nvfp4_set_gemm_experiment(mode: int = 0, max_pairs: int = 0, probe: Optional
 def nvfp4_set_gemm_tile_n(tile_n: int) -> None:
     if lib().nvfp4_set_gemm_tile_n(tile_n) != 0:
         raise ValueError("tile_n must be 0, 128, 256, 512, 640, 642, 644 or 768")
+
+
+def nvfp4_gemm_tile(bf16: bool, M: int, N: int, K: int, d_is_fp32: bool) -> int:
+    """The tile that such a product takes on the current device (see the header); -1 for a size that is refused."""
+    return int(lib().nvfp4_gemm_tile(int(bf16), M, N, K, int(d_is_fp32)))
 
 
 def nvfp4_launch_count() -> int:

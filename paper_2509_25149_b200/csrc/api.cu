@@ -255,6 +255,11 @@ nvfp4_status bf16_prepare(const void* A, int32_t a_layout, int64_t lda, const vo
   return NVFP4_OK;
 }
 
+nvfp4_status bf16_impl(const DenseGemmArgs& g0, const DenseGemmArgs* g1, void* cuda_stream) {
+  const int tile = bf16_tile(g0, g1, g_tile_n.load(std::memory_order_relaxed));
+  return launch_gemm_bf16(g0, g1, tile, static_cast<cudaStream_t>(cuda_stream)) == cudaSuccess ? NVFP4_OK : NVFP4_ERR_CUDA;
+}
+
 inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 inline size_t copy_bytes(int64_t rows, int64_t cols) {
   return align_up((size_t)(rows * cols / 2), 256) + align_up((size_t)(rows * cols / 16), 256) + 256;
@@ -471,7 +476,7 @@ nvfp4_status nvfp4_gemm_bf16(const void* A, int32_t a_layout, int64_t lda, const
   DenseGemmArgs g;
   const nvfp4_status st = bf16_prepare(A, a_layout, lda, B, b_layout, ldb, M, N, K, D, d_is_fp32, ldd, accumulate, g);
   if (st != NVFP4_OK) return st;
-  return launch_gemm_bf16(g, nullptr, static_cast<cudaStream_t>(cuda_stream)) == cudaSuccess ? NVFP4_OK : NVFP4_ERR_CUDA;
+  return bf16_impl(g, nullptr, cuda_stream);
 }
 
 nvfp4_status nvfp4_linear_bf16_fwd(const void* X, const void* W, int64_t M, int64_t N, int64_t K, void* Y_bf16,
@@ -495,10 +500,7 @@ nvfp4_status nvfp4_linear_bf16_bwd(const void* dY, const void* X, const void* W,
     return st;
   // both: one launch, the longer contraction first
   const bool both = dX_bf16 && dW_fp32, dgrad_first = dX_bf16 && (!both || gd.K >= gw.K);
-  return launch_gemm_bf16(dgrad_first ? gd : gw, both ? (dgrad_first ? &gw : &gd) : nullptr,
-                          static_cast<cudaStream_t>(cuda_stream)) == cudaSuccess
-             ? NVFP4_OK
-             : NVFP4_ERR_CUDA;
+  return bf16_impl(dgrad_first ? gd : gw, both ? (dgrad_first ? &gw : &gd) : nullptr, cuda_stream);
 }
 
 nvfp4_status nvfp4_quant_error(const void* x_bf16, int64_t rows, int64_t cols, int64_t ld, const nvfp4_tensor* q,
@@ -587,6 +589,20 @@ int32_t nvfp4_set_gemm_tile_n(int32_t tile_n) {
     return -1;
   g_tile_n.store(tile_n, std::memory_order_relaxed);
   return 0;
+}
+
+int32_t nvfp4_gemm_tile(int32_t bf16, int64_t M, int64_t N, int64_t K, int32_t d_is_fp32) {
+  if (M <= 0 || N <= 0 || K <= 0 || M > 0x7fffff00 || N > 0x7fffff00 || K > 0x7fffff00) return -1;
+  if (bf16 ? (M % 8 || N % 8 || K % 8) : (M % 128 || N % 128 || K % 256)) return -1;
+  if (bf16) {
+    DenseGemmArgs g{};
+    g.M = (int)M; g.N = (int)N; g.K = (int)K;
+    return bf16_tile(g, nullptr, g_tile_n.load(std::memory_order_relaxed));
+  }
+  GemmArgs g{};
+  g.M = (int)M; g.N = (int)N; g.K = (int)K;
+  g.d_is_fp32 = d_is_fp32 != 0;
+  return gemm_tile(g);
 }
 
 const char* nvfp4_status_string(nvfp4_status s) {

@@ -763,14 +763,12 @@ static cudaError_t launch_bf16_t(const DenseGemmArgs& g0, const DenseGemmArgs* g
             : launch_bf16_problems<BN, SPLIT, false>(g0, nullptr, max_pairs, s);
 }
 
-cudaError_t launch_gemm_bf16(const DenseGemmArgs& g0, const DenseGemmArgs* g1, cudaStream_t s) {
+int bf16_tile(const DenseGemmArgs& g0, const DenseGemmArgs* g1, int forced) {
   int num_sms = 0;
-  cudaError_t e = sm_count(&num_sms);
-  if (e != cudaSuccess) return e;
+  if (sm_count(&num_sms) != cudaSuccess) return kTilePair256;
   // 256 x 128 tiles while every one of them has a pair to itself: less to load per k-block and half the epilogue (1000 x
   // 2000 x 3000 22.9 -> 19.0 us, 512 x 4096 x 4096 24.2 -> 23.2, 512 x 1024 x 1024 9.1 -> 8.1).  Beyond one round they lose:
   // an instruction 128 columns wide takes as long as one 256 wide (264 x 7168 x 5120 30 -> 50 us).
-  const int pairs = num_sms / 2;
   const int64_t tiles128 = (int64_t)bf16_tiles(g0, 128) + (g1 ? bf16_tiles(*g1, 128) : 0);
   // Fewer tiles than clusters of several pairs: each tile's contraction is shared by two or four pairs, where what that saves
   // of the longest contraction (0.305 us per 64 deep) exceeds the exchange, 1.1 us (1.5 where most of the chip takes part) |
@@ -781,15 +779,26 @@ cudaError_t launch_gemm_bf16(const DenseGemmArgs& g0, const DenseGemmArgs* g1, c
     return resident_clusters<dense::gemm_bf16_pair_kernel<128, kSplit>, kSplit>(dense::kThreads,
                                                                              dense::Cfg<128, kSplit>::kSmemBytes);
   };
-  const int kb0 = (g0.K + 63) / 64, kb1 = g1 ? (g1->K + 63) / 64 : kb0, kb = kb0 > kb1 ? kb0 : kb1;
+  const int kb0 = (g0.K + 63) / 64, kb1 = g1 ? (g1->K + 63) / 64 : kb0, kb = std::max(kb0, kb1), least = std::min(kb0, kb1);
+  if ((forced == kTileSplit2 && least >= 2) || (forced == kTileSplit4 && least >= 4)) return forced;
   auto gain = [&](int split) {
     return 0.305 * (kb - (kb + split - 1) / split) - (split == 4 ? 1.6 : tiles128 > 16 ? 1.5 : 1.1);
   };
-  if (tiles128 <= 64 && (kb0 < kb1 ? kb0 : kb1) >= 4 && gain(2) > 0.2) {
-    if (gain(4) > gain(2) && tiles128 <= clusters(std::integral_constant<int, 4>())) return launch_bf16_t<128, 4>(g0, g1, pairs, s);
-    if (tiles128 <= clusters(std::integral_constant<int, 2>())) return launch_bf16_t<128, 2>(g0, g1, pairs, s);
+  if (tiles128 <= 64 && least >= 4 && gain(2) > 0.2) {
+    if (gain(4) > gain(2) && tiles128 <= clusters(std::integral_constant<int, 4>())) return kTileSplit4;
+    if (tiles128 <= clusters(std::integral_constant<int, 2>())) return kTileSplit2;
   }
-  return tiles128 <= pairs ? launch_bf16_t<128>(g0, g1, pairs, s) : launch_bf16_t<256>(g0, g1, pairs, s);
+  return tiles128 <= num_sms / 2 ? kTilePair128 : kTilePair256;
+}
+
+cudaError_t launch_gemm_bf16(const DenseGemmArgs& g0, const DenseGemmArgs* g1, int tile, cudaStream_t s) {
+  int num_sms = 0;
+  const cudaError_t e = sm_count(&num_sms);
+  if (e != cudaSuccess) return e;
+  const int pairs = num_sms / 2;
+  if (tile == kTileSplit4) return launch_bf16_t<128, 4>(g0, g1, pairs, s);
+  if (tile == kTileSplit2) return launch_bf16_t<128, 2>(g0, g1, pairs, s);
+  return tile == kTilePair128 ? launch_bf16_t<128>(g0, g1, pairs, s) : launch_bf16_t<256>(g0, g1, pairs, s);
 }
 
 // Test aid: one warp waits, with the given limit, on a barrier nobody arrives at.  The wait runs out, the code lands

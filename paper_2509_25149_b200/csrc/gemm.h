@@ -56,7 +56,8 @@ cudaError_t device_status_word(unsigned int** word);
 
 // BF16 GEMM D[M x N] = A B^T on CTA pairs (gemm_bf16.cuh) for layers kept in higher precision.
 // a_mn / b_mn = 0: the operand is stored [M or N][K] (contraction contiguous); 1: stored [K][M or N].
-// M, N, K multiples of 8 (tiles of 256 x 256 x 64 with zero-filled / clipped edges); leading dimensions in elements.
+// M, N, K multiples of 8 (tiles of 256 x 256 or 256 x 128, 64 deep, with zero-filled / clipped edges); leading dimensions in
+// elements.
 struct DenseGemmArgs {
   const void* a;
   const void* b;
@@ -67,6 +68,8 @@ struct DenseGemmArgs {
   int d_is_fp32, accumulate;
 };
 // g1 (may be NULL): a second, independent product in the same launch, its tiles after those of g0
-cudaError_t launch_gemm_bf16(const DenseGemmArgs& g0, const DenseGemmArgs* g1, cudaStream_t s);
+// The tile of such a launch: kTilePair256, kTilePair128 or a split one (`forced`, where every share has a k-block, or by size)
+int bf16_tile(const DenseGemmArgs& g0, const DenseGemmArgs* g1, int forced);
+cudaError_t launch_gemm_bf16(const DenseGemmArgs& g0, const DenseGemmArgs* g1, int tile, cudaStream_t s);
 
 }  // namespace nvfp4

@@ -54,7 +54,7 @@ cudaError_t launch_amax(const QuantArgs& a, bool has_row, bool has_col, bool rht
 cudaError_t launch_quantize(const QuantArgs& a, bool has_row, bool has_col, bool block2d, bool rht_row,
                             bool rht_col, bool sr, cudaStream_t s);
 // The copies of an activation (1x16 blocks, the transposed one, if wanted, with the 16-point transform) and of a weight (16x16
-// blocks), round-to-nearest, both passes of both in three launches
+// blocks), round-to-nearest, both passes of both: clearing the words, pass 1, pass 2, or the last two where pass 1 leaves parts
 cudaError_t launch_quantize_x_and_w(const QuantArgs& x, bool x_col, const QuantArgs& w, bool w_col, cudaStream_t s);
 // MXFP4 outputs (quantize_mx.cu): one pass, no tensor-level scale
 cudaError_t launch_quantize_mx(const QuantArgs& a, bool has_row, bool has_col, bool block2d, bool rht_col, bool sr,

@@ -51,7 +51,8 @@ def test_odd_multiples_of_128(shape, tile, fp32, fmt):
 @pytest.mark.parametrize("shape", [(256, 512, 256), (768, 1280, 1024)])
 @pytest.mark.parametrize("tile", [512, 640, 768])
 def test_layer_is_the_same_on_every_tile(shape, tile):
-    """Dgrad and Wgrad share a launch; the sums are exact enough that every tile gives the same bits here."""
+    """Dgrad and Wgrad share a launch: on every tile, forced or chosen by size, Y, dX and dW are the same up to the order of
+    FP32 sums (and a bf16 boundary crossed here and there): 5e-5 of their norm."""
     M, N, K = shape
     X, W = synth.normal_bf16((M, K), 1.0, 1).cuda(), synth.normal_bf16((N, K), 0.02, 2).cuda()
     dY = synth.normal_bf16((M, N), 1e-3, 3).cuda()

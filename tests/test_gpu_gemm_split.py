@@ -124,3 +124,60 @@ def test_backward_call_sums_as_its_products_do(size, tile, fmt):
     finally:
         B.nvfp4_set_gemm_tile_n(0)
     assert torch.equal(dx1, dx0) and torch.equal(dw1, dw0) and torch.equal(dx2, dx0) and torch.equal(dw2, dw0)
+
+
+# one k-block or an unequal number of them to a share, ragged in every direction, more clusters than are resident
+@pytest.mark.parametrize("shape", [(8, 8, 256), (264, 520, 328), (776, 264, 1000), (1032, 2056, 264)])
+@pytest.mark.parametrize("tile", [642, 644])
+def test_bf16_products_on_split_tiles(shape, tile):
+    """Both forms are forced: all four operand layouts, both outputs, accumulation, and two problems in one launch."""
+    M, N, K = shape
+    gen = torch.Generator("cuda").manual_seed(M + N + K)
+    a, b = (torch.randn(s, generator=gen, device="cuda").to(torch.bfloat16) for s in ((M, K), (N, K)))
+    want, T = a.double() @ b.double().T, a.double().abs() @ b.double().abs().T
+    B.nvfp4_set_gemm_tile_n(tile)
+    try:
+        assert B.nvfp4_gemm_tile(True, M, N, K, False) == tile
+        for layouts in ((0, 0), (0, 1), (1, 0), (1, 1)):
+            ops = [t.T.contiguous() if mn else t for t, mn in zip((a, b), layouts)]
+            for dtype in (torch.float32, torch.bfloat16):
+                wide = torch.full((M + 8, N + 8), 7.0, dtype=dtype, device="cuda")
+                D = wide[:M, :N]
+                B.nvfp4_gemm_bf16(*ops, D, *layouts)
+                B.nvfp4_device_status()
+                # K roundings of what the magnitudes add up to at most, and the rounding of the output
+                bound = K * 2.0 ** -23 * T + (2.0 ** -8 * want.abs() if dtype == torch.bfloat16 else 0)
+                assert torch.all((D.double() - want).abs() <= bound + 1e-30)
+                assert torch.all(wide[M:] == 7.0) and torch.all(wide[:, N:] == 7.0)
+                if dtype == torch.float32:
+                    once = D.clone()
+                    B.nvfp4_gemm_bf16(*ops, D, *layouts, accumulate=True)
+                    assert torch.equal(D, once + once)
+        # as a layer's backward call: dX = dY W and dW = dY^T X with dY [M x N], W [N x K], X [M x K], each as by itself
+        dy = want.to(torch.bfloat16)
+        dx, dw = torch.empty_like(a), torch.empty((N, K), device="cuda")
+        B.nvfp4_linear_bf16_bwd(dy, a, b, K, dx, dw, False)
+        if N > 192 and M > 192:  # (otherwise a share would be empty, and the call is not split)
+            one, two = torch.empty_like(dx), torch.empty_like(dw)
+            B.nvfp4_linear_bf16_bwd(dy, None, b, K, one, None, False)
+            B.nvfp4_linear_bf16_bwd(dy, a, None, K, None, two, False)
+            assert torch.equal(dx, one) and torch.equal(dw, two)
+        B.nvfp4_device_status()
+        T = dy.double().abs() @ b.double().abs()
+        assert torch.all((dx.double() - dy.double() @ b.double()).abs() <= N * 2.0 ** -23 * T + 2.0 ** -7 * T)
+        T = dy.double().abs().T @ a.double().abs()
+        assert torch.all((dw.double() - dy.double().T @ a.double()).abs() <= M * 2.0 ** -23 * T + 1e-30)
+    finally:
+        B.nvfp4_set_gemm_tile_n(0)
+
+
+def test_the_rule_splits_where_it_says():
+    """Few tiles and a long contraction, by size alone (any GPU keeps two clusters resident); short ones and many tiles stay whole."""
+    split = {642, 644}
+    for bf16, size, want in [(False, (256, 256, 5120), split), (False, (128, 128, 20480), split), (True, (256, 128, 4096), split),
+                             (True, (264, 128, 1032), split), (False, (256, 256, 1280), {640}), (True, (256, 128, 256), {640}),
+                             (False, (4096, 4096, 4096), {512, 640, 768}), (True, (4096, 4096, 4096), {512})]:
+        for fp32 in (False, True):
+            assert B.nvfp4_gemm_tile(bf16, *size, fp32) in want, (bf16, size)
+    for bf16, size in [(False, (64, 128, 256)), (False, (128, 128, 128)), (True, (4, 8, 8)), (True, (8, 8, 0))]:
+        assert B.nvfp4_gemm_tile(bf16, *size, False) == -1
