@@ -370,8 +370,9 @@ __device__ __forceinline__ float encode_scale_of_byte(uint32_t byte, float s_dec
   return (byte == 0u) ? 0.0f : fminf(__frcp_rn(d), kFltMax);
 }
 
+// OWN_DRAWS: 16x16 blocks whose transposed copy is rounded with draws of its own.
 template <bool HAS_ROW, bool HAS_COL, bool BLOCK2D, bool RHT_ROW, bool RHT_COL, bool SR, int TC, bool F32 = false,
-          bool PARTS = false>
+          bool PARTS = false, bool OWN_DRAWS = false>
 __device__ __forceinline__ void quantize_tiles(const CUtensorMap* src_map, const QuantArgs& a, const int block,
                                                const int blocks) {  // this CTA among those of the tensor
   using S = QuantSmem<TC, F32>;
@@ -385,7 +386,7 @@ __device__ __forceinline__ void quantize_tiles(const CUtensorMap* src_map, const
   const int n_rb = (int)(a.rows >> 4);  // 16-blocks per source column
   // 16x16 blocks with both copies requested: the transposed copy holds the very codes of the row-wise one
   // (Section 4.3), so it is made by transposing nibbles; the raw tile is not needed a second time
-  constexpr bool kNibbleTranspose = BLOCK2D && HAS_ROW && HAS_COL;
+  constexpr bool kNibbleTranspose = BLOCK2D && HAS_ROW && HAS_COL && !OWN_DRAWS;
   volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(smem + S::kBars + 16);
   const uint32_t bar0 = smem_u32(smem + S::kBars), tile0 = smem_u32(smem + S::kTile);
 
@@ -795,10 +796,11 @@ __device__ __forceinline__ void quantize_tiles(const CUtensorMap* src_map, const
 }
 
 template <bool HAS_ROW, bool HAS_COL, bool BLOCK2D, bool RHT_ROW, bool RHT_COL, bool SR, int TC, bool F32 = false,
-          bool PARTS = false>
+          bool PARTS = false, bool OWN_DRAWS = false>
 __global__ void __launch_bounds__(256, 2) quantize_kernel(const __grid_constant__ CUtensorMap src_map,
                                                           const __grid_constant__ QuantArgs a) {
-  quantize_tiles<HAS_ROW, HAS_COL, BLOCK2D, RHT_ROW, RHT_COL, SR, TC, F32, PARTS>(&src_map, a, (int)blockIdx.x, (int)gridDim.x);
+  quantize_tiles<HAS_ROW, HAS_COL, BLOCK2D, RHT_ROW, RHT_COL, SR, TC, F32, PARTS, OWN_DRAWS>(&src_map, a, (int)blockIdx.x,
+                                                                                            (int)gridDim.x);
 }
 
 // The activation (1x16 blocks, the transposed copy with the transform) and the weight (16x16 blocks) of a forward call in one
@@ -1004,12 +1006,12 @@ static bool quant_source_map(CUtensorMap* map, const QuantArgs& a, int tc, bool 
                      (uint64_t)a.cols, (uint64_t)a.rows, (uint64_t)a.ld * (f32 ? 4 : 2), tc, 128, false);
 }
 
-template <bool HR, bool HC, bool B2, bool RR, bool RC, bool SR, int TC, bool F32 = false, bool PARTS = false>
+template <bool HR, bool HC, bool B2, bool RR, bool RC, bool SR, int TC, bool F32 = false, bool PARTS = false, bool OWN = false>
 static cudaError_t launch_quant_tc(const QuantArgs& a_in, int slots, cudaStream_t s) {
-  auto kern = quantize_kernel<HR, HC, B2, RR, RC, SR, TC, F32, PARTS>;
+  auto kern = quantize_kernel<HR, HC, B2, RR, RC, SR, TC, F32, PARTS, OWN>;
   QuantArgs a = a_in;
   a.tiles_c = (int)((a.cols + TC - 1) / TC);
-  constexpr bool kRowCodes = B2 && HR && HC;
+  constexpr bool kRowCodes = B2 && HR && HC && !OWN;
   constexpr int smem = QuantSmem<TC, F32>::bytes(SR && HC && !kRowCodes, kRowCodes);
   CUtensorMap map;
   if (!quant_source_map(&map, a, TC, F32)) return cudaErrorInvalidValue;
@@ -1158,13 +1160,11 @@ cudaError_t launch_amax_f32(const QuantArgs& a, bool has_row, bool has_col, cuda
 // binary32 source (Appendix B names FP32 as well as BF16 as the precision converted from), e.g. weights quantized straight from
 // their FP32 master copy; no transform (the recipe transforms activations and gradients, which are bf16)
 cudaError_t launch_quantize_f32(const QuantArgs& a, bool has_row, bool has_col, bool block2d, bool sr, cudaStream_t s) {
-  if (block2d && sr && has_row && has_col && a.off_hi_col != a.off_hi) {  // independent draws: the copies' codes differ
-    const cudaError_t e = launch_quantize_f32(a, true, false, true, true, s);
-    return e != cudaSuccess ? e : launch_quantize_f32(a, false, true, true, true, s);
-  }
   int sms = 0;
   const cudaError_t e = sm_count(&sms);
   if (e != cudaSuccess) return e;
+  if (block2d && sr && has_row && has_col && a.off_hi_col != a.off_hi)  // independent draws: the copies' codes differ
+    return launch_quant_tc<true, true, true, false, false, true, 64, true, false, true>(a, 2 * sms, s);
 #define NVFP4_F32Q(HR, HC, B2, SRV)                                              \
   if (has_row == HR && has_col == HC && block2d == B2 && sr == SRV)              \
     return launch_quant_tc<HR, HC, B2, false, false, SRV, 64, true>(a, 2 * sms, s);

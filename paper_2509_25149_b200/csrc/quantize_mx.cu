@@ -60,16 +60,16 @@ constexpr float kInvSqrt32 = 0.176776695296636893f;  // fl(1 / sqrt(32))
 //   phase 2  each thread owns 32 rows x 2 columns of the tile and produces the transposed copy: a pair of warps reads what
 //            the same pair staged, so the 64 threads meet at a barrier of their own;
 //   phase 3  staged codes and scale bytes leave with 16-byte stores (staging double buffered: one CTA barrier per tile).
-template <bool HAS_ROW, bool HAS_COL, bool BLOCK2D, bool RHT_COL, bool SR>
+// OWN_DRAWS: 32x32 blocks whose transposed copy is rounded with draws of its own.
+template <bool HAS_ROW, bool HAS_COL, bool BLOCK2D, bool RHT_COL, bool SR, bool OWN_DRAWS>
 __global__ void __launch_bounds__(256, 2) quantize_mx_kernel(const __grid_constant__ CUtensorMap src_map,
                                                              const QuantArgs a) {
   using S = MxSmem;
   extern __shared__ __align__(128) uint8_t smem[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t n_cb = a.cols >> 4;  // 16-chunks per source row (index of the random draws)
-  // 32x32 blocks with both copies requested: the transposed copy holds the very codes of the row-wise one (with draws of its
-  // own it is made by a launch of its own, see launch_quantize_mx)
-  constexpr bool kNibbleTranspose = BLOCK2D && HAS_ROW && HAS_COL;
+  // 32x32 blocks with both copies requested: the transposed copy holds the very codes of the row-wise one
+  constexpr bool kNibbleTranspose = BLOCK2D && HAS_ROW && HAS_COL && !OWN_DRAWS;
   constexpr bool kStageRand = SR && HAS_COL && !kNibbleTranspose;
   volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(smem + S::kBars + 16);
   const uint32_t bar0 = smem_u32(smem + S::kBars), tile0 = smem_u32(smem + S::kTile);
@@ -319,10 +319,10 @@ __global__ void __launch_bounds__(256, 2) quantize_mx_kernel(const __grid_consta
   }
 }
 
-template <bool HR, bool HC, bool B2, bool RC, bool SR>
+template <bool HR, bool HC, bool B2, bool RC, bool SR, bool OWN = false>
 static cudaError_t launch_mx_t(const QuantArgs& a, cudaStream_t s) {
-  auto kern = quantize_mx_kernel<HR, HC, B2, RC, SR>;
-  constexpr bool kRowCodes = B2 && HR && HC;
+  auto kern = quantize_mx_kernel<HR, HC, B2, RC, SR, OWN>;
+  constexpr bool kRowCodes = B2 && HR && HC && !OWN;
   constexpr int smem = MxSmem::bytes(SR && HC && !kRowCodes, kRowCodes);
   CUtensorMap map;
   if (!make_map_2d(&map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, a.x, (uint64_t)a.cols, (uint64_t)a.rows,
@@ -345,10 +345,8 @@ static cudaError_t launch_mx_t(const QuantArgs& a, cudaStream_t s) {
 cudaError_t launch_quantize_mx(const QuantArgs& a, bool has_row, bool has_col, bool block2d, bool rht_col, bool sr,
                                cudaStream_t s) {
   rht_col = rht_col && has_col;
-  if (block2d && sr && has_row && has_col && a.off_hi_col != a.off_hi) {  // independent draws: the copies' codes differ
-    const cudaError_t e = launch_quantize_mx(a, true, false, true, false, true, s);
-    return e != cudaSuccess ? e : launch_quantize_mx(a, false, true, true, false, true, s);
-  }
+  if (block2d && sr && has_row && has_col && a.off_hi_col != a.off_hi)  // independent draws: the copies' codes differ
+    return launch_mx_t<true, true, true, false, true, true>(a, s);
 #define NVFP4_MXQ(HR, HC, B2, RC, SRV)                                                        \
   if (has_row == HR && has_col == HC && block2d == B2 && rht_col == RC && sr == SRV)         \
     return launch_mx_t<HR, HC, B2, RC, SRV>(a, s);
