@@ -112,6 +112,28 @@ def test_quantize_1x32_is_bit_exact(shape, which, rounding):
         P.assert_exact_mx(col, oracle.quantize_mx(synth.bits(x), colwise=True, **kw), f"col {shape}")
 
 
+# 144, 160, 272 | 306 and 450 tiles: one, two, three CTAs per SM of 148, and more tiles than CTAs
+@pytest.mark.parametrize("shape", [(2048, 1152), (2048, 1280), (2176, 2048), (2176, 2304), (1280, 5760)])
+@pytest.mark.parametrize("which", ["row", "both"])
+def test_every_way_the_tiles_are_spread(shape, which):
+    """The calls behind one another start while the one before drains."""
+    x = synth.normal_with_outliers_bf16(shape, 0.01, 50.0, shape[1], 3)
+    xd = x.cuda()
+    opts = B.quant_opts(rounding=B.ROUND_STOCHASTIC, seed=7, sr_offset=3)
+    rows = [B.alloc_tensor(*shape, format=B.FORMAT_MXFP4) for _ in range(4)]
+    cols = [B.alloc_tensor(*shape[::-1], format=B.FORMAT_MXFP4) if which == "both" else None for _ in range(4)]
+    for row, col in zip(rows, cols):
+        B.nvfp4_quantize(xd, opts, row, col)
+    B.nvfp4_device_status()
+    kw = dict(rounding=oracle.SR, seed=7, sr_offset=3)
+    want = oracle.quantize_mx(synth.bits(x), **kw)
+    want_col = oracle.quantize_mx(synth.bits(x), colwise=True, **kw)
+    for row, col in zip(rows, cols):
+        P.assert_exact_mx(row, want, "row")
+        if col is not None:
+            P.assert_exact_mx(col, want_col, "col")
+
+
 @pytest.mark.parametrize("shape", [(128, 128), (256, 384), (160, 224)])
 @pytest.mark.parametrize("rounding", [B.ROUND_NEAREST_EVEN, B.ROUND_STOCHASTIC])
 def test_quantize_32x32_weights_bit_exact_and_consistent(shape, rounding):
