@@ -36,23 +36,26 @@ __device__ __forceinline__ void fwht32_pairs(float2 v[32]) {
   }
 }
 
+// COL: the transposed copy is made
+template <bool COL>
 struct MxSmem {
   static constexpr int kTileBytes = 32768;
   static constexpr int kTile = 0;                       // 2 x (128 rows x 256 B of bf16), filled by TMA
   static constexpr int kColCodes = 2 * kTileBytes;      // 2 x (64 column pairs x 128 B)
-  static constexpr int kSfRow = kColCodes + 2 * 8192;   // 2 x one 512-byte atom: 128 rows x 4 blocks of 32
+  static constexpr int kSfRow = kColCodes + (COL ? 2 * 8192 : 0);  // 2 x one 512-byte atom: 128 rows x 4 blocks of 32
   static constexpr int kSfCol = kSfRow + 2 * 512;
-  static constexpr int kBlk = kSfCol + 2 * 512;         // 32x32 mode: amax of (warp's 16 rows) x (4 column blocks)
+  static constexpr int kBlk = kSfCol + (COL ? 2 * 512 : 0);  // 32x32 mode: amax of (warp's 16 rows) x (4 column blocks)
   static constexpr int kBlkByte = kBlk + 128;           // 32x32 mode: scale byte by (32-row group, column block)
   static constexpr int kBars = kBlkByte + 32;           // two "tile landed" barriers, then the abort word
   static constexpr int kRand = kBars + 32;              // 128 rows x 128 B of complemented draws (stochastic rounding),
                                                         // or 128 rows x 64 B of row-wise codes (32x32, both copies)
   static constexpr int bytes(bool rand, bool row_codes) { return kRand + (rand ? 16384 : row_codes ? 8192 : 0); }
+  static constexpr int kCtas = COL ? 2 : 3;             // resident per SM (the row-wise copy alone stages no codes)
 };
 
 constexpr float kInvSqrt32 = 0.176776695296636893f;  // fl(1 / sqrt(32))
 
-// Persistent CTAs (two per SM) going through 128 x 128 tiles of the source that arrive by TMA in a ring of two buffers, as
+// Persistent CTAs (two per SM, three for the row-wise copy alone) going through 128 x 128 tiles of the source that arrive by TMA in a ring of two buffers, as
 // in quantize_kernel; bound by instruction issue.  One CTA per tile, each loading its own registers and waiting for them,
 // took 45 us for a 8192 x 5120 activation, 80 us for a 8192 x 7168 gradient and 27 us for a 7168 x 5120 weight.
 //   phase 1  each thread owns four 1x16 chunks of the tile; a 1x32 block is the two chunks of an even / odd lane pair;
@@ -62,9 +65,9 @@ constexpr float kInvSqrt32 = 0.176776695296636893f;  // fl(1 / sqrt(32))
 //   phase 3  staged codes and scale bytes leave with 16-byte stores (staging double buffered: one CTA barrier per tile).
 // OWN_DRAWS: 32x32 blocks whose transposed copy is rounded with draws of its own.
 template <bool HAS_ROW, bool HAS_COL, bool BLOCK2D, bool RHT_COL, bool SR, bool OWN_DRAWS>
-__global__ void __launch_bounds__(256, 2) quantize_mx_kernel(const __grid_constant__ CUtensorMap src_map,
-                                                             const QuantArgs a) {
-  using S = MxSmem;
+__global__ void __launch_bounds__(256, MxSmem<HAS_COL>::kCtas)
+    quantize_mx_kernel(const __grid_constant__ CUtensorMap src_map, const QuantArgs a) {
+  using S = MxSmem<HAS_COL>;
   extern __shared__ __align__(128) uint8_t smem[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t n_cb = a.cols >> 4;  // 16-chunks per source row (index of the random draws)
@@ -319,14 +322,14 @@ __global__ void __launch_bounds__(256, 2) quantize_mx_kernel(const __grid_consta
   }
 }
 
-// just more dynamic shared memory than two CTAs of an SM (228 KB, 1 KB of it taken per CTA) can have
-constexpr int kSmemOfHalf = 116 * 1024;
+// just more dynamic shared memory than two | three CTAs of an SM (228 KB, 1 KB of it taken per CTA) can have
+constexpr int kSmemOfHalf = 116 * 1024, kSmemOfThird = 76 * 1024;
 
 template <bool HR, bool HC, bool B2, bool RC, bool SR, bool OWN = false>
 static cudaError_t launch_mx_t(const QuantArgs& a, cudaStream_t s) {
   auto kern = quantize_mx_kernel<HR, HC, B2, RC, SR, OWN>;
   constexpr bool kRowCodes = B2 && HR && HC && !OWN;
-  constexpr int smem = MxSmem::bytes(SR && HC && !kRowCodes, kRowCodes);
+  constexpr int smem = MxSmem<HC>::bytes(SR && HC && !kRowCodes, kRowCodes);
   CUtensorMap map;
   if (!make_map_2d(&map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, a.x, (uint64_t)a.cols, (uint64_t)a.rows,
                    (uint64_t)a.ld * 2, 128, 128, 0))
@@ -342,11 +345,14 @@ static cudaError_t launch_mx_t(const QuantArgs& a, cudaStream_t s) {
     device_configured(configured, dev);
   }
   const int64_t tiles = (int64_t)a.tiles_r * a.tiles_c;
+  // Resident CTAs.  Row-wise copy alone, two / three per SM: gradient of 1024 x 6784 (424 tiles) 6.4 / 5.3 us, activation of 8192 x
+  // 5120 17.1 / 16.4; 256 tiles are best off with two (gradient of 2048 x 2048 4.0 / 5.0).
+  const int slots = MxSmem<HC>::kCtas * sms;
   // The kernel becomes resident while the one before it drains, and few CTAs would crowd on the SMs that drain first: no more
-  // on an SM than the tiles take when they are spread evenly (the shared memory that is left keeps others out).  Backward call
-  // of 1024 x 2304 x 2560 19.4 -> 18.0 us, 3584 x 256 x 4352 22.9 -> 21.1, in a loop of such calls.
-  const int room = tiles <= sms ? kSmemOfHalf : 0;
-  e = launch_kernel(kern, dim3((unsigned)(tiles < 2 * sms ? tiles : 2 * sms)), dim3(256), room > smem ? room : smem, s, map, a);
+  // on an SM than the tiles take when they are spread evenly (the shared memory that is left keeps others out).  Backward call of
+  // 1024 x 2304 x 2560 19.4 -> 18.0 us, 3584 x 256 x 4352 22.9 -> 21.1, in a loop of such calls.
+  const int room = tiles <= sms ? kSmemOfHalf : tiles <= 2 * sms ? kSmemOfThird : 0;
+  e = launch_kernel(kern, dim3((unsigned)(tiles < slots ? tiles : slots)), dim3(256), room > smem ? room : smem, s, map, a);
   count_launch();
   return e;
 }
