@@ -229,25 +229,11 @@ __global__ void __launch_bounds__(256, MxSmem<HAS_COL>::kCtas)
         else
           am2 = amax_pairs(v);
         // Section 5, transform size 32: y = fl(sum * c), c = fl(1 / sqrt(32)).  Rounding is monotone, so the block's amax is
-        // fl(max |sum| * c); the encode scale is a power of two, so fl(y * enc) = fl(sum * (c * enc)) and y need not be formed.
-        // That holds while both are normal numbers.  y is subnormal for 724 sums of bf16 values alone, and none of them gets
-        // another code at any scale or draw; c * enc is so where a sum has overflowed: there y is formed.  (The branch costs
-        // 0.5 of 30 us, 8192 x 5120 rounded to nearest.)
-        if (RHT_COL) {
-          const bool overflow = fmaxf(am2.x, am2.y) > kFltMax;
-          if (overflow) {
-#pragma unroll
-            for (int k = 0; k < 32; ++k) v[k] = mul2(v[k], make_float2(kInvSqrt32, kInvSqrt32));
-          }
-          am2 = mul2(am2, make_float2(kInvSqrt32, kInvSqrt32));
-          mx_scales(am2.x, byte0, enc.x);
-          mx_scales(am2.y, byte1, enc.y);
-          const float left = overflow ? 1.0f : kInvSqrt32;
-          enc = mul2(enc, make_float2(left, left));
-        } else {
-          mx_scales(am2.x, byte0, enc.x);
-          mx_scales(am2.y, byte1, enc.y);
-        }
+        // fl(max |sum| * c); the encode scale is a power of two, so fl(y * enc) = fl(sum * (c * enc)): y is never formed.
+        if (RHT_COL) am2 = mul2(am2, make_float2(kInvSqrt32, kInvSqrt32));
+        mx_scales(am2.x, byte0, enc.x);
+        mx_scales(am2.y, byte1, enc.y);
+        if (RHT_COL) enc = mul2(enc, make_float2(kInvSqrt32, kInvSqrt32));
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
           uint2 c0, c1;
