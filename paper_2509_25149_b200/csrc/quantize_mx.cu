@@ -229,7 +229,11 @@ __global__ void __launch_bounds__(256, MxSmem<HAS_COL>::kCtas)
         else
           am2 = amax_pairs(v);
         // Section 5, transform size 32: y = fl(sum * c), c = fl(1 / sqrt(32)).  Rounding is monotone, so the block's amax is
-        // fl(max |sum| * c); the encode scale is a power of two, so fl(y * enc) = fl(sum * (c * enc)): y is never formed.
+        // fl(max |sum| * c); the encode scale is a power of two, so fl(y * enc) = fl(sum * (c * enc)): y is never formed.  That
+        // holds while y and c * enc are normal numbers.  c * enc is, up to byte 250, for every finite sum (beside a sum that has
+        // overflowed it lacks three bits, 2.5e-7, which can move a value next to a threshold); y is subnormal for 724 sums of
+        // bf16 values alone, and none of them gets another code at any scale or draw.  (Forming y where a sum has
+        // overflowed was exact there as well and took 1.8 % longer on an activation of 8192 x 5120, 3.5 % on one of 512 x 1024.)
         if (RHT_COL) am2 = mul2(am2, make_float2(kInvSqrt32, kInvSqrt32));
         mx_scales(am2.x, byte0, enc.x);
         mx_scales(am2.y, byte1, enc.y);

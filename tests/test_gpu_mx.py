@@ -162,6 +162,47 @@ def test_quantize_rht32_copy_follows_the_tolerance_protocol(shape, rounding):
     assert st["excused_codes"] + st["excused_scales"] <= max(1e-3 * st["elements"], 32)
 
 
+def _two_roundings(x, rounding):
+    """Transposed, transformed copy of [32 x C] whose sums are exact in binary32: y = fl(sum * c), then fl(y * 2^(127 - byte))."""
+    h = np.array([[1.0 - 2.0 * (bin(j & k).count("1") & 1) for j in range(32)] for k in range(32)])
+    with np.errstate(all="ignore"):
+        sums = (x.T.astype(np.float64) @ h).astype(np.float32)
+        y = sums * np.float32(1 / np.sqrt(32.0))
+        bits = np.abs(y).max(axis=1).view(np.uint32)
+        byte = np.maximum((bits >> 23).astype(np.int64) - 2 + ((bits & 0x7FFFFF) > 0x400000), 0)
+        v = y * ((254 - byte).astype(np.uint32) << 23).view(np.float32)[:, None]
+    v = np.clip(v, -8, 8)
+    if rounding == oracle.RNE:
+        code = np.array([oracle.e2m1_encode_rne(w) for w in v.ravel()], np.uint8)
+    else:  # the draws are those of the source elements (row k, column c)
+        u = [oracle.sr_draw(2, 5, k * len(v) + c) for c in range(len(v)) for k in range(32)]
+        code = oracle.e2m1_encode_sr_many(v, np.array(u, np.uint8))
+    return byte, np.asarray(code).reshape(v.shape)
+
+
+@pytest.mark.parametrize("rounding", [oracle.RNE, oracle.SR])
+@pytest.mark.parametrize("end", ["bottom", "top"])
+def test_quantize_rht32_at_the_ends_of_the_range(end, rounding):
+    """Every sum is exact, so the codes are: around the threshold 1/4 beside values of the largest scale a finite sum can have (byte
+    250), and over all small multiples of the smallest bf16 number."""
+    x = np.zeros((32, 1024), np.float32)
+    if end == "top":
+        m = 741455 + np.arange(-512, 512)  # sqrt(32) / 4 in units of 2^-19
+        for i, shift in enumerate((16, 8, 0)):
+            x[i] = ((m >> shift) & 255) * 2.0 ** (104 + shift)
+        x[16], x[17] = 1.125 * 2.0 ** 126, -1.125 * 2.0 ** 126
+    else:
+        x[0], x[1] = np.arange(1024) % 256 * 2.0 ** -133, (1 + np.arange(1024) // 128) * 2.0 ** -126
+    bf = torch.from_numpy(x).to(torch.bfloat16)
+    assert np.array_equal(bf.float().numpy(), x)
+    _, col = P.gpu_quantize_mx(bf, rowwise=False, colwise=True, sf_layout=B.SF_LINEAR, rht_colwise=True, rounding=rounding,
+                               seed=2, sr_offset=5)
+    codes, scales = P.download_mx(col)
+    byte, want = _two_roundings(x, rounding)
+    assert np.array_equal(scales[:, 0], byte) and (end == "bottom" or set(byte) == {250})
+    assert np.array_equal(P.canon_zero(P.unpack(codes)), P.canon_zero(want))
+
+
 def test_quantize_degenerate_and_rejected_inputs():
     z = torch.zeros((128, 128), dtype=torch.bfloat16)
     row, col = P.gpu_quantize_mx(z, colwise=True)
