@@ -50,12 +50,11 @@ struct MxSmem {
   static constexpr int kRand = kBars + 32;              // 128 rows x 128 B of complemented draws (stochastic rounding),
                                                         // or 128 rows x 64 B of row-wise codes (32x32, both copies)
   static constexpr int bytes(bool rand, bool row_codes) { return kRand + (rand ? 16384 : row_codes ? 8192 : 0); }
-  static constexpr int kCtas = COL ? 2 : 3;             // resident per SM (the row-wise copy alone stages no codes)
 };
 
 constexpr float kInvSqrt32 = 0.176776695296636893f;  // fl(1 / sqrt(32))
 
-// Persistent CTAs (two per SM, three for the row-wise copy alone) going through 128 x 128 tiles of the source that arrive by TMA in a ring of two buffers, as
+// Persistent CTAs (CTAS per SM: two, or three for the row-wise copy alone) going through 128 x 128 tiles of the source that arrive by TMA in a ring of two buffers, as
 // in quantize_kernel; bound by instruction issue.  One CTA per tile, each loading its own registers and waiting for them,
 // took 45 us for a 8192 x 5120 activation, 80 us for a 8192 x 7168 gradient and 27 us for a 7168 x 5120 weight.
 //   phase 1  each thread owns four 1x16 chunks of the tile; a 1x32 block is the two chunks of an even / odd lane pair;
@@ -64,8 +63,8 @@ constexpr float kInvSqrt32 = 0.176776695296636893f;  // fl(1 / sqrt(32))
 //            the same pair staged, so the 64 threads meet at a barrier of their own;
 //   phase 3  staged codes and scale bytes leave with 16-byte stores (staging double buffered: one CTA barrier per tile).
 // OWN_DRAWS: 32x32 blocks whose transposed copy is rounded with draws of its own.
-template <bool HAS_ROW, bool HAS_COL, bool BLOCK2D, bool RHT_COL, bool SR, bool OWN_DRAWS>
-__global__ void __launch_bounds__(256, MxSmem<HAS_COL>::kCtas)
+template <bool HAS_ROW, bool HAS_COL, bool BLOCK2D, bool RHT_COL, bool SR, bool OWN_DRAWS, int CTAS>
+__global__ void __launch_bounds__(256, CTAS)
     quantize_mx_kernel(const __grid_constant__ CUtensorMap src_map, const QuantArgs a) {
   using S = MxSmem<HAS_COL>;
   extern __shared__ __align__(128) uint8_t smem[];
@@ -315,9 +314,9 @@ __global__ void __launch_bounds__(256, MxSmem<HAS_COL>::kCtas)
 // just more dynamic shared memory than two | three CTAs of an SM (228 KB, 1 KB of it taken per CTA) can have
 constexpr int kSmemOfHalf = 116 * 1024, kSmemOfThird = 76 * 1024;
 
-template <bool HR, bool HC, bool B2, bool RC, bool SR, bool OWN = false>
-static cudaError_t launch_mx_t(const QuantArgs& a, cudaStream_t s) {
-  auto kern = quantize_mx_kernel<HR, HC, B2, RC, SR, OWN>;
+template <bool HR, bool HC, bool B2, bool RC, bool SR, bool OWN, int CTAS>
+static cudaError_t launch_mx_ctas(const QuantArgs& a, int sms, cudaStream_t s) {
+  auto kern = quantize_mx_kernel<HR, HC, B2, RC, SR, OWN, CTAS>;
   constexpr bool kRowCodes = B2 && HR && HC && !OWN;
   constexpr int smem = MxSmem<HC>::bytes(SR && HC && !kRowCodes, kRowCodes);
   CUtensorMap map;
@@ -325,9 +324,8 @@ static cudaError_t launch_mx_t(const QuantArgs& a, cudaStream_t s) {
                    (uint64_t)a.ld * 2, 128, 128, 0))
     return cudaErrorInvalidValue;
   static std::atomic<uint64_t> configured{0};  // per call site (template instantiation) and device
-  int dev, sms = 0;
-  cudaError_t e = sm_count(&sms);
-  if (e != cudaSuccess) return e;
+  int dev;
+  cudaError_t e;
   if (device_needs_config(configured, &dev)) {
     if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem > kSmemOfHalf ? smem : kSmemOfHalf)) !=
         cudaSuccess)
@@ -335,16 +333,30 @@ static cudaError_t launch_mx_t(const QuantArgs& a, cudaStream_t s) {
     device_configured(configured, dev);
   }
   const int64_t tiles = (int64_t)a.tiles_r * a.tiles_c;
-  // Resident CTAs.  Row-wise copy alone, two / three per SM: gradient of 1024 x 6784 (424 tiles) 6.4 / 5.3 us, activation of 8192 x
-  // 5120 17.1 / 16.4; 256 tiles are best off with two (gradient of 2048 x 2048 4.0 / 5.0).
-  const int slots = MxSmem<HC>::kCtas * sms;
+  const int slots = CTAS * sms;
   // The kernel becomes resident while the one before it drains, and few CTAs would crowd on the SMs that drain first: no more
   // on an SM than the tiles take when they are spread evenly (the shared memory that is left keeps others out).  Backward call of
   // 1024 x 2304 x 2560 19.4 -> 18.0 us, 3584 x 256 x 4352 22.9 -> 21.1, in a loop of such calls.
-  const int room = tiles <= sms ? kSmemOfHalf : tiles <= 2 * sms ? kSmemOfThird : 0;
+  const int room = tiles <= sms ? kSmemOfHalf : CTAS == 2 ? kSmemOfThird : 0;
   e = launch_kernel(kern, dim3((unsigned)(tiles < slots ? tiles : slots)), dim3(256), room > smem ? room : smem, s, map, a);
   count_launch();
   return e;
+}
+
+template <bool HR, bool HC, bool B2, bool RC, bool SR, bool OWN = false>
+static cudaError_t launch_mx_t(const QuantArgs& a, cudaStream_t s) {
+  int sms = 0;
+  const cudaError_t e = sm_count(&sms);
+  if (e != cudaSuccess) return e;
+  // Without a transposed copy three CTAs fit an SM; they take 1.5 times as long for a round of tiles as two, so they pay where that many
+  // rounds go: 297 to 444 tiles above all (two / three per SM: gradient of 1024 x 6784 6.4 / 5.3 us, activation of 896 x 7936 4.3 /
+  // 3.6; but gradient of 2048 x 2048 4.0 / 5.0, 11680 x 896 8.2 / 9.3).
+  if constexpr (!HC) {
+    const int64_t tiles = (int64_t)a.tiles_r * a.tiles_c;
+    if (3 * ((tiles + 3 * sms - 1) / (3 * sms)) < 2 * ((tiles + 2 * sms - 1) / (2 * sms)))
+      return launch_mx_ctas<HR, HC, B2, RC, SR, OWN, 3>(a, sms, s);
+  }
+  return launch_mx_ctas<HR, HC, B2, RC, SR, OWN, 2>(a, sms, s);
 }
 
 cudaError_t launch_quantize_mx(const QuantArgs& a, bool has_row, bool has_col, bool block2d, bool rht_col, bool sr,
