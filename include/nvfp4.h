@@ -155,7 +155,8 @@ NVFP4_API nvfp4_status nvfp4_quantize(const void* x_bf16, int64_t rows, int64_t 
  * nvfp4_gemm -- Eq. 5: D[i][j] = s_dec^A * s_dec^B * sum_blocks S^A[i,b] S^B[j,b] sum_{k in b} a[i,k] b[j,k]
  *   A [M x K], B [N x K]: quantized copies whose columns are the contraction dimension, scales in
  *   the NVFP4_SF_SWIZZLED layout, M % 128 == 0, N % 128 == 0, K % 256 == 0 (K = A->cols = B->cols).
- *   Runs on CTA pairs with 256 x 128, 256 x 256 or 256 x 384 tiles, whichever schedule is estimated shorter.
+ *   Runs on CTA pairs with 256 x 128, 256 x 256 or 256 x 384 tiles, or on single CTAs with 128 x 128 tiles, whichever schedule is
+ *   estimated shorter.
  *   D: device, row-major [M x N] with leading dimension ldd (elements, >= N, ldd*elemsize % 16 == 0),
  *   bf16 (round-to-nearest-even) when d_is_fp32 == 0, else fp32.  Partial sums are accumulated in
  *   FP32 by the tensor cores; the product of the two tensor decode scales is applied once at the end.
@@ -335,14 +336,14 @@ NVFP4_API nvfp4_status nvfp4_test_cluster_leave(uint64_t delay_ns, uint64_t* tim
  * up to two 256-wide ones per row of tiles (needs N >= 256, otherwise as 512); 642 / 644 = 256 x 128 tiles whose
  * contraction two / four CTA pairs share (K >= 512 / 1024, otherwise as 640; two products in one launch: as 640, summed in
  * the same order); these two are heeded by BF16 products as well (K > 64 / 192, otherwise by size), the others are not;
- * 0 = choose by shape (the CTA-pair tile whose static schedule is estimated shortest; whether a contraction is
+ * 0 = choose by shape (the tile whose static schedule is estimated shortest; whether a contraction is
  * shared, and so the order of the FP32 sums, also depends on how many such clusters the GPU keeps resident).
  * Returns 0, or -1 for any other value.  Process-wide; results do not depend on it
  * beyond FP32 summation order. */
 NVFP4_API int32_t nvfp4_set_gemm_tile_n(int32_t tile_n);
 
-/* The tile (a value of nvfp4_set_gemm_tile_n) of one M x N x K product with a launch to itself on the current device: nvfp4_gemm,
- * or nvfp4_gemm_bf16 when bf16 != 0.  -1 for a size that the call would refuse.  Launches nothing. */
+/* The tile (a value of nvfp4_set_gemm_tile_n) of one M x N x K product with a launch to itself on the current device: nvfp4_gemm
+ * (NVFP4, D written), or nvfp4_gemm_bf16 when bf16 != 0.  -1 for a size that the call would refuse.  Launches nothing. */
 NVFP4_API int32_t nvfp4_gemm_tile(int32_t bf16, int64_t M, int64_t N, int64_t K, int32_t d_is_fp32);
 
 /*

@@ -215,10 +215,10 @@ nvfp4_status gemm_prepare(const nvfp4_tensor* A, const nvfp4_tensor* B, void* D,
   return NVFP4_OK;
 }
 
-// The tile of a launch: the caller's (nvfp4_set_gemm_tile_n), or the CTA-pair tile with the shortest estimated schedule
+// The tile of a launch: the caller's (nvfp4_set_gemm_tile_n), or the one with the shortest estimated schedule
 int gemm_tile(const GemmArgs& g0, const GemmArgs* g1 = nullptr) {
   const int forced = g_tile_n.load(std::memory_order_relaxed);
-  return forced ? forced : best_pair_tile(g0, g1);
+  return forced ? forced : best_tile(g0, g1);
 }
 
 nvfp4_status gemm_impl(const nvfp4_tensor* A, const nvfp4_tensor* B, void* D, int32_t d_is_fp32, int64_t ldd,

@@ -12,8 +12,8 @@
 // Every wait is bounded: when one expires the kernel records a code in a device status word, every role
 // leaves its loop, tensor memory is released and the kernel returns.
 //
-// This file holds the one-CTA kernel (only on request, nvfp4_set_gemm_tile_n), the tensor-map helpers and the launchers of
-// all kernels; the CTA-pair kernels that take every shape are in gemm_2cta.cuh and gemm_wide.cuh.
+// This file holds the one-CTA kernel (for odd multiples of 128, see one_cta_time, and on request), the tensor-map helpers and the
+// launchers of all kernels; the CTA-pair kernels that take every shape are in gemm_2cta.cuh and gemm_wide.cuh.
 #include <cuda.h>
 #include <cuda_bf16.h>
 
@@ -311,8 +311,8 @@ __global__ void __launch_bounds__(kThreads, 1)
           float* dst = reinterpret_cast<float*>(g.d) + row * g.ldd + col;
 #pragma unroll
           for (int v = 0; v < 8; ++v) {
-            float4 o = make_float4(__uint_as_float(r[4 * v]) * alpha, __uint_as_float(r[4 * v + 1]) * alpha,
-                                   __uint_as_float(r[4 * v + 2]) * alpha, __uint_as_float(r[4 * v + 3]) * alpha);
+            float4 o = make_float4(__fmul_rn(__uint_as_float(r[4 * v]), alpha), __fmul_rn(__uint_as_float(r[4 * v + 1]), alpha),
+                                   __fmul_rn(__uint_as_float(r[4 * v + 2]), alpha), __fmul_rn(__uint_as_float(r[4 * v + 3]), alpha));
             if (g.accumulate) {
               float4 old = *reinterpret_cast<const float4*>(dst + 4 * v);
               o.x += old.x; o.y += old.y; o.z += old.z; o.w += old.w;
@@ -676,16 +676,30 @@ cudaError_t launch_gemm_two(const GemmArgs& g0, const void* a0, const void* b0, 
   return launch_pair(g0, a0, b0, &g1, a1, b1, tile == kTilePair256 || tile == kTileWide ? 256 : 128, num_sms, s);
 }
 
-int best_pair_tile(const GemmArgs& g0, const GemmArgs* g1) {
+// 128 x 128 tiles of one CTA each, for one product: its time, or 0 where they are no candidates.  They double the operand
+// traffic of a pair, but where M is an odd multiple of 128 the pairs compute a row of half tiles: if that takes the narrow pair
+// tiles over one round of the chip and the single ones fit it, those win.  Single / pair tiles: 1152 x 2048 x 2048 7.2 / 9.0
+// us, x 5120 12.3 / 13.3, MXFP4 6.4 / 8.8 and 10.0 / 13.1; 1664 x 1408 x 5120 13.3 / 13.3, MXFP4 10.9 / 13.0, fp32 output 15.4 /
+// 14.8 and 13.2 / 14.3.  (Not for an accumulated output: its read-modify-write in the epilogue costs 3 us.)
+static double one_cta_time(const GemmArgs& g, int num_sms) {
+  const int64_t tiles = (int64_t)(g.M / 128) * (g.N / 128);
+  if (g.accumulate || g.a_rows || g.b_rows || tiles > num_sms || pair_tiles(g, 128) <= num_sms / 2) return 0.0;
+  const double kb = g.K / 256.0;
+  return (g.mx ? 0.29 : 0.40) * kb + (g.d_is_fp32 ? 3.7 : 1.4);
+}
+
+int best_tile(const GemmArgs& g0, const GemmArgs* g1) {
   int num_sms = 0;
   if (sm_count(&num_sms) != cudaSuccess) return kTilePair256;
   const bool wide_fits = wide_eligible(g0) && (!g1 || wide_eligible(*g1));
   int dev = 0, best = kTilePair256;
   if (cudaGetDevice(&dev) != cudaSuccess) return best;
   static TileMemo memo;
+  const double single = g1 ? 0.0 : one_cta_time(g0, num_sms);
   // (the output type is part of the key: an fp32 output changes the hand-over cost and with it the choice)
   const int key[TileMemo::kKey] = {g0.M, g0.N, g0.K, g1 ? g1->M : 0, g1 ? g1->N : 0, g1 ? g1->K : 0,
-                                   (g0.d_is_fp32 ? 1 : 0) | (g1 && g1->d_is_fp32 ? 2 : 0), dev};
+                                   (g0.d_is_fp32 ? 1 : 0) | (g1 && g1->d_is_fp32 ? 2 : 0) | (single > 0.0 ? 4 : 0) | (g0.mx ? 8 : 0),
+                                   dev};
   if (memo.find(key, &best)) return best;
   const GemmArgs* gs[2] = {&g0, g1};
   const int n = g1 ? 2 : 1, pairs = num_sms / 2;
@@ -699,8 +713,13 @@ int best_pair_tile(const GemmArgs& g0, const GemmArgs* g1) {
       best = tile;
     }
   }
-  if (!g1)
+  if (!g1) {
+    if (single > 0.0 && single + 0.2 < least) {
+      least = single;
+      best = kTileOne128;
+    }
     if (const int tile = split_tile(g0, least)) best = tile;
+  }
   memo.put(key, best);
   return best;
 }

@@ -22,6 +22,7 @@ struct GemmArgs {
 
 // Tiles: 128 or 256 = one CTA per 128 x 128 / 128 x 256 tile (256 needs N % 256 == 0, otherwise 128 is used); the others
 // run on CTA pairs and take any M and N that are multiples of 128 (a half beyond the edge is computed on zeros and clipped).
+constexpr int kTileOne128 = 128;   // 128 x 128, one CTA
 constexpr int kTilePair256 = 512;  // 256 x 256
 constexpr int kTilePair128 = 640;  // 256 x 128
 constexpr int kTileWide = 768;     // 256 x 384, needs N >= 256
@@ -35,8 +36,8 @@ int split_of(const GemmArgs& g, int tile);
 // in the same order here, on 256 x 128 tiles whatever `tile` says.
 cudaError_t launch_gemm_two(const GemmArgs& g0, const void* a0, const void* b0, const GemmArgs& g1, const void* a1,
                             const void* b1, int tile, cudaStream_t s);
-// Scheduling estimate: the CTA-pair tile for this problem (or pair of problems in one launch, then no split one)
-int best_pair_tile(const GemmArgs& g0, const GemmArgs* g1);
+// Scheduling estimate: the tile for this problem (or for two problems in one launch, then a whole CTA-pair one)
+int best_tile(const GemmArgs& g0, const GemmArgs* g1);
 // Measurement aids of the CTA-pair kernel with 256 x 256 tiles (0, 0, NULL = normal operation): mode bit 0 = no MMAs,
 // bit 1 = no operand loads, bit 2 = no scale loads / copies, bit 3 = accumulator handed back unread and nothing
 // stored, bit 4 = the issuer does not wait for the accumulator (results meaningless with any bit set); max_pairs caps the

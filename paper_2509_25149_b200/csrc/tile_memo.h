@@ -1,4 +1,4 @@
-// Remembered tile choices (host code, see best_pair_tile): a training loop repeats a handful of shapes, and the estimate walks every
+// Remembered tile choices (host code, see best_tile): a training loop repeats a handful of shapes, and the estimate walks every
 // tile of every schedule.  The newest kEntries shapes are kept, whatever came before them; a shape's choice belongs to
 // a device, because how many clusters are resident at once differs between GPUs with the same number of SMs.
 #pragma once

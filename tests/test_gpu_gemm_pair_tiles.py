@@ -149,3 +149,44 @@ def test_measurement_aids_leave_the_other_tiles_alone(tile):
         B.nvfp4_set_gemm_experiment()
         B.nvfp4_set_gemm_tile_n(0)
     assert torch.equal(D, want) and not probe.any()
+
+
+# 143, 144 and 148 tiles of 128 x 128 (one round of 148 CTAs) where 256 x 128 would take two rounds of 74 pairs; then 150, and 72 pairs
+@pytest.mark.parametrize("shape,single", [((1664, 1408, 512), True), ((1152, 2048, 2048), True), ((128, 18944, 768), True),
+                                          ((1280, 1920, 512), False), ((1536, 1536, 512), False), ((1664, 1408, 8192), False)])
+@pytest.mark.parametrize("fmt", [B.FORMAT_NVFP4, B.FORMAT_MXFP4])
+@pytest.mark.parametrize("fp32", [False, True])
+def test_single_tiles_where_pairs_would_go_round_twice(shape, single, fmt, fp32):
+    """Chosen by size; the bits are those of the pair tiles, accumulated outputs included.  Blocks far apart in magnitude, so that
+    the order of the additions shows."""
+    M, N, K = shape
+    if torch.cuda.get_device_properties(0).multi_processor_count == 148 and not fp32 and fmt == B.FORMAT_NVFP4:
+        assert (B.nvfp4_gemm_tile(False, M, N, K, False) == 128) == single
+    gen = torch.Generator("cuda").manual_seed(M + K)
+    ops = []
+    for rows in (M, N):
+        x = torch.randn((rows, K), generator=gen, device="cuda")
+        e = torch.randint(-9, 10, (rows // 32, K // 32), generator=gen, device="cuda").float()
+        x = (x * torch.exp2(e).repeat_interleave(32, 0).repeat_interleave(32, 1)).to(torch.bfloat16)
+        ops.append(B.alloc_tensor(rows, K, format=fmt))
+        B.nvfp4_quantize(x, B.quant_opts(), ops[-1])
+    dtype = torch.float32 if fp32 else torch.bfloat16
+    wide = torch.full((M + 8, N + 64), 7.0, dtype=dtype, device="cuda")
+    D, want = wide[:M, :N], torch.empty((M, N), dtype=dtype, device="cuda")
+    for accumulate in (False, True)[:1 + fp32]:
+        B.nvfp4_gemm(*ops, D, accumulate=accumulate)
+        B.nvfp4_set_gemm_tile_n(512)
+        try:
+            B.nvfp4_gemm(*ops, want, accumulate=accumulate)
+        finally:
+            B.nvfp4_set_gemm_tile_n(0)
+        B.nvfp4_device_status()
+        assert torch.equal(D, want) and torch.all(wide[M:] == 7.0) and torch.all(wide[:, N:] == 7.0)
+    if fp32:  # the forced kernel adds a rounded product, as the others do
+        B.nvfp4_set_gemm_tile_n(128)
+        try:
+            B.nvfp4_gemm(*ops, D, accumulate=True)
+        finally:
+            B.nvfp4_set_gemm_tile_n(0)
+        B.nvfp4_gemm(*ops, want, accumulate=True)
+        assert torch.equal(D, want)

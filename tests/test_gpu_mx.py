@@ -61,7 +61,7 @@ def test_gemm_against_fp64_product_of_decoded_operands(shape, fp32):
 @pytest.mark.parametrize("tile_n", [128, 256])
 @pytest.mark.parametrize("fp32", [False, True])
 def test_gemm_one_cta_kernel(shape, tile_n, fp32):
-    """Shapes with M or N not a multiple of 256 (and the forced tile widths) take the one-CTA kernel."""
+    """The forced tile widths take the one-CTA kernel."""
     M, N, K = shape
     a = oracle.quantize_mx(synth.bits(synth.normal_with_outliers_bf16((M, K), 0.01, 50.0, 35, 36)))
     b = oracle.quantize_mx(synth.bits(synth.normal_bf16((N, K), 0.02, 37)), block_rows=32)
