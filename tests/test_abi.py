@@ -164,10 +164,18 @@ def test_stream_handle_comes_from_the_public_call_where_it_has_to(monkeypatch, m
     monkeypatch.setattr(torch.cuda, "is_initialized", lambda: missing != "CUDA not initialised")
     monkeypatch.setattr(B, "_get_device", lambda: 0)
     monkeypatch.setattr(B, "_raw_stream", lambda device: 0x5678)
-    assert B._stream() == (0x1234 if missing == "CUDA not initialised" else 0x5678)
+    monkeypatch.setattr(B, "_stream_is_raw", False)
     if missing.startswith("_"):
         monkeypatch.setattr(B, missing, None)
-        assert B._stream() == 0x1234
+    assert B._stream() == 0x1234
+
+
+def test_stream_handle_is_the_raw_one_once_cuda_is_initialised(monkeypatch):
+    monkeypatch.setattr(torch.cuda, "is_initialized", lambda: True)
+    monkeypatch.setattr(B, "_get_device", lambda: 3)
+    monkeypatch.setattr(B, "_raw_stream", lambda device: 0x5678 + device)
+    monkeypatch.setattr(B, "_stream_is_raw", False)
+    assert B._stream() == B._stream() == 0x567B
 
 
 def test_tensor_structs_are_taken_in_every_form():
