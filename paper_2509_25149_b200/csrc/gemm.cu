@@ -577,7 +577,7 @@ int split_clusters() {
 // The split of a product that has a launch to itself, or 0 (`least`: the estimate of the best tile).  A split pays where a
 // tile's contraction is long and the clusters of all tiles are resident at once; its exchange costs 1.4 us (2.1 where most of
 // the chip takes part) and it has to win by half a microsecond.  The two products of a backward call fill one launch
-// together: with one of them split and the other behind it, 512 x 3584 x 768 took 38.0 us instead of 31.8.
+// together: with one of them split and the other behind it, 512 x 3584 x 768 took 22.6 us instead of 16.0.
 // Time of a product, 256 x 128 tiles / two pairs / four pairs per tile: 256 x 512 x 5120 10.5 / 8.5 / 7.3 us, 256 x 512 x 20480
 // 29.1 / 17.8 / 12.2, 512 x 1024 x 4096 9.5 / 8.1 / 14.1 (two rounds), 1024 x 1024 x 10240 17.6 / 12.9 / 27.6; 256 x 1024 x 2048
 // 6.7 / 6.7 / 6.4, 256 x 2048 x 1024 5.5 / 6.2 / 12.1.

@@ -12,7 +12,7 @@
 // soon as it has been read).
 // M and N may be odd multiples of 128: the half of the last tile beyond the edge reads zero codes (tensor map) and its
 // output is clipped.  Half a tile of padding costs less than the one-CTA kernel that used to take these shapes:
-// 4224 x 5248 x 5120 85 -> 60 us, 2176 x 4992 x 1024 15.5 -> 12.2 us.
+// 4224 x 5248 x 5120 85 -> 60 us, 2176 x 4992 x 1024 15.5 -> 12.2 us (it keeps some, see one_cta_time).
 // Included by gemm.cu only.
 #pragma once
 
