@@ -53,13 +53,19 @@ __device__ __forceinline__ void global_scales(float amax, float& s_enc, float& s
 // the correction term is off by only 2^-25 relative, so q' is the correctly rounded quotient whenever the residual is
 // exact, i.e. outside the denormal range (checked exhaustively over whole binades on the host); tiny inputs take the
 // IEEE division.
-__device__ __forceinline__ float div6_rn(float x) {
+__device__ __forceinline__ float div6_fast(float x) {
   const float c = 0.16666667163372039794921875f;  // fl(1/6)
   const float q = __fmul_rn(x, c);
   const float r = __fmaf_rn(-6.0f, q, x);
-  const float fast = __fmaf_rn(r, c, q);
+  return __fmaf_rn(r, c, q);
+}
+__device__ __forceinline__ float div6_rn(float x) {
+  const float fast = div6_fast(x);
   return (x != 0.0f && x < 1.0e-30f) ? __fdiv_rn(x, 6.0f) : fast;
 }
+// Largest s_enc with which every block amax below 1e-30 gets the scale byte 0 whichever way it is divided: the quotient is below
+// 1.7e-31 and fl(quotient * s_enc) below 2^-10, half of the smallest E4M3 value.
+constexpr float kPlainDivisionLimit = 5.0e27f;
 
 __device__ __forceinline__ void block_scales(float amax_b, float s_enc, float s_dec, uint32_t& byte,
                                              float& s_enc_b) {

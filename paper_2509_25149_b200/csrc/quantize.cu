@@ -63,7 +63,7 @@ __device__ __forceinline__ void amax_tile(const uint16_t* __restrict__ x, int64_
       acc = absmax_bf16x2(acc, raw[j].z);
       acc = absmax_bf16x2(acc, raw[j].w);
     }
-    m_plain = fmaxf(bf16_lo(acc), bf16_hi(acc));
+    m_plain = amax_of_pair(acc);
   }
   if (ROT_COL) {
     // chunks run down the 16 rows of the warp's slab: one transform per column
@@ -228,7 +228,7 @@ __device__ __forceinline__ void amax_rot_col_tile(const uint16_t* __restrict__ x
     }
   }
   m_col *= norm;
-  float m_plain = PLAIN ? fmaxf(bf16_lo(acc), bf16_hi(acc)) : 0.f;
+  float m_plain = PLAIN ? amax_of_pair(acc) : 0.f;
 
   __shared__ float red[2][8];
   m_plain = warp_max(m_plain);
@@ -354,12 +354,16 @@ struct QuantSmem {
   static constexpr int bytes(bool rand, bool row_codes) { return kRand + (rand ? 128 * TC : row_codes ? 64 * TC : 0); }
 };
 
-// Eq. 2-3: the stored E4M3 byte of a block, S_b = e4m3(fl(fl(amax_b / 6) * s_enc))
+// Eq. 2-3: the stored E4M3 byte of a block, S_b = e4m3(fl(fl(amax_b / 6) * s_enc)).  TINY: s_enc > kPlainDivisionLimit; the other
+// form has no branch.  A branch per block (this one, and one around the transposed copy's own draws) cut the code of a tile into
+// pieces that could not overlap, at four warps per scheduler: activation of 8192 x 5120 43.5 -> 41.0 us without, gradient 59.2 ->
+// 55.6, 4096 x 4096 20.2 -> 19.4 and 26.4 -> 24.5.
+template <bool TINY>
 __device__ __forceinline__ uint32_t block_scale_byte(float amax_b, float s_enc) {
-  const float t = __fmul_rn(div6_rn(amax_b), s_enc);
+  const float t = __fmul_rn(TINY ? div6_rn(amax_b) : div6_fast(amax_b), s_enc);
   uint16_t packed;
-  asm("cvt.rn.satfinite.e4m3x2.f32 %0, %1, %1;" : "=h"(packed) : "f"(t));
-  return packed & 0xffu;
+  asm("cvt.rn.satfinite.e4m3x2.f32 %0, %1, %2;" : "=h"(packed) : "f"(0.f), "f"(t));
+  return packed;
 }
 // the text after Eq. 3: encode scale of a block from its stored byte, fl(1 / fl(fp32(S_b) * s_dec)), 0 for S_b = 0
 __device__ __forceinline__ float encode_scale_of_byte(uint32_t byte, float s_dec) {
@@ -459,6 +463,7 @@ __device__ __forceinline__ void quantize_tiles(const CUtensorMap* src_map, const
   __syncthreads();
   griddep_launch_dependents();
   const float r_senc = g_sc[0], r_sdec = g_sc[1], c_senc = g_sc[2], c_sdec = g_sc[3];
+  const bool tiny = !BLOCK2D && fmaxf(HAS_ROW ? r_senc : 0.f, HAS_COL ? c_senc : 0.f) > kPlainDivisionLimit;
   const float* enc_row = reinterpret_cast<const float*>(smem + S::kEncRow);
   const float* enc_col = reinterpret_cast<const float*>(smem + S::kEncCol);
   if (!BLOCK2D) {
@@ -517,8 +522,8 @@ __device__ __forceinline__ void quantize_tiles(const CUtensorMap* src_map, const
     uint8_t* const sf_row = smem + S::kSfRow + buf * S::kSfBytes;
     uint8_t* const sf_col = smem + S::kSfCol + buf * S::kSfBytes;
 
-    auto phases_1_2 = [&](auto full_c) {
-      constexpr bool FULL = decltype(full_c)::value;
+    auto phases_1_2 = [&](auto full_c, auto tiny_c) {
+      constexpr bool FULL = decltype(full_c)::value, TINY = decltype(tiny_c)::value;
       // ---------------------------------------------------------------- phase 1 ----
       const int rows_left = FULL ? 128 : (int)(a.rows - row0) - rl;         // chunk i exists iff RPP * i < rows_left
       const bool col_ok = FULL || (col0 + cb * 16 < a.cols);
@@ -547,7 +552,7 @@ __device__ __forceinline__ void quantize_tiles(const CUtensorMap* src_map, const
             uint32_t acc = 0;
 #pragma unroll
             for (int k = 0; k < 8; ++k) acc = absmax_bf16x2(acc, raw[i][k]);
-            blk_amax = fmaxf(blk_amax, fmaxf(bf16_lo(acc), bf16_hi(acc)));
+            blk_amax = fmaxf(blk_amax, amax_of_pair(acc));
           }
         }
 #pragma unroll
@@ -567,15 +572,10 @@ __device__ __forceinline__ void quantize_tiles(const CUtensorMap* src_map, const
         uint32_t rnd[4] = {0u, 0u, 0u, 0u};
         if (SR) {
           const uint64_t gi = g + (uint64_t)(RPP * i) * (uint64_t)n_cb;
-          uint4 q = philox4x32_10((uint32_t)gi, (uint32_t)(gi >> 32), a.off_lo, a.off_hi, a.rk);
+          const uint4 q = philox4x32_10((uint32_t)gi, (uint32_t)(gi >> 32), a.off_lo, HAS_ROW ? a.off_hi : a.off_hi_col, a.rk);
           rnd[0] = q.x; rnd[1] = q.y; rnd[2] = q.z; rnd[3] = q.w;
-          if (HAS_COL && !kNibbleTranspose) {
-            uint4 qc = q;
-            if (a.off_hi_col != a.off_hi)
-              qc = philox4x32_10((uint32_t)gi, (uint32_t)(gi >> 32), a.off_lo, a.off_hi_col, a.rk);
-            // staged complemented: the conversion wants 255 - draw
-            *reinterpret_cast<uint4*>(smem + rand_st + i * (RPP * TC)) = make_uint4(~qc.x, ~qc.y, ~qc.z, ~qc.w);
-          }
+          if (HAS_COL && !kNibbleTranspose)  // staged complemented: the conversion wants 255 - draw
+            *reinterpret_cast<uint4*>(smem + rand_st + i * (RPP * TC)) = make_uint4(~q.x, ~q.y, ~q.z, ~q.w);
         }
         if (HAS_ROW) {
           float f[16];
@@ -605,7 +605,7 @@ __device__ __forceinline__ void quantize_tiles(const CUtensorMap* src_map, const
             enc = blk_enc;
           } else {
             const float m = amax16_3(f);
-            byte = block_scale_byte(RHT_ROW ? 0.25f * m : m, r_senc);
+            byte = block_scale_byte<TINY>(RHT_ROW ? 0.25f * m : m, r_senc);
             enc = enc_row[byte];
           }
           uint2 codes = convert16<SR>(f, enc, Nu14FromWords{rnd});
@@ -620,6 +620,14 @@ __device__ __forceinline__ void quantize_tiles(const CUtensorMap* src_map, const
             *reinterpret_cast<uint2*>(smem + S::kRand + (rl + RPP * i) * (TC / 2) + cb * 8) =
                 (FULL || (col_ok && RPP * i < rows_left)) ? codes : make_uint2(0u, 0u);
           sf_row[sf_row_pos + i * sf_row_step] = (uint8_t)byte;
+        }
+      }
+      if (SR && HAS_ROW && HAS_COL && !kNibbleTranspose && a.off_hi_col != a.off_hi) {  // draws of its own for the transposed copy
+#pragma unroll 1
+        for (int i = 0; i < NP; ++i) {
+          const uint64_t gi = g + (uint64_t)(RPP * i) * (uint64_t)n_cb;
+          const uint4 q = philox4x32_10((uint32_t)gi, (uint32_t)(gi >> 32), a.off_lo, a.off_hi_col, a.rk);
+          *reinterpret_cast<uint4*>(smem + rand_st + i * (RPP * TC)) = make_uint4(~q.x, ~q.y, ~q.z, ~q.w);
         }
       }
       // Phase 2 of a warp reads only what the same warp staged in phase 1 (its own 16 rows of the tile, their random
@@ -677,8 +685,8 @@ __device__ __forceinline__ void quantize_tiles(const CUtensorMap* src_map, const
             byte0 = byte1 = smem[S::kBlkByte + q * CH + (cp >> 3)];
           } else {
             const float2 m = amax_pairs(v);
-            byte0 = block_scale_byte(RHT_COL ? 0.25f * m.x : m.x, c_senc);
-            byte1 = block_scale_byte(RHT_COL ? 0.25f * m.y : m.y, c_senc);
+            byte0 = block_scale_byte<TINY>(RHT_COL ? 0.25f * m.x : m.x, c_senc);
+            byte1 = block_scale_byte<TINY>(RHT_COL ? 0.25f * m.y : m.y, c_senc);
             enc = make_float2(enc_col[byte0], enc_col[byte1]);
           }
           uint2 codes0, codes1;
@@ -701,10 +709,12 @@ __device__ __forceinline__ void quantize_tiles(const CUtensorMap* src_map, const
         }
       }
     };
-    if (full_tile)
-      phases_1_2(std::true_type{});
+    if (tiny)
+      phases_1_2(std::false_type{}, std::true_type{});
+    else if (full_tile)
+      phases_1_2(std::true_type{}, std::false_type{});
     else
-      phases_1_2(std::false_type{});
+      phases_1_2(std::false_type{}, std::false_type{});
     __syncthreads();
     if (*abort_flag) break;  // a wait expired (the word is read after the barrier: the same for every thread)
     if (threadIdx.x == 0 && j + 2 < n_mine) issue(j + 2);  // every warp is done with this buffer

@@ -26,13 +26,12 @@ __device__ __forceinline__ uint4 ldg128_stream(const void* p) {
   return r;
 }
 
+// magnitudes of `acc` become the larger ones of both operands; its signs mean nothing (amax_of_pair drops them)
 __device__ __forceinline__ uint32_t absmax_bf16x2(uint32_t acc, uint32_t v) {
-  __nv_bfloat162 a = *reinterpret_cast<__nv_bfloat162*>(&acc);
-  uint32_t m = v & 0x7fff7fffu;
-  __nv_bfloat162 b = *reinterpret_cast<__nv_bfloat162*>(&m);
-  __nv_bfloat162 r = __hmax2(a, b);
-  return *reinterpret_cast<uint32_t*>(&r);
+  asm("max.xorsign.abs.bf16x2 %0, %0, %1;" : "+r"(acc) : "r"(v));
+  return acc;
 }
+__device__ __forceinline__ float amax_of_pair(uint32_t acc) { return fmaxf(fabsf(bf16_lo(acc)), fabsf(bf16_hi(acc))); }
 
 __device__ __forceinline__ float warp_max(float v) {
 #pragma unroll

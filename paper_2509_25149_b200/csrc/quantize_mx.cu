@@ -141,7 +141,7 @@ __global__ void __launch_bounds__(256, CTAS)
         uint32_t acc = 0;
 #pragma unroll
         for (int k = 0; k < 8; ++k) acc = absmax_bf16x2(acc, raw[i][k]);
-        const float own = fmaxf(bf16_lo(acc), bf16_hi(acc));
+        const float own = amax_of_pair(acc);
         am[i] = fmaxf(own, __shfl_xor_sync(0xffffffffu, own, 1));
       }
     }

@@ -34,7 +34,7 @@ __device__ __forceinline__ void encode_chunk(const QuantArgs& a, const uint32_t 
   for (int k = 0; k < 8; ++k) acc = absmax_bf16x2(acc, raw[k]);
   uint32_t byte;
   float enc;
-  block_scales(fmaxf(bf16_lo(acc), bf16_hi(acc)), s_enc, s_dec, byte, enc);
+  block_scales(amax_of_pair(acc), s_enc, s_dec, byte, enc);
   float f[16];
 #pragma unroll
   for (int k = 0; k < 8; ++k) {
@@ -86,7 +86,7 @@ __global__ void __launch_bounds__(128, ctas_per_sm(kKeep)) quantize_rowscale_ker
     for (int i = 0; i < kKeep; ++i)
 #pragma unroll
       for (int k = 0; k < 8; ++k) acc = absmax_bf16x2(acc, keep[i][k]);
-    float amax = warp_max(fmaxf(bf16_lo(acc), bf16_hi(acc)));
+    float amax = warp_max(amax_of_pair(acc));
     if (WPR > 1) {
       if (lane == 0) part[it & 1][warp] = amax;
       __syncthreads();
@@ -134,7 +134,7 @@ __global__ void __launch_bounds__(256) quantize_rowscale_long_kernel(const Quant
 #pragma unroll
         for (int k = 0; k < 8; ++k) acc = absmax_bf16x2(acc, raw[u][k]);
     }
-    const float amax = warp_max(fmaxf(bf16_lo(acc), bf16_hi(acc)));
+    const float amax = warp_max(amax_of_pair(acc));
     float s_enc, s_dec;
     global_scales(amax, s_enc, s_dec);
     if (lane == 0) {

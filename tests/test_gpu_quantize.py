@@ -165,6 +165,24 @@ def test_extreme_magnitudes_stay_bit_exact(scale, rounding):
         P.assert_exact(col, oracle.quantize(synth.bits(x), colwise=True, **kw), f"col scale {scale} blocks {block_rows}")
 
 
+@pytest.mark.parametrize("amax", [5.0e-25, 5.8e-25])
+@pytest.mark.parametrize("shape", [(128, 128), (144, 208)])
+@pytest.mark.parametrize("rounding", [B.ROUND_NEAREST_EVEN, B.ROUND_STOCHASTIC])
+def test_blocks_beside_the_limit_of_the_plain_division(amax, shape, rounding):
+    """amax_b / 6 is divided without a branch while s_enc = 2688 / amax is at most 5e27 (amax 5.4e-25): tensors on either side,
+    with blocks whose amax is 1, 1e-3 ... 1e-12 of the tensor's, i.e. above and below 1e-30 and below the smallest normal."""
+    x = rand_bf16(shape, 77).float()
+    decades = torch.arange(shape[0] // 16).repeat_interleave(16)[:, None] + torch.arange(shape[1] // 16).repeat_interleave(16)
+    x = x / x.abs().max() * amax * 10.0 ** (-3.0 * (decades % 5))
+    x[0, 0] = amax
+    x = x.bfloat16()
+    layout = B.SF_SWIZZLED if shape[0] % 128 == 0 else B.SF_LINEAR
+    row, col = P.gpu_quantize(x, rowwise=True, colwise=True, sf_layout=layout, rounding=rounding, seed=3, sr_offset=2)
+    kw = dict(rounding=oracle.RNE if rounding == B.ROUND_NEAREST_EVEN else oracle.SR, seed=3, sr_offset=2)
+    P.assert_exact(row, oracle.quantize(synth.bits(x), **kw), "row")
+    P.assert_exact(col, oracle.quantize(synth.bits(x), colwise=True, **kw), "col")
+
+
 def test_gpu_sr_is_unbiased_over_seeds():
     x = rand_bf16((128, 128), 8, std=1e-3)
     xd = x.cuda()
