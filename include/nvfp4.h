@@ -179,7 +179,7 @@ NVFP4_API nvfp4_status nvfp4_gemm(const nvfp4_tensor* A, const nvfp4_tensor* B, 
  *   B: device bf16.  b_layout NVFP4_K_MAJOR : stored [N][K], ldb >= K;  NVFP4_MN_MAJOR: stored [K][N], ldb >= N.
  *   D: device, row-major [M x N], ldd >= N, bf16 (round-to-nearest-even) or fp32 (d_is_fp32 != 0);
  *      accumulate != 0 adds into an fp32 D.
- *   M, N, K multiples of 8 (the kernel works on 256 x 256 or 256 x 128 tiles, 64 deep, and a narrow tile's contraction may be
+ *   M, N, K multiples of 8 (the kernel works on 256 x 512, 256 x 256 or 256 x 128 tiles, 64 deep, and a narrow tile's contraction may be
  *   shared by two or four CTA pairs; ragged edges are zero-filled on load and clipped on store by the tensor maps); pointers 16-byte aligned, lda, ldb multiples of 8, ldd * elemsize of 16.
  *   Nothing is enqueued on error.
  */
@@ -343,7 +343,8 @@ NVFP4_API nvfp4_status nvfp4_test_cluster_leave(uint64_t delay_ns, uint64_t* tim
 NVFP4_API int32_t nvfp4_set_gemm_tile_n(int32_t tile_n);
 
 /* The tile (a value of nvfp4_set_gemm_tile_n) of one M x N x K product with a launch to itself on the current device: nvfp4_gemm
- * (NVFP4, D written), or nvfp4_gemm_bf16 when bf16 != 0.  -1 for a size that the call would refuse.  Launches nothing. */
+ * (NVFP4, D written), or nvfp4_gemm_bf16 of packed K-major operands when bf16 != 0 (which has 1024 besides: 256 x 512 tiles, and
+ * 256 x 256 ones for the columns that are left; chosen by size alone).  -1 for a size that the call would refuse.  Launches nothing. */
 NVFP4_API int32_t nvfp4_gemm_tile(int32_t bf16, int64_t M, int64_t N, int64_t K, int32_t d_is_fp32);
 
 /*

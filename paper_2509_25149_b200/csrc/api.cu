@@ -597,6 +597,7 @@ int32_t nvfp4_gemm_tile(int32_t bf16, int64_t M, int64_t N, int64_t K, int32_t d
   if (bf16) {
     DenseGemmArgs g{};
     g.M = (int)M; g.N = (int)N; g.K = (int)K;
+    g.lda = g.ldb = K;
     return bf16_tile(g, nullptr, g_tile_n.load(std::memory_order_relaxed));
   }
   GemmArgs g{};

@@ -730,7 +730,8 @@ static bool make_bf16_maps(const DenseGemmArgs& g, CUtensorMap* m) {  // A, B, D
   bool ok = g.a_mn ? make_map_2d(&m[0], bf, 2, g.a, (uint64_t)g.M, (uint64_t)g.K, (uint64_t)g.lda * 2, 64, 64, true)
                    : make_map_2d(&m[0], bf, 2, g.a, (uint64_t)g.K, (uint64_t)g.M, (uint64_t)g.lda * 2, 64, 128, true);
   ok = ok && (g.b_mn ? make_map_2d(&m[1], bf, 2, g.b, (uint64_t)g.N, (uint64_t)g.K, (uint64_t)g.ldb * 2, 64, 64, true)
-                     : make_map_2d(&m[1], bf, 2, g.b, (uint64_t)g.K, (uint64_t)g.N, (uint64_t)g.ldb * 2, 64, BN / 2, true));
+                     : make_map_2d(&m[1], bf, 2, g.b, (uint64_t)g.K, (uint64_t)g.N, (uint64_t)g.ldb * 2, 64,
+                                   BN == 512 ? 128 : BN / 2, true));
   if (g.d_is_fp32)
     ok = ok && make_map_2d(&m[2], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, g.d, (uint64_t)g.N, (uint64_t)g.M,
                            (uint64_t)g.ldd * 4, 16, 128, 2);
@@ -743,7 +744,8 @@ static bool make_bf16_maps(const DenseGemmArgs& g, CUtensorMap* m) {  // A, B, D
 static int bf16_tiles(const DenseGemmArgs& g, int bn) { return ((g.M + 255) / 256) * ((g.N + bn - 1) / bn); }
 
 template <int BN, int SPLIT, bool TWO>
-static cudaError_t launch_bf16_problems(const DenseGemmArgs& g0, const DenseGemmArgs* g1, int max_pairs, cudaStream_t s) {
+static cudaError_t launch_bf16_problems(const DenseGemmArgs& g0, const DenseGemmArgs* g1, const int (&wide_n)[2], int max_pairs,
+                                        cudaStream_t s) {
   auto kern = dense::gemm_bf16_pair_kernel<BN, SPLIT, TWO>;
   constexpr int smem = dense::Cfg<BN, SPLIT>::kSmemBytes;
   CUtensorMap m[6];
@@ -766,8 +768,20 @@ static cudaError_t launch_bf16_problems(const DenseGemmArgs& g0, const DenseGemm
   dense::Args a{};
   a.p[0] = problem(g0);
   a.p[1] = problem(g1 ? *g1 : g0);
-  a.n_tiles0 = bf16_tiles(g0, BN);
-  a.n_tiles = a.n_tiles0 + (g1 ? bf16_tiles(*g1, BN) : 0);
+  if (BN == 512) {
+    for (int i = 0; i < (g1 ? 2 : 1); ++i) {
+      const DenseGemmArgs& g = i ? *g1 : g0;
+      const int tiles_m = (g.M + 255) / 256, wide = std::min(wide_n[i], (g.N + 255) / 512);
+      a.wide_n[i] = wide;
+      a.seg_end[i] = tiles_m * wide;
+      a.seg_end[2 + i] = tiles_m * ((g.N + 255) / 256 - 2 * wide);
+    }
+    for (int i = 1; i < 4; ++i) a.seg_end[i] += a.seg_end[i - 1];
+    a.n_tiles0 = a.n_tiles = a.seg_end[3];
+  } else {
+    a.n_tiles0 = bf16_tiles(g0, BN);
+    a.n_tiles = a.n_tiles0 + (g1 ? bf16_tiles(*g1, BN) : 0);
+  }
   const int pairs = a.n_tiles < max_pairs || SPLIT > 1 ? a.n_tiles : max_pairs;  // SPLIT > 1: a cluster for each tile
   const cudaError_t e = launch_kernel(kern, dim3(2 * SPLIT * pairs), dim3(dense::kThreads), smem, s, m[0], m[1], m[2],
                                       m[3], m[4], m[5], a);
@@ -777,9 +791,81 @@ static cudaError_t launch_bf16_problems(const DenseGemmArgs& g0, const DenseGemm
 
 // g1 == nullptr: one problem
 template <int BN, int SPLIT = 1>
-static cudaError_t launch_bf16_t(const DenseGemmArgs& g0, const DenseGemmArgs* g1, int max_pairs, cudaStream_t s) {
-  return g1 ? launch_bf16_problems<BN, SPLIT, true>(g0, g1, max_pairs, s)
-            : launch_bf16_problems<BN, SPLIT, false>(g0, nullptr, max_pairs, s);
+static cudaError_t launch_bf16_t(const DenseGemmArgs& g0, const DenseGemmArgs* g1, const int (&wide_n)[2], int max_pairs,
+                                 cudaStream_t s) {
+  return g1 ? launch_bf16_problems<BN, SPLIT, true>(g0, g1, wide_n, max_pairs, s)
+            : launch_bf16_problems<BN, SPLIT, false>(g0, nullptr, wide_n, max_pairs, s);
+}
+
+// Column tiles 512 wide of each problem (the other columns in tiles of 256, behind them) whose schedule is estimated shortest;
+// {0, 0}: 256-wide tiles everywhere.  A k-block of a tile takes as long as its MMAs (530 SM cycles per 256 columns) or as its
+// loads: 63 bytes per clock, 1.375 x the bytes where the rows of an operand are no multiple of 128 bytes apart.  Where the MMAs
+// are longer, what 512 columns gain is fewer hand-overs and, with tiles of two sizes, shorter last rounds.  256 wide / chosen:
+// forward of 4088 x 5128 x 5112 214 / 184 us, backward 401 / 341, forward of 2048 x 7168 x 2056 68 / 55, of 3000 x 3000 x 1000
+// 21.3 / 19.0; rows 128 bytes apart: backward of 8192 x 5120 x 5120 696 / 671, of 4096 x 4096 x 4096 221 / 208, forward of 16384 x
+// 2560 x 1288 113 / 105.  Contractions of fewer than 14 k-blocks keep 256 columns: there the epilogue of the last tile, whose
+// halves leave one after the other, costs more than the loads (1112 x 3672 x 552 11.5 / 12.7, 2344 x 1856 x 264 9.2 / 10.3).
+static void bf16_wide_tiles(const DenseGemmArgs& g0, const DenseGemmArgs* g1, int pairs, int (&wide_n)[2]) {
+  static TileMemo memo;
+  const int key[TileMemo::kKey] = {g0.M, g0.N, g0.K, g1 ? g1->M : 0, g1 ? g1->N : 0, g1 ? g1->K : 0,
+                                   (g0.lda % 64 ? 1 : 0) | (g0.ldb % 64 ? 2 : 0) | (g1 && g1->lda % 64 ? 4 : 0) |
+                                       (g1 && g1->ldb % 64 ? 8 : 0),
+                                   pairs};
+  int both = 0;
+  if (memo.find(key, &both)) {
+    wide_n[0] = both & 0xffff;
+    wide_n[1] = both >> 16;
+    return;
+  }
+  const DenseGemmArgs* const gs[2] = {&g0, g1};
+  const int n = g1 ? 2 : 1;
+  std::vector<double> load((size_t)pairs);
+  auto makespan = [&](int w0, int w1) {
+    std::fill(load.begin(), load.end(), 0.0);
+    const bool snake = w0 + w1 > 0;
+    int64_t t = 0;
+    for (int seg = 0; seg < 4; ++seg) {
+      if ((seg & 1) >= n) continue;
+      const DenseGemmArgs& g = *gs[seg & 1];
+      const int w = seg & 1 ? w1 : w0, halves = seg < 2 ? 2 : 1;
+      auto bytes = [](int64_t ld) { return ld % 64 ? 1.375 * 16384.0 : 16384.0; };
+      const double k_block = std::max(halves * 530.0, (bytes(g.lda) + halves * bytes(g.ldb)) / 63.0);
+      const double cost = k_block * ((g.K + 63) / 64) + (halves == 2 ? 1500.0 : 500.0);
+      const int64_t end = t + (int64_t)((g.M + 255) / 256) * (seg < 2 ? w : (g.N + 255) / 256 - 2 * w);
+      // whole rounds of the pairs at once
+      const int64_t first = (t + pairs - 1) / pairs, last = end / pairs;
+      auto one = [&](int64_t i) {
+        const int64_t p = i % pairs;
+        load[(size_t)(snake && (i / pairs & 1) ? pairs - 1 - p : p)] += cost;
+      };
+      if (first < last) {
+        for (int64_t i = t; i < first * pairs; ++i) one(i);
+        for (double& v : load) v += cost * (double)(last - first);
+        for (int64_t i = last * pairs; i < end; ++i) one(i);
+      } else {
+        for (int64_t i = t; i < end; ++i) one(i);
+      }
+      t = end;
+    }
+    return *std::max_element(load.begin(), load.end());
+  };
+  wide_n[0] = wide_n[1] = 0;
+  double least = 0.98 * makespan(0, 0);
+  auto most_of = [](const DenseGemmArgs& g) { return g.K > 13 * 64 ? (g.N + 255) / 512 : 0; };
+  const int most[2] = {most_of(g0), g1 ? most_of(*g1) : 0};
+  for (int i = 0; i <= most[0]; ++i)
+    for (int j = 0; j <= most[1]; ++j) {
+      if (g1 && i % (1 + most[0] / 16) != most[0] % (1 + most[0] / 16)) continue;  // two problems: at most 17 x 17 of them
+      if (j % (1 + most[1] / 16) != most[1] % (1 + most[1] / 16)) continue;
+      if (i + j == 0) continue;
+      const double v = makespan(i, j);
+      if (v < least) {
+        least = v;
+        wide_n[0] = i;
+        wide_n[1] = j;
+      }
+    }
+  memo.put(key, wide_n[0] | wide_n[1] << 16);
 }
 
 int bf16_tile(const DenseGemmArgs& g0, const DenseGemmArgs* g1, int forced) {
@@ -807,7 +893,10 @@ int bf16_tile(const DenseGemmArgs& g0, const DenseGemmArgs* g1, int forced) {
     if (gain(4) > gain(2) && tiles128 <= clusters(std::integral_constant<int, 4>())) return kTileSplit4;
     if (tiles128 <= clusters(std::integral_constant<int, 2>())) return kTileSplit2;
   }
-  return tiles128 <= num_sms / 2 ? kTilePair128 : kTilePair256;
+  if (tiles128 <= num_sms / 2) return kTilePair128;
+  int wide_n[2];
+  bf16_wide_tiles(g0, g1, num_sms / 2, wide_n);
+  return wide_n[0] + wide_n[1] ? kTileDouble : kTilePair256;
 }
 
 cudaError_t launch_gemm_bf16(const DenseGemmArgs& g0, const DenseGemmArgs* g1, int tile, cudaStream_t s) {
@@ -815,9 +904,13 @@ cudaError_t launch_gemm_bf16(const DenseGemmArgs& g0, const DenseGemmArgs* g1, i
   const cudaError_t e = sm_count(&num_sms);
   if (e != cudaSuccess) return e;
   const int pairs = num_sms / 2;
-  if (tile == kTileSplit4) return launch_bf16_t<128, 4>(g0, g1, pairs, s);
-  if (tile == kTileSplit2) return launch_bf16_t<128, 2>(g0, g1, pairs, s);
-  return tile == kTilePair128 ? launch_bf16_t<128>(g0, g1, pairs, s) : launch_bf16_t<256>(g0, g1, pairs, s);
+  int wide_n[2] = {0, 0};
+  if (tile == kTileSplit4) return launch_bf16_t<128, 4>(g0, g1, wide_n, pairs, s);
+  if (tile == kTileSplit2) return launch_bf16_t<128, 2>(g0, g1, wide_n, pairs, s);
+  if (tile == kTilePair128) return launch_bf16_t<128>(g0, g1, wide_n, pairs, s);
+  if (tile != kTileDouble) return launch_bf16_t<256>(g0, g1, wide_n, pairs, s);
+  bf16_wide_tiles(g0, g1, pairs, wide_n);
+  return launch_bf16_t<512>(g0, g1, wide_n, pairs, s);
 }
 
 // Test aid: one warp waits, with the given limit, on a barrier nobody arrives at.  The wait runs out, the code lands

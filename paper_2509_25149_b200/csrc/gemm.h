@@ -26,6 +26,7 @@ constexpr int kTileOne128 = 128;   // 128 x 128, one CTA
 constexpr int kTilePair256 = 512;  // 256 x 256
 constexpr int kTilePair128 = 640;  // 256 x 128
 constexpr int kTileWide = 768;     // 256 x 384, needs N >= 256
+constexpr int kTileDouble = 1024;  // BF16: 256 x 512, and 256 x 256 for the columns that are left (chosen by size alone)
 constexpr int kTileSplit2 = 642;   // 256 x 128, a cluster of two pairs per tile shares its contraction (K >= 512)
 constexpr int kTileSplit4 = 644;   // the same with four pairs (K >= 1024)
 cudaError_t launch_gemm(const GemmArgs& g, const void* a_codes, const void* b_codes, int tile, cudaStream_t s);
@@ -57,7 +58,7 @@ cudaError_t device_status_word(unsigned int** word);
 
 // BF16 GEMM D[M x N] = A B^T on CTA pairs (gemm_bf16.cuh) for layers kept in higher precision.
 // a_mn / b_mn = 0: the operand is stored [M or N][K] (contraction contiguous); 1: stored [K][M or N].
-// M, N, K multiples of 8 (tiles of 256 x 256 or 256 x 128, 64 deep, with zero-filled / clipped edges); leading dimensions in
+// M, N, K multiples of 8 (tiles of 256 x 512, 256 x 256 or 256 x 128, 64 deep, with zero-filled / clipped edges); leading dimensions in
 // elements.
 struct DenseGemmArgs {
   const void* a;
@@ -69,7 +70,7 @@ struct DenseGemmArgs {
   int d_is_fp32, accumulate;
 };
 // g1 (may be NULL): a second, independent product in the same launch, its tiles after those of g0
-// The tile of such a launch: kTilePair256, kTilePair128 or a split one (`forced`, where every share has a k-block, or by size)
+// The tile of such a launch: kTilePair256, kTilePair128, kTileDouble or a split one (`forced`, where every share has a k-block, or by size)
 int bf16_tile(const DenseGemmArgs& g0, const DenseGemmArgs* g1, int forced);
 cudaError_t launch_gemm_bf16(const DenseGemmArgs& g0, const DenseGemmArgs* g1, int tile, cudaStream_t s);
 

@@ -25,11 +25,12 @@ namespace dense {
 constexpr int kThreads = 320;       // producer, MMA issuer, 2 x 4 epilogue warps
 constexpr int kOperandBytes = 128 * 128;           // 128 rows (or output indices) x 64 bf16
 constexpr int kStagingBytes = 2 * 16384;
-constexpr int kStages = 6;
 template <int BN, int SPLIT>
 struct Cfg {
+  static constexpr int kStages = BN == 512 ? 4 : 6;
   // A, this CTA's half of B.  (32 KB for the narrow tile as well: 24 KB apart, 1024 x 1280 x 4096 takes 24.3 us, not 23.9)
-  static constexpr int kStageBytes = SPLIT > 1 ? kOperandBytes + BN / 2 * 128 : 2 * kOperandBytes;
+  static constexpr int kStageBytes =
+      SPLIT > 1 ? kOperandBytes + BN / 2 * 128 : BN == 512 ? 3 * kOperandBytes : 2 * kOperandBytes;
   static constexpr int kRecvBytes = (SPLIT - 1) * 128 * (BN / SPLIT) * 4;
   static constexpr int kSmemBytes = kStages * kStageBytes + kStagingBytes + 1024 /*alignment*/ + 256 /*barriers*/ + kRecvBytes;
   static_assert(kSmemBytes <= 232448, "shared memory budget");
@@ -47,6 +48,9 @@ struct Args {
   Problem p[2];
   int n_tiles0;  // tiles of problem 0
   int n_tiles;   // tiles of both problems
+  // BN = 512: tiles 512 columns wide of problem 0 and 1, then the tiles 256 wide of both, and where each of these four ends
+  int wide_n[2];  // column tiles 512 wide of each problem
+  int seg_end[4];
 };
 
 // kind::f16 instruction descriptor: FP32 accumulator (bit 4), BF16 x BF16 (format 1 at bits 7 and 10), operand
@@ -66,7 +70,12 @@ __device__ __forceinline__ void tc2_mma_bf16(uint32_t d_tmem, uint64_t adesc, ui
       : "memory");
 }
 
-// BN: columns of a tile (256 or 128).  SPLIT > 1 (BN = 128): a cluster of SPLIT pairs takes one tile, the only one of its life,
+// BN: columns of a tile (512, 256 or 128).  BN = 512: two accumulators side by side share the loads of A, 48 KB per k-block and
+// CTA instead of 64; what is left of the columns, and what balances the rounds better, is taken in tiles of 256 (bf16_wide_tiles).
+// That is for operands whose rows are no multiple of 128 bytes apart: a 128-byte row of a box then lies across two lines, the SM's
+// path to L2 carries 1.375 x as much in 64-byte pieces (mean over the offsets), and 256-wide tiles wait for it.
+// The two halves of such a tile begin and end apart (kLead): the epilogue drains one while the tensor pipe works on the other.
+// SPLIT > 1 (BN = 128): a cluster of SPLIT pairs takes one tile, the only one of its life,
 // each pair a share of the k-blocks (the exchange: pair::exchange_columns).
 // TWO: the launch has two problems.
 template <int BN, int SPLIT = 1, bool TWO = true>
@@ -76,7 +85,9 @@ __global__ void __cluster_dims__(2 * SPLIT, 1, 1) __launch_bounds__(kThreads, 1)
                           const __grid_constant__ CUtensorMap map_b1, const __grid_constant__ CUtensorMap map_d1,
                           const __grid_constant__ Args g) {
   using namespace pair;
-  constexpr int S = dense::kStages, kStageBytes = dense::Cfg<BN, SPLIT>::kStageBytes;
+  constexpr int S = dense::Cfg<BN, SPLIT>::kStages, kStageBytes = dense::Cfg<BN, SPLIT>::kStageBytes;
+  constexpr bool kDouble = BN == 512;        // two 256-column halves
+  constexpr int HN = kDouble ? 256 : BN;     // columns of an accumulator
   extern __shared__ uint8_t smem_raw[];
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t* base_ptr = smem_raw + (base - smem_u32(smem_raw));
@@ -102,22 +113,43 @@ __global__ void __cluster_dims__(2 * SPLIT, 1, 1) __launch_bounds__(kThreads, 1)
   const int pair_id = blockIdx.x / (2 * SPLIT), n_pairs = gridDim.x / (2 * SPLIT);  // (SPLIT > 1: clusters)
   // ragged edges: loads beyond the operands read zeros, stores beyond D are clipped (both by the tensor maps)
   const int n_tiles = g.n_tiles;
+  auto prob_of = [&](int tile) {
+    if (kDouble) return TWO ? ((tile >= g.seg_end[0] && tile < g.seg_end[1]) || tile >= g.seg_end[2] ? 1 : 0) : 0;
+    return TWO && tile >= g.n_tiles0 ? 1 : 0;
+  };
+  auto halves_of = [&](int tile) { return kDouble && tile < g.seg_end[1] ? 2 : 1; };
   auto k_begin = [&](int tile, int s) {  // first k-block of share s
-    const int n = (g.p[TWO && tile >= g.n_tiles0 ? 1 : 0].K + 63) / 64;
+    const int n = (g.p[prob_of(tile)].K + 63) / 64;
     return SPLIT > 1 ? n * s / SPLIT : n * s;
   };
-  // groups of eight row-blocks sweep all column-blocks before the next group starts (L2 reuse of A and B)
+  // rounds of the pairs; kDouble: odd ones in reverse order, which evens out tiles of different cost
+  auto next_tile = [&](int rnd) { return rnd * n_pairs + (kDouble && (rnd & 1) ? n_pairs - 1 - pair_id : pair_id); };
+  // groups of eight row-blocks sweep all column-blocks before the next group starts (L2 reuse of A and B);
+  // n_blk: the tile's first column in units of HN
   constexpr int kGroupM = 8;
   auto tile_coords = [&](int tile, int& prob, int& m_blk, int& n_blk) {
-    prob = TWO && tile >= g.n_tiles0 ? 1 : 0;
-    if (prob) tile -= g.n_tiles0;
-    const int tiles_m = (g.p[prob].M + 255) / 256, tiles_n = (g.p[prob].N + BN - 1) / BN;
+    prob = prob_of(tile);
+    int tiles_n = (g.p[prob].N + HN - 1) / HN, n_first = 0, n_step = 1;
+    if constexpr (kDouble) {
+      const int seg = (tile >= g.seg_end[0]) + (tile >= g.seg_end[1]) + (tile >= g.seg_end[2]);
+      if (seg) tile -= g.seg_end[seg - 1];
+      if (seg < 2) {
+        tiles_n = g.wide_n[prob];
+        n_step = 2;
+      } else {
+        n_first = 2 * g.wide_n[prob];
+        tiles_n -= n_first;
+      }
+    } else if (prob) {
+      tile -= g.n_tiles0;
+    }
+    const int tiles_m = (g.p[prob].M + 255) / 256;
     const int per_group = kGroupM * tiles_n;
     const int grp = tile / per_group, in_grp = tile - grp * per_group;
     const int m0 = grp * kGroupM;
     const int gm = (tiles_m - m0 < kGroupM) ? (tiles_m - m0) : kGroupM;
     m_blk = m0 + in_grp % gm;
-    n_blk = in_grp / gm;
+    n_blk = n_first + n_step * (in_grp / gm);
   };
 
   if (threadIdx.x == 0) {
@@ -156,11 +188,12 @@ __global__ void __cluster_dims__(2 * SPLIT, 1, 1) __launch_bounds__(kThreads, 1)
       int stage = 0;
       uint32_t phase = 0;
       bool ok = true;
-      for (int tile = pair_id; tile < n_tiles && ok; tile += n_pairs) {
+      for (int rnd = 0, tile = pair_id; tile < n_tiles && ok; tile = next_tile(++rnd)) {
         int prob, m_blk, n_blk;
         tile_coords(tile, prob, m_blk, n_blk);
         const int row_a = m_blk * 256 + (int)rank * 128;  // this CTA's rows of A
-        const int row_b = n_blk * BN + (int)rank * (BN / 2);  // this CTA's half of the B tile
+        const int row_b = n_blk * HN + (int)rank * (HN / 2);  // this CTA's half of the B tile (of its first 256 columns)
+        const int halves = halves_of(tile);
         const int k_end = k_begin(tile, split + 1);
         // One copy of the loop for each problem of the launch, with its tensor maps and layouts at fixed places of the parameter
         // bank: with the maps picked by pointer the loads of a stage were issued so late that a pair could not go faster even
@@ -170,18 +203,23 @@ __global__ void __cluster_dims__(2 * SPLIT, 1, 1) __launch_bounds__(kThreads, 1)
             if (!(ok = mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag, 0x900u + stage))) break;
             const uint32_t st = base + stage * kStageBytes;
             const uint32_t bar = map_to_cta(full_bar(stage), leader_cta);  // the leader's barrier counts both CTAs' operands
-            mbar_expect_tx_cluster(bar, dense::kOperandBytes + BN / 2 * 128);
+            mbar_expect_tx_cluster(bar, dense::kOperandBytes + (kDouble ? halves * dense::kOperandBytes : BN / 2 * 128));
             if (pr.a_mn) {
               tma_load_2d_pair(st, map_a, row_a, kb * 64, bar);
               tma_load_2d_pair(st + 8192, map_a, row_a + 64, kb * 64, bar);
             } else {
               tma_load_2d_pair(st, map_a, kb * 64, row_a, bar);
             }
-            if (pr.b_mn) {
-              tma_load_2d_pair(st + dense::kOperandBytes, map_b, row_b, kb * 64, bar);
-              if (BN == 256) tma_load_2d_pair(st + dense::kOperandBytes + 8192, map_b, row_b + 64, kb * 64, bar);
-            } else {
-              tma_load_2d_pair(st + dense::kOperandBytes, map_b, kb * 64, row_b, bar);
+#pragma unroll
+            for (int h = 0; h < (kDouble ? 2 : 1); ++h) {
+              if (h >= halves) break;
+              const uint32_t st_b = st + (1 + h) * dense::kOperandBytes;
+              if (pr.b_mn) {
+                tma_load_2d_pair(st_b, map_b, row_b + 256 * h, kb * 64, bar);
+                if (HN == 256) tma_load_2d_pair(st_b + 8192, map_b, row_b + 256 * h + 64, kb * 64, bar);
+              } else {
+                tma_load_2d_pair(st_b, map_b, kb * 64, row_b + 256 * h, bar);
+              }
             }
             if (++stage == S) {
               stage = 0;
@@ -205,43 +243,89 @@ __global__ void __cluster_dims__(2 * SPLIT, 1, 1) __launch_bounds__(kThreads, 1)
       // 128-byte swizzle (high word).  K-major: 8-row groups 1024 bytes apart, leading offset unused.  MN-major:
       // 64-index boxes 8192 bytes apart (leading), 8-row k groups 1024 bytes apart (stride).
       const uint32_t a_lo_base = (base >> 4) & 0x3fffu, b_lo_base = ((base + dense::kOperandBytes) >> 4) & 0x3fffu;
-      int it = 0;
-      for (int tile = pair_id; tile < n_tiles && ok; tile += n_pairs, ++it) {
-        const int buf = it & 1;
-        if (!(ok = mbar_wait_cluster(acce_bar(buf), ((acc_phase >> buf) & 1u) ^ 1u, abort_flag, 0xB00u + buf))) break;
+      int buf = 0;
+      auto acc_free = [&](int b) {
+        return mbar_wait_cluster(acce_bar(b), ((acc_phase >> b) & 1u) ^ 1u, abort_flag, 0xB00u + b);
+      };
+      for (int rnd = 0, tile = pair_id; tile < n_tiles && ok; tile = next_tile(++rnd)) {
+        const bool both = halves_of(tile) == 2;
+        if (both) buf = 0;
+        if (!(ok = acc_free(buf))) break;
         tc_fence_after();
-        const uint32_t d_t = tmem + buf * 256;
         const int k_blocks = k_begin(tile, split + 1) - k_begin(tile, split);
         // (one copy of the loop for each problem, as in the producer)
         auto main_loop = [&](const Problem& pr) {
-          const uint32_t idesc = instr_desc_bf16(256, BN, pr.a_mn, pr.b_mn);
+          const uint32_t idesc = instr_desc_bf16(256, HN, pr.a_mn, pr.b_mn);
           const uint32_t a_lo0 = a_lo_base | ((pr.a_mn ? (8192u >> 4) : 1u) << 16);
           const uint32_t b_lo0 = b_lo_base | ((pr.b_mn ? (8192u >> 4) : 1u) << 16);
           const uint32_t a_step = pr.a_mn ? (2048u >> 4) : (32u >> 4);  // one K = 16 instruction further
           const uint32_t b_step = pr.b_mn ? (2048u >> 4) : (32u >> 4);
-          for (int kb = 0; kb < k_blocks; ++kb) {
-            if (!(ok = mbar_wait_cluster(full_bar(stage), phase, abort_flag, 0xA00u + stage))) break;
-            tc_fence_after();
-            const uint32_t a_lo = a_lo0 + stage * (kStageBytes >> 4);
-            const uint32_t b_lo = b_lo0 + stage * (kStageBytes >> 4);
+          auto mma = [&](int st, int half, int acc, bool first) {  // a k-block of one half
+            const uint32_t a_lo = a_lo0 + st * (kStageBytes >> 4);
+            const uint32_t b_lo = b_lo0 + st * (kStageBytes >> 4) + half * (dense::kOperandBytes >> 4);
 #pragma unroll
             for (int j = 0; j < 4; ++j)
-              tc2_mma_bf16(d_t, make_desc(a_lo + j * a_step, kDescHiOperand), make_desc(b_lo + j * b_step, kDescHiOperand),
-                           idesc, (kb > 0 || j > 0) ? 1u : 0u);
+              tc2_mma_bf16(tmem + acc * 256, make_desc(a_lo + j * a_step, kDescHiOperand),
+                           make_desc(b_lo + j * b_step, kDescHiOperand), idesc, (!first || j > 0) ? 1u : 0u);
+          };
+          auto landed = [&](int st, uint32_t ph) {
+            if (!(ok = mbar_wait_cluster(full_bar(st), ph, abort_flag, 0xA00u + st))) return false;
+            tc_fence_after();
+            return true;
+          };
+          auto release = [&] {
             tc2_commit_both(empty_bar(stage), pair_mask);  // both CTAs' stages are free once these MMAs have read them
             if (++stage == S) {
               stage = 0;
               phase ^= 1u;
             }
+          };
+          if constexpr (kDouble) {
+            if (both) {
+              // runs of up to kLead k-blocks of the first half and then of the second at either end of the tile, half by
+              // half in between
+              constexpr int kLead = 3;
+              for (int kb = 0; kb < k_blocks;) {
+                const int left = k_blocks - kb;
+                const int run = kb == 0 || left <= kLead ? min(left, kLead) : 1;
+                for (int i = 0; i < run; ++i) {
+                  const int st = stage + i < S ? stage + i : stage + i - S;
+                  if (!landed(st, phase ^ (stage + i < S ? 0u : 1u))) return;
+                  mma(st, 0, 0, kb + i == 0);
+                }
+                if (kb + run == k_blocks) tc2_commit_both(accf_bar(0), pair_mask);  // the first accumulator is complete
+                if (kb == 0) {
+                  if (!(ok = acc_free(1))) return;
+                  tc_fence_after();
+                }
+                for (int i = 0; i < run; ++i) {
+                  mma(stage, 1, 1, kb + i == 0);
+                  release();
+                }
+                kb += run;
+              }
+              return;
+            }
+          }
+          for (int kb = 0; kb < k_blocks; ++kb) {
+            if (!landed(stage, phase)) return;
+            mma(stage, 0, buf, kb == 0);
+            release();
           }
         };
-        if (!TWO || tile < g.n_tiles0)
+        if (!TWO || prob_of(tile) == 0)
           main_loop(g.p[0]);
         else
           main_loop(g.p[1]);
         if (!ok) break;
-        tc2_commit_both(accf_bar(buf), pair_mask);  // this accumulator is complete in both CTAs
-        acc_phase ^= 1u << buf;
+        if (both) {
+          tc2_commit_both(accf_bar(1), pair_mask);
+          acc_phase ^= 3u;
+        } else {
+          tc2_commit_both(accf_bar(buf), pair_mask);  // this accumulator is complete in both CTAs
+          acc_phase ^= 1u << buf;
+          buf ^= 1;
+        }
       }
     }
   } else {
@@ -253,11 +337,18 @@ __global__ void __cluster_dims__(2 * SPLIT, 1, 1) __launch_bounds__(kThreads, 1)
     uint32_t acc_phase = 0;
     const int row_in_tile = quad * 32 + lane;
     const uint32_t stage_buf = staging + half * 16384;
-    int it = 0, last_prob = 0;
-    for (int tile = pair_id; tile < n_tiles; tile += n_pairs, ++it) {
-      const int buf = it & 1;
+    int buf = 0, last_prob = 0, halves = 1;
+    // (kDouble: a tile comes up once for each of its halves, the second time without a step of the walk)
+    for (int rnd = 0, half_no = 0, tile = pair_id; tile < n_tiles; tile = half_no ? tile : next_tile(++rnd)) {
       int prob, m_blk, n_blk;
       tile_coords(tile, prob, m_blk, n_blk);
+      if constexpr (kDouble) {
+        halves = halves_of(tile);
+        if (halves == 2) {
+          buf = half_no;
+          n_blk += half_no;
+        }
+      }
       const CUtensorMap* map_d = prob ? &map_d1 : &map_d0;
       const bool drain = prob != last_prob;  // the problems of a launch may have different output types
       last_prob = prob;
@@ -266,10 +357,10 @@ __global__ void __cluster_dims__(2 * SPLIT, 1, 1) __launch_bounds__(kThreads, 1)
       if (group_gave_up(abort_flag, bar_id, 128)) break;
       tc_fence_after();
       const int row0 = m_blk * 256 + (int)rank * 128;
-      const uint32_t t_row = tmem + ((uint32_t)(quad * 32) << 16) + buf * 256 + half * (BN / 2);
-      uint32_t r[BN / 2];
+      const uint32_t t_row = tmem + ((uint32_t)(quad * 32) << 16) + buf * 256 + half * (HN / 2);
+      uint32_t r[HN / 2];
 #pragma unroll
-      for (int q = 0; q < BN / 32; ++q) tc_ld16(t_row + q * 16, *reinterpret_cast<uint32_t(*)[16]>(&r[q * 16]));
+      for (int q = 0; q < HN / 32; ++q) tc_ld16(t_row + q * 16, *reinterpret_cast<uint32_t(*)[16]>(&r[q * 16]));
       tc_wait_ld();
       tc_fence_before();
       __syncwarp();
@@ -286,12 +377,14 @@ __global__ void __cluster_dims__(2 * SPLIT, 1, 1) __launch_bounds__(kThreads, 1)
         else
           store_half<false, false, kCols>(v, 1.0f, et, bar_id, row_in_tile, stage_buf, map_d, xs, row0, g.p[prob].accumulate, drain);
       } else if (g.p[prob].d_is_fp32)
-        store_half<true, false, BN / 2>(r, 1.0f, et, bar_id, row_in_tile, stage_buf, map_d, n_blk * BN + half * (BN / 2),
+        store_half<true, false, HN / 2>(r, 1.0f, et, bar_id, row_in_tile, stage_buf, map_d, n_blk * HN + half * (HN / 2),
                                         row0, g.p[prob].accumulate, drain);
       else
-        store_half<false, false, BN / 2>(r, 1.0f, et, bar_id, row_in_tile, stage_buf, map_d, n_blk * BN + half * (BN / 2),
+        store_half<false, false, HN / 2>(r, 1.0f, et, bar_id, row_in_tile, stage_buf, map_d, n_blk * HN + half * (HN / 2),
                                          row0, g.p[prob].accumulate, drain);
       acc_phase ^= 1u << buf;
+      buf = halves == 2 ? 0 : buf ^ 1;
+      if (kDouble) half_no = halves == 2 ? half_no ^ 1 : 0;
     }
     if (et == 0) bulk_wait_all<0>();  // all stores have left shared memory and are visible
   }

@@ -181,3 +181,49 @@ def test_the_rule_splits_where_it_says():
             assert B.nvfp4_gemm_tile(bf16, *size, fp32) in want, (bf16, size)
     for bf16, size in [(False, (64, 128, 256)), (False, (128, 128, 128)), (True, (4, 8, 8)), (True, (8, 8, 0))]:
         assert B.nvfp4_gemm_tile(bf16, *size, False) == -1
+
+
+# one column tile of 512 and many of 256; three and several; only such tiles and eight columns; 15 to 17 k-blocks, the last of 8,
+# 32 and 40 elements; none of the row lengths a multiple of 128 bytes
+@pytest.mark.parametrize("shape", [(1040, 3664, 904), (1384, 3624, 928), (2056, 7176, 1064)])
+def test_bf16_products_on_512_wide_tiles(shape):
+    M, N, K = shape
+    gen = torch.Generator("cuda").manual_seed(M + N + K)
+    a, b = (torch.randn(s, generator=gen, device="cuda").to(torch.bfloat16) for s in ((M, K), (N, K)))
+    want, T = a.double() @ b.double().T, a.double().abs() @ b.double().abs().T
+    if torch.cuda.get_device_properties(0).multi_processor_count == 148:
+        assert B.nvfp4_gemm_tile(True, M, N, K, False) == 1024
+    for layouts in ((0, 0), (0, 1), (1, 0), (1, 1)):
+        ops = [t.T.contiguous() if mn else t for t, mn in zip((a, b), layouts)]
+        for dtype in (torch.float32, torch.bfloat16):
+            wide = torch.full((M + 8, N + 8), 7.0, dtype=dtype, device="cuda")
+            D = wide[:M, :N]
+            B.nvfp4_gemm_bf16(*ops, D, *layouts)
+            B.nvfp4_device_status()
+            # K roundings of what the magnitudes add up to at most, and the rounding of the output
+            bound = K * 2.0 ** -23 * T + (2.0 ** -8 * want.abs() if dtype == torch.bfloat16 else 0)
+            assert torch.all((D.double() - want).abs() <= bound + 1e-30)
+            assert torch.all(wide[M:] == 7.0) and torch.all(wide[:, N:] == 7.0)
+            if dtype == torch.float32:
+                once = D.clone()
+                B.nvfp4_gemm_bf16(*ops, D, *layouts, accumulate=True)
+                assert torch.equal(D, once + once)
+
+
+@pytest.mark.parametrize("shape", [(1592, 1392, 2040), (1544, 1680, 1912), (1592, 1552, 2128)])
+def test_bf16_backward_call_on_512_wide_tiles(shape):
+    """Tiles of both widths and of both products in one launch; each product has the bits that it has alone."""
+    M, N, K = shape
+    gen = torch.Generator("cuda").manual_seed(M + N + K)
+    dy, x, w = (torch.randn(s, generator=gen, device="cuda").to(torch.bfloat16) for s in ((M, N), (M, K), (N, K)))
+    dx, dw = torch.empty_like(x), torch.empty((N, K), device="cuda")
+    one, two = torch.empty_like(dx), torch.empty_like(dw)
+    B.nvfp4_linear_bf16_bwd(dy, x, w, K, dx, dw, False)
+    B.nvfp4_linear_bf16_bwd(dy, None, w, K, one, None, False)
+    B.nvfp4_linear_bf16_bwd(dy, x, None, K, None, two, False)
+    B.nvfp4_device_status()
+    T = dy.double().abs() @ w.double().abs()
+    assert torch.all((dx.double() - dy.double() @ w.double()).abs() <= N * 2.0 ** -23 * T + 2.0 ** -8 * T)
+    T = dy.double().abs().T @ x.double().abs()
+    assert torch.all((dw.double() - dy.double().T @ x.double()).abs() <= M * 2.0 ** -23 * T + 1e-30)
+    assert torch.equal(dx, one) and torch.equal(dw, two)
