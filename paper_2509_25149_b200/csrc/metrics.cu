@@ -92,16 +92,15 @@ __global__ void __launch_bounds__(kThreads, 2) quant_error_kernel(const uint16_t
   const int64_t n_sb = MX ? (cols >> 5) : n_cb;   // scale blocks per row
   const float s_dec_t = MX ? 1.f : global[1];
   double err = 0.0, ref = 0.0;
-  Walk w(blockIdx.x * (int64_t)blockDim.x + threadIdx.x, (int64_t)gridDim.x * blockDim.x, n_cb);
-  constexpr int kDepth = 3;  // chunks whose loads are in flight
-  uint32_t raw[kDepth][8];
-  uint2 codes2[kDepth];
-  uint32_t byte[kDepth];
-  float s_dec[kDepth];
-  bool live[kDepth];
+  const int64_t first = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
+  Walk w(first, step, n_cb);
+  constexpr int kDepth = 2;  // chunks whose loads are in flight
+  uint32_t raw[kDepth][8] = {};
+  uint2 codes2[kDepth] = {};
+  uint32_t byte[kDepth] = {};
+  float s_dec[kDepth] = {};
   auto load = [&](int u) {
-    live[u] = w.r < rows;
-    if (live[u]) {
+    if (w.r < rows) {
       const int64_t r = w.r, cb = w.c, sb = MX ? (cb >> 1) : cb;
       ldg256_stream(x + r * ld + cb * 16, raw[u]);
       codes2[u] = __ldg(reinterpret_cast<const uint2*>(codes + r * (cols >> 1) + cb * 8));
@@ -110,36 +109,41 @@ __global__ void __launch_bounds__(kThreads, 2) quant_error_kernel(const uint16_t
     }
     w.next();
   };
+  auto add = [&](int u) {
+    float sf;
+    if (MX) {
+      sf = byte[u] == 0 ? __uint_as_float(0x00400000u) : __uint_as_float(byte[u] << 23);  // 2^(byte - 127)
+    } else {
+      uint32_t h2;
+      asm("cvt.rn.f16x2.e4m3x2 %0, %1;" : "=r"(h2) : "h"((uint16_t)byte[u]));
+      sf = __half2float(__ushort_as_half((unsigned short)(h2 & 0xffffu)));
+    }
+    const float neg = -__fmul_rn(sf, s_dec[u]);
+    float2 e = make_float2(0.f, 0.f), n = e;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const float2 q = e2m1x2_values(((k < 4 ? codes2[u].x : codes2[u].y) >> (8 * (k & 3))) & 0xffu);
+      const float2 xv = make_float2(bf16_lo(raw[u][k]), bf16_hi(raw[u][k]));
+      const float2 d = fma2(q, make_float2(neg, neg), xv);
+      e = fma2(d, d, e);
+      n = fma2(xv, xv, n);
+    }
+    err += (double)(e.x + e.y);
+    ref += (double)(n.x + n.y);
+  };
+  const int64_t units = rows * n_cb;
+  int64_t left = first < units ? (units - first + step - 1) / step : 0;  // chunks of this thread
 #pragma unroll
   for (int u = 0; u < kDepth; ++u) load(u);
-  while (live[0]) {
-#pragma unroll
-    for (int u = 0; u < kDepth; ++u) {
-      if (live[u]) {
-        float sf;
-        if (MX) {
-          sf = byte[u] == 0 ? __uint_as_float(0x00400000u) : __uint_as_float(byte[u] << 23);  // 2^(byte - 127)
-        } else {
-          uint32_t h2;
-          asm("cvt.rn.f16x2.e4m3x2 %0, %1;" : "=r"(h2) : "h"((uint16_t)byte[u]));
-          sf = __half2float(__ushort_as_half((unsigned short)(h2 & 0xffffu)));
-        }
-        const float neg = -__fmul_rn(sf, s_dec[u]);
-        float2 e = make_float2(0.f, 0.f), n = e;
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-          const float2 q = e2m1x2_values(((k < 4 ? codes2[u].x : codes2[u].y) >> (8 * (k & 3))) & 0xffu);
-          const float2 xv = make_float2(bf16_lo(raw[u][k]), bf16_hi(raw[u][k]));
-          const float2 d = fma2(q, make_float2(neg, neg), xv);
-          e = fma2(d, d, e);
-          n = fma2(xv, xv, n);
-        }
-        err += (double)(e.x + e.y);
-        ref += (double)(n.x + n.y);
-      }
-      load(u);  // the slot's next chunk, while the other slots' are worked on
-    }
+  // Two chunks a turn without a branch between them, so that they overlap (three, each in a branch of its own: 8192 x 5120 21.2
+  // us, now 20.4; 20480 x 5120 53.5, now 50.5)
+  for (; left > 1; left -= 2) {
+    add(0);
+    load(0);  // the slot's next chunk, while the other's is worked on
+    add(1);
+    load(1);
   }
+  if (left > 0) add(0);
   block_reduce_add(err, ref, out);
 }
 
