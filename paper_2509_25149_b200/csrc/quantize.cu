@@ -354,26 +354,6 @@ struct QuantSmem {
   static constexpr int bytes(bool rand, bool row_codes) { return kRand + (rand ? 128 * TC : row_codes ? 64 * TC : 0); }
 };
 
-// Eq. 2-3: the stored E4M3 byte of a block, S_b = e4m3(fl(fl(amax_b / 6) * s_enc)).  TINY: s_enc > kPlainDivisionLimit; the other
-// form has no branch.  A branch per block (this one, and one around the transposed copy's own draws) cut the code of a tile into
-// pieces that could not overlap, at four warps per scheduler: activation of 8192 x 5120 43.5 -> 41.0 us without, gradient 59.2 ->
-// 55.6, 4096 x 4096 20.2 -> 19.4 and 26.4 -> 24.5.
-template <bool TINY>
-__device__ __forceinline__ uint32_t block_scale_byte(float amax_b, float s_enc) {
-  const float t = __fmul_rn(TINY ? div6_rn(amax_b) : div6_fast(amax_b), s_enc);
-  uint16_t packed;
-  asm("cvt.rn.satfinite.e4m3x2.f32 %0, %1, %2;" : "=h"(packed) : "f"(0.f), "f"(t));
-  return packed;
-}
-// the text after Eq. 3: encode scale of a block from its stored byte, fl(1 / fl(fp32(S_b) * s_dec)), 0 for S_b = 0
-__device__ __forceinline__ float encode_scale_of_byte(uint32_t byte, float s_dec) {
-  uint32_t h2;
-  asm("cvt.rn.f16x2.e4m3x2 %0, %1;" : "=r"(h2) : "h"((uint16_t)byte));
-  const float sf = __half2float(__ushort_as_half((unsigned short)(h2 & 0xffffu)));
-  const float d = __fmul_rn(sf, s_dec);
-  return (byte == 0u) ? 0.0f : fminf(__frcp_rn(d), kFltMax);
-}
-
 // OWN_DRAWS: 16x16 blocks whose transposed copy is rounded with draws of its own.
 template <bool HAS_ROW, bool HAS_COL, bool BLOCK2D, bool RHT_ROW, bool RHT_COL, bool SR, int TC, bool F32 = false,
           bool PARTS = false, bool OWN_DRAWS = false>
