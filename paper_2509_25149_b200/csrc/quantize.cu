@@ -611,8 +611,9 @@ __device__ __forceinline__ void quantize_tiles(const CUtensorMap* src_map, const
         }
       }
       // Phase 2 of a warp reads only what the same warp staged in phase 1 (its own 16 rows of the tile, their random
-      // bytes, its 16x16 scales), so the warps need not wait for each other here
-      __syncwarp();
+      // bytes, its 16x16 scales), so the warps need not wait for each other here.  (An activation's reads the tile alone, and the
+      // two phases may overlap: 4096 x 4096 19.4 -> 19.1 us.)
+      if (SR || BLOCK2D) __syncwarp();
 
       // ---------------------------------------------------------------- phase 2 ----
       if constexpr (kNibbleTranspose) {
