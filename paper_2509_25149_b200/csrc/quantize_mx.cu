@@ -4,6 +4,8 @@
 // The recipe options are those of Section 4 at this format's block size: 1x32 blocks for activations and gradients,
 // 32x32 blocks for weights, a 32-point random Hadamard transform on the transposed (weight-gradient) copy, stochastic
 // rounding with the same Philox draws as the NVFP4 kernel.
+#include <type_traits>
+
 #include "async_ptx.cuh"
 #include "quantize.h"
 #include "quantize_common.cuh"
@@ -125,146 +127,163 @@ __global__ void __launch_bounds__(256, CTAS)
     uint8_t* const sf_col = smem + S::kSfCol + buf * 512;
     quant_wait(bar0 + 8 * buf, (uint32_t)(j >> 1) & 1u, abort_flag, a.status);
 
-    // ---------------------------------------------------------------- phase 1 ----
-    uint32_t raw[4][8];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const uint4 h0 = *reinterpret_cast<const uint4*>(tile_buf + rl * 256 + cb * 32 + i * 1024);
-      const uint4 h1 = *reinterpret_cast<const uint4*>(tile_buf + rl * 256 + cb * 32 + i * 1024 + 16);
-      raw[i][0] = h0.x; raw[i][1] = h0.y; raw[i][2] = h0.z; raw[i][3] = h0.w;
-      raw[i][4] = h1.x; raw[i][5] = h1.y; raw[i][6] = h1.z; raw[i][7] = h1.w;
-    }
-    float am[4];  // amax of the 1x32 block each chunk belongs to (the chunk of the neighbouring lane completes it)
-    if (HAS_ROW || BLOCK2D) {
+    const bool full_tile = row0 + 128 <= a.rows && col0 + 128 <= a.cols;
+    // Two copies: a full tile's code has no branch around its stores (nor, now, one around the transposed copy's own draws), and a
+    // chunk overlaps with the next: gradient of 4096 x 4096 19.8 -> 17.7 us, 8192 x 20480 166 -> 152; activation of 8192 x 5120
+    // 31.0 -> 29.2.  Not for weights: few tiles lose what many gain (2304 x 3328 6.0 -> 6.2 us, 8192 x 5120 24.9 -> 24.4).
+    auto phases_1_2 = [&](auto full_c) {
+      constexpr bool FULL = decltype(full_c)::value;
+      // ---------------------------------------------------------------- phase 1 ----
+      uint32_t raw[4][8];
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
-        uint32_t acc = 0;
-#pragma unroll
-        for (int k = 0; k < 8; ++k) acc = absmax_bf16x2(acc, raw[i][k]);
-        const float own = amax_of_pair(acc);
-        am[i] = fmaxf(own, __shfl_xor_sync(0xffffffffu, own, 1));
+        const uint4 h0 = *reinterpret_cast<const uint4*>(tile_buf + rl * 256 + cb * 32 + i * 1024);
+        const uint4 h1 = *reinterpret_cast<const uint4*>(tile_buf + rl * 256 + cb * 32 + i * 1024 + 16);
+        raw[i][0] = h0.x; raw[i][1] = h0.y; raw[i][2] = h0.z; raw[i][3] = h0.w;
+        raw[i][4] = h1.x; raw[i][5] = h1.y; raw[i][6] = h1.z; raw[i][7] = h1.w;
       }
-    }
-    if (BLOCK2D) {
-      // 32x32 blocks: the warp's 16 rows first, then the other warp of the pair's through shared memory
-      float m = fmaxf(fmaxf(am[0], am[1]), fmaxf(am[2], am[3]));
-      m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 8));
-      m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 16));
-      if (lane < 8 && !(lane & 1)) blk[warp * 4 + (cb >> 1)] = m;
-      pair_sync();
-      m = fmaxf(blk[warp * 4 + (cb >> 1)], blk[(warp ^ 1) * 4 + (cb >> 1)]);
+      float am[4];  // amax of the 1x32 block each chunk belongs to (the chunk of the neighbouring lane completes it)
+      if (HAS_ROW || BLOCK2D) {
 #pragma unroll
-      for (int i = 0; i < 4; ++i) am[i] = m;
-    }
-    const bool col_ok = col0 + cb * 16 < a.cols;
-    uint64_t g = 0;
-    if (SR) g = (uint64_t)(row0 + rl) * (uint64_t)n_cb + (uint64_t)((col0 >> 4) + cb);
-    uint8_t* r_out = HAS_ROW ? a.r_codes + (row0 + rl) * r_pitch + ((col0 + cb * 16) >> 1) : nullptr;
+        for (int i = 0; i < 4; ++i) {
+          uint32_t acc = 0;
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const bool ok = col_ok && row0 + rl + 4 * i < a.rows;
-      uint32_t rnd[4] = {0u, 0u, 0u, 0u};
-      if (SR) {
-        const uint64_t gi = g + (uint64_t)(4 * i) * (uint64_t)n_cb;
-        const uint4 q = philox4x32_10((uint32_t)gi, (uint32_t)(gi >> 32), a.off_lo, a.off_hi, a.rk);
-        rnd[0] = q.x; rnd[1] = q.y; rnd[2] = q.z; rnd[3] = q.w;
-        if (kStageRand) {
-          uint4 qc = q;
-          if (a.off_hi_col != a.off_hi)
-            qc = philox4x32_10((uint32_t)gi, (uint32_t)(gi >> 32), a.off_lo, a.off_hi_col, a.rk);
-          *reinterpret_cast<uint4*>(smem + S::kRand + (rl + 4 * i) * 128 + cb * 16) = make_uint4(~qc.x, ~qc.y, ~qc.z, ~qc.w);
+          for (int k = 0; k < 8; ++k) acc = absmax_bf16x2(acc, raw[i][k]);
+          const float own = amax_of_pair(acc);
+          am[i] = fmaxf(own, __shfl_xor_sync(0xffffffffu, own, 1));
         }
       }
-      if (HAS_ROW) {
-        float f[16];
+      if (BLOCK2D) {
+        // 32x32 blocks: the warp's 16 rows first, then the other warp of the pair's through shared memory
+        float m = fmaxf(fmaxf(am[0], am[1]), fmaxf(am[2], am[3]));
+        m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 8));
+        m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 16));
+        if (lane < 8 && !(lane & 1)) blk[warp * 4 + (cb >> 1)] = m;
+        pair_sync();
+        m = fmaxf(blk[warp * 4 + (cb >> 1)], blk[(warp ^ 1) * 4 + (cb >> 1)]);
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
-          f[2 * k] = bf16_lo(raw[i][k]);
-          f[2 * k + 1] = bf16_hi(raw[i][k]);
-        }
-        uint32_t byte;
-        float enc;
-        mx_scales(am[i], byte, enc);
-        const uint2 codes = convert16<SR>(f, enc, Nu14FromWords{rnd});
-        if (ok) *reinterpret_cast<uint2*>(r_out + (int64_t)(4 * i) * r_pitch) = codes;
-        if (kNibbleTranspose)
-          *reinterpret_cast<uint2*>(smem + S::kRand + (rl + 4 * i) * 64 + cb * 8) = ok ? codes : make_uint2(0u, 0u);
-        if (!(cb & 1)) sf_row[sf_row_pos + i * sf_row_step] = (uint8_t)byte;
-        if (kNibbleTranspose && i == 0 && lane < 8 && !(cb & 1)) smem[S::kBlkByte + warp * 4 + (cb >> 1)] = (uint8_t)byte;
+        for (int i = 0; i < 4; ++i) am[i] = m;
       }
-    }
-    if (kStageRand || kNibbleTranspose) pair_sync();  // (otherwise phase 2 reads the tile alone)
+      const bool col_ok = FULL || col0 + cb * 16 < a.cols;
+      const int rows_left = FULL ? 128 : (int)(a.rows - row0) - rl;
+      uint64_t g = 0;
+      if (SR) g = (uint64_t)(row0 + rl) * (uint64_t)n_cb + (uint64_t)((col0 >> 4) + cb);
+      uint8_t* r_out = HAS_ROW ? a.r_codes + (row0 + rl) * r_pitch + ((col0 + cb * 16) >> 1) : nullptr;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const bool ok = FULL || (col_ok && 4 * i < rows_left);
+        uint32_t rnd[4] = {0u, 0u, 0u, 0u};
+        if (SR) {
+          const uint64_t gi = g + (uint64_t)(4 * i) * (uint64_t)n_cb;
+          const uint4 q = philox4x32_10((uint32_t)gi, (uint32_t)(gi >> 32), a.off_lo,
+                                        HAS_ROW ? a.off_hi : a.off_hi_col, a.rk);
+          rnd[0] = q.x; rnd[1] = q.y; rnd[2] = q.z; rnd[3] = q.w;
+          if (kStageRand)
+            *reinterpret_cast<uint4*>(smem + S::kRand + (rl + 4 * i) * 128 + cb * 16) = make_uint4(~q.x, ~q.y, ~q.z, ~q.w);
+        }
+        if (HAS_ROW) {
+          float f[16];
+#pragma unroll
+          for (int k = 0; k < 8; ++k) {
+            f[2 * k] = bf16_lo(raw[i][k]);
+            f[2 * k + 1] = bf16_hi(raw[i][k]);
+          }
+          uint32_t byte;
+          float enc;
+          mx_scales(am[i], byte, enc);
+          const uint2 codes = convert16<SR>(f, enc, Nu14FromWords{rnd});
+          if (ok) *reinterpret_cast<uint2*>(r_out + (int64_t)(4 * i) * r_pitch) = codes;
+          if (kNibbleTranspose)
+            *reinterpret_cast<uint2*>(smem + S::kRand + (rl + 4 * i) * 64 + cb * 8) = ok ? codes : make_uint2(0u, 0u);
+          if (!(cb & 1)) sf_row[sf_row_pos + i * sf_row_step] = (uint8_t)byte;
+          if (kNibbleTranspose && i == 0 && lane < 8 && !(cb & 1)) smem[S::kBlkByte + warp * 4 + (cb >> 1)] = (uint8_t)byte;
+        }
+      }
+      if (kStageRand && HAS_ROW && a.off_hi_col != a.off_hi) {  // draws of its own for the transposed copy
+#pragma unroll 1
+        for (int i = 0; i < 4; ++i) {
+          const uint64_t gi = g + (uint64_t)(4 * i) * (uint64_t)n_cb;
+          const uint4 q = philox4x32_10((uint32_t)gi, (uint32_t)(gi >> 32), a.off_lo, a.off_hi_col, a.rk);
+          *reinterpret_cast<uint4*>(smem + S::kRand + (rl + 4 * i) * 128 + cb * 16) = make_uint4(~q.x, ~q.y, ~q.z, ~q.w);
+        }
+      }
+      if (kStageRand || kNibbleTranspose) pair_sync();  // (otherwise phase 2 reads the tile alone)
 
-    // ---------------------------------------------------------------- phase 2 ----
-    if (HAS_COL) {
-      uint4 out0, out1;  // 32 nibbles of column 2cp / 2cp + 1
-      uint32_t byte0, byte1;
-      if (kNibbleTranspose) {
-        // nibbles of the row-wise copy, 8 rows x 8 columns per thread, see transpose_nibbles()
-        byte0 = byte1 = smem[S::kBlkByte + 2 * q32 * 4 + (cp >> 4)];
-        const int o = lane & 15, rg = cp >> 4;  // columns 8 o .., rows 8 rg .. of the group
-        const uint8_t* const src = smem + S::kRand + (q32 * 32 + rg * 8) * 64 + o * 4;
-        uint32_t w[8], col[8];
+      // ---------------------------------------------------------------- phase 2 ----
+      if (HAS_COL) {
+        uint4 out0, out1;  // 32 nibbles of column 2cp / 2cp + 1
+        uint32_t byte0, byte1;
+        if (kNibbleTranspose) {
+          // nibbles of the row-wise copy, 8 rows x 8 columns per thread, see transpose_nibbles()
+          byte0 = byte1 = smem[S::kBlkByte + 2 * q32 * 4 + (cp >> 4)];
+          const int o = lane & 15, rg = cp >> 4;  // columns 8 o .., rows 8 rg .. of the group
+          const uint8_t* const src = smem + S::kRand + (q32 * 32 + rg * 8) * 64 + o * 4;
+          uint32_t w[8], col[8];
 #pragma unroll
-        for (int k = 0; k < 8; ++k) w[k] = *reinterpret_cast<const uint32_t*>(src + k * 64);
-        transpose_nibbles(w, col);
+          for (int k = 0; k < 8; ++k) w[k] = *reinterpret_cast<const uint32_t*>(src + k * 64);
+          transpose_nibbles(w, col);
 #pragma unroll
-        for (int k = 0; k < 8; ++k)
-          *reinterpret_cast<uint32_t*>(col_codes + (4 * o + (k >> 1)) * 128 +
-                                       ((((k & 1) * 4 + q32) ^ spread(4 * o + (k >> 1))) & 7) * 16 + rg * 4) = col[k];
-      } else {
-        float2 v[32];
-        const uint8_t* tp = tile_buf + q32 * 32 * 256 + cp * 4;
+          for (int k = 0; k < 8; ++k)
+            *reinterpret_cast<uint32_t*>(col_codes + (4 * o + (k >> 1)) * 128 +
+                                         ((((k & 1) * 4 + q32) ^ spread(4 * o + (k >> 1))) & 7) * 16 + rg * 4) = col[k];
+        } else {
+          float2 v[32];
+          const uint8_t* tp = tile_buf + q32 * 32 * 256 + cp * 4;
 #pragma unroll
-        for (int k = 0; k < 32; ++k) {
-          uint32_t word = *reinterpret_cast<const uint32_t*>(tp + k * 256);
-          if (RHT_COL) word ^= a.row_sign[k];
-          v[k] = make_float2(bf16_lo(word), bf16_hi(word));
-        }
-        if (RHT_COL) fwht32_pairs(v);
-        float2 am2, enc;
-        if (BLOCK2D)
-          am2.x = am2.y = fmaxf(blk[(2 * q32) * 4 + (cp >> 4)], blk[(2 * q32 + 1) * 4 + (cp >> 4)]);
-        else
-          am2 = amax_pairs(v);
-        // Section 5, transform size 32: y = fl(sum * c), c = fl(1 / sqrt(32)).  Rounding is monotone, so the block's amax is
-        // fl(max |sum| * c); the encode scale is a power of two, so fl(y * enc) = fl(sum * (c * enc)): y is never formed.  That
-        // holds while y and c * enc are normal numbers.  c * enc is, up to byte 250, for every finite sum (beside a sum that has
-        // overflowed it lacks three bits, 2.5e-7, which can move a value next to a threshold); y is subnormal for 724 sums of
-        // bf16 values alone, and none of them gets another code at any scale or draw.  (Forming y where a sum has
-        // overflowed was exact there as well and took 1.8 % longer on an activation of 8192 x 5120, 3.5 % on one of 512 x 1024.)
-        if (RHT_COL) am2 = mul2(am2, make_float2(kInvSqrt32, kInvSqrt32));
-        mx_scales(am2.x, byte0, enc.x);
-        mx_scales(am2.y, byte1, enc.y);
-        if (RHT_COL) enc = mul2(enc, make_float2(kInvSqrt32, kInvSqrt32));
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          uint2 c0, c1;
-          if (SR) {
-            // low / high byte of ntwo[k] = 255 - draw of source element (row 32 q32 + 16 h + k, column 2cp / 2cp + 1)
-            uint32_t ntwo[16];
-            const uint8_t* rp = smem + S::kRand + (q32 * 32 + 16 * h) * 128 + cp * 2;
-#pragma unroll
-            for (int k = 0; k < 16; ++k) ntwo[k] = *reinterpret_cast<const uint16_t*>(rp + k * 128);
-            convert16x2_sr(&v[16 * h], enc, ntwo, c0, c1);
-          } else {
-            convert16x2_rne(&v[16 * h], enc, c0, c1);
+          for (int k = 0; k < 32; ++k) {
+            uint32_t word = *reinterpret_cast<const uint32_t*>(tp + k * 256);
+            if (RHT_COL) word ^= a.row_sign[k];
+            v[k] = make_float2(bf16_lo(word), bf16_hi(word));
           }
-          if (h == 0) {
-            out0.x = c0.x; out0.y = c0.y; out1.x = c1.x; out1.y = c1.y;
-          } else {
-            out0.z = c0.x; out0.w = c0.y; out1.z = c1.x; out1.w = c1.y;
+          if (RHT_COL) fwht32_pairs(v);
+          float2 am2, enc;
+          if (BLOCK2D)
+            am2.x = am2.y = fmaxf(blk[(2 * q32) * 4 + (cp >> 4)], blk[(2 * q32 + 1) * 4 + (cp >> 4)]);
+          else
+            am2 = amax_pairs(v);
+          // Section 5, transform size 32: y = fl(sum * c), c = fl(1 / sqrt(32)).  Rounding is monotone, so the block's amax is
+          // fl(max |sum| * c); the encode scale is a power of two, so fl(y * enc) = fl(sum * (c * enc)): y is never formed.  That
+          // holds while y and c * enc are normal numbers.  c * enc is, up to byte 250, for every finite sum (beside a sum that has
+          // overflowed it lacks three bits, 2.5e-7, which can move a value next to a threshold); y is subnormal for 724 sums of
+          // bf16 values alone, and none of them gets another code at any scale or draw.  (Forming y where a sum has
+          // overflowed was exact there as well and took 1.8 % longer on an activation of 8192 x 5120, 3.5 % on one of 512 x 1024.)
+          if (RHT_COL) am2 = mul2(am2, make_float2(kInvSqrt32, kInvSqrt32));
+          mx_scales(am2.x, byte0, enc.x);
+          mx_scales(am2.y, byte1, enc.y);
+          if (RHT_COL) enc = mul2(enc, make_float2(kInvSqrt32, kInvSqrt32));
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            uint2 c0, c1;
+            if (SR) {
+              // low / high byte of ntwo[k] = 255 - draw of source element (row 32 q32 + 16 h + k, column 2cp / 2cp + 1)
+              uint32_t ntwo[16];
+              const uint8_t* rp = smem + S::kRand + (q32 * 32 + 16 * h) * 128 + cp * 2;
+#pragma unroll
+              for (int k = 0; k < 16; ++k) ntwo[k] = *reinterpret_cast<const uint16_t*>(rp + k * 128);
+              convert16x2_sr(&v[16 * h], enc, ntwo, c0, c1);
+            } else {
+              convert16x2_rne(&v[16 * h], enc, c0, c1);
+            }
+            if (h == 0) {
+              out0.x = c0.x; out0.y = c0.y; out1.x = c1.x; out1.y = c1.y;
+            } else {
+              out0.z = c0.x; out0.w = c0.y; out1.z = c1.x; out1.w = c1.y;
+            }
           }
         }
+        // staging: a column pair has 128 bytes, eight 16-byte units (column parity, 32-row group); unit u sits at u ^ spread(cp)
+        if (!kNibbleTranspose) {
+          *reinterpret_cast<uint4*>(col_codes + cp * 128 + (((q32 ^ spread(cp)) & 7) << 4)) = out0;
+          *reinterpret_cast<uint4*>(col_codes + cp * 128 + ((((4 + q32) ^ spread(cp)) & 7) << 4)) = out1;
+        }
+        sf_col[sf_col_pos] = (uint8_t)byte0;
+        sf_col[sf_col_pos + sf_col_odd] = (uint8_t)byte1;
       }
-      // staging: a column pair has 128 bytes, eight 16-byte units (column parity, 32-row group); unit u sits at u ^ spread(cp)
-      if (!kNibbleTranspose) {
-        *reinterpret_cast<uint4*>(col_codes + cp * 128 + (((q32 ^ spread(cp)) & 7) << 4)) = out0;
-        *reinterpret_cast<uint4*>(col_codes + cp * 128 + ((((4 + q32) ^ spread(cp)) & 7) << 4)) = out1;
-      }
-      sf_col[sf_col_pos] = (uint8_t)byte0;
-      sf_col[sf_col_pos + sf_col_odd] = (uint8_t)byte1;
-    }
+    };
+    if (!BLOCK2D && full_tile)
+      phases_1_2(std::integral_constant<bool, !BLOCK2D>{});
+    else
+      phases_1_2(std::false_type{});
     __syncthreads();
     if (*abort_flag) break;  // a wait expired (the word is read after the barrier: the same for every thread)
     if (threadIdx.x == 0 && j + 2 < n_mine) issue(j + 2);  // every warp is done with this buffer
@@ -276,7 +295,7 @@ __global__ void __launch_bounds__(256, CTAS)
       for (int k = 0; k < 2; ++k) {
         const int unit = threadIdx.x + 256 * k;
         const int c = unit >> 2, m = unit & 3;  // column, 32-row group
-        if (col0 + c >= a.cols || row0 + 32 * m >= a.rows) continue;  // rows % 32 == 0: a group is inside or outside
+        if (!full_tile && (col0 + c >= a.cols || row0 + 32 * m >= a.rows)) continue;  // rows % 32 == 0: a group is in or out
         const uint4 val = *reinterpret_cast<const uint4*>(col_codes + (c >> 1) * 128 +
                                                           (((((c & 1) * 4 + m) ^ spread(c >> 1)) & 7) << 4));
         *reinterpret_cast<uint4*>(a.c_codes + (col0 + c) * pitch + (row0 >> 1) + m * 16) = val;
@@ -296,7 +315,7 @@ __global__ void __launch_bounds__(256, CTAS)
           *reinterpret_cast<uint4*>(dst + off) = *reinterpret_cast<const uint4*>(src + threadIdx.x * 16);
         }
       } else {
-        store_linear_scales<128, 4>(src, dst, R0, K0, Rn, n_kb, row0 + 128 <= a.rows && col0 + 128 <= a.cols);
+        store_linear_scales<128, 4>(src, dst, R0, K0, Rn, n_kb, full_tile);
       }
     }
   }
