@@ -183,9 +183,9 @@ def test_the_rule_splits_where_it_says():
         assert B.nvfp4_gemm_tile(bf16, *size, False) == -1
 
 
-# one column tile of 512 and many of 256; three and several; only such tiles and eight columns; 15 to 17 k-blocks, the last of 8,
-# 32 and 40 elements; none of the row lengths a multiple of 128 bytes
-@pytest.mark.parametrize("shape", [(1040, 3664, 904), (1384, 3624, 928), (2056, 7176, 1064)])
+# one column tile of 512 and nine of 256; two and twelve; many and a ragged few; 16 and 17 k-blocks, the last of 8 and 40 elements;
+# row lengths that are odd multiples of 16 bytes
+@pytest.mark.parametrize("shape", [(1608, 2600, 968), (1056, 3960, 1032), (2056, 7176, 1064)])
 def test_bf16_products_on_512_wide_tiles(shape):
     M, N, K = shape
     gen = torch.Generator("cuda").manual_seed(M + N + K)
@@ -210,7 +210,7 @@ def test_bf16_products_on_512_wide_tiles(shape):
                 assert torch.equal(D, once + once)
 
 
-@pytest.mark.parametrize("shape", [(1592, 1392, 2040), (1544, 1680, 1912), (1592, 1552, 2128)])
+@pytest.mark.parametrize("shape", [(1040, 3664, 904), (1544, 1680, 1912), (1592, 1552, 2128)])
 def test_bf16_backward_call_on_512_wide_tiles(shape):
     """Tiles of both widths and of both products in one launch; each product has the bits that it has alone."""
     M, N, K = shape
