@@ -170,7 +170,8 @@ __device__ __forceinline__ uint32_t movmatrix_trans(uint32_t v) {
 
 // d, norm: size of the transform (2, 4, 8 or 16: H_16 is replaced by the block-diagonal matrix of 16 / d copies of
 // H_d) and its normalisation 1 / sqrt(d), applied to the maximum.
-template <bool PLAIN, bool PARTS>
+// FIRST: the source leaves L2 before anything else, see kEvictFirstBytes.
+template <bool PLAIN, bool PARTS, bool FIRST>
 __device__ __forceinline__ void amax_rot_col_tile(const uint16_t* __restrict__ x, int64_t rows, int64_t cols, int64_t ld,
                                                   uint32_t sign_mask, int tile, int tiles_c, float* __restrict__ out_plain0,
                                                   float* __restrict__ out_plain1, float* __restrict__ out_rot_col, int d,
@@ -182,13 +183,20 @@ __device__ __forceinline__ void amax_rot_col_tile(const uint16_t* __restrict__ x
   if (PARTS) griddep_wait();  // as in amax_tile
   griddep_launch_dependents();
 
+  uint64_t policy = 0;
+  if constexpr (FIRST) asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
   uint32_t lo[4][8], hi[4][8];  // rows g and g + 8 of the slab, 16 columns each, four 64-column steps
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     const int64_t c = tc * 256 + q * 64 + t * 16;
     if (r0 < rows && c < cols) {  // rows % 16 == 0, cols % 16 == 0
-      ldg256_stream(x + (r0 + g) * ld + c, lo[q]);
-      ldg256_stream(x + (r0 + 8 + g) * ld + c, hi[q]);
+      if constexpr (FIRST) {
+        ldg256_hint(x + (r0 + g) * ld + c, lo[q], policy);
+        ldg256_hint(x + (r0 + 8 + g) * ld + c, hi[q], policy);
+      } else {
+        ldg256_stream(x + (r0 + g) * ld + c, lo[q]);
+        ldg256_stream(x + (r0 + 8 + g) * ld + c, hi[q]);
+      }
     } else {
 #pragma unroll
       for (int w = 0; w < 8; ++w) lo[q][w] = hi[q][w] = 0u;
@@ -254,13 +262,19 @@ __device__ __forceinline__ void amax_rot_col_tile(const uint16_t* __restrict__ x
   }
 }
 
-template <bool PLAIN, bool PARTS>
+// A source of 64 MiB or more, read with the policy "evict first": calls on four tensors in turn, gradient of 8192 x 5120 60.1 -> 57.5
+// us, of 8192 x 20480 217 -> 209, activation 45.3 -> 42.9 and 166 -> 158.  Smaller ones gain 1 to 4 % by themselves, but a backward
+// call of 2816 x 3328 x 2304, which finds its gradient in L2 again, loses 2 %.  (Weights, whose pass 1 is amax_kernel, lose 1 to
+// 3 %; the priority as a qualifier of the load, without a policy, gained nothing and cost 5 % between 27 and 52 MB; keeping the
+// end of the source with "evict last" lost 2 to 5 % against this.)
+constexpr int64_t kEvictFirstBytes = 64ll << 20;
+template <bool PLAIN, bool PARTS, bool FIRST = false>
 __global__ void __launch_bounds__(256) amax_rot_col_kernel(const uint16_t* __restrict__ x, int64_t rows, int64_t cols,
                                                            int64_t ld, uint32_t sign_mask, int tiles_c,
                                                            float* __restrict__ out_plain0, float* __restrict__ out_plain1,
                                                            float* __restrict__ out_rot_col, int d, float norm,
                                                            float2* __restrict__ parts) {
-  amax_rot_col_tile<PLAIN, PARTS>(x, rows, cols, ld, sign_mask, (int)blockIdx.x, tiles_c, out_plain0, out_plain1,
+  amax_rot_col_tile<PLAIN, PARTS, FIRST>(x, rows, cols, ld, sign_mask, (int)blockIdx.x, tiles_c, out_plain0, out_plain1,
                                   out_rot_col, d, norm, parts);
 }
 
@@ -274,7 +288,7 @@ __global__ void __launch_bounds__(256) amax_x_and_w_kernel(const __grid_constant
     amax_tile<true, false, false, PARTS>(w.x, w.rows, w.cols, w.ld, 0u, b - n_x, w_tiles_c, w.r_global, W_COL ? w.c_global : nullptr,
                                   nullptr, nullptr, w.parts);
   else if (X_COL)
-    amax_rot_col_tile<true, PARTS>(x.x, x.rows, x.cols, x.ld, x.sign_mask, b, x_tiles_c, x.r_global, nullptr, x.c_global, 16, 0.25f,
+    amax_rot_col_tile<true, PARTS, false>(x.x, x.rows, x.cols, x.ld, x.sign_mask, b, x_tiles_c, x.r_global, nullptr, x.c_global, 16, 0.25f,
                                    x.parts);
   else
     amax_tile<true, false, false, PARTS>(x.x, x.rows, x.cols, x.ld, 0u, b, x_tiles_c, x.r_global, nullptr, nullptr, nullptr,
@@ -948,8 +962,10 @@ static cudaError_t launch_amax_rot_col(const QuantArgs& a, uint32_t mask16, floa
   const cudaError_t e =
       a.parts ? launch_amax_parts<amax_rot_col_kernel<PLAIN, true>>(tiles, s, a.x, a.rows, a.cols, a.ld, mask16, tiles_c, plain0,
                                                                     plain1, rot_col, d, norm, a.parts)
-              : launch_kernel(amax_rot_col_kernel<PLAIN, false>, dim3(tiles), dim3(256), 0, s, a.x, a.rows, a.cols, a.ld,
-                              mask16, tiles_c, plain0, plain1, rot_col, d, norm, (float2*)nullptr);
+              : launch_kernel(2 * a.rows * a.cols >= kEvictFirstBytes ? amax_rot_col_kernel<PLAIN, false, true>
+                                                                      : amax_rot_col_kernel<PLAIN, false>,
+                              dim3(tiles), dim3(256), 0, s, a.x, a.rows, a.cols, a.ld, mask16, tiles_c, plain0, plain1, rot_col,
+                              d, norm, (float2*)nullptr);
   count_launch();
   return e;
 }
