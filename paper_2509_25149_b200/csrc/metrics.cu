@@ -135,8 +135,8 @@ __global__ void __launch_bounds__(kThreads, 2) quant_error_kernel(const uint16_t
   int64_t left = first < units ? (units - first + step - 1) / step : 0;  // chunks of this thread
 #pragma unroll
   for (int u = 0; u < kDepth; ++u) load(u);
-  // Two chunks a turn without a branch between them, so that they overlap (three, each in a branch of its own: 8192 x 5120 21.2
-  // us, now 20.4; 20480 x 5120 53.5, now 50.5)
+  // Two chunks a turn without a branch between them, so that they overlap (three, each in a branch of its own: 8192 x 5120 20.5
+  // us, now 19.3; 20480 x 5120 52.5, now 49.3)
   for (; left > 1; left -= 2) {
     add(0);
     load(0);  // the slot's next chunk, while the other's is worked on
