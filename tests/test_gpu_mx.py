@@ -358,3 +358,17 @@ def test_full_size_layer_in_mxfp4_sampled():
     n12 = np.sort(rng.choice(N, 12, replace=False))
     check(dW, rows_of(gb, n12, colwise=True, rht=True, **sr), rows_of(xb, k256, colwise=True, rht=True), n12, k256, False,
           True, "Wgrad")
+
+
+@pytest.mark.parametrize("which", ["both", "col"])
+@pytest.mark.parametrize("shape", [(128, 128), (256, 384), (160, 224)])
+def test_1x32_blocks_with_draws_of_their_own(shape, which):
+    """The transposed copy rounded with the second stream: staged after the row-wise copy's own, full tiles and partial ones."""
+    x = synth.normal_bf16(shape, 1e-3, 71)
+    layout = B.SF_SWIZZLED if shape[0] % 128 == 0 else B.SF_LINEAR
+    row, col = P.gpu_quantize_mx(x, rowwise=which == "both", colwise=True, sf_layout=layout, rounding=B.ROUND_STOCHASTIC, seed=11,
+                                 sr_offset=6, flags=B.SR_INDEPENDENT_COPIES)
+    sr = dict(rounding=oracle.SR, seed=11)
+    if row is not None:
+        P.assert_exact_mx(row, oracle.quantize_mx(synth.bits(x), sr_offset=6, **sr), "row")
+    P.assert_exact_mx(col, oracle.quantize_mx(synth.bits(x), colwise=True, sr_offset=6 | (1 << 63), **sr), "col")

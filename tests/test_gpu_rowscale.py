@@ -46,6 +46,19 @@ def test_quantizer_bit_exact(shape, rounding):
     assert_rows_exact(t, oracle.quantize_rowscale(synth.bits(x), rounding=rounding, seed=3, sr_offset=9), f"{shape}")
 
 
+@pytest.mark.parametrize("cols", [10256, 12304, 20480])
+def test_long_rows_beside_the_limit_of_the_plain_division(cols):
+    """Rows on either side of s_enc = 5e27 (amax 5.4e-25: from the table of encode scales, block by block), whose blocks' amaxes are
+    1, 1e-3 ... 1e-12 of the row's; rows that end inside a pair of chunk groups."""
+    x = synth.normal_bf16((16, cols), 1.0, 23).float()
+    x = x / x.abs().amax(dim=1, keepdim=True) * 10.0 ** (-3.0 * (torch.arange(cols) // 16 % 5))
+    x[:, 0] = 1.0
+    x *= torch.tensor([5.0e-25, 5.8e-25, 1e-30, 1.0])[torch.arange(16) % 4][:, None]
+    x = x.bfloat16()
+    t = gpu_rowscale(x, sf_layout=B.SF_LINEAR)
+    assert_rows_exact(t, oracle.quantize_rowscale(synth.bits(x)), f"{cols}")
+
+
 def test_linear_scale_layout_ragged_rows_and_argument_checks():
     x = synth.normal_bf16((48, 208), 1.0, 21)  # rows not a multiple of 8 warps x n, cols not of 512
     t = gpu_rowscale(x, sf_layout=B.SF_LINEAR)
