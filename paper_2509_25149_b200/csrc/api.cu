@@ -256,8 +256,9 @@ nvfp4_status bf16_prepare(const void* A, int32_t a_layout, int64_t lda, const vo
 }
 
 nvfp4_status bf16_impl(const DenseGemmArgs& g0, const DenseGemmArgs* g1, void* cuda_stream) {
-  const int tile = bf16_tile(g0, g1, g_tile_n.load(std::memory_order_relaxed));
-  return launch_gemm_bf16(g0, g1, tile, static_cast<cudaStream_t>(cuda_stream)) == cudaSuccess ? NVFP4_OK : NVFP4_ERR_CUDA;
+  Bf16Wide wide;
+  const int tile = bf16_tile(g0, g1, g_tile_n.load(std::memory_order_relaxed), &wide);
+  return launch_gemm_bf16(g0, g1, tile, wide, static_cast<cudaStream_t>(cuda_stream)) == cudaSuccess ? NVFP4_OK : NVFP4_ERR_CUDA;
 }
 
 inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
@@ -598,7 +599,8 @@ int32_t nvfp4_gemm_tile(int32_t bf16, int64_t M, int64_t N, int64_t K, int32_t d
     DenseGemmArgs g{};
     g.M = (int)M; g.N = (int)N; g.K = (int)K;
     g.lda = g.ldb = K;
-    return bf16_tile(g, nullptr, g_tile_n.load(std::memory_order_relaxed));
+    Bf16Wide wide;
+    return bf16_tile(g, nullptr, g_tile_n.load(std::memory_order_relaxed), &wide);
   }
   GemmArgs g{};
   g.M = (int)M; g.N = (int)N; g.K = (int)K;

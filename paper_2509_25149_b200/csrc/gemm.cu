@@ -744,7 +744,7 @@ static bool make_bf16_maps(const DenseGemmArgs& g, CUtensorMap* m) {  // A, B, D
 static int bf16_tiles(const DenseGemmArgs& g, int bn) { return ((g.M + 255) / 256) * ((g.N + bn - 1) / bn); }
 
 template <int BN, int SPLIT, bool TWO>
-static cudaError_t launch_bf16_problems(const DenseGemmArgs& g0, const DenseGemmArgs* g1, const int (&wide_n)[2], int max_pairs,
+static cudaError_t launch_bf16_problems(const DenseGemmArgs& g0, const DenseGemmArgs* g1, const Bf16Wide& wide_cols, int max_pairs,
                                         cudaStream_t s) {
   auto kern = dense::gemm_bf16_pair_kernel<BN, SPLIT, TWO>;
   constexpr int smem = dense::Cfg<BN, SPLIT>::kSmemBytes;
@@ -771,7 +771,7 @@ static cudaError_t launch_bf16_problems(const DenseGemmArgs& g0, const DenseGemm
   if (BN == 512) {
     for (int i = 0; i < (g1 ? 2 : 1); ++i) {
       const DenseGemmArgs& g = i ? *g1 : g0;
-      const int tiles_m = (g.M + 255) / 256, wide = std::min(wide_n[i], (g.N + 255) / 512);
+      const int tiles_m = (g.M + 255) / 256, wide = std::min(wide_cols.n[i], (g.N + 255) / 512);
       a.wide_n[i] = wide;
       a.seg_end[i] = tiles_m * wide;
       a.seg_end[2 + i] = tiles_m * ((g.N + 255) / 256 - 2 * wide);
@@ -791,92 +791,24 @@ static cudaError_t launch_bf16_problems(const DenseGemmArgs& g0, const DenseGemm
 
 // g1 == nullptr: one problem
 template <int BN, int SPLIT = 1>
-static cudaError_t launch_bf16_t(const DenseGemmArgs& g0, const DenseGemmArgs* g1, const int (&wide_n)[2], int max_pairs,
+static cudaError_t launch_bf16_t(const DenseGemmArgs& g0, const DenseGemmArgs* g1, const Bf16Wide& wide_cols, int max_pairs,
                                  cudaStream_t s) {
-  return g1 ? launch_bf16_problems<BN, SPLIT, true>(g0, g1, wide_n, max_pairs, s)
-            : launch_bf16_problems<BN, SPLIT, false>(g0, nullptr, wide_n, max_pairs, s);
+  return g1 ? launch_bf16_problems<BN, SPLIT, true>(g0, g1, wide_cols, max_pairs, s)
+            : launch_bf16_problems<BN, SPLIT, false>(g0, nullptr, wide_cols, max_pairs, s);
 }
 
-// Column tiles 512 wide of each problem (the other columns in tiles of 256, behind them) whose schedule is estimated shortest;
-// {0, 0}: 256-wide tiles everywhere.  A k-block of a tile takes as long as its MMAs (530 SM cycles per 256 columns) or as its
-// loads: 63 bytes per clock, in pieces of 64, of which a 128-byte row of a box takes three where it does not begin on one: with rows
-// P bytes apart 1.5 - gcd(P, 64) / 128 times the bytes.  Where the MMAs are longer, what 512 columns gain is fewer hand-overs and,
-// with tiles of two sizes, shorter last rounds.  256 wide / chosen: forward of 4088 x 5128 x 5112 208 / 179 us, backward 414 / 330,
-// forward of 2048 x 7168 x 2056 68 / 55, of 3000 x 3000 x 1000 20.3 / 18.6, backward 45.2 / 39.6; rows 128 bytes apart: backward of
-// 4096 x 2048 x 1024 38.5 / 27.1, of 8192 x 5120 x 5120 696 / 671.  A hand-over of two accumulators takes 3000 cycles and a pair whose
-// last tile is such a one 3000 more, its halves leaving one after the other: with half of that forward of 1040 x 3664 x 904 came out at
-// 14.8 / 15.6, 1384 x 3624 x 928 at 14.8 / 15.4.  Contractions of fewer than 14 k-blocks keep 256 columns (1112 x 3672 x 552 11.5 /
-// 12.7, 2344 x 1856 x 264 9.2 / 10.3).
-static void bf16_wide_tiles(const DenseGemmArgs& g0, const DenseGemmArgs* g1, int pairs, int (&wide_n)[2]) {
-  const DenseGemmArgs* const gs[2] = {&g0, g1};
-  const int n = g1 ? 2 : 1;
-  int most[2] = {0, 0};
-  for (int i = 0; i < n; ++i)
-    if (gs[i]->K > 13 * 64) most[i] = std::min((gs[i]->N + 255) / 512, 0x7fff);
-  wide_n[0] = wide_n[1] = 0;
-  if (most[0] + most[1] == 0) return;
-  static TileMemo memo;
-  auto piece = [](int64_t ld) { return (int)std::min<int64_t>(ld & -ld, 32); };  // elements: gcd(P, 64) / 2
-  int pitches = 0;
-  for (int i = 0; i < n; ++i) pitches = (pitches << 12) | piece(gs[i]->lda) << 6 | piece(gs[i]->ldb);
-  const int key[TileMemo::kKey] = {g0.M, g0.N, g0.K, g1 ? g1->M : 0, g1 ? g1->N : 0, g1 ? g1->K : 0, pitches, pairs};
-  int both = 0;
-  if (memo.find(key, &both)) {
-    wide_n[0] = both & 0xffff;
-    wide_n[1] = both >> 16;
-    return;
+static Bf16Wide bf16_wide_tiles(const DenseGemmArgs& g0, const DenseGemmArgs* g1, int pairs) {
+  Bf16Walk w[2];
+  for (int i = 0; i < (g1 ? 2 : 1); ++i) {
+    const DenseGemmArgs& g = i ? *g1 : g0;
+    w[i] = bf16_walk(g.M, g.N, g.K, g.lda, g.ldb);
   }
-  std::vector<double> load((size_t)pairs), tail((size_t)pairs);
-  auto makespan = [&](int w0, int w1) {
-    std::fill(load.begin(), load.end(), 0.0);
-    std::fill(tail.begin(), tail.end(), 0.0);
-    const bool snake = w0 + w1 > 0;
-    int64_t t = 0;
-    for (int seg = 0; seg < 4; ++seg) {  // tiles 512 wide of both problems, then 256 wide
-      if ((seg & 1) >= n) continue;
-      const DenseGemmArgs& g = *gs[seg & 1];
-      const int w = seg & 1 ? w1 : w0, halves = seg < 2 ? 2 : 1;
-      auto bytes = [&](int64_t ld) { return 16384.0 * (1.5 - piece(ld) / 64.0); };
-      const double k_block = std::max(halves * 530.0, (bytes(g.lda) + halves * bytes(g.ldb)) / 63.0);
-      const double cost = k_block * ((g.K + 63) / 64) + (halves == 2 ? 3000.0 : 500.0), last_cost = halves == 2 ? 3000.0 : 0.0;
-      const int64_t end = t + (int64_t)((g.M + 255) / 256) * (seg < 2 ? w : (g.N + 255) / 256 - 2 * w);
-      const int64_t first = (t + pairs - 1) / pairs, last = end / pairs;
-      auto one = [&](int64_t i) {
-        const size_t p = (size_t)(snake && (i / pairs & 1) ? pairs - 1 - i % pairs : i % pairs);
-        load[p] += cost;
-        tail[p] = last_cost;
-      };
-      if (first < last) {  // whole rounds of the pairs at once
-        for (int64_t i = t; i < first * pairs; ++i) one(i);
-        for (double& v : load) v += cost * (double)(last - first);
-        std::fill(tail.begin(), tail.end(), last_cost);
-        for (int64_t i = last * pairs; i < end; ++i) one(i);
-      } else {
-        for (int64_t i = t; i < end; ++i) one(i);
-      }
-      t = end;
-    }
-    double worst = 0.0;
-    for (int p = 0; p < pairs; ++p) worst = std::max(worst, load[(size_t)p] + tail[(size_t)p]);
-    return worst;
-  };
-  double least = 0.98 * makespan(0, 0);
-  const int step[2] = {1 + most[0] / (g1 ? 16 : 64), 1 + most[1] / 16};  // (at most 65, or 17 x 17 of them)
-  for (int i = most[0] % step[0]; i <= most[0]; i += step[0])
-    for (int j = most[1] % step[1]; j <= most[1]; j += step[1]) {
-      if (i + j == 0) continue;
-      const double v = makespan(i, j);
-      if (v < least) {
-        least = v;
-        wide_n[0] = i;
-        wide_n[1] = j;
-      }
-    }
-  memo.put(key, wide_n[0] | wide_n[1] << 16);
+  return bf16_wide_tiles(w, g1 ? 2 : 1, pairs);
 }
 
-int bf16_tile(const DenseGemmArgs& g0, const DenseGemmArgs* g1, int forced) {
+int bf16_tile(const DenseGemmArgs& g0, const DenseGemmArgs* g1, int forced, Bf16Wide* wide) {
   int num_sms = 0;
+  *wide = Bf16Wide{{0, 0}};
   if (sm_count(&num_sms) != cudaSuccess) return kTilePair256;
   // 256 x 128 tiles while every one of them has a pair to itself: less to load per k-block and half the epilogue (1000 x
   // 2000 x 3000 22.9 -> 19.0 us, 512 x 4096 x 4096 24.2 -> 23.2, 512 x 1024 x 1024 9.1 -> 8.1).  Beyond one round they lose:
@@ -901,23 +833,19 @@ int bf16_tile(const DenseGemmArgs& g0, const DenseGemmArgs* g1, int forced) {
     if (tiles128 <= clusters(std::integral_constant<int, 2>())) return kTileSplit2;
   }
   if (tiles128 <= num_sms / 2) return kTilePair128;
-  int wide_n[2];
-  bf16_wide_tiles(g0, g1, num_sms / 2, wide_n);
-  return wide_n[0] + wide_n[1] ? kTileDouble : kTilePair256;
+  *wide = bf16_wide_tiles(g0, g1, num_sms / 2);
+  return wide->n[0] + wide->n[1] ? kTileDouble : kTilePair256;
 }
 
-cudaError_t launch_gemm_bf16(const DenseGemmArgs& g0, const DenseGemmArgs* g1, int tile, cudaStream_t s) {
+cudaError_t launch_gemm_bf16(const DenseGemmArgs& g0, const DenseGemmArgs* g1, int tile, const Bf16Wide& wide, cudaStream_t s) {
   int num_sms = 0;
   const cudaError_t e = sm_count(&num_sms);
   if (e != cudaSuccess) return e;
   const int pairs = num_sms / 2;
-  int wide_n[2] = {0, 0};
-  if (tile == kTileSplit4) return launch_bf16_t<128, 4>(g0, g1, wide_n, pairs, s);
-  if (tile == kTileSplit2) return launch_bf16_t<128, 2>(g0, g1, wide_n, pairs, s);
-  if (tile == kTilePair128) return launch_bf16_t<128>(g0, g1, wide_n, pairs, s);
-  if (tile != kTileDouble) return launch_bf16_t<256>(g0, g1, wide_n, pairs, s);
-  bf16_wide_tiles(g0, g1, pairs, wide_n);
-  return launch_bf16_t<512>(g0, g1, wide_n, pairs, s);
+  if (tile == kTileSplit4) return launch_bf16_t<128, 4>(g0, g1, wide, pairs, s);
+  if (tile == kTileSplit2) return launch_bf16_t<128, 2>(g0, g1, wide, pairs, s);
+  if (tile == kTilePair128) return launch_bf16_t<128>(g0, g1, wide, pairs, s);
+  return tile == kTileDouble ? launch_bf16_t<512>(g0, g1, wide, pairs, s) : launch_bf16_t<256>(g0, g1, wide, pairs, s);
 }
 
 // Test aid: one warp waits, with the given limit, on a barrier nobody arrives at.  The wait runs out, the code lands

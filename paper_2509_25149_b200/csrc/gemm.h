@@ -3,6 +3,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "bf16_schedule.h"
+
 namespace nvfp4 {
 
 struct GemmArgs {
@@ -70,8 +72,9 @@ struct DenseGemmArgs {
   int d_is_fp32, accumulate;
 };
 // g1 (may be NULL): a second, independent product in the same launch, its tiles after those of g0
-// The tile of such a launch: kTilePair256, kTilePair128, kTileDouble or a split one (`forced`, where every share has a k-block, or by size)
-int bf16_tile(const DenseGemmArgs& g0, const DenseGemmArgs* g1, int forced);
-cudaError_t launch_gemm_bf16(const DenseGemmArgs& g0, const DenseGemmArgs* g1, int tile, cudaStream_t s);
+// The tile of such a launch: kTilePair256, kTilePair128, kTileDouble (*wide: how many column tiles of each product are 512 wide) or a
+// split one (`forced`, where every share has a k-block, or by size)
+int bf16_tile(const DenseGemmArgs& g0, const DenseGemmArgs* g1, int forced, Bf16Wide* wide);
+cudaError_t launch_gemm_bf16(const DenseGemmArgs& g0, const DenseGemmArgs* g1, int tile, const Bf16Wide& wide, cudaStream_t s);
 
 }  // namespace nvfp4
