@@ -369,8 +369,9 @@ struct QuantSmem {
 };
 
 // OWN_DRAWS: 16x16 blocks whose transposed copy is rounded with draws of its own.
+// WHOLE: no tile is cut off (rows a multiple of 128, columns of TC).
 template <bool HAS_ROW, bool HAS_COL, bool BLOCK2D, bool RHT_ROW, bool RHT_COL, bool SR, int TC, bool F32 = false,
-          bool PARTS = false, bool OWN_DRAWS = false>
+          bool PARTS = false, bool OWN_DRAWS = false, bool WHOLE = false>
 __device__ __forceinline__ void quantize_tiles(const CUtensorMap* src_map, const QuantArgs& a, const int block,
                                                const int blocks) {  // this CTA among those of the tensor
   using S = QuantSmem<TC, F32>;
@@ -511,7 +512,7 @@ __device__ __forceinline__ void quantize_tiles(const CUtensorMap* src_map, const
     const uint8_t* const tile_buf = smem + S::kTile + buf * S::kTileBytes;
     quant_wait(bar0 + 8 * buf, (uint32_t)(j >> 1) & 1u, abort_flag, a.status);  // the tile has landed
     const int64_t row0 = (int64_t)tr * 128, col0 = (int64_t)tc * TC;
-    const bool full_tile = (row0 + 128 <= a.rows) && (col0 + TC <= a.cols);
+    const bool full_tile = WHOLE || ((row0 + 128 <= a.rows) && (col0 + TC <= a.cols));
     uint8_t* const col_codes = smem + S::kColCodes + buf * S::kColBytes;
     uint8_t* const sf_row = smem + S::kSfRow + buf * S::kSfBytes;
     uint8_t* const sf_col = smem + S::kSfCol + buf * S::kSfBytes;
@@ -705,11 +706,11 @@ __device__ __forceinline__ void quantize_tiles(const CUtensorMap* src_map, const
       }
     };
     if (tiny)
-      phases_1_2(std::false_type{}, std::true_type{});
+      phases_1_2(std::bool_constant<WHOLE>{}, std::true_type{});
     else if (full_tile)
       phases_1_2(std::true_type{}, std::false_type{});
     else
-      phases_1_2(std::false_type{}, std::false_type{});
+      phases_1_2(std::bool_constant<WHOLE>{}, std::false_type{});
     __syncthreads();
     if (*abort_flag) break;  // a wait expired (the word is read after the barrier: the same for every thread)
     if (threadIdx.x == 0 && j + 2 < n_mine) issue(j + 2);  // every warp is done with this buffer
@@ -812,7 +813,9 @@ __global__ void __launch_bounds__(256, 2) quantize_kernel(const __grid_constant_
 // launch, the first n_x CTAs on the activation: one ramp and one tail instead of two.  Carrying the weight's memory-bound
 // pass 1 on the activation's pass 2 and quantizing the weight behind it measured the same for many tiles (8192 x 20480 x 5120)
 // and lost for few: fwd + bwd of 512 x 1024 x 1024 27.6 -> 24.2 us of GPU time, 1024 x 2048 x 2048 41.7 -> 39.7, 2048 x 4096 x
-// 3072 93.8 -> 91.5.
+// 3072 93.8 -> 91.5.  The layer's sizes are multiples of 256, so no tile is cut off and the code for those that are is left out: with
+// it (five copies of a tile's code in one kernel) the forward call of 4096 x 4096 x 4096 took 73.1 us, now 72.1, 1024 x 4096 x 3840
+// 36.1, now 35.4, 2048 x 4096 x 3072 41.1, now 39.9, 3584 x 2048 x 3840 46.6, now 45.3.
 template <bool X_COL, bool W_COL, int TC, bool PARTS>
 __global__ void __launch_bounds__(256, 2) quantize_x_and_w_kernel(const __grid_constant__ CUtensorMap x_map,
                                                                   const __grid_constant__ CUtensorMap w_map,
@@ -820,9 +823,9 @@ __global__ void __launch_bounds__(256, 2) quantize_x_and_w_kernel(const __grid_c
                                                                   const __grid_constant__ QuantArgs w, int n_x) {
   const int b = (int)blockIdx.x;
   if (b < n_x)
-    quantize_tiles<true, X_COL, false, false, X_COL, false, TC, false, PARTS>(&x_map, x, b, n_x);
+    quantize_tiles<true, X_COL, false, false, X_COL, false, TC, false, PARTS, false, true>(&x_map, x, b, n_x);
   else
-    quantize_tiles<true, W_COL, true, false, false, false, TC, false, PARTS>(&w_map, w, b - n_x, (int)gridDim.x - n_x);
+    quantize_tiles<true, W_COL, true, false, false, false, TC, false, PARTS, false, true>(&w_map, w, b - n_x, (int)gridDim.x - n_x);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1097,6 +1100,7 @@ static cudaError_t launch_x_and_w_t(const QuantArgs& x, const QuantArgs& w, cuda
   int sms = 0;
   cudaError_t e = sm_count(&sms);
   if (e != cudaSuccess) return e;
+  if ((x.rows | x.cols | w.rows | w.cols) % 128 != 0) return cudaErrorInvalidValue;  // (a layer's sizes: multiples of 256)
   if (!x.parts) {
     e = launch_zero_words(x.r_global, X_COL ? x.c_global : nullptr, w.r_global, W_COL ? w.c_global : nullptr, s);
     if (e != cudaSuccess) return e;

@@ -121,3 +121,27 @@ def test_forward_call_quantizes_w_exactly_like_the_standalone_call(M, N, K, with
             assert torch.equal(a.glob, b.glob)
         assert float(W_row.glob[0]) == 3.0
         assert torch.equal(Y, Y2)
+
+
+@pytest.mark.parametrize("amax", [5.0e-25, 5.8e-25])
+@pytest.mark.parametrize("M,N,K", [(256, 512, 768), (1024, 1024, 2560), (4096, 2048, 2560)])  # parts; 64 and 128 columns a tile
+def test_forward_call_of_a_tiny_activation(M, N, K, amax):
+    """On either side of the limit below which amax_b / 6 is divided exactly, the merged kernel against the standalone one."""
+    g = torch.Generator(device="cuda").manual_seed(M + N + K)
+    X = torch.randn((M, K), generator=g, device="cuda").clamp_(-4, 4) * 10.0 ** (-3.0 * (torch.arange(M, device="cuda") // 16 % 5))[:, None]
+    X = X / X.abs().max() * amax
+    X[0, 0] = amax
+    X = X.to(torch.bfloat16)
+    W = (torch.randn((N, K), generator=g, device="cuda") * 0.02).to(torch.bfloat16)
+    opts = B.quant_opts(rht_sign_mask=synth.DEFAULT_RHT_SIGN_MASK)
+    X_col, W_row, W_col, Y = B.alloc_tensor(K, M), B.alloc_tensor(N, K), B.alloc_tensor(K, N), torch.empty((M, N), dtype=torch.bfloat16, device="cuda")
+    ws = torch.empty(B.nvfp4_linear_fwd_workspace_bytes(M, K), dtype=torch.uint8, device="cuda")
+    B.nvfp4_linear_fwd(X, W, opts, Y, X_col, W_row, W_col, False, ws)
+    X_row2, X_col2, W_row2, Y2 = B.alloc_tensor(M, K), B.alloc_tensor(K, M), B.alloc_tensor(N, K), torch.empty_like(Y)
+    B.nvfp4_quantize(X, B.quant_opts(rht_colwise=True, rht_sign_mask=synth.DEFAULT_RHT_SIGN_MASK), X_row2, X_col2)
+    B.nvfp4_quantize(W, B.quant_opts(block_rows=16), W_row2, None)
+    B.nvfp4_gemm(X_row2, W_row2, Y2)
+    B.nvfp4_device_status()
+    for a, b in ((X_col, X_col2), (W_row, W_row2)):
+        assert torch.equal(a.codes, b.codes) and torch.equal(a.scales, b.scales) and torch.equal(a.glob, b.glob)
+    assert torch.equal(Y, Y2)
