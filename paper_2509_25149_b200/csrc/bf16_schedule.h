@@ -17,11 +17,17 @@ struct Bf16Wide {
   int n[2];  // column tiles 512 wide of each product of the launch
 };
 
-// elements: gcd(P, 64) / 2 for rows P bytes apart
-inline int bf16_piece(int64_t ld) { return (int)std::min<int64_t>(ld & -ld, 32); }
+// Of 32 neighbouring rows of an operand, those that begin on 64 bytes.  With rows ld elements (P bytes) apart every remainder of 64
+// that is a multiple of g = gcd(P, 64) comes up equally often, counted from the first row's.  (Judged by P alone, slices 16 bytes
+// behind a boundary kept 256 columns: 4096 x 4096 x 4096 with rows 8256 bytes apart 188.7 us, now 152.4, 8192 x 2048 x 1024 48.0,
+// now 41.2.)
+inline int bf16_piece(uint64_t base, int64_t ld) {
+  const int g = (int)std::min<int64_t>(ld & -ld, 32);  // gcd(P, 64) / 2
+  return base % (uint64_t)(2 * g) == 0 ? g : 0;
+}
 
-inline Bf16Walk bf16_walk(int64_t M, int64_t N, int64_t K, int64_t lda, int64_t ldb) {
-  return Bf16Walk{(int)((M + 255) / 256), (int)((N + 255) / 256), (int)((K + 63) / 64), bf16_piece(lda), bf16_piece(ldb)};
+inline Bf16Walk bf16_walk(int64_t M, int64_t N, int64_t K, uint64_t a, int64_t lda, uint64_t b, int64_t ldb) {
+  return Bf16Walk{(int)((M + 255) / 256), (int)((N + 255) / 256), (int)((K + 63) / 64), bf16_piece(a, lda), bf16_piece(b, ldb)};
 }
 
 // Estimated SM cycles of a launch of one or two products on `pairs` CTA pairs.
@@ -84,8 +90,8 @@ class Bf16Estimate {
 
 // Column tiles 512 wide of each product (the other columns in tiles of 256, behind them) whose schedule is estimated shortest;
 // {0, 0}: 256-wide tiles everywhere.  A k-block of a tile takes as long as its MMAs (530 SM cycles per 256 columns) or as its
-// loads: 63 bytes per clock, in pieces of 64, of which a 128-byte row of a box takes three where it does not begin on one: with rows
-// P bytes apart 1.5 - gcd(P, 64) / 128 times the bytes.  Where the MMAs are longer, what 512 columns gain is fewer hand-overs and,
+// loads: 63 bytes per clock, in pieces of 64, of which a 128-byte row of a box takes three where it does not begin on one: 1.5 -
+// bf16_piece() / 64 times the bytes.  Where the MMAs are longer, what 512 columns gain is fewer hand-overs and,
 // with tiles of two sizes, shorter last rounds.  256 wide / chosen: forward of 4088 x 5128 x 5112 208 / 179 us, backward 414 / 330,
 // forward of 2048 x 7168 x 2056 68 / 55, of 3000 x 3000 x 1000 20.3 / 18.6, backward 45.2 / 39.6; rows 128 bytes apart: backward of
 // 4096 x 2048 x 1024 38.5 / 27.1, of 8192 x 5120 x 5120 696 / 671.  A hand-over of two accumulators takes 3000 cycles and a pair whose

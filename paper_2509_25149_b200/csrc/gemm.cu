@@ -801,7 +801,7 @@ static Bf16Wide bf16_wide_tiles(const DenseGemmArgs& g0, const DenseGemmArgs* g1
   Bf16Walk w[2];
   for (int i = 0; i < (g1 ? 2 : 1); ++i) {
     const DenseGemmArgs& g = i ? *g1 : g0;
-    w[i] = bf16_walk(g.M, g.N, g.K, g.lda, g.ldb);
+    w[i] = bf16_walk(g.M, g.N, g.K, reinterpret_cast<uintptr_t>(g.a), g.lda, reinterpret_cast<uintptr_t>(g.b), g.ldb);
   }
   return bf16_wide_tiles(w, g1 ? 2 : 1, pairs);
 }

@@ -12,18 +12,19 @@ from conftest import ROOT
 SOURCE = """
 #include "bf16_schedule.h"
 using namespace nvfp4;
-static void walks(const int* p, int n, Bf16Walk* w) {
-  for (int i = 0; i < n; ++i) w[i] = bf16_walk(p[5 * i], p[5 * i + 1], p[5 * i + 2], p[5 * i + 3], p[5 * i + 4]);
+static void walks(const int* p, int n, Bf16Walk* w, int base = 4096) {
+  for (int i = 0; i < n; ++i) w[i] = bf16_walk(p[5 * i], p[5 * i + 1], p[5 * i + 2], base, p[5 * i + 3], base, p[5 * i + 4]);
 }
+extern "C" int piece(unsigned long long base, long long ld) { return bf16_piece(base, ld); }
 extern "C" long long estimate(const int* p, int n, int pairs, int w0, int w1, int lower) {
   Bf16Walk w[2];
   walks(p, n, w);
   const Bf16Estimate e(w, n, pairs);
   return lower ? e.least(Bf16Wide{{w0, w1}}) : e.until_the_last(Bf16Wide{{w0, w1}});
 }
-extern "C" int choose(const int* p, int n, int pairs, int remember, int* wide) {
+extern "C" int choose(const int* p, int n, int pairs, int remember, int base, int* wide) {
   Bf16Walk w[2];
-  walks(p, n, w);
+  walks(p, n, w, base);
   int walked = 0;
   const Bf16Wide v = remember ? bf16_wide_tiles(w, n, pairs, &walked) : bf16_wide_search(w, n, pairs, &walked);
   wide[0] = v.n[0];
@@ -56,9 +57,9 @@ def _flat(products):
     return (ctypes.c_int * 10)(*[v for p in products for v in p])
 
 
-def choose(lib, products, pairs=74, remember=False):
+def choose(lib, products, pairs=74, remember=False, base=4096):
     wide = (ctypes.c_int * 2)()
-    walked = lib.choose(_flat(products), len(products), pairs, int(remember), wide)
+    walked = lib.choose(_flat(products), len(products), pairs, int(remember), base, wide)
     return (wide[0], wide[1]), walked
 
 
@@ -94,6 +95,16 @@ def test_the_estimate_is_a_walk_of_every_tile(lib):
         got, least = lib.estimate(*args, 0), lib.estimate(*args, 1)
         assert abs(got - want) <= tiles, (products, pairs, wide)  # (a tile's cycles are whole numbers there)
         assert least <= got + 1
+
+
+def test_rows_that_begin_on_64_bytes(lib):
+    """Operands need 16-byte alignment only: a slice whose rows are a multiple of 64 bytes apart may begin beside one."""
+    lib.piece.argtypes = [ctypes.c_ulonglong, ctypes.c_longlong]
+    for base in range(4096, 4096 + 128, 16):
+        for ld in (8, 16, 24, 32, 40, 48, 64, 96, 1024, 5120, 5128, 5136, 5152):
+            assert lib.piece(base, ld) == sum((base + 2 * ld * r) % 64 == 0 for r in range(32)), (base, ld)
+    aligned, beside = (choose(lib, [(1536, 4608, 1024, 1056, 1056)], base=b, remember=True)[0] for b in (4096, 4112))
+    assert aligned == (0, 0) and beside[0] > 0
 
 
 def test_no_schedule_is_estimated_shorter_than_the_chosen_one(lib):

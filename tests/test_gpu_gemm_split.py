@@ -227,3 +227,22 @@ def test_bf16_backward_call_on_512_wide_tiles(shape):
     T = dy.double().abs().T @ x.double().abs()
     assert torch.all((dw.double() - dy.double().T @ x.double()).abs() <= M * 2.0 ** -23 * T + 1e-30)
     assert torch.equal(dx, one) and torch.equal(dw, two)
+
+
+def test_bf16_products_of_slices_that_begin_beside_64_bytes():
+    """Rows a multiple of 64 bytes apart, the first one 16 bytes behind a boundary (tiles 512 wide on 148 SMs), in every layout."""
+    M, N, K = 1536, 4608, 1024
+    gen = torch.Generator("cuda").manual_seed(9)
+
+    def slice_(rows, cols):
+        buf = torch.randn((rows, cols + 32), generator=gen, device="cuda").to(torch.bfloat16)
+        return buf[:, 8:8 + cols]
+
+    for layouts in ((0, 0), (0, 1), (1, 0), (1, 1)):
+        a, b = (slice_(K, n) if mn else slice_(n, K) for n, mn in zip((M, N), layouts))
+        D = torch.empty((M, N), device="cuda")
+        B.nvfp4_gemm_bf16(a, b, D, *layouts)
+        B.nvfp4_device_status()
+        A64, B64 = (t.double().T if mn else t.double() for t, mn in zip((a, b), layouts))
+        # K roundings of what the magnitudes add up to at most
+        assert torch.all((D.double() - A64 @ B64.T).abs() <= K * 2.0 ** -23 * (A64.abs() @ B64.abs().T))
