@@ -183,6 +183,70 @@ def test_blocks_beside_the_limit_of_the_plain_division(amax, shape, rounding):
     P.assert_exact(col, oracle.quantize(synth.bits(x), colwise=True, **kw), "col")
 
 
+@pytest.mark.parametrize("case", ["both_tiny", "transformed_tiny", "plain_tiny"])
+@pytest.mark.parametrize("shape", [(128, 128), (144, 208)])
+@pytest.mark.parametrize("rounding,flags", [(B.ROUND_NEAREST_EVEN, 0), (B.ROUND_STOCHASTIC, 0),
+                                            (B.ROUND_STOCHASTIC, B.SR_INDEPENDENT_COPIES)])
+def test_transformed_copies_beside_the_limit_of_the_plain_division(case, shape, rounding, flags):
+    """The limit is an amax of 5.4e-25, and either copy's decides for both: a transformed copy below it beside a plain one above
+    (one large element: its transform has a quarter of it), the reverse (a chunk whose signs are the transform's: four times)."""
+    x = rand_bf16(shape, 78).float()
+    decades = torch.arange(shape[0] // 16).repeat_interleave(16)[:, None] + torch.arange(shape[1] // 16).repeat_interleave(16)
+    x = x / x.abs().max() * (2.0e-25 if case == "both_tiny" else 2.0e-26) * 10.0 ** (-3.0 * (decades % 5))
+    if case == "transformed_tiny":
+        x[5, 7] = 9.0e-25
+    if case == "plain_tiny":
+        x[16:32, 9] = 3.0e-25 * torch.tensor([1.0 - 2.0 * (MASK >> j & 1) for j in range(16)])
+    x = x.bfloat16()
+    layout = B.SF_SWIZZLED if shape[0] % 128 == 0 else B.SF_LINEAR
+    row, col = P.gpu_quantize(x, rowwise=True, colwise=True, sf_layout=layout, rounding=rounding, seed=3, sr_offset=2, flags=flags,
+                              rht_colwise=True, rht_sign_mask=MASK)
+    amaxes = float(row.glob[0]), float(col.glob[0])
+    assert [a < 5.37e-25 for a in amaxes] == [case != "transformed_tiny", case != "plain_tiny"], amaxes
+    kw = dict(rounding=oracle.RNE if rounding == B.ROUND_NEAREST_EVEN else oracle.SR, seed=3)
+    P.assert_exact(row, oracle.quantize(synth.bits(x), sr_offset=2, **kw), "row")
+    y = B.nvfp4_rht16(x.cuda(), True, MASK).cpu().numpy()
+    P.assert_rht_close(synth.bits(x), col, y, colwise=True, sign_mask=MASK, sr_offset=2 | (1 << 63 if flags else 0), what="col", **kw)
+
+
+@pytest.mark.parametrize("kind", ["activation", "weight", "rows", "mxfp4"])
+def test_a_nan_changes_no_other_element(kind):
+    """What an element that is no number becomes is unspecified, but the maxima pass over it, in either half of a word and with
+    either sign: scales and other codes are those of the tensor with zeros there."""
+    x = rand_bf16((128, 256), 79)
+    where = torch.zeros(x.shape, dtype=torch.bool)
+    for r, c in ((0, 0), (3, 17), (3, 18), (40, 255), (127, 128)):
+        where[r, c] = True
+    where[64, 32:64] = True  # whole blocks
+    nan = torch.where(torch.arange(256) % 3 == 0, -torch.tensor(float("nan")), torch.tensor(float("nan")))
+    fmt = {"rows": B.FORMAT_NVFP4_ROWSCALE, "mxfp4": B.FORMAT_MXFP4}.get(kind, B.FORMAT_NVFP4)
+    got = []
+    for src in (torch.where(where, nan, x.float()).bfloat16(), torch.where(where, 0.0, x.float()).bfloat16()):
+        row, col = B.alloc_tensor(128, 256, format=fmt), None if kind == "rows" else B.alloc_tensor(256, 128, format=fmt)
+        B.nvfp4_quantize(src.cuda(), B.quant_opts(block_rows=16 if kind == "weight" else 1), row, col)
+        got.append((row, col))
+    for (a, b), elsewhere in zip(zip(*got), (~where, ~where.T)):
+        if a is None:
+            continue
+        assert torch.equal(a.glob, b.glob) and torch.equal(a.scales, b.scales)
+        nibbles = [P.unpack(t.codes.cpu().numpy()) for t in (a, b)]
+        assert np.array_equal(nibbles[0][elsewhere.numpy()], nibbles[1][elsewhere.numpy()])
+
+
+def test_an_infinite_row_leaves_the_others_their_scales():
+    x = rand_bf16((32, 10304), 80)
+    row = []
+    for v in (float("inf"), 0.0):
+        x[9, 4000] = v
+        row.append(B.alloc_tensor(32, 10304, B.SF_LINEAR, format=B.FORMAT_NVFP4_ROWSCALE))
+        B.nvfp4_quantize(x.cuda(), B.quant_opts(), row[-1], None)
+    keep = torch.arange(32) != 9
+    for name, width in (("codes", 5152), ("scales", 644), ("glob", 2)):
+        a, b = (getattr(t, name).reshape(32, width)[keep.cuda()] for t in row)
+        assert torch.equal(a, b), name
+    assert float(row[0].glob.reshape(32, 2)[9, 0]) == float("inf")
+
+
 def test_gpu_sr_is_unbiased_over_seeds():
     x = rand_bf16((128, 128), 8, std=1e-3)
     xd = x.cuda()
