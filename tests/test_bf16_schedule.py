@@ -118,6 +118,14 @@ def test_no_schedule_is_estimated_shorter_than_the_chosen_one(lib):
         assert lib.estimate(*args, *wide, 0) == (all_ if all_ < int(0.98 * narrow) else narrow)
 
 
+def test_launches_of_both_widths(lib):
+    """What 74 pairs get for the shapes that the GPU tests name for their tiles of both widths: column tiles 512 wide of each product."""
+    for shape, want in {(1608, 2600, 968): 1, (1056, 3960, 1032): 2, (2056, 7176, 1064): 13}.items():
+        assert choose(lib, forward(*shape))[0] == (want, 0), shape
+    for shape, want in {(1040, 3664, 904): (0, 1), (1544, 1680, 1912): (2, 4), (1592, 1552, 2128): (4, 4)}.items():
+        assert choose(lib, backward(*shape))[0] == want, shape
+
+
 def test_what_a_new_shape_costs(lib):
     """A call searches where its shape is new: schedules that cannot be the shortest are not walked through, and token counts that
     differ within a tile are one shape."""

@@ -183,7 +183,7 @@ def test_the_rule_splits_where_it_says():
         assert B.nvfp4_gemm_tile(bf16, *size, False) == -1
 
 
-# one column tile of 512 and nine of 256; two and twelve; many and a ragged few; 16 and 17 k-blocks, the last of 8 and 40 elements;
+# one column tile of 512 and nine of 256; two and twelve; thirteen and three; 16 and 17 k-blocks, the last of 8 and 40 elements;
 # row lengths that are odd multiples of 16 bytes
 @pytest.mark.parametrize("shape", [(1608, 2600, 968), (1056, 3960, 1032), (2056, 7176, 1064)])
 def test_bf16_products_on_512_wide_tiles(shape):
