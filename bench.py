@@ -28,10 +28,9 @@ if ROOT not in sys.path:
 METRIC = "NVFP4 GEMM TFLOP/s vs FP4 peak; quantize+RHT+SR GB/s vs HBM peak"
 M, N, K = 8192, 20480, 5120
 WORKLOAD = "cfg3_ffn_up_fwd_bwd_M8192_K5120_N20480"
-# DRAM bytes (read + write).  GEMMs: one-pass ncu capture of this workload at full size, cold caches
-# (profiles/dram_traffic_cfg3_step.md): the step's two GEMM launches divided by its three GEMMs.  Quantizer: ncu
-# captures of the three pass-2 kernels on the reduced --case shapes (profiles/quantize_kernel_dy_x_w.md), 2.80 / 2.73 /
-# 2.72 B per element for W / X / dY, scaled to the step's tensors by their element counts (traffic grows in
+# DRAM bytes (read + write).  GEMMs: one-pass ncu capture of this workload at full size, cold caches: the step's two GEMM
+# launches divided by its three GEMMs.  Quantizer: ncu captures of the three pass-2 kernels on the reduced --case shapes, 2.80 /
+# 2.73 / 2.72 B per element for W / X / dY, scaled to the step's tensors by their element counts (traffic grows in
 # proportion), plus the amax passes at the 2 B per element the earlier full-size capture measured for them.
 GEMM_DRAM_BYTES_PER_LAUNCH = (547.2e6 + 1092.6e6) / 3  # Fprop launch + merged Dgrad/Wgrad launch, per GEMM
 QUANT_DRAM_BYTES_PER_STEP = (N * K) * (2.80 + 2.0) + (M * K) * (2.73 + 2.0) + (M * N) * (2.72 + 2.0)
@@ -490,7 +489,7 @@ def run_cuda(args):
                          "achieved": gemm_tflops, "peak": fp4_peak, "unit": "TFLOP/s",
                          "frac": gemm_tflops / fp4_peak, "traffic": None if mx else GEMM_DRAM_BYTES_PER_LAUNCH,
                          "traffic_source": "ncu dram__bytes_read.sum + dram__bytes_write.sum, full-size one-pass "
-                                           "capture, mean of the three GEMMs (profiles/dram_traffic_cfg3_step.md)",
+                                           "capture, mean of the three GEMMs",
                          "peak_source": f"4 x {peaks['source']} burst bf16 cuBLAS ({peaks['bf16_tflops']} TFLOP/s)",
                          "frac_of_sustained": gemm_tflops / (4.0 * peaks["bf16_tflops_sustained"]),
                          "frac_of_datasheet_9pf": gemm_tflops / 9000.0,

@@ -71,7 +71,8 @@ struct DenseGemmArgs {
   int a_mn, b_mn;
   int d_is_fp32, accumulate;
 };
-// g1 (may be NULL): a second, independent product in the same launch, its tiles after those of g0
+// g1 (may be NULL): a second, independent product in the same launch, its tiles after those of g0 (kTileDouble: 512-wide ones of
+// both, then 256-wide ones of both)
 // The tile of such a launch: kTilePair256, kTilePair128, kTileDouble (*wide: how many column tiles of each product are 512 wide) or a
 // split one (`forced`, where every share has a k-block, or by size)
 int bf16_tile(const DenseGemmArgs& g0, const DenseGemmArgs* g1, int forced, Bf16Wide* wide);

@@ -42,11 +42,11 @@ struct Problem {
   int a_mn, b_mn;  // 1 = the operand is stored with the output index contiguous
   int d_is_fp32, accumulate;
 };
-// One launch works through the tiles of up to two independent products (problem 0 first): Dgrad and Wgrad of a layer fill
-// each other's partial last round (4088 x 5128 x 5112: 5 + 6 rounds of tiles on 74 pairs become 10).
+// One launch works through the tiles of up to two independent products: Dgrad and Wgrad of a layer fill each other's partial last
+// round (4088 x 5128 x 5112: 5 + 6 rounds of 256-wide tiles on 74 pairs become 10).
 struct Args {
   Problem p[2];
-  int n_tiles0;  // tiles of problem 0
+  int n_tiles0;  // tiles of problem 0, which come first (BN < 512)
   int n_tiles;   // tiles of both problems
   // BN = 512: tiles 512 columns wide of problem 0 and 1, then the tiles 256 wide of both, and where each of these four ends
   int wide_n[2];  // column tiles 512 wide of each problem
