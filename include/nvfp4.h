@@ -343,7 +343,7 @@ NVFP4_API nvfp4_status nvfp4_test_cluster_leave(uint64_t delay_ns, uint64_t* tim
 NVFP4_API int32_t nvfp4_set_gemm_tile_n(int32_t tile_n);
 
 /* The tile (a value of nvfp4_set_gemm_tile_n) of one M x N x K product with a launch to itself on the current device: nvfp4_gemm
- * (NVFP4, D written), or nvfp4_gemm_bf16 of packed K-major operands that begin on 64 bytes when bf16 != 0 (which has 1024
+ * (NVFP4, D written), or nvfp4_gemm_bf16 of packed K-major operands that begin on 32 bytes when bf16 != 0 (which has 1024
  * besides: 256 x 512 tiles, and 256 x 256 ones for other columns; chosen by the sizes and by where the operands' rows begin).
  * -1 for a size that the call would refuse.  Launches nothing. */
 NVFP4_API int32_t nvfp4_gemm_tile(int32_t bf16, int64_t M, int64_t N, int64_t K, int32_t d_is_fp32);

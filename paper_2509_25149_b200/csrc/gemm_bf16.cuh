@@ -72,8 +72,8 @@ __device__ __forceinline__ void tc2_mma_bf16(uint32_t d_tmem, uint64_t adesc, ui
 
 // BN: columns of a tile (512, 256 or 128).  BN = 512: two accumulators side by side share the loads of A, 48 KB per k-block and
 // CTA instead of 64; what is left of the columns, and what balances the rounds better, is taken in tiles of 256 (bf16_wide_tiles).
-// That is for operands whose rows do not all begin on 64 bytes: a 128-byte row of a box then takes three 64-byte pieces of the
-// SM's path to L2 (with rows an odd multiple of 16 bytes apart 2.75 on average), and 256-wide tiles wait for it.
+// That is for operands whose rows do not all begin on 32 bytes: a 128-byte row of a box that does not takes 1.75 times as long on the
+// SM's path to L2 (with rows an odd multiple of 16 bytes apart 1.375 on average), and 256-wide tiles wait for it.
 // The two halves of such a tile begin and end apart (kLead): the epilogue drains one while the tensor pipe works on the other.
 // SPLIT > 1 (BN = 128): a cluster of SPLIT pairs takes one tile, the only one of its life,
 // each pair a share of the k-blocks (the exchange: pair::exchange_columns).

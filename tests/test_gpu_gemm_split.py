@@ -210,7 +210,7 @@ def test_bf16_products_on_512_wide_tiles(shape):
                 assert torch.equal(D, once + once)
 
 
-@pytest.mark.parametrize("shape", [(1040, 3664, 904), (1544, 1680, 1912), (1592, 1552, 2128)])
+@pytest.mark.parametrize("shape", [(1040, 3664, 904), (1544, 1680, 1912), (1592, 1552, 2128), (1112, 1144, 2344), (1224, 1192, 2328)])
 def test_bf16_backward_call_on_512_wide_tiles(shape):
     """Tiles of both widths and of both products in one launch; each product has the bits that it has alone."""
     M, N, K = shape
@@ -230,7 +230,7 @@ def test_bf16_backward_call_on_512_wide_tiles(shape):
 
 
 def test_bf16_products_of_slices_that_begin_beside_64_bytes():
-    """Rows a multiple of 64 bytes apart, the first one 16 bytes behind a boundary (tiles 512 wide on 148 SMs), in every layout."""
+    """Rows a multiple of 64 bytes apart, the first one 16 bytes behind such a boundary (tiles 512 wide on 148 SMs), in every layout."""
     M, N, K = 1536, 4608, 1024
     gen = torch.Generator("cuda").manual_seed(9)
 
