@@ -815,7 +815,8 @@ __global__ void __launch_bounds__(256, 2) quantize_kernel(const __grid_constant_
 // and lost for few: fwd + bwd of 512 x 1024 x 1024 27.6 -> 24.2 us of GPU time, 1024 x 2048 x 2048 41.7 -> 39.7, 2048 x 4096 x
 // 3072 93.8 -> 91.5.  The layer's sizes are multiples of 256, so no tile is cut off and the code for those that are is left out: with
 // it (five copies of a tile's code in one kernel) the forward call of 4096 x 4096 x 4096 took 73.1 us, now 72.1, 1024 x 4096 x 3840
-// 36.1, now 35.4, 2048 x 4096 x 3072 41.1, now 39.9, 3584 x 2048 x 3840 46.6, now 45.3.
+// 36.1, now 35.4, 2048 x 4096 x 3072 41.1, now 39.9, 3584 x 2048 x 3840 46.6, now 45.3.  Not for an activation without its transposed
+// copy, whose code is short and came out slower so: 768 x 3840 x 1536 17.9 / 18.6 us, 512 x 5120 x 1024 16.2 / 16.8.
 template <bool X_COL, bool W_COL, int TC, bool PARTS>
 __global__ void __launch_bounds__(256, 2) quantize_x_and_w_kernel(const __grid_constant__ CUtensorMap x_map,
                                                                   const __grid_constant__ CUtensorMap w_map,
@@ -823,7 +824,7 @@ __global__ void __launch_bounds__(256, 2) quantize_x_and_w_kernel(const __grid_c
                                                                   const __grid_constant__ QuantArgs w, int n_x) {
   const int b = (int)blockIdx.x;
   if (b < n_x)
-    quantize_tiles<true, X_COL, false, false, X_COL, false, TC, false, PARTS, false, true>(&x_map, x, b, n_x);
+    quantize_tiles<true, X_COL, false, false, X_COL, false, TC, false, PARTS, false, X_COL>(&x_map, x, b, n_x);
   else
     quantize_tiles<true, W_COL, true, false, false, false, TC, false, PARTS, false, true>(&w_map, w, b - n_x, (int)gridDim.x - n_x);
 }
@@ -1044,10 +1045,12 @@ static cudaError_t launch_quant_t(const QuantArgs& a, cudaStream_t s) {
   int sms = 0;
   const cudaError_t e = sm_count(&sms);
   if (e != cudaSuccess) return e;
-  // Tiles 64 columns wide when they go round the resident CTAs in less time: a tile of half the width takes 0.535 of the time
-  // (16x16 blocks: 0.58), and the CTAs take whole rounds.  Measured (128 / 64 wide): gradient of 512 x 1024 8.6 / 7.0 us, 2048 x
-  // 1024 10.6 / 8.3, 2816 x 2304 16.4 / 14.7, 4096 x 4096 31.7 / 30.4, 8192 x 5120 63.3 / 67.2; weight of 2048 x 1024 7.0 / 6.0,
-  // 4096 x 2304 11.1 / 12.1.
+  // Tiles 64 columns wide when they go round the resident CTAs in less time: a tile of half the width counts as 0.535 of a whole
+  // one (16x16 blocks: 0.58), and the CTAs take whole rounds.  Measured (128 / 64 wide, three tensors in turn): gradient of 2816 x
+  // 2304 15.3 / 13.6 us, 1024 x 9728 21.8 / 19.8, 4096 x 4096 29.8 / 28.5, 8192 x 5120 57.6 / 60.4; activation of 4096 x 4096 23.2 /
+  // 22.8, 8192 x 5120 42.9 / 46.9; weight of 4096 x 2304 10.6 / 11.7, 8192 x 5120 37.9 / 43.8.  (The factors were fitted when a
+  // tile took 5 to 8 % longer; of 90 drawn tensors they give one the slower width by more than 1 %: activation of 2304 x 11008
+  // 30.5 / 31.6.)
   const int slots = 2 * sms;  // resident CTAs
   if constexpr (!B2 && !RR && RC == HC)  // an activation or a gradient of a layer
     if (a.parts) return launch_quant_tc<HR, HC, B2, RR, RC, SR, 64, false, true>(a, slots, s);
@@ -1074,7 +1077,8 @@ static cudaError_t launch_x_and_w_tc(QuantArgs x, QuantArgs w, int slots, cudaSt
     if (e != cudaSuccess) return e;
     device_configured(configured, dev);
   }
-  // CTAs in proportion to the work (a weight's tile takes three quarters of an activation's), at whole rounds of either
+  // CTAs in proportion to the work (a weight's tile counts as three quarters of an activation's), at whole rounds of either.  Anything
+  // from 0.65 to 0.8 measures the same within 1 %; 0.85 costs 8192 x 6144 x 1536 70.4 -> 71.4 us, 4352 x 2048 x 2560 38.6 -> 39.6.
   const int tx = x.tiles_r * x.tiles_c, tw = w.tiles_r * w.tiles_c;
   int n_x = tx, n_w = tw;
   if (tx + tw > slots) {
@@ -1119,8 +1123,8 @@ static cudaError_t launch_x_and_w_t(const QuantArgs& x, const QuantArgs& w, cuda
   if (x.parts) return launch_x_and_w_tc<X_COL, W_COL, 64, true>(xa, wa, slots, s);
   const int64_t t128 = (int64_t)x.tiles_r * x.tiles_c + (int64_t)w.tiles_r * w.tiles_c;
   const int64_t t64 = (int64_t)x.tiles_r * ((x.cols + 63) / 64) + (int64_t)w.tiles_r * ((w.cols + 63) / 64);
-  // (0.6: the forward call of 1024 x 4096 x 4096 took 34.3 us in nine rounds of narrow
-  // tiles, 32.2 in five of wide ones)
+  // (0.6: the forward call of 1024 x 4096 x 4096 takes 38.4 us in nine rounds of narrow tiles, 35.6 in five of wide ones.  Of 34
+  // shapes two would gain more than 1 % by the other width: 6144 x 512 x 2560 35.1 / 34.5, 2048 x 4608 x 512 19.8 / 19.5.)
   return 0.6 * (double)((t64 + slots - 1) / slots) < (double)((t128 + slots - 1) / slots)
              ? launch_x_and_w_tc<X_COL, W_COL, 64>(xa, wa, slots, s)
              : launch_x_and_w_tc<X_COL, W_COL, 128>(xa, wa, slots, s);
