@@ -173,7 +173,7 @@ nvfp4_status quantize_impl(const void* x, int64_t rows, int64_t cols, int64_t ld
       a.parts = parts;
       a.n_parts = (int)amax_parts(rows, cols);
     }
-    if (launch_amax(a, hr, hc, o->rht_rowwise != 0, o->rht_colwise != 0, s) != cudaSuccess) return NVFP4_ERR_CUDA;
+    if (launch_amax(a, hr, hc, o->rht_rowwise != 0, o->rht_colwise != 0, sr, s) != cudaSuccess) return NVFP4_ERR_CUDA;
     a.chained = 1;
   }
   if (launch_quantize(a, hr, hc, b2, o->rht_rowwise != 0, o->rht_colwise != 0, sr, s) != cudaSuccess)

@@ -267,7 +267,13 @@ __device__ __forceinline__ void amax_rot_col_tile(const uint16_t* __restrict__ x
 // call of 2816 x 3328 x 2304, which finds its gradient in L2 again, loses 2 %.  (Weights, whose pass 1 is amax_kernel, lose 1 to
 // 3 %; the priority as a qualifier of the load, without a policy, gained nothing and cost 5 % between 27 and 52 MB; keeping the
 // end of the source with "evict last" lost 2 to 5 % against this.)
+// Nor an activation whose scale bytes leave one by one in both copies (sizes that are no multiples of 64, see store_linear_scales):
+// with the policy / without 9360 x 7920 96.4 / 93.1 us, 8736 x 12720 146.7 / 139.4, 4880 x 11216 72.5 / 68.8; one side a multiple, 9344 x
+// 7920 80.0 / 84.0, 9360 x 7936 80.1 / 83.8; gradients gain either way (9360 x 7920 107.8 / 112.0).
 constexpr int64_t kEvictFirstBytes = 64ll << 20;
+static bool evict_first(const QuantArgs& a, bool sr) {
+  return 2 * a.rows * a.cols >= kEvictFirstBytes && (sr || a.rows % 64 == 0 || a.cols % 64 == 0);
+}
 template <bool PLAIN, bool PARTS, bool FIRST = false>
 __global__ void __launch_bounds__(256) amax_rot_col_kernel(const uint16_t* __restrict__ x, int64_t rows, int64_t cols,
                                                            int64_t ld, uint32_t sign_mask, int tiles_c,
@@ -960,21 +966,20 @@ cudaError_t launch_zero_words(float* w0, float* w1, float* w2, float* w3, cudaSt
 
 template <bool PLAIN>
 static cudaError_t launch_amax_rot_col(const QuantArgs& a, uint32_t mask16, float* plain0, float* plain1, float* rot_col,
-                                       int d, float norm, cudaStream_t s) {
+                                       int d, float norm, bool sr, cudaStream_t s) {
   const int tiles_c = (int)((a.cols + 255) / 256);
   const unsigned tiles = (unsigned)(((a.rows + 127) / 128) * tiles_c);
   const cudaError_t e =
       a.parts ? launch_amax_parts<amax_rot_col_kernel<PLAIN, true>>(tiles, s, a.x, a.rows, a.cols, a.ld, mask16, tiles_c, plain0,
                                                                     plain1, rot_col, d, norm, a.parts)
-              : launch_kernel(2 * a.rows * a.cols >= kEvictFirstBytes ? amax_rot_col_kernel<PLAIN, false, true>
-                                                                      : amax_rot_col_kernel<PLAIN, false>,
+              : launch_kernel(evict_first(a, sr) ? amax_rot_col_kernel<PLAIN, false, true> : amax_rot_col_kernel<PLAIN, false>,
                               dim3(tiles), dim3(256), 0, s, a.x, a.rows, a.cols, a.ld, mask16, tiles_c, plain0, plain1, rot_col,
                               d, norm, (float2*)nullptr);
   count_launch();
   return e;
 }
 
-cudaError_t launch_amax(const QuantArgs& a, bool has_row, bool has_col, bool rht_row, bool rht_col,
+cudaError_t launch_amax(const QuantArgs& a, bool has_row, bool has_col, bool rht_row, bool rht_col, bool sr,
                         cudaStream_t s) {
   if (!a.parts) {
     const cudaError_t e = launch_zero_words(has_row ? a.r_global : nullptr, has_col ? a.c_global : nullptr, nullptr, nullptr, s);
@@ -987,8 +992,8 @@ cudaError_t launch_amax(const QuantArgs& a, bool has_row, bool has_col, bool rht
   float* rot_row = rr ? a.r_global : nullptr;
   float* rot_col = rc ? a.c_global : nullptr;
   if (rc && !rr)  // tensor-core transform for the transposed copy
-    return plain ? launch_amax_rot_col<true>(a, a.sign_mask, plain0, plain1, rot_col, 16, 0.25f, s)
-                 : launch_amax_rot_col<false>(a, a.sign_mask, plain0, plain1, rot_col, 16, 0.25f, s);
+    return plain ? launch_amax_rot_col<true>(a, a.sign_mask, plain0, plain1, rot_col, 16, 0.25f, sr, s)
+                 : launch_amax_rot_col<false>(a, a.sign_mask, plain0, plain1, rot_col, 16, 0.25f, sr, s);
 #define NVFP4_AMAX(P, R, C) \
   if (plain == P && rr == R && rc == C) return launch_amax_t<P, R, C>(a, plain0, plain1, rot_row, rot_col, s);
   NVFP4_AMAX(true, false, false)
@@ -1007,8 +1012,8 @@ cudaError_t launch_amax_rot_col_small(const QuantArgs& a, bool has_row, uint32_t
                                       cudaStream_t s) {
   const cudaError_t e = launch_zero_words(has_row ? a.r_global : nullptr, a.c_global, nullptr, nullptr, s);
   if (e != cudaSuccess) return e;
-  return has_row ? launch_amax_rot_col<true>(a, mask16, a.r_global, nullptr, a.c_global, d, norm, s)
-                 : launch_amax_rot_col<false>(a, mask16, nullptr, nullptr, a.c_global, d, norm, s);
+  return has_row ? launch_amax_rot_col<true>(a, mask16, a.r_global, nullptr, a.c_global, d, norm, false, s)
+                 : launch_amax_rot_col<false>(a, mask16, nullptr, nullptr, a.c_global, d, norm, false, s);
 }
 
 // the source as a 2-D tensor map: boxes of 128 rows x tc elements (no swizzle), zero fill outside

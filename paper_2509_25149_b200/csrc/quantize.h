@@ -49,7 +49,7 @@ int64_t amax_parts(int64_t rows, int64_t cols);
 bool pass1_in_parts(int64_t parts);
 // Clears the words the reductions of a call add into (any of them may be NULL) in one launch, the first of the call.
 cudaError_t launch_zero_words(float* w0, float* w1, float* w2, float* w3, cudaStream_t s);
-cudaError_t launch_amax(const QuantArgs& a, bool has_row, bool has_col, bool rht_row, bool rht_col,
+cudaError_t launch_amax(const QuantArgs& a, bool has_row, bool has_col, bool rht_row, bool rht_col, bool sr,
                         cudaStream_t s);
 cudaError_t launch_quantize(const QuantArgs& a, bool has_row, bool has_col, bool block2d, bool rht_row,
                             bool rht_col, bool sr, cudaStream_t s);

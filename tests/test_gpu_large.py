@@ -102,3 +102,20 @@ def test_bf16_gemm_with_more_than_2_pow_31_outputs_and_row_scaled_copy_past_the_
         assert np.array_equal(t.glob.view(R, 2)[r0:r0 + 128].cpu().numpy().view(np.uint32), ref.glob.view(np.uint32))
         sc = t.scales.view(-1)[(r0 // 128) * (C // 64) * 512:((r0 // 128) + 1) * (C // 64) * 512].cpu().numpy()
         assert np.array_equal(oracle.sf_unswizzle(sc, 128, C // 16), ref.scales), f"scales of rows {r0}.."
+
+
+@pytest.mark.parametrize("rounding", [B.ROUND_NEAREST_EVEN, B.ROUND_STOCHASTIC])
+@pytest.mark.parametrize("rows,cols", [(4112, 8176), (4112, 8192), (4160, 8080)])
+def test_tensor_amax_of_large_ragged_sources(rows, cols, rounding):
+    """Sources of 64 MiB and more, which pass 1 reads with an L2 policy or without, by the rounding and by whether either size is a
+    multiple of 64: the words it leaves, with the maximum in the last partial tile."""
+    x = synth.normal_bf16_device((rows, cols), 1.0, rows + cols)
+    x[rows - 1, cols - 1] = -9.0
+    row, col = B.alloc_tensor(rows, cols, B.SF_LINEAR), B.alloc_tensor(cols, rows, B.SF_LINEAR)
+    mask = synth.DEFAULT_RHT_SIGN_MASK
+    B.nvfp4_quantize(x, B.quant_opts(rounding=rounding, rht_colwise=True, rht_sign_mask=mask, seed=3), row, col)
+    B.nvfp4_device_status()
+    assert float(row.glob[0]) == 9.0
+    y = B.nvfp4_rht16(x, True, mask)
+    # sixteen terms summed in another order
+    assert abs(float(col.glob[0]) - float(y.abs().max())) <= 16 * 2.0 ** -23 * float(col.glob[0]) * 4
