@@ -12,6 +12,9 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
+#include <utility>
+
+#include "async_ptx.cuh"
 #include "common.cuh"
 #include "quantize.h"
 #include "quantize_common.cuh"
@@ -59,8 +62,9 @@ __device__ __forceinline__ void encode_chunk(const QuantArgs& a, const uint32_t 
   a.r_scales[a.r_swz ? sf_swizzled_offset(row, cb, n_cb) : (row * n_cb + cb)] = (uint8_t)byte;
 }
 
-// CTAs resident per SM by what a lane keeps (registers)
-constexpr int ctas_per_sm(int keep) { return keep <= 2 ? 8 : keep <= 5 ? 6 : 4; }
+// CTAs resident per SM by what a lane keeps (registers).  Five chunks: 64 registers, two of which spill, and eight CTAs read 16384 x
+// 5120 in 38.9 us, six with 74 registers in 40.8 (ordinary launches).
+constexpr int ctas_per_sm(int keep) { return keep <= 5 ? 8 : 4; }
 
 // WPR warps per row (1, 2 or 4): row (4 / WPR) * i + w / WPR of iteration i belongs to warp w, whose lanes take every WPR-th
 // group of 32 chunks, so that a row of any length is spread evenly.
@@ -77,6 +81,8 @@ __global__ void __launch_bounds__(128, ctas_per_sm(kKeep)) quantize_rowscale_ker
   constexpr int kRowsPerCta = 4 / WPR;
   const int seg = warp % WPR, sub = warp / WPR;
   const int64_t n_cb = a.cols >> 4;
+  griddep_wait();
+  griddep_launch_dependents();
   int it = 0;
   // every warp of a CTA runs the same number of iterations (rows are padded), so the barriers below are uniform
   for (int64_t base = (int64_t)blockIdx.x * kRowsPerCta; base < a.rows; base += (int64_t)gridDim.x * kRowsPerCta, ++it) {
@@ -142,6 +148,8 @@ template <bool SR>
 __global__ void __launch_bounds__(256) quantize_rowscale_long_kernel(const QuantArgs a) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t n_cb = a.cols >> 4;
+  griddep_wait();
+  griddep_launch_dependents();
   for (int64_t row = (int64_t)blockIdx.x * 8 + warp; row < a.rows; row += (int64_t)gridDim.x * 8) {
     const uint16_t* src = a.x + row * a.ld;
     uint32_t acc = 0;
@@ -185,11 +193,29 @@ __global__ void __launch_bounds__(256) quantize_rowscale_long_kernel(const Quant
   }
 }
 
+// Programmatic launch: behind an ordinary one the next kernel begins on a grid of 2.05 us (a row-wise copy of 8192 x 1536 took 10.24 us
+// by the side of 7.47, 1024 x 7168 6.15 / 5.14, 16384 x 2560 20.5 / 19.0).  Without an ordinary launch's pause, though, the SMs stay
+// divided the way the kernel before wanted them, nearly all shared memory behind a product, and the loads in flight do not fit what
+// is left as L1: forward of 16384 x 1024 x 5120 88 us with an ordinary launch, 96 with a programmatic one, 85.4 where the kernel
+// asks for 7 % of the SM as shared memory (16 KB, eight CTAs of 1.1 KB); 16384 x 5120 x 5120 243 / 250 / 237, 1024 x 2048 x 2048
+// 12.3 / 10.9 / 9.9.  (15 % and more do not make an SM change, and with none at all rows of 20480, whose CTAs have 3 KB, lose 40 %.)
+constexpr int kCarveoutPercent = 7;
+template <auto KERN, typename... Args>
+cudaError_t launch_streaming(unsigned grid, unsigned block, cudaStream_t s, Args&&... args) {
+  static std::atomic<uint64_t> configured{0};  // per kernel and device
+  int dev;
+  if (device_needs_config(configured, &dev)) {
+    const cudaError_t e = cudaFuncSetAttribute(KERN, cudaFuncAttributePreferredSharedMemoryCarveout, kCarveoutPercent);
+    if (e != cudaSuccess) return e;
+    device_configured(configured, dev);
+  }
+  return launch_kernel(KERN, dim3(grid), dim3(block), 0, s, std::forward<Args>(args)...);
+}
+
 template <bool SR, int WPR, int KEEP>
 cudaError_t launch_kept(const QuantArgs& a, int sms, cudaStream_t s) {
   const int64_t want = (a.rows * WPR + 3) / 4, cap = (int64_t)sms * ctas_per_sm(KEEP) * 4;  // up to four rounds of CTAs
-  quantize_rowscale_kernel<SR, WPR, KEEP><<<(unsigned)(want < cap ? want : cap), 128, 0, s>>>(a);
-  return cudaGetLastError();
+  return launch_streaming<quantize_rowscale_kernel<SR, WPR, KEEP>>((unsigned)(want < cap ? want : cap), 128, s, a);
 }
 
 template <bool SR>
@@ -205,8 +231,7 @@ cudaError_t launch_t(const QuantArgs& a, int sms, cudaStream_t s) {
   if (chunks <= 32 * 20) return launch_kept<SR, 4, 5>(a, sms, s);
   if (chunks <= 32 * 40) return launch_kept<SR, 4, 10>(a, sms, s);
   const int64_t want = (a.rows + 7) / 8, cap = (int64_t)sms * 6;
-  quantize_rowscale_long_kernel<SR><<<(unsigned)(want < cap ? want : cap), 256, 0, s>>>(a);
-  return cudaGetLastError();
+  return launch_streaming<quantize_rowscale_long_kernel<SR>>((unsigned)(want < cap ? want : cap), 256, s, a);
 }
 
 }  // namespace

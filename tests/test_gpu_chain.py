@@ -88,3 +88,31 @@ def test_a_call_sees_what_precedes_it(kind, before):
         for got, ref in zip(res, want):
             assert torch.equal(got, ref)
     B.nvfp4_device_status()
+
+
+# chunks of 16 a lane keeps: 2 | 2 of two warps | 5 | 5 of two | 5 of four | 10 of four | rows read twice
+@pytest.mark.parametrize("cols", [1024, 2048, 2560, 5120, 10240, 20480, 20608])
+@pytest.mark.parametrize("rounding", [B.ROUND_NEAREST_EVEN, B.ROUND_STOCHASTIC])
+def test_row_scaled_copies_of_any_length_in_a_chain(cols, rounding):
+    """The row-scaled quantizer is resident before the kernel that makes its source and the product that reads its last copy have
+    finished: the source and the copy are those of a quiet GPU all the same."""
+    rows = 128
+    src = torch.randn((rows, cols), generator=torch.Generator("cuda").manual_seed(cols), device="cuda").to(torch.bfloat16)
+    opts = B.quant_opts(rounding=rounding, seed=7, sr_offset=3)
+    layout = B.SF_SWIZZLED if cols % 64 == 0 else B.SF_LINEAR
+    want = B.alloc_tensor(rows, cols, layout, format=B.FORMAT_NVFP4_ROWSCALE)
+    B.nvfp4_quantize(src, opts, want, None)
+    torch.cuda.synchronize()
+    x, got = torch.empty_like(src), B.alloc_tensor(rows, cols, layout, format=B.FORMAT_NVFP4_ROWSCALE)
+    big = torch.randn((2048, 2048), device="cuda")
+    total = torch.zeros(2, dtype=torch.float64, device="cuda")
+    for _ in range(10):
+        x.fill_(float("nan"))
+        torch.mm(big, big)
+        torch.mul(src, 1.0, out=x)
+        B.nvfp4_quantize(x, opts, got, None)
+        first = B.nvfp4_quant_error(x, got, total).clone()  # reads the copy while the next call is resident
+        B.nvfp4_quantize(x, opts, got, None)
+        for a, b in ((got.codes, want.codes), (got.scales, want.scales), (got.glob, want.glob)):
+            assert torch.equal(a, b)
+        assert float(first[0]) < 0.02 * float(first[1])
