@@ -69,21 +69,32 @@ __device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wa
 __device__ __forceinline__ void griddep_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 #ifdef __CUDACC__
+// carveout: per cent of the SM that the kernel wants as shared memory, or -1 for whatever there is.  Between kernels launched this way
+// an SM stays divided as the one before wanted it, nearly all shared memory behind a product or a quantizer's pass 2, and a kernel
+// that streams with loads of its own finds little L1 for those in flight.
 template <typename... Params, typename... Args>
-inline cudaError_t launch_kernel(void (*kern)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
-                                 Args&&... args) {
+inline cudaError_t launch_divided(int carveout, void (*kern)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                                  Args&&... args) {
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = grid;
   cfg.blockDim = block;
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+  attr[1].val.sharedMemCarveout = (unsigned)carveout;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = carveout < 0 ? 1 : 2;
   return cudaLaunchKernelEx(&cfg, kern, static_cast<Params>(args)...);
 }
+template <typename... Params, typename... Args>
+inline cudaError_t launch_kernel(void (*kern)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                                 Args&&... args) {
+  return launch_divided(-1, kern, grid, block, smem, s, static_cast<Args&&>(args)...);
+}
+constexpr int kStreamingCarveout = 7;  // 16 KB; with 15 per cent or more an SM was not divided again (see quantize_rowscale.cu)
 #endif
 
 // ---- host-side tensor-map encoder (driver entry point fetched through the runtime) ----

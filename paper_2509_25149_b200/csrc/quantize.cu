@@ -1171,7 +1171,10 @@ cudaError_t launch_amax_f32(const QuantArgs& a, bool has_row, bool has_col, cuda
   if (e != cudaSuccess) return e;
   const int tiles_c = (int)((a.cols + 127) / 128);
   const unsigned tiles = (unsigned)(((a.rows + 127) / 128) * tiles_c);
-  e = launch_kernel(amax_f32_kernel, dim3(tiles), dim3(256), 0, s, reinterpret_cast<const float*>(a.x), a.rows, a.cols,
+  // Its loads do not fit the L1 beside the shared memory of the pass 2 before it (calls on three tensors in turn, 7168 x 5120: 55.5 us ->
+  // 54.5).  The bf16 kernels of pass 1 gain nothing: behind a product within the measurement's 1 %, behind another quantizer's pass 2
+  // they lose 0.3 to 0.8 % (their first CTAs then fit beside the last ones of that pass only as the SM is).
+  e = launch_divided(kStreamingCarveout, amax_f32_kernel, dim3(tiles), dim3(256), 0, s, reinterpret_cast<const float*>(a.x), a.rows, a.cols,
                     a.ld, tiles_c, has_row ? a.r_global : nullptr, has_col ? a.c_global : nullptr);
   count_launch();
   return e;

@@ -12,8 +12,6 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
-#include <utility>
-
 #include "async_ptx.cuh"
 #include "common.cuh"
 #include "quantize.h"
@@ -199,23 +197,11 @@ __global__ void __launch_bounds__(256) quantize_rowscale_long_kernel(const Quant
 // is left as L1: forward of 16384 x 1024 x 5120 88 us with an ordinary launch, 96 with a programmatic one, 85.4 where the kernel
 // asks for 7 % of the SM as shared memory (16 KB, eight CTAs of 1.1 KB); 16384 x 5120 x 5120 243 / 250 / 237, 1024 x 2048 x 2048
 // 12.3 / 10.9 / 9.9.  (15 % and more do not make an SM change, and with none at all rows of 20480, whose CTAs have 3 KB, lose 40 %.)
-constexpr int kCarveoutPercent = 7;
-template <auto KERN, typename... Args>
-cudaError_t launch_streaming(unsigned grid, unsigned block, cudaStream_t s, Args&&... args) {
-  static std::atomic<uint64_t> configured{0};  // per kernel and device
-  int dev;
-  if (device_needs_config(configured, &dev)) {
-    const cudaError_t e = cudaFuncSetAttribute(KERN, cudaFuncAttributePreferredSharedMemoryCarveout, kCarveoutPercent);
-    if (e != cudaSuccess) return e;
-    device_configured(configured, dev);
-  }
-  return launch_kernel(KERN, dim3(grid), dim3(block), 0, s, std::forward<Args>(args)...);
-}
-
 template <bool SR, int WPR, int KEEP>
 cudaError_t launch_kept(const QuantArgs& a, int sms, cudaStream_t s) {
   const int64_t want = (a.rows * WPR + 3) / 4, cap = (int64_t)sms * ctas_per_sm(KEEP) * 4;  // up to four rounds of CTAs
-  return launch_streaming<quantize_rowscale_kernel<SR, WPR, KEEP>>((unsigned)(want < cap ? want : cap), 128, s, a);
+  return launch_divided(kStreamingCarveout, quantize_rowscale_kernel<SR, WPR, KEEP>, dim3((unsigned)(want < cap ? want : cap)), dim3(128), 0,
+                        s, a);
 }
 
 template <bool SR>
@@ -231,7 +217,7 @@ cudaError_t launch_t(const QuantArgs& a, int sms, cudaStream_t s) {
   if (chunks <= 32 * 20) return launch_kept<SR, 4, 5>(a, sms, s);
   if (chunks <= 32 * 40) return launch_kept<SR, 4, 10>(a, sms, s);
   const int64_t want = (a.rows + 7) / 8, cap = (int64_t)sms * 6;
-  return launch_streaming<quantize_rowscale_long_kernel<SR>>((unsigned)(want < cap ? want : cap), 256, s, a);
+  return launch_divided(kStreamingCarveout, quantize_rowscale_long_kernel<SR>, dim3((unsigned)(want < cap ? want : cap)), dim3(256), 0, s, a);
 }
 
 }  // namespace
