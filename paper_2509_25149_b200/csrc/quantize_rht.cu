@@ -64,6 +64,7 @@ __global__ void __launch_bounds__(256, 3) quantize_rht_kernel(const RhtArgs ra) 
   extern __shared__ __align__(128) uint8_t smem[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int tile = MODE == 0 ? (int)blockIdx.x : (int)(gridDim.x - 1 - blockIdx.x);  // pass 2 walks backwards (L2)
+  griddep_wait();               // (nothing to wait for after an ordinary launch)
   griddep_launch_dependents();  // the GEMM of a composed call may set itself up while the last CTAs run
   const int64_t row0 = (int64_t)(tile / a.tiles_c) * 128;
   const int64_t col0 = (int64_t)(tile % a.tiles_c) * 128;
@@ -332,8 +333,15 @@ cudaError_t launch_mode(const RhtArgs& ra, cudaStream_t s) {
     device_configured(configured, dev);
   }
   const int smem = (ra.d == 128 && ra.has_col && ra.rht_col) ? RhtSmem::kBytesBig : RhtSmem::kBytesSmall;
-  kern<<<(unsigned)((int64_t)ra.q.tiles_r * ra.q.tiles_c), 256, smem, s>>>(ra);
+  const dim3 grid((unsigned)((int64_t)ra.q.tiles_r * ra.q.tiles_c));
   count_launch();
+  // Programmatic, because the next kernel behind an ordinary launch begins on a grid of 2.05 us: d = 4, gradient of 2816 x 2304 20.5 ->
+  // 18.7 us, of 8192 x 5120 92.4 -> 91.0, fwd + bwd of 512 x 1024 x 1024 44.0 -> 39.8, 4096 x 4096 x 4096 200.4 -> 196.8.  Not with the
+  // tile in FP32 for d = 128 (90 KB a CTA): by itself the call gains as well (41.0 -> 36.3, 185 -> 182), but behind a product an SM then
+  // keeps less L1 for the loads of a tile, and fwd + bwd of 2816 x 3328 x 2304 goes from 142.4 to 144.6, 4096 x 4096 x 4096 from 279.2 to
+  // 282.6, whatever division of the SM is asked for.
+  if (smem == RhtSmem::kBytesSmall) return launch_kernel(kern, grid, dim3(256), smem, s, ra);
+  kern<<<grid, 256, smem, s>>>(ra);
   return cudaGetLastError();
 }
 

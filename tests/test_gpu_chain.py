@@ -116,3 +116,28 @@ def test_row_scaled_copies_of_any_length_in_a_chain(cols, rounding):
         for a, b in ((got.codes, want.codes), (got.scales, want.scales), (got.glob, want.glob)):
             assert torch.equal(a, b)
         assert float(first[0]) < 0.02 * float(first[1])
+
+
+@pytest.mark.parametrize("dim", [2, 8, 128])
+@pytest.mark.parametrize("copies", ["both", "row"])
+def test_other_transform_sizes_in_a_chain(dim, copies):
+    """The same for the kernel of the other transform sizes, which is launched either way (d = 128: by whether the transposed copy is
+    asked for)."""
+    rows, cols = 384, 640
+    src = torch.randn((rows, cols), generator=torch.Generator("cuda").manual_seed(dim), device="cuda").to(torch.bfloat16)
+    opts = B.quant_opts(rounding=1, rht_colwise=copies == "both", rht_rowwise=copies == "row", rht_sign_mask=0x73E5, rht_dim=dim, seed=1)
+
+    def quantize(x):
+        row, col = B.alloc_tensor(rows, cols), B.alloc_tensor(cols, rows) if copies == "both" else None
+        B.nvfp4_quantize(x, opts, row, col)
+        return [t for c in (row, col) if c for t in (c.codes, c.scales, c.glob)]
+
+    want = quantize(src)
+    torch.cuda.synchronize()
+    x, big = torch.empty_like(src), torch.randn((2048, 2048), device="cuda")
+    for _ in range(10):
+        x.fill_(float("nan"))
+        torch.mm(big, big)
+        torch.mul(src, 1.0, out=x)
+        first, second = quantize(x), quantize(x)
+        assert all(torch.equal(a, b) and torch.equal(a, c) for a, b, c in zip(want, first, second))
