@@ -12,21 +12,23 @@ namespace nvfp4 {
 // ---------------------------------------------------------------------------------------------
 // small PTX helpers
 // ---------------------------------------------------------------------------------------------
+// Loads of a tensor that is read once.  Coherent ones (no .nc): a kernel that is resident before its source has been written may read it
+// only that way, and the non-coherent path was no faster (quantizers of every role: within the 1 % that two runs differ).
 __device__ __forceinline__ void ldg256_stream(const void* p, uint32_t (&r)[8]) {
-  asm volatile("ld.global.nc.L1::no_allocate.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+  asm volatile("ld.global.L1::no_allocate.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
                  "=r"(r[7])
                : "l"(p));
 }
 __device__ __forceinline__ void ldg256_hint(const void* p, uint32_t (&r)[8], uint64_t policy) {
-  asm volatile("ld.global.nc.L1::no_allocate.L2::cache_hint.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8], %9;"
+  asm volatile("ld.global.L1::no_allocate.L2::cache_hint.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8], %9;"
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
                  "=r"(r[7])
                : "l"(p), "l"(policy));
 }
 __device__ __forceinline__ uint4 ldg128_stream(const void* p) {
   uint4 r;
-  asm volatile("ld.global.nc.L1::no_allocate.v4.b32 {%0,%1,%2,%3}, [%4];"
+  asm volatile("ld.global.L1::no_allocate.v4.b32 {%0,%1,%2,%3}, [%4];"
                : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w)
                : "l"(p));
   return r;

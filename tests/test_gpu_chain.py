@@ -141,3 +141,79 @@ def test_other_transform_sizes_in_a_chain(dim, copies):
         torch.mul(src, 1.0, out=x)
         first, second = quantize(x), quantize(x)
         assert all(torch.equal(a, b) and torch.equal(a, c) for a, b, c in zip(want, first, second))
+
+
+def _quantized(rows, cols, seed, scale):
+    t = B.alloc_tensor(rows, cols)
+    x = torch.randn((rows, cols), generator=torch.Generator("cuda").manual_seed(seed), device="cuda") * scale
+    B.nvfp4_quantize(x.to(torch.bfloat16), B.quant_opts(block_rows=16), t, None)
+    return t
+
+
+class _Chain:
+    """Two products write D in turn (one in FP4, one in BF16), `quantize` turns D into the shared copies, and a product on each copy
+    reads them: every kernel is this library's own and resident before the one before it has finished, D and the copies are
+    overwritten while the kernels that read them may still run."""
+
+    def __init__(self, rows, cols, quantize, copies, fp32=False):
+        g = torch.Generator("cuda").manual_seed(rows + cols)
+        self.a, self.w = _quantized(rows, 256, 1, 1.0), _quantized(cols, 256, 2, 0.1)
+        self.x, self.y = (torch.randn((n, 256), generator=g, device="cuda").to(torch.bfloat16) for n in (rows, cols))
+        self.D = torch.empty((rows, cols), dtype=torch.float32 if fp32 else torch.bfloat16, device="cuda")
+        self.quantize, self.copies = quantize, copies
+        # products of 1024 columns, four tiles and more: they leave the GPU's SMs at different times
+        self.other = [_quantized(1024, c.cols, 3, 1.0) for c in copies]
+        self.out = [[torch.empty((c.rows, 1024), dtype=torch.bfloat16, device="cuda") for c in copies] for _ in range(2)]
+
+    def round(self, i, sync=lambda: None):
+        if i == 0:
+            B.nvfp4_gemm(self.a, self.w, self.D)
+        else:
+            B.nvfp4_gemm_bf16(self.x, self.y, self.D)
+        sync()
+        self.quantize(self.D)
+        sync()
+        for c, o, e in zip(self.copies, self.other, self.out[i]):
+            B.nvfp4_gemm(c, o, e)
+            sync()
+
+    def bytes(self):
+        return [e.clone() for o in self.out for e in o] + [t.clone() for c in self.copies for t in (c.codes, c.scales, c.glob)]
+
+    def check(self):
+        for i in (0, 1):
+            self.round(i, torch.cuda.synchronize)
+        want = self.bytes()
+        assert not torch.equal(self.out[0][0], self.out[1][0])
+        for _ in range(5):
+            for t in [e for o in self.out for e in o] + [c.codes for c in self.copies]:
+                t.zero_()
+            self.D.fill_(float("nan"))
+            torch.cuda.synchronize()
+            for _ in range(2):
+                for i in (0, 1):
+                    self.round(i)
+            assert all(torch.equal(a, b) for a, b in zip(self.bytes(), want))
+        graph, side = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+        with torch.cuda.stream(side):
+            with torch.cuda.graph(graph, stream=side):
+                for i in (0, 1):
+                    self.round(i)
+        for _ in range(3):
+            for o in self.out:
+                for e in o:
+                    e.zero_()
+            graph.replay()
+        torch.cuda.synchronize()
+        assert all(torch.equal(a, b) for a, b in zip(self.bytes(), want))
+        B.nvfp4_device_status()
+
+
+# the row lengths of the test above (multiples of 256, as the product on the copy contracts over them)
+@pytest.mark.parametrize("cols", [1024, 2048, 2560, 5120, 10240, 20480, 20736])
+@pytest.mark.parametrize("rounding", [B.ROUND_NEAREST_EVEN, B.ROUND_STOCHASTIC])
+def test_row_scaled_copies_between_products(cols, rounding):
+    rows = 256
+    copy = B.alloc_tensor(rows, cols, format=B.FORMAT_NVFP4_ROWSCALE)
+    opts = B.quant_opts(rounding=rounding, seed=7, sr_offset=3)
+    _Chain(rows, cols, lambda x: B.nvfp4_quantize(x, opts, copy, None), [copy]).check()
