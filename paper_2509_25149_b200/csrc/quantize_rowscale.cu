@@ -66,8 +66,11 @@ __device__ __forceinline__ void encode_chunk(const QuantArgs& a, const uint32_t 
   a.r_scales[a.r_swz ? sf_swizzled_offset(row, cb, n_cb) : (row * n_cb + cb)] = (uint8_t)byte;
 }
 
-// CTAs resident per SM by what a lane keeps (registers).  Five chunks: 64 registers, two of which spill, and eight CTAs read 16384 x
-// 5120 in 38.9 us, six with 74 registers in 40.8 (ordinary launches).
+// CTAs resident per SM by what a lane keeps (registers).  Eight with five chunks: 64 registers, and with one or two warps a row 8 to 24
+// bytes of a thread spill; six: 71 to 78 and none.  Six / eight, sources in turn that exceed L2: 16384 x 2064 16.7 / 16.0 us, 16384 x 5120
+// 37.1 / 35.6, 16384 x 7168 54.7 / 52.1, 8192 x 10240 36.1 / 34.8, with stochastic rounding 25.7 / 25.5, 53.4 / 52.3, 80.9 / 76.3, 52.6 /
+// 51.2.  Six would be faster where 1024 CTAs all fit at once but not evenly: 4096 x 2560 7.1 / 7.7, 1024 x 10240 6.8 / 7.5, with
+// stochastic rounding 10.0 / 10.7 and 10.2 / 10.7, behind a product 16.4 / 16.6 and 19.4 / 19.9.
 constexpr int ctas_per_sm(int keep) { return keep <= 5 ? 8 : 4; }
 
 // WPR warps per row (1, 2 or 4): row (4 / WPR) * i + w / WPR of iteration i belongs to warp w, whose lanes take every WPR-th
@@ -198,17 +201,36 @@ __global__ void __launch_bounds__(256) quantize_rowscale_long_kernel(const Quant
   }
 }
 
-// Programmatic launch: behind an ordinary one the next kernel begins on a grid of 2.05 us (a row-wise copy of 8192 x 1536 took 10.24 us
-// by the side of 7.47, 1024 x 7168 6.15 / 5.14, 16384 x 2560 20.5 / 19.0).  Without an ordinary launch's pause, though, the SMs stay
-// divided the way the kernel before wanted them, nearly all shared memory behind a product, and the loads in flight do not fit what
-// is left as L1: forward of 16384 x 1024 x 5120 88 us with an ordinary launch, 96 with a programmatic one, 85.4 where the kernel
-// asks for 7 % of the SM as shared memory (16 KB, eight CTAs of 1.1 KB); 16384 x 5120 x 5120 243 / 250 / 237, 1024 x 2048 x 2048
-// 12.3 / 10.9 / 9.9.  (15 % and more do not make an SM change, and with none at all rows of 20480, whose CTAs have 3 KB, lose 40 %.)
+// Programmatic launch: behind an ordinary one the next kernel begins on a grid of 2.05 us.  Without an ordinary launch's pause, though, the
+// SMs stay divided the way the kernel before wanted them, nearly all shared memory behind a product, and the loads in flight do not fit
+// what is left as L1; so the kernel asks for 7 % of the SM as shared memory (15 % and more do not make an SM change, and with none at all
+// rows of 20480, whose CTAs have 3 KB, lose 40 %).  Sources in turn that exceed L2, ordinary / programmatic / that with the division, all
+// with eight CTAs: copies of 8192 x 1536 10.3 / 8.6 / 8.6 us, 16384 x 2560 20.5 / 18.8 / 18.8, 16384 x 5120 37.0 / 35.7 / 35.9; forward
+// calls of 16384 x 1024 x 5120 82.2 to 84.2 / 94.8 to 97.9 / 80.5 to 82.6, 4096 x 4096 x 4096 47.1 / 49.0 / 45.2, 16384 x 5120 x 5120
+// 231 / 251 / 230 (two runs of one build differ by 1 %).
+//
+// Few CTAs crowd that way: they become resident while a product still runs, as many as fit an SM on each that has none of its tiles.  So
+// up to four CTAs per SM have a share of 16 KB each as shared memory, and no more of them fit an SM than an even spread puts there.  Behind
+// a product of 64 tiles, ordinary / crowded / spread: 512 x 20608 39.6 / 51.2 / 36.7 us, 512 x 5120 14.4 / 15.1 / 12.5, with stochastic
+// rounding 44.4 / 73.6 / 39.1 and 14.4 / 18.0 / 13.4; forward of 256 x 1024 x 24576 with a fresh weight 65.1 / 86.2 / 61.3, of 1024 x 2048
+// x 2048 10.3 / 10.4 / 9.3.  For this the kernel asks for 5 %: CTAs of 3.5 KB and more then meet an SM divided at 16 KB; with 7 % some
+// sizes meet 32 KB (seen by how many were resident: of 4 KB eight).  From five CTAs per SM on the even shares would be below that; there
+// nothing lost against an ordinary launch of six (1024 x 7168 to 20480 x 5120, alone and behind a product 1.5 to 35 % faster).
+constexpr int kSpreadCarveout = 5, kSpreadBytes = 16384, kSpreadCtas = 4;
+
+template <typename Kernel>
+cudaError_t launch_spread(Kernel kern, int64_t want, int64_t cap, int threads, int static_smem, const QuantArgs& a, int sms, cudaStream_t s) {
+  const int64_t per_sm = (want + sms - 1) / sms;
+  const bool few = per_sm <= kSpreadCtas;
+  const size_t smem = few ? (size_t)((kSpreadBytes / per_sm) & ~127) - (size_t)static_smem - 1024 : 0;  // (1 KB a CTA is the system's)
+  return launch_divided(few ? kSpreadCarveout : kStreamingCarveout, kern, dim3((unsigned)(want < cap ? want : cap)), dim3((unsigned)threads),
+                        smem, s, a);
+}
+
 template <bool SR, int WPR, int KEEP>
 cudaError_t launch_kept(const QuantArgs& a, int sms, cudaStream_t s) {
   const int64_t want = (a.rows * WPR + 3) / 4, cap = (int64_t)sms * ctas_per_sm(KEEP) * 4;  // up to four rounds of CTAs
-  return launch_divided(kStreamingCarveout, quantize_rowscale_kernel<SR, WPR, KEEP>, dim3((unsigned)(want < cap ? want : cap)), dim3(128), 0,
-                        s, a);
+  return launch_spread(quantize_rowscale_kernel<SR, WPR, KEEP>, want, cap, 128, KEEP >= 10 && !SR ? 2176 : 128, a, sms, s);
 }
 
 template <bool SR>
@@ -223,8 +245,7 @@ cudaError_t launch_t(const QuantArgs& a, int sms, cudaStream_t s) {
   if (chunks <= 32 * 10) return launch_kept<SR, 2, 5>(a, sms, s);
   if (chunks <= 32 * 20) return launch_kept<SR, 4, 5>(a, sms, s);
   if (chunks <= 32 * 40) return launch_kept<SR, 4, 10>(a, sms, s);
-  const int64_t want = (a.rows + 7) / 8, cap = (int64_t)sms * 6;
-  return launch_divided(kStreamingCarveout, quantize_rowscale_long_kernel<SR>, dim3((unsigned)(want < cap ? want : cap)), dim3(256), 0, s, a);
+  return launch_spread(quantize_rowscale_long_kernel<SR>, (a.rows + 7) / 8, (int64_t)sms * 6, 256, 0, a, sms, s);
 }
 
 }  // namespace

@@ -149,3 +149,55 @@ def test_forward_only_layer_with_row_scaled_activations():
     P.assert_gemm_close(Y.float().cpu().numpy(), Dref, T, True, "forward-only layer")
     with pytest.raises(B.NVFP4Error):  # a saved transposed copy cannot be made with row scales
         B.nvfp4_linear_fwd(x.cuda(), w.cuda(), o, Y, B.alloc_tensor(K, M), W_row, None, False, ws)
+
+
+# CTAs of one, two or four rows (eight of the longest rows): as many as SMs and some more, four times that and some more (the most that
+# are given a share of shared memory each), and more than the grid has (rows of a second turn; beside it the row where that begins)
+@pytest.mark.parametrize("rounding", [oracle.RNE, oracle.SR])
+@pytest.mark.parametrize("rows,cols", [(592, 1024), (608, 1024), (2368, 1024), (2384, 1024), (144, 20480), (160, 20480), (592, 20480),
+                                       (608, 20480), (1184, 20608), (1200, 20608), (4736, 20608), (4752, 20608), (18960, 1024),
+                                       (9488, 2048), (18960, 2560), (9488, 5120), (4768, 10240), (2384, 20480), (7120, 20608)])
+def test_numbers_of_ctas(rows, cols, rounding):
+    x = synth.normal_with_outliers_bf16_device((rows, cols), 0.01, 40.0, rows)
+    t = B.alloc_tensor(rows, cols, B.SF_LINEAR, format=B.FORMAT_NVFP4_ROWSCALE)
+    B.nvfp4_quantize(x, B.quant_opts(rounding=rounding, seed=3, sr_offset=9), t, None)
+    torch.cuda.synchronize()
+    for r0 in {0, rows // 2 // 16 * 16, rows - 32, rows - 16}:  # (a second turn takes the last 16 rows or the last 32)
+        ref = oracle.quantize_rowscale(synth.bits(x[r0:r0 + 16].cpu()), rounding=rounding, seed=3, sr_offset=9, sr_row0=r0, sr_cols=cols)
+        part = B.NVFP4Tensor(t.codes[r0:r0 + 16], t.scales.view(rows, -1)[r0:r0 + 16], t.glob.view(rows, 2)[r0:r0 + 16], 16, cols, B.SF_LINEAR,
+                             t.format)
+        assert_rows_exact(part, ref, f"rows {r0}..")
+
+
+@pytest.mark.parametrize("rounding", [oracle.RNE, oracle.SR])
+def test_few_ctas_do_not_crowd_where_a_product_has_left_room(rounding):
+    """64 CTAs behind a product of 64 tiles on 74 pairs of SMs: the two together take no longer than one after the other (crowded onto
+    the 20 SMs that are free they took 1.3 and 1.7 times as long)."""
+    A, W = B.alloc_tensor(2048, 2048), B.alloc_tensor(2048, 2048)
+    for t, seed in ((A, 1), (W, 2)):
+        B.nvfp4_quantize(synth.normal_bf16_device((2048, 2048), 1.0, seed), B.quant_opts(), t, None)
+    D = torch.empty((2048, 2048), dtype=torch.bfloat16, device="cuda")
+    x = synth.normal_bf16_device((512, 20608), 1.0, 3)
+    copy, opts = B.alloc_tensor(512, 20608, format=B.FORMAT_NVFP4_ROWSCALE), B.quant_opts(rounding=rounding, seed=1)
+
+    def product():
+        B.nvfp4_gemm(A, W, D)
+
+    def quantizer():
+        B.nvfp4_quantize(x, opts, copy, None)
+
+    def time(*calls):
+        best = []
+        for _ in range(7):
+            start, end = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            start.record()
+            for _ in range(200):
+                for c in calls:
+                    c()
+            end.record()
+            end.synchronize()
+            best.append(start.elapsed_time(end))
+        return sorted(best)[3]
+
+    time(product, quantizer)
+    assert time(product, quantizer) <= 1.15 * (time(product) + time(quantizer))
