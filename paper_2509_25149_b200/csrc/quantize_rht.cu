@@ -322,42 +322,65 @@ __global__ void __launch_bounds__(256, 3) quantize_rht_kernel(const RhtArgs ra) 
   }
 }
 
+// Shared memory with which one CTA, or two, fit an SM (228 KB, of which 1 KB a CTA is the system's)
+constexpr int kOnePerSm = 116 * 1024, kTwoPerSm = 77 * 1024;
+
+// Pass 2 with no more CTAs than SMs, or than twice as many, is given the shared memory with which no more fit an SM than an even spread
+// puts there: launched programmatically it becomes resident while a product or pass 1 still runs, and three crowd on each SM that is
+// free.  d = 4, ordinary launch / crowded / spread: gradient of 512 x 2048 with its amax provided, behind a product of 64 tiles, 20.4 /
+// 23.3 / 18.5 us, activation 18.4 / 19.4 / 16.7; with pass 1, gradient of 2048 x 2048 16.4 / 17.6 / 14.6; fwd + bwd of 2048 x 2048 x 2048
+// 69.6 / 67.7 / 63.5.
 template <int MODE, bool SR>
-cudaError_t launch_mode(const RhtArgs& ra, cudaStream_t s) {
+cudaError_t launch_mode(const RhtArgs& ra, bool programmatic, int sms, cudaStream_t s) {
   auto kern = quantize_rht_kernel<MODE, SR>;
   static std::atomic<uint64_t> configured{0};  // per call site (template instantiation) and device
   int dev;
   if (device_needs_config(configured, &dev)) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, RhtSmem::kBytesBig);
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kOnePerSm);
     if (e != cudaSuccess) return e;
     device_configured(configured, dev);
   }
-  const int smem = (ra.d == 128 && ra.has_col && ra.rht_col) ? RhtSmem::kBytesBig : RhtSmem::kBytesSmall;
-  const dim3 grid((unsigned)((int64_t)ra.q.tiles_r * ra.q.tiles_c));
+  const bool big = ra.d == 128 && ra.has_col && ra.rht_col;
+  const int64_t tiles = (int64_t)ra.q.tiles_r * ra.q.tiles_c;
+  const dim3 grid((unsigned)tiles);
   count_launch();
-  // Programmatic, because the next kernel behind an ordinary launch begins on a grid of 2.05 us: d = 4, gradient of 2816 x 2304 20.5 ->
-  // 18.7 us, of 8192 x 5120 92.4 -> 91.0, fwd + bwd of 512 x 1024 x 1024 44.0 -> 39.8, 4096 x 4096 x 4096 200.4 -> 196.8.  Not with the
-  // tile in FP32 for d = 128 (90 KB a CTA): by itself the call gains as well (41.0 -> 36.3, 185 -> 182), but behind a product an SM then
-  // keeps less L1 for the loads of a tile, and fwd + bwd of 2816 x 3328 x 2304 goes from 142.4 to 144.6, 4096 x 4096 x 4096 from 279.2 to
-  // 282.6, whatever division of the SM is asked for.
-  if (smem == RhtSmem::kBytesSmall) return launch_kernel(kern, grid, dim3(256), smem, s, ra);
-  kern<<<grid, 256, smem, s>>>(ra);
+  if (programmatic && !big) {
+    const int smem = MODE == 1 && tiles <= sms ? kOnePerSm : MODE == 1 && tiles <= 2 * sms ? kTwoPerSm : RhtSmem::kBytesSmall;
+    return launch_kernel(kern, grid, dim3(256), smem, s, ra);
+  }
+  kern<<<grid, 256, big ? RhtSmem::kBytesBig : RhtSmem::kBytesSmall, s>>>(ra);
   return cudaGetLastError();
 }
 
 }  // namespace
 
+// Which launches are programmatic: the next kernel behind an ordinary one begins on a grid of 2.05 us, but without an ordinary one's pause
+// an SM keeps little L1 behind a product or another quantizer's pass 2, too little for the loads of more than one tile.
+//   Pass 2 is, in the recipe's case, where a pass 1 on the tensor cores comes before it (d = 4, ordinary / programmatic: gradient of 2816 x
+//   2304 21.9 / 19.9 us, of 8192 x 5120 96.7 / 95.2, fwd + bwd of 512 x 1024 x 1024 43.6 / 39.9, 4096 x 4096 x 4096 201.4 / 196.1; d = 2
+//   and d = 8 the same within 1 %), behind pass 1 of this file and where the amax is provided (8192 x 5120 64.1 / 62.5).
+//   Not with the tile in FP32 for d = 128 (90 KB a CTA): by itself the call gains as well (41.0 / 36.3, 185 / 182), but fwd + bwd of 2816 x
+//   3328 x 2304 goes from 142.4 to 144.6, 4096 x 4096 x 4096 from 279.2 to 282.6, whatever division of the SM is asked for.
+//   Neither pass of a row-wise transform with stochastic rounding on few tiles: behind a product 512 x 1024, both copies, 26.7 / 28.6 (d =
+//   128 30.7 / 32.4), although by itself 18.5 / 14.4.
+//   Pass 1 of this file is with at most a tile per SM: forward of 512 x 1024 x 1024 with a cached weight, d = 4, no transposed copy, 16.4 /
+//   14.3.  Not with more: the same with a fresh weight, 2048 x 4096 x 4096, 51.8 / 54.7, 4096 x 4096 x 4096 78.6 / 82.4, although by itself
+//   an activation of 2816 x 2304 takes 12.5 / 11.2.
 cudaError_t launch_quantize_rht(const RhtArgs& ra, bool amax_provided, bool sr, cudaStream_t s) {
-  cudaError_t e;
+  int sms = 0;
+  cudaError_t e = sm_count(&sms);
+  if (e != cudaSuccess) return e;
+  const bool few = (int64_t)ra.q.tiles_r * ra.q.tiles_c <= sms;
+  const bool held = few && sr && ra.rht_row && !amax_provided;
   if (!amax_provided && ra.d <= 16 && ra.has_col && ra.rht_col && !ra.rht_row) {
     // the recipe's case (plain row-wise copy, transformed transposed copy): pass 1 on the tensor cores, HBM-bound
     if ((e = launch_amax_rot_col_small(ra.q, ra.has_row != 0, ra.mask16, ra.d, ra.norm, s)) != cudaSuccess) return e;
   } else if (!amax_provided) {
     e = launch_zero_words(ra.has_row ? ra.q.r_global : nullptr, ra.has_col ? ra.q.c_global : nullptr, nullptr, nullptr, s);
     if (e != cudaSuccess) return e;
-    if ((e = launch_mode<0, false>(ra, s)) != cudaSuccess) return e;
+    if ((e = launch_mode<0, false>(ra, few && !held, sms, s)) != cudaSuccess) return e;
   }
-  return sr ? launch_mode<1, true>(ra, s) : launch_mode<1, false>(ra, s);
+  return sr ? launch_mode<1, true>(ra, !held, sms, s) : launch_mode<1, false>(ra, true, sms, s);
 }
 
 }  // namespace nvfp4

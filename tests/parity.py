@@ -263,3 +263,31 @@ def assert_mx_rht_close(x_bits: np.ndarray, gpu: B.NVFP4Tensor, *, colwise, sign
         excused += 1
     assert excused + int(np.count_nonzero(sdiff)) * 32 <= max(1e-3 * R * C, 32), f"{what}: too many excused items"
     return {"excused_codes": excused, "excused_scales": int(np.count_nonzero(sdiff)), "elements": R * C}
+
+
+def crowding(quantizer):
+    """Time of a product of 64 tiles (on 64 of 74 pairs of SMs) and `quantizer` behind it, over that of one after the other (medians of
+    loops of 200): kernels that become resident while a product still runs may crowd on the SMs that it leaves free."""
+    A, W = B.alloc_tensor(2048, 2048), B.alloc_tensor(2048, 2048)
+    for t, seed in ((A, 1), (W, 2)):
+        B.nvfp4_quantize(synth.normal_bf16_device((2048, 2048), 1.0, seed), B.quant_opts(), t, None)
+    D = torch.empty((2048, 2048), dtype=torch.bfloat16, device="cuda")
+
+    def product():
+        B.nvfp4_gemm(A, W, D)
+
+    def time(*calls):
+        took = []
+        for _ in range(7):
+            start, end = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            start.record()
+            for _ in range(200):
+                for c in calls:
+                    c()
+            end.record()
+            end.synchronize()
+            took.append(start.elapsed_time(end))
+        return sorted(took)[3]
+
+    time(product, quantizer)
+    return time(product, quantizer) / (time(product) + time(quantizer))

@@ -217,3 +217,19 @@ def test_row_scaled_copies_between_products(cols, rounding):
     copy = B.alloc_tensor(rows, cols, format=B.FORMAT_NVFP4_ROWSCALE)
     opts = B.quant_opts(rounding=rounding, seed=7, sr_offset=3)
     _Chain(rows, cols, lambda x: B.nvfp4_quantize(x, opts, copy, None), [copy]).check()
+
+
+# 8 tiles, 192 and 396 (one CTA per SM, two, as many as fit)
+@pytest.mark.parametrize("rows,cols", [(256, 512), (1536, 2048), (2816, 2304)])
+@pytest.mark.parametrize("dim", [4, 128])
+@pytest.mark.parametrize("form", ["col", "row", "both rotated", "provided"])
+def test_other_transform_sizes_between_products(rows, cols, dim, form):
+    """The forms that differ in which of their launches are programmatic: the recipe's two copies, a row-wise one, two transformed ones,
+    and two whose amax is provided, so that pass 2 is the call's first kernel."""
+    row, col = B.alloc_tensor(rows, cols), B.alloc_tensor(cols, rows)
+    kw = dict(rounding=B.ROUND_STOCHASTIC, rht_colwise=form != "row", rht_rowwise=form != "col", rht_sign_mask=0x73E5, rht_dim=dim, seed=1)
+    opts = B.quant_opts(flags=B.AMAX_PROVIDED if form == "provided" else 0, **kw)
+    for t in (row, col):
+        t.glob[0] = 400.0  # (a bound on both products' outputs, and on their transforms')
+    copies = [row] if form == "row" else [row, col]
+    _Chain(rows, cols, lambda x: B.nvfp4_quantize(x, opts, row, col if form != "row" else None), copies).check()

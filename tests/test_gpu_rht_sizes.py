@@ -131,3 +131,56 @@ def test_linear_layer_with_another_transform_size(d):
     Dref, T = oracle.gemm_tn(oracle.dequantize(gg), oracle.dequantize(gx))
     err = np.abs(dW.cpu().numpy() - Dref)
     assert np.count_nonzero(err > 1e-3 * T + 1e-30) <= 1e-3 * err.size and np.all(err <= 2e-2 * T + 1e-30)
+
+
+def test_few_tiles_do_not_crowd_where_a_product_has_left_room():
+    """64 tiles behind a product, amax provided: no slower than one after the other (crowded they took 1.3 times as long)."""
+    x = synth.normal_bf16_device((512, 2048), 1e-4, 3)
+    row, col = B.alloc_tensor(512, 2048), B.alloc_tensor(2048, 512)
+    kw = dict(rounding=B.ROUND_STOCHASTIC, rht_colwise=True, rht_sign_mask=0x5, rht_dim=4, seed=5)
+    B.nvfp4_quantize(x, B.quant_opts(**kw), row, col)
+    opts = B.quant_opts(flags=B.AMAX_PROVIDED, **kw)
+    assert P.crowding(lambda: B.nvfp4_quantize(x, opts, row, col)) <= 1.15
+
+
+# 24 tiles; 148 and 152 (pass 1 programmatic or not, one CTA per SM or two); 296 and 304 (two or as many as fit); 666
+@pytest.mark.parametrize("rows,cols", [(384, 1024), (512, 4736), (512, 4864), (1024, 4736), (1024, 4864), (4736, 2304)])
+@pytest.mark.parametrize("rounding", [oracle.RNE, oracle.SR])
+def test_numbers_of_tiles(rows, cols, rounding):
+    """Every launch of a call with another transform size, by its number of tiles and the copies: the untransformed row-wise copy against
+    the oracle's first and last rows, transformed ones against those of calls that take other launches (a copy on its own; the amax
+    provided, from the words that pass 1 has left)."""
+    x = synth.normal_with_outliers_bf16_device((rows, cols), 0.01, 40.0, rows + cols)
+    for d in (2, 128):
+        kw = dict(rounding=rounding, rht_sign_mask=mask_for(d), rht_dim=d, seed=9, sr_offset=3)
+
+        def quantize(row=True, col=True, amax=None, **opt):
+            r, c = B.alloc_tensor(rows, cols) if row else None, B.alloc_tensor(cols, rows) if col else None
+            if amax:
+                for t, a in zip((r, c), amax):
+                    t.glob[0] = a
+            B.nvfp4_quantize(x, B.quant_opts(flags=B.AMAX_PROVIDED if amax else 0, **kw, **opt), r, c)
+            return [[t.codes, t.scales, t.glob] for t in (r, c) if t], r
+
+        def same(a, b):
+            assert all(torch.equal(s, t) for s, t in zip(a, b))
+
+        (plain, col), r = quantize(rht_colwise=True)
+        amax = float(plain[2][0]), float(col[2][0])
+        assert amax[0] == float(x.float().abs().max())
+        codes, scales, glob = P.download(r)
+        for r0 in (0, rows - 16):
+            ref = oracle.quantize(synth.bits(x[r0:r0 + 16].cpu()), rounding=rounding, seed=9, sr_offset=3, sr_row0=r0, sr_cols=cols,
+                                  amax_override=amax[0])
+            assert np.array_equal(codes[r0:r0 + 16], ref.codes) and np.array_equal(scales[r0:r0 + 16], ref.scales)
+        same(quantize(col=False, rht_colwise=True)[0][0], plain)
+        same(quantize(row=False, rht_colwise=True)[0][0], col)
+        for a, b in zip(quantize(amax=amax, rht_colwise=True)[0], (plain, col)):
+            same(a, b)
+        (rot, col2), _ = quantize(rht_rowwise=True, rht_colwise=True)
+        same(quantize(col=False, rht_rowwise=True)[0][0], rot)
+        for a, b in zip(quantize(amax=(float(rot[2][0]), float(col2[2][0])), rht_rowwise=True, rht_colwise=True)[0], (rot, col2)):
+            same(a, b)
+        if d == 128:  # (with d = 2 the first col's maximum comes from the tensor cores, which sum in another order)
+            same(col2, col)
+    B.nvfp4_device_status()

@@ -171,33 +171,7 @@ def test_numbers_of_ctas(rows, cols, rounding):
 
 @pytest.mark.parametrize("rounding", [oracle.RNE, oracle.SR])
 def test_few_ctas_do_not_crowd_where_a_product_has_left_room(rounding):
-    """64 CTAs behind a product of 64 tiles on 74 pairs of SMs: the two together take no longer than one after the other (crowded onto
-    the 20 SMs that are free they took 1.3 and 1.7 times as long)."""
-    A, W = B.alloc_tensor(2048, 2048), B.alloc_tensor(2048, 2048)
-    for t, seed in ((A, 1), (W, 2)):
-        B.nvfp4_quantize(synth.normal_bf16_device((2048, 2048), 1.0, seed), B.quant_opts(), t, None)
-    D = torch.empty((2048, 2048), dtype=torch.bfloat16, device="cuda")
+    """64 CTAs behind a product: no slower than one after the other (crowded they took 1.3 and 2 times as long)."""
     x = synth.normal_bf16_device((512, 20608), 1.0, 3)
     copy, opts = B.alloc_tensor(512, 20608, format=B.FORMAT_NVFP4_ROWSCALE), B.quant_opts(rounding=rounding, seed=1)
-
-    def product():
-        B.nvfp4_gemm(A, W, D)
-
-    def quantizer():
-        B.nvfp4_quantize(x, opts, copy, None)
-
-    def time(*calls):
-        best = []
-        for _ in range(7):
-            start, end = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-            start.record()
-            for _ in range(200):
-                for c in calls:
-                    c()
-            end.record()
-            end.synchronize()
-            best.append(start.elapsed_time(end))
-        return sorted(best)[3]
-
-    time(product, quantizer)
-    assert time(product, quantizer) <= 1.15 * (time(product) + time(quantizer))
+    assert P.crowding(lambda: B.nvfp4_quantize(x, opts, copy, None)) <= 1.15
