@@ -55,7 +55,7 @@ __device__ __forceinline__ void fence_mbarrier_init() {
 // orders this thread's earlier generic-proxy accesses to shared memory before later asynchronous-proxy ones (TMA)
 __device__ __forceinline__ void fence_proxy_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
-// ---- programmatic dependent launch: every kernel launched with `launch_kernel` may become resident while the previous
+// ---- programmatic dependent launch: every kernel launched with `launch_divided` or `launch_kernel` may become resident while the previous
 // kernel of the stream drains; it runs its set-up (barriers, tensor memory, descriptor prefetch) and then waits here for
 // that kernel to finish with all its writes visible.  Behind a kernel that does not know the scheme (a caller's own) the
 // launch is held until that kernel's CTAs have exited, and the wait covers its writes.  Rules that keep it transitive:
@@ -87,7 +87,9 @@ inline cudaError_t launch_divided(int carveout, void (*kern)(Params...), dim3 gr
   attr[1].val.sharedMemCarveout = (unsigned)carveout;
   cfg.attrs = attr;
   cfg.numAttrs = carveout < 0 ? 1 : 2;
-  return cudaLaunchKernelEx(&cfg, kern, static_cast<Params>(args)...);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, static_cast<Params>(args)...);
+  if (e != cudaSuccess) (void)cudaGetLastError();  // reported here, and not left for a later ordinary launch to find
+  return e;
 }
 template <typename... Params, typename... Args>
 inline cudaError_t launch_kernel(void (*kern)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
