@@ -96,7 +96,7 @@ inline cudaError_t launch_kernel(void (*kern)(Params...), dim3 grid, dim3 block,
                                  Args&&... args) {
   return launch_divided(-1, kern, grid, block, smem, s, static_cast<Args&&>(args)...);
 }
-constexpr int kStreamingCarveout = 7;  // 16 KB; with 15 per cent or more an SM was not divided again (see quantize_rowscale.cu)
+constexpr int kStreamingCarveout = 7;  // an SM then has 32 KB; with 15 per cent or more it was not divided again (see quantize_rowscale.cu)
 #endif
 
 // ---- host-side tensor-map encoder (driver entry point fetched through the runtime) ----

@@ -1171,9 +1171,11 @@ cudaError_t launch_amax_f32(const QuantArgs& a, bool has_row, bool has_col, cuda
   if (e != cudaSuccess) return e;
   const int tiles_c = (int)((a.cols + 127) / 128);
   const unsigned tiles = (unsigned)(((a.rows + 127) / 128) * tiles_c);
-  // Its loads do not fit the L1 beside the shared memory of the pass 2 before it (calls on three tensors in turn, 7168 x 5120: 55.5 us ->
-  // 54.5).  The bf16 kernels of pass 1 gain nothing: behind a product within the measurement's 1 %, behind another quantizer's pass 2
-  // they lose 0.3 to 0.8 % (their first CTAs then fit beside the last ones of that pass only as the SM is).
+  // Its loads do not fit the L1 beside the shared memory of the pass 2, or the product, before it.  The whole call without the division /
+  // with it, sources in turn that exceed L2: 2304 x 3328 15.0 / 14.5 us, 4096 x 4096 26.0 / 25.6, 7168 x 5120 55.0 / 54.1, 20480 x 5120 139.4
+  // / 138.3, up to 2048 x 2048 the same; behind a product 2048 x 2048 20.3 / 19.8, 4096 x 4096 37.3 / 37.2, 7168 x 5120 65.3 / 64.7.  The
+  // bf16 kernels of pass 1 gain nothing: behind a product within the measurement's 1 %, behind another quantizer's pass 2 they lose 0.3 to
+  // 0.8 % (their first CTAs then fit beside the last ones of that pass only as the SM is).
   e = launch_divided(kStreamingCarveout, amax_f32_kernel, dim3(tiles), dim3(256), 0, s, reinterpret_cast<const float*>(a.x), a.rows, a.cols,
                     a.ld, tiles_c, has_row ? a.r_global : nullptr, has_col ? a.c_global : nullptr);
   count_launch();

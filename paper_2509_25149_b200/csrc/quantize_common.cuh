@@ -9,6 +9,9 @@
 
 namespace nvfp4 {
 
+// just more dynamic shared memory than two | three CTAs of an SM (228 KB, 1 KB of it taken per CTA) can have
+constexpr int kSmemOfHalf = 116 * 1024, kSmemOfThird = 76 * 1024;
+
 // ---------------------------------------------------------------------------------------------
 // small PTX helpers
 // ---------------------------------------------------------------------------------------------

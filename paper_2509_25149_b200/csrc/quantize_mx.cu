@@ -330,9 +330,6 @@ __global__ void __launch_bounds__(256, CTAS)
   }
 }
 
-// just more dynamic shared memory than two | three CTAs of an SM (228 KB, 1 KB of it taken per CTA) can have
-constexpr int kSmemOfHalf = 116 * 1024, kSmemOfThird = 76 * 1024;
-
 template <bool HR, bool HC, bool B2, bool RC, bool SR, bool OWN, int CTAS>
 static cudaError_t launch_mx_ctas(const QuantArgs& a, int sms, cudaStream_t s) {
   auto kern = quantize_mx_kernel<HR, HC, B2, RC, SR, OWN, CTAS>;

@@ -322,9 +322,6 @@ __global__ void __launch_bounds__(256, 3) quantize_rht_kernel(const RhtArgs ra) 
   }
 }
 
-// Shared memory with which one CTA, or two, fit an SM (228 KB, of which 1 KB a CTA is the system's)
-constexpr int kOnePerSm = 116 * 1024, kTwoPerSm = 77 * 1024;
-
 // Pass 2 with no more CTAs than SMs, or than twice as many, is given the shared memory with which no more fit an SM than an even spread
 // puts there: launched programmatically it becomes resident while a product or pass 1 still runs, and three crowd on each SM that is
 // free.  d = 4, ordinary launch / crowded / spread: gradient of 512 x 2048 with its amax provided, behind a product of 64 tiles, 20.4 /
@@ -336,7 +333,7 @@ cudaError_t launch_mode(const RhtArgs& ra, bool programmatic, int sms, cudaStrea
   static std::atomic<uint64_t> configured{0};  // per call site (template instantiation) and device
   int dev;
   if (device_needs_config(configured, &dev)) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kOnePerSm);
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemOfHalf);
     if (e != cudaSuccess) return e;
     device_configured(configured, dev);
   }
@@ -345,7 +342,7 @@ cudaError_t launch_mode(const RhtArgs& ra, bool programmatic, int sms, cudaStrea
   const dim3 grid((unsigned)tiles);
   count_launch();
   if (programmatic && !big) {
-    const int smem = MODE == 1 && tiles <= sms ? kOnePerSm : MODE == 1 && tiles <= 2 * sms ? kTwoPerSm : RhtSmem::kBytesSmall;
+    const int smem = MODE == 1 && tiles <= sms ? kSmemOfHalf : MODE == 1 && tiles <= 2 * sms ? kSmemOfThird : RhtSmem::kBytesSmall;
     return launch_kernel(kern, grid, dim3(256), smem, s, ra);
   }
   kern<<<grid, 256, big ? RhtSmem::kBytesBig : RhtSmem::kBytesSmall, s>>>(ra);

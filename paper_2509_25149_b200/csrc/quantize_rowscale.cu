@@ -213,7 +213,7 @@ __global__ void __launch_bounds__(256) quantize_rowscale_long_kernel(const Quant
 // up to four CTAs per SM have a share of 16 KB each as shared memory, and no more of them fit an SM than an even spread puts there.  Behind
 // a product of 64 tiles, ordinary / crowded / spread: 512 x 20608 39.6 / 51.2 / 36.7 us, 512 x 5120 14.4 / 15.1 / 12.5, with stochastic
 // rounding 44.4 / 73.6 / 39.1 and 14.4 / 18.0 / 13.4; forward of 256 x 1024 x 24576 with a fresh weight 65.1 / 86.2 / 61.3, of 1024 x 2048
-// x 2048 10.3 / 10.4 / 9.3.  For this the kernel asks for 5 %: CTAs of 3.5 KB and more then meet an SM divided at 16 KB; with 7 % some
+// x 2048 10.3 / 10.4 / 9.3.  For this the kernel asks for 5 %: CTAs of 3.5 KB and more then meet an SM divided at 16 KB; with 7 % most
 // sizes meet 32 KB (seen by how many were resident: of 4 KB eight).  From five CTAs per SM on the even shares would be below that; there
 // nothing lost against an ordinary launch of six (1024 x 7168 to 20480 x 5120, alone and behind a product 1.5 to 35 % faster).
 constexpr int kSpreadCarveout = 5, kSpreadBytes = 16384, kSpreadCtas = 4;
