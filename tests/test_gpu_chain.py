@@ -94,8 +94,9 @@ def test_a_call_sees_what_precedes_it(kind, before):
 @pytest.mark.parametrize("cols", [1024, 2048, 2560, 5120, 10240, 20480, 20608])
 @pytest.mark.parametrize("rounding", [B.ROUND_NEAREST_EVEN, B.ROUND_STOCHASTIC])
 def test_row_scaled_copies_of_any_length_in_a_chain(cols, rounding):
-    """The row-scaled quantizer is resident before the kernel that makes its source and the product that reads its last copy have
-    finished: the source and the copy are those of a quiet GPU all the same."""
+    """Behind kernels of torch's, whose end the quantizer waits for, and before the metric, which reads the copy without a pause: source and
+    copy are those of a quiet GPU.  (Copies that are overwritten while a kernel of this library may still read them:
+    test_row_scaled_copies_between_products.)"""
     rows = 128
     src = torch.randn((rows, cols), generator=torch.Generator("cuda").manual_seed(cols), device="cuda").to(torch.bfloat16)
     opts = B.quant_opts(rounding=rounding, seed=7, sr_offset=3)
@@ -121,8 +122,8 @@ def test_row_scaled_copies_of_any_length_in_a_chain(cols, rounding):
 @pytest.mark.parametrize("dim", [2, 8, 128])
 @pytest.mark.parametrize("copies", ["both", "row"])
 def test_other_transform_sizes_in_a_chain(dim, copies):
-    """The same for the kernel of the other transform sizes, which is launched either way (d = 128: by whether the transposed copy is
-    asked for)."""
+    """The order of the launches inside a call (words, pass 1, pass 2), behind kernels of torch's and into fresh copies.  (Shared copies:
+    test_other_transform_sizes_between_products.)"""
     rows, cols = 384, 640
     src = torch.randn((rows, cols), generator=torch.Generator("cuda").manual_seed(dim), device="cuda").to(torch.bfloat16)
     opts = B.quant_opts(rounding=1, rht_colwise=copies == "both", rht_rowwise=copies == "row", rht_sign_mask=0x73E5, rht_dim=dim, seed=1)
@@ -233,3 +234,14 @@ def test_other_transform_sizes_between_products(rows, cols, dim, form):
         t.glob[0] = 400.0  # (a bound on both products' outputs, and on their transforms')
     copies = [row] if form == "row" else [row, col]
     _Chain(rows, cols, lambda x: B.nvfp4_quantize(x, opts, row, col if form != "row" else None), copies).check()
+
+
+@pytest.mark.parametrize("rows,cols", [(256, 512), (2816, 2304)])
+@pytest.mark.parametrize("provided", [False, True])
+def test_binary32_weights_between_products(rows, cols, provided):
+    """Pass 1 of a binary32 source, which divides an SM for its loads, and pass 2 as the call's first kernel."""
+    row, col = B.alloc_tensor(rows, cols), B.alloc_tensor(cols, rows)
+    opts = B.quant_opts(block_rows=16, flags=B.INPUT_FP32 | (B.AMAX_PROVIDED if provided else 0))
+    for t in (row, col):
+        t.glob[0] = 400.0  # (a bound on both products' outputs)
+    _Chain(rows, cols, lambda x: B.nvfp4_quantize(x, opts, row, col), [row, col], fp32=True).check()
